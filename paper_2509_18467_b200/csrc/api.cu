@@ -67,13 +67,13 @@ __global__ void narrow_kernel(const float* __restrict__ x, bf16* __restrict__ y,
   if (i < n) y[i] = __float2bfloat16_rn(x[i]);
 }
 
-// Scratch of the exact layer backward: the chain conv_fwd -> gla_fwd -> gla_bwd -> conv_bwd in fp32. bf16 tensors are
+// Scratch of the exact layer backward: the chain conv_fwd -> gla_bwd -> conv_bwd in fp32. bf16 tensors are
 // widened to fp32 copies first and the four activation gradients narrowed at the end, so that no feature and no feature
 // gradient is rounded to bf16 between the stages.
 struct ExactBwdLayout {
   size_t in[10];    // q k v gate w_q w_k W dO cache_q cache_k  (fp32 copies; only for bf16 storage)
   size_t out[4];    // dq dk dv dgate (fp32; only for bf16 storage)
-  size_t qd, kd, dqd, dkd, o, den, ws_g, ws_c, total;
+  size_t qd, kd, dqd, dkd, ws_g, ws_c, total;
 };
 ExactBwdLayout exact_bwd_layout(const lawcat_params* p) {
   ExactBwdLayout L{};
@@ -90,7 +90,6 @@ ExactBwdLayout exact_bwd_layout(const lawcat_params* p) {
   for (int i = 0; i < 10; ++i) L.in[i] = take(widen ? 4 * n_in[i] : 0);
   for (int i = 0; i < 4; ++i) L.out[i] = take(widen ? 4 * n_in[i] : 0);
   L.qd = take(4 * n_in[0]); L.kd = take(4 * n_in[0]); L.dqd = take(4 * n_in[0]); L.dkd = take(4 * n_in[0]);
-  L.o = take(4 * n_in[7]); L.den = take(4 * elems(p, p->H, 1));
   L.ws_g = take(lawcat_workspace_bytes(&p32, LAWCAT_OP_GLA_BWD));
   L.ws_c = take(lawcat_workspace_bytes(&p32, LAWCAT_OP_CONV_BWD));
   L.total = off;
@@ -130,13 +129,15 @@ size_t lawcat_workspace_bytes(const lawcat_params* p, int op) {
   switch (op) {
     case LAWCAT_OP_CONV_BWD:
       return align_up(sizeof(float) * elems(p, p->H, p->d_k), 256) + align_up(sizeof(float) * elems(p, p->H_kv, p->d_k), 256);
+    case LAWCAT_OP_GLA_FWD:
+      return gla_tc_supported(*p) ? 0 : align_up(gla_fwd_rec_workspace_bytes(*p), 256);
     case LAWCAT_OP_GLA_BWD:
       if (gla_tc_bwd_supported(*p)) return gla_tc_bwd_workspace_bytes(*p);
       return align_up(sizeof(float) * elems(p, p->H, p->d_v), 256) + 2 * align_up(sizeof(float) * elems(p, p->H, 1), 256) +
              align_up(sizeof(float) * elems(p, p->H, p->d_k), 256);
     case LAWCAT_OP_LAYER_FWD:
       if (layer_tc_supported(*p)) return align_up(layer_tc_workspace_bytes(*p), 256);
-      return 2 * align_up(sizeof(float) * elems(p, p->H, p->d_k), 256);
+      return 2 * align_up(sizeof(float) * elems(p, p->H, p->d_k), 256) + align_up(gla_fwd_rec_workspace_bytes(*p), 256);
     case LAWCAT_OP_DECODE_STEP:
       return align_up(decode_workspace_bytes(*p), 256);
     case LAWCAT_OP_LAYER_BWD:
@@ -206,16 +207,15 @@ int lawcat_conv_bwd(const lawcat_params* p, const void* q, const void* k, const 
 int lawcat_gla_fwd(const lawcat_params* p, const void* qdot, const void* kdot, const void* v, const void* gate,
                    const float* S0, const float* z0, void* o, float* den, float* S_T, float* z_T, void* ws,
                    size_t ws_bytes, void* stream, int* dev_status) {
-  (void)ws; (void)ws_bytes;
   int r = check_params(p, true);
   if (r) return r;
   const void* const req[] = {qdot, kdot, v, gate, o};
-  const void* const opt[] = {S0, z0, den, S_T, z_T};
+  const void* const opt[] = {S0, z0, den, S_T, z_T, ws};
   if ((r = check_ptrs(req, opt, (size_t)p->B * p->T == 0))) return r;
   Ctx c{p, (cudaStream_t)stream, dev_status};
   if ((size_t)p->B * p->T != 0 && gla_tc_supported(*p))  // chunkwise tensor-core kernel
     return launch_gla_fwd_tc(c, qdot, kdot, v, gate, S0, z0, o, den, S_T, z_T);
-  return launch_gla_fwd_rec(c, qdot, kdot, false, v, gate, S0, z0, o, den, S_T, z_T);
+  return launch_gla_fwd_rec(c, qdot, kdot, false, v, gate, S0, z0, o, den, S_T, z_T, ws, ws_bytes);
 }
 
 int lawcat_gla_bwd(const lawcat_params* p, const void* qdot, const void* kdot, const void* v, const void* gate,
@@ -256,7 +256,8 @@ int lawcat_layer_fwd(const lawcat_params* p, const void* q, const void* k, const
                            z_T, ws);
   }
   float* qdot = (float*)ws;
-  float* kdot = (float*)((char*)ws + align_up(sizeof(float) * elems(p, p->H, p->d_k), 256));
+  const size_t nf = align_up(sizeof(float) * elems(p, p->H, p->d_k), 256);
+  float* kdot = (float*)((char*)ws + nf);
   // The feature maps of Section 2 other than the softmax (1 + ELU, identity) on head width 64: tensor-core conv + mix +
   // phi into fp32 scratch, then the chunkwise tensor-core attention on those features.
   if ((size_t)p->B * p->T != 0 && (p->phi != LAWCAT_PHI_SOFTMAX || p->mix_unshared) && p->chunk != 1 &&
@@ -267,7 +268,8 @@ int lawcat_layer_fwd(const lawcat_params* p, const void* q, const void* k, const
   }
   // exact path: conv + mix + phi into fp32 scratch, then the recurrent GLA
   if ((r = launch_convmix_fwd(c, q, k, w_q, w_k, W, cache_q_in, cache_k_in, qdot, kdot, true, true))) return r;
-  if ((r = launch_gla_fwd_rec(c, qdot, kdot, true, v, gate, S0, z0, o, nullptr, S_T, z_T))) return r;
+  if ((r = launch_gla_fwd_rec(c, qdot, kdot, true, v, gate, S0, z0, o, nullptr, S_T, z_T,
+                              (char*)ws + 2 * nf, ws_bytes - 2 * nf))) return r;
   return launch_cache_out(c, q, k, cache_q_in, cache_k_in, cache_q_out, cache_k_out);
 }
 
@@ -380,8 +382,7 @@ int lawcat_layer_bwd(const lawcat_params* p, const void* q, const void* k, const
   }
   if ((size_t)p->B * p->T != 0) {
     if ((r = launch_convmix_fwd(c32, in[0], in[1], in[4], in[5], in[6], in[8], in[9], w + L.qd, w + L.kd, false, true))) return r;
-    if ((r = launch_gla_fwd_rec(c32, w + L.qd, w + L.kd, false, in[2], in[3], S0, z0, w + L.o, (float*)(w + L.den), nullptr, nullptr))) return r;
-    if ((r = launch_gla_bwd_rec(c32, w + L.qd, w + L.kd, in[2], in[3], S0, z0, w + L.o, (const float*)(w + L.den), in[7],
+    if ((r = launch_gla_bwd_rec(c32, w + L.qd, w + L.kd, in[2], in[3], S0, z0, nullptr, nullptr, in[7],
                                 w + L.dqd, w + L.dkd, out[2], out[3], w + L.ws_g)))
       return r;
   }

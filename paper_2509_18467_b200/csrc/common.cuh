@@ -61,7 +61,8 @@ int launch_cache_out(const Ctx& c, const void* q, const void* k, const void* cac
                      void* cache_q_out, void* cache_k_out);
 int launch_gla_fwd_rec(const Ctx& c, const void* qdot, const void* kdot, bool qk_f32, const void* v,
                        const void* gate, const float* S0, const float* z0, void* o, float* den, float* S_T,
-                       float* z_T);
+                       float* z_T, void* ws, size_t ws_bytes);
+size_t gla_fwd_rec_workspace_bytes(const lawcat_params& p);  // (without it the call runs one block per head)
 int launch_gla_bwd_rec(const Ctx& c, const void* qdot, const void* kdot, const void* v, const void* gate,
                        const float* S0, const float* z0, const void* o, const float* den, const void* dO,
                        void* d_qdot, void* d_kdot, void* dv, void* dgate, void* ws);
@@ -71,6 +72,7 @@ int launch_decode(const Ctx& c, const void* q_t, const void* k_t, const void* v_
 size_t decode_workspace_bytes(const lawcat_params& p);
 
 // Host-side check of a parameter block (api.cu): LAWCAT_OK, LAWCAT_ERR_INVALID_ARG or LAWCAT_ERR_UNSUPPORTED.
+int sm_count();  // of the current device (layer_tc.cu)
 int validate_params(const lawcat_params* p, bool need_T);
 
 // Chunkwise tensor-core layer forward (layer_tc.cu): whether it takes these parameters, and its launcher.

@@ -12,6 +12,7 @@
 //   dg_s    = sum_{t>=s} (qdot_t*dqdot_t - kdot_t*dkdot_t)   (o' depends on the log-decays only through their running
 //             sum), accumulated in the same reverse sweep that produces dkdot.
 #include "common.cuh"
+#include "tc_common.cuh"
 
 namespace lawcat {
 
@@ -28,113 +29,6 @@ struct GlaArgs {
   float inv_tau, eps;
 };
 
-// ------------------------------------------------------------------------------------------------ forward
-// Thread (rg, col): column col of S' (col == dv is the z column), rows [rg*R, rg*R+R). o'_t[col] is a sum over rows:
-// in-thread over R rows, then over the row groups through shared memory once per staged batch.
-template <typename TQ, typename TS, int R>
-__global__ void gla_fwd_rec_kernel(GlaArgs a) {
-  extern __shared__ __align__(16) float smem[];
-  const int dk = a.dk, dv = a.dv, Tn = a.T, H = a.H;
-  const int CW = (dv + 1 + 31) / 32 * 32, RG = dk / R;
-  float* s_alpha = smem;               // [TB][dk]
-  float* s_k = s_alpha + TB * dk;      // [TB][dk]
-  float* s_q = s_k + TB * dk;          // [TB][dk]
-  float* s_v = s_q + TB * dk;          // [TB][CW]
-  float* s_part = s_v + TB * CW;       // [TB][RG][CW]
-  const int b = blockIdx.x / H, h = blockIdx.x % H, j = h / (H / a.Hkv);
-  const int tid = threadIdx.x, nthr = blockDim.x;
-  const int rg = tid / CW, col = tid % CW;
-  const bool active = col <= dv;
-  const TQ* qdot = (const TQ*)a.qdot;
-  const TQ* kdot = (const TQ*)a.kdot;
-  const TS* v = (const TS*)a.v;
-  const TS* gate = (const TS*)a.gate;
-  TS* o = (TS*)a.out_o;
-  float S[R];
-#pragma unroll
-  for (int r = 0; r < R; ++r) {
-    const int row = rg * R + r;
-    float s0 = 0.f;
-    if (col < dv && a.S0) s0 = a.S0[(((size_t)b * H + h) * dk + row) * dv + col];
-    if (col == dv && a.z0) s0 = a.z0[((size_t)b * H + h) * dk + row];
-    S[r] = s0;
-  }
-  for (int t0 = 0; t0 < Tn; t0 += TB) {
-    const int nt = min(TB, Tn - t0);
-    for (int i = tid; i < nt * dk; i += nthr) {
-      const int tok = i / dk, c = i % dk;
-      const size_t th = ((size_t)b * Tn + t0 + tok) * H + h;
-      s_q[i] = ldf(qdot + th * dk + c);
-      s_k[i] = ldf(kdot + th * dk + c);
-      s_alpha[i] = expf(log_decay(ldf(gate + th * a.gd + (a.gd == 1 ? 0 : c)), a.gate_mode, a.inv_tau));
-    }
-    for (int i = tid; i < nt * CW; i += nthr) {
-      const int tok = i / CW, e = i % CW;
-      s_v[i] = e < dv ? ldf(v + (((size_t)b * Tn + t0 + tok) * a.Hkv + j) * dv + e) : (e == dv ? 1.f : 0.f);
-    }
-    __syncthreads();
-    if (active) {
-      for (int tok = 0; tok < nt; ++tok) {
-        const float vc = s_v[tok * CW + col];
-        const float4* a4 = reinterpret_cast<const float4*>(s_alpha + tok * dk + rg * R);
-        const float4* k4 = reinterpret_cast<const float4*>(s_k + tok * dk + rg * R);
-        const float4* q4 = reinterpret_cast<const float4*>(s_q + tok * dk + rg * R);
-        float acc = 0.f;
-#pragma unroll
-        for (int r4 = 0; r4 < R / 4; ++r4) {
-          const float4 al = a4[r4], kk = k4[r4], qq = q4[r4];
-          S[4 * r4 + 0] = fmaf(al.x, S[4 * r4 + 0], kk.x * vc); acc = fmaf(qq.x, S[4 * r4 + 0], acc);
-          S[4 * r4 + 1] = fmaf(al.y, S[4 * r4 + 1], kk.y * vc); acc = fmaf(qq.y, S[4 * r4 + 1], acc);
-          S[4 * r4 + 2] = fmaf(al.z, S[4 * r4 + 2], kk.z * vc); acc = fmaf(qq.z, S[4 * r4 + 2], acc);
-          S[4 * r4 + 3] = fmaf(al.w, S[4 * r4 + 3], kk.w * vc); acc = fmaf(qq.w, S[4 * r4 + 3], acc);
-        }
-        s_part[(tok * RG + rg) * CW + col] = acc;
-      }
-    }
-    __syncthreads();
-    for (int i = tid; i < nt * dv; i += nthr) {
-      const int tok = i / dv, e = i % dv;
-      float num = 0.f, dn = a.eps;
-      for (int g = 0; g < RG; ++g) {
-        num += s_part[(tok * RG + g) * CW + e];
-        dn += s_part[(tok * RG + g) * CW + dv];
-      }
-      const size_t th = ((size_t)b * Tn + t0 + tok) * H + h;
-      stf(o + th * dv + e, a.normalize ? num / dn : num);
-      if (e == 0 && a.out_den) a.out_den[th] = dn;
-    }
-    __syncthreads();
-  }
-  if (active) {
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const int row = rg * R + r;
-      if (col < dv && a.S_T) a.S_T[(((size_t)b * H + h) * dk + row) * dv + col] = S[r];
-      if (col == dv && a.z_T) a.z_T[((size_t)b * H + h) * dk + row] = S[r];
-    }
-  }
-}
-
-template <typename TQ, typename TS>
-static int gla_fwd_launch(const Ctx& c, GlaArgs& a) {
-  const lawcat_params& p = *c.p;
-  if (p.B * p.H == 0) return LAWCAT_OK;
-  const int RG = p.d_k >= 64 ? 4 : (p.d_k >= 32 ? 2 : 1), R = p.d_k / RG;  // (at most 4 x 160 threads)
-  const int CW = (p.d_v + 1 + 31) / 32 * 32;
-  const size_t smem = sizeof(float) * ((size_t)3 * TB * p.d_k + (size_t)TB * CW + (size_t)TB * RG * CW);
-  const int threads = RG * CW;
-  const unsigned grid = p.B * p.H;
-  LaunchScope _ls("gla_fwd_rec", c.stream);
-  switch (R) {
-    case 16: gla_fwd_rec_kernel<TQ, TS, 16><<<grid, threads, smem, c.stream>>>(a); break;
-    case 32: gla_fwd_rec_kernel<TQ, TS, 32><<<grid, threads, smem, c.stream>>>(a); break;
-    case 64: gla_fwd_rec_kernel<TQ, TS, 64><<<grid, threads, smem, c.stream>>>(a); break;
-    default: return LAWCAT_ERR_UNSUPPORTED;
-  }
-  LAWCAT_CHECK_LAUNCH();
-  return LAWCAT_OK;
-}
-
 static GlaArgs base_args(const lawcat_params& p) {
   GlaArgs a{};
   a.B = p.B; a.T = p.T; a.H = p.H; a.Hkv = p.H_kv; a.dk = p.d_k; a.dv = p.d_v; a.gd = p.gate_dim;
@@ -142,9 +36,312 @@ static GlaArgs base_args(const lawcat_params& p) {
   return a;
 }
 
+// ------------------------------------------------------------------------------------------------ forward
+// The recurrence is cut along T into segments that run at the same time: (1) every segment but the last computes its end
+// state from a zero state, and its total decay (MODE 1); (2) every segment folds the pieces in front of it into its start
+// state (Eq. 4 unrolled over whole segments) and runs the recurrence with its read-out (MODE 0). One block per head, as
+// the recurrence alone would give, leaves a 32-head call at 1.2 us per token (T = 4096, d = 128: 4.27 ms); what bounds
+// the cut form is the fp32 pipe: two multiply-adds per token and state entry, one more for the first pass.
+//
+// Thread (rg, column pair): rows [rg*R, rg*R+R) x 2 columns of S in registers, rows in packed pairs. Tokens are taken in
+// batches of TBF. Inside a batch the state is kept divided by the decay A_t since the batch's start, S~ = S / A_t, so that
+// a token costs S~ += (k_t / A_t) v_t and o_t += (q_t A_t) S~ -- the decay itself multiplies S once per batch. A batch in
+// which some A falls below 2^-80 (1/A would approach the end of the fp32 range) runs the plain S = alpha S + k v instead.
+// The normalizer row z is a prefix over (A, k) pairs formed by the threads that stage the batch.
+constexpr int TBF = 16;                  // tokens per batch
+constexpr int TPP_MAX = 8;               // tokens a thread stages per batch, at most (fwd_threads)
+constexpr float A_MIN = 8.2718061e-25f;  // 2^-80
+constexpr int MAX_FWD_SEG = 16;          // (a segment reads the pieces of all segments in front of it)
+
+struct SegArgs {
+  int nseg, seg_len;            // segments per sequence, tokens per segment (a multiple of TBF)
+  float *loc_S, *loc_z, *dec;   // pieces: [B,H,nseg-1,dk,dv], [B,H,nseg-1,dk], total decay [B,H,nseg-1,dk]
+};
+
+// decay of one token: sigmoid(a)^(1/tau), or exp(a)
+__device__ __forceinline__ float decay_of(float a, int gate_mode, float inv_tau) {
+  if (gate_mode != LAWCAT_GATE_LOGDECAY && inv_tau == 1.f) {
+    const float e = expf(-fabsf(a)), r = 1.f / (1.f + e);
+    return a >= 0.f ? r : e * r;
+  }
+  return expf(log_decay(a, gate_mode, inv_tau));
+}
+
+template <typename TQ, typename TS, int R, int MODE>
+__global__ void __launch_bounds__(256, 2) gla_fwd_rec_kernel(const GlaArgs a, const SegArgs sgm) {
+  using namespace tc;
+  extern __shared__ __align__(16) float smem[];
+  const int dk = a.dk, dv = a.dv, H = a.H;
+  const int CP = dv / 2, RG = dk / R;
+  const int tid = threadIdx.x, nthr = blockDim.x;
+  const int P = nthr / dk, TPP = TBF / P;  // staging: P threads per channel, TPP consecutive tokens each
+  float* s_k = smem;                    // [TBF][dk]  k / A  (plain batch: k)
+  float* s_v = s_k + TBF * dk;          // [TBF][dv]
+  float* s_al = s_v + TBF * dv;         // [TBF][dk]  alpha (plain batch only)
+  float* s_pA = s_al + TBF * dk;        // [P][dk] decay of each part of the batch, [P][dk] its own z
+  float* s_ab = s_pA + 2 * nthr;        // [dk] decay of the batch
+  float* s_q = s_ab + dk;               // [TBF][dk]  q A  (plain batch: q)
+  float* s_den = s_q + TBF * dk;        // [TBF][4] partial q.z
+  float* s_part = s_den + TBF * 4;      // [TBF][RG][dv]
+  const int nseg_run = MODE == 1 ? sgm.nseg - 1 : sgm.nseg;
+  const int bh = blockIdx.x / nseg_run, seg = blockIdx.x % nseg_run;
+  const int b = bh / H, h = bh % H, j = h / (H / a.Hkv);
+  const int t_begin = seg * sgm.seg_len, t_end = min(a.T, t_begin + sgm.seg_len);
+  const int cp = tid % CP, rg = tid / CP;
+  const bool active = rg < RG;
+  const int row0 = rg * R, c0 = 2 * cp;
+  const int sc = tid % dk, sp = tid / dk;  // staging: channel, part
+  const TQ* qdot = (const TQ*)a.qdot;
+  const TQ* kdot = (const TQ*)a.kdot;
+  const TS* v = (const TS*)a.v;
+  const TS* gate = (const TS*)a.gate;
+  TS* o = (TS*)a.out_o;
+
+  // start state
+  float S[R][2];
+  float z = 0.f, dtot = 1.f;
+#pragma unroll
+  for (int r = 0; r < R; ++r) S[r][0] = S[r][1] = 0.f;
+  if (MODE == 0) {
+    if (active && a.S0) {
+      const float* src = a.S0 + ((size_t)bh * dk + row0) * dv + c0;
+#pragma unroll
+      for (int r = 0; r < R; ++r) { S[r][0] = src[(size_t)r * dv]; S[r][1] = src[(size_t)r * dv + 1]; }
+    }
+    if (a.z0) z = a.z0[(size_t)bh * dk + sc];
+    for (int i = 0; i < seg; ++i) {
+      const size_t pi = (size_t)bh * (sgm.nseg - 1) + i;
+      if (active) {
+        const float* src = sgm.loc_S + (pi * dk + row0) * dv + c0;
+        const float* dc = sgm.dec + pi * dk + row0;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const float2 l = *reinterpret_cast<const float2*>(src + (size_t)r * dv);
+          const float d = dc[r];
+          S[r][0] = fmaf(d, S[r][0], l.x);
+          S[r][1] = fmaf(d, S[r][1], l.y);
+        }
+      }
+      z = fmaf(sgm.dec[pi * dk + sc], z, sgm.loc_z[pi * dk + sc]);
+    }
+  }
+  uint64_t S2[R / 2][2];
+#pragma unroll
+  for (int r = 0; r < R / 2; ++r) {
+    S2[r][0] = f2_pack(S[2 * r][0], S[2 * r + 1][0]);
+    S2[r][1] = f2_pack(S[2 * r][1], S[2 * r + 1][1]);
+  }
+
+  for (int t0 = t_begin; t0 < t_end; t0 += TBF) {
+    const int nt = min(TBF, t_end - t0);
+    // ---- staging: this thread's channel, tokens [sp TPP, sp TPP + TPP) of the batch (tokens past the end: no decay, k = 0)
+    float al[TPP_MAX], kk[TPP_MAX], qq[TPP_MAX];
+#pragma unroll
+    for (int i = 0; i < TPP_MAX; ++i) {
+      if (i >= TPP) break;
+      const int tok = sp * TPP + i;
+      al[i] = 1.f; kk[i] = 0.f; qq[i] = 0.f;
+      if (tok < nt) {
+        const size_t th = ((size_t)b * a.T + t0 + tok) * H + h;
+        kk[i] = ldf(kdot + th * dk + sc);
+        if (MODE == 0) qq[i] = ldf(qdot + th * dk + sc);
+        al[i] = ldf(gate + th * a.gd + (a.gd == 1 ? 0 : sc));
+      }
+    }
+    for (int i = tid; i < TBF * dv; i += nthr) {
+      const int tok = i / dv, e = i % dv;
+      s_v[i] = tok < nt ? ldf(v + (((size_t)b * a.T + t0 + tok) * a.Hkv + j) * dv + e) : 0.f;
+    }
+    float A = 1.f, zl = 0.f;
+#pragma unroll
+    for (int i = 0; i < TPP_MAX; ++i) {
+      if (i >= TPP) break;
+      al[i] = sp * TPP + i < nt ? decay_of(al[i], a.gate_mode, a.inv_tau) : 1.f;
+      A *= al[i];
+      zl = fmaf(al[i], zl, kk[i]);
+    }
+    s_pA[tid] = A;
+    s_pA[nthr + tid] = zl;
+    __syncthreads();
+    float Ain = 1.f, zin = z, Aall = 1.f;  // decay since the batch's start and z in front of this thread's first token
+    for (int p = 0; p < P; ++p) {
+      const float Ap = s_pA[p * dk + sc], zp = s_pA[nthr + p * dk + sc];
+      if (p < sp) { zin = fmaf(Ap, zin, zp); Ain *= Ap; }
+      z = fmaf(Ap, z, zp);
+      Aall *= Ap;
+    }
+    dtot *= Aall;
+    if (sp == 0) s_ab[sc] = Aall;
+    const bool plain = __syncthreads_or(Aall < A_MIN);
+    A = Ain;
+#pragma unroll
+    for (int i = 0; i < TPP_MAX; ++i) {
+      if (i >= TPP) break;
+      const int tok = sp * TPP + i;
+      A *= al[i];
+      zin = fmaf(al[i], zin, kk[i]);
+      if (plain) {
+        s_k[tok * dk + sc] = kk[i];
+        s_al[tok * dk + sc] = al[i];
+        if (MODE == 0) s_q[tok * dk + sc] = qq[i];
+      } else {
+        s_k[tok * dk + sc] = kk[i] / A;
+        if (MODE == 0) s_q[tok * dk + sc] = qq[i] * A;
+      }
+      if (MODE == 0) {
+        float d = qq[i] * zin;
+        for (int off = min(16, dk >> 1); off > 0; off >>= 1) d += __shfl_xor_sync(0xffffffffu, d, off);
+        if ((sc & 31) == 0) s_den[tok * 4 + (sc >> 5)] = d;
+      }
+    }
+    __syncthreads();
+    // ---- the recurrence over the batch
+    if (active) {
+#pragma unroll 1
+      for (int tok = 0; tok < TBF; ++tok) {
+        const float2 vv = *reinterpret_cast<const float2*>(s_v + tok * dv + c0);
+        const uint64_t v0 = f2_pack(vv.x, vv.x), v1 = f2_pack(vv.y, vv.y);
+        const ulonglong2* k4 = reinterpret_cast<const ulonglong2*>(s_k + tok * dk + row0);
+        const ulonglong2* q4 = reinterpret_cast<const ulonglong2*>(s_q + tok * dk + row0);
+        const ulonglong2* a4 = reinterpret_cast<const ulonglong2*>(s_al + tok * dk + row0);
+        uint64_t acc0 = 0ull, acc1 = 0ull;
+#pragma unroll
+        for (int r4 = 0; r4 < R / 4; ++r4) {
+          const ulonglong2 k2 = k4[r4];
+          if (plain) {
+            const ulonglong2 al2 = a4[r4];
+            S2[2 * r4][0] = f2_fma(al2.x, S2[2 * r4][0], f2_mul(k2.x, v0));
+            S2[2 * r4][1] = f2_fma(al2.x, S2[2 * r4][1], f2_mul(k2.x, v1));
+            S2[2 * r4 + 1][0] = f2_fma(al2.y, S2[2 * r4 + 1][0], f2_mul(k2.y, v0));
+            S2[2 * r4 + 1][1] = f2_fma(al2.y, S2[2 * r4 + 1][1], f2_mul(k2.y, v1));
+          } else {
+            S2[2 * r4][0] = f2_fma(k2.x, v0, S2[2 * r4][0]);
+            S2[2 * r4][1] = f2_fma(k2.x, v1, S2[2 * r4][1]);
+            S2[2 * r4 + 1][0] = f2_fma(k2.y, v0, S2[2 * r4 + 1][0]);
+            S2[2 * r4 + 1][1] = f2_fma(k2.y, v1, S2[2 * r4 + 1][1]);
+          }
+          if (MODE == 0) {
+            const ulonglong2 q2 = q4[r4];
+            acc0 = f2_fma(q2.x, S2[2 * r4][0], acc0);
+            acc1 = f2_fma(q2.x, S2[2 * r4][1], acc1);
+            acc0 = f2_fma(q2.y, S2[2 * r4 + 1][0], acc0);
+            acc1 = f2_fma(q2.y, S2[2 * r4 + 1][1], acc1);
+          }
+        }
+        if (MODE == 0) {
+          float x0, y0, x1, y1;
+          f2_unpack(acc0, x0, y0);
+          f2_unpack(acc1, x1, y1);
+          *reinterpret_cast<float2*>(s_part + (tok * RG + rg) * dv + c0) = make_float2(x0 + y0, x1 + y1);
+        }
+      }
+      if (!plain) {  // back to the state itself
+        const ulonglong2* d4 = reinterpret_cast<const ulonglong2*>(s_ab + row0);
+#pragma unroll
+        for (int r4 = 0; r4 < R / 4; ++r4) {
+          const ulonglong2 d2 = d4[r4];
+          S2[2 * r4][0] = f2_mul(d2.x, S2[2 * r4][0]);
+          S2[2 * r4][1] = f2_mul(d2.x, S2[2 * r4][1]);
+          S2[2 * r4 + 1][0] = f2_mul(d2.y, S2[2 * r4 + 1][0]);
+          S2[2 * r4 + 1][1] = f2_mul(d2.y, S2[2 * r4 + 1][1]);
+        }
+      }
+    }
+    __syncthreads();
+    if (MODE == 0) {
+      for (int i = tid; i < nt * dv; i += nthr) {
+        const int tok = i / dv, e = i % dv;
+        float num = 0.f, dn = a.eps;
+        for (int g = 0; g < RG; ++g) num += s_part[(tok * RG + g) * dv + e];
+        for (int g = 0; g < (dk + 31) / 32; ++g) dn += s_den[tok * 4 + g];
+        const size_t th = ((size_t)b * a.T + t0 + tok) * H + h;
+        stf(o + th * dv + e, a.normalize ? num / dn : num);
+        if (e == 0 && a.out_den) a.out_den[th] = dn;
+      }
+      // (the next batch writes s_den and s_part behind barriers of its own; s_v is read by nobody here)
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < R / 2; ++r) {
+    f2_unpack(S2[r][0], S[2 * r][0], S[2 * r + 1][0]);
+    f2_unpack(S2[r][1], S[2 * r][1], S[2 * r + 1][1]);
+  }
+  float* const dS = MODE == 1 ? sgm.loc_S + (size_t)blockIdx.x * dk * dv
+                              : (a.S_T && seg == sgm.nseg - 1) ? a.S_T + (size_t)bh * dk * dv : nullptr;
+  float* const dz = MODE == 1 ? sgm.loc_z + (size_t)blockIdx.x * dk
+                              : (a.z_T && seg == sgm.nseg - 1) ? a.z_T + (size_t)bh * dk : nullptr;
+  if (dS && active) {
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+      *reinterpret_cast<float2*>(dS + (size_t)(row0 + r) * dv + c0) = make_float2(S[r][0], S[r][1]);
+  }
+  if (sp == 0) {
+    if (dz) dz[sc] = z;
+    if (MODE == 1) sgm.dec[(size_t)blockIdx.x * dk + sc] = dtot;
+  }
+}
+
+// threads of the forward kernel: RG row groups x dv / 2 column pairs, at least 128, and at least two per channel at dk = 128
+static int fwd_rows(int dk) { return dk >= 64 ? dk / 4 : 16; }
+static int fwd_threads(const lawcat_params& p) {
+  const int n = (p.d_k / fwd_rows(p.d_k)) * (p.d_v / 2), lo = p.d_k == 128 ? 256 : 128;
+  return n < lo ? lo : n;
+}
+
+// Segments per sequence: two blocks per SM are resident; a segment has at least two batches, and more than 16 segments
+// would spend longer on reading the pieces in front than the cut saves.
+static SegArgs fwd_plan(const lawcat_params& p) {
+  SegArgs s{};
+  const int slots = 2 * sm_count(), batches = (p.T + TBF - 1) / TBF;
+  int n = slots / (p.B * p.H);
+  if (n > MAX_FWD_SEG) n = MAX_FWD_SEG;
+  if (n > batches / 2) n = batches / 2;
+  if (n < 1) n = 1;
+  s.seg_len = (batches + n - 1) / n * TBF;
+  s.nseg = (p.T + s.seg_len - 1) / s.seg_len;
+  if (s.nseg < 1) s.nseg = 1;
+  return s;
+}
+
+size_t gla_fwd_rec_workspace_bytes(const lawcat_params& p) {
+  if (p.B * p.H == 0 || p.T == 0) return 0;
+  const SegArgs s = fwd_plan(p);
+  return sizeof(float) * (size_t)p.B * p.H * (s.nseg - 1) * ((size_t)p.d_k * p.d_v + 2 * p.d_k);
+}
+
+template <typename TQ, typename TS>
+static int gla_fwd_launch(const Ctx& c, GlaArgs& a, void* ws, size_t ws_bytes) {
+  const lawcat_params& p = *c.p;
+  if (p.B * p.H == 0) return LAWCAT_OK;
+  SegArgs s = fwd_plan(p);
+  if (s.nseg > 1 && (!ws || ws_bytes < gla_fwd_rec_workspace_bytes(p))) {  // (a caller without scratch: one segment)
+    s.nseg = 1;
+    s.seg_len = (p.T + TBF - 1) / TBF * TBF;
+  }
+  const int BH = p.B * p.H, R = fwd_rows(p.d_k), RG = p.d_k / R, thr = fwd_threads(p);
+  const size_t pieces = (size_t)BH * (s.nseg - 1);
+  s.loc_S = (float*)ws;
+  s.loc_z = s.loc_S + pieces * p.d_k * p.d_v;
+  s.dec = s.loc_z + pieces * p.d_k;
+  const size_t smem1 = sizeof(float) * ((size_t)TBF * (2 * p.d_k + p.d_v) + 2 * thr + p.d_k);
+  const size_t smem0 = smem1 + sizeof(float) * ((size_t)TBF * p.d_k + 4 * TBF + (size_t)TBF * RG * p.d_v);
+  auto* const k_state = R == 32 ? gla_fwd_rec_kernel<TQ, TS, 32, 1> : gla_fwd_rec_kernel<TQ, TS, 16, 1>;
+  auto* const k_full = R == 32 ? gla_fwd_rec_kernel<TQ, TS, 32, 0> : gla_fwd_rec_kernel<TQ, TS, 16, 0>;
+  if (cudaFuncSetAttribute(k_full, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem0) != cudaSuccess) return LAWCAT_ERR_CUDA;
+  if (s.nseg > 1) {
+    LaunchScope _ls("gla_fwd_rec_state", c.stream);
+    k_state<<<(unsigned)pieces, thr, smem1, c.stream>>>(a, s);
+    LAWCAT_CHECK_LAUNCH();
+  }
+  LaunchScope _ls("gla_fwd_rec", c.stream);
+  k_full<<<(unsigned)(BH * s.nseg), thr, smem0, c.stream>>>(a, s);
+  LAWCAT_CHECK_LAUNCH();
+  return LAWCAT_OK;
+}
+
 int launch_gla_fwd_rec(const Ctx& c, const void* qdot, const void* kdot, bool qk_f32, const void* v,
                        const void* gate, const float* S0, const float* z0, void* o, float* den, float* S_T,
-                       float* z_T) {
+                       float* z_T, void* ws, size_t ws_bytes) {
   const lawcat_params& p = *c.p;
   GlaArgs a = base_args(p);
   a.qdot = qdot; a.kdot = kdot; a.v = v; a.gate = gate; a.S0 = S0; a.z0 = z0;
@@ -157,9 +354,9 @@ int launch_gla_fwd_rec(const Ctx& c, const void* qdot, const void* kdot, bool qk
       return LAWCAT_ERR_CUDA;
     return LAWCAT_OK;
   }
-  if (p.dtype == LAWCAT_F32) return gla_fwd_launch<float, float>(c, a);
-  if (qk_f32) return gla_fwd_launch<float, bf16>(c, a);
-  return gla_fwd_launch<bf16, bf16>(c, a);
+  if (p.dtype == LAWCAT_F32) return gla_fwd_launch<float, float>(c, a, ws, ws_bytes);
+  if (qk_f32) return gla_fwd_launch<float, bf16>(c, a, ws, ws_bytes);
+  return gla_fwd_launch<bf16, bf16>(c, a, ws, ws_bytes);
 }
 
 // ------------------------------------------------------------------------------------------------ backward sweeps

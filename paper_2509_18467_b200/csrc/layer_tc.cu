@@ -95,7 +95,7 @@ __global__ void segment_scan_kernel(const float* __restrict__ S0, const float* _
 }  // namespace tc
 
 // Number of SMs of the current device (cached per device; 148 on a B200).
-static int sm_count() {
+int sm_count() {
   static int cached[64] = {};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 148;
