@@ -11,6 +11,8 @@
 //   dv'_t   = kdot_t dS'_t                        columns owned by threads
 //   dg_s    = sum_{t>=s} (qdot_t*dqdot_t - kdot_t*dkdot_t)   (o' depends on the log-decays only through their running
 //             sum), accumulated in the same reverse sweep that produces dkdot.
+#include <type_traits>
+
 #include "common.cuh"
 #include "tc_common.cuh"
 
@@ -43,248 +45,357 @@ static GlaArgs base_args(const lawcat_params& p) {
 // the recurrence alone would give, leaves a 32-head call at 1.2 us per token (T = 4096, d = 128: 4.27 ms); what bounds
 // the cut form is the fp32 pipe: two multiply-adds per token and state entry, one more for the first pass.
 //
-// Thread (rg, column pair): rows [rg*R, rg*R+R) x 2 columns of S in registers, rows in packed pairs. Tokens are taken in
-// batches of TBF. Inside a batch the state is kept divided by the decay A_t since the batch's start, S~ = S / A_t, so that
+// Thread (rg, column quad): R rows x 4 columns of S in registers, rows in packed pairs: rows 4 (rg + RG i) .. + 3, so that the
+// RG neighbouring lanes of a row read 16 RG consecutive bytes of k and q per step, and the sum over the rows of a column ends
+// in a few shuffles. Tokens are taken in batches of TBF. Inside a batch the state is kept divided by the decay A_t since the batch's start, S~ = S / A_t, so that
 // a token costs S~ += (k_t / A_t) v_t and o_t += (q_t A_t) S~ -- the decay itself multiplies S once per batch. A batch in
 // which some A falls below 2^-80 (1/A would approach the end of the fp32 range) runs the plain S = alpha S + k v instead.
 // The normalizer row z is a prefix over (A, k) pairs formed by the threads that stage the batch.
 constexpr int TBF = 16;                  // tokens per batch
-constexpr int TPP_MAX = 8;               // tokens a thread stages per batch, at most (fwd_threads)
 constexpr float A_MIN = 8.2718061e-25f;  // 2^-80
 constexpr int MAX_FWD_SEG = 16;          // (a segment reads the pieces of all segments in front of it)
+
+constexpr __host__ __device__ int fwd_groups(int dk) { return dk >= 64 ? 8 : dk / 8; }  // row groups
 
 struct SegArgs {
   int nseg, seg_len;            // segments per sequence, tokens per segment (a multiple of TBF)
   float *loc_S, *loc_z, *dec;   // pieces: [B,H,nseg-1,dk,dv], [B,H,nseg-1,dk], total decay [B,H,nseg-1,dk]
 };
 
-// decay of one token: sigmoid(a)^(1/tau), or exp(a)
-__device__ __forceinline__ float decay_of(float a, int gate_mode, float inv_tau) {
-  if (gate_mode != LAWCAT_GATE_LOGDECAY && inv_tau == 1.f) {
-    const float e = expf(-fabsf(a)), r = 1.f / (1.f + e);
-    return a >= 0.f ? r : e * r;
+// decays of N tokens: sigmoid(a)^(1/tau), or exp(a). (tau = 1: e / (1 + e) by one exponential and one reciprocal; else only
+// the absolute error of log(1 + e^-|a|) / tau counts, so the logarithm may be the hardware's.)
+template <int N>
+__device__ __forceinline__ void decays_of(float (&a)[N], int gate_mode, float inv_tau) {
+  if (gate_mode == LAWCAT_GATE_LOGDECAY) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) a[i] = expf(a[i]);
+  } else if (inv_tau == 1.f) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const float e = expf(-fabsf(a[i])), r = tc::rcpf(1.f + e);
+      a[i] = a[i] >= 0.f ? r : e * r;
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+      a[i] = expf((fminf(a[i], 0.f) - 0.69314718f * tc::lg2f(1.f + expf(-fabsf(a[i])))) * inv_tau);
   }
-  return expf(log_decay(a, gate_mode, inv_tau));
 }
 
-template <typename TQ, typename TS, int R, int MODE>
+// Sums d[0..N) over W neighbouring lanes; afterwards lane l of the group holds the sum of token tok_of_lane<N, W>(l): every
+// step halves the number of tokens a lane still carries, N + log2(W / N) - 1 shuffles instead of N log2(W).
+template <int N, int W>
+__device__ __forceinline__ float sum_tokens(float (&d)[N], int lane) {
+  int n = N;
+#pragma unroll
+  for (int off = W / 2; off > 0; off >>= 1) {
+    if (n > 1) {
+      n >>= 1;
+      const bool up = lane & off;
+#pragma unroll
+      for (int i = 0; i < N / 2; ++i)
+        if (i < n) d[i] = (up ? d[i + n] : d[i]) + __shfl_xor_sync(0xffffffffu, up ? d[i] : d[i + n], off);
+    } else {
+      d[0] += __shfl_xor_sync(0xffffffffu, d[0], off);
+    }
+  }
+  return d[0];
+}
+template <int N, int W>
+__device__ __forceinline__ int tok_of_lane(int lane) { return (lane & (W - 1)) / (W / N); }
+
+__device__ __forceinline__ void store4(float* p, float x, float y, float z, float w) { *reinterpret_cast<float4*>(p) = make_float4(x, y, z, w); }
+__device__ __forceinline__ void store4(bf16* p, float x, float y, float z, float w) {
+  *reinterpret_cast<uint2*>(p) = make_uint2(tc::pack_bf16(x, y), tc::pack_bf16(z, w));
+}
+
+// rows [row0, row0 + TBF) of a strided tensor into shared memory, 16 bytes per copy; rows from nt on are zero-filled
+__device__ __forceinline__ void copy_rows(uint32_t dst, const void* src, size_t row_stride, int row_bytes_log2, int nt, int tid,
+                                          int nthr) {
+  const int cl = row_bytes_log2 - 4;
+  for (int idx = tid; idx < (TBF << cl); idx += nthr) {
+    const int r = idx >> cl, c = idx & ((1 << cl) - 1);
+    const char* g = (const char*)src + (r < nt ? (size_t)r * row_stride : 0) + c * 16;
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst + idx * 16), "l"(g), "r"(r < nt ? 16 : 0) : "memory");
+  }
+}
+
+template <typename TQ, typename TS, int DK, int MODE>
 __global__ void __launch_bounds__(256, 2) gla_fwd_rec_kernel(const GlaArgs a, const SegArgs sgm) {
   using namespace tc;
   extern __shared__ __align__(16) float smem[];
-  const int dk = a.dk, dv = a.dv, H = a.H;
-  const int CP = dv / 2, RG = dk / R;
+  constexpr int dk = DK, RG = fwd_groups(DK), R = DK / RG;
+  // staging: P threads per channel take TPP consecutive tokens each (the first P * DK threads of the block)
+  constexpr int P = DK >= 64 ? 2 : 128 / DK, TPP = TBF / P, SUMW = DK < 32 ? DK : 32;
+  const int dv = a.dv, H = a.H;
   const int tid = threadIdx.x, nthr = blockDim.x;
-  const int P = nthr / dk, TPP = TBF / P;  // staging: P threads per channel, TPP consecutive tokens each
   float* s_k = smem;                    // [TBF][dk]  k / A  (plain batch: k)
   float* s_v = s_k + TBF * dk;          // [TBF][dv]
   float* s_al = s_v + TBF * dv;         // [TBF][dk]  alpha (plain batch only)
   float* s_pA = s_al + TBF * dk;        // [P][dk] decay of each part of the batch, [P][dk] its own z
-  float* s_ab = s_pA + 2 * nthr;        // [dk] decay of the batch
+  float* s_ab = s_pA + 2 * P * dk;      // [dk] decay of the batch
   float* s_q = s_ab + dk;               // [TBF][dk]  q A  (plain batch: q)
-  float* s_den = s_q + TBF * dk;        // [TBF][4] partial q.z
-  float* s_part = s_den + TBF * 4;      // [TBF][RG][dv]
+  float* s_den = s_q + (MODE == 0 ? TBF * dk : 0);   // [TBF][4] partial q.z
+  float* s_inv = s_den + (MODE == 0 ? TBF * 4 : 0);  // [TBF] 1 / denominator
+  float* s_o = s_inv + (MODE == 0 ? TBF : 0);        // [TBF][dv] numerators
+  // raw rows of the next batch, copied while the current one is computed
+  TQ* r_k = (TQ*)(s_o + (MODE == 0 ? TBF * dv : 0));
+  TS* r_v = (TS*)(r_k + TBF * dk);
+  TS* r_g = r_v + TBF * dv;
+  TQ* r_q = (TQ*)(r_g + TBF * dk);
+  const int ldv = 31 - __clz(dv);  // (a power of two)
+  constexpr int ldk = DK == 128 ? 7 : DK == 64 ? 6 : DK == 32 ? 5 : 4;
   const int nseg_run = MODE == 1 ? sgm.nseg - 1 : sgm.nseg;
   const int bh = blockIdx.x / nseg_run, seg = blockIdx.x % nseg_run;
   const int b = bh / H, h = bh % H, j = h / (H / a.Hkv);
   const int t_begin = seg * sgm.seg_len, t_end = min(a.T, t_begin + sgm.seg_len);
-  const int cp = tid % CP, rg = tid / CP;
-  const bool active = rg < RG;
-  const int row0 = rg * R, c0 = 2 * cp;
+  // (whole warps take part in the recurrence; lanes beyond the last column quad repeat it and store nothing)
+  const int rg = tid % RG, c0 = 4 * min(tid / RG, dv / 4 - 1);
+  const bool active = (tid & ~31) < RG * (dv / 4), own = tid / RG < dv / 4;
   const int sc = tid % dk, sp = tid / dk;  // staging: channel, part
-  const TQ* qdot = (const TQ*)a.qdot;
-  const TQ* kdot = (const TQ*)a.kdot;
-  const TS* v = (const TS*)a.v;
+  const bool stager = sp < P;              // (whole warps)
   const TS* gate = (const TS*)a.gate;
   TS* o = (TS*)a.out_o;
-
-  // start state
-  float S[R][2];
-  float z = 0.f, dtot = 1.f;
-#pragma unroll
-  for (int r = 0; r < R; ++r) S[r][0] = S[r][1] = 0.f;
-  if (MODE == 0) {
-    if (active && a.S0) {
-      const float* src = a.S0 + ((size_t)bh * dk + row0) * dv + c0;
-#pragma unroll
-      for (int r = 0; r < R; ++r) { S[r][0] = src[(size_t)r * dv]; S[r][1] = src[(size_t)r * dv + 1]; }
+  auto fetch = [&](int t0) {
+    if (t0 < t_end) {
+      const int nt = min(TBF, t_end - t0);
+      const size_t th = ((size_t)b * a.T + t0) * H + h, tv = ((size_t)b * a.T + t0) * a.Hkv + j;
+      constexpr int LQ = sizeof(TQ) == 4 ? 2 : 1, LS = sizeof(TS) == 4 ? 2 : 1;
+      copy_rows(smem_u32(r_k), (const TQ*)a.kdot + th * dk, (size_t)H * dk * sizeof(TQ), ldk + LQ, nt, tid, nthr);
+      if (MODE == 0) copy_rows(smem_u32(r_q), (const TQ*)a.qdot + th * dk, (size_t)H * dk * sizeof(TQ), ldk + LQ, nt, tid, nthr);
+      if (a.gd != 1) copy_rows(smem_u32(r_g), gate + th * dk, (size_t)H * dk * sizeof(TS), ldk + LS, nt, tid, nthr);
+      copy_rows(smem_u32(r_v), (const TS*)a.v + tv * dv, (size_t)a.Hkv * dv * sizeof(TS), ldv + LS, nt, tid, nthr);
     }
-    if (a.z0) z = a.z0[(size_t)bh * dk + sc];
-    for (int i = 0; i < seg; ++i) {
-      const size_t pi = (size_t)bh * (sgm.nseg - 1) + i;
-      if (active) {
-        const float* src = sgm.loc_S + (pi * dk + row0) * dv + c0;
-        const float* dc = sgm.dec + pi * dk + row0;
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  fetch(t_begin);
+
+  // start state: S2[i][c] = rows 2 (i % 2) + {0, 1} of the thread's row quad i / 2, column c0 + c
+  uint64_t S2[R / 2][4];
+  float z = 0.f, dtot = 1.f;
+  auto row_of = [&](int i) { return 4 * (rg + RG * (i >> 1)) + 2 * (i & 1); };
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-          const float2 l = *reinterpret_cast<const float2*>(src + (size_t)r * dv);
-          const float d = dc[r];
-          S[r][0] = fmaf(d, S[r][0], l.x);
-          S[r][1] = fmaf(d, S[r][1], l.y);
+  for (int i = 0; i < R / 2; ++i) {
+    float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
+    if (MODE == 0 && active && a.S0) {
+      const float* src = a.S0 + ((size_t)bh * dk + row_of(i)) * dv + c0;
+      lo = *reinterpret_cast<const float4*>(src);
+      hi = *reinterpret_cast<const float4*>(src + dv);
+    }
+    S2[i][0] = f2_pack(lo.x, hi.x); S2[i][1] = f2_pack(lo.y, hi.y); S2[i][2] = f2_pack(lo.z, hi.z); S2[i][3] = f2_pack(lo.w, hi.w);
+  }
+  if (MODE == 0) {
+    if (a.z0) z = a.z0[(size_t)bh * dk + sc];
+    for (int pc = 0; pc < seg; ++pc) {
+      const size_t pi = (size_t)bh * (sgm.nseg - 1) + pc;
+      if (active) {
+#pragma unroll
+        for (int i = 0; i < R / 2; ++i) {
+          const float* src = sgm.loc_S + (pi * dk + row_of(i)) * dv + c0;
+          const float4 lo = *reinterpret_cast<const float4*>(src), hi = *reinterpret_cast<const float4*>(src + dv);
+          const uint64_t d = *reinterpret_cast<const uint64_t*>(sgm.dec + pi * dk + row_of(i));
+          S2[i][0] = f2_fma(d, S2[i][0], f2_pack(lo.x, hi.x)); S2[i][1] = f2_fma(d, S2[i][1], f2_pack(lo.y, hi.y));
+          S2[i][2] = f2_fma(d, S2[i][2], f2_pack(lo.z, hi.z)); S2[i][3] = f2_fma(d, S2[i][3], f2_pack(lo.w, hi.w));
         }
       }
       z = fmaf(sgm.dec[pi * dk + sc], z, sgm.loc_z[pi * dk + sc]);
     }
   }
-  uint64_t S2[R / 2][2];
-#pragma unroll
-  for (int r = 0; r < R / 2; ++r) {
-    S2[r][0] = f2_pack(S[2 * r][0], S[2 * r + 1][0]);
-    S2[r][1] = f2_pack(S[2 * r][1], S[2 * r + 1][1]);
-  }
 
   for (int t0 = t_begin; t0 < t_end; t0 += TBF) {
     const int nt = min(TBF, t_end - t0);
     // ---- staging: this thread's channel, tokens [sp TPP, sp TPP + TPP) of the batch (tokens past the end: no decay, k = 0)
-    float al[TPP_MAX], kk[TPP_MAX], qq[TPP_MAX];
-#pragma unroll
-    for (int i = 0; i < TPP_MAX; ++i) {
-      if (i >= TPP) break;
-      const int tok = sp * TPP + i;
-      al[i] = 1.f; kk[i] = 0.f; qq[i] = 0.f;
-      if (tok < nt) {
-        const size_t th = ((size_t)b * a.T + t0 + tok) * H + h;
-        kk[i] = ldf(kdot + th * dk + sc);
-        if (MODE == 0) qq[i] = ldf(qdot + th * dk + sc);
-        al[i] = ldf(gate + th * a.gd + (a.gd == 1 ? 0 : sc));
-      }
-    }
-    for (int i = tid; i < TBF * dv; i += nthr) {
-      const int tok = i / dv, e = i % dv;
-      s_v[i] = tok < nt ? ldf(v + (((size_t)b * a.T + t0 + tok) * a.Hkv + j) * dv + e) : 0.f;
-    }
-    float A = 1.f, zl = 0.f;
-#pragma unroll
-    for (int i = 0; i < TPP_MAX; ++i) {
-      if (i >= TPP) break;
-      al[i] = sp * TPP + i < nt ? decay_of(al[i], a.gate_mode, a.inv_tau) : 1.f;
-      A *= al[i];
-      zl = fmaf(al[i], zl, kk[i]);
-    }
-    s_pA[tid] = A;
-    s_pA[nthr + tid] = zl;
+    float al[TPP], kk[TPP], qq[TPP];
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
-    float Ain = 1.f, zin = z, Aall = 1.f;  // decay since the batch's start and z in front of this thread's first token
-    for (int p = 0; p < P; ++p) {
-      const float Ap = s_pA[p * dk + sc], zp = s_pA[nthr + p * dk + sc];
-      if (p < sp) { zin = fmaf(Ap, zin, zp); Ain *= Ap; }
-      z = fmaf(Ap, z, zp);
-      Aall *= Ap;
-    }
-    dtot *= Aall;
-    if (sp == 0) s_ab[sc] = Aall;
-    const bool plain = __syncthreads_or(Aall < A_MIN);
-    A = Ain;
+    if (stager) {
+      const TQ *rk = r_k + sp * (TPP * dk) + sc, *rq = r_q + sp * (TPP * dk) + sc;
+      const TS* rg_ = r_g + sp * (TPP * dk) + sc;
 #pragma unroll
-    for (int i = 0; i < TPP_MAX; ++i) {
-      if (i >= TPP) break;
-      const int tok = sp * TPP + i;
-      A *= al[i];
-      zin = fmaf(al[i], zin, kk[i]);
-      if (plain) {
-        s_k[tok * dk + sc] = kk[i];
-        s_al[tok * dk + sc] = al[i];
-        if (MODE == 0) s_q[tok * dk + sc] = qq[i];
+      for (int i = 0; i < TPP; ++i) {
+        kk[i] = ldf(rk + i * dk);
+        if (MODE == 0) qq[i] = ldf(rq + i * dk);
+      }
+      if (a.gd != 1) {
+#pragma unroll
+        for (int i = 0; i < TPP; ++i) al[i] = ldf(rg_ + i * dk);
       } else {
-        s_k[tok * dk + sc] = kk[i] / A;
-        if (MODE == 0) s_q[tok * dk + sc] = qq[i] * A;
+#pragma unroll
+        for (int i = 0; i < TPP; ++i)
+          al[i] = sp * TPP + i < nt ? ldf(gate + ((size_t)b * a.T + t0 + sp * TPP + i) * H + h) : 0.f;
       }
+    }
+    for (int i = 4 * tid; i < TBF * dv; i += 4 * nthr)
+      *reinterpret_cast<float4*>(s_v + i) = make_float4(ldf(r_v + i), ldf(r_v + i + 1), ldf(r_v + i + 2), ldf(r_v + i + 3));
+    float A = 1.f, zl = 0.f;
+    if (stager) {
+      decays_of<TPP>(al, a.gate_mode, a.inv_tau);
+      if (nt < TBF) {
+#pragma unroll
+        for (int i = 0; i < TPP; ++i)
+          if (sp * TPP + i >= nt) al[i] = 1.f;
+      }
+#pragma unroll
+      for (int i = 0; i < TPP; ++i) {
+        A *= al[i];
+        zl = fmaf(al[i], zl, kk[i]);
+      }
+      s_pA[tid] = A;
+      s_pA[P * dk + tid] = zl;
+    }
+    __syncthreads();
+    fetch(t0 + TBF);  // (every thread has read its raw values)
+    float Ain = 1.f, zin = z, Aall = 1.f;  // decay since the batch's start and z in front of this thread's first token
+    if (stager) {
+#pragma unroll
+      for (int p = 0; p < P; ++p) {
+        const float Ap = s_pA[p * dk + sc], zp = s_pA[P * dk + p * dk + sc];
+        if (p < sp) { zin = fmaf(Ap, zin, zp); Ain *= Ap; }
+        z = fmaf(Ap, z, zp);
+        Aall *= Ap;
+      }
+      dtot *= Aall;
+      if (sp == 0) s_ab[sc] = Aall;
+    }
+    const bool plain = __syncthreads_or(Aall < A_MIN);
+    if (stager) {
+      float* const wk = s_k + sp * (TPP * dk) + sc;
+      float* const wq = s_q + sp * (TPP * dk) + sc;
       if (MODE == 0) {
-        float d = qq[i] * zin;
-        for (int off = min(16, dk >> 1); off > 0; off >>= 1) d += __shfl_xor_sync(0xffffffffu, d, off);
-        if ((sc & 31) == 0) s_den[tok * 4 + (sc >> 5)] = d;
+        float d[TPP];
+#pragma unroll
+        for (int i = 0; i < TPP; ++i) {
+          zin = fmaf(al[i], zin, kk[i]);
+          d[i] = qq[i] * zin;
+        }
+        const float den = sum_tokens<TPP, SUMW>(d, tid & 31);
+        s_den[(sp * TPP + tok_of_lane<TPP, SUMW>(tid)) * 4 + (sc >> 5)] = den;  // (lanes of one token hold the same sum)
+      }
+      if (plain) {
+        float* const wa = s_al + sp * (TPP * dk) + sc;
+#pragma unroll
+        for (int i = 0; i < TPP; ++i) {
+          wk[i * dk] = kk[i];
+          wa[i * dk] = al[i];
+          if (MODE == 0) wq[i * dk] = qq[i];
+        }
+      } else {
+        A = Ain;
+#pragma unroll
+        for (int i = 0; i < TPP; ++i) {
+          A *= al[i];
+          wk[i * dk] = kk[i] * rcpf(A);
+          if (MODE == 0) wq[i * dk] = qq[i] * A;
+        }
       }
     }
     __syncthreads();
+    if (MODE == 0 && tid < TBF) {
+      float dn = a.eps;
+#pragma unroll
+      for (int g = 0; g < (dk + 31) / 32; ++g) dn += s_den[tid * 4 + g];
+      s_inv[tid] = a.normalize ? 1.f / dn : 1.f;
+      if (a.out_den && tid < nt) a.out_den[((size_t)b * a.T + t0 + tid) * H + h] = dn;
+    }
     // ---- the recurrence over the batch
     if (active) {
-#pragma unroll 1
-      for (int tok = 0; tok < TBF; ++tok) {
-        const float2 vv = *reinterpret_cast<const float2*>(s_v + tok * dv + c0);
-        const uint64_t v0 = f2_pack(vv.x, vv.x), v1 = f2_pack(vv.y, vv.y);
-        const ulonglong2* k4 = reinterpret_cast<const ulonglong2*>(s_k + tok * dk + row0);
-        const ulonglong2* q4 = reinterpret_cast<const ulonglong2*>(s_q + tok * dk + row0);
-        const ulonglong2* a4 = reinterpret_cast<const ulonglong2*>(s_al + tok * dk + row0);
-        uint64_t acc0 = 0ull, acc1 = 0ull;
+      auto run = [&](auto plain_c) {
+        constexpr bool PLAIN = decltype(plain_c)::value;
+#pragma unroll 2
+        for (int tok = 0; tok < TBF; ++tok) {
+          const float4 vv = *reinterpret_cast<const float4*>(s_v + tok * dv + c0);
+          const uint64_t vc[4] = {f2_pack(vv.x, vv.x), f2_pack(vv.y, vv.y), f2_pack(vv.z, vv.z), f2_pack(vv.w, vv.w)};
+          const ulonglong2* k4 = reinterpret_cast<const ulonglong2*>(s_k + tok * dk) + rg;
+          const ulonglong2* q4 = reinterpret_cast<const ulonglong2*>(s_q + tok * dk) + rg;
+          const ulonglong2* a4 = reinterpret_cast<const ulonglong2*>(s_al + tok * dk) + rg;
+          uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
 #pragma unroll
-        for (int r4 = 0; r4 < R / 4; ++r4) {
-          const ulonglong2 k2 = k4[r4];
-          if (plain) {
-            const ulonglong2 al2 = a4[r4];
-            S2[2 * r4][0] = f2_fma(al2.x, S2[2 * r4][0], f2_mul(k2.x, v0));
-            S2[2 * r4][1] = f2_fma(al2.x, S2[2 * r4][1], f2_mul(k2.x, v1));
-            S2[2 * r4 + 1][0] = f2_fma(al2.y, S2[2 * r4 + 1][0], f2_mul(k2.y, v0));
-            S2[2 * r4 + 1][1] = f2_fma(al2.y, S2[2 * r4 + 1][1], f2_mul(k2.y, v1));
-          } else {
-            S2[2 * r4][0] = f2_fma(k2.x, v0, S2[2 * r4][0]);
-            S2[2 * r4][1] = f2_fma(k2.x, v1, S2[2 * r4][1]);
-            S2[2 * r4 + 1][0] = f2_fma(k2.y, v0, S2[2 * r4 + 1][0]);
-            S2[2 * r4 + 1][1] = f2_fma(k2.y, v1, S2[2 * r4 + 1][1]);
+          for (int i = 0; i < R / 4; ++i) {
+            const ulonglong2 k2 = k4[RG * i];
+            ulonglong2 al2, q2;
+            if (PLAIN) al2 = a4[RG * i];
+            if (MODE == 0) q2 = q4[RG * i];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+              uint64_t &sx = S2[2 * i][c], &sy = S2[2 * i + 1][c];
+              sx = PLAIN ? f2_fma(al2.x, sx, f2_mul(k2.x, vc[c])) : f2_fma(k2.x, vc[c], sx);
+              sy = PLAIN ? f2_fma(al2.y, sy, f2_mul(k2.y, vc[c])) : f2_fma(k2.y, vc[c], sy);
+              if (MODE == 0) acc[c] = f2_fma(q2.y, sy, f2_fma(q2.x, sx, acc[c]));
+            }
           }
           if (MODE == 0) {
-            const ulonglong2 q2 = q4[r4];
-            acc0 = f2_fma(q2.x, S2[2 * r4][0], acc0);
-            acc1 = f2_fma(q2.x, S2[2 * r4][1], acc1);
-            acc0 = f2_fma(q2.y, S2[2 * r4 + 1][0], acc0);
-            acc1 = f2_fma(q2.y, S2[2 * r4 + 1][1], acc1);
+            // sum over the RG row groups (neighbouring lanes), a lane keeping ever fewer columns: 2, then 1
+            float x[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+              float lo, hi;
+              f2_unpack(acc[c], lo, hi);
+              x[c] = lo + hi;
+            }
+            const bool b0 = rg & 1, b1 = rg & 2;
+            float y0 = (b0 ? x[2] : x[0]) + __shfl_xor_sync(0xffffffffu, b0 ? x[0] : x[2], 1);
+            float y1 = (b0 ? x[3] : x[1]) + __shfl_xor_sync(0xffffffffu, b0 ? x[1] : x[3], 1);
+            float* const dst = s_o + tok * dv + c0 + (b0 ? 2 : 0);
+            if (RG == 2) {
+              if (own) *reinterpret_cast<float2*>(dst) = make_float2(y0, y1);
+            } else {
+              float w = (b1 ? y1 : y0) + __shfl_xor_sync(0xffffffffu, b1 ? y0 : y1, 2);
+              if (RG == 8) w += __shfl_xor_sync(0xffffffffu, w, 4);
+              if (own && rg < 4) dst[b1 ? 1 : 0] = w;
+            }
           }
         }
-        if (MODE == 0) {
-          float x0, y0, x1, y1;
-          f2_unpack(acc0, x0, y0);
-          f2_unpack(acc1, x1, y1);
-          *reinterpret_cast<float2*>(s_part + (tok * RG + rg) * dv + c0) = make_float2(x0 + y0, x1 + y1);
-        }
-      }
+      };
+      if (plain) run(std::true_type{});
+      else run(std::false_type{});
       if (!plain) {  // back to the state itself
-        const ulonglong2* d4 = reinterpret_cast<const ulonglong2*>(s_ab + row0);
+        const ulonglong2* d4 = reinterpret_cast<const ulonglong2*>(s_ab) + rg;
 #pragma unroll
-        for (int r4 = 0; r4 < R / 4; ++r4) {
-          const ulonglong2 d2 = d4[r4];
-          S2[2 * r4][0] = f2_mul(d2.x, S2[2 * r4][0]);
-          S2[2 * r4][1] = f2_mul(d2.x, S2[2 * r4][1]);
-          S2[2 * r4 + 1][0] = f2_mul(d2.y, S2[2 * r4 + 1][0]);
-          S2[2 * r4 + 1][1] = f2_mul(d2.y, S2[2 * r4 + 1][1]);
+        for (int i = 0; i < R / 4; ++i) {
+          const ulonglong2 d2 = d4[RG * i];
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            S2[2 * i][c] = f2_mul(d2.x, S2[2 * i][c]);
+            S2[2 * i + 1][c] = f2_mul(d2.y, S2[2 * i + 1][c]);
+          }
         }
       }
     }
     __syncthreads();
     if (MODE == 0) {
-      for (int i = tid; i < nt * dv; i += nthr) {
-        const int tok = i / dv, e = i % dv;
-        float num = 0.f, dn = a.eps;
-        for (int g = 0; g < RG; ++g) num += s_part[(tok * RG + g) * dv + e];
-        for (int g = 0; g < (dk + 31) / 32; ++g) dn += s_den[tok * 4 + g];
-        const size_t th = ((size_t)b * a.T + t0 + tok) * H + h;
-        stf(o + th * dv + e, a.normalize ? num / dn : num);
-        if (e == 0 && a.out_den) a.out_den[th] = dn;
+      TS* const ob = o + (((size_t)b * a.T + t0) * H + h) * dv;
+      for (int i = 4 * tid; i < nt * dv; i += 4 * nthr) {
+        const int tok = i >> ldv, e = i & (dv - 1);
+        const float4 x = *reinterpret_cast<const float4*>(s_o + i);
+        const float inv = s_inv[tok];
+        store4(ob + (size_t)tok * H * dv + e, x.x * inv, x.y * inv, x.z * inv, x.w * inv);
       }
-      // (the next batch writes s_den and s_part behind barriers of its own; s_v is read by nobody here)
+      // (the next batch writes s_den and s_o behind barriers of its own; s_v is read by nobody here)
     }
-  }
-#pragma unroll
-  for (int r = 0; r < R / 2; ++r) {
-    f2_unpack(S2[r][0], S[2 * r][0], S[2 * r + 1][0]);
-    f2_unpack(S2[r][1], S[2 * r][1], S[2 * r + 1][1]);
   }
   float* const dS = MODE == 1 ? sgm.loc_S + (size_t)blockIdx.x * dk * dv
                               : (a.S_T && seg == sgm.nseg - 1) ? a.S_T + (size_t)bh * dk * dv : nullptr;
   float* const dz = MODE == 1 ? sgm.loc_z + (size_t)blockIdx.x * dk
                               : (a.z_T && seg == sgm.nseg - 1) ? a.z_T + (size_t)bh * dk : nullptr;
-  if (dS && active) {
+  if (dS && own) {
 #pragma unroll
-    for (int r = 0; r < R; ++r)
-      *reinterpret_cast<float2*>(dS + (size_t)(row0 + r) * dv + c0) = make_float2(S[r][0], S[r][1]);
+    for (int i = 0; i < R / 2; ++i) {
+      float4 lo, hi;
+      f2_unpack(S2[i][0], lo.x, hi.x); f2_unpack(S2[i][1], lo.y, hi.y); f2_unpack(S2[i][2], lo.z, hi.z); f2_unpack(S2[i][3], lo.w, hi.w);
+      float* dst = dS + (size_t)row_of(i) * dv + c0;
+      *reinterpret_cast<float4*>(dst) = lo;
+      *reinterpret_cast<float4*>(dst + dv) = hi;
+    }
   }
-  if (sp == 0) {
+  if (sp == 0) {  // (dk <= 128 <= threads)
     if (dz) dz[sc] = z;
     if (MODE == 1) sgm.dec[(size_t)blockIdx.x * dk + sc] = dtot;
   }
 }
 
-// threads of the forward kernel: RG row groups x dv / 2 column pairs, at least 128, and at least two per channel at dk = 128
-static int fwd_rows(int dk) { return dk >= 64 ? dk / 4 : 16; }
+// threads of the forward kernel: RG row groups x dv / 4 column quads, and at least the P * d_k staging threads
 static int fwd_threads(const lawcat_params& p) {
-  const int n = (p.d_k / fwd_rows(p.d_k)) * (p.d_v / 2), lo = p.d_k == 128 ? 256 : 128;
+  const int n = fwd_groups(p.d_k) * (p.d_v / 4), lo = p.d_k == 128 ? 256 : 128;
   return n < lo ? lo : n;
 }
 
@@ -318,16 +429,22 @@ static int gla_fwd_launch(const Ctx& c, GlaArgs& a, void* ws, size_t ws_bytes) {
     s.nseg = 1;
     s.seg_len = (p.T + TBF - 1) / TBF * TBF;
   }
-  const int BH = p.B * p.H, R = fwd_rows(p.d_k), RG = p.d_k / R, thr = fwd_threads(p);
+  const int BH = p.B * p.H, thr = fwd_threads(p);
   const size_t pieces = (size_t)BH * (s.nseg - 1);
   s.loc_S = (float*)ws;
   s.loc_z = s.loc_S + pieces * p.d_k * p.d_v;
   s.dec = s.loc_z + pieces * p.d_k;
-  const size_t smem1 = sizeof(float) * ((size_t)TBF * (2 * p.d_k + p.d_v) + 2 * thr + p.d_k);
-  const size_t smem0 = smem1 + sizeof(float) * ((size_t)TBF * p.d_k + 4 * TBF + (size_t)TBF * RG * p.d_v);
-  auto* const k_state = R == 32 ? gla_fwd_rec_kernel<TQ, TS, 32, 1> : gla_fwd_rec_kernel<TQ, TS, 16, 1>;
-  auto* const k_full = R == 32 ? gla_fwd_rec_kernel<TQ, TS, 32, 0> : gla_fwd_rec_kernel<TQ, TS, 16, 0>;
-  if (cudaFuncSetAttribute(k_full, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem0) != cudaSuccess) return LAWCAT_ERR_CUDA;
+  const size_t raw = (size_t)TBF * (p.d_k * sizeof(TQ) + (p.d_k + p.d_v) * sizeof(TS));
+  const size_t smem1 = raw + sizeof(float) * ((size_t)TBF * (2 * p.d_k + p.d_v) + 2 * (p.d_k == 128 ? 256 : 128) + p.d_k);
+  const size_t smem0 = smem1 + (size_t)TBF * p.d_k * sizeof(TQ) + sizeof(float) * ((size_t)TBF * (p.d_k + p.d_v) + 5 * TBF);
+  auto* k_state = gla_fwd_rec_kernel<TQ, TS, 128, 1>;
+  auto* k_full = gla_fwd_rec_kernel<TQ, TS, 128, 0>;
+  if (p.d_k == 64) { k_state = gla_fwd_rec_kernel<TQ, TS, 64, 1>; k_full = gla_fwd_rec_kernel<TQ, TS, 64, 0>; }
+  if (p.d_k == 32) { k_state = gla_fwd_rec_kernel<TQ, TS, 32, 1>; k_full = gla_fwd_rec_kernel<TQ, TS, 32, 0>; }
+  if (p.d_k == 16) { k_state = gla_fwd_rec_kernel<TQ, TS, 16, 1>; k_full = gla_fwd_rec_kernel<TQ, TS, 16, 0>; }
+  if (cudaFuncSetAttribute(k_full, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem0) != cudaSuccess ||
+      cudaFuncSetAttribute(k_state, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1) != cudaSuccess)
+    return LAWCAT_ERR_CUDA;
   if (s.nseg > 1) {
     LaunchScope _ls("gla_fwd_rec_state", c.stream);
     k_state<<<(unsigned)pieces, thr, smem1, c.stream>>>(a, s);
