@@ -2,9 +2,9 @@
 // through them (distillation step, Section 5.1), bf16 storage.
 //
 // Forward: one thread block = one (batch, query head, tile of 128 tokens), both streams one after the other (they share
-// W_h): raw rows (with the conv_k - 1 rows in front) into shared memory, depthwise causal conv in fp32 -> fp16 operand,
-// Y = u W_h as one tcgen05 product per 16 channels (fp32 accumulator in tensor memory), phi (softmax over the row, or the
-// elementwise 1 + ELU / identity of Section 2) by the thread that owns the row's TMEM lane, 16-bit or fp32 store.
+// W_h): depthwise causal conv in fp32 -> operand, Y = u W_h by tcgen05 (fp32 accumulator in tensor memory), phi (softmax over
+// the row, or the elementwise 1 + ELU / identity of Section 2) by the threads that own the row's TMEM lane, 16-bit or fp32
+// store.
 // Backward (head width 64): one block = one (batch, key head, tile); for each query head of
 // the group and each stream it recomputes u and p = softmax(u W_h), applies the softmax Jacobian dy = p (dp - p . dp),
 // and forms du = dy W_h^T (the key stream summed over the group in registers) and dW_h += u^T dy (accumulators of two
@@ -98,19 +98,70 @@ __device__ __forceinline__ void conv_tile(const uint8_t* s_raw, const float* s_w
   }
 }
 
+// conv of 8 channels (octet o) of N consecutive tokens from t on, straight from global memory with a window of raw rows
+// (rows before the sequence come from the conv cache or are zero, rows past its end are zero); emit(i, u) takes token t + i.
+// s_w: the head's taps, fp32 [D][4], in shared memory.
+template <int D, int N, typename F>
+__device__ __forceinline__ void conv_run(const bf16* x, const bf16* cache, const float* s_w, int b, int t, int T, int NH,
+                                         int head, int K, int o, F emit) {
+  uint4 raw[N + HALO];
+#pragma unroll
+  for (int i = 0; i < N + HALO; ++i) {
+    const int tt = t - HALO + i;
+    raw[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (tt >= 0 && tt < T)
+      raw[i] = *reinterpret_cast<const uint4*>(x + (((size_t)b * T + tt) * NH + head) * D + o * 8);
+    else if (tt < 0 && cache != nullptr && tt + (K - 1) >= 0)
+      raw[i] = *reinterpret_cast<const uint4*>(cache + (((size_t)b * (K - 1) + tt + (K - 1)) * NH + head) * D + o * 8);
+  }
+  float w[8][4];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const float4 t4 = *reinterpret_cast<const float4*>(s_w + (o * 8 + i) * 4);
+    w[i][0] = t4.x; w[i][1] = t4.y; w[i][2] = t4.z; w[i][3] = t4.w;
+  }
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    float u[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int dl = 0; dl < 4; ++dl) {
+      float xv[8];
+      unpack8b(raw[i + HALO - dl], xv);
+#pragma unroll
+      for (int c = 0; c < 8; ++c) u[c] = fmaf(w[c][dl], xv[c], u[c]);
+    }
+    emit(i, u);
+  }
+}
+
+// v rounded to bf16, and v -= the rounded value
+__device__ __forceinline__ uint4 take_bf16(float* v) {
+  const uint4 p = pack8bf16(v);
+  float h[8];
+  unpack8b(p, h);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] -= h[i];
+  return p;
+}
+
+// Forward. 256 threads walk one (batch, query head, tile of 128 tokens), query stream then key stream. bf16 outputs take
+// the conv output as one fp16 operand. fp32 outputs (features that a fused caller keeps in fp32, and those of the exact
+// recurrence) take it as three bf16 terms, u = b1 + b2 + b3 exactly, with W_h exact in bf16: the products are those of
+// fp32 numbers over the full fp32 range, summed in fp32.
+// Bound by HBM writes (fp32 features) and by the dependent phases of a tile: raw rows go from global memory through the
+// conv straight into the operand (no staging tile), and the outputs leave through the drained operand tile as whole rows.
 template <int D, typename TO>
-__global__ void __launch_bounds__(128) convmix_tc_fwd_kernel(const CArgs a) {
+__global__ void __launch_bounds__(256) convmix_tc_fwd_kernel(const CArgs a) {
   using L = Lay<D>;
   extern __shared__ __align__(128) uint8_t sg[];
-  // fp32 outputs (the features a fused caller keeps in fp32) take the conv output as a two-term fp16 pair: about 21 bits
-  // instead of 11, so that the features carry no visible rounding into the gradients computed from them
-  constexpr bool TWO = sizeof(TO) == 4;
-  constexpr uint32_t OFF_WT = 0, OFF_U = OFF_WT + L::TILE_W, OFF_UL = OFF_U + L::TILE_U;
-  constexpr uint32_t OFF_RAW = OFF_UL + (TWO ? L::TILE_U : 0) + 2048 /* rows past the tile */;
-  constexpr uint32_t OFF_TAPS = OFF_RAW + (L::RAW_BYTES + 15) / 16 * 16, OFF_BAR = OFF_TAPS + D * 4 * 4;
+  constexpr int NT = sizeof(TO) == 4 ? 3 : 1, FMT = NT == 3 ? FMT_BF16 : FMT_F16;
+  constexpr uint32_t OFF_WT = 0, OFF_U = OFF_WT + L::TILE_W;
+  constexpr uint32_t OFF_TAPS = OFF_U + NT * L::TILE_U, OFF_RED = OFF_TAPS + D * 16, OFF_BAR = OFF_RED + 4 * TT * 4;
   const uint32_t sb = smem_u32(sg);
-  const int tid = threadIdx.x, warp = tid >> 5;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   volatile int* const s_flags = reinterpret_cast<volatile int*>(sg + OFF_BAR + 16);  // [0] tmem base, [1] abort
+  float* const s_taps = reinterpret_cast<float*>(sg + OFF_TAPS);
+  float* const s_red = reinterpret_cast<float*>(sg + OFF_RED);  // [max, sum][2 halves][128 rows]
   const int t0 = blockIdx.x * TT, bh = blockIdx.y, h = bh % a.H, b = bh / a.H;
   const int G = a.H / a.Hkv, j = h / G;
   if (tid == 0) {
@@ -122,100 +173,132 @@ __global__ void __launch_bounds__(128) convmix_tc_fwd_kernel(const CArgs a) {
     tmem_alloc(sb + OFF_BAR + 16, D);
     tmem_relinquish();
   }
-  load_w_tile<D>(sg + OFF_WT, a.W + (size_t)h * D * D, tid, 128);
-  tc_fence_before_sync();
-  __syncthreads();
-  tc_fence_after_sync();
-  const uint32_t tmem = (uint32_t)s_flags[0];
-  const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16);
+  auto load_w = [&](const bf16* Wh) {
+    if (NT == 1) {
+      load_w_tile<D>(sg + OFF_WT, Wh, tid, 256);
+    } else {
+      for (int idx = tid; idx < D * L::OPR; idx += 256) {
+        const int c = idx / L::OPR, o = idx % L::OPR;
+        *reinterpret_cast<uint4*>(sg + OFF_WT + toff(L::SLAB_W, c, o * 8)) = *reinterpret_cast<const uint4*>(Wh + (size_t)c * D + o * 8);
+      }
+    }
+  };
+  load_w(a.W + (size_t)h * D * D);
+  const int row = (warp & 3) * 32 + lane, half = warp >> 2;  // epilogue: row of the tile, half of its columns
+  constexpr int HC = D / 2;
+  uint32_t lane_base = 0, tmem = 0;
   Waiter wt{sb + OFF_BAR, 0u, s_flags + 1, a.dev_status};
 #pragma unroll 1
   for (int stream = 0; stream < 2; ++stream) {
     const bf16* x = stream ? a.k : a.q;
+    const bf16* w = stream ? a.w_k : a.w_q;
+    const bf16* cache = stream ? a.cache_k : a.cache_q;
     const int NH = stream ? a.Hkv : a.H, head = stream ? j : h;
-    // (a separate linear layer per stream: the key stream's W_h replaces the tile; the product that read the query
-    // stream's has completed, and the barriers below publish the new tile together with the conv output)
-    if (stream == 1 && a.unshared) load_w_tile<D>(sg + OFF_WT, a.W + ((size_t)a.H + h) * D * D, tid, 128);
-    load_raw_and_taps<D>(sg + OFF_RAW, reinterpret_cast<float*>(sg + OFF_TAPS), x, stream ? a.w_k : a.w_q,
-                         stream ? a.cache_k : a.cache_q, b, t0, a.T, NH, head, a.K, tid, 128);
-    if (stream == 0 && t0 + tid < a.T) {  // the key stream's raw row of this thread, towards L2 meanwhile
+    // (a separate linear layer per stream: the product that read the query stream's W_h has completed)
+    if (stream == 1 && a.unshared) load_w(a.W + ((size_t)a.H + h) * D * D);
+    for (int idx = tid; idx < D * 4; idx += 256) {
+      const int c = idx >> 2, dl = idx & 3;
+      s_taps[idx] = dl < a.K ? __bfloat162float(w[((size_t)head * D + c) * a.K + dl]) : 0.f;
+    }
+    if (stream == 0 && tid < TT && t0 + tid < a.T) {  // the key stream's raw row of this thread, towards L2 meanwhile
       const bf16* kr = a.k + (((size_t)b * a.T + t0 + tid) * a.Hkv + j) * D;
       prefetch_l2(kr);
       if (D * 2 > 128) prefetch_l2(kr + 64);
     }
+    tc_fence_before_sync();
     __syncthreads();
-    conv_tile<D>(sg + OFF_RAW, reinterpret_cast<const float*>(sg + OFF_TAPS), sg + OFF_U, tid, 128,
-                 TWO ? sg + OFF_UL : nullptr);
+    tc_fence_after_sync();
+    {
+      constexpr int RPT = TT * L::OPR / 256, STEP = 4;  // rows per thread, rows per run
+      const int o = tid % L::OPR, r0 = tid / L::OPR * RPT;
+#pragma unroll 1
+      for (int rr = 0; rr < RPT; rr += STEP)
+        conv_run<D, STEP>(x, cache, s_taps, b, t0 + r0 + rr, a.T, NH, head, a.K, o, [&](int i, float* u) {
+          uint8_t* dst = sg + OFF_U + toff(L::SLAB_U, r0 + rr + i, o * 8);
+          if (NT == 1) {
+            *reinterpret_cast<uint4*>(dst) = pack8f16(u);
+          } else {
+            *reinterpret_cast<uint4*>(dst) = take_bf16(u);
+            *reinterpret_cast<uint4*>(dst + L::TILE_U) = take_bf16(u);
+            *reinterpret_cast<uint4*>(dst + 2 * L::TILE_U) = pack8bf16(u);
+          }
+        });
+    }
     fence_proxy_async();
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
+    tmem = (uint32_t)s_flags[0];
+    lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16) + half * HC;
     if (tid == 0) {
-      const uint32_t idesc = instr_desc(128, D, FMT_F16, MAJOR_K, MAJOR_MN);
-      const uint64_t da = kview(sb + OFF_U, L::SLAB_U), db = mview(sb + OFF_WT, L::SLAB_W);
-      for (int kk = 0; kk < D / 16; ++kk) mma_f16(tmem, dadv(da, 2 * L::SLAB_U * kk), dadv(db, 256 * kk), idesc, kk > 0);
-      if (TWO) {
-        const uint64_t dl = kview(sb + OFF_UL, L::SLAB_U);
-        for (int kk = 0; kk < D / 16; ++kk) mma_f16(tmem, dadv(dl, 2 * L::SLAB_U * kk), dadv(db, 256 * kk), idesc, 1);
+      const uint32_t idesc = instr_desc(128, D, FMT, MAJOR_K, MAJOR_MN);
+      const uint64_t db = mview(sb + OFF_WT, L::SLAB_W);
+      for (int term = NT - 1; term >= 0; --term) {  // (smallest terms first)
+        const uint64_t da = kview(sb + OFF_U + term * L::TILE_U, L::SLAB_U);
+        for (int kk = 0; kk < D / 16; ++kk)
+          mma_f16(tmem, dadv(da, 2 * L::SLAB_U * kk), dadv(db, 256 * kk), idesc, term < NT - 1 || kk > 0);
       }
       mma_commit(sb + OFF_BAR);
     }
     wt.wait();
-    // phi over the row this thread owns (row = token t0 + tid): softmax, or elementwise 1 + ELU / identity
-    if (a.phi != LAWCAT_PHI_SOFTMAX) {
-      const int t = t0 + tid;
-      float y[32];
-      TO* out = reinterpret_cast<TO*>(stream ? a.kdot : a.qdot) + (((size_t)b * a.T + t) * a.H + h) * D;
-#pragma unroll 1
-      for (int c0 = 0; c0 < D; c0 += 32) {
-        tmem_ld32(lane_base + c0, y);
-        tmem_wait_ld();
-        if (a.phi == LAWCAT_PHI_ELU1) {
+    // phi over the row: softmax (the two threads of a row exchange max and sum), or elementwise 1 + ELU / identity
+    float y[HC];
 #pragma unroll
-          for (int i = 0; i < 32; ++i) y[i] = y[i] > 0.f ? y[i] + 1.f : __expf(y[i]);
-        }
-        if (t < a.T) {
+    for (int c0 = 0; c0 < HC; c0 += 32) tmem_ld32(lane_base + c0, y + c0);
+    tmem_wait_ld();
+    if (a.phi == LAWCAT_PHI_SOFTMAX) {
+      float m = -INFINITY, sum = 0.f;
 #pragma unroll
-          for (int i = 0; i < 32; i += 8) store_row8(out + c0 + i, y + i);
-        }
+      for (int i = 0; i < HC; ++i) m = fmaxf(m, y[i]);
+      s_red[half * TT + row] = m;
+      __syncthreads();
+      m = fmaxf(m, s_red[(half ^ 1) * TT + row]);
+      if (NT == 3) {
+#pragma unroll
+        for (int i = 0; i < HC; ++i) { y[i] = expf(y[i] - m); sum += y[i]; }
+      } else {
+        const float mb = m * 1.4426950408889634f;
+#pragma unroll
+        for (int i = 0; i < HC; ++i) { y[i] = ex2f(fmaf(y[i], 1.4426950408889634f, -mb)); sum += y[i]; }
       }
-    } else {
-      const int t = t0 + tid;
-      float y[32], m = -INFINITY, sum = 0.f;
-#pragma unroll 1
-      for (int c0 = 0; c0 < D; c0 += 32) {
-        tmem_ld32(lane_base + c0, y);
-        tmem_wait_ld();
+      s_red[(2 + half) * TT + row] = sum;
+      __syncthreads();
+      const float inv = 1.f / (sum + s_red[(2 + (half ^ 1)) * TT + row]);
 #pragma unroll
-        for (int i = 0; i < 32; ++i) m = fmaxf(m, y[i]);
-      }
-      const float mb = m * 1.4426950408889634f;
-#pragma unroll 1
-      for (int c0 = 0; c0 < D; c0 += 32) {
-        tmem_ld32(lane_base + c0, y);
-        tmem_wait_ld();
+      for (int i = 0; i < HC; ++i) y[i] *= inv;
+    } else if (a.phi == LAWCAT_PHI_ELU1) {
 #pragma unroll
-        for (int i = 0; i < 32; ++i) sum += ex2f(fmaf(y[i], 1.4426950408889634f, -mb));
-      }
-      const float inv = 1.f / sum;
-      TO* out = reinterpret_cast<TO*>(stream ? a.kdot : a.qdot) + (((size_t)b * a.T + t) * a.H + h) * D;
-#pragma unroll 1
-      for (int c0 = 0; c0 < D; c0 += 32) {
-        tmem_ld32(lane_base + c0, y);
-        tmem_wait_ld();
+      for (int i = 0; i < HC; ++i) y[i] = y[i] > 0.f ? y[i] + 1.f : (NT == 3 ? expf(y[i]) : __expf(y[i]));
+    }
+    // out through the drained operand tile: rows of 16-byte pieces, XOR-swizzled, then whole rows to global memory
+    constexpr int EPP = 16 / sizeof(TO), PPR = D / EPP;  // elements per piece, pieces per row
 #pragma unroll
-        for (int i = 0; i < 32; ++i) y[i] = ex2f(fmaf(y[i], 1.4426950408889634f, -mb)) * inv;
-        if (t < a.T) {
-#pragma unroll
-          for (int i = 0; i < 32; i += 8) store_row8(out + c0 + i, y + i);
-        }
-      }
+    for (int i = 0; i < HC; i += EPP) {
+      const int pc = (half * HC + i) / EPP;
+      uint4 v;
+      if (NT == 3) v = make_uint4(__float_as_uint(y[i]), __float_as_uint(y[i + 1]), __float_as_uint(y[i + 2]), __float_as_uint(y[i + 3]));
+      else v = pack8bf16(y + i);
+      *reinterpret_cast<uint4*>(sg + OFF_U + (row * PPR + (pc ^ (row & 7))) * 16) = v;
     }
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
+    TO* out = reinterpret_cast<TO*>(stream ? a.kdot : a.qdot);
+#pragma unroll 4
+    for (int idx = tid; idx < TT * PPR; idx += 256) {
+      const int r = idx / PPR, pc = idx % PPR;
+      if (t0 + r < a.T)
+        *reinterpret_cast<uint4*>(out + (((size_t)b * a.T + t0 + r) * a.H + h) * D + pc * EPP) =
+            *reinterpret_cast<const uint4*>(sg + OFF_U + (r * PPR + (pc ^ (r & 7))) * 16);
+    }
+    // (the barrier in front of the next stream's conv keeps its writes behind these reads)
   }
-  if (warp == 0) tmem_dealloc(tmem, D);
+  tc_fence_before_sync();
+  __syncthreads();
+  if (warp == 0) {
+    tc_fence_after_sync();
+    tmem_dealloc(tmem, D);
+  }
 }
 
 // Backward through phi and the mix for head width 64: du_q [B,T,H,64], du_k [B,T,Hkv,64] (fp32), dW [H,64,64] (atomic adds
@@ -418,7 +501,7 @@ __global__ void __launch_bounds__(128, 2) convmix_tc_bwd_kernel(const CArgs a) {
 template <int D, typename TO>
 constexpr uint32_t fwd_smem() {
   using L = Lay<D>;
-  return L::TILE_W + (sizeof(TO) == 4 ? 2 : 1) * L::TILE_U + 2048 + (L::RAW_BYTES + 15) / 16 * 16 + D * 16 + 64;
+  return L::TILE_W + (sizeof(TO) == 4 ? 3 : 1) * L::TILE_U + D * 16 + 4 * TT * 4 + 64;
 }
 constexpr uint32_t bwd_smem() {
   using L = Lay<64>;
@@ -474,11 +557,11 @@ int launch_convmix_tc_fwd(const Ctx& c, const void* q, const void* k, const void
   const dim3 grid((unsigned)((p.T + TT - 1) / TT), (unsigned)(p.B * p.H));
   LaunchScope _ls("convmix_tc_fwd", c.stream);
   if (p.d_k == 64) {
-    if (out_f32) convmix_tc_fwd_kernel<64, float><<<grid, 128, fwd_smem<64, float>(), c.stream>>>(a);
-    else convmix_tc_fwd_kernel<64, bf16><<<grid, 128, fwd_smem<64, bf16>(), c.stream>>>(a);
+    if (out_f32) convmix_tc_fwd_kernel<64, float><<<grid, 256, fwd_smem<64, float>(), c.stream>>>(a);
+    else convmix_tc_fwd_kernel<64, bf16><<<grid, 256, fwd_smem<64, bf16>(), c.stream>>>(a);
   } else {
-    if (out_f32) convmix_tc_fwd_kernel<128, float><<<grid, 128, fwd_smem<128, float>(), c.stream>>>(a);
-    else convmix_tc_fwd_kernel<128, bf16><<<grid, 128, fwd_smem<128, bf16>(), c.stream>>>(a);
+    if (out_f32) convmix_tc_fwd_kernel<128, float><<<grid, 256, fwd_smem<128, float>(), c.stream>>>(a);
+    else convmix_tc_fwd_kernel<128, bf16><<<grid, 256, fwd_smem<128, bf16>(), c.stream>>>(a);
   }
   LAWCAT_CHECK_LAUNCH();
   return LAWCAT_OK;
