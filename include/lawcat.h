@@ -242,8 +242,9 @@ int lawcat_layer_fwd(const lawcat_params* p, const void* q, const void* k, const
  *     boundary; a chunk of a longer sequence passes the state and caches its previous chunk returned)
  *   S_T, z_T, cache_q_out, cache_k_out: the same per sequence after its last token (nullable)
  * No token of one sequence reaches another: neither through the conv (its first conv_k - 1 tokens see the sequence's own
- * cache or zeros) nor through the state. An empty sequence hands its state and caches through. The sequences are
- * enqueued one after the other on `stream`, sharing `ws` (lawcat_layer_fwd_varlen_workspace_bytes: the largest need).
+ * cache or zeros) nor through the state. An empty sequence hands its state and caches through. The sequences that the
+ * chunkwise tensor-core kernel serves (see lawcat_layer_fwd) run together, up to 64 per launch; the others are enqueued one
+ * after the other. All share `ws` (lawcat_layer_fwd_varlen_workspace_bytes: the largest need).
  */
 size_t lawcat_layer_fwd_varlen_workspace_bytes(const lawcat_params* p, const int32_t* cu_seqlens, int nseq);
 int lawcat_layer_fwd_varlen(const lawcat_params* p, const int32_t* cu_seqlens, int nseq, const void* q, const void* k,

@@ -275,12 +275,12 @@ int lawcat_layer_fwd(const lawcat_params* p, const void* q, const void* k, const
 
 size_t lawcat_layer_fwd_varlen_workspace_bytes(const lawcat_params* p, const int32_t* cu_seqlens, int nseq) {
   if (check_params(p, true) != LAWCAT_OK || !cu_seqlens || nseq < 0) return 0;
-  size_t need = 0;
+  size_t need = layer_tc_packed_workspace_bytes(*p, cu_seqlens, nseq);
   for (int i = 0; i < nseq; ++i) {
     lawcat_params pi = *p;
     pi.B = 1;
     pi.T = cu_seqlens[i + 1] - cu_seqlens[i];
-    if (pi.T <= 0) continue;
+    if (pi.T <= 0 || layer_tc_supported(pi)) continue;
     const size_t n = lawcat_workspace_bytes(&pi, LAWCAT_OP_LAYER_FWD);
     if (n > need) need = n;
   }
@@ -305,10 +305,20 @@ int lawcat_layer_fwd_varlen(const lawcat_params* p, const int32_t* cu_seqlens, i
   auto at = [](const void* base, size_t bytes) -> const void* { return base ? (const char*)base + bytes : nullptr; };
   auto atw = [](void* base, size_t bytes) -> void* { return base ? (char*)base + bytes : nullptr; };
   cudaStream_t st = (cudaStream_t)stream;
+  const void* const req[] = {q, k, v, gate, w_q, w_k, W, o};
+  const void* const opt[] = {cache_q_in, cache_k_in, S0, z0, cache_q_out, cache_k_out, S_T, z_T, ws};
+  if ((r = check_ptrs(req, opt, p->T == 0))) return r;
+  if ((cache_q_out && cache_q_out == cache_q_in) || (cache_k_out && cache_k_out == cache_k_in)) return LAWCAT_ERR_INVALID_ARG;
+  // the sequences that the chunkwise layer kernel serves run together; the rest one by one
+  Ctx c{p, st, dev_status};
+  if ((r = launch_layer_tc_packed(c, cu_seqlens, nseq, q, k, v, gate, w_q, w_k, W, cache_q_in, cache_k_in, S0, z0, o,
+                                  cache_q_out, cache_k_out, S_T, z_T, ws)))
+    return r;
   for (int i = 0; i < nseq; ++i) {
     const size_t t0 = (size_t)cu_seqlens[i];
     lawcat_params pi = *p;
     pi.T = cu_seqlens[i + 1] - cu_seqlens[i];
+    if (layer_tc_supported(pi)) continue;
     const float* S0i = S0 ? S0 + i * nS : nullptr;
     const float* z0i = z0 ? z0 + i * nz : nullptr;
     float* STi = S_T ? S_T + i * nS : nullptr;

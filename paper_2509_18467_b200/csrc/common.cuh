@@ -77,11 +77,16 @@ int validate_params(const lawcat_params* p, bool need_T);
 
 // Chunkwise tensor-core layer forward (layer_tc.cu): whether it takes these parameters, and its launcher.
 bool layer_tc_supported(const lawcat_params& p);
-int layer_tc_segments(const lawcat_params& p);
 size_t layer_tc_workspace_bytes(const lawcat_params& p);
 int launch_layer_tc(const Ctx& c, const void* q, const void* k, const void* v, const void* gate, const void* w_q,
                     const void* w_k, const void* W, const void* cache_q_in, const void* cache_k_in, const float* S0,
                     const float* z0, void* o, void* cache_q_out, void* cache_k_out, float* S_T, float* z_T, void* ws);
+// The sequences of a packed batch that the layer kernel serves, in as few launches as their table allows (the others are left).
+size_t layer_tc_packed_workspace_bytes(const lawcat_params& p, const int32_t* cu_seqlens, int nseq);
+int launch_layer_tc_packed(const Ctx& c, const int32_t* cu_seqlens, int nseq, const void* q, const void* k, const void* v,
+                           const void* gate, const void* w_q, const void* w_k, const void* W, const void* cache_q_in,
+                           const void* cache_k_in, const float* S0, const float* z0, void* o, void* cache_q_out,
+                           void* cache_k_out, float* S_T, float* z_T, void* ws);
 
 // Chunkwise tensor-core GLA on given features and its backward (gla_tc.cu).
 bool gla_tc_supported(const lawcat_params& p);

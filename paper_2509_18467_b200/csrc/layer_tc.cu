@@ -1,6 +1,8 @@
 // Host side of the chunkwise tensor-core layer forward: tensor maps, segment split, launches.
+#include <algorithm>
 #include <atomic>
 #include <mutex>
+#include <vector>
 
 #include "layer_tc_kernel.cuh"
 
@@ -60,34 +62,49 @@ static bool make_map(CUtensorMap* m, const void* ptr, int heads, int T, int B, i
   return true;
 }
 
-// State at the start of every segment from the end states of its pieces (each computed from a zero state) and their
-// total decays: running state cur = given state; after piece i: cur = decay[i] * cur + local[i] (Eq. 4 unrolled over
-// whole pieces); start[seg] = cur in front of the segment's first piece.
-// One thread per state entry (the d_k x d_v entries of S, then the d_k entries of z) of one (batch, head).
-__global__ void segment_scan_kernel(const float* __restrict__ S0, const float* __restrict__ z0,
-                                    const float* __restrict__ loc_S, const float* __restrict__ loc_z,
-                                    const float* __restrict__ dtot, float* __restrict__ start_S,
-                                    float* __restrict__ start_z, int BH, int nseg, int nsub, int dh) {
+// State at the start of every segment but a sequence's first from the end states of the pieces in front (each computed from a
+// zero state) and their total decays: running state cur = given state; after piece i: cur = decay[i] * cur + local[i] (Eq. 4
+// unrolled over whole pieces). One thread per four state entries (the d_k x d_v entries of S, then the d_k entries of z) of one
+// (sequence, head).
+__global__ void segment_scan_kernel(const TcArgs a, const __grid_constant__ PackTab tab, const float* __restrict__ loc_S,
+                                    const float* __restrict__ loc_z, const float* __restrict__ dtot, float* __restrict__ start_S,
+                                    float* __restrict__ start_z, int nseq, int nsub, int dh) {
   const int D = dh;  // (rows and columns of the state as stored)
-  const int per = D * D + D;
+  const int per = (D * D + D) / 4;
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // the layer kernel may start its set-up
-  asm volatile("griddepcontrol.wait;" ::: "memory");               // (this kernel itself: behind the state-only pass)
-  if (idx >= BH * per) return;
-  const int bh = idx / per, r = idx % per;
-  const bool isz = r >= D * D;
-  const int c = isz ? r - D * D : r / D;  // key channel: the decay is per row of the state
-  const int e = isz ? 0 : r % D;
-  float cur = isz ? (z0 ? z0[(size_t)bh * D + c] : 0.f) : (S0 ? S0[((size_t)bh * D + c) * D + e] : 0.f);
-  for (int sgm = 0; sgm < nseg; ++sgm) {
-    const size_t so = (size_t)bh * nseg + sgm;
-    if (isz) start_z[so * D + c] = cur; else start_S[(so * D + c) * D + e] = cur;
-    if (sgm + 1 < nseg) {
-      for (int sb = 0; sb < nsub; ++sb) {
-        const size_t si = so * nsub + sb;
-        const float loc = isz ? loc_z[si * D + c] : loc_S[(si * D + c) * D + e];
-        cur = fmaf(exp2f(dtot[si * D + c]), cur, loc);
-      }
+  asm volatile("griddepcontrol.wait;" ::: "memory");               // behind the state-only pass
+  if (idx >= nseq * a.H * per) return;
+  const int e = idx % per * 4, h = idx / per % a.H;
+  const int i = idx / (per * a.H);
+  const int seg0 = tab.n ? tab.seg0[i] : i * a.nseg, nseg = tab.n ? tab.seg0[i + 1] - seg0 : a.nseg;
+  const int seq = tab.n ? tab.seq[i] : i;
+  const bool isz = e >= D * D;
+  const float* const init = isz ? a.z0 : a.S0;
+  const size_t n = isz ? D : (size_t)D * D, off = isz ? e - D * D : e;  // entries per state, this thread's first
+  const float* const loc = isz ? loc_z : loc_S;
+  float* const start = isz ? start_z : start_S;
+  float4 cur = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (init) cur = *reinterpret_cast<const float4*>(init + ((size_t)seq * a.H + h) * n + off);
+  const int np = (nseg - 1) * nsub;
+  constexpr int U = 4;  // pieces whose loads are in flight together
+  for (int i0 = 0; i0 < np; i0 += U) {
+    float4 l[U], d[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (i0 + u >= np) break;
+      const size_t si = ((size_t)seg0 * nsub + i0 + u) * a.H + h;
+      l[u] = *reinterpret_cast<const float4*>(loc + si * n + off);
+      // (the decay is per row of the state)
+      if (isz) d[u] = *reinterpret_cast<const float4*>(dtot + si * D + off);
+      else d[u].x = d[u].y = d[u].z = d[u].w = dtot[si * D + off / D];
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (i0 + u >= np) break;
+      cur.x = fmaf(exp2f(d[u].x), cur.x, l[u].x); cur.y = fmaf(exp2f(d[u].y), cur.y, l[u].y);
+      cur.z = fmaf(exp2f(d[u].z), cur.z, l[u].z); cur.w = fmaf(exp2f(d[u].w), cur.w, l[u].w);
+      if ((i0 + u + 1) % nsub == 0)
+        *reinterpret_cast<float4*>(start + ((size_t)(seg0 + (i0 + u + 1) / nsub) * a.H + h) * n + off) = cur;
     }
   }
 }
@@ -146,16 +163,91 @@ static TcPlan layer_tc_plan(const lawcat_params& p) {
   return pl;
 }
 
-int layer_tc_segments(const lawcat_params& p) { return layer_tc_plan(p).nseg; }
-
 // Limit of the kernels' device-side waits in clock cycles (about two seconds); a test hook may shorten it.
 static std::atomic<long long> g_wait_limit{4000000000LL};
 
+// scratch of a launch with `segs` segments in all (none when every sequence is one segment)
+static size_t layer_tc_scratch(const lawcat_params& p, size_t segs, int nsub) {
+  const size_t pieces = segs * nsub;
+  return sizeof(float) * (size_t)p.H * ((pieces + segs) * ((size_t)p.d_k * p.d_k + p.d_k) + pieces * p.d_k);
+}
+
 size_t layer_tc_workspace_bytes(const lawcat_params& p) {
   const TcPlan pl = layer_tc_plan(p);
-  if (pl.nseg == 1) return 0;
-  const size_t pieces = (size_t)pl.nseg * pl.nsub;
-  return sizeof(float) * (size_t)p.B * p.H * ((pieces + pl.nseg) * ((size_t)p.d_k * p.d_k + p.d_k) + pieces * p.d_k);
+  return pl.nseg == 1 ? 0 : layer_tc_scratch(p, (size_t)p.B * pl.nseg, pl.nsub);
+}
+
+// Packed sequences: how one launch cuts them. All sequences of the group share the SMs, so the segments are only as short as
+// it takes to keep the longest from being the tail: L, the longest segment allowed, is the one with the smallest estimate of
+// chunk times over {longest / 1 .. longest / 8}: per block its chunks and about three more for set-up and pipeline fill, the
+// total spread over the SMs but never less than the longest block and half a block of unevenness; when something is cut, the
+// state-only pass over all but the last segments (0.65 of a chunk time each) and its two extra launches (about two).
+static void layer_tc_pack(const lawcat_params& p, const int32_t* cu, const int* order, int n, tc::PackTab& t, int& nsub) {
+  const double sms = sm_count(), Hn = layer_tc_paired(p) ? p.H / 2 : p.H;
+  auto chunks = [&](int i) { return (cu[order[i] + 1] - cu[order[i]] + tc::C - 1) / tc::C; };
+  const int longest = chunks(0);
+  int best_L = longest, best_sub = 1;
+  double best = 1e30;
+  for (int k = 1; k <= 8 && (k == 1 || longest / k >= 4); ++k) {
+    const int L = (longest + k - 1) / k;
+    double work = 0, pre = 0, pieces = 0;
+    int seg_max = 0;
+    for (int i = 0; i < n; ++i) {
+      const int ch = chunks(i), ns = (ch + L - 1) / L, sl = (ch + ns - 1) / ns;
+      work += ch + 3.0 * ns;
+      pre += (double)(ns - 1) * sl;
+      pieces += ns - 1;
+      if (sl > seg_max) seg_max = sl;
+    }
+    auto span = [&](double total, double one) { return total * Hn / sms > one ? total * Hn / sms + 0.5 * one : one; };
+    const double main_cost = span(work, seg_max + 3.0);
+    if (pieces == 0) {
+      if (main_cost < best) { best = main_cost; best_L = L; best_sub = 1; }
+      continue;
+    }
+    for (int sub = 1; sub <= 4 && sub * 4 <= seg_max; ++sub) {
+      const double cost = main_cost + 2.0 + span(0.65 * (pre + 2.0 * sub * pieces), 0.65 * ((double)seg_max / sub + 2.0));
+      if (cost < best) { best = cost; best_L = L; best_sub = sub; }
+    }
+  }
+  nsub = best_sub;
+  t.n = n;
+  t.seg0[0] = 0;
+  for (int i = 0; i < n; ++i) {
+    const int ch = chunks(i), ns = (ch + best_L - 1) / best_L, sl = (ch + ns - 1) / ns;
+    t.tok0[i] = cu[order[i]];
+    t.len[i] = cu[order[i] + 1] - cu[order[i]];
+    t.seg_len[i] = sl * tc::C;
+    t.seg0[i + 1] = t.seg0[i] + (ch + sl - 1) / sl;
+    t.seq[i] = order[i];
+  }
+}
+
+// the sequences that the packed launches take (those the layer kernel serves: at least 16 tokens), the longest first
+static std::vector<int> layer_tc_pack_order(const lawcat_params& p, const int32_t* cu, int nseq) {
+  std::vector<int> order;
+  lawcat_params q = p;
+  q.B = 1;
+  for (int i = 0; i < nseq; ++i) {
+    q.T = cu[i + 1] - cu[i];
+    if (layer_tc_supported(q)) order.push_back(i);
+  }
+  std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return cu[x + 1] - cu[x] > cu[y + 1] - cu[y]; });
+  return order;
+}
+
+size_t layer_tc_packed_workspace_bytes(const lawcat_params& p, const int32_t* cu, int nseq) {
+  const std::vector<int> order = layer_tc_pack_order(p, cu, nseq);
+  size_t need = 0;
+  for (size_t o = 0; o < order.size(); o += tc::PACK_MAX) {
+    const int n = (int)(order.size() - o < tc::PACK_MAX ? order.size() - o : tc::PACK_MAX);
+    tc::PackTab t;
+    int nsub = 1;
+    layer_tc_pack(p, cu, order.data() + o, n, t, nsub);
+    const size_t b = t.seg0[n] == n ? 0 : layer_tc_scratch(p, (size_t)t.seg0[n], nsub);
+    if (b > need) need = b;
+  }
+  return need;
 }
 
 bool layer_tc_supported(const lawcat_params& p) {
@@ -173,9 +265,11 @@ bool layer_tc_supported(const lawcat_params& p) {
          !p.mix_unshared;  // (one W_h is what lets both streams share the M = 128 mix)
 }
 
-int launch_layer_tc(const Ctx& c, const void* q, const void* k, const void* v, const void* gate, const void* w_q,
-                    const void* w_k, const void* W, const void* cache_q_in, const void* cache_k_in, const float* S0,
-                    const float* z0, void* o, void* cache_q_out, void* cache_k_out, float* S_T, float* z_T, void* ws) {
+// One launch set over a uniform batch (tab.n = 0) or a group of packed sequences; `segs` segments in all, of `nseq` sequences.
+static int run_layer_tc(const Ctx& c, const void* q, const void* k, const void* v, const void* gate, const void* w_q,
+                        const void* w_k, const void* W, const void* cache_q_in, const void* cache_k_in, const float* S0,
+                        const float* z0, void* o, void* cache_q_out, void* cache_k_out, float* S_T, float* z_T, void* ws,
+                        const TcPlan& pl, const tc::PackTab& tab, int nseq, int segs) {
   using namespace tc;
   const lawcat_params& p = *c.p;
   CUtensorMap tq, tk, tv, tg;
@@ -198,10 +292,11 @@ int launch_layer_tc(const Ctx& c, const void* q, const void* k, const void* v, c
   a.T = p.T; a.H = p.H; a.Hkv = p.H_kv; a.K = p.conv_k;
   a.gate_mode = p.gate_mode; a.normalize = p.normalize; a.inv_tau = 1.f / p.gate_tau; a.eps = p.eps;
   a.wait_limit = g_wait_limit.load();
-  const TcPlan pl = layer_tc_plan(p);
-  const int nseg = pl.nseg;
-  a.nseg = nseg;
+  const int nsub = pl.nsub;
+  a.nseg = pl.nseg;
   a.seg_len = pl.seg_len;
+  a.nsub = 1;
+  a.S0 = S0; a.z0 = z0; a.S_T = S_T; a.z_T = z_T;
   auto* const k_layer = paired ? layer_tc_kernel<0, 2> : dh == 64 ? layer_tc_kernel<0, 1> : layer_tc_kernel<0, 0>;
   auto* const k_state = paired ? layer_tc_kernel<1, 2> : dh == 64 ? layer_tc_kernel<1, 1> : layer_tc_kernel<1, 0>;
   {
@@ -222,67 +317,80 @@ int launch_layer_tc(const Ctx& c, const void* q, const void* k, const void* v, c
       done[dev] = true;
     }
   }
-  const int BH = p.B * p.H;                       // real heads: the states in the workspace are per real head
-  const int NB = paired ? BH / 2 : BH;            // sequences of thread blocks
-  if (nseg == 1) {
-    a.S0 = S0; a.z0 = z0; a.S_T = S_T; a.z_T = z_T; a.dtot = nullptr;
-    a.grid_nseg = 1; a.nsub = 1; a.seg_in = 0; a.seg_out = 0;
+  const int Hn = paired ? p.H / 2 : p.H;          // thread blocks per segment
+  if (segs == nseq) {
     LaunchScope _ls("layer_tc", c.stream);
-    k_layer<<<NB, THREADS, SMEM_ALLOC, c.stream>>>(tq, tk, tv, tg, a);
+    k_layer<<<Hn * segs, THREADS, SMEM_ALLOC, c.stream>>>(tq, tk, tv, tg, a, tab);
     LAWCAT_CHECK_LAUNCH();
     return LAWCAT_OK;
   }
-  // Several segments per sequence: (1) every segment but the last computes its end state from a zero state, and the
+  // Several segments per sequence: (1) every segment but a sequence's last computes its end state from a zero state, and the
   // total decay of the segment; (2) a scan over the segments turns these into the state at each segment's start;
   // (3) the layer runs on all segments at once, each from its start state.
-  const int nsub = pl.nsub;
-  const size_t nS = (size_t)BH * nseg * dh * dh, nz = (size_t)BH * nseg * dh;
-  float* loc_S = (float*)ws;              // [BH, nseg, nsub, D, D]
-  float* loc_z = loc_S + nS * nsub;       // [BH, nseg, nsub, D]
-  float* dtot = loc_z + nz * nsub;        // [BH, nseg, nsub, D]
-  float* start_S = dtot + nz * nsub;      // [BH, nseg, D, D]
-  float* start_z = start_S + nS;          // [BH, nseg, D]
+  const size_t nS = (size_t)p.H * segs * dh * dh, nz = (size_t)p.H * segs * dh;
+  float* loc_S = (float*)ws;              // [segs, nsub, H, D, D]
+  float* loc_z = loc_S + nS * nsub;       // [segs, nsub, H, D]
+  float* dtot = loc_z + nz * nsub;        // [segs, nsub, H, D]
+  float* start_S = dtot + nz * nsub;      // [segs, H, D, D]
+  float* start_z = start_S + nS;          // [segs, H, D]
   {
     TcArgs b1 = a;
-    b1.S0 = nullptr; b1.z0 = nullptr; b1.S_T = loc_S; b1.z_T = loc_z; b1.dtot = dtot;
-    b1.grid_nseg = nseg - 1; b1.nsub = nsub; b1.seg_in = 1; b1.seg_out = 1;
+    b1.S_T = loc_S; b1.z_T = loc_z; b1.dtot = dtot; b1.nsub = nsub;
     LaunchScope _ls("layer_tc_state", c.stream);
-    k_state<<<NB * (nseg - 1) * nsub, THREADS, SMEM_ALLOC, c.stream>>>(tq, tk, tv, tg, b1);
+    k_state<<<Hn * (segs - nseq) * nsub, THREADS, SMEM_ALLOC, c.stream>>>(tq, tk, tv, tg, b1, tab);
     LAWCAT_CHECK_LAUNCH();
   }
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.stream = c.stream;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
   {
-    const int total = BH * (dh * dh + dh);
+    const int total = nseq * p.H * (dh * dh + dh) / 4;
     LaunchScope _ls("segment_scan", c.stream);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((total + 255) / 256));
-    cfg.blockDim = dim3(256);
-    cfg.stream = c.stream;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, segment_scan_kernel, S0, z0, (const float*)loc_S, (const float*)loc_z, (const float*)dtot,
-                       start_S, start_z, BH, nseg, nsub, dh);
+    cfg.gridDim = dim3((unsigned)((total + 127) / 128));
+    cfg.blockDim = dim3(128);
+    cudaLaunchKernelEx(&cfg, segment_scan_kernel, a, tab, (const float*)loc_S, (const float*)loc_z, (const float*)dtot,
+                       start_S, start_z, nseq, nsub, dh);
     LAWCAT_CHECK_LAUNCH();
   }
-  a.S0 = start_S; a.z0 = start_z; a.S_T = S_T; a.z_T = z_T; a.dtot = nullptr;
-  a.grid_nseg = nseg; a.nsub = 1; a.seg_in = 1; a.seg_out = 0;
-  LaunchScope _ls("layer_tc", c.stream);
+  a.seg_S = start_S; a.seg_z = start_z;
   {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(NB * nseg));
-    cfg.blockDim = dim3(THREADS);
-    cfg.dynamicSmemBytes = SMEM_ALLOC;
-    cfg.stream = c.stream;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, k_layer, tq, tk, tv, tg, a);
+    // (an ordinary launch: as a dependent of the scan its blocks land while scan blocks still hold registers of most SMs,
+    // and the call at T = 32768 took 1.34 ms instead of 1.11)
+    LaunchScope _ls("layer_tc", c.stream);
+    k_layer<<<Hn * segs, THREADS, SMEM_ALLOC, c.stream>>>(tq, tk, tv, tg, a, tab);
   }
   LAWCAT_CHECK_LAUNCH();
+  return LAWCAT_OK;
+}
+
+int launch_layer_tc(const Ctx& c, const void* q, const void* k, const void* v, const void* gate, const void* w_q,
+                    const void* w_k, const void* W, const void* cache_q_in, const void* cache_k_in, const float* S0,
+                    const float* z0, void* o, void* cache_q_out, void* cache_k_out, float* S_T, float* z_T, void* ws) {
+  const TcPlan pl = layer_tc_plan(*c.p);
+  tc::PackTab tab;
+  tab.n = 0;
+  return run_layer_tc(c, q, k, v, gate, w_q, w_k, W, cache_q_in, cache_k_in, S0, z0, o, cache_q_out, cache_k_out, S_T, z_T, ws,
+                      pl, tab, c.p->B, c.p->B * pl.nseg);
+}
+
+int launch_layer_tc_packed(const Ctx& c, const int32_t* cu, int nseq, const void* q, const void* k, const void* v,
+                           const void* gate, const void* w_q, const void* w_k, const void* W, const void* cache_q_in,
+                           const void* cache_k_in, const float* S0, const float* z0, void* o, void* cache_q_out,
+                           void* cache_k_out, float* S_T, float* z_T, void* ws) {
+  const std::vector<int> order = layer_tc_pack_order(*c.p, cu, nseq);
+  for (size_t at = 0; at < order.size(); at += tc::PACK_MAX) {
+    const int n = (int)(order.size() - at < tc::PACK_MAX ? order.size() - at : tc::PACK_MAX);
+    tc::PackTab tab;
+    TcPlan pl{};
+    layer_tc_pack(*c.p, cu, order.data() + at, n, tab, pl.nsub);
+    const int r = run_layer_tc(c, q, k, v, gate, w_q, w_k, W, cache_q_in, cache_k_in, S0, z0, o, cache_q_out, cache_k_out, S_T,
+                               z_T, ws, pl, tab, n, tab.seg0[n]);
+    if (r) return r;
+  }
   return LAWCAT_OK;
 }
 

@@ -25,7 +25,10 @@
 // +-8 and the state within +-3e4 -- the usual case -- and bf16 otherwise (range first). bf16 score weights would
 // cost up to 2^-9 relative error per weight, which the first tokens of a sequence do not average out.
 // Every MMA uses M = 128; where only 64 rows are meaningful (P, O') the upper 64 TMEM lanes hold unused results.
-// Loops over column blocks are deliberately NOT unrolled: each role's loop must stay inside the instruction cache.
+// Loops over column blocks are deliberately NOT unrolled, and a sweep keeps ONE copy of its body (16 columns, the next load
+// issued into the registers it has just copied out of): the roles together are near the size of the instruction cache. With two
+// copies per sweep, moving a few unrelated instructions cost up to a quarter of the kernel's time (770 -> 950 us at T = 32768;
+// warps without an instruction 0.81 -> 1.12 per issue slot); with one copy it takes 750 us.
 // Every wait is bounded: a wait that runs out raises the abort flag, every role leaves its loop, the CTA frees its
 // tensor memory and reports LAWCAT_ERR_TIMEOUT through dev_status.
 #pragma once
@@ -135,6 +138,28 @@ enum {
   NUM_BARS
 };
 
+// Packed sequences of different lengths in one launch: one entry per sequence (the longest first, so that the last wave of
+// thread blocks is the short ones). The tokens of the batch lie back to back along T of ONE batch element.
+constexpr int PACK_MAX = 64;   // sequences per launch (the table travels as a kernel parameter)
+struct PackTab {
+  int n;                       // entries; 0: a uniform batch, described by TcArgs alone
+  int tok0[PACK_MAX];          // first token
+  int len[PACK_MAX];           // tokens
+  int seg0[PACK_MAX + 1];      // segments of the entries in front
+  int seg_len[PACK_MAX];       // tokens per segment (a multiple of the chunk)
+  int seq[PACK_MAX];           // index of the sequence among the caller's states and caches
+};
+
+// What a thread block works on.
+struct SeqView {
+  int seq;                     // sequence: index into states and caches
+  int T;                       // its length
+  int nseg, seg_len;           // its segments
+  int seg0;                    // segments of the sequences in front: index of its first state in the workspace
+  int tm_t, tm_b;              // tensor-map coordinates of its first token
+  size_t row0;                 // first token as a row of the [tokens, heads, channels] tensors
+};
+
 struct TcArgs {
   const bf16 *q, *k;     // raw streams (for the halo rows in front of a segment)
   const bf16* gate;      // gate logits; read directly when there is one per token and head (gate_dim = 1)
@@ -143,23 +168,41 @@ struct TcArgs {
                          // channels (of q, k, gate, v, W, the state) are zero: the tiles' second 64-channel slabs are
                          // zeroed once and never loaded, and the feature map leaves the padded outputs out
   const bf16 *w_q, *w_k, *W, *cache_q, *cache_k;
-  const float *S0, *z0;  // state before the first token of the CTA's segment
-  float *S_T, *z_T;      // state after the last token of the CTA's segment
-  float* dtot;           // [B,H,nseg,128]: log2 of the total decay of the segment per key channel (nullable)
+  const float *S0, *z0;  // [seq,H,..]: state in front of each sequence (nullable: zero)
+  const float *seg_S, *seg_z;  // (MODE 0) [segment,H,..]: state in front of every segment but a sequence's first
+  float *S_T, *z_T;      // MODE 0: [seq,H,..] state after the last token; MODE 1: [segment piece,H,..] state of the piece
+  float* dtot;           // (MODE 1) [segment piece,H,128]: log2 of the total decay of the piece per key channel
   bf16* o;               // [B,T,H,128]
   bf16 *cache_q_out, *cache_k_out;  // conv caches after the last token (nullable): [B,K-1,H*dh], [B,K-1,Hkv*dh]
   int* dev_status;
   int T, H, Hkv, K;
-  int nseg, seg_len;     // segments per sequence and tokens per segment (a multiple of C)
-  int grid_nseg;         // segments of each sequence covered by this launch (the first grid_nseg of nseg)
-  int nsub;              // pieces each segment is cut into by this launch (whole chunks; 1 = the segment itself)
-  int seg_in;            // 1: S0/z0 are indexed [b,h,seg*nsub+sub]; 0: [b,h] and they apply to segment 0 only
-  int seg_out;           // 1: S_T/z_T (and dtot) are indexed [b,h,seg*nsub+sub]; 0: [b,h], written by the last segment
+  int nseg, seg_len;     // uniform batch: segments per sequence and tokens per segment (a multiple of C)
+  int nsub;              // MODE 1: pieces each segment is cut into (whole chunks); MODE 0: 1
   int gate_mode;
   int normalize;         // 1: Eq. 8; 0: the numerator alone (the query features then carry their softmax normalizer)
   float inv_tau, eps;
   long long wait_limit;  // clock cycles a device-side wait may take before the block gives up (about 2 s by default)
 };
+
+// The sequence that block `blk` of a launch works on, with `per_seg` blocks per segment and `skip` segments of each sequence
+// left out (MODE 1 leaves out the last); blk becomes the block's index inside the sequence.
+__device__ __forceinline__ SeqView seq_of_block(const TcArgs& a, const PackTab& tab, int per_seg, int skip, int& blk) {
+  SeqView v;
+  if (tab.n == 0) {
+    const int per_seq = (a.nseg - skip) * per_seg;
+    v.seq = blk / per_seq;
+    blk -= v.seq * per_seq;
+    v.T = a.T; v.nseg = a.nseg; v.seg_len = a.seg_len; v.seg0 = v.seq * a.nseg;
+    v.tm_t = 0; v.tm_b = v.seq; v.row0 = (size_t)v.seq * a.T;
+  } else {
+    int i = 0;
+    while (i + 1 < tab.n && blk >= (tab.seg0[i + 1] - skip * (i + 1)) * per_seg) ++i;
+    blk -= (tab.seg0[i] - skip * i) * per_seg;
+    v.seq = tab.seq[i]; v.T = tab.len[i]; v.nseg = tab.seg0[i + 1] - tab.seg0[i]; v.seg_len = tab.seg_len[i]; v.seg0 = tab.seg0[i];
+    v.tm_t = tab.tok0[i]; v.tm_b = 0; v.row0 = (size_t)tab.tok0[i];
+  }
+  return v;
+}
 
 __device__ __forceinline__ void unpack8(const uint4& v, float* f) {
   f[0] = bf16_lo(v.x); f[1] = bf16_hi(v.x); f[2] = bf16_lo(v.y); f[3] = bf16_hi(v.y);
@@ -273,7 +316,8 @@ __device__ __forceinline__ bool wait_set_or_abort(uint32_t bar0, uint32_t mask, 
 template <int MODE, int WIDTH>
 __global__ void __launch_bounds__(THREADS, 1)
 layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-                const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_g, const TcArgs a) {
+                const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_g, const TcArgs a,
+                const __grid_constant__ PackTab tab) {
   extern __shared__ __align__(1024) uint8_t sg[];
   const uint32_t sb = smem_u32(sg);
   volatile int* const s_flags = reinterpret_cast<volatile int*>(sg + OFF_BAR + 8 * NUM_BARS);  // [0] tmem base, [1] abort
@@ -302,22 +346,25 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   // tensor memory columns (the pair keeps two read-out and two score accumulators where the state needs half the columns)
   constexpr uint32_t cS = COL_S, cSZ = pair ? 192u : COL_SZ, cO = pair ? 208u : COL_O, cO2 = 288u;
   constexpr uint32_t cP = pair ? 368u : COL_P, cP2 = 432u, cMAIL = pair ? 496u : COL_MAIL;
-  const int sub = blockIdx.x % a.nsub;
-  const int seg = (blockIdx.x / a.nsub) % a.grid_nseg;
-  const int bh = blockIdx.x / (a.nsub * a.grid_nseg);
   const int Hn = pair ? a.H / 2 : a.H;   // heads as addressed (units of dh channels)
-  const int h = bh % Hn, b = bh / Hn;
+  // blocks of a sequence: head (outer), segment, piece
+  int blk = blockIdx.x;
+  const SeqView sq = seq_of_block(a, tab, Hn * a.nsub, MODE == 1 ? 1 : 0, blk);
+  const int segs_run = sq.nseg - (MODE == 1 ? 1 : 0);
+  const int sub = blk % a.nsub;
+  const int seg = (blk / a.nsub) % segs_run;
+  const int h = blk / (a.nsub * segs_run), b = sq.seq, T = sq.T;
   const int h0 = pair ? 2 * h : h;       // first real head of this block
   const int G = a.H / a.Hkv, j = h0 / G;
-  const int cps = a.seg_len / C;  // chunks per segment; piece `sub` covers chunks [sub cps / nsub, (sub + 1) cps / nsub)
-  const int t_begin = min(a.T, seg * a.seg_len + (sub * cps / a.nsub) * C);
-  const int t_end = min(a.T, seg * a.seg_len + ((sub + 1) * cps / a.nsub) * C);
+  const int cps = sq.seg_len / C;  // chunks per segment; piece `sub` covers chunks [sub cps / nsub, (sub + 1) cps / nsub)
+  const int t_begin = min(T, seg * sq.seg_len + (sub * cps / a.nsub) * C);
+  const int t_end = min(T, seg * sq.seg_len + ((sub + 1) * cps / a.nsub) * C);
   const int nchunks = max(0, (t_end - t_begin + C - 1) / C);
-  // index of the state of the real head that owns state row c (rows 64-127 of a pair: the second head)
-  auto state_idx = [&](int c, int per_segment) -> size_t {
-    const size_t hr = (size_t)b * a.H + h0 + (pair ? (c >> 6) : 0);
-    return per_segment ? (hr * a.nseg + seg) * a.nsub + sub : hr;
-  };
+  // index of the state of the real head that owns state row c (rows 64-127 of a pair: the second head): among the caller's
+  // states (one per sequence), or among the workspace's (one per segment piece)
+  auto head_of_row = [&](int c) -> size_t { return h0 + (pair ? (c >> 6) : 0); };
+  auto seq_state = [&](int c) -> size_t { return (size_t)b * a.H + head_of_row(c); };
+  auto seg_state = [&](int c) -> size_t { return ((size_t)(sq.seg0 + seg) * a.nsub + sub) * a.H + head_of_row(c); };
 
   if ((sb & 1023u) != 0) {  // the swizzled tiles need a 1024-byte aligned base
     if (tid == 0 && a.dev_status) atomicMax(a.dev_status, (int)LAWCAT_ERR_CUDA);
@@ -399,7 +446,7 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     if (oc * 8 >= dh) {
       // padded channels: zero
     } else if (t >= 0) {
-      v = *reinterpret_cast<const uint4*>((st ? a.k : a.q) + ((size_t)b * a.T + t) * rstride + coff);
+      v = *reinterpret_cast<const uint4*>((st ? a.k : a.q) + (sq.row0 + t) * rstride + coff);
     } else {
       const bf16* cache = st ? a.cache_k : a.cache_q;
       const int ci = t + (a.K - 1);  // the cache holds tokens -(K-1) .. -1, oldest first
@@ -410,7 +457,7 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   __syncthreads();
   // conv caches after the last token (Section 4.1: the last K - 1 raw rows of [cache_in, x]): they depend on the raw
   // inputs alone, so the block of a head's last segment writes them here (the key stream by the first head of a group)
-  if (MODE == 0 && seg == a.nseg - 1 && sub == 0 && a.K > 1 && tid < PREP_THREADS) {
+  if (MODE == 0 && seg == sq.nseg - 1 && sub == 0 && a.K > 1 && tid < PREP_THREADS) {
     const int per = (a.K - 1) * (dh / 8);  // 16-byte units per stream (the key stream of a pair uses the first hd / 8 per row)
     for (int idx = tid; idx < 2 * per; idx += PREP_THREADS) {
       const int st = idx / per, r = (idx % per) / (dh / 8), oc = idx % (dh / 8);
@@ -418,11 +465,11 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       if (dst == nullptr || (st == 1 && (h0 % G != 0 || oc * 8 >= hd))) continue;
       const size_t rstride = st ? (size_t)a.Hkv * hd : (size_t)Hn * dh;
       const size_t coff = (st ? (size_t)j * hd : (size_t)h * dh) + (size_t)oc * 8;
-      const int tok = a.T - (a.K - 1) + r;
+      const int tok = T - (a.K - 1) + r;
       const bf16* x = st ? a.k : a.q;
       const bf16* cin = st ? a.cache_k : a.cache_q;
       uint4 v = make_uint4(0u, 0u, 0u, 0u);
-      if (tok >= 0) v = *reinterpret_cast<const uint4*>(x + ((size_t)b * a.T + tok) * rstride + coff);
+      if (tok >= 0) v = *reinterpret_cast<const uint4*>(x + (sq.row0 + tok) * rstride + coff);
       else if (cin != nullptr) v = *reinterpret_cast<const uint4*>(cin + ((size_t)b * (a.K - 1) + tok + a.K - 1) * rstride + coff);
       *reinterpret_cast<uint4*>(dst + ((size_t)b * (a.K - 1) + r) * rstride + coff) = v;
     }
@@ -435,15 +482,16 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   const uint32_t tmem = (uint32_t)s_flags[0];
   const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
 
-  // Launched with programmatic stream serialization: the set-up above may run beside the tail of the kernel in front
-  // (the scan over the segments, whose results are the start states read next); from here on that kernel has completed.
-  asm volatile("griddepcontrol.wait;" ::: "memory");
   // initial state into tensor memory: row thread (c, half) owns 64 columns of row c of [S | z]
   if (warp >= ROW_WARP0 && warp < ROW_WARP0 + 8) {
     // (pair: the state is [128 key channels x 64 value columns], the thread owns 32 columns; rows 64-127 are the second head)
     const int tw = tid - ROW_WARP0 * 32, c = tw & 127, chh = tw >> 7;
-    const bool have = a.S0 != nullptr && (a.seg_in || seg == 0);
-    const size_t in_idx = state_idx(c, a.seg_in);
+    // a sequence's first segment starts from the caller's state, the others from the scan's; pieces from zero
+    const bool first = seg == 0;
+    const float* const srcS = MODE == 1 ? nullptr : first ? a.S0 : a.seg_S;
+    const float* const srcz = MODE == 1 ? nullptr : first ? a.z0 : a.seg_z;
+    const bool have = srcS != nullptr, havez = srcz != nullptr;
+    const size_t in_idx = first ? seq_state(c) : seg_state(c);
     const int cr = c & (hd - 1);  // row inside the real head's state
     float s[32], mx = 0.f;
 #pragma unroll 1
@@ -451,14 +499,13 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       const int blk = pair ? chh : chh * 2 + b2;
 #pragma unroll
       for (int i = 0; i < 32; ++i) {
-        s[i] = (have && c < dh && blk * 32 < hd) ? a.S0[(in_idx * hd + cr) * hd + blk * 32 + i] : 0.f;
+        s[i] = (have && c < dh && blk * 32 < hd) ? srcS[(in_idx * hd + cr) * hd + blk * 32 + i] : 0.f;
         mx = fmaxf(mx, fabsf(s[i]));
       }
       tmem_st32(lane_base + cS + blk * 32, s);
     }
     if (chh == 1) {
-      const bool havez = a.z0 != nullptr && (a.seg_in || seg == 0);
-      const float z0v = (havez && c < dh) ? a.z0[in_idx * hd + cr] : 0.f;
+      const float z0v = (havez && c < dh) ? srcz[in_idx * hd + cr] : 0.f;
       tmem_st1(lane_base + cSZ, z0v);
       mx = fmaxf(mx, fabsf(z0v));
     }
@@ -488,28 +535,28 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     if (lane == 0) {
       int ar_raw = -1, ar_g = -1, ar_v = -1;  // last chunk whose copies were started, per tile
       for (int n = 0; n < nchunks; ++n) {
-        const int t0 = t_begin + n * C;
+        const int tt0 = sq.tm_t + t_begin + n * C;
         const uint32_t pp = (uint32_t)((n - 1) & 1);
         if (n > 0) WAIT(B_MMA1, pp);  // MMA 1 of the previous chunk has read the in-place conv output
         mbar_arrive_expect_tx(bar(B_RAW_FULL), (MODE == 0 ? 16384u : 8192u) * (uint32_t)nslab);
 #pragma unroll 1
         for (int s = 0; s < nslab; ++s) {
-          if (MODE == 0) tma_load_4d(sb + OFF_AU + s * 16384, &tm_q, bar(B_RAW_FULL), s * 64, h, t0, b);
+          if (MODE == 0) tma_load_4d(sb + OFF_AU + s * 16384, &tm_q, bar(B_RAW_FULL), s * 64, h, tt0, sq.tm_b);
           // (pair: the same 64 key channels into both halves of the tile)
-          tma_load_4d(sb + OFF_AU + s * 16384 + 8192, &tm_k, bar(B_RAW_FULL), pair ? 0 : s * 64, j, t0, b);
+          tma_load_4d(sb + OFF_AU + s * 16384 + 8192, &tm_k, bar(B_RAW_FULL), pair ? 0 : s * 64, j, tt0, sq.tm_b);
         }
         ar_raw = n;
         if (a.gate_dim != 1) {
           if (n > 0) WAIT(B_G_FREE, pp);
           mbar_arrive_expect_tx(bar(B_G_FULL), 8192u * (uint32_t)nslab);
-          tma_load_4d(sb + OFF_G, &tm_g, bar(B_G_FULL), 0, h, t0, b);
-          if (nslab == 2) tma_load_4d(sb + OFF_G + 8192, &tm_g, bar(B_G_FULL), 64, h, t0, b);
+          tma_load_4d(sb + OFF_G, &tm_g, bar(B_G_FULL), 0, h, tt0, sq.tm_b);
+          if (nslab == 2) tma_load_4d(sb + OFF_G + 8192, &tm_g, bar(B_G_FULL), 64, h, tt0, sq.tm_b);
           ar_g = n;
         }
         if (n > 0) WAIT(MODE == 0 ? B_MMA3 : B_MMA2, pp);  // the last MMA that reads v
         mbar_arrive_expect_tx(bar(B_V_FULL), 8192u * (uint32_t)vslab);
-        tma_load_4d(sb + OFF_V, &tm_v, bar(B_V_FULL), 0, j, t0, b);
-        if (vslab == 2) tma_load_4d(sb + OFF_V + 8192, &tm_v, bar(B_V_FULL), 64, j, t0, b);
+        tma_load_4d(sb + OFF_V, &tm_v, bar(B_V_FULL), 0, j, tt0, sq.tm_b);
+        if (vslab == 2) tma_load_4d(sb + OFF_V + 8192, &tm_v, bar(B_V_FULL), 64, j, tt0, sq.tm_b);
         ar_v = n;
       }
       if (*s_abort) {
@@ -659,6 +706,7 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       tc_fence_before_sync();
       mbar_arrive(bar(B_O_FREE));
     };
+    bf16* const obase = a.o + (sq.row0 * Hn + h) * dh;
     auto out_pass = [&](int m) {
       if ((warp & 3) >= 2) return;
       const int orow_i = (warp & 3) * 32 + lane, och = tid >> 7;
@@ -684,21 +732,24 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       tmem_wait_ld();
       den += den_p0 + den_p1;
       const float inv = 1.f / (a.normalize ? fmaf(a.eps, qs, den) : qs);
-      bf16* orow = a.o + (((size_t)b * a.T + ot0 + orow_i) * Hn + h) * dh + och * 64;
-      float y[32];
+      bf16* orow = obase + (size_t)(ot0 + orow_i) * (Hn * dh) + och * 64;
+      // (columns at a time: 16 keep the code small; the pair, whose other roles are smaller, is faster with 32)
+      constexpr int NC = pair ? 32 : 16;
+      float y[NC];
 #pragma unroll 1
-      for (int b2 = 0; b2 < 2; ++b2) {
-        tmem_ld32(lane_base + ocol + b2 * 32, y);
+      for (int c0 = 0; c0 < 64; c0 += NC) {
+        if constexpr (pair) tmem_ld32(lane_base + ocol + c0, y);
+        else tmem_ld16(lane_base + ocol + c0, y);
         tmem_wait_ld();
-        if (b2 == 1) {  // O' is in registers: the next chunk's products may overwrite it
+        if (c0 == 64 - NC) {  // O' is in registers: the next chunk's products may overwrite it
           tc_fence_before_sync();
           mbar_arrive(bar(B_O_FREE));
         }
 #pragma unroll
-        for (int i = 0; i < 32; ++i) y[i] *= inv;
+        for (int i = 0; i < NC; ++i) y[i] *= inv;
         if (orow_i < onvalid && och * 64 < dh) {
 #pragma unroll
-          for (int q4 = 0; q4 < 4; ++q4) *reinterpret_cast<uint4*>(orow + b2 * 32 + q4 * 8) = pack8(y + 8 * q4, false);
+          for (int i = 0; i < NC; i += 8) *reinterpret_cast<uint4*>(orow + c0 + i) = pack8(y + i, false);
         }
       }
     };
@@ -708,7 +759,7 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     auto gate1_load = [&](int m) -> float {
       const int t = t_begin + m * C + tid;
       return (a.gate_dim == 1 && tid < C && m < nchunks && t < t_end)
-                 ? __bfloat162float(a.gate[((size_t)b * a.T + t) * a.H + h]) : 0.f;
+                 ? __bfloat162float(a.gate[(sq.row0 + t) * a.H + h]) : 0.f;
     };
     float g1_next = gate1_load(0);
     bool fail = false;
@@ -849,7 +900,7 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         const int vthreads = MODE == 1 ? PREP_THREADS : PREP_THREADS / 2;
         const int vt = MODE == 1 ? tid : (tid >> 7) * 64 + ((warp & 3) - 2) * 32 + lane;
         float vm = 0.f;
-#pragma unroll 4
+#pragma unroll 2
         for (int i = 0; i < vslab * 512 / vthreads; ++i) {
           const uint32_t ad = sb + OFF_V + (uint32_t)(vt + vthreads * i) * 16;
           float x[8];
@@ -977,23 +1028,15 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
           // key rows: e = exp(y - max) and its sum; e is parked in Y's own columns for the writing sweep
           if (!fail && !padded) {
 #pragma unroll 1
-            for (int b2 = 0; b2 < 2; ++b2) {
+            for (int b4 = 0; b4 < 4; ++b4) {
               tmem_wait_ld();
-              tmem_ld16(ycol + b2 * 32 + 16, yb);
 #pragma unroll
               for (int i = 0; i < 16; ++i) {
-                ya[i] = ex2f(fmaf(ya[i], L2E, -mb));
-                sum += ya[i];
-              }
-              tmem_st16(ycol + b2 * 32, ya);
-              tmem_wait_ld();
-              if (b2 < 1) tmem_ld16(ycol + b2 * 32 + 32, ya);
-#pragma unroll
-              for (int i = 0; i < 16; ++i) {
-                yb[i] = ex2f(fmaf(yb[i], L2E, -mb));
+                yb[i] = ex2f(fmaf(ya[i], L2E, -mb));
                 sum += yb[i];
               }
-              tmem_st16(ycol + b2 * 32 + 16, yb);
+              if (b4 < 3) tmem_ld16(ycol + b4 * 16 + 16, ya);
+              tmem_st16(ycol + b4 * 16, yb);
             }
           }
           if (wide) {
@@ -1097,13 +1140,12 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
           };
           // (`ya` holds the first 16 columns since the row-max sweep)
 #pragma unroll 1
-          for (int b2 = 0; b2 < 2; ++b2) {
+          for (int b4 = 0; b4 < 4; ++b4) {
             tmem_wait_ld();
-            tmem_ld16(ycol + b2 * 32 + 16, yb);
-            q_block(ya, ch * 8 + b2 * 4);
-            tmem_wait_ld();
-            if (b2 < 1) tmem_ld16(ycol + b2 * 32 + 32, ya);
-            q_block(yb, ch * 8 + b2 * 4 + 2);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) yb[i] = ya[i];
+            if (b4 < 3) tmem_ld16(ycol + b4 * 16 + 16, ya);
+            q_block(yb, ch * 8 + b4 * 2);
           }
           if (need_qsum) {
             // the dropped normalizer travels to the output pass through tensor memory: each half adds its part
@@ -1132,14 +1174,25 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             }
           };
           tmem_ld16(ycol, ya);
+          if (MODE == 0) {
 #pragma unroll 1
-          for (int b2 = 0; b2 < 2; ++b2) {
-            tmem_wait_ld();
-            tmem_ld16(ycol + b2 * 32 + 16, yb);
-            k_block(ya, ch * 8 + b2 * 4);
-            tmem_wait_ld();
-            if (b2 < 1) tmem_ld16(ycol + b2 * 32 + 32, ya);
-            k_block(yb, ch * 8 + b2 * 4 + 2);
+            for (int b4 = 0; b4 < 4; ++b4) {
+              tmem_wait_ld();
+#pragma unroll
+              for (int i = 0; i < 16; ++i) yb[i] = ya[i];
+              if (b4 < 3) tmem_ld16(ycol + b4 * 16 + 16, ya);
+              k_block(yb, ch * 8 + b4 * 2);
+            }
+          } else {  // (the state-only pass is small enough to afford two copies, with a load in flight across both)
+#pragma unroll 1
+            for (int b2 = 0; b2 < 2; ++b2) {
+              tmem_wait_ld();
+              tmem_ld16(ycol + b2 * 32 + 16, yb);
+              k_block(ya, ch * 8 + b2 * 4);
+              tmem_wait_ld();
+              if (b2 < 1) tmem_ld16(ycol + b2 * 32 + 32, ya);
+              k_block(yb, ch * 8 + b2 * 4 + 2);
+            }
           }
         }
       }
@@ -1170,9 +1223,15 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     if (!fail && !*s_abort && (nchunks == 0 || wait_or_abort(bar(B_MMA2), (uint32_t)((nchunks - 1) & 1), s_abort, a.wait_limit))) {
       tc_fence_after_sync();
       const int c = r128, cr = c & (hd - 1);  // state row, and the row inside its real head's state
-      const size_t out_idx = state_idx(c, a.seg_out);
-      if (a.dtot != nullptr && ch == 0 && c < dh) a.dtot[state_idx(c, 1) * hd + cr] = dsum;
-      const bool last = a.seg_out || seg == a.nseg - 1;  // (each of the two outputs is optional on its own)
+      // (the block's place among the sequences is worked out again: kept across the chunk loop it would cost spills)
+      int blk2 = blockIdx.x;
+      asm volatile("" : "+r"(blk2));
+      const SeqView sv = seq_of_block(a, tab, Hn * a.nsub, MODE == 1 ? 1 : 0, blk2);
+      const int nrun = sv.nseg - (MODE == 1 ? 1 : 0), seg2 = (blk2 / a.nsub) % nrun, hh = blk2 / (a.nsub * nrun);
+      const size_t hr = (pair ? 2 * hh : hh) + (pair ? (c >> 6) : 0);
+      const size_t out_idx = (MODE == 1 ? (size_t)(sv.seg0 + seg2) * a.nsub + blk2 % a.nsub : (size_t)sv.seq) * a.H + hr;
+      if (MODE == 1 && ch == 0 && c < dh) a.dtot[out_idx * hd + cr] = dsum;
+      const bool last = MODE == 1 || seg2 == sv.nseg - 1;  // (each of the two outputs is optional on its own)
       if (a.S_T != nullptr && last) {
         float s[32];
 #pragma unroll 1

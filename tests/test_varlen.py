@@ -50,6 +50,39 @@ def test_packed_sequences_match_the_oracle_one_by_one(dtype, d, with_state):
         assert np.array_equal(r["cache_k"][i:i + 1].float().cpu().numpy(), ref["cache_k"].astype(np.float32))
 
 
+@pytest.mark.gpu
+@pytest.mark.parametrize("d,gate_dim", [(128, 0), (64, 0), (128, 1)])
+def test_many_sequences_share_the_launches(d, gate_dim):
+    """More sequences than one launch's table holds, one long enough to be cut into segments, the others around the chunk
+    length and too short for the chunkwise kernel."""
+    import dataclasses
+    import torch
+    from paper_2509_18467_b200 import api
+    lens = [16, 64, 65, 20 if gate_dim else 1, 0, 2100, 127, 128, 129] + [17 + 5 * (i % 13) for i in range(66)]
+    cu = np.concatenate([[0], np.cumsum(lens)]).tolist()
+    s = I.LayerShape(1, cu[-1], 4, 2, d, d, gate_dim=gate_dim, dtype="bf16", config_id=96)
+    x = I.make(s, NAMES)
+    st = I.make(dataclasses.replace(s, B=len(lens)), ["S0", "z0", "cache_q", "cache_k"])
+    dv = {n: api.to_device(v, "bf16") for n, v in x.items()}
+    ds = {n: api.to_device(v, "f32" if n in ("S0", "z0") else "bf16") for n, v in st.items()}
+    p = api.params(1, s.T, s.H, s.H_kv, d, d, gate_dim=gate_dim)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    n0 = api.launch_count()
+    r = api.lawcat_layer_fwd_varlen(p, cu, *[dv[n] for n in NAMES], ds["cache_q"], ds["cache_k"], ds["S0"], ds["z0"],
+                                    dev_status=status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0 and api.launch_count() - n0 <= 14
+    for i in [0, 1, 2, 3, 5, 6, 7, 8, 9, 40, 73, 74]:
+        lo, hi = cu[i], cu[i + 1]
+        ref = O.layer_fwd(oracle_params(dataclasses.replace(s, T=hi - lo)), *[x[m][:, lo:hi] for m in NAMES[:4]],
+                          *[x[m] for m in NAMES[4:]], *[st[m][i:i + 1] for m in ("cache_q", "cache_k", "S0", "z0")])
+        check(r["o"][:, lo:hi], ref["o"], "bf16", f"o of sequence {i}")
+        check(r["S_T"][i:i + 1], ref["S_T"], "bf16", f"S_T of sequence {i}", f32_store=True)
+        check(r["z_T"][i:i + 1], ref["z_T"], "bf16", f"z_T of sequence {i}", f32_store=True)
+        assert np.array_equal(r["cache_q"][i:i + 1].float().cpu().numpy(), ref["cache_q"].astype(np.float32))
+        assert np.array_equal(r["cache_k"][i:i + 1].float().cpu().numpy(), ref["cache_k"].astype(np.float32))
+
+
 def test_bad_offsets_are_refused_on_the_host():
     import ctypes
     from paper_2509_18467_b200 import api
