@@ -1,4 +1,5 @@
-"""Thin ctypes binding of ``liblawcat.so``: argument marshalling only, every step of the layer runs in the CUDA kernels.
+"""Thin binding of ``liblawcat.so``: argument marshalling only, every step of the layer runs in the CUDA kernels. The tensors of
+a call are turned into pointers by the native module ``_binding``; ctypes serves the rest.
 
 The functions carry the names of the C entry points declared in ``include/lawcat.h`` and take ``torch`` CUDA tensors
 (PyTorch serves as the device allocator and stream provider). Outputs that the caller does not pass are allocated with
@@ -82,6 +83,10 @@ def lib() -> ctypes.CDLL:
         L.lawcat_layer_fwd_host.argtypes = [ctypes.POINTER(Params)] + [ctypes.c_void_p] * 9 + \
                                            [ctypes.c_size_t, ctypes.c_void_p]
         L.lawcat_trace_end.argtypes = [ctypes.c_char_p, ctypes.c_size_t]
+        L.lawcat_gate_fn_workspace_bytes.restype = ctypes.c_size_t
+        L.lawcat_gate_fn_workspace_bytes.argtypes = [ctypes.POINTER(Params), ctypes.c_int32, ctypes.c_int32]
+        L.lawcat_layer_fwd_varlen_workspace_bytes.restype = ctypes.c_size_t
+        L.lawcat_layer_fwd_varlen_workspace_bytes.argtypes = [ctypes.POINTER(Params), ctypes.c_void_p, ctypes.c_int]
         for name, nptr in (("lawcat_conv_fwd", 9), ("lawcat_conv_bwd", 14), ("lawcat_gla_fwd", 10),
                            ("lawcat_gla_bwd", 13), ("lawcat_layer_fwd", 16), ("lawcat_layer_bwd", 19),
                            ("lawcat_decode_step", 12)):
@@ -145,48 +150,61 @@ def _stream(stream):
     return ctypes.c_void_p(s.cuda_stream)
 
 
-def _ws(p: Params, op: int, ws: Optional[torch.Tensor], dev):
-    need = workspace_bytes(p, op)
-    if ws is None and need:
-        ws = torch.empty(need, dtype=torch.uint8, device=dev)
-    return ws, (0 if ws is None else ws.numel() * ws.element_size())
+_binding = None
+_addr = {}
 
 
-def _call(name, p, ptrs, ws, ws_bytes, stream, dev_status):
-    st = getattr(lib(), name)(ctypes.byref(p), *[_ptr(t) for t in ptrs], _ptr(ws), ws_bytes, _stream(stream),
-                              _ptr(dev_status))
+def _bind():
+    """The native marshalling module and the addresses of the entry points; fails loudly when either has not been built."""
+    global _binding
+    L = lib()
+    try:
+        from . import _binding as b
+    except ImportError as e:
+        raise RuntimeError("the native module _binding is missing or does not load: build it with "
+                           f"`python -m paper_2509_18467_b200.build` ({e})") from e
+    for name in EXPORTS:
+        _addr[name] = ctypes.cast(getattr(L, name), ctypes.c_void_p).value
+    _binding = b
+    return b
+
+
+def _call(name, p, op, args, ws, stream, dev_status):
+    """op: the entry point's LAWCAT_OP (its scratch is taken from torch's allocator when ws is None), or None for no scratch."""
+    b = _binding or _bind()
+    if op is None:
+        st = b.call(_addr[name], ctypes.addressof(p), 0, -1, args, ws, stream and stream.cuda_stream, dev_status)
+    else:
+        st = b.call(_addr[name], ctypes.addressof(p), _addr["lawcat_workspace_bytes"], op, args, ws,
+                    stream and stream.cuda_stream, dev_status)
     if st != 0:
         raise LawcatError(st, name)
 
 
+def _empty(like, dtype, *sizes):
+    """Uninitialised tensor on like's device; dtype: F32 or BF16."""
+    return (_binding or _bind()).empty(like, dtype, *sizes)
+
+
 def lawcat_conv_fwd(p: Params, q, k, w_q, w_k, W=None, cache_q=None, cache_k=None, qdot=None, kdot=None, ws=None,
                     stream=None, dev_status=None):
-    dt, dev = torch_dtype(p), q.device
     if qdot is None:
-        qdot = torch.empty(p.B, p.T, p.H, p.d_k, dtype=dt, device=dev)
+        qdot = _empty(q, p.dtype, p.B, p.T, p.H, p.d_k)
     if kdot is None:
-        kdot = torch.empty(p.B, p.T, p.H if W is not None else p.H_kv, p.d_k, dtype=dt, device=dev)
-    ws, nb = _ws(p, OP_CONV_FWD, ws, dev)
-    _call("lawcat_conv_fwd", p, [q, k, w_q, w_k, W, cache_q, cache_k, qdot, kdot], ws, nb, stream, dev_status)
+        kdot = _empty(q, p.dtype, p.B, p.T, p.H if W is not None else p.H_kv, p.d_k)
+    _call("lawcat_conv_fwd", p, OP_CONV_FWD, (q, k, w_q, w_k, W, cache_q, cache_k, qdot, kdot), ws, stream, dev_status)
     return qdot, kdot
 
 
 def lawcat_gate_fn_fwd(p: Params, d_model: int, rank: int, x, A1, A2, bias=None, gate=None, ws=None, stream=None,
                        dev_status=None):
     """x [B,T,d_model], A1 [rank,d_model], A2 [H*gate_dim,rank], bias [H*gate_dim] -> gate logits [B,T,H,gate_dim]."""
-    dt, dev = torch_dtype(p), x.device
     if gate is None:
-        gate = torch.empty(p.B, p.T, p.H, p.gate_dim, dtype=dt, device=dev)
-    f = lib().lawcat_gate_fn_workspace_bytes
-    f.restype = ctypes.c_size_t
-    f.argtypes = [ctypes.POINTER(Params), ctypes.c_int32, ctypes.c_int32]
-    need = f(ctypes.byref(p), d_model, rank)
-    if ws is None and need:
-        ws = torch.empty(need, dtype=torch.uint8, device=dev)
-    nb = 0 if ws is None else ws.numel() * ws.element_size()
-    st = lib().lawcat_gate_fn_fwd(ctypes.byref(p), ctypes.c_int32(d_model), ctypes.c_int32(rank), _ptr(x), _ptr(A1),
-                                  _ptr(A2), _ptr(bias), _ptr(gate), _ptr(ws), ctypes.c_size_t(nb), _stream(stream),
-                                  _ptr(dev_status))
+        gate = _empty(x, p.dtype, p.B, p.T, p.H, p.gate_dim)
+    b = _binding or _bind()
+    need = 0 if ws is not None else lib().lawcat_gate_fn_workspace_bytes(ctypes.byref(p), d_model, rank)
+    st = b.call(_addr["lawcat_gate_fn_fwd"], ctypes.addressof(p), need, -1,
+                (int(d_model), int(rank), x, A1, A2, bias, gate), ws, stream and stream.cuda_stream, dev_status)
     if st != 0:
         raise LawcatError(st, "lawcat_gate_fn_fwd")
     return gate
@@ -194,52 +212,43 @@ def lawcat_gate_fn_fwd(p: Params, d_model: int, rank: int, x, A1, A2, bias=None,
 
 def lawcat_conv_bwd(p: Params, q, k, w_q, w_k, W, d_qdot, d_kdot, cache_q=None, cache_k=None, ws=None, stream=None,
                     dev_status=None):
-    dev = q.device
     dq, dk = torch.empty_like(q), torch.empty_like(k)
-    dw_q = torch.empty(w_q.shape, dtype=torch.float32, device=dev)
-    dw_k = torch.empty(w_k.shape, dtype=torch.float32, device=dev)
-    dW = None if W is None else torch.empty(W.shape, dtype=torch.float32, device=dev)
-    ws, nb = _ws(p, OP_CONV_BWD, ws, dev)
-    _call("lawcat_conv_bwd", p, [q, k, w_q, w_k, W, cache_q, cache_k, d_qdot, d_kdot, dq, dk, dw_q, dw_k, dW], ws,
-          nb, stream, dev_status)
+    dw_q, dw_k = _empty(q, F32, *w_q.shape), _empty(q, F32, *w_k.shape)
+    dW = None if W is None else _empty(q, F32, *W.shape)
+    _call("lawcat_conv_bwd", p, OP_CONV_BWD, (q, k, w_q, w_k, W, cache_q, cache_k, d_qdot, d_kdot, dq, dk, dw_q, dw_k, dW), ws,
+          stream, dev_status)
     return dict(dq=dq, dk=dk, dw_q=dw_q, dw_k=dw_k, dW=dW)
 
 
 def lawcat_gla_fwd(p: Params, qdot, kdot, v, gate, S0=None, z0=None, o=None, want_den=True, want_state=True, ws=None,
                    stream=None, dev_status=None):
-    dt, dev = torch_dtype(p), qdot.device
     if o is None:
-        o = torch.empty(p.B, p.T, p.H, p.d_v, dtype=dt, device=dev)
-    den = torch.empty(p.B, p.T, p.H, dtype=torch.float32, device=dev) if want_den else None
-    S_T = torch.empty(p.B, p.H, p.d_k, p.d_v, dtype=torch.float32, device=dev) if want_state else None
-    z_T = torch.empty(p.B, p.H, p.d_k, dtype=torch.float32, device=dev) if want_state else None
-    ws, nb = _ws(p, OP_GLA_FWD, ws, dev)
-    _call("lawcat_gla_fwd", p, [qdot, kdot, v, gate, S0, z0, o, den, S_T, z_T], ws, nb, stream, dev_status)
+        o = _empty(qdot, p.dtype, p.B, p.T, p.H, p.d_v)
+    den = _empty(qdot, F32, p.B, p.T, p.H) if want_den else None
+    S_T = _empty(qdot, F32, p.B, p.H, p.d_k, p.d_v) if want_state else None
+    z_T = _empty(qdot, F32, p.B, p.H, p.d_k) if want_state else None
+    _call("lawcat_gla_fwd", p, OP_GLA_FWD, (qdot, kdot, v, gate, S0, z0, o, den, S_T, z_T), ws, stream, dev_status)
     return dict(o=o, den=den, S_T=S_T, z_T=z_T)
 
 
 def lawcat_gla_bwd(p: Params, qdot, kdot, v, gate, o, den, dO, S0=None, z0=None, ws=None, stream=None,
                    dev_status=None):
-    dev = qdot.device
     d_qdot, d_kdot, dv, dgate = (torch.empty_like(x) for x in (qdot, kdot, v, gate))
-    ws, nb = _ws(p, OP_GLA_BWD, ws, dev)
-    _call("lawcat_gla_bwd", p, [qdot, kdot, v, gate, S0, z0, o, den, dO, d_qdot, d_kdot, dv, dgate], ws, nb, stream,
+    _call("lawcat_gla_bwd", p, OP_GLA_BWD, (qdot, kdot, v, gate, S0, z0, o, den, dO, d_qdot, d_kdot, dv, dgate), ws, stream,
           dev_status)
     return dict(d_qdot=d_qdot, d_kdot=d_kdot, dv=dv, dgate=dgate)
 
 
 def lawcat_layer_fwd(p: Params, q, k, v, gate, w_q, w_k, W, cache_q=None, cache_k=None, S0=None, z0=None, o=None,
                      want_state=True, want_cache=True, ws=None, stream=None, dev_status=None):
-    dt, dev = torch_dtype(p), q.device
     if o is None:
-        o = torch.empty(p.B, p.T, p.H, p.d_v, dtype=dt, device=dev)
+        o = _empty(q, p.dtype, p.B, p.T, p.H, p.d_v)
     # want_state: True / False, or "S" / "z" for one of the two state outputs alone (each is optional on its own)
-    S_T = torch.empty(p.B, p.H, p.d_k, p.d_v, dtype=torch.float32, device=dev) if want_state in (True, "S") else None
-    z_T = torch.empty(p.B, p.H, p.d_k, dtype=torch.float32, device=dev) if want_state in (True, "z") else None
-    cq = torch.empty(p.B, p.conv_k - 1, p.H * p.d_k, dtype=dt, device=dev) if want_cache else None
-    ck = torch.empty(p.B, p.conv_k - 1, p.H_kv * p.d_k, dtype=dt, device=dev) if want_cache else None
-    ws, nb = _ws(p, OP_LAYER_FWD, ws, dev)
-    _call("lawcat_layer_fwd", p, [q, k, v, gate, w_q, w_k, W, cache_q, cache_k, S0, z0, o, cq, ck, S_T, z_T], ws, nb,
+    S_T = _empty(q, F32, p.B, p.H, p.d_k, p.d_v) if want_state in (True, "S") else None
+    z_T = _empty(q, F32, p.B, p.H, p.d_k) if want_state in (True, "z") else None
+    cq = _empty(q, p.dtype, p.B, p.conv_k - 1, p.H * p.d_k) if want_cache else None
+    ck = _empty(q, p.dtype, p.B, p.conv_k - 1, p.H_kv * p.d_k) if want_cache else None
+    _call("lawcat_layer_fwd", p, OP_LAYER_FWD, (q, k, v, gate, w_q, w_k, W, cache_q, cache_k, S0, z0, o, cq, ck, S_T, z_T), ws,
           stream, dev_status)
     return dict(o=o, cache_q=cq, cache_k=ck, S_T=S_T, z_T=z_T)
 
@@ -248,26 +257,18 @@ def lawcat_layer_fwd_varlen(p: Params, cu_seqlens, q, k, v, gate, w_q, w_k, W, c
                             stream=None, dev_status=None):
     """Packed sequences (B = 1): cu_seqlens is a host sequence of nseq + 1 token offsets. Returns dict(o, cache_q, cache_k,
     S_T, z_T) with the state outputs per sequence."""
-    L = lib()
+    b = _binding or _bind()
     nseq = len(cu_seqlens) - 1
     cu = (ctypes.c_int32 * (nseq + 1))(*[int(x) for x in cu_seqlens])
-    dt, dev = torch_dtype(p), q.device
-    o = torch.empty(1, p.T, p.H, p.d_v, dtype=dt, device=dev)
-    S_T = torch.empty(nseq, p.H, p.d_k, p.d_v, dtype=torch.float32, device=dev)
-    z_T = torch.empty(nseq, p.H, p.d_k, dtype=torch.float32, device=dev)
-    cq = torch.empty(nseq, p.conv_k - 1, p.H * p.d_k, dtype=dt, device=dev)
-    ck = torch.empty(nseq, p.conv_k - 1, p.H_kv * p.d_k, dtype=dt, device=dev)
-    L.lawcat_layer_fwd_varlen_workspace_bytes.restype = ctypes.c_size_t
-    L.lawcat_layer_fwd_varlen_workspace_bytes.argtypes = [ctypes.POINTER(Params), ctypes.c_void_p, ctypes.c_int]
-    need = int(L.lawcat_layer_fwd_varlen_workspace_bytes(ctypes.byref(p), cu, nseq))
-    ws = torch.empty(max(need, 16), dtype=torch.uint8, device=dev)
-    f = L.lawcat_layer_fwd_varlen
-    f.restype = ctypes.c_int
-    f.argtypes = [ctypes.POINTER(Params), ctypes.c_void_p, ctypes.c_int] + [ctypes.c_void_p] * 17 + \
-                 [ctypes.c_size_t, ctypes.c_void_p, ctypes.c_void_p]
-    st = f(ctypes.byref(p), cu, nseq, *[_ptr(t) for t in (q, k, v, gate, w_q, w_k, W, cache_q, cache_k, S0, z0, o, cq, ck,
-                                                          S_T, z_T)], _ptr(ws), ws.numel(), _stream(stream),
-           _ptr(dev_status))
+    o = _empty(q, p.dtype, 1, p.T, p.H, p.d_v)
+    S_T = _empty(q, F32, nseq, p.H, p.d_k, p.d_v)
+    z_T = _empty(q, F32, nseq, p.H, p.d_k)
+    cq = _empty(q, p.dtype, nseq, p.conv_k - 1, p.H * p.d_k)
+    ck = _empty(q, p.dtype, nseq, p.conv_k - 1, p.H_kv * p.d_k)
+    need = lib().lawcat_layer_fwd_varlen_workspace_bytes(ctypes.byref(p), cu, nseq)
+    st = b.call(_addr["lawcat_layer_fwd_varlen"], ctypes.addressof(p), max(need, 16), -1,
+                (ctypes.addressof(cu), nseq, q, k, v, gate, w_q, w_k, W, cache_q, cache_k, S0, z0, o, cq, ck, S_T, z_T), None,
+                stream and stream.cuda_stream, dev_status)
     if st != 0:
         raise LawcatError(st, "lawcat_layer_fwd_varlen")
     return dict(o=o, cache_q=cq, cache_k=ck, S_T=S_T, z_T=z_T)
@@ -276,14 +277,10 @@ def lawcat_layer_fwd_varlen(p: Params, cu_seqlens, q, k, v, gate, w_q, w_k, W, c
 def lawcat_layer_bwd(p: Params, q, k, v, gate, w_q, w_k, W, dO, cache_q=None, cache_k=None, S0=None, z0=None, ws=None,
                      stream=None, dev_status=None):
     """Gradients of the whole layer for the upstream gradient dO: dict(dq, dk, dv, dgate, dw_q, dw_k, dW)."""
-    dev = q.device
     dq, dk, dv, dgate = (torch.empty_like(x) for x in (q, k, v, gate))
-    dw_q = torch.empty(w_q.shape, dtype=torch.float32, device=dev)
-    dw_k = torch.empty(w_k.shape, dtype=torch.float32, device=dev)
-    dW = torch.empty(W.shape, dtype=torch.float32, device=dev)
-    ws, nb = _ws(p, OP_LAYER_BWD, ws, dev)
-    _call("lawcat_layer_bwd", p, [q, k, v, gate, w_q, w_k, W, cache_q, cache_k, S0, z0, dO, dq, dk, dv, dgate, dw_q, dw_k,
-                                  dW], ws, nb, stream, dev_status)
+    dw_q, dw_k, dW = _empty(q, F32, *w_q.shape), _empty(q, F32, *w_k.shape), _empty(q, F32, *W.shape)
+    _call("lawcat_layer_bwd", p, OP_LAYER_BWD, (q, k, v, gate, w_q, w_k, W, cache_q, cache_k, S0, z0, dO, dq, dk, dv, dgate,
+                                                dw_q, dw_k, dW), ws, stream, dev_status)
     return dict(dq=dq, dk=dk, dv=dv, dgate=dgate, dw_q=dw_q, dw_k=dw_k, dW=dW)
 
 
@@ -291,9 +288,8 @@ def lawcat_decode_step(p: Params, q_t, k_t, v_t, gate_t, w_q, w_k, W, S, z, cach
                        stream=None, dev_status=None):
     """S, z, cache_q, cache_k are updated in place; returns o_t [B,H,d_v]."""
     if o_t is None:
-        o_t = torch.empty(p.B, p.H, p.d_v, dtype=torch_dtype(p), device=q_t.device)
-    ws, nb = _ws(p, OP_DECODE_STEP, ws, q_t.device)
-    _call("lawcat_decode_step", p, [q_t, k_t, v_t, gate_t, w_q, w_k, W, S, z, cache_q, cache_k, o_t], ws, nb, stream,
+        o_t = _empty(q_t, p.dtype, p.B, p.H, p.d_v)
+    _call("lawcat_decode_step", p, OP_DECODE_STEP, (q_t, k_t, v_t, gate_t, w_q, w_k, W, S, z, cache_q, cache_k, o_t), ws, stream,
           dev_status)
     return o_t
 
