@@ -1,5 +1,6 @@
 // Recurrent single-token decode (streaming inference, Section 6): the layer at one token with the conv cache of
-// Section 4.1 and the constant-size state of Eq. 4. Two launches:
+// Section 4.1 and the constant-size state of Eq. 4. One launch where decode_one_kernel applies (bf16, d_k = d_v = 64 or 128,
+// conv width up to 4, 1, 2, 4 or 8 query heads per key/value head), else two launches:
 //   decode_features  conv -> shared linear layer -> feature map for the token's query and key, decay alpha = exp(g), the
 //                    normalizer state z (Eq. 8's denominator) advanced in place; writes qdot, kdot, alpha and the
 //                    denominator to the workspace. Two kernels: decode_features_tc_kernel (bf16, d_k = 64 or 128: one
@@ -572,6 +573,172 @@ __global__ void __launch_bounds__(DEC_THREADS, 3) decode_state_kernel(DecodeArgs
   }
 }
 
+// ---- the whole step in one launch -------------------------------------------------------------------------------------------
+// One block per (sequence, query head) does everything: conv, mix, phi, decay, normalizer, state update, read-out, cache shift.
+// A step is a chain of memory round trips in front of one pass over the states, so every global read of the block (W_h, raw
+// rows, taps, gate, z, v and the whole state tile) is issued before anything waits for any of them: one launch and one trip
+// where the two-launch form pays two of each, and nothing of the state's traffic waits for another kernel's features. The G
+// query heads of a key/value head form a cluster: all of them read the key stream's cache, and the first of them shifts it
+// once the cluster has met. W_h is read once per sequence, from L2 after the first.
+// Bound by latency up to about 12 sequences and by HBM beyond. Two launches -> one, 32 heads, us per step:
+//   d = 64:  B = 1 9.8 -> 3.6   B = 16 15.1 -> 6.0   B = 64 29.5 -> 22.1
+//   d = 128: B = 1 11.6 -> 5.0  B = 16 25.6 -> 16.7  B = 64 60.5 -> 58.9 (268 MB of state: 4.6 TB/s)
+// (The state tile as one bulk copy into shared memory, three blocks per SM instead of two: 66 us at B = 64, d = 128.)
+// Thread (row group cg, output octet): 256 / (D / 8) row groups; the mix of both streams in fp32, partial sums over the row
+// groups through shared memory.
+template <int D>
+__global__ void __launch_bounds__(DEC_THREADS) decode_one_kernel(const DecodeArgs a) {
+  using namespace ctc;
+  constexpr int OCT = D / 8, NCG = DEC_THREADS / OCT, RPT = D / NCG;  // octets per row, row groups, W rows per thread
+  constexpr int C4 = D / 4, NRG = DEC_THREADS / C4, NR = D / NRG;     // state: column quads, row groups, rows per thread
+  __shared__ __align__(16) float s_u[2][D], s_alpha[D], s_z[D], s_q[D], s_k[D], s_v[D], s_red[16];
+  __shared__ __align__(16) float s_part[2][NCG][D + 4];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int bh = blockIdx.x, b = bh / a.H, h = bh % a.H, G = a.H / a.Hkv, j = h / G, K = a.K;
+  // ---- every global read
+  const int oc = tid % OCT, cg = tid / OCT;
+  uint4 w[RPT];
+  {
+    const uint4* Wh = reinterpret_cast<const uint4*>((const bf16*)a.W + (size_t)h * D * D) + oc;
+#pragma unroll
+    for (int r = 0; r < RPT; ++r) w[r] = __ldg(Wh + (size_t)(cg * RPT + r) * OCT);
+  }
+  // conv: thread (stream, channel) of the first 2 D threads
+  const int st = tid / D, ch = tid % D;
+  const bool conv_thr = st < 2;
+  bf16 x[4], tap[4];
+  const int NH = st ? a.Hkv : a.H, hd = st ? j : h;
+  bf16* const cache = (bf16*)(st ? a.cache_k : a.cache_q) + ((size_t)b * (K - 1) * NH + hd) * D + ch;  // row r: + r NH D
+  const bf16 zero = __float2bfloat16_rn(0.f);
+#pragma unroll
+  for (int dl = 0; dl < 4; ++dl) {
+    x[dl] = tap[dl] = zero;
+    if (conv_thr && dl < K) {
+      x[dl] = dl == 0 ? ((const bf16*)(st ? a.k_t : a.q_t))[((size_t)b * NH + hd) * D + ch] : cache[(size_t)(K - 1 - dl) * NH * D];
+      tap[dl] = ((const bf16*)(st ? a.w_k : a.w_q))[((size_t)hd * D + ch) * K + dl];
+    }
+  }
+  float graw = 0.f, zold = 0.f, vv = 0.f;
+  if (tid < D) {
+    graw = __bfloat162float(((const bf16*)a.gate_t)[(size_t)bh * a.gd + (a.gd == 1 ? 0 : tid)]);
+    zold = a.z[(size_t)bh * D + tid];
+    vv = __bfloat162float(((const bf16*)a.v_t)[((size_t)b * a.Hkv + j) * D + tid]);
+  }
+  float* const Sbh = a.S + (size_t)bh * D * D;
+  const int e4 = tid % C4, rg = tid / C4;
+  float4 s[NR];
+#pragma unroll
+  for (int i = 0; i < NR; ++i) s[i] = __ldcs(reinterpret_cast<const float4*>(Sbh + (size_t)(rg + NRG * i) * D) + e4);
+  // ---- conv, decay
+  if (conv_thr) {
+    float u = 0.f;
+#pragma unroll
+    for (int dl = 0; dl < 4; ++dl) u = fmaf(__bfloat162float(tap[dl]), __bfloat162float(x[dl]), u);
+    s_u[st][ch] = u;
+  }
+  float alpha = 0.f;
+  if (tid < D) {
+    alpha = expf(log_decay(graw, a.gate_mode, a.inv_tau));
+    s_alpha[tid] = alpha;
+    s_v[tid] = vv;
+  }
+  __syncthreads();
+  // every block of the cluster has its copy of the cache rows: the owners may shift them (the wait is at the shift)
+  asm volatile("barrier.cluster.arrive.aligned;" ::: "memory");
+  // ---- mix
+  {
+    float yq[8], yk[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) yq[i] = yk[i] = 0.f;
+#pragma unroll
+    for (int r = 0; r < RPT; ++r) {
+      float f[8];
+      unpack8b(w[r], f);
+      const float uq = s_u[0][cg * RPT + r], uk = s_u[1][cg * RPT + r];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) { yq[i] = fmaf(uq, f[i], yq[i]); yk[i] = fmaf(uk, f[i], yk[i]); }
+    }
+    store_row8(&s_part[0][cg][oc * 8], yq);
+    store_row8(&s_part[1][cg][oc * 8], yk);
+  }
+  __syncthreads();
+  // ---- phi: warps of stream st own its D outputs, one per thread
+  float y = 0.f;
+  if (conv_thr) {
+#pragma unroll
+    for (int g = 0; g < NCG; ++g) y += s_part[st][g][ch];
+  }
+  constexpr int WPS = D / 32;  // warps per stream
+  if (a.phi == LAWCAT_PHI_SOFTMAX) {
+    float m = conv_thr ? warp_max(y) : 0.f;
+    if (conv_thr && lane == 0) s_red[warp] = m;
+    __syncthreads();
+    if (conv_thr) {
+#pragma unroll
+      for (int i = 0; i < WPS; ++i) m = fmaxf(m, s_red[st * WPS + i]);
+      y = expf(y - m);
+    }
+    const float t = warp_sum(y);
+    if (conv_thr && lane == 0) s_red[8 + warp] = t;
+    __syncthreads();
+    if (conv_thr) {
+      float tot = 0.f;
+#pragma unroll
+      for (int i = 0; i < WPS; ++i) tot += s_red[8 + st * WPS + i];
+      y /= tot;
+    }
+  } else if (a.phi == LAWCAT_PHI_ELU1) {
+    y = y > 0.f ? y + 1.f : expf(y);
+  }
+  if (conv_thr) (st ? s_k : s_q)[ch] = y;
+  __syncthreads();
+  if (tid < D) {
+    const float zn = fmaf(alpha, zold, s_k[tid]);
+    a.z[(size_t)bh * D + tid] = zn;
+    const float t = warp_sum(s_q[tid] * zn);
+    if (lane == 0) s_red[warp] = t;
+  }
+  // ---- state update and read-out
+  float* const s_o = &s_part[0][0][0];  // [NRG][D]: the mix's partial sums have been read
+  {
+    const float4 v4 = *reinterpret_cast<const float4*>(s_v + 4 * e4);
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < NR; ++i) {
+      const int c = rg + NRG * i;
+      const float al = s_alpha[c], kc = s_k[c], qc = s_q[c];
+      s[i].x = fmaf(al, s[i].x, kc * v4.x); s[i].y = fmaf(al, s[i].y, kc * v4.y);
+      s[i].z = fmaf(al, s[i].z, kc * v4.z); s[i].w = fmaf(al, s[i].w, kc * v4.w);
+      __stcs(reinterpret_cast<float4*>(Sbh + (size_t)c * D) + e4, s[i]);
+      acc.x = fmaf(qc, s[i].x, acc.x); acc.y = fmaf(qc, s[i].y, acc.y);
+      acc.z = fmaf(qc, s[i].z, acc.z); acc.w = fmaf(qc, s[i].w, acc.w);
+    }
+    *reinterpret_cast<float4*>(s_o + rg * D + 4 * e4) = acc;
+  }
+  __syncthreads();
+  if (tid < D) {
+    float num = 0.f, den = a.eps;
+#pragma unroll
+    for (int g = 0; g < NRG; ++g) num += s_o[g * D + tid];
+#pragma unroll
+    for (int i = 0; i < WPS; ++i) den += s_red[i];
+    ((bf16*)a.o_t)[(size_t)bh * D + tid] = __float2bfloat16_rn(a.normalize ? num / den : num);
+  }
+  // ---- conv caches: drop the oldest row, append the token (x[] holds token, newest row, ...)
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+  if (conv_thr && (st == 0 || h % G == 0)) {
+#pragma unroll
+    for (int dl = 0; dl < 3; ++dl)
+      if (dl < K - 1) cache[(size_t)(K - 2 - dl) * NH * D] = x[dl];
+  }
+}
+
+// (clusters of 1, 2, 4 or 8 blocks; square states)
+static bool decode_one_supported(const lawcat_params& p) {
+  const int G = p.H / p.H_kv;
+  return decode_tc_supported(p) && p.d_v == p.d_k && G <= 8 && (G & (G - 1)) == 0;
+}
+
 size_t decode_workspace_bytes(const lawcat_params& p) {
   return sizeof(float) * (size_t)p.B * p.H * (3 * (size_t)p.d_k + 1);
 }
@@ -580,6 +747,21 @@ template <typename T>
 static int decode_typed(const Ctx& c, DecodeArgs& a) {
   const lawcat_params& p = *c.p;
   if (p.B * p.H == 0) return LAWCAT_OK;
+  if (std::is_same<T, bf16>::value && decode_one_supported(p)) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(p.B * p.H));
+    cfg.blockDim = dim3(DEC_THREADS);
+    cfg.stream = c.stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)(p.H / p.H_kv);
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    LAWCAT_LAUNCH("decode_one", c.stream, cudaLaunchKernelEx(&cfg, p.d_k == 64 ? decode_one_kernel<64> : decode_one_kernel<128>, a));
+    LAWCAT_CHECK_LAUNCH();
+    return LAWCAT_OK;
+  }
   if (std::is_same<T, bf16>::value && decode_tc_supported(p)) {
     const int r = p.d_k == 64 ? launch_decode_features_tc<64>(c, a) : launch_decode_features_tc<128>(c, a);
     if (r) return r;

@@ -293,3 +293,25 @@ def test_decode_steps_tensor_core_features(api, B, dk, dv, conv_k, gate_dim, kw)
     check(torch.stack(outs, 1), ref["o"], "bf16", "decode o")
     check(S, ref["S_T"], "bf16", "S", f32_store=True)
     check(z, ref["z_T"], "bf16", "z", f32_store=True)
+
+
+@pytest.mark.parametrize("H,Hkv,d,K", [(4, 4, 128, 4), (4, 2, 64, 3), (8, 1, 128, 4), (8, 1, 64, 1), (16, 1, 64, 4), (3, 1, 128, 2)])
+def test_decode_head_groups(api, H, Hkv, d, K):
+    """Every group size of the one-launch decode step (1, 2, 8 query heads per key/value head share the key cache that one of
+    them shifts), and two it does not take (16, 3); three steps, so that the shifted caches are read."""
+    import torch
+    s = shape(5, 3, H, Hkv, d, d, "bf16", conv_k=K, cid=46)
+    x = I.make(s, LAYER_NAMES + ["S0", "z0"] + (["cache_q", "cache_k"] if K > 1 else []))
+    t = dev(api, x, s)
+    S, z, cq, ck = t["S0"].clone(), t["z0"].clone(), t.get("cache_q"), t.get("cache_k")
+    ref = O.layer_fwd(oracle_params(s), *[x[n] for n in LAYER_NAMES], x.get("cache_q"), x.get("cache_k"), x["S0"], x["z0"])
+    api.trace_begin()
+    o = [api.lawcat_decode_step(P(api, s), *[t[n][:, i].contiguous() for n in LAYER_NAMES[:4]], t["w_q"], t["w_k"], t["W"], S, z,
+                                cq, ck) for i in range(3)]
+    assert ("decode_one" in api.trace_end()) == (H // Hkv in (1, 2, 4, 8))
+    check(torch.stack(o, 1), ref["o"], "bf16", "o")
+    check(S, ref["S_T"], "f32", "S")
+    check(z, ref["z_T"], "f32", "z")
+    if K > 1:
+        assert np.array_equal(cq.float().cpu().numpy(), ref["cache_q"].astype(np.float32))
+        assert np.array_equal(ck.float().cpu().numpy(), ref["cache_k"].astype(np.float32))
