@@ -24,9 +24,9 @@
 // its copies land, frees its tensor memory and reports LAWCAT_ERR_TIMEOUT through dev_status.
 //
 // Few tokens (a decode step, a short call; bf16, widths multiples of 8): one block of the tensor-core kernel walks its
-// 64 stages and 32 output tiles one after the other, about 50 us whatever the number of tokens. Up to 1024 tokens
-// gate_fn_small_kernel takes over: one thread block per token (or per four), both layers on the CUDA cores in fp32 with
-// the bottleneck activations in shared memory, every load a 16-byte one and many in flight; the weights come from L2.
+// 64 stages and 32 output tiles one after the other. gate_fn_small_kernel takes over: a cluster of eight blocks per one to
+// eight tokens, both layers on the CUDA cores in fp32, every block an eighth of each layer's weights, every load a 16-byte one
+// and many in flight; the weights come from L2.
 // Above that, while there are fewer token tiles than the SMs hold blocks, the output tiles of a token tile are shared out
 // over several blocks (gridDim.y), each of which repeats the first layer.
 //
@@ -343,86 +343,135 @@ __global__ void __launch_bounds__(256) gate_fn_out_kernel(const float* __restric
 }
 
 // ---------------------------------------------------------------------------------------------------- few tokens
-// One block per TOK tokens, 256 threads. First layer: warp w takes the bottleneck units w, w + 8, ...; its lanes stride
-// over the hidden channels in octets and meet in a shuffle sum. Second layer: a thread takes 8 consecutive outputs at a
-// time (their rows of A2 are contiguous) and keeps TOK x 8 sums.
+constexpr int SMALL_CL = 8;  // blocks per cluster
+
+// Sums v[0..N) over the 32 lanes; afterwards lane l holds the sum of element l / (32 / N) (each step halves what a lane carries).
+template <int N>
+__device__ __forceinline__ float sum_lanes(float (&v)[N], int lane) {
+  int n = N;
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    if (n > 1) {
+      n >>= 1;
+      const bool up = lane & off;
+#pragma unroll
+      for (int i = 0; i < N / 2; ++i)
+        if (i < n) v[i] = (up ? v[i + n] : v[i]) + __shfl_xor_sync(0xffffffffu, up ? v[i] : v[i + n], off);
+    } else {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
+    }
+  }
+  return v[0];
+}
+
+// TOK tokens per cluster: block cr of the cluster takes the cr-th eighth of the hidden width in the first layer and the cr-th
+// eighth of the outputs in the second, so that a cluster reads every weight once, and its blocks exchange the partial sums of
+// the bottleneck activations through distributed shared memory in between. Bound by the latency of one read of each layer's
+// weights from L2 (the second layer's are fetched before the exchange). At the 7B widths and rank 32, 64 tokens: one block per
+// token, reading all 512 KB of weights itself, took 16.6 us; this form takes 6.7 us (one token: 15.6 -> 4.3 us).
 template <int TOK>
-__global__ void __launch_bounds__(256) gate_fn_small_kernel(const bf16* __restrict__ x, const bf16* __restrict__ A1,
+__global__ void __launch_bounds__(256, 2) gate_fn_small_kernel(const bf16* __restrict__ x, const bf16* __restrict__ A1,
                                                             const bf16* __restrict__ A2, const bf16* __restrict__ bias,
                                                             bf16* __restrict__ out, int N, int dm, int rank, int n_out) {
-  extern __shared__ __align__(16) uint8_t sm_small[];
-  uint4* const s_x = reinterpret_cast<uint4*>(sm_small);                           // [TOK][dm / 8] octets of bf16
-  float* const s_h = reinterpret_cast<float*>(sm_small + (size_t)TOK * dm * 2);    // [TOK][rank]
+  extern __shared__ __align__(16) float sm_small[];
+  float* const s_p = sm_small;                // [rank][TOK] this block's part of the sums
+  float* const s_h = sm_small + rank * TOK;   // [TOK][rank]
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int n0 = blockIdx.x * TOK, oct = dm >> 3;
-  for (int i = tid; i < TOK * oct; i += 256) {
-    const int t = i / oct, o = i - t * oct;
-    s_x[i] = n0 + t < N ? __ldg(reinterpret_cast<const uint4*>(x + (size_t)(n0 + t) * dm) + o) : make_uint4(0u, 0u, 0u, 0u);
-  }
-  __syncthreads();
-  // (four units at a time, so that a lane has 16 loads of A1 in flight)
+  const int cr = blockIdx.x % SMALL_CL, n0 = blockIdx.x / SMALL_CL * TOK;
+  const int oct = dm >> 3, o0 = oct * cr / SMALL_CL, o1 = oct * (cr + 1) / SMALL_CL;
+  const int jo = n_out >> 3, j0 = jo * cr / SMALL_CL * 8, j1 = jo * (cr + 1) / SMALL_CL * 8;
+  // the second layer's first rows: thread = two outputs
+  constexpr int PRE = 4;  // octets of a row fetched ahead
+  uint4 pre[2][PRE];
+  const int ro = rank >> 3, jt = j0 + 2 * tid;
+#pragma unroll
+  for (int e = 0; e < 2; ++e)
+#pragma unroll
+    for (int i = 0; i < PRE; ++i)
+      if (jt < j1 && i < ro) pre[e][i] = __ldg(reinterpret_cast<const uint4*>(A2 + (size_t)(jt + e) * rank) + i);
+  // ---- first layer: warp = four units at a time, lane = octet of the block's slice
   for (int r0 = warp; r0 < rank; r0 += 32) {
-    float acc[4][TOK];
+    float acc[4 * TOK];
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-      for (int t = 0; t < TOK; ++t) acc[u][t] = 0.f;
-#pragma unroll 4
-    for (int c = lane; c < oct; c += 32) {
-      uint4 wa[4];
+    for (int i = 0; i < 4 * TOK; ++i) acc[i] = 0.f;
+#pragma unroll 2
+    for (int c = o0 + lane; c < o1; c += 32) {
+      uint4 wa[4], xv[TOK];
 #pragma unroll
       for (int u = 0; u < 4; ++u)
         wa[u] = r0 + 8 * u < rank ? __ldg(reinterpret_cast<const uint4*>(A1 + (size_t)(r0 + 8 * u) * dm) + c)
                                   : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
+      for (int t = 0; t < TOK; ++t)
+        xv[t] = n0 + t < N ? __ldg(reinterpret_cast<const uint4*>(x + (size_t)(n0 + t) * dm) + c) : make_uint4(0u, 0u, 0u, 0u);
+      float fa[4][8];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) ctc::unpack8b(wa[u], fa[u]);
+#pragma unroll
       for (int t = 0; t < TOK; ++t) {
         float fx[8];
-        ctc::unpack8b(s_x[t * oct + c], fx);
+        ctc::unpack8b(xv[t], fx);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          float fa[8];
-          ctc::unpack8b(wa[u], fa);
+        for (int u = 0; u < 4; ++u)
 #pragma unroll
-          for (int i = 0; i < 8; ++i) acc[u][t] = fmaf(fa[i], fx[i], acc[u][t]);
-        }
+          for (int i = 0; i < 8; ++i) acc[u * TOK + t] = fmaf(fa[u][i], fx[i], acc[u * TOK + t]);
       }
     }
+    const float v = sum_lanes<4 * TOK>(acc, lane);
+    const int i = lane / (32 / (4 * TOK)), u = i / TOK, r = r0 + 8 * u;
+    if (lane % (32 / (4 * TOK)) == 0 && r < rank) s_p[r * TOK + i % TOK] = v;
+  }
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  // ---- the cluster's sums: every block adds up all of them
+  for (int i = tid; i < rank * TOK; i += 256) {
+    const uint32_t addr = smem_u32(s_p + i);
+    float v = 0.f;
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
+    for (int k = 0; k < SMALL_CL; ++k) {
+      uint32_t ra;
+      float w;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(addr), "r"(k));
+      asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(w) : "r"(ra) : "memory");
+      v += w;
+    }
+    s_h[(i % TOK) * rank + i / TOK] = v;
+  }
+  // (nobody reads this block's sums after the wait at the end)
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  __syncthreads();
+  // ---- second layer
+  for (int j = jt; j < j1; j += 512) {
+    float acc[TOK][2];
+    const float b0 = bias ? __bfloat162float(bias[j]) : 0.f, b1 = bias ? __bfloat162float(bias[j + 1]) : 0.f;
+#pragma unroll
+    for (int t = 0; t < TOK; ++t) { acc[t][0] = b0; acc[t][1] = b1; }
+    auto step = [&](const uint4& w0, const uint4& w1, int i) {
+      float f0[8], f1[8];
+      ctc::unpack8b(w0, f0);
+      ctc::unpack8b(w1, f1);
 #pragma unroll
       for (int t = 0; t < TOK; ++t) {
-        const float v = warp_sum(acc[u][t]);
-        if (lane == 0 && r0 + 8 * u < rank) s_h[t * rank + r0 + 8 * u] = v;
+        const float4 ha = *reinterpret_cast<const float4*>(s_h + t * rank + 8 * i), hb = *reinterpret_cast<const float4*>(s_h + t * rank + 8 * i + 4);
+        const float hv[8] = {ha.x, ha.y, ha.z, ha.w, hb.x, hb.y, hb.z, hb.w};
+#pragma unroll
+        for (int e = 0; e < 8; ++e) { acc[t][0] = fmaf(f0[e], hv[e], acc[t][0]); acc[t][1] = fmaf(f1[e], hv[e], acc[t][1]); }
       }
-  }
-  __syncthreads();
-  for (int jo = tid; jo * 8 < n_out; jo += 256) {
-    const int j0 = jo * 8;
-    float acc[TOK][8];
-    {
-      float fb[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-      if (bias) ctc::unpack8b(__ldg(reinterpret_cast<const uint4*>(bias + j0)), fb);
+    };
+    const uint4 *r0 = reinterpret_cast<const uint4*>(A2 + (size_t)j * rank), *r1 = r0 + ro;
+    int i0 = 0;
+    if (j == jt) {
 #pragma unroll
-      for (int t = 0; t < TOK; ++t)
-#pragma unroll
-        for (int e = 0; e < 8; ++e) acc[t][e] = fb[e];
+      for (int i = 0; i < PRE; ++i)
+        if (i < ro) step(pre[0][i], pre[1][i], i);
+      i0 = PRE;
     }
 #pragma unroll 4
-    for (int rr = 0; rr < rank; rr += 8) {
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        float fa[8];
-        ctc::unpack8b(__ldg(reinterpret_cast<const uint4*>(A2 + (size_t)(j0 + e) * rank + rr)), fa);
-#pragma unroll
-        for (int t = 0; t < TOK; ++t)
-#pragma unroll
-          for (int i = 0; i < 8; ++i) acc[t][e] = fmaf(fa[i], s_h[t * rank + rr + i], acc[t][e]);
-      }
-    }
+    for (int i = i0; i < ro; ++i) step(__ldg(r0 + i), __ldg(r1 + i), i);
 #pragma unroll
     for (int t = 0; t < TOK; ++t)
-      if (n0 + t < N) *reinterpret_cast<uint4*>(out + (size_t)(n0 + t) * n_out + j0) = ctc::pack8bf16(acc[t]);
+      if (n0 + t < N) *reinterpret_cast<uint32_t*>(out + (size_t)(n0 + t) * n_out + j) = pack_bf16(acc[t][0], acc[t][1]);
   }
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 // ---------------------------------------------------------------------------------------------------- host side
@@ -495,14 +544,24 @@ static int launch_tc(const Ctx& c, int d_model, const void* x, const void* A1, c
 template <int TOK>
 static int launch_small(const Ctx& c, int d_model, int rank, const void* x, const void* A1, const void* A2,
                         const void* bias, void* gate, size_t N, int n_out) {
-  const size_t smem = (size_t)TOK * d_model * 2 + sizeof(float) * (size_t)TOK * rank;
+  const size_t smem = 2 * sizeof(float) * (size_t)TOK * rank;
   if (smem > 48 * 1024 &&
       cudaFuncSetAttribute(gate_fn_small_kernel<TOK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return LAWCAT_ERR_CUDA;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((N + TOK - 1) / TOK) * SMALL_CL);
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = c.stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = SMALL_CL;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
   LAWCAT_LAUNCH("gate_fn_small", c.stream,
-                gate_fn_small_kernel<TOK><<<(unsigned)((N + TOK - 1) / TOK), 256, smem, c.stream>>>(
-                    (const bf16*)x, (const bf16*)A1, (const bf16*)A2, (const bf16*)bias, (bf16*)gate, (int)N, d_model, rank,
-                    n_out));
+                cudaLaunchKernelEx(&cfg, gate_fn_small_kernel<TOK>, (const bf16*)x, (const bf16*)A1, (const bf16*)A2,
+                                   (const bf16*)bias, (bf16*)gate, (int)N, d_model, rank, n_out));
   LAWCAT_CHECK_LAUNCH();
   return LAWCAT_OK;
 }
@@ -533,17 +592,20 @@ bool gate_fn_tc_supported(const lawcat_params& p, int d_model, int rank) {
          n_out % 8 == 0 && p.chunk != 1;
 }
 
-// Few tokens: the latency-oriented CUDA-core kernel (see the head of this file). SMALL_1: tokens up to which one block per
-// token is used, SMALL_4: up to which one block per four tokens; beyond, the tensor-core kernel where it applies.
-constexpr size_t SMALL_1 = 128, SMALL_4 = 1024;
-// tokens per block of the few-token kernel for this call, 0 = not its case
+// Few tokens: the latency-oriented CUDA-core kernel (see the head of this file) while its arithmetic is small: it loses to the
+// tensor-core kernel, whose 26 us at the 7B widths hardly depend on the number of tokens up to 3000, at about 256 tokens of
+// rank 32 there (12.9 us; 512 tokens 25.1), and in proportion to rank and widths elsewhere. Where the tensor-core kernel does
+// not apply it serves up to 1024 tokens.
+constexpr size_t SMALL_MAX = 1024, SMALL_WORK = (size_t)256 * 32 * 8192;
+// tokens per cluster for this call, 0 = not its case: as few as keep the call at 32 clusters, which are resident together
+// (64 tokens at the 7B widths: 6.7 us with 2 tokens per cluster, 8.4 with 4, 11.0 with 1)
 static int gate_fn_small_tok(const lawcat_params& p, int d_model, int rank) {
   const long long n_out = (long long)p.H * p.gate_dim;
   const size_t N = (size_t)p.B * p.T;
   if (p.dtype != LAWCAT_BF16 || rank % 8 != 0 || d_model % 8 != 0 || n_out % 8 != 0 || p.chunk == 1) return 0;
-  if (N <= SMALL_1) return 1;
-  if (N <= SMALL_4 && d_model <= 8192) return 4;
-  return 0;
+  if (N > SMALL_MAX) return 0;
+  if (gate_fn_tc_supported(p, d_model, rank) && N * rank * ((size_t)d_model + (size_t)n_out) > SMALL_WORK) return 0;
+  return N <= 8 ? 1 : N <= 64 ? 2 : N <= 128 ? 4 : 8;
 }
 
 size_t gate_fn_workspace_bytes(const lawcat_params& p, int d_model, int rank) {
@@ -560,7 +622,9 @@ int launch_gate_fn(const Ctx& c, int d_model, int rank, const void* x, const voi
   if (N == 0) return LAWCAT_OK;
   switch (gate_fn_small_tok(p, d_model, rank)) {
     case 1: return gfn::launch_small<1>(c, d_model, rank, x, A1, A2, bias, gate, N, n_out);
+    case 2: return gfn::launch_small<2>(c, d_model, rank, x, A1, A2, bias, gate, N, n_out);
     case 4: return gfn::launch_small<4>(c, d_model, rank, x, A1, A2, bias, gate, N, n_out);
+    case 8: return gfn::launch_small<8>(c, d_model, rank, x, A1, A2, bias, gate, N, n_out);
     default: break;
   }
   if (gate_fn_tc_supported(p, d_model, rank)) {

@@ -160,3 +160,11 @@ def test_empty_and_invalid_calls():
     with pytest.raises(api.LawcatError) as e:                 # a weight pointer off the 16-byte grid
         api.lawcat_gate_fn_fwd(p, 64, 16, x, buf[4:4 + 16 * 64], A2)
     assert e.value.status == 1
+
+
+@pytest.mark.parametrize("N", [1, 8, 9, 64, 65, 127, 129, 256])
+@pytest.mark.parametrize("rank,H,dm", [(8, 1, 72), (32, 3, 520), (40, 9, 200), (16, 1, 4096)])
+def test_clusters_of_the_few_tokens_kernel(N, rank, H, dm):
+    """Every number of tokens per cluster (1, 2, 4, 8) at its edges; widths that eight blocks share unevenly."""
+    got, want = run(1, N, H, 64, 0, dm, rank, expect_tc=False, expect_kernel="gate_fn_small", cfg=960)
+    assert err_bf16(got, want)[1] <= 1e-4
