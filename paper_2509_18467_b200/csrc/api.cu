@@ -53,11 +53,6 @@ int validate_params(const lawcat_params* p, bool need_T) { return check_params(p
 extern "C" size_t lawcat_workspace_bytes(const lawcat_params* p, int op);
 
 namespace {
-// whether the fused layer backward runs on the tensor-core kernels (fp32 features between its stages)
-bool layer_bwd_tc(const lawcat_params& p) {
-  return p.chunk != 1 && gla_tc_bwd_supported(p) && convmix_tc_fwd_supported(p) && convmix_tc_bwd_supported(p);
-}
-
 __global__ void widen_kernel(const bf16* __restrict__ x, float* __restrict__ y, size_t n) {
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) y[i] = __bfloat162float(x[i]);
@@ -97,11 +92,7 @@ ExactBwdLayout exact_bwd_layout(const lawcat_params* p) {
 }
 
 size_t layer_bwd_workspace(const lawcat_params* p) {
-  if (layer_bwd_tc(*p)) {
-    // fp32 features and their gradients between the stages, then the scratch of the attention and the conv backward
-    return 4 * align_up(4 * elems(p, p->H, p->d_k), 256) + lawcat_workspace_bytes(p, LAWCAT_OP_GLA_BWD) +
-           lawcat_workspace_bytes(p, LAWCAT_OP_CONV_BWD);
-  }
+  if (layer_bwd_tc_supported(*p)) return layer_bwd_tc_workspace_bytes(*p);
   return exact_bwd_layout(p).total;
 }
 }  // namespace
@@ -354,17 +345,8 @@ int lawcat_layer_bwd(const lawcat_params* p, const void* q, const void* k, const
   const size_t need = lawcat_workspace_bytes(p, LAWCAT_OP_LAYER_BWD);
   if (need && (!ws || ws_bytes < need)) return LAWCAT_ERR_WORKSPACE_TOO_SMALL;
   Ctx c{p, (cudaStream_t)stream, dev_status};
-  if ((size_t)p->B * p->T != 0 && layer_bwd_tc(*p)) {
-    char* w = (char*)ws;
-    const size_t nf = align_up(4 * elems(p, p->H, p->d_k), 256);
-    void* qd = w; void* kd = w + nf; void* dqd = w + 2 * nf; void* dkd = w + 3 * nf;
-    void* ws_g = w + 4 * nf;
-    void* ws_c = (char*)ws_g + lawcat_workspace_bytes(p, LAWCAT_OP_GLA_BWD);
-    // features recomputed in fp32, attention backward on them (it runs its own forward sweep), mix / softmax / conv backward
-    if ((r = launch_convmix_tc_fwd(c, q, k, w_q, w_k, W, cache_q, cache_k, qd, kd, true))) return r;
-    if ((r = launch_gla_bwd_tc(c, qd, kd, v, gate, S0, z0, dO, dqd, dkd, dv, dgate, ws_g, true))) return r;
-    return launch_conv_bwd(c, q, k, w_q, w_k, W, cache_q, cache_k, dqd, dkd, dq, dk, dw_q, dw_k, dW, ws_c, true);
-  }
+  if (layer_bwd_tc_supported(*p))
+    return launch_layer_bwd_tc(c, q, k, v, gate, w_q, w_k, W, cache_q, cache_k, S0, z0, dO, dq, dk, dv, dgate, dw_q, dw_k, dW, ws);
   // exact kernels, the whole chain in fp32
   const ExactBwdLayout L = exact_bwd_layout(p);
   char* w = (char*)ws;

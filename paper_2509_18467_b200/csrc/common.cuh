@@ -107,6 +107,16 @@ int launch_convmix_tc_bwd(const Ctx& c, const void* q, const void* k, const void
                           const void* cache_q, const void* cache_k, const void* d_qdot, const void* d_kdot, bool grads_f32,
                           float* du_q, float* du_k, float* dW);
 
+// The whole layer's backward on the tensor cores (layer_bwd_tc.cu), and the conv's own backward that ends it (conv.cu).
+bool layer_bwd_tc_supported(const lawcat_params& p);
+size_t layer_bwd_tc_workspace_bytes(const lawcat_params& p);
+int launch_layer_bwd_tc(const Ctx& c, const void* q, const void* k, const void* v, const void* gate, const void* w_q,
+                        const void* w_k, const void* W, const void* cache_q, const void* cache_k, const float* S0,
+                        const float* z0, const void* dO, void* dq, void* dk, void* dv, void* dgate, float* dw_q, float* dw_k,
+                        float* dW, void* ws);
+int launch_conv_only_bwd(const Ctx& c, const void* q, const void* k, const void* w_q, const void* w_k, const void* cache_q,
+                         const void* cache_k, const float* du_q, const float* du_k, void* dq, void* dk, float* dw_q, float* dw_k);
+
 // The gate function in front of the layer: two consecutive low-rank linear layers producing the gate logits (gate_fn.cu).
 bool gate_fn_tc_supported(const lawcat_params& p, int d_model, int rank);
 size_t gate_fn_workspace_bytes(const lawcat_params& p, int d_model, int rank);

@@ -514,6 +514,14 @@ int launch_conv_bwd(const Ctx& c, const void* q, const void* k, const void* w_q,
   return conv_bwd_typed<bf16>(c, q, k, w_q, w_k, W, cache_q, cache_k, d_qdot, d_kdot, dq, dk, dw_q, dw_k, dW, ws, grads_f32);
 }
 
+// the conv's own backward alone, on fp32 gradients of both conv outputs (bf16 storage)
+int launch_conv_only_bwd(const Ctx& c, const void* q, const void* k, const void* w_q, const void* w_k, const void* cache_q,
+                         const void* cache_k, const float* du_q, const float* du_k, void* dq, void* dk, float* dw_q, float* dw_k) {
+  const int r = conv_bwd_stream<bf16, float>(c, du_q, (const bf16*)q, (const bf16*)w_q, (const bf16*)cache_q, (bf16*)dq, dw_q, c.p->H);
+  if (r) return r;
+  return conv_bwd_stream<bf16, float>(c, du_k, (const bf16*)k, (const bf16*)w_k, (const bf16*)cache_k, (bf16*)dk, dw_k, c.p->H_kv);
+}
+
 // ------------------------------------------------------------------------------------------------ conv cache out
 // cache_out[b,r,:] = token T-(K-1)+r of the stream [cache_in, x] (Section 4.1: the cache is bounded by the kernel size)
 template <typename T>

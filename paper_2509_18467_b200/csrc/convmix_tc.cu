@@ -33,10 +33,6 @@ struct CArgs {
   int unshared;  // 1: W is [2,H,D,D], the key stream mixes with the second set (forward kernel only)
 };
 
-// hint: fetch the 128-byte line at p towards L2 (these kernels walk their tiles in lock-step; the hint lets the next
-// tile's rows travel while the current one is computed)
-__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
-
 // raw rows [t0 - HALO, t0 + TT) of one head into shared memory (rows before the sequence come from the conv cache or are
 // zero, rows past its end are zero), and the head's taps as fp32 [D][4] (zero beyond the conv width)
 template <int D>
@@ -96,52 +92,6 @@ __device__ __forceinline__ void conv_tile(const uint8_t* s_raw, const float* s_w
       *reinterpret_cast<uint4*>(s_ul + toff(L::SLAB_U, r, o * 8)) = pack8f16(lo);
     }
   }
-}
-
-// conv of 8 channels (octet o) of N consecutive tokens from t on, straight from global memory with a window of raw rows
-// (rows before the sequence come from the conv cache or are zero, rows past its end are zero); emit(i, u) takes token t + i.
-// s_w: the head's taps, fp32 [D][4], in shared memory.
-template <int D, int N, typename F>
-__device__ __forceinline__ void conv_run(const bf16* x, const bf16* cache, const float* s_w, int b, int t, int T, int NH,
-                                         int head, int K, int o, F emit) {
-  uint4 raw[N + HALO];
-#pragma unroll
-  for (int i = 0; i < N + HALO; ++i) {
-    const int tt = t - HALO + i;
-    raw[i] = make_uint4(0u, 0u, 0u, 0u);
-    if (tt >= 0 && tt < T)
-      raw[i] = *reinterpret_cast<const uint4*>(x + (((size_t)b * T + tt) * NH + head) * D + o * 8);
-    else if (tt < 0 && cache != nullptr && tt + (K - 1) >= 0)
-      raw[i] = *reinterpret_cast<const uint4*>(cache + (((size_t)b * (K - 1) + tt + (K - 1)) * NH + head) * D + o * 8);
-  }
-  float w[8][4];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const float4 t4 = *reinterpret_cast<const float4*>(s_w + (o * 8 + i) * 4);
-    w[i][0] = t4.x; w[i][1] = t4.y; w[i][2] = t4.z; w[i][3] = t4.w;
-  }
-#pragma unroll
-  for (int i = 0; i < N; ++i) {
-    float u[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-    for (int dl = 0; dl < 4; ++dl) {
-      float xv[8];
-      unpack8b(raw[i + HALO - dl], xv);
-#pragma unroll
-      for (int c = 0; c < 8; ++c) u[c] = fmaf(w[c][dl], xv[c], u[c]);
-    }
-    emit(i, u);
-  }
-}
-
-// v rounded to bf16, and v -= the rounded value
-__device__ __forceinline__ uint4 take_bf16(float* v) {
-  const uint4 p = pack8bf16(v);
-  float h[8];
-  unpack8b(p, h);
-#pragma unroll
-  for (int i = 0; i < 8; ++i) v[i] -= h[i];
-  return p;
 }
 
 // Forward. 256 threads walk one (batch, query head, tile of 128 tokens), query stream then key stream. bf16 outputs take

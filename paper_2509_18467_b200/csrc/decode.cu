@@ -591,7 +591,7 @@ __global__ void __launch_bounds__(DEC_THREADS) decode_one_kernel(const DecodeArg
   using namespace ctc;
   constexpr int OCT = D / 8, NCG = DEC_THREADS / OCT, RPT = D / NCG;  // octets per row, row groups, W rows per thread
   constexpr int C4 = D / 4, NRG = DEC_THREADS / C4, NR = D / NRG;     // state: column quads, row groups, rows per thread
-  __shared__ __align__(16) float s_u[2][D], s_alpha[D], s_z[D], s_q[D], s_k[D], s_v[D], s_red[16];
+  __shared__ __align__(16) float s_u[2][D], s_alpha[D], s_q[D], s_k[D], s_v[D], s_red[16];
   __shared__ __align__(16) float s_part[2][NCG][D + 4];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int bh = blockIdx.x, b = bh / a.H, h = bh % a.H, G = a.H / a.Hkv, j = h / G, K = a.K;

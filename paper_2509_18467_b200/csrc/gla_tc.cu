@@ -36,12 +36,14 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "octet_tile.cuh"
 #include "tc_common.cuh"
 
 namespace lawcat {
 namespace gtc {
 
 using namespace tc;
+using namespace ctc;
 
 #ifdef LAWCAT_TIMELINE
 __device__ long long g_gla_timeline[32];
@@ -114,65 +116,6 @@ struct GArgs {
   int B, T, H, Hkv, gate_dim, gate_mode, normalize;
   float inv_tau, eps;
 };
-
-__device__ __forceinline__ uint32_t toff(uint32_t slab, int r, int c) { return (uint32_t)(c >> 3) * slab + (uint32_t)r * 16u + (uint32_t)(c & 7) * 2u; }
-// K-major view (rows = M or N, columns = K) and MN-major view (rows = K, columns = M or N) of a tile
-__device__ __forceinline__ uint64_t kview(uint32_t addr, uint32_t slab) { return smem_desc(addr, slab, 128, LAYOUT_NONE); }
-__device__ __forceinline__ uint64_t mview(uint32_t addr, uint32_t slab) { return smem_desc(addr, 128, slab, LAYOUT_NONE); }
-__device__ __forceinline__ uint64_t dadv(uint64_t d, uint32_t bytes) {
-  return (d & 0xFFFFFFFF00000000ull) | (uint64_t)((uint32_t)d + (bytes >> 4));
-}
-__device__ __forceinline__ float log2_sigmoid(float a) {
-  const float x = -a * 1.4426950408889634f;
-  return -fmaxf(x, lg2f(1.f + ex2f(fminf(x, 126.f))));
-}
-__device__ __forceinline__ uint4 pack8h(const float* v, bool f16) {
-  return f16 ? make_uint4(pack_f16(v[0], v[1]), pack_f16(v[2], v[3]), pack_f16(v[4], v[5]), pack_f16(v[6], v[7]))
-             : make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
-}
-// 16-bit values back to fp32
-__device__ __forceinline__ void unpack8h(const uint4& v, bool f16, float* f) {
-  if (f16) {
-    const __half2* h = reinterpret_cast<const __half2*>(&v);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const float2 x = __half22float2(h[i]);
-      f[2 * i] = x.x; f[2 * i + 1] = x.y;
-    }
-  } else {
-    f[0] = bf16_lo(v.x); f[1] = bf16_hi(v.x); f[2] = bf16_lo(v.y); f[3] = bf16_hi(v.y);
-    f[4] = bf16_lo(v.z); f[5] = bf16_hi(v.z); f[6] = bf16_lo(v.w); f[7] = bf16_hi(v.w);
-  }
-}
-// v = hi + lo with hi the 16-bit rounding of v and lo the 16-bit rounding of the rest
-__device__ __forceinline__ void split8h(const float* v, bool f16, uint4& hi, uint4& lo) {
-  hi = pack8h(v, f16);
-  float h[8], r[8];
-  unpack8h(hi, f16, h);
-#pragma unroll
-  for (int i = 0; i < 8; ++i) r[i] = v[i] - h[i];
-  lo = pack8h(r, f16);
-}
-__device__ __forceinline__ void unpack8b(const uint4& v, float* f) {
-  f[0] = bf16_lo(v.x); f[1] = bf16_hi(v.x); f[2] = bf16_lo(v.y); f[3] = bf16_hi(v.y);
-  f[4] = bf16_lo(v.z); f[5] = bf16_hi(v.z); f[6] = bf16_lo(v.w); f[7] = bf16_hi(v.w);
-}
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
-  uint32_t r[8];
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-               : "r"(taddr)
-               : "memory");
-#pragma unroll
-  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
-}
-__device__ __forceinline__ void tmem_st8(uint32_t taddr, const float* v) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
-               ::"r"(taddr), "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])),
-                 "r"(__float_as_uint(v[3])), "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])),
-                 "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7]))
-               : "memory");
-}
 
 // MODE 0: the forward (o, den, S_T, z_T). The backward is two launches: MODE 1, the forward sweep for the scratch quantities
 // (state operand of every chunk, 1 / den, dO . o, the scale of do'), two thread blocks per SM; MODE 2, the reverse sweep. In

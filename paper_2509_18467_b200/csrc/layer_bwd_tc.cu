@@ -1,0 +1,1075 @@
+// The attention part of the whole layer's backward (lawcat_layer_bwd; Section 5.1's distillation step) on the tensor cores,
+// bf16 storage, d_k = d_v = 64 or 128, softmax feature map. The features qdot, kdot come in fp32 from the recomputed conv +
+// mix; what goes out towards the mix is not their gradients but the products
+//     wq = qdot * dqdot,   wk = kdot * dkdot   (elementwise)
+// because that is all the softmax Jacobian needs (dy = w - p sum(w)) and all the gate gradient needs (dg_s = sum_{t>=s} wq_t -
+// wk_t): the decay factors 2^{+-x} of the chunkwise form cancel in them and never have to be undone.
+//
+// With b_t the running sum of the log2-decays inside a chunk of C = 64 tokens, m = 31, x_t = b_t - b_m, bm = b_m, ft = b_C - b_m:
+//   qs_t = qdot_t 2^{x_t},  ks_i = kdot_i 2^{-x_i},  S16 = 2^bm S (S the state in front of the chunk, z its normalizer column)
+//   forward sweep   P = mask(qs ks^T)    num | den = P [v|1] + qs [S16|z16]    W <- S16 + ks^T [v|1]   (next state = 2^ft W)
+//                   inv_t = 1 / den_t, delta_t = dO_t . o_t; the operand S16 of every chunk is kept for the reverse sweep
+//   reverse sweep   qn_t = qs_t inv_t      P' = mask(qn ks^T)      E = mask(dO v^T - delta_t)
+//                   dQ = E ks + dO S16^T - delta z16             wq = qn * dQ
+//                   dK = E^T qn + v R16^T + r16                  wk = ks * dK      (R16 = 2^ft R, R the adjoint of the state
+//                   dV = P'^T dO + ks R16                                           behind the chunk, r its normalizer column)
+//                   W' <- R16 + qn^T dO  (adjoint in front of the chunk = 2^bm W')   r likewise with -delta
+// Dividing by den is folded into qn and into the row terms, so dO and v enter every product unrounded (both are exact in 16
+// bits); qn, ks, S16, R16, P' and E are two-term 16-bit pairs hi + lo (hi hi + lo hi + hi lo: about 21 bits). Powers of two keep
+// the pairs in the fp16 range and away from its subnormals: 2^kap on ks and S16 (per chunk, from a bound on the state), 2^al on
+// inv (per chunk, from its largest inv and the largest adjoint entry), 2^sc on dO (per head). Chunks whose decay exponents leave
+// +-8 use bf16 pairs.
+//
+// One thread block walks one (batch, query head), lock-step: every phase of a chunk by all threads, products by one thread
+// (tcgen05.mma, fp32 accumulators in tensor memory), bounded waits on mbarriers. What bounds it is that chain of phases:
+// instruction issue in the operand and epilogue passes, the products second. Head width 64: two blocks per SM (<= 113 KB, 256
+// tensor memory columns); 128: one block of 512 threads.
+#include <cuda.h>
+#include <cuda_fp16.h>
+
+#include <mutex>
+
+#include "common.cuh"
+#include "octet_tile.cuh"
+#include "tc_common.cuh"
+
+namespace lawcat {
+namespace lbt {
+
+using namespace tc;
+using namespace ctc;
+
+constexpr int C = 64, MID = 31;
+constexpr float RMAX_F16 = 8.f;
+constexpr int QSC = 4;       // power of two on qs in the forward sweep
+constexpr int KAP_MAX = 4;   // largest power of two on ks and S16 (ks <= 2^8 in fp16 chunks)
+
+struct Args {
+  const float *qd, *kd;                 // [B,T,H,D] features
+  const bf16 *v, *gate, *dO;
+  const float *S0, *z0;
+  float *wq, *wk;                       // [B,T,H,D]
+  float* dvh;                           // [B,T,H,D] per-head dv, reduced over the heads of a group afterwards
+  bf16* dgate;
+  float *inv, *delta;                   // [B,T,H]
+  float* domax;                         // [B*H] largest |dO| of the head
+  float* z16;                           // [B*H][chunks][D]
+  int* meta;                            // [B*H][chunks][2]: kap, operand format
+  uint8_t* s16;                         // [B*H][chunks][2 * D * D * 2] operand tiles, hi then lo
+  int* wmax;                            // [1] largest |wq|, |wk| of the call as float bits (caller-zeroed)
+  int* dev_status;
+  int B, T, H, Hkv, gate_dim, gate_mode, normalize;
+  float inv_tau, eps;
+};
+
+template <int D>
+struct Cfg {
+  static constexpr int THREADS = D == 128 ? 512 : 256, OCT = D / 8, NCG = THREADS / 128;  // NCG: column groups of row threads
+  static constexpr uint32_t SL_T = C * 16 + 16;  // slab stride of token tiles written eight lanes to a row (padded: the slabs
+                                                 // then start in different banks)
+  static constexpr uint32_t SL_U = C * 16;       // ... of token tiles written a lane to a row
+  static constexpr uint32_t SL_C = D * 16;       // ... of tiles with D rows
+  static constexpr uint32_t T_TOK = OCT * SL_T, T_P = 8 * SL_U, T_C = OCT * SL_C;
+  // forward sweep
+  static constexpr uint32_t F_QS = 0, F_KS = F_QS + 2 * T_TOK, F_V = F_KS + 2 * T_TOK, F_PM = F_V + (OCT + 2) * SL_T;
+  static constexpr uint32_t F_S = F_PM + 2 * T_P, T_SZ = (OCT + 2) * SL_C, F_VEC = F_S + 2 * T_SZ;
+  static constexpr uint32_t F_BYTES = F_VEC + 4 * D * 4 + NCG * C * 4 + 64;
+  static constexpr uint32_t F_X = F_S;           // exponents, fp32 [C][D]: dead before the state operand is written
+  // reverse sweep
+  static constexpr uint32_t R_QS = 0, R_KS = R_QS + 2 * T_TOK, R_V = R_KS + 2 * T_TOK, R_DO = R_V + T_TOK, R_PM = R_DO + T_TOK;
+  static constexpr uint32_t R_E = R_PM + 2 * T_P, R_S = R_E + 2 * T_P, R_VEC = R_S + 2 * T_C;
+  static constexpr uint32_t R_BYTES = R_VEC + 8 * D * 4 + 2 * C * 4 + (THREADS / 32) * D * 4 + 96;
+  static constexpr uint32_t R_X = R_S;
+  // fp32 [C][D] result tiles over operands that are dead by then
+  static constexpr uint32_t R_WQ = R_S, R_WK = D == 128 ? R_S + C * D * 4 : R_PM, R_DV = D == 128 ? R_PM : R_E, R_DG = R_QS;
+  static_assert(C * D * 4 <= 2 * T_SZ && C * D * 4 <= 2 * T_TOK && 2 * T_P >= C * 64 * 4, "aliases");
+  static_assert(R_BYTES <= (D == 128 ? 232448 : 115000) && F_BYTES <= (D == 128 ? 232448 : 115000), "shared memory budget");
+  // tensor memory
+  static constexpr uint32_t F_ST = 0, F_O = D + 16, F_P = 2 * (D + 16), COLS = D == 128 ? 512 : 256;
+  static constexpr uint32_t R_R = 0, R_DQ = D, R_DK = 2 * D, R_DVC = 3 * D, R_P = R_DQ, R_EP = R_DQ + 64;
+};
+
+__device__ __forceinline__ float pow2i(int e) { return __int_as_float((min(max(e, -126), 127) + 127) << 23); }
+// smallest e with |x| < 2^e (x > 0)
+__device__ __forceinline__ int exp_above(float x) { return ((__float_as_int(x) >> 23) & 0xff) - 126; }
+// piece pc (16 bytes) of row r of an fp32 [C][D] tile, swizzled so that lanes that own rows spread over the banks
+template <int D>
+__device__ __forceinline__ uint32_t foff(int r, int pc) { return (uint32_t)(r * (D * 4) + ((pc ^ (r & 7)) << 4)); }
+
+// Log-decays of a chunk scanned outwards from the middle token: exponents x into s_x (fp32, rows of D), bm and ft per channel,
+// the largest |x| into *rmax. Ends with a barrier; the caller has one between the last readers of s_x and this call.
+template <int D>
+__device__ __forceinline__ void gate_pass(const Args& a, size_t row0, int h, int nvalid, float* s_x, float* s_bm, float* s_ft,
+                                          int* rmax, int tid) {
+  using F = Cfg<D>;
+  const float L2E = 1.4426950408889634f;
+  if (tid == 0) *rmax = 0;
+  for (int idx = tid; idx < C * F::OCT; idx += F::THREADS) {
+    const int o = idx % F::OCT, r = idx / F::OCT;
+    float g[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (r < nvalid) {
+      const size_t gi = (row0 + r) * a.H + h;
+      if (a.gate_dim == 1) {
+        const float av = __bfloat162float(a.gate[gi]);
+        const float gv = a.gate_mode == LAWCAT_GATE_LOGDECAY ? av * L2E : log2_sigmoid(av) * a.inv_tau;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) g[i] = gv;
+      } else {
+        unpack8b(*reinterpret_cast<const uint4*>(a.gate + gi * D + o * 8), g);
+        if (a.gate_mode == LAWCAT_GATE_LOGDECAY) {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) g[i] *= L2E;
+        } else {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) g[i] = log2_sigmoid(g[i]) * a.inv_tau;
+        }
+      }
+    }
+    store_row8(s_x + r * D + o * 8, g);
+  }
+  __syncthreads();
+  if (tid < 2 * D) {
+    const int c = tid & (D - 1), gh = tid / D;
+    float g[32], acc = 0.f;
+#pragma unroll
+    for (int i = 0; i < 32; ++i) g[i] = s_x[(gh * 32 + i) * D + c];
+    if (gh) {
+#pragma unroll
+      for (int i = 0; i < 32; ++i) {
+        acc += g[i];
+        s_x[(32 + i) * D + c] = fmaxf(acc, -120.f);
+      }
+      s_ft[c] = acc;
+    } else {
+      s_x[MID * D + c] = 0.f;
+#pragma unroll
+      for (int i = MID - 1; i >= 0; --i) {
+        acc += g[i + 1];
+        s_x[i * D + c] = fminf(-acc, 120.f);
+      }
+      s_bm[c] = acc + g[0];
+    }
+    if (-acc > 120.f && a.dev_status) atomicMax(a.dev_status, (int)LAWCAT_ERR_NUMERIC);
+    const float am = warp_max(-acc);
+    if ((tid & 31) == 0) atomicMax(rmax, __float_as_int(am));
+  }
+  __syncthreads();
+}
+
+// products on two-term operands, issued by one thread: D (+)= A B with A = ah + al, B = bh + bl (a missing low part is 0)
+struct Mma {
+  uint32_t tmem;
+  __device__ __forceinline__ void chain(uint32_t col, uint64_t da, uint32_t as, uint64_t db, uint32_t bs, int ks, uint32_t id, bool acc) const {
+    for (int k = 0; k < ks; ++k) mma_f16(tmem + col, dadv(da, as * k), dadv(db, bs * k), id, (acc || k > 0) ? 1u : 0u);
+  }
+  __device__ __forceinline__ void split(uint32_t col, uint64_t ah, uint64_t al, uint32_t as, uint64_t bh, uint64_t bl, uint32_t bs,
+                                        int ks, uint32_t id, bool acc) const {
+    chain(col, ah, as, bh, bs, ks, id, acc);
+    if (al) chain(col, al, as, bh, bs, ks, id, true);
+    if (bl) chain(col, ah, as, bl, bs, ks, id, true);
+  }
+};
+
+// ------------------------------------------------------------------------------------------------ forward sweep
+template <int D>
+__global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) sweep_kernel(const Args a) {
+  using F = Cfg<D>;
+  constexpr int NV = D + 16;
+  extern __shared__ __align__(128) uint8_t sg[];
+  const uint32_t sb = smem_u32(sg);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  float* const s_x = reinterpret_cast<float*>(sg + F::F_X);
+  float* const s_bm = reinterpret_cast<float*>(sg + F::F_VEC);
+  float *const s_ft = s_bm + D, *const s_pe = s_ft + D;  // s_pe: ft of the chunk in front (its state is still 2^-ft short)
+  float* const s_row = s_pe + 2 * D;                     // [NCG][C]
+  volatile int* const s_fl = reinterpret_cast<volatile int*>(s_row + F::NCG * C);  // tmem base, abort, rmax, smax, vmax, domax
+  const uint32_t bar = smem_u32(const_cast<int*>(s_fl)) + 32;
+  const int bh = blockIdx.x, h = bh % a.H, b = bh / a.H, G = a.H / a.Hkv, j = h / G;
+  const int nch = (a.T + C - 1) / C;
+  if (tid == 0) {
+    mbar_init(bar, 1);
+    mbar_fence_init();
+    for (int i = 1; i < 6; ++i) s_fl[i] = 0;
+  }
+  if (warp == 0) {
+    tmem_alloc(smem_u32(const_cast<int*>(s_fl)), F::COLS);
+    tmem_relinquish();
+  }
+  // the two extra slabs of [v | 1] (column D: the 1) and of the state operand (column D: z; the rest zero)
+  for (int i = tid; i < 2 * C; i += F::THREADS)
+    *reinterpret_cast<uint4*>(sg + F::F_V + toff(F::SL_T, i & (C - 1), D + 8 * (i >> 6))) = make_uint4(0u, 0u, 0u, 0u);
+  for (int i = tid; i < D; i += F::THREADS) s_pe[i] = 0.f;
+  tc_fence_before_sync();
+  __syncthreads();
+  tc_fence_after_sync();
+  const Mma mm{(uint32_t)s_fl[0]};
+  const uint32_t lane_base = mm.tmem + ((uint32_t)((warp & 3) * 32) << 16);
+  const int row = (warp & 3) * 32 + lane, cg = warp >> 2;  // TMEM lane, column group
+  const bool tok_thr = row < C, st_thr = row < D;          // owns a token row / a state row
+  Waiter wt{bar, 0u, s_fl + 1, a.dev_status};
+  constexpr int SW = D / F::NCG, TW = 64 / F::NCG;         // columns per thread of a state row, of a score row
+  auto publish = [&]() {
+    fence_proxy_async();
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+  };
+  float smx = 0.f;
+  if (st_thr) {
+    float s[8];
+#pragma unroll 1
+    for (int c0 = cg * SW; c0 < (cg + 1) * SW; c0 += 8) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        s[i] = a.S0 ? a.S0[((size_t)bh * D + row) * D + c0 + i] : 0.f;
+        smx = fmaxf(smx, fabsf(s[i]));
+      }
+      tmem_st8(lane_base + F::F_ST + c0, s);
+    }
+    if (cg == 0) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) s[i] = 0.f;
+      tmem_st8(lane_base + F::F_ST + D + 8, s);
+      s[0] = a.z0 ? a.z0[(size_t)bh * D + row] : 0.f;
+      smx = fmaxf(smx, fabsf(s[0]));
+      tmem_st8(lane_base + F::F_ST + D, s);
+    }
+    tmem_wait_st();
+  }
+  if (!(smx < 1.0e30f)) smx = 1.0e30f;
+  smx = warp_max(smx);
+  if (lane == 0) atomicMax(const_cast<int*>(&s_fl[3]), __float_as_int(smx));
+  __syncthreads();
+  float sbound = __int_as_float(s_fl[3]), domax = 0.f;
+  int kap_prev = 0;
+  auto KV = [&](uint32_t off, uint32_t slab) -> uint64_t { return kview(sb + off, slab); };
+  auto MV = [&](uint32_t off, uint32_t slab) -> uint64_t { return mview(sb + off, slab); };
+
+  for (int n = 0; n < nch; ++n) {
+    const int t0 = n * C, nvalid = min(C, a.T - t0);
+    const size_t row0 = (size_t)b * a.T + t0;
+    gate_pass<D>(a, row0, h, nvalid, s_x, s_bm, s_ft, const_cast<int*>(&s_fl[2]), tid);
+    const bool f16 = __int_as_float(s_fl[2]) <= RMAX_F16;
+    const int fmt = f16 ? FMT_F16 : FMT_BF16;
+    const int kap = max(-100, min(KAP_MAX, 14 - exp_above(fmaxf(sbound, 1e-30f))));
+    const float ksc = pow2i(kap);
+    // ---- operands
+    float vmax = 0.f;
+    for (int idx = tid; idx < C * F::OCT; idx += F::THREADS) {
+      const int o = idx % F::OCT, r = idx / F::OCT;
+      float q[8], k[8], vv[8], x[8];
+      uint4 zv = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) q[i] = k[i] = 0.f;
+      if (r < nvalid) {
+        const size_t tq = ((row0 + r) * a.H + h) * D + o * 8;
+        load_row8(a.qd + tq, q);
+        load_row8(a.kd + tq, k);
+        zv = *reinterpret_cast<const uint4*>(a.v + ((row0 + r) * a.Hkv + j) * D + o * 8);
+      }
+      load_row8(s_x + r * D + o * 8, x);
+      unpack8b(zv, vv);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        q[i] *= ex2f(x[i]) * (float)(1 << QSC);
+        k[i] *= ex2f(-x[i]) * ksc;
+        vmax = fmaxf(vmax, fabsf(vv[i]));
+      }
+      uint4 hi, lo;
+      const uint32_t at = toff(F::SL_T, r, o * 8);
+      split8h(q, f16, hi, lo);
+      *reinterpret_cast<uint4*>(sg + F::F_QS + at) = hi;
+      *reinterpret_cast<uint4*>(sg + F::F_QS + F::T_TOK + at) = lo;
+      split8h(k, f16, hi, lo);
+      *reinterpret_cast<uint4*>(sg + F::F_KS + at) = hi;
+      *reinterpret_cast<uint4*>(sg + F::F_KS + F::T_TOK + at) = lo;
+      *reinterpret_cast<uint4*>(sg + F::F_V + at) = pack8h(vv, f16);
+      if (o == 0) {
+        const float one[8] = {1.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        *reinterpret_cast<uint4*>(sg + F::F_V + toff(F::SL_T, r, D)) = pack8h(one, f16);
+      }
+    }
+    vmax = warp_max(vmax);
+    if (lane == 0) atomicMax(const_cast<int*>(&s_fl[4]), __float_as_int(vmax < 1.0e30f ? vmax : 1.0e30f));
+    __syncthreads();  // (the exponents have been read: the state operand may overwrite them)
+    // ---- state pass: W = 2^(bm + ft of the chunk in front) S, kept in tensor memory and as the two-term operand, scaled 2^kap
+    smx = 0.f;
+    if (st_thr) {
+      const float f = ex2f(fmaxf(s_bm[row] + s_pe[row], -126.f)) * pow2i(kap - kap_prev);
+      float s[8];
+      uint4 hi, lo;
+#pragma unroll 2
+      for (int c0 = cg * SW; c0 < (cg + 1) * SW; c0 += 8) {
+        tmem_ld8(lane_base + F::F_ST + c0, s);
+        tmem_wait_ld();
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          s[i] *= f;
+          smx = fmaxf(smx, fabsf(s[i]));
+        }
+        split8h(s, f16, hi, lo);
+        *reinterpret_cast<uint4*>(sg + F::F_S + toff(F::SL_C, row, c0)) = hi;
+        *reinterpret_cast<uint4*>(sg + F::F_S + F::T_SZ + toff(F::SL_C, row, c0)) = lo;
+        tmem_st8(lane_base + F::F_ST + c0, s);
+      }
+      if (cg == F::NCG - 1) {
+        tmem_ld8(lane_base + F::F_ST + D, s);
+        tmem_wait_ld();
+        s[0] *= f;
+        smx = fmaxf(smx, fabsf(s[0]));
+#pragma unroll
+        for (int i = 1; i < 8; ++i) s[i] = 0.f;
+        split8h(s, f16, hi, lo);
+        *reinterpret_cast<uint4*>(sg + F::F_S + toff(F::SL_C, row, D)) = hi;
+        *reinterpret_cast<uint4*>(sg + F::F_S + F::T_SZ + toff(F::SL_C, row, D)) = lo;
+        *reinterpret_cast<uint4*>(sg + F::F_S + toff(F::SL_C, row, D + 8)) = make_uint4(0u, 0u, 0u, 0u);
+        *reinterpret_cast<uint4*>(sg + F::F_S + F::T_SZ + toff(F::SL_C, row, D + 8)) = make_uint4(0u, 0u, 0u, 0u);
+        tmem_st8(lane_base + F::F_ST + D, s);
+        a.z16[((size_t)bh * nch + n) * D + row] = s[0];
+      }
+      tmem_wait_st();
+    }
+    smx = warp_max(smx);
+    if (lane == 0) atomicMax(const_cast<int*>(&s_fl[3]), __float_as_int(smx < 1.0e30f ? smx : 1.0e30f));
+    publish();
+    if (tid == 0) {
+      uint8_t* dst = a.s16 + ((size_t)bh * nch + n) * (2 * F::T_C);
+      asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(sb + F::F_S), "r"(F::T_C) : "memory");
+      asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst + F::T_C), "r"(sb + F::F_S + F::T_SZ), "r"(F::T_C) : "memory");
+      tma_store_commit();
+      a.meta[((size_t)bh * nch + n) * 2] = kap;
+      a.meta[((size_t)bh * nch + n) * 2 + 1] = fmt;
+      mm.split(F::F_P, KV(F::F_QS, F::SL_T), KV(F::F_QS + F::T_TOK, F::SL_T), 2 * F::SL_T, KV(F::F_KS, F::SL_T),
+               KV(F::F_KS + F::T_TOK, F::SL_T), 2 * F::SL_T, D / 16, instr_desc(128, C, fmt, MAJOR_K, MAJOR_K), false);
+      mm.split(F::F_O, KV(F::F_QS, F::SL_T), KV(F::F_QS + F::T_TOK, F::SL_T), 2 * F::SL_T, MV(F::F_S, F::SL_C),
+               MV(F::F_S + F::T_SZ, F::SL_C), 256, D / 16, instr_desc(128, NV, fmt, MAJOR_K, MAJOR_MN), false);
+      // (the state in tensor memory is 2^kap-scaled like ks)
+      mm.split(F::F_ST, MV(F::F_KS, F::SL_T), MV(F::F_KS + F::T_TOK, F::SL_T), 256, MV(F::F_V, F::SL_T), 0, 256, C / 16,
+               instr_desc(128, NV, fmt, MAJOR_MN, MAJOR_MN), true);
+      mma_commit(bar);
+    }
+    wt.wait();
+    // ---- mask
+    if (tok_thr) {
+      float s[8];
+      uint4 hi, lo;
+#pragma unroll 2
+      for (int c0 = cg * TW; c0 < (cg + 1) * TW; c0 += 8) {
+        tmem_ld8(lane_base + F::F_P + c0, s);
+        tmem_wait_ld();
+#pragma unroll
+        for (int i = 0; i < 8; ++i) s[i] = c0 + i <= row ? s[i] : 0.f;
+        split8h(s, f16, hi, lo);
+        *reinterpret_cast<uint4*>(sg + F::F_PM + toff(F::SL_U, row, c0)) = hi;
+        *reinterpret_cast<uint4*>(sg + F::F_PM + F::T_P + toff(F::SL_U, row, c0)) = lo;
+      }
+    }
+    for (int i = tid; i < D; i += F::THREADS) s_pe[i] = s_ft[i];
+    publish();
+    if (tid == 0) {
+      mm.split(F::F_O, KV(F::F_PM, F::SL_U), KV(F::F_PM + F::T_P, F::SL_U), 2 * F::SL_U, MV(F::F_V, F::SL_T), 0, 256, C / 16,
+               instr_desc(128, NV, fmt, MAJOR_K, MAJOR_MN), true);
+      mma_commit(bar);
+    }
+    // |next state| <= |2^bm state| + 64 max|v|: every key enters with a factor <= 1
+    const float vm = __int_as_float(s_fl[4]), sm = __int_as_float(s_fl[3]) * pow2i(-kap);
+    wt.wait();
+    // ---- 1 / den and dO . o of the chunk's rows
+    float inv = 1.f, dot = 0.f;
+    if (tok_thr) {
+      const float den = tmem_ld1(lane_base + F::F_O + D);
+      tmem_wait_ld();
+      const float osc = pow2i(-(QSC + kap));
+      inv = a.normalize ? 1.f / fmaf(den, osc, a.eps) : 1.f;
+      const float oi = inv * osc;
+      const bf16* g = a.dO + ((row0 + min(row, nvalid - 1)) * a.H + h) * D;
+#pragma unroll 2
+      for (int c0 = cg * SW; c0 < (cg + 1) * SW; c0 += 8) {
+        float s[8], gv[8];
+        tmem_ld8(lane_base + F::F_O + c0, s);
+        unpack8b(*reinterpret_cast<const uint4*>(g + c0), gv);
+        tmem_wait_ld();
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          dot = fmaf(gv[i], s[i] * oi, dot);
+          domax = fmaxf(domax, fabsf(gv[i]));
+        }
+      }
+      s_row[cg * C + row] = dot;
+    }
+    if (tid == 0) tma_store_wait_read();  // (the state operand has left: the next chunk's exponents may overwrite it)
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+    if (tid == 0) { s_fl[3] = 0; s_fl[4] = 0; }
+    if (tok_thr && cg == 0 && row < nvalid) {
+      float d = 0.f;
+#pragma unroll
+      for (int i = 0; i < F::NCG; ++i) d += s_row[i * C + row];
+      const size_t th = (row0 + row) * a.H + h;
+      a.inv[th] = inv;
+      a.delta[th] = a.normalize ? d : 0.f;
+    }
+    sbound = sm + 64.f * fmaxf(vm, 1.f);
+    kap_prev = kap;
+    __syncthreads();
+  }
+  domax = warp_max(domax);
+  if (lane == 0) atomicMax(const_cast<int*>(&s_fl[5]), __float_as_int(domax < 1.0e30f ? domax : 1.0e30f));
+  tc_fence_before_sync();
+  __syncthreads();
+  if (tid == 0) {
+    a.domax[bh] = __int_as_float(s_fl[5]);
+    tma_store_wait_all();
+  }
+  if (warp == 0) {
+    tc_fence_after_sync();
+    tmem_dealloc(mm.tmem, F::COLS);
+  }
+}
+
+// ------------------------------------------------------------------------------------------------ reverse sweep
+template <int D>
+__global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_kernel(const Args a) {
+  using F = Cfg<D>;
+  constexpr int NW = F::THREADS / 32;
+  extern __shared__ __align__(128) uint8_t sg[];
+  const uint32_t sb = smem_u32(sg);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  float* const s_x = reinterpret_cast<float*>(sg + F::R_X);
+  float* const s_bm = reinterpret_cast<float*>(sg + F::R_VEC);
+  float *const s_ft = s_bm + D, *const s_pe = s_ft + D;  // s_pe: bm of the chunk behind (its adjoint is still 2^-bm short)
+  float *const s_z = s_pe + D, *const s_r16 = s_z + D, *const s_r = s_r16 + D, *const s_car = s_r + D;
+  float *const s_tot = s_car + D;                        // (unused tail of D floats keeps the row scalars aligned)
+  float *const s_inv = s_tot + D, *const s_dl = s_inv + C;
+  float* const s_rp = s_dl + C;                          // [NW][D] partial sums of r
+  volatile int* const s_fl = reinterpret_cast<volatile int*>(s_rp + NW * D);  // tmem base, abort, rmax, imax, Rmax, wmax
+  const uint32_t bar = smem_u32(const_cast<int*>(s_fl)) + 32, bar_s = bar + 8;
+  const int bh = blockIdx.x, h = bh % a.H, b = bh / a.H, G = a.H / a.Hkv, j = h / G;
+  const int nch = (a.T + C - 1) / C;
+  if (tid == 0) {
+    mbar_init(bar, 1);
+    mbar_init(bar_s, 1);
+    mbar_fence_init();
+    for (int i = 1; i < 6; ++i) s_fl[i] = 0;
+  }
+  if (warp == 0) {
+    tmem_alloc(smem_u32(const_cast<int*>(s_fl)), F::COLS);
+    tmem_relinquish();
+  }
+  for (int i = tid; i < D; i += F::THREADS) s_pe[i] = s_r[i] = s_car[i] = 0.f;
+  tc_fence_before_sync();
+  __syncthreads();
+  tc_fence_after_sync();
+  const Mma mm{(uint32_t)s_fl[0]};
+  const uint32_t lane_base = mm.tmem + ((uint32_t)((warp & 3) * 32) << 16);
+  const int row = (warp & 3) * 32 + lane, cg = warp >> 2;
+  const bool tok_thr = row < C, st_thr = row < D;
+  Waiter wt{bar, 0u, s_fl + 1, a.dev_status}, ws{bar_s, 0u, s_fl + 1, a.dev_status};
+  constexpr int SW = D / F::NCG, TW = 64 / F::NCG;
+  auto publish = [&]() {
+    fence_proxy_async();
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+  };
+  auto KV = [&](uint32_t off, uint32_t slab) -> uint64_t { return kview(sb + off, slab); };
+  auto MV = [&](uint32_t off, uint32_t slab) -> uint64_t { return mview(sb + off, slab); };
+  if (st_thr) {  // the adjoint starts at zero
+    float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
+    for (int c0 = cg * SW; c0 < (cg + 1) * SW; c0 += 8) tmem_st8(lane_base + F::R_R + c0, s);
+    tmem_wait_st();
+  }
+  // 2^sc: the largest |dO| of the head becomes 2^4 .. 2^5 (every gradient is linear in dO)
+  const int sc = 5 - exp_above(fmaxf(a.domax[bh], 1e-30f));
+  const float osc = pow2i(sc);
+  int al_prev = 0;
+  float wmax = 0.f;
+
+  for (int n = nch - 1; n >= 0; --n) {
+    const int t0 = n * C, nvalid = min(C, a.T - t0);
+    const size_t row0 = (size_t)b * a.T + t0;
+    const int kap = a.meta[((size_t)bh * nch + n) * 2], fmt = a.meta[((size_t)bh * nch + n) * 2 + 1];
+    const bool f16 = fmt == FMT_F16;
+    // ---- row scalars; the largest inv of the chunk and the largest entry of the adjoint decide 2^al
+    if (tid == 0) s_fl[3] = s_fl[4] = 0;
+    __syncthreads();
+    if (tid < C) {
+      float inv = 0.f, dl = 0.f;
+      if (tid < nvalid) {
+        const size_t th = (row0 + tid) * a.H + h;
+        inv = a.inv[th];
+        dl = a.delta[th];
+      }
+      s_inv[tid] = inv;
+      s_dl[tid] = dl * osc;
+      const float m = warp_max(fabsf(inv));
+      if (lane == 0) atomicMax(const_cast<int*>(&s_fl[3]), __float_as_int(m < 1.0e30f ? m : 1.0e30f));
+    }
+    if (tid >= C && tid < C + D) s_z[tid - C] = a.z16[((size_t)bh * nch + n) * D + tid - C];
+    if (n < nch - 1 && st_thr) {
+      const float f = ex2f(fmaxf(s_pe[row], -126.f));
+      float m = 0.f, s[32];
+#pragma unroll 1
+      for (int c0 = cg * SW; c0 < (cg + 1) * SW; c0 += 32) {
+        tmem_ld32(lane_base + F::R_R + c0, s);
+        tmem_wait_ld();
+#pragma unroll
+        for (int i = 0; i < 32; ++i) m = fmaxf(m, fabsf(s[i]));
+      }
+      m = warp_max(m * f);
+      if (lane == 0) atomicMax(const_cast<int*>(&s_fl[4]), __float_as_int(m < 1.0e30f ? m : 1.0e30f));
+    }
+    gate_pass<D>(a, row0, h, nvalid, s_x, s_bm, s_ft, const_cast<int*>(&s_fl[2]), tid);  // (two barriers)
+    int al = min(5 - exp_above(fmaxf(__int_as_float(s_fl[3]), 1e-30f)), 10 - kap);
+    const float rm = __int_as_float(s_fl[4]);
+    if (rm > 0.f) al = min(al, al_prev + 14 - exp_above(rm));
+    al = max(al, -100);
+    const float asc = pow2i(al), ksc = pow2i(kap);
+    // ---- operands: qn, ks (two-term), v, dO; partial sums of r
+    float rp[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) rp[i] = 0.f;
+    for (int idx = tid; idx < C * F::OCT; idx += F::THREADS) {
+      const int o = idx % F::OCT, r = idx / F::OCT;  // (o is the same in every iteration)
+      float q[8], k[8], vv[8], g[8], x[8];
+      uint4 zv = make_uint4(0u, 0u, 0u, 0u), zg = zv;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) q[i] = k[i] = 0.f;
+      if (r < nvalid) {
+        const size_t tq = ((row0 + r) * a.H + h) * D + o * 8;
+        load_row8(a.qd + tq, q);
+        load_row8(a.kd + tq, k);
+        zv = *reinterpret_cast<const uint4*>(a.v + ((row0 + r) * a.Hkv + j) * D + o * 8);
+        zg = *reinterpret_cast<const uint4*>(a.dO + tq);
+      }
+      load_row8(s_x + r * D + o * 8, x);
+      unpack8b(zv, vv);
+      unpack8b(zg, g);
+      const float inv = s_inv[r] * asc, dl = s_dl[r];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        q[i] *= ex2f(x[i]) * inv;
+        k[i] *= ex2f(-x[i]) * ksc;
+        g[i] *= osc;
+        rp[i] = fmaf(-dl, q[i], rp[i]);
+      }
+      uint4 hi, lo;
+      const uint32_t at = toff(F::SL_T, r, o * 8);
+      split8h(q, f16, hi, lo);
+      *reinterpret_cast<uint4*>(sg + F::R_QS + at) = hi;
+      *reinterpret_cast<uint4*>(sg + F::R_QS + F::T_TOK + at) = lo;
+      split8h(k, f16, hi, lo);
+      *reinterpret_cast<uint4*>(sg + F::R_KS + at) = hi;
+      *reinterpret_cast<uint4*>(sg + F::R_KS + F::T_TOK + at) = lo;
+      *reinterpret_cast<uint4*>(sg + F::R_V + at) = pack8h(vv, f16);
+      *reinterpret_cast<uint4*>(sg + F::R_DO + at) = pack8h(g, f16);
+    }
+#pragma unroll
+    for (int off = F::OCT; off < 32; off <<= 1) {  // (the lanes of a warp that hold the same channels)
+#pragma unroll
+      for (int i = 0; i < 8; ++i) rp[i] += __shfl_xor_sync(0xffffffffu, rp[i], off);
+    }
+    if (lane < F::OCT) store_row8(s_rp + warp * D + lane * 8, rp);
+    publish();
+    if (tid == 0) {
+      // the state operand of this chunk (needed behind the mask pass), over the exponents
+      mbar_arrive_expect_tx(bar_s, 2 * F::T_C);
+      const uint8_t* src = a.s16 + ((size_t)bh * nch + n) * (2 * F::T_C);
+      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(sb + F::R_S),
+                   "l"(src), "r"(2 * F::T_C), "r"(bar_s)
+                   : "memory");
+      mm.split(F::R_P, KV(F::R_QS, F::SL_T), KV(F::R_QS + F::T_TOK, F::SL_T), 2 * F::SL_T, KV(F::R_KS, F::SL_T),
+               KV(F::R_KS + F::T_TOK, F::SL_T), 2 * F::SL_T, D / 16, instr_desc(128, C, fmt, MAJOR_K, MAJOR_K), false);
+      mm.chain(F::R_EP, KV(F::R_DO, F::SL_T), 2 * F::SL_T, KV(F::R_V, F::SL_T), 2 * F::SL_T, D / 16,
+               instr_desc(128, C, fmt, MAJOR_K, MAJOR_K), false);
+      mma_commit(bar);
+    }
+    // factor that brings the adjoint behind the chunk to 2^ft R 2^(al + sc)
+    const float rfac = pow2i(al - al_prev);
+    if (tid < D) {
+      const float w = ex2f(fmaxf(s_pe[tid] + s_ft[tid], -126.f)) * rfac * s_r[tid];
+      float p = 0.f;
+#pragma unroll
+      for (int i = 0; i < NW; ++i) p += s_rp[i * D + tid];
+      s_r16[tid] = w;
+      s_r[tid] = w + p;
+    }
+    wt.wait();
+    // ---- mask: P' and E = dO v^T - delta, two-term
+    if (tok_thr) {
+      const float dl = s_dl[row];
+      float s[8], e[8];
+      uint4 hi, lo;
+#pragma unroll 2
+      for (int c0 = cg * TW; c0 < (cg + 1) * TW; c0 += 8) {
+        tmem_ld8(lane_base + F::R_P + c0, s);
+        tmem_ld8(lane_base + F::R_EP + c0, e);
+        tmem_wait_ld();
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const bool on = c0 + i <= row;
+          s[i] = on ? s[i] : 0.f;
+          e[i] = on ? fminf(fmaxf(e[i] - dl, -65000.f), 65000.f) : 0.f;
+        }
+        const uint32_t at = toff(F::SL_U, row, c0);
+        split8h(s, f16, hi, lo);
+        *reinterpret_cast<uint4*>(sg + F::R_PM + at) = hi;
+        *reinterpret_cast<uint4*>(sg + F::R_PM + F::T_P + at) = lo;
+        split8h(e, f16, hi, lo);
+        *reinterpret_cast<uint4*>(sg + F::R_E + at) = hi;
+        *reinterpret_cast<uint4*>(sg + F::R_E + F::T_P + at) = lo;
+      }
+    }
+    publish();
+    const uint32_t ID_KM = instr_desc(128, D, fmt, MAJOR_K, MAJOR_MN), ID_MM = instr_desc(128, D, fmt, MAJOR_MN, MAJOR_MN),
+                   ID_KK = instr_desc(128, D, fmt, MAJOR_K, MAJOR_K);
+    if (tid == 0) {
+      ws.wait();  // the state operand has landed
+      mm.split(F::R_DQ, KV(F::R_E, F::SL_U), KV(F::R_E + F::T_P, F::SL_U), 2 * F::SL_U, MV(F::R_KS, F::SL_T),
+               MV(F::R_KS + F::T_TOK, F::SL_T), 256, C / 16, ID_KM, false);
+      mm.split(F::R_DQ, KV(F::R_DO, F::SL_T), 0, 2 * F::SL_T, KV(F::R_S, F::SL_C), KV(F::R_S + F::T_C, F::SL_C), 2 * F::SL_C,
+               D / 16, ID_KK, true);
+      mm.split(F::R_DK, MV(F::R_E, F::SL_U), MV(F::R_E + F::T_P, F::SL_U), 256, MV(F::R_QS, F::SL_T),
+               MV(F::R_QS + F::T_TOK, F::SL_T), 256, C / 16, ID_MM, false);
+      mm.split(F::R_DVC, MV(F::R_PM, F::SL_U), MV(F::R_PM + F::T_P, F::SL_U), 256, MV(F::R_DO, F::SL_T), 0, 256, C / 16, ID_MM,
+               false);
+      mma_commit(bar);
+    }
+    wt.wait();
+    // ---- adjoint pass, over the consumed state operand
+    if (st_thr) {
+      const float f = ex2f(fmaxf(s_pe[row] + s_ft[row], -126.f)) * rfac;
+      float s[8];
+      uint4 hi, lo;
+#pragma unroll 2
+      for (int c0 = cg * SW; c0 < (cg + 1) * SW; c0 += 8) {
+        tmem_ld8(lane_base + F::R_R + c0, s);
+        tmem_wait_ld();
+#pragma unroll
+        for (int i = 0; i < 8; ++i) s[i] *= f;
+        split8h(s, f16, hi, lo);
+        *reinterpret_cast<uint4*>(sg + F::R_S + toff(F::SL_C, row, c0)) = hi;
+        *reinterpret_cast<uint4*>(sg + F::R_S + F::T_C + toff(F::SL_C, row, c0)) = lo;
+        tmem_st8(lane_base + F::R_R + c0, s);
+      }
+      tmem_wait_st();
+    }
+    publish();
+    if (tid == 0) {
+      mm.split(F::R_DK, KV(F::R_V, F::SL_T), 0, 2 * F::SL_T, KV(F::R_S, F::SL_C), KV(F::R_S + F::T_C, F::SL_C), 2 * F::SL_C,
+               D / 16, ID_KK, true);
+      mm.split(F::R_DVC, KV(F::R_KS, F::SL_T), KV(F::R_KS + F::T_TOK, F::SL_T), 2 * F::SL_T, MV(F::R_S, F::SL_C),
+               MV(F::R_S + F::T_C, F::SL_C), 256, D / 16, ID_KM, true);
+      mm.split(F::R_R, MV(F::R_QS, F::SL_T), MV(F::R_QS + F::T_TOK, F::SL_T), 256, MV(F::R_DO, F::SL_T), 0, 256, C / 16, ID_MM,
+               true);
+      mma_commit(bar);
+    }
+    for (int i = tid; i < D; i += F::THREADS) s_pe[i] = s_bm[i];  // (read again behind the next barrier at the earliest)
+    wt.wait();
+    // ---- wq, wk, dv of the chunk's rows into fp32 tiles over the dead operands
+    const float usc = pow2i(-(al + kap + sc));
+    float wqv[SW > 32 ? 1 : SW], wkv[SW > 32 ? 1 : SW];
+    static_assert(SW == 32, "32 columns per thread");
+    if (tok_thr) {
+      const float dl = s_dl[row];
+#pragma unroll
+      for (int i8 = 0; i8 < SW; i8 += 8) {
+        const int c0 = cg * SW + i8;
+        float d[8], hi[8], lo[8];
+        const uint32_t at = toff(F::SL_T, row, c0);
+        tmem_ld8(lane_base + F::R_DQ + c0, d);
+        unpack8h(*reinterpret_cast<const uint4*>(sg + F::R_QS + at), f16, hi);
+        unpack8h(*reinterpret_cast<const uint4*>(sg + F::R_QS + F::T_TOK + at), f16, lo);
+        tmem_wait_ld();
+#pragma unroll
+        for (int i = 0; i < 8; ++i) wqv[i8 + i] = (hi[i] + lo[i]) * fmaf(-dl, s_z[c0 + i], d[i]) * usc;
+        tmem_ld8(lane_base + F::R_DK + c0, d);
+        unpack8h(*reinterpret_cast<const uint4*>(sg + F::R_KS + at), f16, hi);
+        unpack8h(*reinterpret_cast<const uint4*>(sg + F::R_KS + F::T_TOK + at), f16, lo);
+        tmem_wait_ld();
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          wkv[i8 + i] = (hi[i] + lo[i]) * (d[i] + s_r16[c0 + i]) * usc;
+          wmax = fmaxf(wmax, fmaxf(fabsf(wqv[i8 + i]), fabsf(wkv[i8 + i])));
+        }
+      }
+#pragma unroll
+      for (int i8 = 0; i8 < SW; i8 += 8) {
+        float d[8];
+        tmem_ld8(lane_base + F::R_DVC + cg * SW + i8, d);
+        tmem_wait_ld();
+#pragma unroll
+        for (int i4 = 0; i4 < 8; i4 += 4) {
+          const int c = cg * SW + i8 + i4;
+          *reinterpret_cast<float4*>(sg + F::R_WQ + foff<D>(row, c >> 2)) = make_float4(wqv[i8 + i4], wqv[i8 + i4 + 1], wqv[i8 + i4 + 2], wqv[i8 + i4 + 3]);
+          *reinterpret_cast<float4*>(sg + F::R_WK + foff<D>(row, c >> 2)) = make_float4(wkv[i8 + i4], wkv[i8 + i4 + 1], wkv[i8 + i4 + 2], wkv[i8 + i4 + 3]);
+          *reinterpret_cast<float4*>(sg + F::R_DV + foff<D>(row, c >> 2)) = make_float4(d[i4] * usc, d[i4 + 1] * usc, d[i4 + 2] * usc, d[i4 + 3] * usc);
+        }
+      }
+    }
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+    // ---- gate gradient: reverse running sum of wq - wk over the chunk's tokens on top of what lies behind it; thread =
+    // (channel, run of tokens); the runs' totals meet in shared memory
+    {
+      constexpr int RUNS = F::THREADS / D, RT = C / RUNS;  // 4 runs of 16 tokens
+      const int c = tid % D, run = tid / D;
+      float v[RT], acc = 0.f;
+#pragma unroll
+      for (int i = RT - 1; i >= 0; --i) {
+        const uint32_t at = foff<D>(run * RT + i, c >> 2) + (c & 3) * 4;
+        acc += *reinterpret_cast<const float*>(sg + F::R_WQ + at) - *reinterpret_cast<const float*>(sg + F::R_WK + at);
+        v[i] = acc;
+      }
+      s_rp[run * D + c] = acc;  // (NW >= RUNS rows)
+      __syncthreads();
+      float off = s_car[c], all = off;
+#pragma unroll
+      for (int r = RUNS - 1; r >= 0; --r) {
+        const float t = s_rp[r * D + c];
+        if (r > run) off += t;
+        all += t;
+      }
+#pragma unroll
+      for (int i = 0; i < RT; ++i) *reinterpret_cast<float*>(sg + F::R_DG + foff<D>(run * RT + i, c >> 2) + (c & 3) * 4) = v[i] + off;
+      __syncthreads();
+      if (run == 0) s_car[c] = all;
+    }
+    // ---- whole rows to global memory
+    for (int idx = tid; idx < nvalid * (D / 4); idx += F::THREADS) {
+      const int pc = idx % (D / 4), r = idx / (D / 4);
+      const size_t at = ((row0 + r) * a.H + h) * D + pc * 4;
+      const uint32_t so = foff<D>(r, pc);
+      *reinterpret_cast<float4*>(a.wq + at) = *reinterpret_cast<const float4*>(sg + F::R_WQ + so);
+      *reinterpret_cast<float4*>(a.wk + at) = *reinterpret_cast<const float4*>(sg + F::R_WK + so);
+      *reinterpret_cast<float4*>(a.dvh + at) = *reinterpret_cast<const float4*>(sg + F::R_DV + so);
+    }
+    auto dlog = [&](float av) { return a.gate_mode == LAWCAT_GATE_LOGDECAY ? 1.f : (1.f - 1.f / (1.f + __expf(-av))) * a.inv_tau; };
+    if (a.gate_dim == 1) {
+      for (int r = warp; r < nvalid; r += NW) {
+        float s = 0.f;
+        for (int c = lane; c < D; c += 32) s += *reinterpret_cast<const float*>(sg + F::R_DG + foff<D>(r, c >> 2) + (c & 3) * 4);
+        s = warp_sum(s);
+        if (lane == 0) {
+          const size_t gi = (row0 + r) * a.H + h;
+          a.dgate[gi] = __float2bfloat16_rn(s * dlog(__bfloat162float(a.gate[gi])));
+        }
+      }
+    } else {
+      for (int idx = tid; idx < nvalid * F::OCT; idx += F::THREADS) {
+        const int o = idx % F::OCT, r = idx / F::OCT;
+        const size_t gi = ((row0 + r) * a.H + h) * D + o * 8;
+        float av[8], d[8];
+        unpack8b(*reinterpret_cast<const uint4*>(a.gate + gi), av);
+        const float4 x = *reinterpret_cast<const float4*>(sg + F::R_DG + foff<D>(r, 2 * o)), y = *reinterpret_cast<const float4*>(sg + F::R_DG + foff<D>(r, 2 * o + 1));
+        d[0] = x.x; d[1] = x.y; d[2] = x.z; d[3] = x.w; d[4] = y.x; d[5] = y.y; d[6] = y.z; d[7] = y.w;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) d[i] *= dlog(av[i]);
+        store_row8(a.dgate + gi, d);
+      }
+    }
+    al_prev = al;
+    __syncthreads();
+  }
+  wmax = warp_max(wmax);
+  if (lane == 0) atomicMax(a.wmax, __float_as_int(wmax < 1.0e30f ? wmax : 1.0e30f));
+  tc_fence_before_sync();
+  __syncthreads();
+  if (warp == 0) {
+    tc_fence_after_sync();
+    tmem_dealloc(mm.tmem, F::COLS);
+  }
+}
+
+// ------------------------------------------------------------------------------------------------ mix backward
+// From w = p * dp of both streams (p the features) back through the softmax and the shared linear layer:
+//   dy = w - p sum(w),   du = dy W_h^T (query stream; key stream summed over the heads of the group),   dW_h += u^T dy
+// One block = one (batch, key head, tile of 128 tokens), walking the group's heads and both streams. dy (scaled by a power of
+// two from the largest |w| of the call) and u, the recomputed conv output, are two-term fp16 pairs; the key stream's du is
+// accumulated over the heads in tensor memory. du of the query stream overwrites wq in place.
+struct MArgs {
+  const bf16 *q, *k, *w_q, *w_k, *W, *cache_q, *cache_k;
+  const float *qd, *kd, *wk;
+  float *wq;                 // in: wq; out: du of the query stream
+  float *du_k, *dW;          // [B,T,Hkv,D]; [H,D,D] (atomic adds into zeros)
+  const int* wmax;
+  int* dev_status;
+  int B, T, H, Hkv, K;
+};
+
+template <int D>
+struct MCfg {
+  using L = Lay<D>;
+  static constexpr uint32_t WT = 0, U = L::TILE_W, DY = U + 2 * L::TILE_U, TAPS = DY + 2 * L::TILE_U, BAR = TAPS + D * 16;
+  static constexpr uint32_t BYTES = BAR + 64;
+  static constexpr uint32_t DUQ = 0, DUK = D, DWC = 2 * D, COLS = D == 128 ? 512 : 256;
+};
+
+template <int D>
+__global__ void __launch_bounds__(256, D == 128 ? 1 : 2) mix_bwd_kernel(const MArgs a) {
+  using L = Lay<D>;
+  using M = MCfg<D>;
+  extern __shared__ __align__(128) uint8_t sg[];
+  const uint32_t sb = smem_u32(sg);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  volatile int* const s_fl = reinterpret_cast<volatile int*>(sg + M::BAR + 16);  // tmem base, abort
+  float* const s_taps = reinterpret_cast<float*>(sg + M::TAPS);
+  const int t0 = blockIdx.x * TT, bj = blockIdx.y, j = bj % a.Hkv, b = bj / a.Hkv, G = a.H / a.Hkv;
+  const int nvalid = min(TT, a.T - t0);
+  if (tid == 0) {
+    mbar_init(sb + M::BAR, 1);
+    mbar_fence_init();
+    s_fl[1] = 0;
+  }
+  if (warp == 0) {
+    tmem_alloc(sb + M::BAR + 16, M::COLS);
+    tmem_relinquish();
+  }
+  tc_fence_before_sync();
+  __syncthreads();
+  tc_fence_after_sync();
+  const Mma mm{(uint32_t)s_fl[0]};
+  const uint32_t lane_base = mm.tmem + ((uint32_t)((warp & 3) * 32) << 16);
+  const int row = (warp & 3) * 32 + lane, half = warp >> 2;
+  constexpr int HC = D / 2;
+  Waiter wt{sb + M::BAR, 0u, s_fl + 1, a.dev_status};
+  // 2^sg: the largest |w| becomes 2^7 .. 2^8, which leaves |dy| <= |w| + sum |w| below the fp16 maximum for every row
+  const int sgm = 8 - exp_above(fmaxf(__int_as_float(*a.wmax), 1e-30f));
+  const float sc = pow2i(sgm), isc = pow2i(-sgm);
+  const int o = tid % L::OPR, rr0 = tid / L::OPR;
+  constexpr int RSTEP = 256 / L::OPR;
+  // fp32 [128][D] accumulator to global rows through the (dead) dy tiles
+  auto rows_out = [&](uint32_t col, float* dst, int NH, int head) {
+    float d[8];
+#pragma unroll 1
+    for (int c0 = half * HC; c0 < (half + 1) * HC; c0 += 8) {
+      tmem_ld8(lane_base + col + c0, d);
+      tmem_wait_ld();
+#pragma unroll
+      for (int i = 0; i < 8; i += 4)
+        *reinterpret_cast<float4*>(sg + M::DY + foff<D>(row, (c0 + i) >> 2)) = make_float4(d[i] * isc, d[i + 1] * isc, d[i + 2] * isc, d[i + 3] * isc);
+    }
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+    for (int idx = tid; idx < nvalid * (D / 4); idx += 256) {
+      const int pc = idx % (D / 4), r = idx / (D / 4);
+      *reinterpret_cast<float4*>(dst + (((size_t)b * a.T + t0 + r) * NH + head) * D + pc * 4) =
+          *reinterpret_cast<const float4*>(sg + M::DY + foff<D>(r, pc));
+    }
+    __syncthreads();
+  };
+#pragma unroll 1
+  for (int g = 0; g < G; ++g) {
+    const int h = j * G + g;
+    load_w_tile<D>(sg + M::WT, a.W + (size_t)h * D * D, tid, 256);
+#pragma unroll 1
+    for (int stream = 0; stream < 2; ++stream) {
+      const bf16* x = stream ? a.k : a.q;
+      const bf16* w = stream ? a.w_k : a.w_q;
+      const int NH = stream ? a.Hkv : a.H, head = stream ? j : h;
+      for (int idx = tid; idx < D * 4; idx += 256) {
+        const int c = idx >> 2, dl = idx & 3;
+        s_taps[idx] = dl < a.K ? __bfloat162float(w[((size_t)head * D + c) * a.K + dl]) : 0.f;
+      }
+      // ---- dy
+      {
+        const float* wp = stream ? a.wk : a.wq;
+        const float* pp = stream ? a.kd : a.qd;
+#pragma unroll 2
+        for (int r = rr0; r < TT; r += RSTEP) {
+          float wv[8], pv[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) wv[i] = pv[i] = 0.f;
+          if (r < nvalid) {
+            const size_t at = (((size_t)b * a.T + t0 + r) * a.H + h) * D + o * 8;
+            load_row8(wp + at, wv);
+            load_row8(pp + at, pv);
+          }
+          float s = 0.f;
+#pragma unroll
+          for (int i = 0; i < 8; ++i) s += wv[i];
+#pragma unroll
+          for (int off = 1; off < L::OPR; off <<= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) wv[i] = fmaf(-pv[i], s, wv[i]) * sc;
+          uint4 hi, lo;
+          split8h(wv, true, hi, lo);
+          *reinterpret_cast<uint4*>(sg + M::DY + toff(L::SLAB_U, r, o * 8)) = hi;
+          *reinterpret_cast<uint4*>(sg + M::DY + L::TILE_U + toff(L::SLAB_U, r, o * 8)) = lo;
+        }
+      }
+      __syncthreads();  // (the taps)
+      // ---- u
+      {
+        constexpr int RPT = TT / RSTEP, STEP = 4;
+#pragma unroll 1
+        for (int rr = 0; rr < RPT; rr += STEP)
+          conv_run<D, STEP>(x, stream ? a.cache_k : a.cache_q, s_taps, b, t0 + rr0 * RPT + rr, a.T, NH, head, a.K, o,
+                            [&](int i, float* u) {
+                              uint4 hi, lo;
+                              split8h(u, true, hi, lo);
+                              const uint32_t at = toff(L::SLAB_U, rr0 * RPT + rr + i, o * 8);
+                              *reinterpret_cast<uint4*>(sg + M::U + at) = hi;
+                              *reinterpret_cast<uint4*>(sg + M::U + L::TILE_U + at) = lo;
+                            });
+      }
+      fence_proxy_async();
+      tc_fence_before_sync();
+      __syncthreads();
+      tc_fence_after_sync();
+      if (tid == 0) {
+        mm.split(stream ? M::DUK : M::DUQ, kview(sb + M::DY, L::SLAB_U), kview(sb + M::DY + L::TILE_U, L::SLAB_U), 2 * L::SLAB_U,
+                 kview(sb + M::WT, L::SLAB_W), 0, 2 * L::SLAB_W, D / 16, instr_desc(128, D, FMT_F16, MAJOR_K, MAJOR_K),
+                 stream == 1 && g > 0);
+        mm.split(M::DWC, mview(sb + M::U, L::SLAB_U), mview(sb + M::U + L::TILE_U, L::SLAB_U), 256, mview(sb + M::DY, L::SLAB_U),
+                 mview(sb + M::DY + L::TILE_U, L::SLAB_U), 256, TT / 16, instr_desc(128, D, FMT_F16, MAJOR_MN, MAJOR_MN), stream == 1);
+        mma_commit(sb + M::BAR);
+      }
+      wt.wait();
+      if (stream == 0) rows_out(M::DUQ, a.wq, a.H, h);
+    }
+    // dW of the head: row c of the accumulator belongs to lane c
+    if (a.dW && row < D) {
+      float d[8];
+#pragma unroll 1
+      for (int c0 = half * HC; c0 < (half + 1) * HC; c0 += 8) {
+        tmem_ld8(lane_base + M::DWC + c0, d);
+        tmem_wait_ld();
+        float* dst = a.dW + ((size_t)h * D + row) * D + c0;
+#pragma unroll
+        for (int i = 0; i < 8; i += 4)
+          asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + i), "f"(d[i] * isc), "f"(d[i + 1] * isc),
+                       "f"(d[i + 2] * isc), "f"(d[i + 3] * isc)
+                       : "memory");
+      }
+    }
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+  }
+  rows_out(M::DUK, a.du_k, a.Hkv, j);
+  tc_fence_before_sync();
+  __syncthreads();
+  if (warp == 0) {
+    tc_fence_after_sync();
+    tmem_dealloc(mm.tmem, M::COLS);
+  }
+}
+
+// dv[b,t,j,:] = sum over the query heads of group j of the per-head gradients; one thread per 8 channels
+__global__ void dv_sum_kernel(const float* __restrict__ dvh, bf16* __restrict__ dv, size_t total, int G, int oct) {
+  const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= total) return;
+  const size_t btj = idx / oct;
+  const int o8 = (int)(idx % oct);
+  float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  for (int g = 0; g < G; ++g) {
+    float x[8];
+    load_row8(dvh + ((btj * G + g) * oct + o8) * 8, x);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) s[i] += x[i];
+  }
+  store_row8(dv + (btj * oct + o8) * 8, s);
+}
+
+struct Plan {
+  size_t qd, kd, wq, wk, dvh, du_k, inv, delta, domax, z16, meta, s16, wmax, total;
+};
+static Plan plan(const lawcat_params& p) {
+  Plan L;
+  size_t off = 0;
+  auto take = [&](size_t n) { const size_t o = off; off += align_up(n, 256); return o; };
+  const size_t bth = (size_t)p.B * p.T * p.H, nf = 4 * bth * p.d_k, ch = (size_t)p.B * p.H * ((p.T + C - 1) / C);
+  L.qd = take(nf); L.kd = take(nf); L.wq = take(nf); L.wk = take(nf); L.dvh = take(nf);
+  L.du_k = take(nf / (p.H / p.H_kv));
+  L.inv = take(4 * bth); L.delta = take(4 * bth); L.domax = take(4 * (size_t)p.B * p.H);
+  L.z16 = take(4 * ch * p.d_k); L.meta = take(8 * ch); L.s16 = take(ch * 4 * p.d_k * p.d_k); L.wmax = take(4);
+  L.total = off;
+  return L;
+}
+
+static int raise_limits() {
+  static std::mutex mu;
+  static bool done[64] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return LAWCAT_ERR_CUDA;
+  std::lock_guard<std::mutex> lk(mu);
+  if (done[dev]) return LAWCAT_OK;
+  auto up = [](auto* k, uint32_t n) { return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)n) == cudaSuccess; };
+  if (!up(sweep_kernel<64>, Cfg<64>::F_BYTES) || !up(sweep_kernel<128>, Cfg<128>::F_BYTES) || !up(reverse_kernel<64>, Cfg<64>::R_BYTES) ||
+      !up(reverse_kernel<128>, Cfg<128>::R_BYTES) || !up(mix_bwd_kernel<64>, MCfg<64>::BYTES) || !up(mix_bwd_kernel<128>, MCfg<128>::BYTES))
+    return LAWCAT_ERR_CUDA;
+  done[dev] = true;
+  return LAWCAT_OK;
+}
+
+template <int D>
+static int run(const Ctx& c, const Args& a, const MArgs& m) {
+  const lawcat_params& p = *c.p;
+  {
+    LaunchScope _ls("gla_tc_bwd_sweep", c.stream);
+    sweep_kernel<D><<<p.B * p.H, Cfg<D>::THREADS, Cfg<D>::F_BYTES, c.stream>>>(a);
+    LAWCAT_CHECK_LAUNCH();
+  }
+  {
+    LaunchScope _ls("gla_tc_bwd", c.stream);
+    reverse_kernel<D><<<p.B * p.H, Cfg<D>::THREADS, Cfg<D>::R_BYTES, c.stream>>>(a);
+    LAWCAT_CHECK_LAUNCH();
+  }
+  LaunchScope _ls("convmix_tc_bwd", c.stream);
+  mix_bwd_kernel<D><<<dim3((unsigned)((p.T + TT - 1) / TT), (unsigned)(p.B * p.H_kv)), 256, MCfg<D>::BYTES, c.stream>>>(m);
+  LAWCAT_CHECK_LAUNCH();
+  return LAWCAT_OK;
+}
+
+}  // namespace lbt
+
+// (sharp sigmoid gates and short calls: the same exceptions as the forward, see gla_tc_supported)
+bool layer_bwd_tc_supported(const lawcat_params& p) {
+  const bool sharp = p.gate_mode == LAWCAT_GATE_LOGITS && p.gate_tau < 8.f;
+  return p.dtype == LAWCAT_BF16 && (p.d_k == 64 || p.d_k == 128) && p.d_v == p.d_k && (p.gate_dim == p.d_k || p.gate_dim == 1) &&
+         !sharp && p.phi == LAWCAT_PHI_SOFTMAX && p.conv_k <= ctc::HALO + 1 && !p.mix_unshared && p.B > 0 && p.T >= 16 &&
+         (p.chunk == 0 || p.chunk == lbt::C);
+}
+
+size_t layer_bwd_tc_workspace_bytes(const lawcat_params& p) { return lbt::plan(p).total; }
+
+int launch_layer_bwd_tc(const Ctx& c, const void* q, const void* k, const void* v, const void* gate, const void* w_q,
+                        const void* w_k, const void* W, const void* cache_q, const void* cache_k, const float* S0,
+                        const float* z0, const void* dO, void* dq, void* dk, void* dv, void* dgate, float* dw_q, float* dw_k,
+                        float* dW, void* ws) {
+  using namespace lbt;
+  const lawcat_params& p = *c.p;
+  int r = raise_limits();
+  if (r) return r;
+  const Plan L = plan(p);
+  char* w = (char*)ws;
+  Args a{};
+  a.qd = (float*)(w + L.qd); a.kd = (float*)(w + L.kd); a.v = (const bf16*)v; a.gate = (const bf16*)gate; a.dO = (const bf16*)dO;
+  a.S0 = S0; a.z0 = z0; a.wq = (float*)(w + L.wq); a.wk = (float*)(w + L.wk); a.dvh = (float*)(w + L.dvh); a.dgate = (bf16*)dgate;
+  a.inv = (float*)(w + L.inv); a.delta = (float*)(w + L.delta); a.domax = (float*)(w + L.domax); a.z16 = (float*)(w + L.z16);
+  a.meta = (int*)(w + L.meta); a.s16 = (uint8_t*)(w + L.s16); a.wmax = (int*)(w + L.wmax); a.dev_status = c.dev_status;
+  a.B = p.B; a.T = p.T; a.H = p.H; a.Hkv = p.H_kv; a.gate_dim = p.gate_dim; a.gate_mode = p.gate_mode; a.normalize = p.normalize;
+  a.inv_tau = 1.f / p.gate_tau; a.eps = p.eps;
+  MArgs m{(const bf16*)q, (const bf16*)k, (const bf16*)w_q, (const bf16*)w_k, (const bf16*)W, (const bf16*)cache_q,
+          (const bf16*)cache_k, a.qd, a.kd, a.wk, a.wq, (float*)(w + L.du_k), dW, a.wmax, c.dev_status, p.B, p.T, p.H, p.H_kv, p.conv_k};
+  if (cudaMemsetAsync(a.wmax, 0, 4, c.stream) != cudaSuccess ||
+      cudaMemsetAsync(dW, 0, sizeof(float) * (size_t)p.H * p.d_k * p.d_k, c.stream) != cudaSuccess)
+    return LAWCAT_ERR_CUDA;
+  if ((r = launch_convmix_tc_fwd(c, q, k, w_q, w_k, W, cache_q, cache_k, (void*)a.qd, (void*)a.kd, true))) return r;
+  if ((r = p.d_k == 64 ? run<64>(c, a, m) : run<128>(c, a, m))) return r;
+  {
+    const int oct = p.d_v / 8;
+    const size_t total = (size_t)p.B * p.T * p.H_kv * oct;
+    LaunchScope _ls("dv_reduce", c.stream);
+    dv_sum_kernel<<<(unsigned)((total + 255) / 256), 256, 0, c.stream>>>(a.dvh, (bf16*)dv, total, p.H / p.H_kv, oct);
+    LAWCAT_CHECK_LAUNCH();
+  }
+  return launch_conv_only_bwd(c, q, k, w_q, w_k, cache_q, cache_k, a.wq, m.du_k, dq, dk, dw_q, dw_k);
+}
+
+}  // namespace lawcat

@@ -54,6 +54,54 @@ __device__ __forceinline__ void load_row8(const float* p, float* v) {
   v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
 }
 
+__device__ __forceinline__ float log2_sigmoid(float a) {
+  const float x = -a * 1.4426950408889634f;
+  return -fmaxf(x, lg2f(1.f + ex2f(fminf(x, 126.f))));
+}
+__device__ __forceinline__ uint4 pack8h(const float* v, bool f16) {
+  return f16 ? make_uint4(pack_f16(v[0], v[1]), pack_f16(v[2], v[3]), pack_f16(v[4], v[5]), pack_f16(v[6], v[7]))
+             : make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
+}
+// 16-bit values back to fp32
+__device__ __forceinline__ void unpack8h(const uint4& v, bool f16, float* f) {
+  if (f16) {
+    const __half2* h = reinterpret_cast<const __half2*>(&v);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float2 x = __half22float2(h[i]);
+      f[2 * i] = x.x; f[2 * i + 1] = x.y;
+    }
+  } else {
+    f[0] = bf16_lo(v.x); f[1] = bf16_hi(v.x); f[2] = bf16_lo(v.y); f[3] = bf16_hi(v.y);
+    f[4] = bf16_lo(v.z); f[5] = bf16_hi(v.z); f[6] = bf16_lo(v.w); f[7] = bf16_hi(v.w);
+  }
+}
+// v = hi + lo with hi the 16-bit rounding of v and lo the 16-bit rounding of the rest
+__device__ __forceinline__ void split8h(const float* v, bool f16, uint4& hi, uint4& lo) {
+  hi = pack8h(v, f16);
+  float h[8], r[8];
+  unpack8h(hi, f16, h);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) r[i] = v[i] - h[i];
+  lo = pack8h(r, f16);
+}
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr)
+               : "memory");
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const float* v) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+               ::"r"(taddr), "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])),
+                 "r"(__float_as_uint(v[3])), "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])),
+                 "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7]))
+               : "memory");
+}
+
 // one mbarrier, bounded wait (a product batch completes within microseconds; 2e8 cycles is about a tenth of a second)
 struct Waiter {
   uint32_t bar, phase;
@@ -90,6 +138,56 @@ __device__ __forceinline__ void load_w_tile(uint8_t* s_wt, const bf16* Wh, int t
     unpack8b(*reinterpret_cast<const uint4*>(Wh + (size_t)c * D + o * 8), f);
     *reinterpret_cast<uint4*>(s_wt + toff(L::SLAB_W, c, o * 8)) = pack8f16(f);
   }
+}
+
+// hint: fetch the 128-byte line at p towards L2 (these kernels walk their tiles in lock-step; the hint lets the next
+// tile's rows travel while the current one is computed)
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
+// conv of 8 channels (octet o) of N consecutive tokens from t on, straight from global memory with a window of raw rows
+// (rows before the sequence come from the conv cache or are zero, rows past its end are zero); emit(i, u) takes token t + i.
+// s_w: the head's taps, fp32 [D][4], in shared memory.
+template <int D, int N, typename F>
+__device__ __forceinline__ void conv_run(const bf16* x, const bf16* cache, const float* s_w, int b, int t, int T, int NH,
+                                         int head, int K, int o, F emit) {
+  uint4 raw[N + HALO];
+#pragma unroll
+  for (int i = 0; i < N + HALO; ++i) {
+    const int tt = t - HALO + i;
+    raw[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (tt >= 0 && tt < T)
+      raw[i] = *reinterpret_cast<const uint4*>(x + (((size_t)b * T + tt) * NH + head) * D + o * 8);
+    else if (tt < 0 && cache != nullptr && tt + (K - 1) >= 0)
+      raw[i] = *reinterpret_cast<const uint4*>(cache + (((size_t)b * (K - 1) + tt + (K - 1)) * NH + head) * D + o * 8);
+  }
+  float w[8][4];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const float4 t4 = *reinterpret_cast<const float4*>(s_w + (o * 8 + i) * 4);
+    w[i][0] = t4.x; w[i][1] = t4.y; w[i][2] = t4.z; w[i][3] = t4.w;
+  }
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    float u[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int dl = 0; dl < 4; ++dl) {
+      float xv[8];
+      unpack8b(raw[i + HALO - dl], xv);
+#pragma unroll
+      for (int c = 0; c < 8; ++c) u[c] = fmaf(w[c][dl], xv[c], u[c]);
+    }
+    emit(i, u);
+  }
+}
+
+// v rounded to bf16, and v -= the rounded value
+__device__ __forceinline__ uint4 take_bf16(float* v) {
+  const uint4 p = pack8bf16(v);
+  float h[8];
+  unpack8b(p, h);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] -= h[i];
+  return p;
 }
 
 }  // namespace ctc

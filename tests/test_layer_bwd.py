@@ -85,3 +85,34 @@ def test_c4_distillation_step_whole_layer(api):
     """The training configuration at full size (B = 8, T = 1024, 32/8 heads, d = 64): every gradient of the layer, from
     the raw inputs and the seeded upstream gradient, against the oracle's."""
     run(api, I.CONFIGS["c4"], False, True)
+
+
+@pytest.mark.parametrize("T,with_state", [(16, True), (64, False), (65, True), (129, False), (700, True)])
+def test_tensor_core_path_width_128(api, T, with_state):
+    run(api, I.LayerShape(2, T, 8, 2, 128, 128, dtype="bf16", config_id=86), with_state, True)
+
+
+@pytest.mark.parametrize("kw", [dict(gate_dim=1), dict(conv_k=2), dict(H=4, H_kv=4), dict(H=2, H_kv=1), dict(gate_tau=8.0)])
+def test_tensor_core_path_width_128_variants(api, kw):
+    base = dict(B=1, T=300, H=4, H_kv=2, d_k=128, d_v=128, dtype="bf16", config_id=87)
+    base.update(kw)
+    run(api, I.LayerShape(**base), True, True)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("scale", [1e-6, 1e4])
+def test_gradient_scale(api, d, scale):
+    """Every gradient is linear in dO: a power-of-two-free scaling of dO (a loss scale, or the lack of one) must pass through
+    the 16-bit operands unharmed."""
+    import torch
+    s = I.LayerShape(1, 150, 4, 2, d, d, dtype="bf16", config_id=88)
+    x = I.make(s, NAMES + ["dO"])
+    x["dO"] = I.round_to_bf16(x["dO"] * np.float32(scale))
+    t = {n: api.to_device(v, s.dtype) for n, v in x.items()}
+    g = api.lawcat_layer_bwd(P(api, s), *[t[n] for n in NAMES], t["dO"])
+    torch.cuda.synchronize()
+    ref = oracle_layer_gradients(s, x)
+    for n in ("dq", "dk", "dv", "dgate"):
+        check(g[n], ref[n], "bf16", n)
+    for n in ("dw_q", "dw_k", "dW"):
+        check(g[n], ref[n], "bf16", n, f32_store=True)
