@@ -222,7 +222,7 @@ int lawcat_gla_bwd(const lawcat_params* p, const void* qdot, const void* kdot, c
   if (need && (!ws || ws_bytes < need)) return LAWCAT_ERR_WORKSPACE_TOO_SMALL;
   Ctx c{p, (cudaStream_t)stream, dev_status};
   if ((size_t)p->B * p->T != 0 && gla_tc_bwd_supported(*p))  // chunkwise tensor-core kernel
-    return launch_gla_bwd_tc(c, qdot, kdot, v, gate, S0, z0, dO, d_qdot, d_kdot, dv, dgate, ws, false);
+    return launch_gla_bwd_tc(c, qdot, kdot, v, gate, S0, z0, dO, d_qdot, d_kdot, dv, dgate, ws);
   return launch_gla_bwd_rec(c, qdot, kdot, v, gate, S0, z0, o, den, dO, d_qdot, d_kdot, dv, dgate, ws);
 }
 
@@ -379,7 +379,7 @@ int lawcat_layer_bwd(const lawcat_params* p, const void* q, const void* k, const
       return r;
   }
   if ((r = launch_conv_bwd(c32, in[0], in[1], in[4], in[5], in[6], in[8], in[9], w + L.dqd, w + L.dkd, out[0], out[1], dw_q,
-                           dw_k, dW, w + L.ws_c, false)))
+                           dw_k, dW, w + L.ws_c)))
     return r;
   if (widen) {
     void* dst[4] = {dq, dk, dv, dgate};

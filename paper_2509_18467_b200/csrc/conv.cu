@@ -447,11 +447,125 @@ static int conv_bwd_stream(const Ctx& c, const TD* du, const TI* x, const TI* w,
   return LAWCAT_OK;
 }
 
+// The same for bf16 storage, conv width up to 4 and fp32 du (whole-layer and mix backward), both streams in one launch, four
+// channels per thread: 16-byte loads of du and 8-byte loads of x, a group of 8 tokens in flight. Bound by HBM: du and x in, dx
+// out. One channel per thread, a launch per stream: 129 us at 8 x 1024 tokens, 32/8 heads of 64 (166 MB); this form CONVBW_US.
+constexpr int CB4_SPAN = 32;
+struct ConvBwd4 {
+  const float* du[2];
+  const bf16 *x[2], *w[2], *cache[2];
+  bf16* dx[2];
+  float* dw[2];
+  int C[2];      // channels per stream
+  int B, T, K;
+};
+__device__ __forceinline__ void bf16x4(const uint2& r, float* f) {
+  f[0] = __uint_as_float(r.x << 16); f[1] = __uint_as_float(r.x & 0xffff0000u);
+  f[2] = __uint_as_float(r.y << 16); f[3] = __uint_as_float(r.y & 0xffff0000u);
+}
+__global__ void __launch_bounds__(128) conv_bwd4_kernel(const ConvBwd4 a) {
+  int cq = blockIdx.y * 128 + threadIdx.x;
+  const int st = cq >= a.C[0] / 4;
+  if (st) cq -= a.C[0] / 4;
+  const int C = st ? a.C[1] : a.C[0], ch = 4 * cq, K = a.K, T = a.T;
+  if (ch >= C) return;
+  const float* du = st ? a.du[1] : a.du[0];
+  const bf16* x = st ? a.x[1] : a.x[0];
+  const bf16* w = st ? a.w[1] : a.w[0];
+  const bf16* cache = st ? a.cache[1] : a.cache[0];
+  bf16* dx = st ? a.dx[1] : a.dx[0];
+  float* dw = st ? a.dw[1] : a.dw[0];
+  const int spans = (T + CB4_SPAN - 1) / CB4_SPAN, b = blockIdx.x / spans, t0 = blockIdx.x % spans * CB4_SPAN;
+  const int t1 = min(T, t0 + CB4_SPAN);
+  const float* dub = du + (size_t)b * T * C + ch;
+  const bf16* xb = x + (size_t)b * T * C + ch;
+  float tap[4][4], acc[4][4], xw[3][4], dwin[3][4];  // [delta][channel]; x[t - 1 - i], du[t + i]
+#pragma unroll
+  for (int d = 0; d < 4; ++d)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      tap[d][c] = d < K ? ldf(w + (size_t)(ch + c) * K + d) : 0.f;
+      acc[d][c] = 0.f;
+    }
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    uint2 r = make_uint2(0u, 0u);
+    const int t = t0 - 1 - i;
+    if (t >= 0) r = *reinterpret_cast<const uint2*>(xb + (size_t)t * C);
+    else if (cache && t + K - 1 >= 0) r = *reinterpret_cast<const uint2*>(cache + ((size_t)b * (K - 1) + t + K - 1) * C + ch);
+    bf16x4(r, xw[i]);
+    float4 g = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (t0 + i < T) g = *reinterpret_cast<const float4*>(dub + (size_t)(t0 + i) * C);
+    dwin[i][0] = g.x; dwin[i][1] = g.y; dwin[i][2] = g.z; dwin[i][3] = g.w;
+  }
+  for (int tg = t0; tg < t1; tg += 8) {
+    float4 ahead[8];
+    uint2 xin[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int t = tg + i;
+      ahead[i] = t < t1 && t + 3 < T ? *reinterpret_cast<const float4*>(dub + (size_t)(t + 3) * C) : make_float4(0.f, 0.f, 0.f, 0.f);
+      xin[i] = t < t1 ? *reinterpret_cast<const uint2*>(xb + (size_t)t * C) : make_uint2(0u, 0u);
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      if (tg + i >= t1) break;
+      const float ah[4] = {ahead[i].x, ahead[i].y, ahead[i].z, ahead[i].w};
+      float xc[4], o[4];
+      bf16x4(xin[i], xc);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const float g = dwin[0][c];
+        o[c] = fmaf(tap[0][c], g, fmaf(tap[1][c], dwin[1][c], fmaf(tap[2][c], dwin[2][c], tap[3][c] * ah[c])));
+        acc[0][c] = fmaf(g, xc[c], acc[0][c]);
+        acc[1][c] = fmaf(g, xw[0][c], acc[1][c]);
+        acc[2][c] = fmaf(g, xw[1][c], acc[2][c]);
+        acc[3][c] = fmaf(g, xw[2][c], acc[3][c]);
+        dwin[0][c] = dwin[1][c]; dwin[1][c] = dwin[2][c]; dwin[2][c] = ah[c];
+        xw[2][c] = xw[1][c]; xw[1][c] = xw[0][c]; xw[0][c] = xc[c];
+      }
+      if (dx) {
+        const __nv_bfloat162 p0 = __floats2bfloat162_rn(o[0], o[1]), p1 = __floats2bfloat162_rn(o[2], o[3]);
+        *reinterpret_cast<uint2*>(dx + ((size_t)b * T + tg + i) * C + ch) =
+            make_uint2(*reinterpret_cast<const uint32_t*>(&p0), *reinterpret_cast<const uint32_t*>(&p1));
+      }
+    }
+  }
+  if (dw) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+      for (int d = 0; d < 4; ++d)
+        if (d < K) atomicAdd(dw + (size_t)(ch + c) * K + d, acc[d][c]);
+  }
+}
+
+// the conv's backward of both streams from fp32 du
+template <typename TI>
+static int conv_bwd_both(const Ctx& c, const float* du_q, const float* du_k, const void* q, const void* k, const void* w_q,
+                         const void* w_k, const void* cache_q, const void* cache_k, void* dq, void* dk, float* dw_q, float* dw_k) {
+  const lawcat_params& p = *c.p;
+  if (!std::is_same<TI, bf16>::value || p.conv_k > 4) {
+    const int r = conv_bwd_stream<TI, float>(c, du_q, (const TI*)q, (const TI*)w_q, (const TI*)cache_q, (TI*)dq, dw_q, p.H);
+    if (r) return r;
+    return conv_bwd_stream<TI, float>(c, du_k, (const TI*)k, (const TI*)w_k, (const TI*)cache_k, (TI*)dk, dw_k, p.H_kv);
+  }
+  const int Cq = p.H * p.d_k, Ck = p.H_kv * p.d_k;
+  if (dw_q && cudaMemsetAsync(dw_q, 0, sizeof(float) * (size_t)Cq * p.conv_k, c.stream) != cudaSuccess) return LAWCAT_ERR_CUDA;
+  if (dw_k && cudaMemsetAsync(dw_k, 0, sizeof(float) * (size_t)Ck * p.conv_k, c.stream) != cudaSuccess) return LAWCAT_ERR_CUDA;
+  const ConvBwd4 a{{du_q, du_k}, {(const bf16*)q, (const bf16*)k}, {(const bf16*)w_q, (const bf16*)w_k},
+                   {(const bf16*)cache_q, (const bf16*)cache_k}, {(bf16*)dq, (bf16*)dk}, {dw_q, dw_k}, {Cq, Ck}, p.B, p.T, p.conv_k};
+  const dim3 grid(p.B * ((p.T + CB4_SPAN - 1) / CB4_SPAN), ((Cq + Ck) / 4 + 127) / 128);
+  LaunchScope _ls("conv_bwd", c.stream);
+  conv_bwd4_kernel<<<grid, 128, 0, c.stream>>>(a);
+  LAWCAT_CHECK_LAUNCH();
+  return LAWCAT_OK;
+}
+
 template <typename TI>
 static int conv_bwd_typed(const Ctx& c, const void* q, const void* k, const void* w_q, const void* w_k,
                           const void* W, const void* cache_q, const void* cache_k, const void* d_qdot,
-                          const void* d_kdot, void* dq, void* dk, float* dw_q, float* dw_k, float* dW, void* ws,
-                          bool grads_f32) {
+                          const void* d_kdot, void* dq, void* dk, float* dw_q, float* dw_k, float* dW, void* ws) {
   const lawcat_params& p = *c.p;
   if (p.B * p.T == 0) {
     if (dw_q && cudaMemsetAsync(dw_q, 0, sizeof(float) * (size_t)p.H * p.d_k * p.conv_k, c.stream)) return LAWCAT_ERR_CUDA;
@@ -474,13 +588,10 @@ static int conv_bwd_typed(const Ctx& c, const void* q, const void* k, const void
                    p.B, p.T, p.H, p.H_kv, p.conv_k, p.phi, p.mix_unshared};
   if (std::is_same<TI, bf16>::value && convmix_tc_bwd_supported(p) && p.chunk != 1) {
     // tensor-core kernel for the mix and the softmax Jacobian; the conv's own backward follows on du as below
-    int r0 = launch_convmix_tc_bwd(c, q, k, w_q, w_k, W, cache_q, cache_k, d_qdot, d_kdot, grads_f32, du_q, du_k, dW);
+    int r0 = launch_convmix_tc_bwd(c, q, k, w_q, w_k, W, cache_q, cache_k, d_qdot, d_kdot, du_q, du_k, dW);
     if (r0) return r0;
-    r0 = conv_bwd_stream<TI, float>(c, du_q, (const TI*)q, (const TI*)w_q, (const TI*)cache_q, (TI*)dq, dw_q, p.H);
-    if (r0) return r0;
-    return conv_bwd_stream<TI, float>(c, du_k, (const TI*)k, (const TI*)w_k, (const TI*)cache_k, (TI*)dk, dw_k, p.H_kv);
+    return conv_bwd_both<TI>(c, du_q, du_k, q, k, w_q, w_k, cache_q, cache_k, dq, dk, dw_q, dw_k);
   }
-  if (grads_f32) return LAWCAT_ERR_UNSUPPORTED;  // (fp32 gradients only reach the tensor-core kernel)
   dim3 grid(p.B * ((p.T + CB_SPAN - 1) / CB_SPAN), p.H_kv);
 #define LAUNCH_CB(D)                                                                                             \
   do {                                                                                                           \
@@ -500,67 +611,64 @@ static int conv_bwd_typed(const Ctx& c, const void* q, const void* k, const void
   }
 #undef LAUNCH_CB
   LAWCAT_CHECK_LAUNCH();
-  int r = conv_bwd_stream<TI, float>(c, du_q, (const TI*)q, (const TI*)w_q, (const TI*)cache_q, (TI*)dq, dw_q, p.H);
-  if (r) return r;
-  return conv_bwd_stream<TI, float>(c, du_k, (const TI*)k, (const TI*)w_k, (const TI*)cache_k, (TI*)dk, dw_k,
-                                    p.H_kv);
+  return conv_bwd_both<TI>(c, du_q, du_k, q, k, w_q, w_k, cache_q, cache_k, dq, dk, dw_q, dw_k);
 }
 
 int launch_conv_bwd(const Ctx& c, const void* q, const void* k, const void* w_q, const void* w_k, const void* W,
                     const void* cache_q, const void* cache_k, const void* d_qdot, const void* d_kdot, void* dq,
-                    void* dk, float* dw_q, float* dw_k, float* dW, void* ws, bool grads_f32) {
+                    void* dk, float* dw_q, float* dw_k, float* dW, void* ws) {
   if (c.p->dtype == LAWCAT_F32)
-    return conv_bwd_typed<float>(c, q, k, w_q, w_k, W, cache_q, cache_k, d_qdot, d_kdot, dq, dk, dw_q, dw_k, dW, ws, false);
-  return conv_bwd_typed<bf16>(c, q, k, w_q, w_k, W, cache_q, cache_k, d_qdot, d_kdot, dq, dk, dw_q, dw_k, dW, ws, grads_f32);
+    return conv_bwd_typed<float>(c, q, k, w_q, w_k, W, cache_q, cache_k, d_qdot, d_kdot, dq, dk, dw_q, dw_k, dW, ws);
+  return conv_bwd_typed<bf16>(c, q, k, w_q, w_k, W, cache_q, cache_k, d_qdot, d_kdot, dq, dk, dw_q, dw_k, dW, ws);
 }
 
 // the conv's own backward alone, on fp32 gradients of both conv outputs (bf16 storage)
 int launch_conv_only_bwd(const Ctx& c, const void* q, const void* k, const void* w_q, const void* w_k, const void* cache_q,
                          const void* cache_k, const float* du_q, const float* du_k, void* dq, void* dk, float* dw_q, float* dw_k) {
-  const int r = conv_bwd_stream<bf16, float>(c, du_q, (const bf16*)q, (const bf16*)w_q, (const bf16*)cache_q, (bf16*)dq, dw_q, c.p->H);
-  if (r) return r;
-  return conv_bwd_stream<bf16, float>(c, du_k, (const bf16*)k, (const bf16*)w_k, (const bf16*)cache_k, (bf16*)dk, dw_k, c.p->H_kv);
+  return conv_bwd_both<bf16>(c, du_q, du_k, q, k, w_q, w_k, cache_q, cache_k, dq, dk, dw_q, dw_k);
 }
 
 // ------------------------------------------------------------------------------------------------ conv cache out
 // cache_out[b,r,:] = token T-(K-1)+r of the stream [cache_in, x] (Section 4.1: the cache is bounded by the kernel size)
+// Both streams in one launch; thread = one entry of a row of C = (H + H_kv) d_k channels.
 template <typename T>
-__global__ void cache_out_kernel(const T* __restrict__ x, const T* __restrict__ cin, T* __restrict__ cout, int B,
-                                 int Tn, int C, int K) {
+__global__ void cache_out_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ cin_q,
+                                 const T* __restrict__ cin_k, T* __restrict__ cout_q, T* __restrict__ cout_k, int B, int Tn, int Cq,
+                                 int Ck, int K) {
   const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (size_t)B * (K - 1) * C) return;
-  const int ch = (int)(idx % C);
-  const int r = (int)((idx / C) % (K - 1));
-  const int b = (int)(idx / ((size_t)C * (K - 1)));
-  const int tok = Tn - (K - 1) + r;
+  const int Ct = Cq + Ck;
+  if (idx >= (size_t)B * (K - 1) * Ct) return;
+  int ch = (int)(idx % Ct);
+  const int r = (int)((idx / Ct) % (K - 1)), b = (int)(idx / ((size_t)Ct * (K - 1)));
+  const bool key = ch >= Cq;
+  if (key) ch -= Cq;
+  const int C = key ? Ck : Cq, tok = Tn - (K - 1) + r;
+  const T *x = key ? k : q, *cin = key ? cin_k : cin_q;
+  T* cout = key ? cout_k : cout_q;
+  if (!cout) return;
   T val;
   if (tok >= 0) val = x[((size_t)b * Tn + tok) * C + ch];
   else if (cin) val = cin[((size_t)b * (K - 1) + (tok + K - 1)) * C + ch];
   else stf(&val, 0.f);
-  cout[idx] = val;
-}
-
-template <typename T>
-static int cache_out_typed(const Ctx& c, const void* x, const void* cin, void* cout, int NH) {
-  const lawcat_params& p = *c.p;
-  const size_t total = (size_t)p.B * (p.conv_k - 1) * NH * p.d_k;
-  if (!cout || total == 0) return LAWCAT_OK;
-  LaunchScope _ls("cache_out", c.stream);
-  cache_out_kernel<T><<<(unsigned)((total + 255) / 256), 256, 0, c.stream>>>((const T*)x, (const T*)cin, (T*)cout,
-                                                                              p.B, p.T, NH * p.d_k, p.conv_k);
-  LAWCAT_CHECK_LAUNCH();
-  return LAWCAT_OK;
+  cout[((size_t)b * (K - 1) + r) * C + ch] = val;
 }
 
 int launch_cache_out(const Ctx& c, const void* q, const void* k, const void* cache_q_in, const void* cache_k_in,
                      void* cache_q_out, void* cache_k_out) {
-  int r;
-  if (c.p->dtype == LAWCAT_F32) {
-    if ((r = cache_out_typed<float>(c, q, cache_q_in, cache_q_out, c.p->H))) return r;
-    return cache_out_typed<float>(c, k, cache_k_in, cache_k_out, c.p->H_kv);
-  }
-  if ((r = cache_out_typed<bf16>(c, q, cache_q_in, cache_q_out, c.p->H))) return r;
-  return cache_out_typed<bf16>(c, k, cache_k_in, cache_k_out, c.p->H_kv);
+  const lawcat_params& p = *c.p;
+  const int Cq = p.H * p.d_k, Ck = p.H_kv * p.d_k;
+  const size_t total = (size_t)p.B * (p.conv_k - 1) * (Cq + Ck);
+  if ((!cache_q_out && !cache_k_out) || total == 0) return LAWCAT_OK;
+  const unsigned blocks = (unsigned)((total + 255) / 256);
+  LaunchScope _ls("cache_out", c.stream);
+  if (p.dtype == LAWCAT_F32)
+    cache_out_kernel<float><<<blocks, 256, 0, c.stream>>>((const float*)q, (const float*)k, (const float*)cache_q_in, (const float*)cache_k_in,
+                                                          (float*)cache_q_out, (float*)cache_k_out, p.B, p.T, Cq, Ck, p.conv_k);
+  else
+    cache_out_kernel<bf16><<<blocks, 256, 0, c.stream>>>((const bf16*)q, (const bf16*)k, (const bf16*)cache_q_in, (const bf16*)cache_k_in,
+                                                         (bf16*)cache_q_out, (bf16*)cache_k_out, p.B, p.T, Cq, Ck, p.conv_k);
+  LAWCAT_CHECK_LAUNCH();
+  return LAWCAT_OK;
 }
 
 }  // namespace lawcat

@@ -26,7 +26,7 @@ namespace ctc {
 struct CArgs {
   const bf16 *q, *k, *w_q, *w_k, *W, *cache_q, *cache_k;
   void *qdot, *kdot;                 // forward outputs (bf16 or fp32)
-  const void *d_qdot, *d_kdot;       // backward inputs (bf16 or fp32)
+  const void *d_qdot, *d_kdot;       // backward inputs
   float *du_q, *du_k, *dW;           // backward outputs: d(conv out) per stream (fp32), dW (fp32, atomic adds)
   int* dev_status;
   int B, T, H, Hkv, K, phi;
@@ -252,9 +252,9 @@ __global__ void __launch_bounds__(256) convmix_tc_fwd_kernel(const CArgs a) {
 }
 
 // Backward through phi and the mix for head width 64: du_q [B,T,H,64], du_k [B,T,Hkv,64] (fp32), dW [H,64,64] (atomic adds
-// into a zeroed array). TG: type of the incoming gradients d_qdot, d_kdot.
-template <typename TG>
+// into a zeroed array).
 __global__ void __launch_bounds__(128, 2) convmix_tc_bwd_kernel(const CArgs a) {
+  typedef bf16 TG;  // of the incoming gradients
   constexpr int D = 64;
   using L = Lay<D>;
   extern __shared__ __align__(128) uint8_t sg[];
@@ -517,9 +517,9 @@ int launch_convmix_tc_fwd(const Ctx& c, const void* q, const void* k, const void
   return LAWCAT_OK;
 }
 
-// du_q, du_k (fp32) and dW (atomic adds into the caller-zeroed array) from d_qdot, d_kdot (bf16, or fp32 when grads_f32)
+// du_q, du_k (fp32) and dW (atomic adds into the caller-zeroed array) from d_qdot, d_kdot
 int launch_convmix_tc_bwd(const Ctx& c, const void* q, const void* k, const void* w_q, const void* w_k, const void* W,
-                          const void* cache_q, const void* cache_k, const void* d_qdot, const void* d_kdot, bool grads_f32,
+                          const void* cache_q, const void* cache_k, const void* d_qdot, const void* d_kdot,
                           float* du_q, float* du_k, float* dW) {
   using namespace ctc;
   const lawcat_params& p = *c.p;
@@ -532,14 +532,13 @@ int launch_convmix_tc_bwd(const Ctx& c, const void* q, const void* k, const void
   {
     std::lock_guard<std::mutex> lk(mu);
     if (!done[dev]) {
-      if (raise_smem(convmix_tc_bwd_kernel<bf16>, bwd_smem()) || raise_smem(convmix_tc_bwd_kernel<float>, bwd_smem())) return LAWCAT_ERR_CUDA;
+      if (raise_smem(convmix_tc_bwd_kernel, bwd_smem())) return LAWCAT_ERR_CUDA;
       done[dev] = true;
     }
   }
   const dim3 grid((unsigned)((p.T + TT - 1) / TT), (unsigned)(p.B * p.H_kv));
   LaunchScope _ls("convmix_tc_bwd", c.stream);
-  if (grads_f32) convmix_tc_bwd_kernel<float><<<grid, 128, bwd_smem(), c.stream>>>(a);
-  else convmix_tc_bwd_kernel<bf16><<<grid, 128, bwd_smem(), c.stream>>>(a);
+  convmix_tc_bwd_kernel<<<grid, 128, bwd_smem(), c.stream>>>(a);
   LAWCAT_CHECK_LAUNCH();
   return LAWCAT_OK;
 }

@@ -100,12 +100,12 @@ constexpr uint32_t COL_P = 0, COL_A = 64 /* O' | dQ */, COL_ST = 144 /* S' or R 
                    COL_V = 384 /* dV */;
 
 struct GArgs {
-  const void *qdot, *kdot;   // features: bf16, or fp32 when feat_f32 (scratch of the fused layer backward)
+  const void *qdot, *kdot;   // features: bf16, or fp32 when feat_f32 (scratch of a fused layer forward)
   const bf16 *v, *gate, *dO;
   const float *S0, *z0;
   bf16* o;
   float *den, *S_T, *z_T;
-  void *d_qdot, *d_kdot;     // bf16, or fp32 when feat_f32
+  void *d_qdot, *d_kdot;     // bf16
   bf16* dgate;
   int feat_f32;
   float* dvh;         // [B,T,H,D] per-head dv (fp32), reduced over the heads of a group afterwards
@@ -724,17 +724,8 @@ __global__ void __launch_bounds__(THREADS, MODE == 2 ? 1 : 2) gla_tc_kernel(cons
           *reinterpret_cast<float4*>(s_dt + row * D + c0) = make_float4(dd[0], dd[1], dd[2], dd[3]);
           *reinterpret_cast<float4*>(s_dt + row * D + c0 + 4) = make_float4(dd[4], dd[5], dd[6], dd[7]);
           if (valid) {
-            if (a.feat_f32) {
-              float* gq = reinterpret_cast<float*>(a.d_qdot) + th * D + c0;
-              float* gk = reinterpret_cast<float*>(a.d_kdot) + th * D + c0;
-              *reinterpret_cast<float4*>(gq) = make_float4(dq[0], dq[1], dq[2], dq[3]);
-              *reinterpret_cast<float4*>(gq + 4) = make_float4(dq[4], dq[5], dq[6], dq[7]);
-              *reinterpret_cast<float4*>(gk) = make_float4(dk[0], dk[1], dk[2], dk[3]);
-              *reinterpret_cast<float4*>(gk + 4) = make_float4(dk[4], dk[5], dk[6], dk[7]);
-            } else {
-              *reinterpret_cast<uint4*>(reinterpret_cast<bf16*>(a.d_qdot) + th * D + c0) = pack8h(dq, false);
-              *reinterpret_cast<uint4*>(reinterpret_cast<bf16*>(a.d_kdot) + th * D + c0) = pack8h(dk, false);
-            }
+            *reinterpret_cast<uint4*>(reinterpret_cast<bf16*>(a.d_qdot) + th * D + c0) = pack8h(dq, false);
+            *reinterpret_cast<uint4*>(reinterpret_cast<bf16*>(a.d_kdot) + th * D + c0) = pack8h(dk, false);
             *reinterpret_cast<float4*>(a.dvh + th * D + c0) = make_float4(dvv[0], dvv[1], dvv[2], dvv[3]);
             *reinterpret_cast<float4*>(a.dvh + th * D + c0 + 4) = make_float4(dvv[4], dvv[5], dvv[6], dvv[7]);
           }
@@ -887,8 +878,7 @@ int launch_gla_fwd_tc(const Ctx& c, const void* qdot, const void* kdot, const vo
 }
 
 int launch_gla_bwd_tc(const Ctx& c, const void* qdot, const void* kdot, const void* v, const void* gate, const float* S0,
-                      const float* z0, const void* dO, void* d_qdot, void* d_kdot, void* dv, void* dgate, void* ws,
-                      bool feat_f32) {
+                      const float* z0, const void* dO, void* d_qdot, void* d_kdot, void* dv, void* dgate, void* ws) {
   using namespace gtc;
   const lawcat_params& p = *c.p;
   int r = set_smem_once();
@@ -896,7 +886,7 @@ int launch_gla_bwd_tc(const Ctx& c, const void* qdot, const void* kdot, const vo
   GArgs a = gla_tc_args(c);
   a.qdot = qdot; a.kdot = kdot; a.v = (const bf16*)v; a.gate = (const bf16*)gate;
   a.dO = (const bf16*)dO; a.S0 = S0; a.z0 = z0;
-  a.d_qdot = d_qdot; a.d_kdot = d_kdot; a.dgate = (bf16*)dgate; a.feat_f32 = feat_f32 ? 1 : 0;
+  a.d_qdot = d_qdot; a.d_kdot = d_kdot; a.dgate = (bf16*)dgate;
   const size_t bth = (size_t)p.B * p.T * p.H;
   char* w = (char*)ws;
   a.dvh = (float*)w; w += align_up(sizeof(float) * bth * D, 256);

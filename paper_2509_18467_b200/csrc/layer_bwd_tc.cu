@@ -156,6 +156,25 @@ __device__ __forceinline__ void gate_pass(const Args& a, size_t row0, int h, int
   __syncthreads();
 }
 
+// one chunk's rows towards L2: the chunk that follows travels while this one is computed
+template <int D>
+__device__ __forceinline__ void prefetch_chunk(const Args& a, int b, int h, int j, int t0, int tid) {
+  constexpr int LF = D * 4 / 128, LB = D * 2 / 128, PER = 2 * LF + 3 * LB;  // 128-byte lines per token
+  if (t0 < 0) return;
+  for (int idx = tid; idx < C * PER; idx += Cfg<D>::THREADS) {
+    const int r = idx / PER, l = idx % PER;
+    if (t0 + r >= a.T) return;
+    const size_t th = ((size_t)b * a.T + t0 + r) * a.H + h, tv = ((size_t)b * a.T + t0 + r) * a.Hkv + j;
+    const char* p;
+    if (l < LF) p = (const char*)(a.qd + th * D) + l * 128;
+    else if (l < 2 * LF) p = (const char*)(a.kd + th * D) + (l - LF) * 128;
+    else if (l < 2 * LF + LB) p = (const char*)(a.v + tv * D) + (l - 2 * LF) * 128;
+    else if (l < 2 * LF + 2 * LB) p = (const char*)(a.dO + th * D) + (l - 2 * LF - LB) * 128;
+    else p = (const char*)(a.gate + th * a.gate_dim) + (l - 2 * LF - 2 * LB) * 128 * (a.gate_dim > 1);
+    prefetch_l2(p);
+  }
+}
+
 // products on two-term operands, issued by one thread: D (+)= A B with A = ah + al, B = bh + bl (a missing low part is 0)
 struct Mma {
   uint32_t tmem;
@@ -248,6 +267,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) sweep_kerne
   for (int n = 0; n < nch; ++n) {
     const int t0 = n * C, nvalid = min(C, a.T - t0);
     const size_t row0 = (size_t)b * a.T + t0;
+    if (n + 1 < nch) prefetch_chunk<D>(a, b, h, j, t0 + C, tid);
     gate_pass<D>(a, row0, h, nvalid, s_x, s_bm, s_ft, const_cast<int*>(&s_fl[2]), tid);
     const bool f16 = __int_as_float(s_fl[2]) <= RMAX_F16;
     const int fmt = f16 ? FMT_F16 : FMT_BF16;
@@ -492,6 +512,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
     const size_t row0 = (size_t)b * a.T + t0;
     const int kap = a.meta[((size_t)bh * nch + n) * 2], fmt = a.meta[((size_t)bh * nch + n) * 2 + 1];
     const bool f16 = fmt == FMT_F16;
+    prefetch_chunk<D>(a, b, h, j, t0 - C, tid);
     // ---- row scalars; the largest inv of the chunk and the largest entry of the adjoint decide 2^al
     if (tid == 0) s_fl[3] = s_fl[4] = 0;
     __syncthreads();
