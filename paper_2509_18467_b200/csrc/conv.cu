@@ -464,19 +464,20 @@ __device__ __forceinline__ void bf16x4(const uint2& r, float* f) {
   f[2] = __uint_as_float(r.y << 16); f[3] = __uint_as_float(r.y & 0xffff0000u);
 }
 __global__ void __launch_bounds__(128) conv_bwd4_kernel(const ConvBwd4 a) {
-  int cq = blockIdx.y * 128 + threadIdx.x;
-  const int st = cq >= a.C[0] / 4;
-  if (st) cq -= a.C[0] / 4;
-  const int C = st ? a.C[1] : a.C[0], ch = 4 * cq, K = a.K, T = a.T;
-  if (ch >= C) return;
+  // warp = one of four neighbouring spans of the same 128 channels (C is a multiple of 16: a lane may be past the end)
+  __shared__ float s_dw[3][16][33];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, qb = (a.C[0] / 4 + 31) / 32;
+  const int st = (int)blockIdx.y >= qb;
+  const int C = st ? a.C[1] : a.C[0], ch = 4 * (((int)blockIdx.y - (st ? qb : 0)) * 32 + lane), K = a.K, T = a.T;
+  const int spans = (T + CB4_SPAN - 1) / CB4_SPAN, sg = (int)blockIdx.x * 4 + warp;
+  const bool on = ch < C && sg < a.B * spans;
   const float* du = st ? a.du[1] : a.du[0];
   const bf16* x = st ? a.x[1] : a.x[0];
   const bf16* w = st ? a.w[1] : a.w[0];
   const bf16* cache = st ? a.cache[1] : a.cache[0];
   bf16* dx = st ? a.dx[1] : a.dx[0];
   float* dw = st ? a.dw[1] : a.dw[0];
-  const int spans = (T + CB4_SPAN - 1) / CB4_SPAN, b = blockIdx.x / spans, t0 = blockIdx.x % spans * CB4_SPAN;
-  const int t1 = min(T, t0 + CB4_SPAN);
+  const int b = on ? sg / spans : 0, t0 = on ? sg % spans * CB4_SPAN : 0, t1 = on ? min(T, t0 + CB4_SPAN) : 0;
   const float* dub = du + (size_t)b * T * C + ch;
   const bf16* xb = x + (size_t)b * T * C + ch;
   float tap[4][4], acc[4][4], xw[3][4], dwin[3][4];  // [delta][channel]; x[t - 1 - i], du[t + i]
@@ -484,11 +485,12 @@ __global__ void __launch_bounds__(128) conv_bwd4_kernel(const ConvBwd4 a) {
   for (int d = 0; d < 4; ++d)
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-      tap[d][c] = d < K ? ldf(w + (size_t)(ch + c) * K + d) : 0.f;
+      tap[d][c] = on && d < K ? ldf(w + (size_t)(ch + c) * K + d) : 0.f;
       acc[d][c] = 0.f;
     }
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
+    if (!on) break;
     uint2 r = make_uint2(0u, 0u);
     const int t = t0 - 1 - i;
     if (t >= 0) r = *reinterpret_cast<const uint2*>(xb + (size_t)t * C);
@@ -531,12 +533,27 @@ __global__ void __launch_bounds__(128) conv_bwd4_kernel(const ConvBwd4 a) {
       }
     }
   }
-  if (dw) {
+  // dw: the four spans meet in shared memory, one add per channel and tap goes out
+  if (warp > 0) {
 #pragma unroll
     for (int c = 0; c < 4; ++c)
 #pragma unroll
+      for (int d = 0; d < 4; ++d) s_dw[warp - 1][4 * c + d][lane] = acc[d][c];
+  }
+  __syncthreads();
+  if (warp > 0 || ch >= C || !dw) return;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+#pragma unroll
+    for (int d = 0; d < 4; ++d) acc[d][c] += s_dw[0][4 * c + d][lane] + s_dw[1][4 * c + d][lane] + s_dw[2][4 * c + d][lane];
+    float* const dst = dw + (size_t)(ch + c) * K;
+    if (K == 4) {
+      asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst), "f"(acc[0][c]), "f"(acc[1][c]), "f"(acc[2][c]), "f"(acc[3][c]) : "memory");
+    } else {
+#pragma unroll
       for (int d = 0; d < 4; ++d)
-        if (d < K) atomicAdd(dw + (size_t)(ch + c) * K + d, acc[d][c]);
+        if (d < K) atomicAdd(dst + d, acc[d][c]);
+    }
   }
 }
 
@@ -555,7 +572,7 @@ static int conv_bwd_both(const Ctx& c, const float* du_q, const float* du_k, con
   if (dw_k && cudaMemsetAsync(dw_k, 0, sizeof(float) * (size_t)Ck * p.conv_k, c.stream) != cudaSuccess) return LAWCAT_ERR_CUDA;
   const ConvBwd4 a{{du_q, du_k}, {(const bf16*)q, (const bf16*)k}, {(const bf16*)w_q, (const bf16*)w_k},
                    {(const bf16*)cache_q, (const bf16*)cache_k}, {(bf16*)dq, (bf16*)dk}, {dw_q, dw_k}, {Cq, Ck}, p.B, p.T, p.conv_k};
-  const dim3 grid(p.B * ((p.T + CB4_SPAN - 1) / CB4_SPAN), ((Cq + Ck) / 4 + 127) / 128);
+  const dim3 grid((p.B * ((p.T + CB4_SPAN - 1) / CB4_SPAN) + 3) / 4, (Cq / 4 + 31) / 32 + (Ck / 4 + 31) / 32);
   LaunchScope _ls("conv_bwd", c.stream);
   conv_bwd4_kernel<<<grid, 128, 0, c.stream>>>(a);
   LAWCAT_CHECK_LAUNCH();
