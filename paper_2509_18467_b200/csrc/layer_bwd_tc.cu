@@ -104,8 +104,10 @@ __device__ __forceinline__ void gate_pass(const Args& a, size_t row0, int h, int
   using F = Cfg<D>;
   const float L2E = 1.4426950408889634f;
   if (tid == 0) *rmax = 0;
-  for (int idx = tid; idx < C * F::OCT; idx += F::THREADS) {
-    const int o = idx % F::OCT, r = idx / F::OCT;
+  static_assert(C * F::OCT == 2 * F::THREADS, "two octets per thread");
+#pragma unroll
+  for (int it = 0; it < 2; ++it) {
+    const int idx = tid + it * F::THREADS, o = idx % F::OCT, r = idx / F::OCT;
     float g[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if (r < nvalid) {
       const size_t gi = (row0 + r) * a.H + h;
@@ -174,6 +176,33 @@ __device__ __forceinline__ void prefetch_chunk(const Args& a, int b, int h, int 
     prefetch_l2(p);
   }
 }
+
+// A chunk's rows as they lie in memory, two octets per thread, loaded before the gate pass so that they arrive behind it.
+template <int D, bool REV>
+struct Rows {
+  float4 q[2][2], k[2][2];
+  uint4 v[2], g[2];
+  __device__ __forceinline__ void load(const Args& a, size_t row0, int h, int j, int nvalid, int tid) {
+    using F = Cfg<D>;
+#pragma unroll
+    for (int it = 0; it < 2; ++it) {
+      const int idx = tid + it * F::THREADS, o = idx % F::OCT, r = idx / F::OCT;
+      const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+      q[it][0] = q[it][1] = k[it][0] = k[it][1] = z;
+      v[it] = g[it] = make_uint4(0u, 0u, 0u, 0u);
+      if (r < nvalid) {
+        const size_t tq = ((row0 + r) * a.H + h) * D + o * 8;
+        q[it][0] = *reinterpret_cast<const float4*>(a.qd + tq); q[it][1] = *reinterpret_cast<const float4*>(a.qd + tq + 4);
+        k[it][0] = *reinterpret_cast<const float4*>(a.kd + tq); k[it][1] = *reinterpret_cast<const float4*>(a.kd + tq + 4);
+        v[it] = *reinterpret_cast<const uint4*>(a.v + ((row0 + r) * a.Hkv + j) * D + o * 8);
+        if (REV) g[it] = *reinterpret_cast<const uint4*>(a.dO + tq);
+      }
+    }
+  }
+  static __device__ __forceinline__ void f8(const float4 (&x)[2], float* f) {
+    f[0] = x[0].x; f[1] = x[0].y; f[2] = x[0].z; f[3] = x[0].w; f[4] = x[1].x; f[5] = x[1].y; f[6] = x[1].z; f[7] = x[1].w;
+  }
+};
 
 // products on two-term operands, issued by one thread: D (+)= A B with A = ah + al, B = bh + bl (a missing low part is 0)
 struct Mma {
@@ -268,6 +297,8 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) sweep_kerne
     const int t0 = n * C, nvalid = min(C, a.T - t0);
     const size_t row0 = (size_t)b * a.T + t0;
     if (n + 1 < nch) prefetch_chunk<D>(a, b, h, j, t0 + C, tid);
+    Rows<D, false> rows;
+    rows.load(a, row0, h, j, nvalid, tid);
     gate_pass<D>(a, row0, h, nvalid, s_x, s_bm, s_ft, const_cast<int*>(&s_fl[2]), tid);
     const bool f16 = __int_as_float(s_fl[2]) <= RMAX_F16;
     const int fmt = f16 ? FMT_F16 : FMT_BF16;
@@ -275,20 +306,14 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) sweep_kerne
     const float ksc = pow2i(kap);
     // ---- operands
     float vmax = 0.f;
-    for (int idx = tid; idx < C * F::OCT; idx += F::THREADS) {
-      const int o = idx % F::OCT, r = idx / F::OCT;
-      float q[8], k[8], vv[8], x[8];
-      uint4 zv = make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-      for (int i = 0; i < 8; ++i) q[i] = k[i] = 0.f;
-      if (r < nvalid) {
-        const size_t tq = ((row0 + r) * a.H + h) * D + o * 8;
-        load_row8(a.qd + tq, q);
-        load_row8(a.kd + tq, k);
-        zv = *reinterpret_cast<const uint4*>(a.v + ((row0 + r) * a.Hkv + j) * D + o * 8);
-      }
+    for (int it = 0; it < 2; ++it) {
+      const int idx = tid + it * F::THREADS, o = idx % F::OCT, r = idx / F::OCT;
+      float q[8], k[8], vv[8], x[8];
+      rows.f8(rows.q[it], q);
+      rows.f8(rows.k[it], k);
+      unpack8b(rows.v[it], vv);
       load_row8(s_x + r * D + o * 8, x);
-      unpack8b(zv, vv);
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         q[i] *= ex2f(x[i]) * (float)(1 << QSC);
@@ -316,22 +341,23 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) sweep_kerne
     smx = 0.f;
     if (st_thr) {
       const float f = ex2f(fmaxf(s_bm[row] + s_pe[row], -126.f)) * pow2i(kap - kap_prev);
-      float s[8];
+      static_assert(SW == 32, "one wide load");
+      float y[32], s[8];
       uint4 hi, lo;
-#pragma unroll 2
-      for (int c0 = cg * SW; c0 < (cg + 1) * SW; c0 += 8) {
-        tmem_ld8(lane_base + F::F_ST + c0, s);
-        tmem_wait_ld();
+      tmem_ld32(lane_base + F::F_ST + cg * SW, y);
+      tmem_wait_ld();
+#pragma unroll
+      for (int i8 = 0; i8 < 32; i8 += 8) {
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-          s[i] *= f;
-          smx = fmaxf(smx, fabsf(s[i]));
+          y[i8 + i] *= f;
+          smx = fmaxf(smx, fabsf(y[i8 + i]));
         }
-        split8h(s, f16, hi, lo);
-        *reinterpret_cast<uint4*>(sg + F::F_S + toff(F::SL_C, row, c0)) = hi;
-        *reinterpret_cast<uint4*>(sg + F::F_S + F::T_SZ + toff(F::SL_C, row, c0)) = lo;
-        tmem_st8(lane_base + F::F_ST + c0, s);
+        split8h(y + i8, f16, hi, lo);
+        *reinterpret_cast<uint4*>(sg + F::F_S + toff(F::SL_C, row, cg * SW + i8)) = hi;
+        *reinterpret_cast<uint4*>(sg + F::F_S + F::T_SZ + toff(F::SL_C, row, cg * SW + i8)) = lo;
       }
+      tmem_st32(lane_base + F::F_ST + cg * SW, y);
       if (cg == F::NCG - 1) {
         tmem_ld8(lane_base + F::F_ST + D, s);
         tmem_wait_ld();
@@ -371,17 +397,20 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) sweep_kerne
     wt.wait();
     // ---- mask
     if (tok_thr) {
-      float s[8];
+      float s[16];
       uint4 hi, lo;
-#pragma unroll 2
-      for (int c0 = cg * TW; c0 < (cg + 1) * TW; c0 += 8) {
-        tmem_ld8(lane_base + F::F_P + c0, s);
+#pragma unroll 1
+      for (int c0 = cg * TW; c0 < (cg + 1) * TW; c0 += 16) {
+        tmem_ld16(lane_base + F::F_P + c0, s);
         tmem_wait_ld();
 #pragma unroll
-        for (int i = 0; i < 8; ++i) s[i] = c0 + i <= row ? s[i] : 0.f;
-        split8h(s, f16, hi, lo);
-        *reinterpret_cast<uint4*>(sg + F::F_PM + toff(F::SL_U, row, c0)) = hi;
-        *reinterpret_cast<uint4*>(sg + F::F_PM + F::T_P + toff(F::SL_U, row, c0)) = lo;
+        for (int i8 = 0; i8 < 16; i8 += 8) {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) s[i8 + i] = c0 + i8 + i <= row ? s[i8 + i] : 0.f;
+          split8h(s + i8, f16, hi, lo);
+          *reinterpret_cast<uint4*>(sg + F::F_PM + toff(F::SL_U, row, c0 + i8)) = hi;
+          *reinterpret_cast<uint4*>(sg + F::F_PM + F::T_P + toff(F::SL_U, row, c0 + i8)) = lo;
+        }
       }
     }
     for (int i = tid; i < D; i += F::THREADS) s_pe[i] = s_ft[i];
@@ -403,15 +432,19 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) sweep_kerne
       inv = a.normalize ? 1.f / fmaf(den, osc, a.eps) : 1.f;
       const float oi = inv * osc;
       const bf16* g = a.dO + ((row0 + min(row, nvalid - 1)) * a.H + h) * D;
-#pragma unroll 2
-      for (int c0 = cg * SW; c0 < (cg + 1) * SW; c0 += 8) {
-        float s[8], gv[8];
-        tmem_ld8(lane_base + F::F_O + c0, s);
-        unpack8b(*reinterpret_cast<const uint4*>(g + c0), gv);
-        tmem_wait_ld();
+      float s[32];
+      uint4 gr[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) gr[i] = *reinterpret_cast<const uint4*>(g + cg * SW + 8 * i);
+      tmem_ld32(lane_base + F::F_O + cg * SW, s);
+      tmem_wait_ld();
+#pragma unroll
+      for (int i8 = 0; i8 < 4; ++i8) {
+        float gv[8];
+        unpack8b(gr[i8], gv);
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-          dot = fmaf(gv[i], s[i] * oi, dot);
+          dot = fmaf(gv[i], s[8 * i8 + i] * oi, dot);
           domax = fmaxf(domax, fabsf(gv[i]));
         }
       }
@@ -513,6 +546,8 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
     const int kap = a.meta[((size_t)bh * nch + n) * 2], fmt = a.meta[((size_t)bh * nch + n) * 2 + 1];
     const bool f16 = fmt == FMT_F16;
     prefetch_chunk<D>(a, b, h, j, t0 - C, tid);
+    Rows<D, true> rows;
+    rows.load(a, row0, h, j, nvalid, tid);
     // ---- row scalars; the largest inv of the chunk and the largest entry of the adjoint decide 2^al
     if (tid == 0) s_fl[3] = s_fl[4] = 0;
     __syncthreads();
@@ -552,22 +587,15 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
     float rp[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) rp[i] = 0.f;
-    for (int idx = tid; idx < C * F::OCT; idx += F::THREADS) {
-      const int o = idx % F::OCT, r = idx / F::OCT;  // (o is the same in every iteration)
-      float q[8], k[8], vv[8], g[8], x[8];
-      uint4 zv = make_uint4(0u, 0u, 0u, 0u), zg = zv;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) q[i] = k[i] = 0.f;
-      if (r < nvalid) {
-        const size_t tq = ((row0 + r) * a.H + h) * D + o * 8;
-        load_row8(a.qd + tq, q);
-        load_row8(a.kd + tq, k);
-        zv = *reinterpret_cast<const uint4*>(a.v + ((row0 + r) * a.Hkv + j) * D + o * 8);
-        zg = *reinterpret_cast<const uint4*>(a.dO + tq);
-      }
+    for (int it = 0; it < 2; ++it) {
+      const int idx = tid + it * F::THREADS, o = idx % F::OCT, r = idx / F::OCT;  // (o is the same both times)
+      float q[8], k[8], vv[8], g[8], x[8];
+      rows.f8(rows.q[it], q);
+      rows.f8(rows.k[it], k);
+      unpack8b(rows.v[it], vv);
+      unpack8b(rows.g[it], g);
       load_row8(s_x + r * D + o * 8, x);
-      unpack8b(zv, vv);
-      unpack8b(zg, g);
       const float inv = s_inv[r] * asc, dl = s_dl[r];
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
@@ -621,26 +649,29 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
     // ---- mask: P' and E = dO v^T - delta, two-term
     if (tok_thr) {
       const float dl = s_dl[row];
-      float s[8], e[8];
+      float s[16], e[16];
       uint4 hi, lo;
-#pragma unroll 2
-      for (int c0 = cg * TW; c0 < (cg + 1) * TW; c0 += 8) {
-        tmem_ld8(lane_base + F::R_P + c0, s);
-        tmem_ld8(lane_base + F::R_EP + c0, e);
+#pragma unroll 1
+      for (int c0 = cg * TW; c0 < (cg + 1) * TW; c0 += 16) {
+        tmem_ld16(lane_base + F::R_P + c0, s);
+        tmem_ld16(lane_base + F::R_EP + c0, e);
         tmem_wait_ld();
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const bool on = c0 + i <= row;
-          s[i] = on ? s[i] : 0.f;
-          e[i] = on ? fminf(fmaxf(e[i] - dl, -65000.f), 65000.f) : 0.f;
+        for (int i8 = 0; i8 < 16; i8 += 8) {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const bool on = c0 + i8 + i <= row;
+            s[i8 + i] = on ? s[i8 + i] : 0.f;
+            e[i8 + i] = on ? fminf(fmaxf(e[i8 + i] - dl, -65000.f), 65000.f) : 0.f;
+          }
+          const uint32_t at = toff(F::SL_U, row, c0 + i8);
+          split8h(s + i8, f16, hi, lo);
+          *reinterpret_cast<uint4*>(sg + F::R_PM + at) = hi;
+          *reinterpret_cast<uint4*>(sg + F::R_PM + F::T_P + at) = lo;
+          split8h(e + i8, f16, hi, lo);
+          *reinterpret_cast<uint4*>(sg + F::R_E + at) = hi;
+          *reinterpret_cast<uint4*>(sg + F::R_E + F::T_P + at) = lo;
         }
-        const uint32_t at = toff(F::SL_U, row, c0);
-        split8h(s, f16, hi, lo);
-        *reinterpret_cast<uint4*>(sg + F::R_PM + at) = hi;
-        *reinterpret_cast<uint4*>(sg + F::R_PM + F::T_P + at) = lo;
-        split8h(e, f16, hi, lo);
-        *reinterpret_cast<uint4*>(sg + F::R_E + at) = hi;
-        *reinterpret_cast<uint4*>(sg + F::R_E + F::T_P + at) = lo;
       }
     }
     publish();
@@ -662,19 +693,19 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
     // ---- adjoint pass, over the consumed state operand
     if (st_thr) {
       const float f = ex2f(fmaxf(s_pe[row] + s_ft[row], -126.f)) * rfac;
-      float s[8];
+      float y[32];
       uint4 hi, lo;
-#pragma unroll 2
-      for (int c0 = cg * SW; c0 < (cg + 1) * SW; c0 += 8) {
-        tmem_ld8(lane_base + F::R_R + c0, s);
-        tmem_wait_ld();
+      tmem_ld32(lane_base + F::R_R + cg * SW, y);
+      tmem_wait_ld();
 #pragma unroll
-        for (int i = 0; i < 8; ++i) s[i] *= f;
-        split8h(s, f16, hi, lo);
-        *reinterpret_cast<uint4*>(sg + F::R_S + toff(F::SL_C, row, c0)) = hi;
-        *reinterpret_cast<uint4*>(sg + F::R_S + F::T_C + toff(F::SL_C, row, c0)) = lo;
-        tmem_st8(lane_base + F::R_R + c0, s);
+      for (int i8 = 0; i8 < 32; i8 += 8) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) y[i8 + i] *= f;
+        split8h(y + i8, f16, hi, lo);
+        *reinterpret_cast<uint4*>(sg + F::R_S + toff(F::SL_C, row, cg * SW + i8)) = hi;
+        *reinterpret_cast<uint4*>(sg + F::R_S + F::T_C + toff(F::SL_C, row, cg * SW + i8)) = lo;
       }
+      tmem_st32(lane_base + F::R_R + cg * SW, y);
       tmem_wait_st();
     }
     publish();
@@ -691,43 +722,45 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
     wt.wait();
     // ---- wq, wk, dv of the chunk's rows into fp32 tiles over the dead operands
     const float usc = pow2i(-(al + kap + sc));
-    float wqv[SW > 32 ? 1 : SW], wkv[SW > 32 ? 1 : SW];
     static_assert(SW == 32, "32 columns per thread");
     if (tok_thr) {
       const float dl = s_dl[row];
 #pragma unroll
-      for (int i8 = 0; i8 < SW; i8 += 8) {
-        const int c0 = cg * SW + i8;
-        float d[8], hi[8], lo[8];
-        const uint32_t at = toff(F::SL_T, row, c0);
-        tmem_ld8(lane_base + F::R_DQ + c0, d);
-        unpack8h(*reinterpret_cast<const uint4*>(sg + F::R_QS + at), f16, hi);
-        unpack8h(*reinterpret_cast<const uint4*>(sg + F::R_QS + F::T_TOK + at), f16, lo);
+      for (int i16 = 0; i16 < SW; i16 += 16) {
+        float dq[16], dk[16];
+        tmem_ld16(lane_base + F::R_DQ + cg * SW + i16, dq);
+        tmem_ld16(lane_base + F::R_DK + cg * SW + i16, dk);
         tmem_wait_ld();
 #pragma unroll
-        for (int i = 0; i < 8; ++i) wqv[i8 + i] = (hi[i] + lo[i]) * fmaf(-dl, s_z[c0 + i], d[i]) * usc;
-        tmem_ld8(lane_base + F::R_DK + c0, d);
-        unpack8h(*reinterpret_cast<const uint4*>(sg + F::R_KS + at), f16, hi);
-        unpack8h(*reinterpret_cast<const uint4*>(sg + F::R_KS + F::T_TOK + at), f16, lo);
-        tmem_wait_ld();
+        for (int i8 = 0; i8 < 16; i8 += 8) {
+          const int c0 = cg * SW + i16 + i8;
+          float hi[8], lo[8];
+          const uint32_t at = toff(F::SL_T, row, c0);
+          unpack8h(*reinterpret_cast<const uint4*>(sg + F::R_QS + at), f16, hi);
+          unpack8h(*reinterpret_cast<const uint4*>(sg + F::R_QS + F::T_TOK + at), f16, lo);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          wkv[i8 + i] = (hi[i] + lo[i]) * (d[i] + s_r16[c0 + i]) * usc;
-          wmax = fmaxf(wmax, fmaxf(fabsf(wqv[i8 + i]), fabsf(wkv[i8 + i])));
+          for (int i = 0; i < 8; ++i) dq[i8 + i] = (hi[i] + lo[i]) * fmaf(-dl, s_z[c0 + i], dq[i8 + i]) * usc;
+          unpack8h(*reinterpret_cast<const uint4*>(sg + F::R_KS + at), f16, hi);
+          unpack8h(*reinterpret_cast<const uint4*>(sg + F::R_KS + F::T_TOK + at), f16, lo);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            dk[i8 + i] = (hi[i] + lo[i]) * (dk[i8 + i] + s_r16[c0 + i]) * usc;
+            wmax = fmaxf(wmax, fmaxf(fabsf(dq[i8 + i]), fabsf(dk[i8 + i])));
+          }
+#pragma unroll
+          for (int i = 0; i < 8; i += 4) {
+            *reinterpret_cast<float4*>(sg + F::R_WQ + foff<D>(row, (c0 + i) >> 2)) = make_float4(dq[i8 + i], dq[i8 + i + 1], dq[i8 + i + 2], dq[i8 + i + 3]);
+            *reinterpret_cast<float4*>(sg + F::R_WK + foff<D>(row, (c0 + i) >> 2)) = make_float4(dk[i8 + i], dk[i8 + i + 1], dk[i8 + i + 2], dk[i8 + i + 3]);
+          }
         }
       }
-#pragma unroll
-      for (int i8 = 0; i8 < SW; i8 += 8) {
-        float d[8];
-        tmem_ld8(lane_base + F::R_DVC + cg * SW + i8, d);
+      {
+        float d[32];
+        tmem_ld32(lane_base + F::R_DVC + cg * SW, d);
         tmem_wait_ld();
 #pragma unroll
-        for (int i4 = 0; i4 < 8; i4 += 4) {
-          const int c = cg * SW + i8 + i4;
-          *reinterpret_cast<float4*>(sg + F::R_WQ + foff<D>(row, c >> 2)) = make_float4(wqv[i8 + i4], wqv[i8 + i4 + 1], wqv[i8 + i4 + 2], wqv[i8 + i4 + 3]);
-          *reinterpret_cast<float4*>(sg + F::R_WK + foff<D>(row, c >> 2)) = make_float4(wkv[i8 + i4], wkv[i8 + i4 + 1], wkv[i8 + i4 + 2], wkv[i8 + i4 + 3]);
-          *reinterpret_cast<float4*>(sg + F::R_DV + foff<D>(row, c >> 2)) = make_float4(d[i4] * usc, d[i4 + 1] * usc, d[i4 + 2] * usc, d[i4 + 3] * usc);
-        }
+        for (int i = 0; i < 32; i += 4)
+          *reinterpret_cast<float4*>(sg + F::R_DV + foff<D>(row, (cg * SW + i) >> 2)) = make_float4(d[i] * usc, d[i + 1] * usc, d[i + 2] * usc, d[i + 3] * usc);
       }
     }
     tc_fence_before_sync();
@@ -896,11 +929,27 @@ __global__ void __launch_bounds__(256, D == 128 ? 1 : 2) mix_bwd_kernel(const MA
         const int c = idx >> 2, dl = idx & 3;
         s_taps[idx] = dl < a.K ? __bfloat162float(w[((size_t)head * D + c) * a.K + dl]) : 0.f;
       }
+      // the rows of the next (head, stream) step travel towards L2 while this one is computed
+      if (g + stream < G) {
+        const int nh = h + stream;
+        const float* wn = stream ? a.wq : a.wk;
+        const float* pn = stream ? a.qd : a.kd;
+        constexpr int LF = D * 4 / 128;
+        for (int idx = tid; idx < nvalid * 2 * LF; idx += 256) {
+          const int r = idx / (2 * LF), l = idx % (2 * LF);
+          prefetch_l2((l < LF ? wn : pn) + (((size_t)b * a.T + t0 + r) * a.H + nh) * D + (l % LF) * 32);
+        }
+        if (stream && tid < nvalid) {
+          const bf16* xn = a.q + (((size_t)b * a.T + t0 + tid) * a.H + nh) * D;
+          prefetch_l2(xn);
+          if (D == 128) prefetch_l2(xn + 64);
+        }
+      }
       // ---- dy
       {
         const float* wp = stream ? a.wk : a.wq;
         const float* pp = stream ? a.kd : a.qd;
-#pragma unroll 2
+#pragma unroll 4
         for (int r = rr0; r < TT; r += RSTEP) {
           float wv[8], pv[8];
 #pragma unroll
