@@ -96,28 +96,47 @@ __device__ __forceinline__ int exp_above(float x) { return ((__float_as_int(x) >
 template <int D>
 __device__ __forceinline__ uint32_t foff(int r, int pc) { return (uint32_t)(r * (D * 4) + ((pc ^ (r & 7)) << 4)); }
 
-// Log-decays of a chunk scanned outwards from the middle token: exponents x into s_x (fp32, rows of D), bm and ft per channel,
-// the largest |x| into *rmax. Ends with a barrier; the caller has one between the last readers of s_x and this call.
+// A chunk's gate entries as they lie in memory, two octets per thread (gate_dim = 1: the token's entry as fp32 bits), fetched
+// while the chunk in front is computed.
 template <int D>
-__device__ __forceinline__ void gate_pass(const Args& a, size_t row0, int h, int nvalid, float* s_x, float* s_bm, float* s_ft,
+struct Gates {
+  uint4 r[2];
+  __device__ __forceinline__ void load(const Args& a, int b, int h, int t0, int tid) {
+    using F = Cfg<D>;
+    static_assert(C * F::OCT == 2 * F::THREADS, "two octets per thread");
+#pragma unroll
+    for (int it = 0; it < 2; ++it) {
+      const int idx = tid + it * F::THREADS, o = idx % F::OCT, t = t0 + idx / F::OCT;
+      r[it] = make_uint4(0u, 0u, 0u, 0u);
+      if (t0 >= 0 && t < a.T) {
+        const size_t gi = ((size_t)b * a.T + t) * a.H + h;
+        if (a.gate_dim == 1) r[it].x = __float_as_uint(__bfloat162float(a.gate[gi]));
+        else r[it] = *reinterpret_cast<const uint4*>(a.gate + gi * D + o * 8);
+      }
+    }
+  }
+};
+
+// Log-decays of a chunk scanned outwards from the middle token: exponents x into s_x (fp32, rows of D), bm and ft per channel,
+// the largest |x| into *rmax (cleared by the caller behind a barrier). Ends with a barrier; the caller has one between the
+// last readers of s_x and this call.
+template <int D>
+__device__ __forceinline__ void gate_pass(const Args& a, const Gates<D>& raw, int nvalid, float* s_x, float* s_bm, float* s_ft,
                                           int* rmax, int tid) {
   using F = Cfg<D>;
   const float L2E = 1.4426950408889634f;
-  if (tid == 0) *rmax = 0;
-  static_assert(C * F::OCT == 2 * F::THREADS, "two octets per thread");
 #pragma unroll
   for (int it = 0; it < 2; ++it) {
     const int idx = tid + it * F::THREADS, o = idx % F::OCT, r = idx / F::OCT;
     float g[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if (r < nvalid) {
-      const size_t gi = (row0 + r) * a.H + h;
       if (a.gate_dim == 1) {
-        const float av = __bfloat162float(a.gate[gi]);
+        const float av = __uint_as_float(raw.r[it].x);
         const float gv = a.gate_mode == LAWCAT_GATE_LOGDECAY ? av * L2E : log2_sigmoid(av) * a.inv_tau;
 #pragma unroll
         for (int i = 0; i < 8; ++i) g[i] = gv;
       } else {
-        unpack8b(*reinterpret_cast<const uint4*>(a.gate + gi * D + o * 8), g);
+        unpack8b(raw.r[it], g);
         if (a.gate_mode == LAWCAT_GATE_LOGDECAY) {
 #pragma unroll
           for (int i = 0; i < 8; ++i) g[i] *= L2E;
@@ -158,12 +177,14 @@ __device__ __forceinline__ void gate_pass(const Args& a, size_t row0, int h, int
   __syncthreads();
 }
 
-// one chunk's rows towards L2: the chunk that follows travels while this one is computed
+// One chunk's rows towards L2, issued by the warps that wait for a batch of products (the first warp issues them): the chunk
+// that follows travels while this one is computed. Line by line: the bulk prefetch of a row takes hundreds of cycles to issue.
 template <int D>
 __device__ __forceinline__ void prefetch_chunk(const Args& a, int b, int h, int j, int t0, int tid) {
-  constexpr int LF = D * 4 / 128, LB = D * 2 / 128, PER = 2 * LF + 3 * LB;  // 128-byte lines per token
-  if (t0 < 0) return;
-  for (int idx = tid; idx < C * PER; idx += Cfg<D>::THREADS) {
+  constexpr int LF = D * 4 / 128, LB = D * 2 / 128, PER = 2 * LF + 2 * LB, NT = Cfg<D>::THREADS - 32;  // lines per token
+  if (t0 < 0 || tid < 32) return;
+#pragma unroll 2
+  for (int idx = tid - 32; idx < C * PER; idx += NT) {
     const int r = idx / PER, l = idx % PER;
     if (t0 + r >= a.T) return;
     const size_t th = ((size_t)b * a.T + t0 + r) * a.H + h, tv = ((size_t)b * a.T + t0 + r) * a.Hkv + j;
@@ -171,8 +192,7 @@ __device__ __forceinline__ void prefetch_chunk(const Args& a, int b, int h, int 
     if (l < LF) p = (const char*)(a.qd + th * D) + l * 128;
     else if (l < 2 * LF) p = (const char*)(a.kd + th * D) + (l - LF) * 128;
     else if (l < 2 * LF + LB) p = (const char*)(a.v + tv * D) + (l - 2 * LF) * 128;
-    else if (l < 2 * LF + 2 * LB) p = (const char*)(a.dO + th * D) + (l - 2 * LF - LB) * 128;
-    else p = (const char*)(a.gate + th * a.gate_dim) + (l - 2 * LF - 2 * LB) * 128 * (a.gate_dim > 1);
+    else p = (const char*)(a.dO + th * D) + (l - 2 * LF - LB) * 128;
     prefetch_l2(p);
   }
 }
@@ -290,16 +310,17 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) sweep_kerne
   __syncthreads();
   float sbound = __int_as_float(s_fl[3]), domax = 0.f;
   int kap_prev = 0;
+  Gates<D> gates;
+  gates.load(a, b, h, 0, tid);
   auto KV = [&](uint32_t off, uint32_t slab) -> uint64_t { return kview(sb + off, slab); };
   auto MV = [&](uint32_t off, uint32_t slab) -> uint64_t { return mview(sb + off, slab); };
 
   for (int n = 0; n < nch; ++n) {
     const int t0 = n * C, nvalid = min(C, a.T - t0);
     const size_t row0 = (size_t)b * a.T + t0;
-    if (n + 1 < nch) prefetch_chunk<D>(a, b, h, j, t0 + C, tid);
     Rows<D, false> rows;
     rows.load(a, row0, h, j, nvalid, tid);
-    gate_pass<D>(a, row0, h, nvalid, s_x, s_bm, s_ft, const_cast<int*>(&s_fl[2]), tid);
+    gate_pass<D>(a, gates, nvalid, s_x, s_bm, s_ft, const_cast<int*>(&s_fl[2]), tid);
     const bool f16 = __int_as_float(s_fl[2]) <= RMAX_F16;
     const int fmt = f16 ? FMT_F16 : FMT_BF16;
     const int kap = max(-100, min(KAP_MAX, 14 - exp_above(fmaxf(sbound, 1e-30f))));
@@ -394,6 +415,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) sweep_kerne
                instr_desc(128, NV, fmt, MAJOR_MN, MAJOR_MN), true);
       mma_commit(bar);
     }
+    if (n + 1 < nch) prefetch_chunk<D>(a, b, h, j, t0 + C, tid);
     wt.wait();
     // ---- mask
     if (tok_thr) {
@@ -421,6 +443,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) sweep_kerne
       mma_commit(bar);
     }
     // |next state| <= |2^bm state| + 64 max|v|: every key enters with a factor <= 1
+    gates.load(a, b, h, t0 + C, tid);
     const float vm = __int_as_float(s_fl[4]), sm = __int_as_float(s_fl[3]) * pow2i(-kap);
     wt.wait();
     // ---- 1 / den and dO . o of the chunk's rows
@@ -454,7 +477,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) sweep_kerne
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    if (tid == 0) { s_fl[3] = 0; s_fl[4] = 0; }
+    if (tid == 0) s_fl[2] = s_fl[3] = s_fl[4] = 0;
     if (tok_thr && cg == 0 && row < nvalid) {
       float d = 0.f;
 #pragma unroll
@@ -539,31 +562,39 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
   const float osc = pow2i(sc);
   int al_prev = 0;
   float wmax = 0.f;
+  // what the next chunk's first passes need, fetched while the chunk behind it is computed
+  Gates<D> gates;
+  int2 nx_meta = make_int2(0, 0);
+  float nx_inv = 0.f, nx_dl = 0.f, nx_z = 0.f;
+  auto fetch_next = [&](int m) {
+    if (m < 0) return;
+    gates.load(a, b, h, m * C, tid);
+    nx_meta = *reinterpret_cast<const int2*>(a.meta + ((size_t)bh * nch + m) * 2);
+    nx_inv = nx_dl = 0.f;
+    if (tid < C && m * C + tid < a.T) {
+      const size_t th = ((size_t)b * a.T + m * C + tid) * a.H + h;
+      nx_inv = a.inv[th];
+      nx_dl = a.delta[th];
+    }
+    if (tid >= C && tid < C + D) nx_z = a.z16[((size_t)bh * nch + m) * D + tid - C];
+  };
+  fetch_next(nch - 1);
 
   for (int n = nch - 1; n >= 0; --n) {
     const int t0 = n * C, nvalid = min(C, a.T - t0);
     const size_t row0 = (size_t)b * a.T + t0;
-    const int kap = a.meta[((size_t)bh * nch + n) * 2], fmt = a.meta[((size_t)bh * nch + n) * 2 + 1];
+    const int kap = nx_meta.x, fmt = nx_meta.y;
     const bool f16 = fmt == FMT_F16;
-    prefetch_chunk<D>(a, b, h, j, t0 - C, tid);
     Rows<D, true> rows;
     rows.load(a, row0, h, j, nvalid, tid);
     // ---- row scalars; the largest inv of the chunk and the largest entry of the adjoint decide 2^al
-    if (tid == 0) s_fl[3] = s_fl[4] = 0;
-    __syncthreads();
     if (tid < C) {
-      float inv = 0.f, dl = 0.f;
-      if (tid < nvalid) {
-        const size_t th = (row0 + tid) * a.H + h;
-        inv = a.inv[th];
-        dl = a.delta[th];
-      }
-      s_inv[tid] = inv;
-      s_dl[tid] = dl * osc;
-      const float m = warp_max(fabsf(inv));
+      s_inv[tid] = nx_inv;
+      s_dl[tid] = nx_dl * osc;
+      const float m = warp_max(fabsf(nx_inv));
       if (lane == 0) atomicMax(const_cast<int*>(&s_fl[3]), __float_as_int(m < 1.0e30f ? m : 1.0e30f));
     }
-    if (tid >= C && tid < C + D) s_z[tid - C] = a.z16[((size_t)bh * nch + n) * D + tid - C];
+    if (tid >= C && tid < C + D) s_z[tid - C] = nx_z;
     if (n < nch - 1 && st_thr) {
       const float f = ex2f(fmaxf(s_pe[row], -126.f));
       float m = 0.f, s[32];
@@ -577,7 +608,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
       m = warp_max(m * f);
       if (lane == 0) atomicMax(const_cast<int*>(&s_fl[4]), __float_as_int(m < 1.0e30f ? m : 1.0e30f));
     }
-    gate_pass<D>(a, row0, h, nvalid, s_x, s_bm, s_ft, const_cast<int*>(&s_fl[2]), tid);  // (two barriers)
+    gate_pass<D>(a, gates, nvalid, s_x, s_bm, s_ft, const_cast<int*>(&s_fl[2]), tid);  // (two barriers)
     int al = min(5 - exp_above(fmaxf(__int_as_float(s_fl[3]), 1e-30f)), 10 - kap);
     const float rm = __int_as_float(s_fl[4]);
     if (rm > 0.f) al = min(al, al_prev + 14 - exp_above(rm));
@@ -646,6 +677,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
       s_r[tid] = w + p;
     }
     wt.wait();
+    if (tid == 0) s_fl[2] = s_fl[3] = s_fl[4] = 0;  // (read by everybody before the barrier in front of the products)
     // ---- mask: P' and E = dO v^T - delta, two-term
     if (tok_thr) {
       const float dl = s_dl[row];
@@ -689,6 +721,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
                false);
       mma_commit(bar);
     }
+    prefetch_chunk<D>(a, b, h, j, t0 - C, tid);
     wt.wait();
     // ---- adjoint pass, over the consumed state operand
     if (st_thr) {
@@ -718,6 +751,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
                true);
       mma_commit(bar);
     }
+    fetch_next(n - 1);
     for (int i = tid; i < D; i += F::THREADS) s_pe[i] = s_bm[i];  // (read again behind the next barrier at the earliest)
     wt.wait();
     // ---- wq, wk, dv of the chunk's rows into fp32 tiles over the dead operands
@@ -766,6 +800,12 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
+    uint4 graw[2];  // this chunk's gate again, for the derivative of the log-decays
+#pragma unroll
+    for (int it = 0; it < 2; ++it) {
+      const int idx = tid + it * F::THREADS, o = idx % F::OCT, r = idx / F::OCT;
+      if (a.gate_dim != 1 && r < nvalid) graw[it] = *reinterpret_cast<const uint4*>(a.gate + ((row0 + r) * a.H + h) * D + o * 8);
+    }
     // ---- gate gradient: reverse running sum of wq - wk over the chunk's tokens on top of what lies behind it; thread =
     // (channel, run of tokens); the runs' totals meet in shared memory
     {
@@ -793,15 +833,21 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
       if (run == 0) s_car[c] = all;
     }
     // ---- whole rows to global memory
-    for (int idx = tid; idx < nvalid * (D / 4); idx += F::THREADS) {
-      const int pc = idx % (D / 4), r = idx / (D / 4);
+#pragma unroll
+    for (int it = 0; it < C * (D / 4) / F::THREADS; ++it) {
+      const int idx = tid + it * F::THREADS, pc = idx % (D / 4), r = idx / (D / 4);
       const size_t at = ((row0 + r) * a.H + h) * D + pc * 4;
       const uint32_t so = foff<D>(r, pc);
-      *reinterpret_cast<float4*>(a.wq + at) = *reinterpret_cast<const float4*>(sg + F::R_WQ + so);
-      *reinterpret_cast<float4*>(a.wk + at) = *reinterpret_cast<const float4*>(sg + F::R_WK + so);
-      *reinterpret_cast<float4*>(a.dvh + at) = *reinterpret_cast<const float4*>(sg + F::R_DV + so);
+      if (r < nvalid) {
+        *reinterpret_cast<float4*>(a.wq + at) = *reinterpret_cast<const float4*>(sg + F::R_WQ + so);
+        *reinterpret_cast<float4*>(a.wk + at) = *reinterpret_cast<const float4*>(sg + F::R_WK + so);
+        *reinterpret_cast<float4*>(a.dvh + at) = *reinterpret_cast<const float4*>(sg + F::R_DV + so);
+      }
     }
-    auto dlog = [&](float av) { return a.gate_mode == LAWCAT_GATE_LOGDECAY ? 1.f : (1.f - 1.f / (1.f + __expf(-av))) * a.inv_tau; };
+    // d(log-decay) / d(gate entry): 1 - sigmoid(a) = 1 / (1 + e^a)
+    auto dlog = [&](float av) {
+      return a.gate_mode == LAWCAT_GATE_LOGDECAY ? 1.f : rcpf(1.f + ex2f(fminf(av * 1.4426950408889634f, 126.f))) * a.inv_tau;
+    };
     if (a.gate_dim == 1) {
       for (int r = warp; r < nvalid; r += NW) {
         float s = 0.f;
@@ -813,16 +859,17 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
         }
       }
     } else {
-      for (int idx = tid; idx < nvalid * F::OCT; idx += F::THREADS) {
-        const int o = idx % F::OCT, r = idx / F::OCT;
-        const size_t gi = ((row0 + r) * a.H + h) * D + o * 8;
+#pragma unroll
+      for (int it = 0; it < 2; ++it) {
+        const int idx = tid + it * F::THREADS, o = idx % F::OCT, r = idx / F::OCT;
+        if (r >= nvalid) continue;
         float av[8], d[8];
-        unpack8b(*reinterpret_cast<const uint4*>(a.gate + gi), av);
+        unpack8b(graw[it], av);
         const float4 x = *reinterpret_cast<const float4*>(sg + F::R_DG + foff<D>(r, 2 * o)), y = *reinterpret_cast<const float4*>(sg + F::R_DG + foff<D>(r, 2 * o + 1));
         d[0] = x.x; d[1] = x.y; d[2] = x.z; d[3] = x.w; d[4] = y.x; d[5] = y.y; d[6] = y.z; d[7] = y.w;
 #pragma unroll
         for (int i = 0; i < 8; ++i) d[i] *= dlog(av[i]);
-        store_row8(a.dgate + gi, d);
+        store_row8(a.dgate + ((row0 + r) * a.H + h) * D + o * 8, d);
       }
     }
     al_prev = al;
