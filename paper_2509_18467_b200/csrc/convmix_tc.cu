@@ -94,24 +94,28 @@ __device__ __forceinline__ void conv_tile(const uint8_t* s_raw, const float* s_w
   }
 }
 
-// Forward. 256 threads walk one (batch, query head, tile of 128 tokens), query stream then key stream. bf16 outputs take
+// Forward. One block (16 warps per SM) walks one (batch, query head, tile of 128 tokens), query stream then key stream. bf16 outputs take
 // the conv output as one fp16 operand. fp32 outputs (features that a fused caller keeps in fp32, and those of the exact
 // recurrence) take it as three bf16 terms, u = b1 + b2 + b3 exactly, with W_h exact in bf16: the products are those of
 // fp32 numbers over the full fp32 range, summed in fp32.
 // Bound by HBM writes (fp32 features) and by the dependent phases of a tile: raw rows go from global memory through the
 // conv straight into the operand (no staging tile), and the outputs leave through the drained operand tile as whole rows.
 template <int D, typename TO>
-__global__ void __launch_bounds__(256) convmix_tc_fwd_kernel(const CArgs a) {
+__host__ __device__ constexpr int fwd_threads() { return D == 128 && sizeof(TO) == 4 ? 512 : 256; }
+
+template <int D, typename TO>
+__global__ void __launch_bounds__(fwd_threads<D, TO>()) convmix_tc_fwd_kernel(const CArgs a) {
   using L = Lay<D>;
   extern __shared__ __align__(128) uint8_t sg[];
+  constexpr int NTH = fwd_threads<D, TO>(), NCG = NTH / 128;
   constexpr int NT = sizeof(TO) == 4 ? 3 : 1, FMT = NT == 3 ? FMT_BF16 : FMT_F16;
   constexpr uint32_t OFF_WT = 0, OFF_U = OFF_WT + L::TILE_W;
-  constexpr uint32_t OFF_TAPS = OFF_U + NT * L::TILE_U, OFF_RED = OFF_TAPS + D * 16, OFF_BAR = OFF_RED + 4 * TT * 4;
+  constexpr uint32_t OFF_TAPS = OFF_U + NT * L::TILE_U, OFF_RED = OFF_TAPS + D * 16, OFF_BAR = OFF_RED + 2 * NCG * TT * 4;
   const uint32_t sb = smem_u32(sg);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   volatile int* const s_flags = reinterpret_cast<volatile int*>(sg + OFF_BAR + 16);  // [0] tmem base, [1] abort
   float* const s_taps = reinterpret_cast<float*>(sg + OFF_TAPS);
-  float* const s_red = reinterpret_cast<float*>(sg + OFF_RED);  // [max, sum][2 halves][128 rows]
+  float* const s_red = reinterpret_cast<float*>(sg + OFF_RED);  // [max, sum][column group][128 rows]
   const int t0 = blockIdx.x * TT, bh = blockIdx.y, h = bh % a.H, b = bh / a.H;
   const int G = a.H / a.Hkv, j = h / G;
   if (tid == 0) {
@@ -125,17 +129,17 @@ __global__ void __launch_bounds__(256) convmix_tc_fwd_kernel(const CArgs a) {
   }
   auto load_w = [&](const bf16* Wh) {
     if (NT == 1) {
-      load_w_tile<D>(sg + OFF_WT, Wh, tid, 256);
+      load_w_tile<D>(sg + OFF_WT, Wh, tid, NTH);
     } else {
-      for (int idx = tid; idx < D * L::OPR; idx += 256) {
+      for (int idx = tid; idx < D * L::OPR; idx += NTH) {
         const int c = idx / L::OPR, o = idx % L::OPR;
         *reinterpret_cast<uint4*>(sg + OFF_WT + toff(L::SLAB_W, c, o * 8)) = *reinterpret_cast<const uint4*>(Wh + (size_t)c * D + o * 8);
       }
     }
   };
   load_w(a.W + (size_t)h * D * D);
-  const int row = (warp & 3) * 32 + lane, half = warp >> 2;  // epilogue: row of the tile, half of its columns
-  constexpr int HC = D / 2;
+  const int row = (warp & 3) * 32 + lane, cg = warp >> 2;  // epilogue: row of the tile, group of its columns
+  constexpr int HC = D / NCG;
   uint32_t lane_base = 0, tmem = 0;
   Waiter wt{sb + OFF_BAR, 0u, s_flags + 1, a.dev_status};
 #pragma unroll 1
@@ -146,7 +150,7 @@ __global__ void __launch_bounds__(256) convmix_tc_fwd_kernel(const CArgs a) {
     const int NH = stream ? a.Hkv : a.H, head = stream ? j : h;
     // (a separate linear layer per stream: the product that read the query stream's W_h has completed)
     if (stream == 1 && a.unshared) load_w(a.W + ((size_t)a.H + h) * D * D);
-    for (int idx = tid; idx < D * 4; idx += 256) {
+    for (int idx = tid; idx < D * 4; idx += NTH) {
       const int c = idx >> 2, dl = idx & 3;
       s_taps[idx] = dl < a.K ? __bfloat162float(w[((size_t)head * D + c) * a.K + dl]) : 0.f;
     }
@@ -159,7 +163,7 @@ __global__ void __launch_bounds__(256) convmix_tc_fwd_kernel(const CArgs a) {
     __syncthreads();
     tc_fence_after_sync();
     {
-      constexpr int RPT = TT * L::OPR / 256, STEP = 4;  // rows per thread, rows per run
+      constexpr int RPT = TT * L::OPR / NTH, STEP = 4;  // rows per thread, rows per run
       const int o = tid % L::OPR, r0 = tid / L::OPR * RPT;
 #pragma unroll 1
       for (int rr = 0; rr < RPT; rr += STEP)
@@ -179,7 +183,7 @@ __global__ void __launch_bounds__(256) convmix_tc_fwd_kernel(const CArgs a) {
     __syncthreads();
     tc_fence_after_sync();
     tmem = (uint32_t)s_flags[0];
-    lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16) + half * HC;
+    lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16) + cg * HC;
     if (tid == 0) {
       const uint32_t idesc = instr_desc(128, D, FMT, MAJOR_K, MAJOR_MN);
       const uint64_t db = mview(sb + OFF_WT, L::SLAB_W);
@@ -191,7 +195,7 @@ __global__ void __launch_bounds__(256) convmix_tc_fwd_kernel(const CArgs a) {
       mma_commit(sb + OFF_BAR);
     }
     wt.wait();
-    // phi over the row: softmax (the two threads of a row exchange max and sum), or elementwise 1 + ELU / identity
+    // phi over the row: softmax (the threads of a row exchange max and sum), or elementwise 1 + ELU / identity
     float y[HC];
 #pragma unroll
     for (int c0 = 0; c0 < HC; c0 += 32) tmem_ld32(lane_base + c0, y + c0);
@@ -200,9 +204,10 @@ __global__ void __launch_bounds__(256) convmix_tc_fwd_kernel(const CArgs a) {
       float m = -INFINITY, sum = 0.f;
 #pragma unroll
       for (int i = 0; i < HC; ++i) m = fmaxf(m, y[i]);
-      s_red[half * TT + row] = m;
+      s_red[cg * TT + row] = m;
       __syncthreads();
-      m = fmaxf(m, s_red[(half ^ 1) * TT + row]);
+#pragma unroll
+      for (int i = 0; i < NCG; ++i) m = fmaxf(m, s_red[i * TT + row]);
       if (NT == 3) {
 #pragma unroll
         for (int i = 0; i < HC; ++i) { y[i] = expf(y[i] - m); sum += y[i]; }
@@ -211,9 +216,12 @@ __global__ void __launch_bounds__(256) convmix_tc_fwd_kernel(const CArgs a) {
 #pragma unroll
         for (int i = 0; i < HC; ++i) { y[i] = ex2f(fmaf(y[i], 1.4426950408889634f, -mb)); sum += y[i]; }
       }
-      s_red[(2 + half) * TT + row] = sum;
+      s_red[(NCG + cg) * TT + row] = sum;
       __syncthreads();
-      const float inv = 1.f / (sum + s_red[(2 + (half ^ 1)) * TT + row]);
+      float tot = 0.f;
+#pragma unroll
+      for (int i = 0; i < NCG; ++i) tot += s_red[(NCG + i) * TT + row];
+      const float inv = 1.f / tot;
 #pragma unroll
       for (int i = 0; i < HC; ++i) y[i] *= inv;
     } else if (a.phi == LAWCAT_PHI_ELU1) {
@@ -224,7 +232,7 @@ __global__ void __launch_bounds__(256) convmix_tc_fwd_kernel(const CArgs a) {
     constexpr int EPP = 16 / sizeof(TO), PPR = D / EPP;  // elements per piece, pieces per row
 #pragma unroll
     for (int i = 0; i < HC; i += EPP) {
-      const int pc = (half * HC + i) / EPP;
+      const int pc = (cg * HC + i) / EPP;
       uint4 v;
       if (NT == 3) v = make_uint4(__float_as_uint(y[i]), __float_as_uint(y[i + 1]), __float_as_uint(y[i + 2]), __float_as_uint(y[i + 3]));
       else v = pack8bf16(y + i);
@@ -235,7 +243,7 @@ __global__ void __launch_bounds__(256) convmix_tc_fwd_kernel(const CArgs a) {
     tc_fence_after_sync();
     TO* out = reinterpret_cast<TO*>(stream ? a.kdot : a.qdot);
 #pragma unroll 4
-    for (int idx = tid; idx < TT * PPR; idx += 256) {
+    for (int idx = tid; idx < TT * PPR; idx += NTH) {
       const int r = idx / PPR, pc = idx % PPR;
       if (t0 + r < a.T)
         *reinterpret_cast<uint4*>(out + (((size_t)b * a.T + t0 + r) * a.H + h) * D + pc * EPP) =
@@ -451,7 +459,7 @@ __global__ void __launch_bounds__(128, 2) convmix_tc_bwd_kernel(const CArgs a) {
 template <int D, typename TO>
 constexpr uint32_t fwd_smem() {
   using L = Lay<D>;
-  return L::TILE_W + (sizeof(TO) == 4 ? 3 : 1) * L::TILE_U + D * 16 + 4 * TT * 4 + 64;
+  return L::TILE_W + (sizeof(TO) == 4 ? 3 : 1) * L::TILE_U + D * 16 + 2 * (fwd_threads<D, TO>() / 128) * TT * 4 + 64;
 }
 constexpr uint32_t bwd_smem() {
   using L = Lay<64>;
@@ -507,11 +515,11 @@ int launch_convmix_tc_fwd(const Ctx& c, const void* q, const void* k, const void
   const dim3 grid((unsigned)((p.T + TT - 1) / TT), (unsigned)(p.B * p.H));
   LaunchScope _ls("convmix_tc_fwd", c.stream);
   if (p.d_k == 64) {
-    if (out_f32) convmix_tc_fwd_kernel<64, float><<<grid, 256, fwd_smem<64, float>(), c.stream>>>(a);
-    else convmix_tc_fwd_kernel<64, bf16><<<grid, 256, fwd_smem<64, bf16>(), c.stream>>>(a);
+    if (out_f32) convmix_tc_fwd_kernel<64, float><<<grid, fwd_threads<64, float>(), fwd_smem<64, float>(), c.stream>>>(a);
+    else convmix_tc_fwd_kernel<64, bf16><<<grid, fwd_threads<64, bf16>(), fwd_smem<64, bf16>(), c.stream>>>(a);
   } else {
-    if (out_f32) convmix_tc_fwd_kernel<128, float><<<grid, 256, fwd_smem<128, float>(), c.stream>>>(a);
-    else convmix_tc_fwd_kernel<128, bf16><<<grid, 256, fwd_smem<128, bf16>(), c.stream>>>(a);
+    if (out_f32) convmix_tc_fwd_kernel<128, float><<<grid, fwd_threads<128, float>(), fwd_smem<128, float>(), c.stream>>>(a);
+    else convmix_tc_fwd_kernel<128, bf16><<<grid, fwd_threads<128, bf16>(), fwd_smem<128, bf16>(), c.stream>>>(a);
   }
   LAWCAT_CHECK_LAUNCH();
   return LAWCAT_OK;

@@ -904,13 +904,14 @@ struct MArgs {
 template <int D>
 struct MCfg {
   using L = Lay<D>;
+  static constexpr int THREADS = D == 128 ? 512 : 256, NCG = THREADS / 128;  // (16 warps per SM either way)
   static constexpr uint32_t WT = 0, U = L::TILE_W, DY = U + 2 * L::TILE_U, TAPS = DY + 2 * L::TILE_U, BAR = TAPS + D * 16;
   static constexpr uint32_t BYTES = BAR + 64;
   static constexpr uint32_t DUQ = 0, DUK = D, DWC = 2 * D, COLS = D == 128 ? 512 : 256;
 };
 
 template <int D>
-__global__ void __launch_bounds__(256, D == 128 ? 1 : 2) mix_bwd_kernel(const MArgs a) {
+__global__ void __launch_bounds__(MCfg<D>::THREADS, D == 128 ? 1 : 2) mix_bwd_kernel(const MArgs a) {
   using L = Lay<D>;
   using M = MCfg<D>;
   extern __shared__ __align__(128) uint8_t sg[];
@@ -934,19 +935,19 @@ __global__ void __launch_bounds__(256, D == 128 ? 1 : 2) mix_bwd_kernel(const MA
   tc_fence_after_sync();
   const Mma mm{(uint32_t)s_fl[0]};
   const uint32_t lane_base = mm.tmem + ((uint32_t)((warp & 3) * 32) << 16);
-  const int row = (warp & 3) * 32 + lane, half = warp >> 2;
-  constexpr int HC = D / 2;
+  const int row = (warp & 3) * 32 + lane, cg = warp >> 2;
+  constexpr int HC = D / M::NCG, NTH = M::THREADS;
   Waiter wt{sb + M::BAR, 0u, s_fl + 1, a.dev_status};
   // 2^sg: the largest |w| becomes 2^7 .. 2^8, which leaves |dy| <= |w| + sum |w| below the fp16 maximum for every row
   const int sgm = 8 - exp_above(fmaxf(__int_as_float(*a.wmax), 1e-30f));
   const float sc = pow2i(sgm), isc = pow2i(-sgm);
   const int o = tid % L::OPR, rr0 = tid / L::OPR;
-  constexpr int RSTEP = 256 / L::OPR;
+  constexpr int RSTEP = NTH / L::OPR;
   // fp32 [128][D] accumulator to global rows through the (dead) dy tiles
   auto rows_out = [&](uint32_t col, float* dst, int NH, int head) {
     float d[8];
 #pragma unroll 1
-    for (int c0 = half * HC; c0 < (half + 1) * HC; c0 += 8) {
+    for (int c0 = cg * HC; c0 < (cg + 1) * HC; c0 += 8) {
       tmem_ld8(lane_base + col + c0, d);
       tmem_wait_ld();
 #pragma unroll
@@ -956,7 +957,7 @@ __global__ void __launch_bounds__(256, D == 128 ? 1 : 2) mix_bwd_kernel(const MA
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    for (int idx = tid; idx < nvalid * (D / 4); idx += 256) {
+    for (int idx = tid; idx < nvalid * (D / 4); idx += NTH) {
       const int pc = idx % (D / 4), r = idx / (D / 4);
       *reinterpret_cast<float4*>(dst + (((size_t)b * a.T + t0 + r) * NH + head) * D + pc * 4) =
           *reinterpret_cast<const float4*>(sg + M::DY + foff<D>(r, pc));
@@ -966,13 +967,13 @@ __global__ void __launch_bounds__(256, D == 128 ? 1 : 2) mix_bwd_kernel(const MA
 #pragma unroll 1
   for (int g = 0; g < G; ++g) {
     const int h = j * G + g;
-    load_w_tile<D>(sg + M::WT, a.W + (size_t)h * D * D, tid, 256);
+    load_w_tile<D>(sg + M::WT, a.W + (size_t)h * D * D, tid, NTH);
 #pragma unroll 1
     for (int stream = 0; stream < 2; ++stream) {
       const bf16* x = stream ? a.k : a.q;
       const bf16* w = stream ? a.w_k : a.w_q;
       const int NH = stream ? a.Hkv : a.H, head = stream ? j : h;
-      for (int idx = tid; idx < D * 4; idx += 256) {
+      for (int idx = tid; idx < D * 4; idx += NTH) {
         const int c = idx >> 2, dl = idx & 3;
         s_taps[idx] = dl < a.K ? __bfloat162float(w[((size_t)head * D + c) * a.K + dl]) : 0.f;
       }
@@ -982,7 +983,7 @@ __global__ void __launch_bounds__(256, D == 128 ? 1 : 2) mix_bwd_kernel(const MA
         const float* wn = stream ? a.wq : a.wk;
         const float* pn = stream ? a.qd : a.kd;
         constexpr int LF = D * 4 / 128;
-        for (int idx = tid; idx < nvalid * 2 * LF; idx += 256) {
+        for (int idx = tid; idx < nvalid * 2 * LF; idx += NTH) {
           const int r = idx / (2 * LF), l = idx % (2 * LF);
           prefetch_l2((l < LF ? wn : pn) + (((size_t)b * a.T + t0 + r) * a.H + nh) * D + (l % LF) * 32);
         }
@@ -1053,7 +1054,7 @@ __global__ void __launch_bounds__(256, D == 128 ? 1 : 2) mix_bwd_kernel(const MA
     if (a.dW && row < D) {
       float d[8];
 #pragma unroll 1
-      for (int c0 = half * HC; c0 < (half + 1) * HC; c0 += 8) {
+      for (int c0 = cg * HC; c0 < (cg + 1) * HC; c0 += 8) {
         tmem_ld8(lane_base + M::DWC + c0, d);
         tmem_wait_ld();
         float* dst = a.dW + ((size_t)h * D + row) * D + c0;
@@ -1138,7 +1139,7 @@ static int run(const Ctx& c, const Args& a, const MArgs& m) {
     LAWCAT_CHECK_LAUNCH();
   }
   LaunchScope _ls("convmix_tc_bwd", c.stream);
-  mix_bwd_kernel<D><<<dim3((unsigned)((p.T + TT - 1) / TT), (unsigned)(p.B * p.H_kv)), 256, MCfg<D>::BYTES, c.stream>>>(m);
+  mix_bwd_kernel<D><<<dim3((unsigned)((p.T + TT - 1) / TT), (unsigned)(p.B * p.H_kv)), MCfg<D>::THREADS, MCfg<D>::BYTES, c.stream>>>(m);
   LAWCAT_CHECK_LAUNCH();
   return LAWCAT_OK;
 }
