@@ -137,6 +137,10 @@ __global__ void __launch_bounds__(fwd_threads<D, TO>()) convmix_tc_fwd_kernel(co
       }
     }
   };
+  constexpr int RPT = TT * L::OPR / NTH;  // rows of the conv per thread
+  const int co = tid % L::OPR, cr0 = tid / L::OPR * RPT;
+  uint4 raw[RPT + HALO];
+  conv_load<D, RPT>(raw, a.q, a.cache_q, b, t0 + cr0, a.T, a.H, h, a.K, co);
   load_w(a.W + (size_t)h * D * D);
   const int row = (warp & 3) * 32 + lane, cg = warp >> 2;  // epilogue: row of the tile, group of its columns
   constexpr int HC = D / NCG;
@@ -144,10 +148,8 @@ __global__ void __launch_bounds__(fwd_threads<D, TO>()) convmix_tc_fwd_kernel(co
   Waiter wt{sb + OFF_BAR, 0u, s_flags + 1, a.dev_status};
 #pragma unroll 1
   for (int stream = 0; stream < 2; ++stream) {
-    const bf16* x = stream ? a.k : a.q;
     const bf16* w = stream ? a.w_k : a.w_q;
-    const bf16* cache = stream ? a.cache_k : a.cache_q;
-    const int NH = stream ? a.Hkv : a.H, head = stream ? j : h;
+    const int head = stream ? j : h;
     // (a separate linear layer per stream: the product that read the query stream's W_h has completed)
     if (stream == 1 && a.unshared) load_w(a.W + ((size_t)a.H + h) * D * D);
     for (int idx = tid; idx < D * 4; idx += NTH) {
@@ -162,22 +164,16 @@ __global__ void __launch_bounds__(fwd_threads<D, TO>()) convmix_tc_fwd_kernel(co
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    {
-      constexpr int RPT = TT * L::OPR / NTH, STEP = 4;  // rows per thread, rows per run
-      const int o = tid % L::OPR, r0 = tid / L::OPR * RPT;
-#pragma unroll 1
-      for (int rr = 0; rr < RPT; rr += STEP)
-        conv_run<D, STEP>(x, cache, s_taps, b, t0 + r0 + rr, a.T, NH, head, a.K, o, [&](int i, float* u) {
-          uint8_t* dst = sg + OFF_U + toff(L::SLAB_U, r0 + rr + i, o * 8);
-          if (NT == 1) {
-            *reinterpret_cast<uint4*>(dst) = pack8f16(u);
-          } else {
-            *reinterpret_cast<uint4*>(dst) = take_bf16(u);
-            *reinterpret_cast<uint4*>(dst + L::TILE_U) = take_bf16(u);
-            *reinterpret_cast<uint4*>(dst + 2 * L::TILE_U) = pack8bf16(u);
-          }
-        });
-    }
+    conv_emit<RPT>(raw, s_taps, co, [&](int i, float* u) {
+      uint8_t* dst = sg + OFF_U + toff(L::SLAB_U, cr0 + i, co * 8);
+      if (NT == 1) {
+        *reinterpret_cast<uint4*>(dst) = pack8f16(u);
+      } else {
+        *reinterpret_cast<uint4*>(dst) = take_bf16(u);
+        *reinterpret_cast<uint4*>(dst + L::TILE_U) = take_bf16(u);
+        *reinterpret_cast<uint4*>(dst + 2 * L::TILE_U) = pack8bf16(u);
+      }
+    });
     fence_proxy_async();
     tc_fence_before_sync();
     __syncthreads();
@@ -241,6 +237,8 @@ __global__ void __launch_bounds__(fwd_threads<D, TO>()) convmix_tc_fwd_kernel(co
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
+    // (the key stream's rows arrive while the query stream's features leave)
+    if (stream == 0) conv_load<D, RPT>(raw, a.k, a.cache_k, b, t0 + cr0, a.T, a.Hkv, j, a.K, co);
     TO* out = reinterpret_cast<TO*>(stream ? a.kdot : a.qdot);
 #pragma unroll 4
     for (int idx = tid; idx < TT * PPR; idx += NTH) {

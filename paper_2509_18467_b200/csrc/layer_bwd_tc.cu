@@ -942,7 +942,7 @@ __global__ void __launch_bounds__(MCfg<D>::THREADS, D == 128 ? 1 : 2) mix_bwd_ke
   const int sgm = 8 - exp_above(fmaxf(__int_as_float(*a.wmax), 1e-30f));
   const float sc = pow2i(sgm), isc = pow2i(-sgm);
   const int o = tid % L::OPR, rr0 = tid / L::OPR;
-  constexpr int RSTEP = NTH / L::OPR;
+  constexpr int RSTEP = NTH / L::OPR, RPT = TT / RSTEP;
   // fp32 [128][D] accumulator to global rows through the (dead) dy tiles
   auto rows_out = [&](uint32_t col, float* dst, int NH, int head) {
     float d[8];
@@ -970,7 +970,6 @@ __global__ void __launch_bounds__(MCfg<D>::THREADS, D == 128 ? 1 : 2) mix_bwd_ke
     load_w_tile<D>(sg + M::WT, a.W + (size_t)h * D * D, tid, NTH);
 #pragma unroll 1
     for (int stream = 0; stream < 2; ++stream) {
-      const bf16* x = stream ? a.k : a.q;
       const bf16* w = stream ? a.w_k : a.w_q;
       const int NH = stream ? a.Hkv : a.H, head = stream ? j : h;
       for (int idx = tid; idx < D * 4; idx += NTH) {
@@ -1020,21 +1019,17 @@ __global__ void __launch_bounds__(MCfg<D>::THREADS, D == 128 ? 1 : 2) mix_bwd_ke
           *reinterpret_cast<uint4*>(sg + M::DY + L::TILE_U + toff(L::SLAB_U, r, o * 8)) = lo;
         }
       }
+      uint4 raw[RPT + HALO];
+      conv_load<D, RPT>(raw, stream ? a.k : a.q, stream ? a.cache_k : a.cache_q, b, t0 + rr0 * RPT, a.T, NH, head, a.K, o);
       __syncthreads();  // (the taps)
       // ---- u
-      {
-        constexpr int RPT = TT / RSTEP, STEP = 4;
-#pragma unroll 1
-        for (int rr = 0; rr < RPT; rr += STEP)
-          conv_run<D, STEP>(x, stream ? a.cache_k : a.cache_q, s_taps, b, t0 + rr0 * RPT + rr, a.T, NH, head, a.K, o,
-                            [&](int i, float* u) {
-                              uint4 hi, lo;
-                              split8h(u, true, hi, lo);
-                              const uint32_t at = toff(L::SLAB_U, rr0 * RPT + rr + i, o * 8);
-                              *reinterpret_cast<uint4*>(sg + M::U + at) = hi;
-                              *reinterpret_cast<uint4*>(sg + M::U + L::TILE_U + at) = lo;
-                            });
-      }
+      conv_emit<RPT>(raw, s_taps, o, [&](int i, float* u) {
+        uint4 hi, lo;
+        split8h(u, true, hi, lo);
+        const uint32_t at = toff(L::SLAB_U, rr0 * RPT + i, o * 8);
+        *reinterpret_cast<uint4*>(sg + M::U + at) = hi;
+        *reinterpret_cast<uint4*>(sg + M::U + L::TILE_U + at) = lo;
+      });
       fence_proxy_async();
       tc_fence_before_sync();
       __syncthreads();

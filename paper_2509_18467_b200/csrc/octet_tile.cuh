@@ -144,13 +144,11 @@ __device__ __forceinline__ void load_w_tile(uint8_t* s_wt, const bf16* Wh, int t
 // tile's rows travel while the current one is computed)
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
-// conv of 8 channels (octet o) of N consecutive tokens from t on, straight from global memory with a window of raw rows
-// (rows before the sequence come from the conv cache or are zero, rows past its end are zero); emit(i, u) takes token t + i.
-// s_w: the head's taps, fp32 [D][4], in shared memory.
-template <int D, int N, typename F>
-__device__ __forceinline__ void conv_run(const bf16* x, const bf16* cache, const float* s_w, int b, int t, int T, int NH,
-                                         int head, int K, int o, F emit) {
-  uint4 raw[N + HALO];
+// Conv of 8 channels (octet o) of N consecutive tokens from t on, straight from global memory: the window of raw rows (rows
+// before the sequence come from the conv cache or are zero, rows past its end are zero), loaded well before its use ...
+template <int D, int N>
+__device__ __forceinline__ void conv_load(uint4 (&raw)[N + HALO], const bf16* x, const bf16* cache, int b, int t, int T, int NH,
+                                          int head, int K, int o) {
 #pragma unroll
   for (int i = 0; i < N + HALO; ++i) {
     const int tt = t - HALO + i;
@@ -160,6 +158,10 @@ __device__ __forceinline__ void conv_run(const bf16* x, const bf16* cache, const
     else if (tt < 0 && cache != nullptr && tt + (K - 1) >= 0)
       raw[i] = *reinterpret_cast<const uint4*>(cache + (((size_t)b * (K - 1) + tt + (K - 1)) * NH + head) * D + o * 8);
   }
+}
+// ... and the sums; emit(i, u) takes token t + i. s_w: the head's taps, fp32 [D][4], in shared memory.
+template <int N, typename F>
+__device__ __forceinline__ void conv_emit(const uint4 (&raw)[N + HALO], const float* s_w, int o, F emit) {
   float w[8][4];
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
