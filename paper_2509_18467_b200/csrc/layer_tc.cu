@@ -299,6 +299,7 @@ static int run_layer_tc(const Ctx& c, const void* q, const void* k, const void* 
   a.S0 = S0; a.z0 = z0; a.S_T = S_T; a.z_T = z_T;
   auto* const k_layer = paired ? layer_tc_kernel<0, 2> : dh == 64 ? layer_tc_kernel<0, 1> : layer_tc_kernel<0, 0>;
   auto* const k_state = paired ? layer_tc_kernel<1, 2> : dh == 64 ? layer_tc_kernel<1, 1> : layer_tc_kernel<1, 0>;
+  const int threads = threads_of(paired ? 2 : dh == 64 ? 1 : 0);
   {
     // the kernels' shared-memory limit is raised once per device
     static std::mutex mu;
@@ -320,7 +321,7 @@ static int run_layer_tc(const Ctx& c, const void* q, const void* k, const void* 
   const int Hn = paired ? p.H / 2 : p.H;          // thread blocks per segment
   if (segs == nseq) {
     LaunchScope _ls("layer_tc", c.stream);
-    k_layer<<<Hn * segs, THREADS, SMEM_ALLOC, c.stream>>>(tq, tk, tv, tg, a, tab);
+    k_layer<<<Hn * segs, threads, SMEM_ALLOC, c.stream>>>(tq, tk, tv, tg, a, tab);
     LAWCAT_CHECK_LAUNCH();
     return LAWCAT_OK;
   }
@@ -337,7 +338,7 @@ static int run_layer_tc(const Ctx& c, const void* q, const void* k, const void* 
     TcArgs b1 = a;
     b1.S_T = loc_S; b1.z_T = loc_z; b1.dtot = dtot; b1.nsub = nsub;
     LaunchScope _ls("layer_tc_state", c.stream);
-    k_state<<<Hn * (segs - nseq) * nsub, THREADS, SMEM_ALLOC, c.stream>>>(tq, tk, tv, tg, b1, tab);
+    k_state<<<Hn * (segs - nseq) * nsub, threads, SMEM_ALLOC, c.stream>>>(tq, tk, tv, tg, b1, tab);
     LAWCAT_CHECK_LAUNCH();
   }
   cudaLaunchAttribute at[1];
@@ -361,7 +362,7 @@ static int run_layer_tc(const Ctx& c, const void* q, const void* k, const void* 
     // (an ordinary launch: as a dependent of the scan its blocks land while scan blocks still hold registers of most SMs,
     // and the call at T = 32768 took 1.34 ms instead of 1.11)
     LaunchScope _ls("layer_tc", c.stream);
-    k_layer<<<Hn * segs, THREADS, SMEM_ALLOC, c.stream>>>(tq, tk, tv, tg, a, tab);
+    k_layer<<<Hn * segs, threads, SMEM_ALLOC, c.stream>>>(tq, tk, tv, tg, a, tab);
   }
   LAWCAT_CHECK_LAUNCH();
   return LAWCAT_OK;

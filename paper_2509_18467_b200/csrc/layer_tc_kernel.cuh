@@ -11,7 +11,13 @@
 //               gate: g = log2 sigmoid(a) / tau per entry, then a scan outwards from the middle token gives the
 //               exponents x_t = b_t - b_mid (b the running sum of g) in fp32 (the middle reference keeps every factor
 //               2^x within 2^(+-32 max|g|)); v: bf16 -> fp16 in place (exact)
-//   MMA warp    MMA 1: Y = [u_q; u_k] W_h  (fp16 operands, fp32 accumulate in TMEM)
+//   MMA warp    MMA 1: Y = [u_q; u_k] W_h  (fp16 operands, fp32 accumulate in TMEM). For 64-wide heads a warp of its own
+//               issues it: a thread issues a product every hundred cycles or so, about twice what the tensor pipe needs for
+//               one, and the products of the next chunk's mix stand in the middle of the chain score -> read-out -> state
+//               that the next chunk waits for (32 heads of 64, 8192 tokens: 187 -> 178 us, 65536 tokens: 1205 -> 1066 us).
+//               At width 128 the blocks of a long sequence then fall into periods of 9.7k or 11.5k cycles a chunk, both SMs
+//               of a pair alike and differently from launch to launch, where they otherwise all take 10.0k (32768 tokens:
+//               1080 -> 1180 us): there the MMA warp issues it
 //   row warps   (two threads per token row, 64 columns each, straight from tensor memory)
 //               phi: row softmax. Query rows keep exp(y - max) unnormalized: a positive per-token factor cancels in
 //               Eq. 8. The decay factors ride in the exponent of the softmax: qs = 2^(y' + x_t), ks = phi_k 2^(-x_i),
@@ -33,6 +39,8 @@
 // tensor memory and reports LAWCAT_ERR_TIMEOUT through dev_status.
 #pragma once
 #include <cuda.h>
+
+#include <type_traits>
 
 #include "common.cuh"
 #include "tc_common.cuh"
@@ -68,10 +76,11 @@ constexpr int C = 64;        // tokens per chunk
 constexpr int MID = 31;      // reference token of the in-chunk decay factorization
 constexpr int HALO = 3;      // raw rows in front of a chunk that the conv needs (conv width up to 4)
 
-// warps: 0-7 prep, 8-15 row warps (TMEM quadrant = warp & 3, column half = (warp - 8) >> 2), 16 TMA, 17 MMA
+// warps: 0-7 prep, 8-15 row warps (TMEM quadrant = warp & 3, column half = (warp - 8) >> 2), 16 TMA, 17 MMA,
+// 18 mix (64-wide heads only)
 constexpr int PREP_THREADS = 256;
-constexpr int ROW_WARP0 = 8, TMA_WARP = 16, MMA_WARP = 17;
-constexpr int THREADS = 18 * 32;
+constexpr int ROW_WARP0 = 8, TMA_WARP = 16, MMA_WARP = 17, MIX_WARP = 18;
+__host__ __device__ constexpr int threads_of(int width) { return (width != 0 ? 19 : 18) * 32; }
 
 // shared memory map (byte offsets from a 1024-byte aligned base)
 constexpr uint32_t OFF_W = 0;                     // W_h^T fp16, K-major, 2 slabs x [128 x 128 B]
@@ -314,7 +323,7 @@ __device__ __forceinline__ bool wait_set_or_abort(uint32_t bar0, uint32_t mask, 
 // WIDTH: 0 = heads of 128 channels; 1 = one head of 64 channels per block (padded to 128); 2 = two 64-wide heads of one
 // key/value group per block. A compile-time switch, so that the 128-wide kernel carries none of the others' tests.
 template <int MODE, int WIDTH>
-__global__ void __launch_bounds__(THREADS, 1)
+__global__ void __launch_bounds__(threads_of(WIDTH), 1)
 layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                 const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_g, const TcArgs a,
                 const __grid_constant__ PackTab tab) {
@@ -341,6 +350,7 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   // of 128 channels, the shared k is loaded into both halves, W is block-diagonal, and everything that contracts over the
   // channels (scores, read-out) is issued per half into accumulators of its own.
   constexpr bool narrow = WIDTH == 1, pair = WIDTH == 2, wide = WIDTH == 0;
+  constexpr bool mixw = WIDTH != 0;  // MMA 1 issued by a warp of its own
   constexpr int dh = narrow ? 64 : 128, nslab = dh >> 6;  // width of the q / gate / o tiles as addressed, and their slabs
   constexpr int hd = wide ? 128 : 64, vslab = hd >> 6;    // width of a real head: of k and v as stored, of the state's value side
   // tensor memory columns (the pair keeps two read-out and two score accumulators where the state needs half the columns)
@@ -406,7 +416,7 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   {
     const bf16* Wh = a.W + (size_t)h0 * hd * hd;
 #pragma unroll 1
-    for (int idx = tid; idx < 16 * D; idx += THREADS) {
+    for (int idx = tid; idx < 16 * D; idx += threads_of(WIDTH)) {
       const int e = idx & (D - 1), oc = idx >> 7;
       uint32_t w[4] = {0u, 0u, 0u, 0u};
       if (pair) {
@@ -430,10 +440,10 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   // the tiles are never read; the one exception is the kh operand of the state update, whose M = 128 rows are the key
   // channels: its second slab is zeroed here and never written
   if (narrow)
-    for (int i = tid; i < 8192 / 16; i += THREADS) reinterpret_cast<uint4*>(sg + OFF_KH + 8192)[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = tid; i < 8192 / 16; i += threads_of(WIDTH)) reinterpret_cast<uint4*>(sg + OFF_KH + 8192)[i] = make_uint4(0u, 0u, 0u, 0u);
   // constant "ones" operand and the zeroed column blocks of the state operand that carry z (unswizzled 8x8 core matrices)
-  for (int i = tid; i < 2048 / 4; i += THREADS) reinterpret_cast<uint32_t*>(sg + OFF_ONES)[i] = 0u;
-  for (int i = tid; i < 4096 / 4; i += THREADS) reinterpret_cast<uint32_t*>(sg + OFF_SBF + (hd >> 3) * 2048)[i] = 0u;
+  for (int i = tid; i < 2048 / 4; i += threads_of(WIDTH)) reinterpret_cast<uint32_t*>(sg + OFF_ONES)[i] = 0u;
+  for (int i = tid; i < 4096 / 4; i += threads_of(WIDTH)) reinterpret_cast<uint32_t*>(sg + OFF_SBF + (hd >> 3) * 2048)[i] = 0u;
   // raw rows in front of the segment: earlier tokens, or the conv cache, or zeros (Section 4.1)
   if (tid < 96) {
     const int st = tid / 48, r = (tid % 48) / 16, oc = tid % 16;
@@ -592,7 +602,7 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       // (a 64-wide head: 4 instead of 8 K steps over the channels, 64 instead of 128 output columns)
       const int ksteps = narrow ? 4 : 8, NW = narrow ? 64 : 128;  // (the mix: channels contracted, output columns)
       constexpr int NV = hd;  // value columns of the state and of the read-out
-      auto issue_mma1 = [&]() {
+      [[maybe_unused]] auto issue_mma1 = [&]() {
         const uint32_t ID = instr_desc(128, NW, FMT_F16, MAJOR_K, MAJOR_K);
 #pragma unroll
         for (int k = 0; k < 8; ++k)
@@ -600,8 +610,8 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         mma_commit(bar(B_MMA1));
       };
       bool ok = nchunks > 0;
-      if (ok) ok = wait_set_or_abort(bar(0), BIT(B_U_FULL), 0u, lane, s_abort, a.wait_limit);
-      if (ok && lane == 0) {
+      if (!mixw && ok) ok = wait_set_or_abort(bar(0), BIT(B_U_FULL), 0u, lane, s_abort, a.wait_limit);
+      if (!mixw && ok && lane == 0) {
         tc_fence_after_sync();
         issue_mma1();
       }
@@ -625,7 +635,7 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
           mma_commit(bar(B_P));
         }
         TL(0, 1, n, lane == 0);
-        if (n + 1 < nchunks) {
+        if (!mixw && n + 1 < nchunks) {
           // then the mix of the next chunk: its phi sweeps read Y while this chunk's read-out and state update execute
           WAITSET(BIT(B_U_FULL) | BIT(B_Y_FREE), PAR(B_U_FULL, pp) | PAR(B_Y_FREE, p));
           if (lane == 0) {
@@ -677,6 +687,25 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
           TL(0, 5, n, lane == 0);
         }
       }
+    }
+  } else if (mixw && warp == MIX_WARP) {
+    // ================================================================================================ mix issuer
+    const uint64_t dsc_u = smem_desc(sb + OFF_AU, 16, 1024, LAYOUT_SW128);
+    const uint64_t dsc_w = smem_desc(sb + OFF_W, 16, 1024, LAYOUT_SW128);
+    constexpr uint32_t ID = instr_desc(128, narrow ? 64 : 128, FMT_F16, MAJOR_K, MAJOR_K);
+    for (int n = 0; n < nchunks; ++n) {
+      WAITSET(BIT(B_U_FULL) | (n > 0 ? BIT(B_Y_FREE) : 0u), PAR(B_U_FULL, n & 1) | PAR(B_Y_FREE, (n - 1) & 1));
+      if (lane == 0) {
+        tc_fence_after_sync();
+#pragma unroll
+        for (int k = 0; k < (narrow ? 4 : 8); ++k) {
+          const uint32_t off = (uint32_t)((k >> 2) * (16384 >> 4) + (k & 3) * 2);
+          mma_f16(tmem + COL_Y, (dsc_u & 0xFFFFFFFF00000000ull) | (uint64_t)((uint32_t)dsc_u + off),
+                  (dsc_w & 0xFFFFFFFF00000000ull) | (uint64_t)((uint32_t)dsc_w + off), ID, k > 0);
+        }
+        mma_commit(bar(B_MMA1));
+      }
+      __syncwarp();
     }
   } else if (warp < ROW_WARP0) {
     // ================================================================================================ prep warps
@@ -1061,141 +1090,151 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       const bool f16 = __int_as_float(s_rmax[p]) <= RMAX_F16 && __int_as_float(s_sbound[p]) < SMAX_F16;
       // (the 8-bit-mantissa operands keep the range but not the accuracy bound: the caller is told)
       if (MODE == 0 && !f16 && tw == 0 && a.dev_status) atomicMax(a.dev_status, (int)LAWCAT_ERR_NUMERIC);
-      // ---- state pass: 16-bit operand 2^b_mid [S|z], accumulator [S|z] *= 2^b_C (this thread: 64 columns of row r128)
-      // (64-wide head: only the rows and columns that exist)
-      const bool s_on = !narrow || (!padded && r128 < dh);
-      // The largest state entry (which decides between fp16 and bf16 operands) is measured every 8th chunk; in between
-      // its bound grows by 64 max|v| per chunk (kh <= 1), a few thousand at most against the threshold of 3e4.
+      // The passes that write operands exist once per operand type and with or without the dropped softmax sum, picked by one
+      // branch: with the choice at every conversion the code that runs was strewn over twice its size.
       const bool track = (n & 7) == 0;
-      if (!fail && !s_on && !phi_on) mbar_arrive(bar(B_X_FREE));  // (see the end of the pass)
-      if (!fail && s_on) {
-        const int c = r128;
-        const float bm = vec(p, 0)[c], ft = vec(p, 1)[c];
-        const float dm = ex2f(bm), dC = ex2f(bm + ft);
-        if (ch == 0) dsum += bm + ft;
-        float mx = 0.f;
-        // (pair: 64 value columns, 32 per thread)
+      auto write_operands = [&](auto f16c, auto qsumc) {
+        constexpr bool F16 = decltype(f16c)::value, QSUM = decltype(qsumc)::value;
+        // ---- state pass: 16-bit operand 2^b_mid [S|z], accumulator [S|z] *= 2^b_C (this thread: 64 columns of row r128)
+        // (64-wide head: only the rows and columns that exist)
+        const bool s_on = !narrow || (!padded && r128 < dh);
+        // The largest state entry (which decides between fp16 and bf16 operands) is measured every 8th chunk; in between
+        // its bound grows by 64 max|v| per chunk (kh <= 1), a few thousand at most against the threshold of 3e4.
+        if (!fail && !s_on && !phi_on) mbar_arrive(bar(B_X_FREE));  // (see the end of the pass)
+        if (!fail && s_on) {
+          const int c = r128;
+          const float bm = vec(p, 0)[c], ft = vec(p, 1)[c];
+          const float dm = ex2f(bm), dC = ex2f(bm + ft);
+          if (ch == 0) dsum += bm + ft;
+          float mx = 0.f;
+          // (pair: 64 value columns, 32 per thread)
 #pragma unroll 1
-        for (int b2 = 0; b2 < (pair ? 1 : 2); ++b2) {
-          const int blk = pair ? ch : ch * 2 + b2;
-          tmem_ld32(lane_base + cS + blk * 32, y);
-          tmem_wait_ld();
-          if (MODE == 0) {
-            if (track) {
-#pragma unroll
-              for (int i = 0; i < 32; ++i) mx = fmaxf(mx, fabsf(y[i]));
-            }
-            const uint64_t dm2 = f2_pack(dm, dm);
-#pragma unroll
-            for (int q4 = 0; q4 < 4; ++q4) {
-              uint64_t w[4];
-#pragma unroll
-              for (int i = 0; i < 4; ++i) w[i] = f2_mul(dm2, f2_pack(y[8 * q4 + 2 * i], y[8 * q4 + 2 * i + 1]));
-              // columns [8 nb, 8 nb + 8) of row c: block nb of the unswizzled operand (a warp's 32 rows: 512 contiguous bytes)
-              sts128(sb + OFF_SBF + (uint32_t)(blk * 4 + q4) * 2048u + (uint32_t)c * 16u, pack8p(w, f16));
-            }
-          }
-          {
-            const uint64_t dC2 = f2_pack(dC, dC);
-#pragma unroll
-            for (int i = 0; i < 32; i += 2) f2_unpack(f2_mul(dC2, f2_pack(y[i], y[i + 1])), y[i], y[i + 1]);
-          }
-          tmem_st32(lane_base + cS + blk * 32, y);
-        }
-        if (ch == (narrow ? 0 : 1)) {  // (the thread of the row's last existing column half also carries z)
-          const float z = tmem_ld1(lane_base + cSZ);
-          tmem_wait_ld();
-          if (MODE == 0) {
-            *reinterpret_cast<uint16_t*>(sg + OFF_SBF + (hd >> 3) * 2048 + c * 16) = to16(dm * z, f16);
-            if (track) mx = fmaxf(mx, fabsf(z));
-          }
-          tmem_st1(lane_base + cSZ, dC * z);
-        }
-        if (MODE == 0 && track) {
-          mx = warp_max(mx);
-          if (lane == 0) atomicMax(s_smax, __float_as_int(mx < 3.0e38f ? mx : 3.0e38f));
-        }
-        tmem_wait_st();
-        if (!phi_on) mbar_arrive(bar(B_X_FREE));  // (state-only pass) this thread has read bm, ft and reads no exponents
-      }
-      TL(warp == 8 ? 1 : 2, 6, n, (warp == 8 || warp == 10) && lane == 0);
-      // ---- phi, writing sweep -------------------------------------------------------------------------------------------
-      if (phi_on && !fail && !padded) {
-        if (is_q) {
-          float qsum = 0.f;
-          auto q_block = [&](const float* yy, int jj0) {  // 16 columns = channel groups jj0, jj0 + 1
-#pragma unroll
-            for (int h2 = 0; h2 < 2; ++h2) {
-              const int jj = jj0 + h2;
-              float x[8], v[8];
-              load_x8(sb + OFF_X, row, jj, x);
-#pragma unroll
-              for (int i = 0; i < 8; ++i) v[i] = ex2f(fmaf(yy[h2 * 8 + i], L2E, x[i] - mb));
-              if (need_qsum) {
-#pragma unroll
-                for (int i = 0; i < 8; ++i) qsum += ex2f(fmaf(yy[h2 * 8 + i], L2E, -mb));
-              }
-              sts128(sb + OFF_QK + ch * 16384 + sw128(row, jj & 7), pack8(v, f16));
-            }
-          };
-          // (`ya` holds the first 16 columns since the row-max sweep)
-#pragma unroll 1
-          for (int b4 = 0; b4 < 4; ++b4) {
+          for (int b2 = 0; b2 < (pair ? 1 : 2); ++b2) {
+            const int blk = pair ? ch : ch * 2 + b2;
+            tmem_ld32(lane_base + cS + blk * 32, y);
             tmem_wait_ld();
+            if (MODE == 0) {
+              if (track) {
 #pragma unroll
-            for (int i = 0; i < 16; ++i) yb[i] = ya[i];
-            if (b4 < 3) tmem_ld16(ycol + b4 * 16 + 16, ya);
-            q_block(yb, ch * 8 + b4 * 2);
-          }
-          if (need_qsum) {
-            // the dropped normalizer travels to the output pass through tensor memory: each half adds its part
-            tmem_st1(lane_base + cMAIL + 4 * p + ch, qsum);
-            tmem_wait_st();
-          }
-        } else {
-          const float inv = row < nvalid ? 1.f / sum : 0.f;  // tokens past the end contribute nothing
-          const float* e63v = vec(p, 2);
-          auto k_block = [&](const float* ee, int jj0) {  // 16 columns = channel groups jj0, jj0 + 1
+                for (int i = 0; i < 32; ++i) mx = fmaxf(mx, fabsf(y[i]));
+              }
+              const uint64_t dm2 = f2_pack(dm, dm);
 #pragma unroll
-            for (int h2 = 0; h2 < 2; ++h2) {
-              const int jj = jj0 + h2;  // channels [8 jj, 8 jj + 8)
-              float x[8], ks[8];
-              load_x8(sb + OFF_X, row, jj, x);
-              const float4 ea = *reinterpret_cast<const float4*>(e63v + jj * 8);
-              const float4 eb = *reinterpret_cast<const float4*>(e63v + jj * 8 + 4);
-              const float e63[8] = {ea.x, ea.y, ea.z, ea.w, eb.x, eb.y, eb.z, eb.w};
+              for (int q4 = 0; q4 < 4; ++q4) {
+                uint64_t w[4];
 #pragma unroll
-              for (int i = 0; i < 8; ++i) ks[i] = ee[h2 * 8 + i] * inv * ex2f(-x[i]);
-              if (MODE == 0) sts128(sb + OFF_QK + ch * 16384 + sw128(C + row, jj & 7), pack8(ks, f16));
-#pragma unroll
-              for (int i = 0; i < 8; ++i) ks[i] *= e63[i];
-              // kh: row = token, MN-major A operand of the state update (slab = column half)
-              sts128(sb + OFF_KH + ch * 8192 + sw128(row, jj & 7), pack8(ks, true));
+                for (int i = 0; i < 4; ++i) w[i] = f2_mul(dm2, f2_pack(y[8 * q4 + 2 * i], y[8 * q4 + 2 * i + 1]));
+                // columns [8 nb, 8 nb + 8) of row c: block nb of the unswizzled operand (a warp's 32 rows: 512 contiguous bytes)
+                sts128(sb + OFF_SBF + (uint32_t)(blk * 4 + q4) * 2048u + (uint32_t)c * 16u, pack8p(w, F16));
+              }
             }
-          };
-          tmem_ld16(ycol, ya);
-          if (MODE == 0) {
+            {
+              const uint64_t dC2 = f2_pack(dC, dC);
+#pragma unroll
+              for (int i = 0; i < 32; i += 2) f2_unpack(f2_mul(dC2, f2_pack(y[i], y[i + 1])), y[i], y[i + 1]);
+            }
+            tmem_st32(lane_base + cS + blk * 32, y);
+          }
+          if (ch == (narrow ? 0 : 1)) {  // (the thread of the row's last existing column half also carries z)
+            const float z = tmem_ld1(lane_base + cSZ);
+            tmem_wait_ld();
+            if (MODE == 0) {
+              *reinterpret_cast<uint16_t*>(sg + OFF_SBF + (hd >> 3) * 2048 + c * 16) = to16(dm * z, F16);
+              if (track) mx = fmaxf(mx, fabsf(z));
+            }
+            tmem_st1(lane_base + cSZ, dC * z);
+          }
+          if (MODE == 0 && track) {
+            mx = warp_max(mx);
+            if (lane == 0) atomicMax(s_smax, __float_as_int(mx < 3.0e38f ? mx : 3.0e38f));
+          }
+          tmem_wait_st();
+          if (!phi_on) mbar_arrive(bar(B_X_FREE));  // (state-only pass) this thread has read bm, ft and reads no exponents
+        }
+        TL(warp == 8 ? 1 : 2, 6, n, (warp == 8 || warp == 10) && lane == 0);
+        // ---- phi, writing sweep -------------------------------------------------------------------------------------------
+        if (phi_on && !fail && !padded) {
+          if (is_q) {
+            float qsum = 0.f;
+            auto q_block = [&](const float* yy, int jj0) {  // 16 columns = channel groups jj0, jj0 + 1
+#pragma unroll
+              for (int h2 = 0; h2 < 2; ++h2) {
+                const int jj = jj0 + h2;
+                float x[8], v[8];
+                load_x8(sb + OFF_X, row, jj, x);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) v[i] = ex2f(fmaf(yy[h2 * 8 + i], L2E, x[i] - mb));
+                if (QSUM) {
+#pragma unroll
+                  for (int i = 0; i < 8; ++i) qsum += ex2f(fmaf(yy[h2 * 8 + i], L2E, -mb));
+                }
+                sts128(sb + OFF_QK + ch * 16384 + sw128(row, jj & 7), pack8(v, F16));
+              }
+            };
+            // (`ya` holds the first 16 columns since the row-max sweep)
 #pragma unroll 1
             for (int b4 = 0; b4 < 4; ++b4) {
               tmem_wait_ld();
 #pragma unroll
               for (int i = 0; i < 16; ++i) yb[i] = ya[i];
               if (b4 < 3) tmem_ld16(ycol + b4 * 16 + 16, ya);
-              k_block(yb, ch * 8 + b4 * 2);
+              q_block(yb, ch * 8 + b4 * 2);
             }
-          } else {  // (the state-only pass is small enough to afford two copies, with a load in flight across both)
+            if (QSUM) {
+              // the dropped normalizer travels to the output pass through tensor memory: each half adds its part
+              tmem_st1(lane_base + cMAIL + 4 * p + ch, qsum);
+              tmem_wait_st();
+            }
+          } else {
+            const float inv = row < nvalid ? 1.f / sum : 0.f;  // tokens past the end contribute nothing
+            const float* e63v = vec(p, 2);
+            auto k_block = [&](const float* ee, int jj0) {  // 16 columns = channel groups jj0, jj0 + 1
+#pragma unroll
+              for (int h2 = 0; h2 < 2; ++h2) {
+                const int jj = jj0 + h2;  // channels [8 jj, 8 jj + 8)
+                float x[8], ks[8];
+                load_x8(sb + OFF_X, row, jj, x);
+                const float4 ea = *reinterpret_cast<const float4*>(e63v + jj * 8);
+                const float4 eb = *reinterpret_cast<const float4*>(e63v + jj * 8 + 4);
+                const float e63[8] = {ea.x, ea.y, ea.z, ea.w, eb.x, eb.y, eb.z, eb.w};
+#pragma unroll
+                for (int i = 0; i < 8; ++i) ks[i] = ee[h2 * 8 + i] * inv * ex2f(-x[i]);
+                if (MODE == 0) sts128(sb + OFF_QK + ch * 16384 + sw128(C + row, jj & 7), pack8(ks, F16));
+#pragma unroll
+                for (int i = 0; i < 8; ++i) ks[i] *= e63[i];
+                // kh: row = token, MN-major A operand of the state update (slab = column half)
+                sts128(sb + OFF_KH + ch * 8192 + sw128(row, jj & 7), pack8(ks, true));
+              }
+            };
+            tmem_ld16(ycol, ya);
+            if (MODE == 0) {
 #pragma unroll 1
-            for (int b2 = 0; b2 < 2; ++b2) {
-              tmem_wait_ld();
-              tmem_ld16(ycol + b2 * 32 + 16, yb);
-              k_block(ya, ch * 8 + b2 * 4);
-              tmem_wait_ld();
-              if (b2 < 1) tmem_ld16(ycol + b2 * 32 + 32, ya);
-              k_block(yb, ch * 8 + b2 * 4 + 2);
+              for (int b4 = 0; b4 < 4; ++b4) {
+                tmem_wait_ld();
+#pragma unroll
+                for (int i = 0; i < 16; ++i) yb[i] = ya[i];
+                if (b4 < 3) tmem_ld16(ycol + b4 * 16 + 16, ya);
+                k_block(yb, ch * 8 + b4 * 2);
+              }
+            } else {  // (the state-only pass is small enough to afford two copies, with a load in flight across both)
+#pragma unroll 1
+              for (int b2 = 0; b2 < 2; ++b2) {
+                tmem_wait_ld();
+                tmem_ld16(ycol + b2 * 32 + 16, yb);
+                k_block(ya, ch * 8 + b2 * 4);
+                tmem_wait_ld();
+                if (b2 < 1) tmem_ld16(ycol + b2 * 32 + 32, ya);
+                k_block(yb, ch * 8 + b2 * 4 + 2);
+              }
             }
           }
         }
-      }
+      };
+      if (MODE == 1) write_operands(std::true_type{}, std::false_type{});  // (no operand of a choosable type)
+      else if (f16 && !need_qsum) write_operands(std::true_type{}, std::false_type{});
+      else if (f16) write_operands(std::true_type{}, std::true_type{});
+      else if (!need_qsum) write_operands(std::false_type{}, std::false_type{});
+      else write_operands(std::false_type{}, std::true_type{});
       // ---- hand-over to MMA 2: state operand, qs / ks / kh, and the bound on the state for the next chunk ------------
       TL(warp == 8 ? 1 : 2, 7, n, (warp == 8 || warp == 10) && lane == 0);
       WAITF(B_VH_FULL, p);  // the chunk's max|v| is known
