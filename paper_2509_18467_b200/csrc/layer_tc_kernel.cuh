@@ -383,149 +383,147 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
 
   // ---- one-time setup --------------------------------------------------------------------------------------------
   if (MODE == 1) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // (the scan may be scheduled behind)
-  if (tid == 0) {
-    const int nphi = MODE == 0 ? 256 : 128;  // threads of the phi pass: all row threads, or the key rows only
-    mbar_init(bar(B_RAW_FULL), 1);
-    mbar_init(bar(B_G_FULL), 1);
-    mbar_init(bar(B_V_FULL), 1);
-    mbar_init(bar(B_G_FREE), PREP_THREADS);
-    mbar_init(bar(B_U_FULL), PREP_THREADS);
-    mbar_init(bar(B_X_FULL), PREP_THREADS);
-    mbar_init(bar(B_VH_FULL), PREP_THREADS);
-    mbar_init(bar(B_MMA1), 1);
-    mbar_init(bar(B_Y_FREE), nphi);
-    mbar_init(bar(B_X_FREE), 256);  // every row thread: it reads bm, ft and (phi threads) the exponents
-    mbar_init(bar(B_QK_FULL), nphi);
-    mbar_init(bar(B_SBF_FULL), 256);
-    mbar_init(bar(B_P), 1);
-    mbar_init(bar(B_MMA2), 1);
-    mbar_init(bar(B_PH_FULL), 128);
-    mbar_init(bar(B_MMA3), 1);
-    mbar_init(bar(B_O_FREE), 128);
-    mbar_fence_init();
-    s_flags[1] = 0;
-    for (int i = 0; i < 7; ++i) s_rmax[i] = 0;
-    tma_prefetch_desc(&tm_q); tma_prefetch_desc(&tm_k); tma_prefetch_desc(&tm_v); tma_prefetch_desc(&tm_g);
-  }
-  if (warp == MMA_WARP) {
+  // Three groups of warps prepare side by side, with all their loads in flight before the first is used: a block of a short
+  // sequence spent a third of its time here, most of it in loads that waited for one another (given states 18k cycles, now
+  // 2k; W 2k; the first tiles were asked for 3k cycles after the rest).
+  const int tt_first = sq.tm_t + t_begin;  // (token coordinate of the first chunk in the tensor maps)
+  auto load_raw = [&](int tt0) {
+    mbar_arrive_expect_tx(bar(B_RAW_FULL), (MODE == 0 ? 16384u : 8192u) * (uint32_t)nslab);
+#pragma unroll 1
+    for (int s = 0; s < nslab; ++s) {
+      if (MODE == 0) tma_load_4d(sb + OFF_AU + s * 16384, &tm_q, bar(B_RAW_FULL), s * 64, h, tt0, sq.tm_b);
+      // (pair: the same 64 key channels into both halves of the tile)
+      tma_load_4d(sb + OFF_AU + s * 16384 + 8192, &tm_k, bar(B_RAW_FULL), pair ? 0 : s * 64, j, tt0, sq.tm_b);
+    }
+  };
+  auto load_gate = [&](int tt0) {
+    mbar_arrive_expect_tx(bar(B_G_FULL), 8192u * (uint32_t)nslab);
+    tma_load_4d(sb + OFF_G, &tm_g, bar(B_G_FULL), 0, h, tt0, sq.tm_b);
+    if (nslab == 2) tma_load_4d(sb + OFF_G + 8192, &tm_g, bar(B_G_FULL), 64, h, tt0, sq.tm_b);
+  };
+  auto load_v = [&](int tt0) {
+    mbar_arrive_expect_tx(bar(B_V_FULL), 8192u * (uint32_t)vslab);
+    tma_load_4d(sb + OFF_V, &tm_v, bar(B_V_FULL), 0, j, tt0, sq.tm_b);
+    if (vslab == 2) tma_load_4d(sb + OFF_V + 8192, &tm_v, bar(B_V_FULL), 64, j, tt0, sq.tm_b);
+  };
+  // Row warps move states between global memory, where a row is contiguous, and tensor memory, where it belongs to one lane,
+  // through 16-byte units in shared memory: a warp's 32 rows x NC columns, units XOR-swizzled with the row so that both
+  // directions are free of bank conflicts. Lane by lane straight from memory every access would touch 32 lines. (The room:
+  // the qs | ks tile and the S part of the state operand, which only the row warps write and no product reads outside the
+  // chunk loop.)
+  constexpr int NC = pair ? 32 : 64, LPR = NC / 4, RPI = 32 / LPR;  // columns a thread owns; lanes per row, rows per access
+  const int rw = warp - ROW_WARP0, rw_row0 = (rw & 3) * 32, rw_col0 = (rw >> 2) * NC;  // the warp's first row and column
+  const bool rw_on = rw_row0 < dh && rw_col0 < hd;  // (64-wide head: the rows and columns that exist)
+  const uint32_t rw_stage = sb + (pair ? OFF_QK + (uint32_t)rw * 4096u : (rw < 4 ? OFF_QK : OFF_SBF) + (uint32_t)(rw & 3) * 8192u);
+  auto stage_at = [&](int r, int unit) -> uint32_t { return rw_stage + (uint32_t)(r * NC * 4 + ((unit ^ (r & 7)) << 4)); };
+  const bool first = seg == 0;  // a sequence's first segment starts from the caller's state, the others from the scan's
+  const float* const srcS = MODE == 1 ? nullptr : first ? a.S0 : a.seg_S;
+  const float* const srcz = MODE == 1 ? nullptr : first ? a.z0 : a.seg_z;
+  if (warp == TMA_WARP) {
+    if (lane == 0) {
+      const int nphi = MODE == 0 ? 256 : 128;  // threads of the phi pass: all row threads, or the key rows only
+      mbar_init(bar(B_RAW_FULL), 1);
+      mbar_init(bar(B_G_FULL), 1);
+      mbar_init(bar(B_V_FULL), 1);
+      mbar_init(bar(B_G_FREE), PREP_THREADS);
+      mbar_init(bar(B_U_FULL), PREP_THREADS);
+      mbar_init(bar(B_X_FULL), PREP_THREADS);
+      mbar_init(bar(B_VH_FULL), PREP_THREADS);
+      mbar_init(bar(B_MMA1), 1);
+      mbar_init(bar(B_Y_FREE), nphi);
+      mbar_init(bar(B_X_FREE), 256);  // every row thread: it reads bm, ft and (phi threads) the exponents
+      mbar_init(bar(B_QK_FULL), nphi);
+      mbar_init(bar(B_SBF_FULL), 256);
+      mbar_init(bar(B_P), 1);
+      mbar_init(bar(B_MMA2), 1);
+      mbar_init(bar(B_PH_FULL), 128);
+      mbar_init(bar(B_MMA3), 1);
+      mbar_init(bar(B_O_FREE), 128);
+      mbar_fence_init();
+      if (nchunks > 0) {
+        load_raw(tt_first);
+        if (a.gate_dim != 1) load_gate(tt_first);
+        load_v(tt_first);
+      }
+      s_flags[1] = 0;
+      for (int i = 0; i < 7; ++i) s_rmax[i] = 0;
+    }
+  } else if (warp == MMA_WARP) {
     tmem_alloc(sb + OFF_BAR + 8 * NUM_BARS, TMEM_COLS);
     tmem_relinquish();
-  }
-  // W_h^T into its K-major slabs as fp16: row e holds W[h][c][e] over c
-  // (pair: block-diagonal, W of head 2 h in the upper left 64 x 64 block, W of head 2 h + 1 in the lower right)
-  {
-    const bf16* Wh = a.W + (size_t)h0 * hd * hd;
-#pragma unroll 1
-    for (int idx = tid; idx < 16 * D; idx += threads_of(WIDTH)) {
-      const int e = idx & (D - 1), oc = idx >> 7;
-      uint32_t w[4] = {0u, 0u, 0u, 0u};
-      if (pair) {
-        if ((e >> 6) == (oc >> 3)) {
-          const bf16* Wp = Wh + (size_t)(oc >> 3) * hd * hd;
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-            w[i] = pack_f16(__bfloat162float(Wp[(size_t)((oc & 7) * 8 + 2 * i) * hd + (e & 63)]),
-                            __bfloat162float(Wp[(size_t)((oc & 7) * 8 + 2 * i + 1) * hd + (e & 63)]));
-        }
-      } else if (e < dh && oc * 8 < dh) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-          w[i] = pack_f16(__bfloat162float(Wh[(size_t)(oc * 8 + 2 * i) * dh + e]),
-                          __bfloat162float(Wh[(size_t)(oc * 8 + 2 * i + 1) * dh + e]));
+  } else if (warp < ROW_WARP0) {
+    // raw rows in front of the segment: earlier tokens, or the conv cache, or zeros (Section 4.1)
+    uint4 halo = make_uint4(0u, 0u, 0u, 0u);
+    const int hst = tid / 48, hr = (tid % 48) / 16, hoc = tid % 16;
+    if (tid < 96 && hoc * 8 < dh) {  // (padded channels: zero)
+      // row stride and offset of this block's channels in the stream as stored (pair: the key stream's 64 channels serve
+      // both halves of the tile)
+      const size_t rstride = hst ? (size_t)a.Hkv * hd : (size_t)Hn * dh;
+      const size_t coff = (hst ? (size_t)j * hd : (size_t)h * dh) + (size_t)((hst && pair) ? (hoc & 7) : hoc) * 8;
+      const int t = t_begin - HALO + hr;  // token of halo row hr
+      if (t >= 0) {
+        halo = *reinterpret_cast<const uint4*>((hst ? a.k : a.q) + (sq.row0 + t) * rstride + coff);
+      } else {
+        const bf16* cache = hst ? a.cache_k : a.cache_q;
+        const int ci = t + (a.K - 1);  // the cache holds tokens -(K-1) .. -1, oldest first
+        if (cache && ci >= 0) halo = *reinterpret_cast<const uint4*>(cache + ((size_t)b * (a.K - 1) + ci) * rstride + coff);
       }
-      sts128(sb + OFF_W + (oc >> 3) * 16384 + sw128(e, oc & 7), make_uint4(w[0], w[1], w[2], w[3]));
     }
-  }
-  // a 64-wide head: the products run over the first 64 channels / columns only (K = 64, N = 64), so the second slabs of
-  // the tiles are never read; the one exception is the kh operand of the state update, whose M = 128 rows are the key
-  // channels: its second slab is zeroed here and never written
-  if (narrow)
-    for (int i = tid; i < 8192 / 16; i += threads_of(WIDTH)) reinterpret_cast<uint4*>(sg + OFF_KH + 8192)[i] = make_uint4(0u, 0u, 0u, 0u);
-  // constant "ones" operand and the zeroed column blocks of the state operand that carry z (unswizzled 8x8 core matrices)
-  for (int i = tid; i < 2048 / 4; i += threads_of(WIDTH)) reinterpret_cast<uint32_t*>(sg + OFF_ONES)[i] = 0u;
-  for (int i = tid; i < 4096 / 4; i += threads_of(WIDTH)) reinterpret_cast<uint32_t*>(sg + OFF_SBF + (hd >> 3) * 2048)[i] = 0u;
-  // raw rows in front of the segment: earlier tokens, or the conv cache, or zeros (Section 4.1)
-  if (tid < 96) {
-    const int st = tid / 48, r = (tid % 48) / 16, oc = tid % 16;
-    // row stride and offset of this block's channels in the stream as stored (pair: the key stream's 64 channels serve
-    // both halves of the tile)
-    const size_t rstride = st ? (size_t)a.Hkv * hd : (size_t)Hn * dh;
-    const size_t coff = (st ? (size_t)j * hd : (size_t)h * dh) + (size_t)((st && pair) ? (oc & 7) : oc) * 8;
-    const int t = t_begin - HALO + r;  // token of halo row r
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (oc * 8 >= dh) {
-      // padded channels: zero
-    } else if (t >= 0) {
-      v = *reinterpret_cast<const uint4*>((st ? a.k : a.q) + (sq.row0 + t) * rstride + coff);
-    } else {
-      const bf16* cache = st ? a.cache_k : a.cache_q;
-      const int ci = t + (a.K - 1);  // the cache holds tokens -(K-1) .. -1, oldest first
-      if (cache && ci >= 0) v = *reinterpret_cast<const uint4*>(cache + ((size_t)b * (a.K - 1) + ci) * rstride + coff);
+    // W_h^T into its K-major slabs as fp16: row e holds W[h][c][e] over c. Thread: channels 2 lane, 2 lane + 1 of a slab and
+    // eight columns e; a warp fills eight 128-byte rows of a slab.
+    // (pair: block-diagonal, W of head 2 h in the upper left 64 x 64 block, W of head 2 h + 1 in the lower right)
+    uint4 w0[4], w1[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int oct = (warp & 3) * 4 + u, slab = warp >> 2;  // columns [8 oct, 8 oct + 8), channels [64 slab, 64 slab + 64)
+      w0[u] = w1[u] = make_uint4(0u, 0u, 0u, 0u);
+      if (pair ? (oct >> 3) == slab : oct * 8 < dh && slab < nslab) {
+        const bf16* Wc = a.W + (size_t)(h0 + (pair ? slab : 0)) * hd * hd + (size_t)((pair ? 0 : slab * 64) + 2 * lane) * hd +
+                         (pair ? (oct & 7) : oct) * 8;
+        w0[u] = *reinterpret_cast<const uint4*>(Wc);
+        w1[u] = *reinterpret_cast<const uint4*>(Wc + hd);
+      }
     }
-    *reinterpret_cast<uint4*>(sg + OFF_HALO + ((st * 3 + r) * 16 + oc) * 16) = v;
-  }
-  __syncthreads();
-  // conv caches after the last token (Section 4.1: the last K - 1 raw rows of [cache_in, x]): they depend on the raw
-  // inputs alone, so the block of a head's last segment writes them here (the key stream by the first head of a group)
-  if (MODE == 0 && seg == sq.nseg - 1 && sub == 0 && a.K > 1 && tid < PREP_THREADS) {
-    const int per = (a.K - 1) * (dh / 8);  // 16-byte units per stream (the key stream of a pair uses the first hd / 8 per row)
-    for (int idx = tid; idx < 2 * per; idx += PREP_THREADS) {
-      const int st = idx / per, r = (idx % per) / (dh / 8), oc = idx % (dh / 8);
-      bf16* dst = st ? a.cache_k_out : a.cache_q_out;
-      if (dst == nullptr || (st == 1 && (h0 % G != 0 || oc * 8 >= hd))) continue;
-      const size_t rstride = st ? (size_t)a.Hkv * hd : (size_t)Hn * dh;
-      const size_t coff = (st ? (size_t)j * hd : (size_t)h * dh) + (size_t)oc * 8;
-      const int tok = T - (a.K - 1) + r;
-      const bf16* x = st ? a.k : a.q;
-      const bf16* cin = st ? a.cache_k : a.cache_q;
-      uint4 v = make_uint4(0u, 0u, 0u, 0u);
-      if (tok >= 0) v = *reinterpret_cast<const uint4*>(x + (sq.row0 + tok) * rstride + coff);
-      else if (cin != nullptr) v = *reinterpret_cast<const uint4*>(cin + ((size_t)b * (a.K - 1) + tok + a.K - 1) * rstride + coff);
-      *reinterpret_cast<uint4*>(dst + ((size_t)b * (a.K - 1) + r) * rstride + coff) = v;
+    if (tid < 96) *reinterpret_cast<uint4*>(sg + OFF_HALO + ((hst * 3 + hr) * 16 + hoc) * 16) = halo;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int oct = (warp & 3) * 4 + u, slab = warp >> 2;
+      float x[8], y[8];
+      unpack8(w0[u], x);
+      unpack8(w1[u], y);
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        *reinterpret_cast<uint32_t*>(sg + OFF_W + slab * 16384 + sw128(oct * 8 + i, lane >> 2) + (lane & 3) * 4) = pack_f16(x[i], y[i]);
     }
+  } else if (warp < ROW_WARP0 + 8) {
+    const int rt = tid - ROW_WARP0 * 32;
+    if (srcS != nullptr && rw_on) {
+      const float* src = srcS + ((first ? seq_state(rw_row0) : seg_state(rw_row0)) * hd + (rw_row0 & (hd - 1))) * hd + rw_col0;
+#pragma unroll
+      for (int i = 0; i < 32 / RPI; ++i) {
+        const int r = i * RPI + lane / LPR, unit = lane % LPR;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(stage_at(r, unit)), "l"(src + (size_t)r * hd + unit * 4) : "memory");
+      }
+    }
+    // constant "ones" operand ([64 x 16], column 0 is 1) and the zeroed column blocks of the state operand that carry z
+    // (unswizzled 8x8 core matrices)
+    if (rt < 128) sts128(sb + OFF_ONES + rt * 16, make_uint4(rt < 64 ? 0x3C00u : 0u, 0u, 0u, 0u));
+    sts128(sb + OFF_SBF + (hd >> 3) * 2048 + rt * 16, make_uint4(0u, 0u, 0u, 0u));
+    // a 64-wide head: the products run over the first 64 channels / columns only (K = 64, N = 64), so the second slabs of
+    // the tiles are never read; the one exception is the kh operand of the state update, whose M = 128 rows are the key
+    // channels: its second slab is zeroed here and never written
+    if (narrow) {
+      sts128(sb + OFF_KH + 8192 + rt * 16, make_uint4(0u, 0u, 0u, 0u));
+      sts128(sb + OFF_KH + 12288 + rt * 16, make_uint4(0u, 0u, 0u, 0u));
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
   }
-  if (tid < C) *reinterpret_cast<__half*>(sg + OFF_ONES + (tid >> 3) * 128 + (tid & 7) * 16) = __float2half(1.f);
   fence_proxy_async();
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = (uint32_t)s_flags[0];
   const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-
-  // initial state into tensor memory: row thread (c, half) owns 64 columns of row c of [S | z]
-  if (warp >= ROW_WARP0 && warp < ROW_WARP0 + 8) {
-    // (pair: the state is [128 key channels x 64 value columns], the thread owns 32 columns; rows 64-127 are the second head)
-    const int tw = tid - ROW_WARP0 * 32, c = tw & 127, chh = tw >> 7;
-    // a sequence's first segment starts from the caller's state, the others from the scan's; pieces from zero
-    const bool first = seg == 0;
-    const float* const srcS = MODE == 1 ? nullptr : first ? a.S0 : a.seg_S;
-    const float* const srcz = MODE == 1 ? nullptr : first ? a.z0 : a.seg_z;
-    const bool have = srcS != nullptr, havez = srcz != nullptr;
-    const size_t in_idx = first ? seq_state(c) : seg_state(c);
-    const int cr = c & (hd - 1);  // row inside the real head's state
-    float s[32], mx = 0.f;
-#pragma unroll 1
-    for (int b2 = 0; b2 < (pair ? 1 : 2); ++b2) {
-      const int blk = pair ? chh : chh * 2 + b2;
-#pragma unroll
-      for (int i = 0; i < 32; ++i) {
-        s[i] = (have && c < dh && blk * 32 < hd) ? srcS[(in_idx * hd + cr) * hd + blk * 32 + i] : 0.f;
-        mx = fmaxf(mx, fabsf(s[i]));
-      }
-      tmem_st32(lane_base + cS + blk * 32, s);
-    }
-    if (chh == 1) {
-      const float z0v = (havez && c < dh) ? srcz[in_idx * hd + cr] : 0.f;
-      tmem_st1(lane_base + cSZ, z0v);
-      mx = fmaxf(mx, fabsf(z0v));
-    }
-    tmem_wait_st();
-    if (!(mx < 3.0e38f)) mx = 3.0e38f;  // NaN or inf in the given state: no fp16 operand
-    atomicMax(s_sbound, __float_as_int(mx));
-  }
-  tc_fence_before_sync();
-  __syncthreads();
-  tc_fence_after_sync();
 
 #define WAIT(b, par)                                     \
   if (!wait_or_abort(bar(b), (uint32_t)(par), s_abort, a.wait_limit)) break
@@ -543,30 +541,21 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   if (warp == TMA_WARP) {
     // ================================================================================================ TMA producer
     if (lane == 0) {
-      int ar_raw = -1, ar_g = -1, ar_v = -1;  // last chunk whose copies were started, per tile
-      for (int n = 0; n < nchunks; ++n) {
-        const int tt0 = sq.tm_t + t_begin + n * C;
+      const int cp0 = nchunks > 0 ? 0 : -1;  // (the first chunk's copies were started by the set-up)
+      int ar_raw = cp0, ar_g = a.gate_dim != 1 ? cp0 : -1, ar_v = cp0;  // last chunk whose copies were started, per tile
+      for (int n = 1; n < nchunks; ++n) {
+        const int tt0 = tt_first + n * C;
         const uint32_t pp = (uint32_t)((n - 1) & 1);
-        if (n > 0) WAIT(B_MMA1, pp);  // MMA 1 of the previous chunk has read the in-place conv output
-        mbar_arrive_expect_tx(bar(B_RAW_FULL), (MODE == 0 ? 16384u : 8192u) * (uint32_t)nslab);
-#pragma unroll 1
-        for (int s = 0; s < nslab; ++s) {
-          if (MODE == 0) tma_load_4d(sb + OFF_AU + s * 16384, &tm_q, bar(B_RAW_FULL), s * 64, h, tt0, sq.tm_b);
-          // (pair: the same 64 key channels into both halves of the tile)
-          tma_load_4d(sb + OFF_AU + s * 16384 + 8192, &tm_k, bar(B_RAW_FULL), pair ? 0 : s * 64, j, tt0, sq.tm_b);
-        }
+        WAIT(B_MMA1, pp);  // MMA 1 of the previous chunk has read the in-place conv output
+        load_raw(tt0);
         ar_raw = n;
         if (a.gate_dim != 1) {
-          if (n > 0) WAIT(B_G_FREE, pp);
-          mbar_arrive_expect_tx(bar(B_G_FULL), 8192u * (uint32_t)nslab);
-          tma_load_4d(sb + OFF_G, &tm_g, bar(B_G_FULL), 0, h, tt0, sq.tm_b);
-          if (nslab == 2) tma_load_4d(sb + OFF_G + 8192, &tm_g, bar(B_G_FULL), 64, h, tt0, sq.tm_b);
+          WAIT(B_G_FREE, pp);
+          load_gate(tt0);
           ar_g = n;
         }
-        if (n > 0) WAIT(MODE == 0 ? B_MMA3 : B_MMA2, pp);  // the last MMA that reads v
-        mbar_arrive_expect_tx(bar(B_V_FULL), 8192u * (uint32_t)vslab);
-        tma_load_4d(sb + OFF_V, &tm_v, bar(B_V_FULL), 0, j, tt0, sq.tm_b);
-        if (vslab == 2) tma_load_4d(sb + OFF_V + 8192, &tm_v, bar(B_V_FULL), 64, j, tt0, sq.tm_b);
+        WAIT(MODE == 0 ? B_MMA3 : B_MMA2, pp);  // the last MMA that reads v
+        load_v(tt0);
         ar_v = n;
       }
       if (*s_abort) {
@@ -578,6 +567,27 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     }
   } else if (warp == MMA_WARP) {
     // ================================================================================================ MMA issuer
+    // First, while the operands of the first chunk are made, the conv caches after the last token (Section 4.1: the last K - 1
+    // raw rows of [cache_in, x]): they depend on the raw inputs alone, so the block of a head's last segment writes them
+    // (the key stream by the first head of a group).
+    if (MODE == 0 && seg == sq.nseg - 1 && sub == 0 && a.K > 1) {
+      const int per = (a.K - 1) * (dh / 8);  // 16-byte units per stream (the key stream of a pair uses the first hd / 8 per row)
+      for (int idx = lane; idx < 2 * per; idx += 32) {
+        const int st = idx / per, r = (idx % per) / (dh / 8), oc = idx % (dh / 8);
+        bf16* dst = st ? a.cache_k_out : a.cache_q_out;
+        if (dst == nullptr || (st == 1 && (h0 % G != 0 || oc * 8 >= hd))) continue;
+        const size_t rstride = st ? (size_t)a.Hkv * hd : (size_t)Hn * dh;
+        const size_t coff = (st ? (size_t)j * hd : (size_t)h * dh) + (size_t)oc * 8;
+        const int tok = T - (a.K - 1) + r;
+        const bf16* x = st ? a.k : a.q;
+        const bf16* cin = st ? a.cache_k : a.cache_q;
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (tok >= 0) v = *reinterpret_cast<const uint4*>(x + (sq.row0 + tok) * rstride + coff);
+        else if (cin != nullptr) v = *reinterpret_cast<const uint4*>(cin + ((size_t)b * (a.K - 1) + tok + a.K - 1) * rstride + coff);
+        *reinterpret_cast<uint4*>(dst + ((size_t)b * (a.K - 1) + r) * rstride + coff) = v;
+      }
+      __syncwarp();
+    }
     // The whole warp walks the loop and waits (one lane per barrier of a set); lane 0 issues.
     {
       // shared-memory descriptors of the operands (all tiles sit at fixed addresses); a K step adds a constant to the
@@ -955,6 +965,36 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     // scores. The two threads of a row share a TMEM lane and meet through two spare TMEM columns (row max, softmax sum).
     // Order inside a chunk: the sweeps of phi that only READ (row max; key rows: exp and its sum) run while the previous
     // chunk's MMA 2 is still executing; the state pass and the sweep that writes qs / ks / kh wait for it.
+    {
+      // initial state into tensor memory: row thread (c, half) owns the NC columns of its half of row c of [S | z]
+      // (pieces and sequences without a given state start from zero)
+      const int c = rw_row0 + lane;
+      const bool have = srcS != nullptr && rw_on;
+      float s[32], mx = 0.f;
+#pragma unroll 1
+      for (int b2 = 0; b2 < NC / 32; ++b2) {
+#pragma unroll
+        for (int q4 = 0; q4 < 8; ++q4) {
+          uint4 v = make_uint4(0u, 0u, 0u, 0u);
+          if (have) v = lds128(stage_at(lane, b2 * 8 + q4));
+          s[4 * q4] = __uint_as_float(v.x); s[4 * q4 + 1] = __uint_as_float(v.y);
+          s[4 * q4 + 2] = __uint_as_float(v.z); s[4 * q4 + 3] = __uint_as_float(v.w);
+        }
+#pragma unroll
+        for (int i = 0; i < 32; ++i) mx = fmaxf(mx, fabsf(s[i]));
+        tmem_st32(lane_base + cS + rw_col0 + b2 * 32, s);
+      }
+      if (rw >= 4) {
+        const float z0v = (srcz != nullptr && c < dh)
+                              ? srcz[(first ? seq_state(c) : seg_state(c)) * hd + (c & (hd - 1))] : 0.f;
+        tmem_st1(lane_base + cSZ, z0v);
+        mx = fmaxf(mx, fabsf(z0v));
+      }
+      tmem_wait_st();
+      if (!(mx < 3.0e38f)) mx = 3.0e38f;  // NaN or inf in the given state: no fp16 operand
+      atomicMax(s_sbound, __float_as_int(mx));
+      named_bar_sync(2, 256);  // the bound is complete, and the room the state came through may be written
+    }
     const int tw = tid - ROW_WARP0 * 32;
     const int ch = tw >> 7;                       // column half: columns [64 ch, 64 ch + 64)
     const int r128 = (tw & 127);                  // row of Y and of the state (= TMEM lane)
@@ -1272,16 +1312,23 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       if (MODE == 1 && ch == 0 && c < dh) a.dtot[out_idx * hd + cr] = dsum;
       const bool last = MODE == 1 || seg2 == sv.nseg - 1;  // (each of the two outputs is optional on its own)
       if (a.S_T != nullptr && last) {
-        float s[32];
+        if (rw_on) {
+          float s[32];
 #pragma unroll 1
-        for (int b2 = 0; b2 < (pair ? 1 : 2); ++b2) {
-          const int blk = pair ? ch : ch * 2 + b2;
-          tmem_ld32(lane_base + cS + blk * 32, s);
-          tmem_wait_ld();
-          if (c < dh && blk * 32 < hd) {
+          for (int b2 = 0; b2 < NC / 32; ++b2) {
+            tmem_ld32(lane_base + cS + rw_col0 + b2 * 32, s);
+            tmem_wait_ld();
 #pragma unroll
-            for (int i = 0; i < 32; i += 4)
-              *reinterpret_cast<float4*>(a.S_T + (out_idx * hd + cr) * hd + blk * 32 + i) = make_float4(s[i], s[i + 1], s[i + 2], s[i + 3]);
+            for (int q4 = 0; q4 < 8; ++q4)
+              sts128(stage_at(lane, b2 * 8 + q4), make_uint4(__float_as_uint(s[4 * q4]), __float_as_uint(s[4 * q4 + 1]),
+                                                             __float_as_uint(s[4 * q4 + 2]), __float_as_uint(s[4 * q4 + 3])));
+          }
+          __syncwarp();
+          float* dst = a.S_T + (out_idx * hd + (rw_row0 & (hd - 1))) * hd + rw_col0;
+#pragma unroll 4
+          for (int i = 0; i < 32 / RPI; ++i) {
+            const int r = i * RPI + lane / LPR, unit = lane % LPR;
+            *reinterpret_cast<uint4*>(dst + (size_t)r * hd + unit * 4) = lds128(stage_at(r, unit));
           }
         }
       }
