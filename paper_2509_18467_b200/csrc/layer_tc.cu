@@ -85,28 +85,45 @@ __global__ void segment_scan_kernel(const TcArgs a, const __grid_constant__ Pack
   float* const start = isz ? start_z : start_S;
   float4 cur = make_float4(0.f, 0.f, 0.f, 0.f);
   if (init) cur = *reinterpret_cast<const float4*>(init + ((size_t)seq * a.H + h) * n + off);
+  // With few heads the blocks are few and a thread's own instructions are the time: the loop walks pointers and a counter
+  // of the pieces left in the segment, and the decay of a row of S is one exponential.
   const int np = (nseg - 1) * nsub;
-  constexpr int U = 4;  // pieces whose loads are in flight together
-  for (int i0 = 0; i0 < np; i0 += U) {
+  const size_t lstep = (size_t)a.H * n, dstep = (size_t)a.H * D;
+  const float* lp = loc + ((size_t)seg0 * nsub * a.H + h) * n + off;
+  const float* dp = dtot + ((size_t)seg0 * nsub * a.H + h) * D + (isz ? off : off / D);
+  float* sp = start + ((size_t)(seg0 + 1) * a.H + h) * n + off;
+  int left = nsub;
+  auto batch = [&](auto count) {  // pieces whose loads are in flight together
+    constexpr int U = decltype(count)::value;
     float4 l[U], d[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      if (i0 + u >= np) break;
-      const size_t si = ((size_t)seg0 * nsub + i0 + u) * a.H + h;
-      l[u] = *reinterpret_cast<const float4*>(loc + si * n + off);
-      // (the decay is per row of the state)
-      if (isz) d[u] = *reinterpret_cast<const float4*>(dtot + si * D + off);
-      else d[u].x = d[u].y = d[u].z = d[u].w = dtot[si * D + off / D];
+      l[u] = *reinterpret_cast<const float4*>(lp + u * lstep);
+      if (isz) d[u] = *reinterpret_cast<const float4*>(dp + u * dstep);
+      else d[u].x = dp[u * dstep];
     }
+    lp += U * lstep;
+    dp += U * dstep;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      if (i0 + u >= np) break;
-      cur.x = fmaf(exp2f(d[u].x), cur.x, l[u].x); cur.y = fmaf(exp2f(d[u].y), cur.y, l[u].y);
-      cur.z = fmaf(exp2f(d[u].z), cur.z, l[u].z); cur.w = fmaf(exp2f(d[u].w), cur.w, l[u].w);
-      if ((i0 + u + 1) % nsub == 0)
-        *reinterpret_cast<float4*>(start + ((size_t)(seg0 + (i0 + u + 1) / nsub) * a.H + h) * n + off) = cur;
+      const float ex = exp2f(d[u].x);
+      float4 e = make_float4(ex, ex, ex, ex);
+      if (isz) e = make_float4(ex, exp2f(d[u].y), exp2f(d[u].z), exp2f(d[u].w));
+      cur.x = fmaf(e.x, cur.x, l[u].x); cur.y = fmaf(e.y, cur.y, l[u].y);
+      cur.z = fmaf(e.z, cur.z, l[u].z); cur.w = fmaf(e.w, cur.w, l[u].w);
+      if (--left == 0) {
+        left = nsub;
+        *reinterpret_cast<float4*>(sp) = cur;
+        sp += lstep;
+      }
     }
-  }
+  };
+  int i0 = 0;
+  for (; i0 + 8 <= np; i0 += 8) batch(std::integral_constant<int, 8>{});
+  if (i0 + 4 <= np) { batch(std::integral_constant<int, 4>{}); i0 += 4; }
+  if (np - i0 == 3) batch(std::integral_constant<int, 3>{});
+  else if (np - i0 == 2) batch(std::integral_constant<int, 2>{});
+  else if (np - i0 == 1) batch(std::integral_constant<int, 1>{});
 }
 
 }  // namespace tc
