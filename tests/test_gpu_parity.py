@@ -315,3 +315,27 @@ def test_decode_head_groups(api, H, Hkv, d, K):
     if K > 1:
         assert np.array_equal(cq.float().cpu().numpy(), ref["cache_q"].astype(np.float32))
         assert np.array_equal(ck.float().cpu().numpy(), ref["cache_k"].astype(np.float32))
+
+
+@pytest.mark.parametrize("B,H,Hkv,d,K", [(75, 4, 2, 128, 4), (149, 2, 2, 128, 2), (5, 60, 20, 128, 3), (3, 148, 37, 128, 1),
+                                         (99, 6, 2, 64, 4), (298, 2, 1, 64, 1), (20, 30, 10, 128, 4)])
+def test_decode_many_heads(api, B, H, Hkv, d, K):
+    """The streaming decode step: from one or two heads more than fit in a single round of blocks; blocks with one to five
+    sequences (an empty pipeline up to tile slots used twice), groups of 1 to 4; three steps, so that the shifted caches are
+    read."""
+    import torch
+    s = shape(B, 3, H, Hkv, d, d, "bf16", conv_k=K, cid=47)
+    x = I.make(s, LAYER_NAMES + ["S0", "z0"] + (["cache_q", "cache_k"] if K > 1 else []))
+    t = dev(api, x, s)
+    S, z, cq, ck = t["S0"].clone(), t["z0"].clone(), t.get("cache_q"), t.get("cache_k")
+    ref = O.layer_fwd(oracle_params(s), *[x[n] for n in LAYER_NAMES], x.get("cache_q"), x.get("cache_k"), x["S0"], x["z0"])
+    api.trace_begin()
+    o = [api.lawcat_decode_step(P(api, s), *[t[n][:, i].contiguous() for n in LAYER_NAMES[:4]], t["w_q"], t["w_k"], t["W"], S, z,
+                                cq, ck) for i in range(3)]
+    assert "decode_stream" in api.trace_end()
+    check(torch.stack(o, 1), ref["o"], "bf16", "o")
+    check(S, ref["S_T"], "f32", "S")
+    check(z, ref["z_T"], "f32", "z")
+    if K > 1:
+        assert np.array_equal(cq.float().cpu().numpy(), ref["cache_q"].astype(np.float32))
+        assert np.array_equal(ck.float().cpu().numpy(), ref["cache_k"].astype(np.float32))
