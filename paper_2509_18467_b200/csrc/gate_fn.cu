@@ -49,7 +49,7 @@ using ctc::dadv;
 using ctc::kview;
 using ctc::toff;
 
-constexpr int TT = 128;        // tokens per thread block
+constexpr int TT = 128;        // token rows of a product; a block takes up to as many tokens (GArgs::tt)
 constexpr int NT = 128;        // outputs per product of the second layer
 constexpr int KS = 64;         // hidden channels per stage of the first layer
 constexpr int THREADS = 320;   // warp 0 copies, warp 1 products, warps 2-5 and 6-9 epilogue groups (TMEM quadrant = warp & 3)
@@ -88,6 +88,7 @@ struct GArgs {
   const bf16* A2;     // [n_out, rank]
   const bf16* bias;   // [n_out] or null
   int N, dm, n_out;
+  int tt;             // tokens per block, a multiple of 8 (the rows behind them hold whatever the buffers held: never stored)
   int* dev_status;
 };
 
@@ -119,7 +120,7 @@ gate_fn_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
   volatile int* const s_abort = s_flags + 1;
   float* const s_bias = reinterpret_cast<float*>(smem + L::OFF_BIAS);
   auto BAR = [&](int i) { return bars + 8u * (uint32_t)i; };
-  const int n0 = blockIdx.x * TT;
+  const int n0 = blockIdx.x * a.tt;
   // With fewer token tiles than SMs the output tiles of a token tile are shared out over gridDim.y blocks (each repeats the
   // first layer, whose x tile then comes from L2): this block's tiles are nt0 ... nt0 + ntile - 1, `nt` below counts from 0.
   const int nk = (a.dm + KS - 1) / KS, ntile_all = (a.n_out + NT - 1) / NT;
@@ -152,7 +153,7 @@ gate_fn_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         const int s = i % L::ST;
         if (i >= L::ST) ok = gwait(BAR(B_EMPTY0 + s), ((i / L::ST) - 1) & 1, s_abort);
         if (!ok) break;
-        mbar_arrive_expect_tx(BAR(B_FULL0 + s), L::STAGE);
+        mbar_arrive_expect_tx(BAR(B_FULL0 + s), (uint32_t)a.tt * 128u + L::A1_BYTES);
         tma_load_2d(sb + L::OFF_RING + s * L::STAGE, &tm_x, BAR(B_FULL0 + s), i * KS, n0);
         tma_load_2d(sb + L::OFF_RING + s * L::STAGE + L::X_BYTES, &tm_a1, BAR(B_FULL0 + s), i * KS, 0);
       }
@@ -516,9 +517,6 @@ template <int R>
 static int launch_tc(const Ctx& c, int d_model, const void* x, const void* A1, const void* A2, const void* bias,
                      void* gate, size_t N, int n_out) {
   using L = Lay<R>;
-  CUtensorMap tx, ta1, to;
-  if (!map_2d(&tx, x, N, d_model, TT) || !map_2d(&ta1, A1, R, d_model, R) || !map_2d(&to, gate, N, n_out, TT))
-    return LAWCAT_ERR_CUDA;
   static std::atomic<bool> raised[64] = {};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return LAWCAT_ERR_CUDA;
@@ -527,14 +525,27 @@ static int launch_tc(const Ctx& c, int d_model, const void* x, const void* A1, c
       return LAWCAT_ERR_CUDA;
     raised[dev].store(true);
   }
-  GArgs a{(const bf16*)A2, (const bf16*)bias, (int)N, d_model, n_out, c.dev_status};
   // fewer token tiles than the SMs can hold (two blocks each for rank <= 32): share each tile's outputs out over up to 8
   // blocks, every one of them with output tiles of its own
-  const size_t tiles = (N + TT - 1) / TT;
   const int ntile_all = (n_out + NT - 1) / NT, room = (R <= 32 ? 2 : 1) * sm_count_gfn();
+  size_t tiles = (N + TT - 1) / TT;
   int ysplit = (int)std::min<size_t>(8, std::max<size_t>(1, room / tiles));
   ysplit = std::min(ysplit, ntile_all);
   ysplit = (ntile_all + ((ntile_all + ysplit - 1) / ysplit) - 1) / ((ntile_all + ysplit - 1) / ysplit);  // (no empty block)
+  // With one block per tile the tiles come in whole rounds of the blocks that fit: 32768 tokens are 256 tiles of 128, which
+  // leave 40 SMs with one block where the others have two, or 293 tiles of 112 (114.2 -> 112.5 us at rank 32 and the 7B widths;
+  // 26000 tokens 103 -> 99.7, rank 16 92.2 -> 84.9; rank 64, one block per SM, 19000 tokens 136 -> 129.6). Not when the only round is hardly more than half full: blocks of half the
+  // height read A1 and A2 twice as often (19000 tokens, rank 32: 87.9 -> 89.7).
+  int tt = TT;
+  const size_t slots = (tiles + room - 1) / room * room;
+  if (ysplit == 1 && (tiles > (size_t)room || tiles * 20 > slots * 11)) {
+    tt = (int)std::min<size_t>(TT, ((N + slots - 1) / slots + 7) / 8 * 8);
+    tiles = (N + tt - 1) / tt;
+  }
+  GArgs a{(const bf16*)A2, (const bf16*)bias, (int)N, d_model, n_out, tt, c.dev_status};
+  CUtensorMap tx, ta1, to;
+  if (!map_2d(&tx, x, N, d_model, tt) || !map_2d(&ta1, A1, R, d_model, R) || !map_2d(&to, gate, N, n_out, tt))
+    return LAWCAT_ERR_CUDA;
   LAWCAT_LAUNCH("gate_fn_tc", c.stream,
                 gate_fn_tc_kernel<R><<<dim3((unsigned)tiles, (unsigned)ysplit), THREADS, L::BYTES, c.stream>>>(tx, ta1, to, a));
   LAWCAT_CHECK_LAUNCH();

@@ -55,6 +55,14 @@ def test_tensor_core_kernel(rank, B, T, H, d, gd, dm):
     assert e <= 1e-3, f"{e:.3e}"
 
 
+@pytest.mark.parametrize("rank,N", [(16, 21001), (32, 37760), (64, 10501), (128, 22007)])
+def test_tile_heights(rank, N):
+    """Tiles of fewer than 128 tokens (one round of blocks, two rounds; the last tile ragged) and, second, the largest height."""
+    got, want = run(1, N, 3, 64, 0, 72, rank, expect_tc=True, cfg=940)
+    _, e = err_bf16(got, want)
+    assert e <= 1e-3, f"{e:.3e}"
+
+
 @pytest.mark.parametrize("rank", [8, 24, 32, 128])
 @pytest.mark.parametrize("B,T,H,d,gd,dm", [
     (1, 1, 2, 64, 0, 128),       # one token (a decode step of one sequence)
