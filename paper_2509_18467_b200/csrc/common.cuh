@@ -128,6 +128,22 @@ struct LaunchScope {
   cudaStream_t stream;
   int idx;
 };
+// Launch of a kernel that begins with griddepcontrol.wait: its launch overlaps the end of the kernel in front of it on the
+// stream, and the wait holds it until that one's results are there.
+template <typename... P, typename... A>
+inline void launch_behind(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A... args) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
 #define LAWCAT_LAUNCH(name, strm, ...)       \
   do {                                       \
     ::lawcat::LaunchScope _ls(name, strm);   \

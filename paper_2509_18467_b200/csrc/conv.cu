@@ -654,6 +654,7 @@ __global__ void cache_out_kernel(const T* __restrict__ q, const T* __restrict__ 
                                  int Ck, int K) {
   const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int Ct = Cq + Ck;
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // (the caches read by the kernels in front may be the ones written here)
   if (idx >= (size_t)B * (K - 1) * Ct) return;
   int ch = (int)(idx % Ct);
   const int r = (int)((idx / Ct) % (K - 1)), b = (int)(idx / ((size_t)Ct * (K - 1)));
@@ -679,11 +680,11 @@ int launch_cache_out(const Ctx& c, const void* q, const void* k, const void* cac
   const unsigned blocks = (unsigned)((total + 255) / 256);
   LaunchScope _ls("cache_out", c.stream);
   if (p.dtype == LAWCAT_F32)
-    cache_out_kernel<float><<<blocks, 256, 0, c.stream>>>((const float*)q, (const float*)k, (const float*)cache_q_in, (const float*)cache_k_in,
-                                                          (float*)cache_q_out, (float*)cache_k_out, p.B, p.T, Cq, Ck, p.conv_k);
+    launch_behind(cache_out_kernel<float>, dim3(blocks), dim3(256), 0, c.stream, (const float*)q, (const float*)k, (const float*)cache_q_in,
+                  (const float*)cache_k_in, (float*)cache_q_out, (float*)cache_k_out, p.B, p.T, Cq, Ck, p.conv_k);
   else
-    cache_out_kernel<bf16><<<blocks, 256, 0, c.stream>>>((const bf16*)q, (const bf16*)k, (const bf16*)cache_q_in, (const bf16*)cache_k_in,
-                                                         (bf16*)cache_q_out, (bf16*)cache_k_out, p.B, p.T, Cq, Ck, p.conv_k);
+    launch_behind(cache_out_kernel<bf16>, dim3(blocks), dim3(256), 0, c.stream, (const bf16*)q, (const bf16*)k, (const bf16*)cache_q_in,
+                  (const bf16*)cache_k_in, (bf16*)cache_q_out, (bf16*)cache_k_out, p.B, p.T, Cq, Ck, p.conv_k);
   LAWCAT_CHECK_LAUNCH();
   return LAWCAT_OK;
 }

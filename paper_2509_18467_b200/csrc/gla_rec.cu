@@ -168,6 +168,7 @@ __global__ void __launch_bounds__(256, 2) gla_fwd_rec_kernel(const GlaArgs a, co
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // (three short kernels in a row: each is launched behind the one in front)
   fetch(t_begin);
 
   // start state: S2[i][c] = rows 2 (i % 2) + {0, 1} of the thread's row quad i / 2, column c0 + c
@@ -447,11 +448,11 @@ static int gla_fwd_launch(const Ctx& c, GlaArgs& a, void* ws, size_t ws_bytes) {
     return LAWCAT_ERR_CUDA;
   if (s.nseg > 1) {
     LaunchScope _ls("gla_fwd_rec_state", c.stream);
-    k_state<<<(unsigned)pieces, thr, smem1, c.stream>>>(a, s);
+    launch_behind(k_state, dim3((unsigned)pieces), dim3(thr), smem1, c.stream, a, s);
     LAWCAT_CHECK_LAUNCH();
   }
   LaunchScope _ls("gla_fwd_rec", c.stream);
-  k_full<<<(unsigned)(BH * s.nseg), thr, smem0, c.stream>>>(a, s);
+  launch_behind(k_full, dim3((unsigned)(BH * s.nseg)), dim3(thr), smem0, c.stream, a, s);
   LAWCAT_CHECK_LAUNCH();
   return LAWCAT_OK;
 }
