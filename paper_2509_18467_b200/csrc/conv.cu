@@ -466,6 +466,7 @@ __device__ __forceinline__ void bf16x4(const uint2& r, float* f) {
 __global__ void __launch_bounds__(128) conv_bwd4_kernel(const ConvBwd4 a) {
   // warp = one of four neighbouring spans of the same 128 channels (C is a multiple of 16: a lane may be past the end)
   __shared__ float s_dw[3][16][33];
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, qb = (a.C[0] / 4 + 31) / 32;
   const int st = (int)blockIdx.y >= qb;
   const int C = st ? a.C[1] : a.C[0], ch = 4 * (((int)blockIdx.y - (st ? qb : 0)) * 32 + lane), K = a.K, T = a.T;
@@ -557,10 +558,11 @@ __global__ void __launch_bounds__(128) conv_bwd4_kernel(const ConvBwd4 a) {
   }
 }
 
-// the conv's backward of both streams from fp32 du
+// the conv's backward of both streams from fp32 du (zeroed: an earlier kernel of the caller's has cleared dw_q and dw_k)
 template <typename TI>
 static int conv_bwd_both(const Ctx& c, const float* du_q, const float* du_k, const void* q, const void* k, const void* w_q,
-                         const void* w_k, const void* cache_q, const void* cache_k, void* dq, void* dk, float* dw_q, float* dw_k) {
+                         const void* w_k, const void* cache_q, const void* cache_k, void* dq, void* dk, float* dw_q, float* dw_k,
+                         bool zeroed) {
   const lawcat_params& p = *c.p;
   if (!std::is_same<TI, bf16>::value || p.conv_k > 4) {
     const int r = conv_bwd_stream<TI, float>(c, du_q, (const TI*)q, (const TI*)w_q, (const TI*)cache_q, (TI*)dq, dw_q, p.H);
@@ -568,13 +570,13 @@ static int conv_bwd_both(const Ctx& c, const float* du_q, const float* du_k, con
     return conv_bwd_stream<TI, float>(c, du_k, (const TI*)k, (const TI*)w_k, (const TI*)cache_k, (TI*)dk, dw_k, p.H_kv);
   }
   const int Cq = p.H * p.d_k, Ck = p.H_kv * p.d_k;
-  if (dw_q && cudaMemsetAsync(dw_q, 0, sizeof(float) * (size_t)Cq * p.conv_k, c.stream) != cudaSuccess) return LAWCAT_ERR_CUDA;
-  if (dw_k && cudaMemsetAsync(dw_k, 0, sizeof(float) * (size_t)Ck * p.conv_k, c.stream) != cudaSuccess) return LAWCAT_ERR_CUDA;
+  if (!zeroed && dw_q && cudaMemsetAsync(dw_q, 0, sizeof(float) * (size_t)Cq * p.conv_k, c.stream) != cudaSuccess) return LAWCAT_ERR_CUDA;
+  if (!zeroed && dw_k && cudaMemsetAsync(dw_k, 0, sizeof(float) * (size_t)Ck * p.conv_k, c.stream) != cudaSuccess) return LAWCAT_ERR_CUDA;
   const ConvBwd4 a{{du_q, du_k}, {(const bf16*)q, (const bf16*)k}, {(const bf16*)w_q, (const bf16*)w_k},
                    {(const bf16*)cache_q, (const bf16*)cache_k}, {(bf16*)dq, (bf16*)dk}, {dw_q, dw_k}, {Cq, Ck}, p.B, p.T, p.conv_k};
   const dim3 grid((p.B * ((p.T + CB4_SPAN - 1) / CB4_SPAN) + 3) / 4, (Cq / 4 + 31) / 32 + (Ck / 4 + 31) / 32);
   LaunchScope _ls("conv_bwd", c.stream);
-  conv_bwd4_kernel<<<grid, 128, 0, c.stream>>>(a);
+  launch_behind(conv_bwd4_kernel, grid, dim3(128), 0, c.stream, a);
   LAWCAT_CHECK_LAUNCH();
   return LAWCAT_OK;
 }
@@ -607,7 +609,7 @@ static int conv_bwd_typed(const Ctx& c, const void* q, const void* k, const void
     // tensor-core kernel for the mix and the softmax Jacobian; the conv's own backward follows on du as below
     int r0 = launch_convmix_tc_bwd(c, q, k, w_q, w_k, W, cache_q, cache_k, d_qdot, d_kdot, du_q, du_k, dW);
     if (r0) return r0;
-    return conv_bwd_both<TI>(c, du_q, du_k, q, k, w_q, w_k, cache_q, cache_k, dq, dk, dw_q, dw_k);
+    return conv_bwd_both<TI>(c, du_q, du_k, q, k, w_q, w_k, cache_q, cache_k, dq, dk, dw_q, dw_k, false);
   }
   dim3 grid(p.B * ((p.T + CB_SPAN - 1) / CB_SPAN), p.H_kv);
 #define LAUNCH_CB(D)                                                                                             \
@@ -628,7 +630,7 @@ static int conv_bwd_typed(const Ctx& c, const void* q, const void* k, const void
   }
 #undef LAUNCH_CB
   LAWCAT_CHECK_LAUNCH();
-  return conv_bwd_both<TI>(c, du_q, du_k, q, k, w_q, w_k, cache_q, cache_k, dq, dk, dw_q, dw_k);
+  return conv_bwd_both<TI>(c, du_q, du_k, q, k, w_q, w_k, cache_q, cache_k, dq, dk, dw_q, dw_k, false);
 }
 
 int launch_conv_bwd(const Ctx& c, const void* q, const void* k, const void* w_q, const void* w_k, const void* W,
@@ -639,10 +641,10 @@ int launch_conv_bwd(const Ctx& c, const void* q, const void* k, const void* w_q,
   return conv_bwd_typed<bf16>(c, q, k, w_q, w_k, W, cache_q, cache_k, d_qdot, d_kdot, dq, dk, dw_q, dw_k, dW, ws);
 }
 
-// the conv's own backward alone, on fp32 gradients of both conv outputs (bf16 storage)
+// the conv's own backward alone, on fp32 gradients of both conv outputs (bf16 storage); dw_q and dw_k are zero on entry
 int launch_conv_only_bwd(const Ctx& c, const void* q, const void* k, const void* w_q, const void* w_k, const void* cache_q,
                          const void* cache_k, const float* du_q, const float* du_k, void* dq, void* dk, float* dw_q, float* dw_k) {
-  return conv_bwd_both<bf16>(c, du_q, du_k, q, k, w_q, w_k, cache_q, cache_k, dq, dk, dw_q, dw_k);
+  return conv_bwd_both<bf16>(c, du_q, du_k, q, k, w_q, w_k, cache_q, cache_k, dq, dk, dw_q, dw_k, true);
 }
 
 // ------------------------------------------------------------------------------------------------ conv cache out

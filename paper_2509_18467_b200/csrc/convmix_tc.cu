@@ -127,6 +127,7 @@ __global__ void __launch_bounds__(fwd_threads<D, TO>()) convmix_tc_fwd_kernel(co
     tmem_alloc(sb + OFF_BAR + 16, D);
     tmem_relinquish();
   }
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   auto load_w = [&](const bf16* Wh) {
     if (NT == 1) {
       load_w_tile<D>(sg + OFF_WT, Wh, tid, NTH);
@@ -513,11 +514,11 @@ int launch_convmix_tc_fwd(const Ctx& c, const void* q, const void* k, const void
   const dim3 grid((unsigned)((p.T + TT - 1) / TT), (unsigned)(p.B * p.H));
   LaunchScope _ls("convmix_tc_fwd", c.stream);
   if (p.d_k == 64) {
-    if (out_f32) convmix_tc_fwd_kernel<64, float><<<grid, fwd_threads<64, float>(), fwd_smem<64, float>(), c.stream>>>(a);
-    else convmix_tc_fwd_kernel<64, bf16><<<grid, fwd_threads<64, bf16>(), fwd_smem<64, bf16>(), c.stream>>>(a);
+    if (out_f32) launch_behind(convmix_tc_fwd_kernel<64, float>, grid, dim3(fwd_threads<64, float>()), fwd_smem<64, float>(), c.stream, a);
+    else launch_behind(convmix_tc_fwd_kernel<64, bf16>, grid, dim3(fwd_threads<64, bf16>()), fwd_smem<64, bf16>(), c.stream, a);
   } else {
-    if (out_f32) convmix_tc_fwd_kernel<128, float><<<grid, fwd_threads<128, float>(), fwd_smem<128, float>(), c.stream>>>(a);
-    else convmix_tc_fwd_kernel<128, bf16><<<grid, fwd_threads<128, bf16>(), fwd_smem<128, bf16>(), c.stream>>>(a);
+    if (out_f32) launch_behind(convmix_tc_fwd_kernel<128, float>, grid, dim3(fwd_threads<128, float>()), fwd_smem<128, float>(), c.stream, a);
+    else launch_behind(convmix_tc_fwd_kernel<128, bf16>, grid, dim3(fwd_threads<128, bf16>()), fwd_smem<128, bf16>(), c.stream, a);
   }
   LAWCAT_CHECK_LAUNCH();
   return LAWCAT_OK;

@@ -56,7 +56,8 @@ struct Args {
   float* z16;                           // [B*H][chunks][D]
   int* meta;                            // [B*H][chunks][2]: kap, operand format
   uint8_t* s16;                         // [B*H][chunks][2 * D * D * 2] operand tiles, hi then lo
-  int* wmax;                            // [1] largest |wq|, |wk| of the call as float bits (caller-zeroed)
+  int* wmax;                            // [1] largest |wq|, |wk| of the call as float bits (zeroed by the sweep)
+  float* dW;                            // [H,D,D] weight gradient, accumulated by the mix backward: zeroed by the sweep
   int* dev_status;
   int B, T, H, Hkv, gate_dim, gate_mode, normalize;
   float inv_tau, eps;
@@ -263,6 +264,11 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) sweep_kerne
     tmem_alloc(smem_u32(const_cast<int*>(s_fl)), F::COLS);
     tmem_relinquish();
   }
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // (each kernel of the step is launched behind the one in front)
+  // zeroed here and not by memset nodes of their own, which cost microseconds each: dW (every block a part), the largest gradient
+  for (int i = blockIdx.x * F::THREADS + tid; i < a.H * D * D / 4; i += gridDim.x * F::THREADS)
+    reinterpret_cast<float4*>(a.dW)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (blockIdx.x == 0 && tid == 0) *a.wmax = 0;
   // the two extra slabs of [v | 1] (column D: the 1) and of the state operand (column D: z; the rest zero)
   for (int i = tid; i < 2 * C; i += F::THREADS)
     *reinterpret_cast<uint4*>(sg + F::F_V + toff(F::SL_T, i & (C - 1), D + 8 * (i >> 6))) = make_uint4(0u, 0u, 0u, 0u);
@@ -534,6 +540,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
     tmem_relinquish();
   }
   for (int i = tid; i < D; i += F::THREADS) s_pe[i] = s_r[i] = s_car[i] = 0.f;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
@@ -930,6 +937,7 @@ __global__ void __launch_bounds__(MCfg<D>::THREADS, D == 128 ? 1 : 2) mix_bwd_ke
     tmem_alloc(sb + M::BAR + 16, M::COLS);
     tmem_relinquish();
   }
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
@@ -1074,8 +1082,12 @@ __global__ void __launch_bounds__(MCfg<D>::THREADS, D == 128 ? 1 : 2) mix_bwd_ke
 }
 
 // dv[b,t,j,:] = sum over the query heads of group j of the per-head gradients; one thread per 8 channels
-__global__ void dv_sum_kernel(const float* __restrict__ dvh, bf16* __restrict__ dv, size_t total, int G, int oct) {
+// (and zeroes the tap gradients, n0 and n1 floats, for the conv backward that follows)
+__global__ void dv_sum_kernel(const float* __restrict__ dvh, bf16* __restrict__ dv, size_t total, int G, int oct, float* z0, int n0,
+                              float* z1, int n1) {
   const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  for (size_t i = idx; i < (size_t)n0 + n1; i += (size_t)gridDim.x * blockDim.x) (i < (size_t)n0 ? z0[i] : z1[i - n0]) = 0.f;
   if (idx >= total) return;
   const size_t btj = idx / oct;
   const int o8 = (int)(idx % oct);
@@ -1125,16 +1137,17 @@ static int run(const Ctx& c, const Args& a, const MArgs& m) {
   const lawcat_params& p = *c.p;
   {
     LaunchScope _ls("gla_tc_bwd_sweep", c.stream);
-    sweep_kernel<D><<<p.B * p.H, Cfg<D>::THREADS, Cfg<D>::F_BYTES, c.stream>>>(a);
+    launch_behind(sweep_kernel<D>, dim3(p.B * p.H), dim3(Cfg<D>::THREADS), Cfg<D>::F_BYTES, c.stream, a);
     LAWCAT_CHECK_LAUNCH();
   }
   {
     LaunchScope _ls("gla_tc_bwd", c.stream);
-    reverse_kernel<D><<<p.B * p.H, Cfg<D>::THREADS, Cfg<D>::R_BYTES, c.stream>>>(a);
+    launch_behind(reverse_kernel<D>, dim3(p.B * p.H), dim3(Cfg<D>::THREADS), Cfg<D>::R_BYTES, c.stream, a);
     LAWCAT_CHECK_LAUNCH();
   }
   LaunchScope _ls("convmix_tc_bwd", c.stream);
-  mix_bwd_kernel<D><<<dim3((unsigned)((p.T + TT - 1) / TT), (unsigned)(p.B * p.H_kv)), MCfg<D>::THREADS, MCfg<D>::BYTES, c.stream>>>(m);
+  launch_behind(mix_bwd_kernel<D>, dim3((unsigned)((p.T + TT - 1) / TT), (unsigned)(p.B * p.H_kv)), dim3(MCfg<D>::THREADS), MCfg<D>::BYTES,
+                c.stream, m);
   LAWCAT_CHECK_LAUNCH();
   return LAWCAT_OK;
 }
@@ -1165,21 +1178,19 @@ int launch_layer_bwd_tc(const Ctx& c, const void* q, const void* k, const void* 
   a.qd = (float*)(w + L.qd); a.kd = (float*)(w + L.kd); a.v = (const bf16*)v; a.gate = (const bf16*)gate; a.dO = (const bf16*)dO;
   a.S0 = S0; a.z0 = z0; a.wq = (float*)(w + L.wq); a.wk = (float*)(w + L.wk); a.dvh = (float*)(w + L.dvh); a.dgate = (bf16*)dgate;
   a.inv = (float*)(w + L.inv); a.delta = (float*)(w + L.delta); a.domax = (float*)(w + L.domax); a.z16 = (float*)(w + L.z16);
-  a.meta = (int*)(w + L.meta); a.s16 = (uint8_t*)(w + L.s16); a.wmax = (int*)(w + L.wmax); a.dev_status = c.dev_status;
+  a.meta = (int*)(w + L.meta); a.s16 = (uint8_t*)(w + L.s16); a.wmax = (int*)(w + L.wmax); a.dW = dW; a.dev_status = c.dev_status;
   a.B = p.B; a.T = p.T; a.H = p.H; a.Hkv = p.H_kv; a.gate_dim = p.gate_dim; a.gate_mode = p.gate_mode; a.normalize = p.normalize;
   a.inv_tau = 1.f / p.gate_tau; a.eps = p.eps;
   MArgs m{(const bf16*)q, (const bf16*)k, (const bf16*)w_q, (const bf16*)w_k, (const bf16*)W, (const bf16*)cache_q,
           (const bf16*)cache_k, a.qd, a.kd, a.wk, a.wq, (float*)(w + L.du_k), dW, a.wmax, c.dev_status, p.B, p.T, p.H, p.H_kv, p.conv_k};
-  if (cudaMemsetAsync(a.wmax, 0, 4, c.stream) != cudaSuccess ||
-      cudaMemsetAsync(dW, 0, sizeof(float) * (size_t)p.H * p.d_k * p.d_k, c.stream) != cudaSuccess)
-    return LAWCAT_ERR_CUDA;
   if ((r = launch_convmix_tc_fwd(c, q, k, w_q, w_k, W, cache_q, cache_k, (void*)a.qd, (void*)a.kd, true))) return r;
   if ((r = p.d_k == 64 ? run<64>(c, a, m) : run<128>(c, a, m))) return r;
   {
     const int oct = p.d_v / 8;
     const size_t total = (size_t)p.B * p.T * p.H_kv * oct;
     LaunchScope _ls("dv_reduce", c.stream);
-    dv_sum_kernel<<<(unsigned)((total + 255) / 256), 256, 0, c.stream>>>(a.dvh, (bf16*)dv, total, p.H / p.H_kv, oct);
+    launch_behind(dv_sum_kernel, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, c.stream, (const float*)a.dvh, (bf16*)dv, total,
+                  p.H / p.H_kv, oct, dw_q, dw_q ? p.H * p.d_k * p.conv_k : 0, dw_k, dw_k ? p.H_kv * p.d_k * p.conv_k : 0);
     LAWCAT_CHECK_LAUNCH();
   }
   return launch_conv_only_bwd(c, q, k, w_q, w_k, cache_q, cache_k, a.wq, m.du_k, dq, dk, dw_q, dw_k);
