@@ -596,6 +596,7 @@ __global__ void __launch_bounds__(DEC_THREADS) decode_one_kernel(const DecodeArg
   __shared__ __align__(16) float s_part[2][NCG][D + 4];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int bh = blockIdx.x, b = bh / a.H, h = bh % a.H, G = a.H / a.Hkv, j = h / G, K = a.K;
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // (launched behind the kernel in front on the stream)
   // ---- every global read
   const int oc = tid % OCT, cg = tid / OCT;
   uint4 w[RPT];
@@ -800,6 +801,7 @@ __global__ void __launch_bounds__(4 * D, D == 128 ? 1 : 3) decode_stream_kernel(
     mbar_fence_init();
     sm.abort_flag = 0;
   }
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // (launched behind the kernel in front on the stream)
   __syncthreads();
   if (tid >= L::NF) {
     // ============================================================================================== state
@@ -1027,21 +1029,12 @@ static int launch_decode_stream(const Ctx& c, const DecodeArgs& a) {
   }
   const int fit = sm_count() * (D == 128 ? 1 : 3) / p.H;  // blocks per head that run together
   const dim3 grid((unsigned)p.H, (unsigned)(fit < 1 ? 1 : fit < p.B ? fit : p.B));
-  LAWCAT_LAUNCH("decode_stream", c.stream, decode_stream_kernel<D><<<grid, 4 * D, DstLay<D>::SMEM, c.stream>>>(a));
+  LAWCAT_LAUNCH("decode_stream", c.stream, launch_behind(decode_stream_kernel<D>, grid, dim3(4 * D), DstLay<D>::SMEM, c.stream, a));
   LAWCAT_CHECK_LAUNCH();
   if (p.conv_k > 1) {
     const int C = p.H_kv * D, total = p.B * C / 8;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((total + 127) / 128));
-    cfg.blockDim = dim3(128);
-    cfg.stream = c.stream;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    LAWCAT_LAUNCH("key_cache_shift", c.stream,
-                  cudaLaunchKernelEx(&cfg, key_cache_shift_kernel, (bf16*)a.cache_k, (const bf16*)a.k_t, p.B, C, p.conv_k));
+    LAWCAT_LAUNCH("key_cache_shift", c.stream, launch_behind(key_cache_shift_kernel, dim3((unsigned)((total + 127) / 128)), dim3(128), 0,
+                                                             c.stream, (bf16*)a.cache_k, (const bf16*)a.k_t, p.B, C, p.conv_k));
     LAWCAT_CHECK_LAUNCH();
   }
   return LAWCAT_OK;
@@ -1068,12 +1061,14 @@ static int decode_typed(const Ctx& c, DecodeArgs& a) {
     cfg.gridDim = dim3((unsigned)(p.B * p.H));
     cfg.blockDim = dim3(DEC_THREADS);
     cfg.stream = c.stream;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)(p.H / p.H_kv);
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     LAWCAT_LAUNCH("decode_one", c.stream, cudaLaunchKernelEx(&cfg, p.d_k == 64 ? decode_one_kernel<64> : decode_one_kernel<128>, a));
     LAWCAT_CHECK_LAUNCH();
     return LAWCAT_OK;

@@ -140,6 +140,7 @@ gate_fn_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     tmem_alloc(smem_u32(const_cast<int*>(s_flags)), TMEM_COLS);
     tmem_relinquish();
   }
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // (launched behind the kernel in front on the stream)
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
@@ -381,6 +382,7 @@ __global__ void __launch_bounds__(256, 2) gate_fn_small_kernel(const bf16* __res
   const int cr = blockIdx.x % SMALL_CL, n0 = blockIdx.x / SMALL_CL * TOK;
   const int oct = dm >> 3, o0 = oct * cr / SMALL_CL, o1 = oct * (cr + 1) / SMALL_CL;
   const int jo = n_out >> 3, j0 = jo * cr / SMALL_CL * 8, j1 = jo * (cr + 1) / SMALL_CL * 8;
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // (launched behind the kernel in front on the stream)
   // the second layer's first rows: thread = two outputs
   constexpr int PRE = 4;  // octets of a row fetched ahead
   uint4 pre[2][PRE];
@@ -547,7 +549,7 @@ static int launch_tc(const Ctx& c, int d_model, const void* x, const void* A1, c
   if (!map_2d(&tx, x, N, d_model, tt) || !map_2d(&ta1, A1, R, d_model, R) || !map_2d(&to, gate, N, n_out, tt))
     return LAWCAT_ERR_CUDA;
   LAWCAT_LAUNCH("gate_fn_tc", c.stream,
-                gate_fn_tc_kernel<R><<<dim3((unsigned)tiles, (unsigned)ysplit), THREADS, L::BYTES, c.stream>>>(tx, ta1, to, a));
+                launch_behind(gate_fn_tc_kernel<R>, dim3((unsigned)tiles, (unsigned)ysplit), dim3(THREADS), L::BYTES, c.stream, tx, ta1, to, a));
   LAWCAT_CHECK_LAUNCH();
   return LAWCAT_OK;
 }
@@ -564,12 +566,14 @@ static int launch_small(const Ctx& c, int d_model, int rank, const void* x, cons
   cfg.blockDim = dim3(256);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = c.stream;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = SMALL_CL;
   at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   LAWCAT_LAUNCH("gate_fn_small", c.stream,
                 cudaLaunchKernelEx(&cfg, gate_fn_small_kernel<TOK>, (const bf16*)x, (const bf16*)A1, (const bf16*)A2,
                                    (const bf16*)bias, (bf16*)gate, (int)N, d_model, rank, n_out));

@@ -338,7 +338,7 @@ static int run_layer_tc(const Ctx& c, const void* q, const void* k, const void* 
   const int Hn = paired ? p.H / 2 : p.H;          // thread blocks per segment
   if (segs == nseq) {
     LaunchScope _ls("layer_tc", c.stream);
-    k_layer<<<Hn * segs, threads, SMEM_ALLOC, c.stream>>>(tq, tk, tv, tg, a, tab);
+    launch_behind(k_layer, dim3(Hn * segs), dim3(threads), SMEM_ALLOC, c.stream, tq, tk, tv, tg, a, tab);
     LAWCAT_CHECK_LAUNCH();
     return LAWCAT_OK;
   }
@@ -355,7 +355,7 @@ static int run_layer_tc(const Ctx& c, const void* q, const void* k, const void* 
     TcArgs b1 = a;
     b1.S_T = loc_S; b1.z_T = loc_z; b1.dtot = dtot; b1.nsub = nsub;
     LaunchScope _ls("layer_tc_state", c.stream);
-    k_state<<<Hn * (segs - nseq) * nsub, threads, SMEM_ALLOC, c.stream>>>(tq, tk, tv, tg, b1, tab);
+    launch_behind(k_state, dim3(Hn * (segs - nseq) * nsub), dim3(threads), SMEM_ALLOC, c.stream, tq, tk, tv, tg, b1, tab);
     LAWCAT_CHECK_LAUNCH();
   }
   cudaLaunchAttribute at[1];
@@ -376,10 +376,10 @@ static int run_layer_tc(const Ctx& c, const void* q, const void* k, const void* 
   }
   a.seg_S = start_S; a.seg_z = start_z;
   {
-    // (an ordinary launch: as a dependent of the scan its blocks land while scan blocks still hold registers of most SMs,
+    // (the scan gives no early start: with one, blocks land while scan blocks still hold registers of most SMs,
     // and the call at T = 32768 took 1.34 ms instead of 1.11)
     LaunchScope _ls("layer_tc", c.stream);
-    k_layer<<<Hn * segs, threads, SMEM_ALLOC, c.stream>>>(tq, tk, tv, tg, a, tab);
+    launch_behind(k_layer, dim3(Hn * segs), dim3(threads), SMEM_ALLOC, c.stream, tq, tk, tv, tg, a, tab);
   }
   LAWCAT_CHECK_LAUNCH();
   return LAWCAT_OK;

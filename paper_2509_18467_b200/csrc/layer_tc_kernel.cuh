@@ -383,6 +383,7 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
 
   // ---- one-time setup --------------------------------------------------------------------------------------------
   if (MODE == 1) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // (the scan may be scheduled behind)
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // (launched behind the kernel in front on the stream)
   // Three groups of warps prepare side by side, with all their loads in flight before the first is used: a block of a short
   // sequence spent a third of its time here, most of it in loads that waited for one another (given states 18k cycles, now
   // 2k; W 2k; the first tiles were asked for 3k cycles after the rest).
