@@ -255,9 +255,9 @@ int lawcat_layer_fwd_varlen(const lawcat_params* p, const int32_t* cu_seqlens, i
 /*
  * Backward of the whole layer (Fig. 1) for an upstream gradient dO [B,T,H,d_v]: the layer-wise distillation step of
  * Section 5.1 in one call (chain rule on conv -> mix -> phi -> Eq. 4, Eq. 8; the paper prints no formulas). The features
- * qdot, kdot are recomputed from q, k and never stored in the storage type: on the tensor-core path (bf16, d_k = d_v =
- * 64, softmax feature map, conv_k <= 4, gate_tau >= 8 in LOGITS mode, chunk != 1) they
- * and their gradients pass between the stages in fp32 scratch; every other shape runs the exact kernels as the chain
+ * qdot, kdot are recomputed from q, k and never stored in the storage type: on the tensor-core path (bf16, d_k = d_v
+ * in {64, 128}, softmax feature map, conv_k <= 4, gate_tau >= 8 in LOGITS mode, T >= 16, one shared mix, chunk in {0, 64})
+ * they and their gradients pass between the stages in fp32 scratch; every other shape runs the exact kernels as the chain
  * conv -> attention -> attention backward -> conv backward entirely in fp32 (bf16 tensors are widened into scratch
  * first and the four activation gradients narrowed at the end).
  *   in:  the inputs of lawcat_layer_fwd (caches and initial state nullable) and dO
@@ -278,7 +278,10 @@ int lawcat_layer_bwd(const lawcat_params* p, const void* q, const void* k, const
  *   the state advances by one token, the caches drop their oldest row and append q_t, k_t.
  *   out: o_t [B,H,d_v]
  *   ws: device scratch of lawcat_workspace_bytes(p, LAWCAT_OP_DECODE_STEP) bytes (the token's features, decays and
- *   denominators, handed from the first launch of the step to the second); LAWCAT_ERR_WORKSPACE_TOO_SMALL otherwise.
+ *   denominators where the step takes two launches); LAWCAT_ERR_WORKSPACE_TOO_SMALL otherwise.
+ * Kernels: bf16 storage with d_k = d_v in {64, 128}, conv_k <= 4, one shared mix and chunk != 1 is one pass over the state (plus a
+ * small launch that shifts the key caches when there are more heads than run at once); every other case takes two launches.
+ * dev_status receives LAWCAT_ERR_TIMEOUT when a bounded device-side wait ran out (the outputs are then undefined).
  */
 int lawcat_decode_step(const lawcat_params* p, const void* q_t, const void* k_t, const void* v_t,
                        const void* gate_t, const void* w_q, const void* w_k, const void* W, float* S, float* z,
