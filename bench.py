@@ -129,11 +129,11 @@ def kernel_bytes_per_step(name: str, kind: str, s: I.LayerShape) -> float:
         "gla_tc_fwd": f32_feat + b["v"] + b["gate"] + b["o"],
         "gla_tc_bwd_sweep": f32_feat + b["v"] + b["gate"] + b["o"],   # features, v, gate, dO in
         "dv_reduce": f32_dv + b["v"],
-        # raw q, k and the fp32 feature gradients in, fp32 du out (dW is negligible)
-        "convmix_tc_bwd": b["q"] + b["k"] + f32_feat + 4 * (s.H + s.H_kv) * s.d_k,
+        # raw q, k, the fp32 features and their products with the gradients in, fp32 du out (dW is negligible)
+        "convmix_tc_bwd": b["q"] + b["k"] + 2 * f32_feat + 4 * (s.H + s.H_kv) * s.d_k,
         "conv_bwd": 4 * (s.H + s.H_kv) * s.d_k + 2 * (b["q"] + b["k"]),
     }
-    if name in ("decode_state", "decode_features"):
+    if name in ("decode_one", "decode_stream", "decode_state", "decode_features"):
         return alg_bytes_per_step("decode", s)
     if name in table:
         return table[name] * tok
