@@ -259,9 +259,9 @@ int lawcat_layer_fwd(const lawcat_params* p, const void* q, const void* k, const
   }
   // exact path: conv + mix + phi into fp32 scratch, then the recurrent GLA
   if ((r = launch_convmix_fwd(c, q, k, w_q, w_k, W, cache_q_in, cache_k_in, qdot, kdot, true, p->chunk == 1))) return r;
-  if ((r = launch_gla_fwd_rec(c, qdot, kdot, true, v, gate, S0, z0, o, nullptr, S_T, z_T,
-                              (char*)ws + 2 * nf, ws_bytes - 2 * nf))) return r;
-  return launch_cache_out(c, q, k, cache_q_in, cache_k_in, cache_q_out, cache_k_out);
+  const CacheOut caches{q, k, cache_q_in, cache_k_in, cache_q_out, cache_k_out};
+  return launch_gla_fwd_rec(c, qdot, kdot, true, v, gate, S0, z0, o, nullptr, S_T, z_T, (char*)ws + 2 * nf, ws_bytes - 2 * nf,
+                            &caches);
 }
 
 size_t lawcat_layer_fwd_varlen_workspace_bytes(const lawcat_params* p, const int32_t* cu_seqlens, int nseq) {

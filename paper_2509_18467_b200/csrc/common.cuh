@@ -58,9 +58,14 @@ int launch_conv_bwd(const Ctx& c, const void* q, const void* k, const void* w_q,
                     void* dk, float* dw_q, float* dw_k, float* dW, void* ws);
 int launch_cache_out(const Ctx& c, const void* q, const void* k, const void* cache_q_in, const void* cache_k_in,
                      void* cache_q_out, void* cache_k_out);
+// the conv caches after the last token, for a kernel that writes them on the side (see launch_cache_out)
+struct CacheOut {
+  const void *q, *k, *cin_q, *cin_k;
+  void *cout_q, *cout_k;
+};
 int launch_gla_fwd_rec(const Ctx& c, const void* qdot, const void* kdot, bool qk_f32, const void* v,
                        const void* gate, const float* S0, const float* z0, void* o, float* den, float* S_T,
-                       float* z_T, void* ws, size_t ws_bytes);
+                       float* z_T, void* ws, size_t ws_bytes, const CacheOut* caches = nullptr);
 size_t gla_fwd_rec_workspace_bytes(const lawcat_params& p);  // (without it the call runs one block per head)
 int launch_gla_bwd_rec(const Ctx& c, const void* qdot, const void* kdot, const void* v, const void* gate,
                        const float* S0, const float* z0, const void* o, const float* den, const void* dO,

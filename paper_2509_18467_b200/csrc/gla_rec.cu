@@ -60,6 +60,8 @@ constexpr __host__ __device__ int fwd_groups(int dk) { return dk >= 64 ? 8 : dk 
 struct SegArgs {
   int nseg, seg_len;            // segments per sequence, tokens per segment (a multiple of TBF)
   float *loc_S, *loc_z, *dec;   // pieces: [B,H,nseg-1,dk,dv], [B,H,nseg-1,dk], total decay [B,H,nseg-1,dk]
+  CacheOut caches;              // (MODE 0) the layer's conv caches, written by the first segments; null: none
+  int conv_k;
 };
 
 // decays of N tokens: sigmoid(a)^(1/tau), or exp(a). (tau = 1: e / (1 + e) by one exponential and one reciprocal; else only
@@ -170,6 +172,23 @@ __global__ void __launch_bounds__(256, 2) gla_fwd_rec_kernel(const GlaArgs a, co
   };
   asm volatile("griddepcontrol.wait;" ::: "memory");  // (three short kernels in a row: each is launched behind the one in front)
   fetch(t_begin);
+  if (MODE == 0 && seg == 0 && (sgm.caches.cout_q || sgm.caches.cout_k)) {
+    // the last conv_k - 1 raw rows of [cache, x] (Section 4.1), by the blocks that have no pieces to fold: a launch of its own
+    // costs a short call 1.6 us (fp32, 512 tokens, 4 heads of 64: 45.5 -> 43.9)
+    const int K1 = sgm.conv_k - 1;
+    for (int i = tid; i < 2 * K1 * dk; i += nthr) {
+      const int st = i / (K1 * dk), r = i / dk % K1, ch = i % dk, tok = a.T - K1 + r;
+      const int NH = st ? a.Hkv : H, n = st ? j : h;
+      TS* dst = (TS*)(st ? sgm.caches.cout_k : sgm.caches.cout_q);
+      if (!dst || (st && h % (H / a.Hkv) != 0)) continue;
+      const TS *x = (const TS*)(st ? sgm.caches.k : sgm.caches.q), *cin = (const TS*)(st ? sgm.caches.cin_k : sgm.caches.cin_q);
+      TS val;
+      if (tok >= 0) val = x[(((size_t)b * a.T + tok) * NH + n) * dk + ch];
+      else if (cin) val = cin[(((size_t)b * K1 + tok + K1) * NH + n) * dk + ch];
+      else stf(&val, 0.f);
+      dst[(((size_t)b * K1 + r) * NH + n) * dk + ch] = val;
+    }
+  }
 
   // start state: S2[i][c] = rows 2 (i % 2) + {0, 1} of the thread's row quad i / 2, column c0 + c
   uint64_t S2[R / 2][4];
@@ -422,7 +441,7 @@ size_t gla_fwd_rec_workspace_bytes(const lawcat_params& p) {
 }
 
 template <typename TQ, typename TS>
-static int gla_fwd_launch(const Ctx& c, GlaArgs& a, void* ws, size_t ws_bytes) {
+static int gla_fwd_launch(const Ctx& c, GlaArgs& a, void* ws, size_t ws_bytes, const CacheOut* caches) {
   const lawcat_params& p = *c.p;
   if (p.B * p.H == 0) return LAWCAT_OK;
   SegArgs s = fwd_plan(p);
@@ -430,6 +449,8 @@ static int gla_fwd_launch(const Ctx& c, GlaArgs& a, void* ws, size_t ws_bytes) {
     s.nseg = 1;
     s.seg_len = (p.T + TBF - 1) / TBF * TBF;
   }
+  if (caches && p.conv_k > 1) s.caches = *caches;
+  s.conv_k = p.conv_k;
   const int BH = p.B * p.H, thr = fwd_threads(p);
   const size_t pieces = (size_t)BH * (s.nseg - 1);
   s.loc_S = (float*)ws;
@@ -459,7 +480,7 @@ static int gla_fwd_launch(const Ctx& c, GlaArgs& a, void* ws, size_t ws_bytes) {
 
 int launch_gla_fwd_rec(const Ctx& c, const void* qdot, const void* kdot, bool qk_f32, const void* v,
                        const void* gate, const float* S0, const float* z0, void* o, float* den, float* S_T,
-                       float* z_T, void* ws, size_t ws_bytes) {
+                       float* z_T, void* ws, size_t ws_bytes, const CacheOut* caches) {
   const lawcat_params& p = *c.p;
   GlaArgs a = base_args(p);
   a.qdot = qdot; a.kdot = kdot; a.v = v; a.gate = gate; a.S0 = S0; a.z0 = z0;
@@ -470,11 +491,11 @@ int launch_gla_fwd_rec(const Ctx& c, const void* qdot, const void* kdot, bool qk
       return LAWCAT_ERR_CUDA;
     if (z_T && (z0 ? cudaMemcpyAsync(z_T, z0, nz, cudaMemcpyDeviceToDevice, c.stream) : cudaMemsetAsync(z_T, 0, nz, c.stream)))
       return LAWCAT_ERR_CUDA;
-    return LAWCAT_OK;
+    return caches ? launch_cache_out(c, caches->q, caches->k, caches->cin_q, caches->cin_k, caches->cout_q, caches->cout_k) : LAWCAT_OK;
   }
-  if (p.dtype == LAWCAT_F32) return gla_fwd_launch<float, float>(c, a, ws, ws_bytes);
-  if (qk_f32) return gla_fwd_launch<float, bf16>(c, a, ws, ws_bytes);
-  return gla_fwd_launch<bf16, bf16>(c, a, ws, ws_bytes);
+  if (p.dtype == LAWCAT_F32) return gla_fwd_launch<float, float>(c, a, ws, ws_bytes, caches);
+  if (qk_f32) return gla_fwd_launch<float, bf16>(c, a, ws, ws_bytes, caches);
+  return gla_fwd_launch<bf16, bf16>(c, a, ws, ws_bytes, caches);
 }
 
 // ------------------------------------------------------------------------------------------------ backward sweeps
