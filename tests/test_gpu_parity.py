@@ -339,3 +339,16 @@ def test_decode_many_heads(api, B, H, Hkv, d, K):
     if K > 1:
         assert np.array_equal(cq.float().cpu().numpy(), ref["cache_q"].astype(np.float32))
         assert np.array_equal(ck.float().cpu().numpy(), ref["cache_k"].astype(np.float32))
+
+
+@pytest.mark.parametrize("d,K", [(16, 4), (32, 2), (64, 4), (64, 1), (128, 3), (64, 5)])
+@pytest.mark.parametrize("T", [1, 2, 8, 33, 64])
+def test_exact_conv_tiles(api, d, K, T):
+    """The exact conv + mix around its tile of 32 tokens: runs of channels with the window in registers (d = 64, 128, conv width up
+    to 4) and the general loop, with caches in front."""
+    s = shape(2, T, 4, 2, d, d, "f32", conv_k=K, cid=48)
+    x = I.make(s, ["q", "k", "w_q", "w_k", "W"] + (["cache_q", "cache_k"] if K > 1 else []))
+    t = dev(api, x, s)
+    qd, kd = api.lawcat_conv_fwd(P(api, s), t["q"], t["k"], t["w_q"], t["w_k"], t["W"], t.get("cache_q"), t.get("cache_k"))
+    check(qd, O.mix_phi(O.conv(x["q"], x["w_q"], x.get("cache_q"), K), x["W"], s.H, 0), "f32", "qdot")
+    check(kd, O.mix_phi(O.conv(x["k"], x["w_k"], x.get("cache_k"), K), x["W"], s.H, 0), "f32", "kdot")
