@@ -1,6 +1,6 @@
 // Recurrent single-token decode (streaming inference, Section 6): the layer at one token with the conv cache of
-// Section 4.1 and the constant-size state of Eq. 4. bf16, d_k = d_v = 64 or 128, conv width up to 4: many heads go to
-// decode_stream_kernel, few to decode_one_kernel where it applies (1, 2, 4 or 8 query heads per key/value head). Else two
+// Section 4.1 and the constant-size state of Eq. 4. bf16, d_k = d_v = 64 or 128, conv width up to 4: few heads go to
+// decode_one_kernel where it applies (1, 2, 4 or 8 query heads per key/value head), the rest to decode_stream_kernel. Else two
 // launches:
 //   decode_features  conv -> shared linear layer -> feature map for the token's query and key, decay alpha = exp(g), the
 //                    normalizer state z (Eq. 8's denominator) advanced in place; writes qdot, kdot, alpha and the
@@ -1005,11 +1005,19 @@ __global__ void key_cache_shift_kernel(bf16* __restrict__ cache, const bf16* __r
     if (r < K - 1) row0[(size_t)r * per] = x[r];
 }
 
+// (clusters of 1, 2, 4 or 8 blocks; square states)
+static bool decode_one_supported(const lawcat_params& p) {
+  const int G = p.H / p.H_kv;
+  return decode_tc_supported(p) && p.d_v == p.d_k && G <= 8 && (G & (G - 1)) == 0;
+}
+
 // More heads than decode_one blocks run at once (2 per SM for d = 128, 4 for d = 64): up to there its single round is the
-// shorter chain (B = 8, d = 128: 7.3 us against 9.0; B = 16, d = 64: 6.0 against 6.7). Every query head needs a block at once.
+// shorter chain (B = 8, d = 128: 7.3 us against 9.0; B = 16, d = 64: 6.0 against 6.7). Groups that decode_one does not take come
+// here whatever their number (24 heads in groups of 3: 11.6 us as two launches, 6.2 here, d = 128, B = 1). Every query head needs a block at once.
 static bool decode_stream_supported(const lawcat_params& p) {
   const int sms = sm_count();
-  return decode_tc_supported(p) && p.d_v == p.d_k && p.H <= sms && (int64_t)p.B * p.H > (int64_t)sms * (p.d_k == 128 ? 2 : 4);
+  if (!decode_tc_supported(p) || p.d_v != p.d_k || p.H > sms) return false;
+  return !decode_one_supported(p) || (int64_t)p.B * p.H > (int64_t)sms * (p.d_k == 128 ? 2 : 4);
 }
 
 template <int D>
@@ -1038,12 +1046,6 @@ static int launch_decode_stream(const Ctx& c, const DecodeArgs& a) {
     LAWCAT_CHECK_LAUNCH();
   }
   return LAWCAT_OK;
-}
-
-// (clusters of 1, 2, 4 or 8 blocks; square states)
-static bool decode_one_supported(const lawcat_params& p) {
-  const int G = p.H / p.H_kv;
-  return decode_tc_supported(p) && p.d_v == p.d_k && G <= 8 && (G & (G - 1)) == 0;
 }
 
 size_t decode_workspace_bytes(const lawcat_params& p) {
