@@ -837,6 +837,13 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
 #pragma unroll
           for (int cp = 0; cp < 4; ++cp) { x3[cp] = x2[cp]; x2[cp] = x1[cp]; x1[cp] = x0[cp]; }
         }
+        // Rows past the end of the sequence: zeros. In a pack they hold the next sequence's tokens, and a factor of zero further
+        // on would not keep out what is not finite there.
+        if (MODE == 0 && nvalid < C) {
+#pragma unroll 1
+          for (int i = 0; i < 8; ++i)
+            if (cv_rg * 8 + i >= nvalid) sts128(au + sw128(crow0 + i, cjc), make_uint4(0u, 0u, 0u, 0u));
+        }
         if (cv_rg == 7) {  // the last three raw rows of the chunk are the next chunk's halo (bf16 values: exact repack)
           uint4* hl = reinterpret_cast<uint4*>(sg + OFF_HALO) + cv_stream * 48 + cv_oct;
           hl[0] = pack8p(x3, false); hl[16] = pack8p(x2, false); hl[32] = pack8p(x1, false);
@@ -948,6 +955,11 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
 #pragma unroll
           for (int e = 0; e < 8; ++e) vm = fmaxf(vm, fabsf(x[e]));
           sts128(ad, pack8(x, true));
+        }
+        if (MODE == 0 && nvalid < C) {  // (rows past the end, as in the conv)
+#pragma unroll 1
+          for (int u = vt; u < vslab * 512; u += vthreads)
+            if (((u >> 3) & (C - 1)) >= nvalid) sts128(sb + OFF_V + (uint32_t)u * 16, make_uint4(0u, 0u, 0u, 0u));
         }
         vm = warp_max(vm);
         if (lane == 0) atomicMax(&s_vmax[p], __float_as_int(vm < 3.0e38f ? vm : 3.0e38f));

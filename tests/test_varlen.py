@@ -83,6 +83,32 @@ def test_many_sequences_share_the_launches(d, gate_dim):
         assert np.array_equal(r["cache_k"][i:i + 1].float().cpu().numpy(), ref["cache_k"].astype(np.float32))
 
 
+@pytest.mark.gpu
+@pytest.mark.parametrize("d,H,H_kv,gate_dim", [(128, 4, 2, 0), (64, 4, 2, 0), (64, 2, 2, 0), (128, 2, 1, 1)])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf"), 1.0e5, 3.0e38])
+def test_a_sequence_does_not_reach_its_neighbours(d, H, H_kv, gate_dim, bad):
+    """Every token of one sequence of the pack is not finite, or beyond the range of fp16: the sequences in front of it (whose
+    last chunk it shares) and behind it keep their outputs and states bit for bit."""
+    import torch
+    from paper_2509_18467_b200 import api
+    lens = [100, 80, 65, 17, 700, 90, 130]
+    cu = np.concatenate([[0], np.cumsum(lens)]).tolist()
+    s = I.LayerShape(1, cu[-1], H, H_kv, d, d, gate_dim=gate_dim, dtype="bf16", config_id=97)
+    t = {n: api.to_device(v, "bf16") for n, v in I.make(s, NAMES).items()}
+    p = api.params(1, s.T, H, H_kv, d, d, gate_dim=gate_dim)
+    ref = api.lawcat_layer_fwd_varlen(p, cu, *[t[n] for n in NAMES])
+    poisoned = (1, 3, 5)
+    for i in poisoned:
+        for n in ("q", "k", "v") + (("gate",) if bad != bad else ()):
+            t[n][:, cu[i]:cu[i + 1]] = bad
+    r = api.lawcat_layer_fwd_varlen(p, cu, *[t[n] for n in NAMES])
+    torch.cuda.synchronize()
+    for i in set(range(len(lens))) - set(poisoned):
+        assert torch.equal(r["o"][:, cu[i]:cu[i + 1]], ref["o"][:, cu[i]:cu[i + 1]]), f"o of sequence {i}"
+        for n in ("S_T", "z_T"):
+            assert bool(torch.isfinite(ref[n][i]).all()) and torch.equal(r[n][i], ref[n][i]), f"{n} of sequence {i}"
+
+
 def test_bad_offsets_are_refused_on_the_host():
     import ctypes
     from paper_2509_18467_b200 import api
