@@ -926,7 +926,7 @@ __global__ void __launch_bounds__(MCfg<D>::THREADS, D == 128 ? 1 : 2) mix_bwd_ke
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   volatile int* const s_fl = reinterpret_cast<volatile int*>(sg + M::BAR + 16);  // tmem base, abort
   float* const s_taps = reinterpret_cast<float*>(sg + M::TAPS);
-  const int t0 = blockIdx.x * TT, bj = blockIdx.y, j = bj % a.Hkv, b = bj / a.Hkv, G = a.H / a.Hkv;
+  const int tiles = (a.T + TT - 1) / TT, t0 = blockIdx.x % tiles * TT, bj = blockIdx.x / tiles, j = bj % a.Hkv, b = bj / a.Hkv, G = a.H / a.Hkv;
   const int nvalid = min(TT, a.T - t0);
   if (tid == 0) {
     mbar_init(sb + M::BAR, 1);
@@ -1146,7 +1146,8 @@ static int run(const Ctx& c, const Args& a, const MArgs& m) {
     LAWCAT_CHECK_LAUNCH();
   }
   LaunchScope _ls("convmix_tc_bwd", c.stream);
-  launch_behind(mix_bwd_kernel<D>, dim3((unsigned)((p.T + TT - 1) / TT), (unsigned)(p.B * p.H_kv)), dim3(MCfg<D>::THREADS), MCfg<D>::BYTES,
+  // (all blocks along x: the other axes end at 65535)
+  launch_behind(mix_bwd_kernel<D>, dim3((unsigned)((p.T + TT - 1) / TT) * (unsigned)(p.B * p.H_kv)), dim3(MCfg<D>::THREADS), MCfg<D>::BYTES,
                 c.stream, m);
   LAWCAT_CHECK_LAUNCH();
   return LAWCAT_OK;
