@@ -204,7 +204,7 @@ def lawcat_gate_fn_fwd(p: Params, d_model: int, rank: int, x, A1, A2, bias=None,
     b = _binding or _bind()
     need = 0 if ws is not None else lib().lawcat_gate_fn_workspace_bytes(ctypes.byref(p), d_model, rank)
     st = b.call(_addr["lawcat_gate_fn_fwd"], ctypes.addressof(p), need, -1,
-                (int(d_model), int(rank), x, A1, A2, bias, gate), ws, stream and stream.cuda_stream, dev_status)
+                (int(d_model), int(rank), x, A1, A2, bias, gate), ws, stream and stream.cuda_stream, dev_status, 2)
     if st != 0:
         raise LawcatError(st, "lawcat_gate_fn_fwd")
     return gate
@@ -268,7 +268,7 @@ def lawcat_layer_fwd_varlen(p: Params, cu_seqlens, q, k, v, gate, w_q, w_k, W, c
     need = lib().lawcat_layer_fwd_varlen_workspace_bytes(ctypes.byref(p), cu, nseq)
     st = b.call(_addr["lawcat_layer_fwd_varlen"], ctypes.addressof(p), max(need, 16), -1,
                 (ctypes.addressof(cu), nseq, q, k, v, gate, w_q, w_k, W, cache_q, cache_k, S0, z0, o, cq, ck, S_T, z_T), None,
-                stream and stream.cuda_stream, dev_status)
+                stream and stream.cuda_stream, dev_status, 2)
     if st != 0:
         raise LawcatError(st, "lawcat_layer_fwd_varlen")
     return dict(o=o, cache_q=cq, cache_k=ck, S_T=S_T, z_T=z_T)

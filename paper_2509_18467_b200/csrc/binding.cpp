@@ -11,17 +11,12 @@ namespace {
 
 constexpr int MAX_PTRS = 20;
 
-// None and empty tensors are NULL, an integer is passed as it is (a size, or the address of a host array); anything else must
-// be a contiguous CUDA tensor. False with a Python error set otherwise.
+// None and empty tensors are NULL, anything else must be a contiguous CUDA tensor. False with a Python error set otherwise.
 bool argument(PyObject* o, void** out) {
   *out = nullptr;
   if (o == Py_None) return true;
-  if (PyLong_Check(o)) {
-    *out = PyLong_AsVoidPtr(o);
-    return !PyErr_Occurred();
-  }
   if (!THPVariable_Check(o)) {
-    PyErr_SetString(PyExc_TypeError, "expected a tensor, an integer or None");
+    PyErr_SetString(PyExc_TypeError, "expected a tensor or None");
     return false;
   }
   const at::Tensor& t = THPVariable_Unpack(o);
@@ -40,28 +35,34 @@ int call_n(void* fn, const void* p, void* const* a, void* ws, size_t nb, void* s
   return reinterpret_cast<F>(fn)(p, a[I]..., ws, nb, st, ds);
 }
 
-// call(fn, params, ws_fn, op, tensors, ws, stream, dev_status) -> status
-//   fn: address of an entry point fn(params, tensors..., ws, ws_bytes, stream, dev_status)
+// call(fn, params, ws_fn, op, args, ws, stream, dev_status, nint = 0) -> status
+//   fn: address of an entry point fn(params, args..., ws, ws_bytes, stream, dev_status)
+//   args: tensors or None, behind `nint` integers that are passed as they are (sizes, the address of a host array)
 //   ws_fn(params, op): its scratch bytes; op = -1: ws_fn is that number itself
 //   ws: scratch tensor, or None to take it from torch's allocator for the duration of the call
-//   stream: cudaStream_t as an integer, or None for the current stream of the first tensor's device
+//   stream: cudaStream_t as an integer, or None for the current stream of the current device
 PyObject* call(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
-  if (nargs != 8 || !PyTuple_Check(args[4])) {
-    PyErr_SetString(PyExc_TypeError, "call(fn, params, ws_fn, op, tensors, ws, stream, dev_status)");
+  if (nargs < 8 || nargs > 9 || !PyTuple_Check(args[4])) {
+    PyErr_SetString(PyExc_TypeError, "call(fn, params, ws_fn, op, args, ws, stream, dev_status, nint = 0)");
     return nullptr;
   }
   void* fn = PyLong_AsVoidPtr(args[0]);
   const void* p = PyLong_AsVoidPtr(args[1]);
   const size_t ws_arg = PyLong_AsSize_t(args[2]);
   const int op = (int)PyLong_AsLong(args[3]);
+  const Py_ssize_t nint = nargs > 8 ? PyLong_AsSsize_t(args[8]) : 0;
   if (PyErr_Occurred()) return nullptr;
   const Py_ssize_t n = PyTuple_GET_SIZE(args[4]);
-  if (n < 1 || n > MAX_PTRS) {
-    PyErr_SetString(PyExc_TypeError, "number of tensors");
+  if (n < 1 || n > MAX_PTRS || nint < 0 || nint > n) {
+    PyErr_SetString(PyExc_TypeError, "number of arguments");
     return nullptr;
   }
   void* a[MAX_PTRS];
-  for (Py_ssize_t i = 0; i < n; ++i)
+  for (Py_ssize_t i = 0; i < nint; ++i) {
+    a[i] = PyLong_AsVoidPtr(PyTuple_GET_ITEM(args[4], i));
+    if (PyErr_Occurred()) return nullptr;
+  }
+  for (Py_ssize_t i = nint; i < n; ++i)
     if (!argument(PyTuple_GET_ITEM(args[4], i), &a[i])) return nullptr;
   void *ws = nullptr, *ds = nullptr, *st = nullptr;
   if (!argument(args[5], &ws) || !argument(args[7], &ds)) return nullptr;
@@ -74,7 +75,7 @@ PyObject* call(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
       nb = op < 0 ? ws_arg : reinterpret_cast<size_t (*)(const void*, int)>(ws_arg)(p, op);
       if (nb) {
         c10::Device dev(c10::kCUDA);
-        for (Py_ssize_t i = 0; i < n; ++i)
+        for (Py_ssize_t i = nint; i < n; ++i)
           if (THPVariable_Check(PyTuple_GET_ITEM(args[4], i))) {
             dev = THPVariable_Unpack(PyTuple_GET_ITEM(args[4], i)).device();
             break;

@@ -1,0 +1,47 @@
+"""The native module that turns tensors into the pointers of a C entry point: what is not a tensor is a Python error. No GPU:
+nothing here is launched."""
+import ctypes
+
+import pytest
+
+from paper_2509_18467_b200 import api, build
+
+
+@pytest.fixture(scope="module")
+def binding():
+    build.build()
+    return api._bind()
+
+
+ARGS = [None] * 12   # of a decode step, all NULL: refused by the library before anything is launched
+
+
+def call(b, args=ARGS, ws=None, dev_status=None, nint=None):
+    p = api.params(1, 1, 4, 2, 64, 64)
+    extra = () if nint is None else (nint,)
+    return b.call(api._addr["lawcat_decode_step"], ctypes.addressof(p), 0, -1, tuple(args), ws, None, dev_status, *extra)
+
+
+def test_null_tensors_reach_the_library(binding):
+    assert call(binding) == 1   # LAWCAT_ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("bad", [16, 0, True, 1.5, "ws", [0]])
+@pytest.mark.parametrize("where", ["ws", "dev_status", "first", "last"])
+def test_what_is_not_a_tensor_is_a_python_error(binding, bad, where):
+    args = list(ARGS)
+    kw = {}
+    if where in ("ws", "dev_status"):
+        kw[where] = bad
+    else:
+        args[0 if where == "first" else -1] = bad
+    with pytest.raises(TypeError):
+        call(binding, args, **kw)
+
+
+@pytest.mark.parametrize("nint", [-1, 13, "2"])
+def test_number_of_leading_integers(binding, nint):
+    with pytest.raises(TypeError):
+        call(binding, nint=nint)
+    with pytest.raises(TypeError):
+        call(binding, [None] * 12, nint=1)   # (an integer is expected in front)
