@@ -41,6 +41,8 @@ int call_n(void* fn, const void* p, void* const* a, void* ws, size_t nb, void* s
 //   ws_fn(params, op): its scratch bytes; op = -1: ws_fn is that number itself
 //   ws: scratch tensor, or None to take it from torch's allocator for the duration of the call
 //   stream: cudaStream_t as an integer, or None for the current stream of the current device
+// The library's call runs without the interpreter lock: it stands while the device's launch queue is full or a kernel's module
+// is loaded, and other Python threads go on meanwhile.
 PyObject* call(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
   if (nargs < 8 || nargs > 9 || !PyTuple_Check(args[4])) {
     PyErr_SetString(PyExc_TypeError, "call(fn, params, ws_fn, op, args, ws, stream, dev_status, nint = 0)");
@@ -92,11 +94,13 @@ PyObject* call(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
   }
   if (PyErr_Occurred()) return nullptr;
   int r = 0;
+  Py_BEGIN_ALLOW_THREADS
   switch (n) {
 #define N(k) case k: r = call_n(fn, p, a, ws, nb, st, ds, std::make_index_sequence<k>{}); break;
     N(1) N(2) N(3) N(4) N(5) N(6) N(7) N(8) N(9) N(10) N(11) N(12) N(13) N(14) N(15) N(16) N(17) N(18) N(19) N(20)
 #undef N
   }
+  Py_END_ALLOW_THREADS
   return PyLong_FromLong(r);
 }
 

@@ -1,6 +1,8 @@
-"""The native module that turns tensors into the pointers of a C entry point: what is not a tensor is a Python error. No GPU:
-nothing here is launched."""
+"""The native module that turns tensors into the pointers of a C entry point: what is not a tensor is a Python error, and other
+Python threads run while the library does. No GPU: nothing here is launched."""
 import ctypes
+import threading
+import time
 
 import pytest
 
@@ -45,3 +47,27 @@ def test_number_of_leading_integers(binding, nint):
         call(binding, nint=nint)
     with pytest.raises(TypeError):
         call(binding, [None] * 12, nint=1)   # (an integer is expected in front)
+
+
+def test_other_threads_run_during_a_call(binding):
+    """usleep stands in for an entry point that waits for room in the launch queue (it reads its first argument only)."""
+    usleep = ctypes.cast(ctypes.CDLL(None).usleep, ctypes.c_void_p).value
+    stamps, stop = [], threading.Event()
+
+    def tick():
+        while not stop.is_set():
+            stamps.append(time.perf_counter())
+            time.sleep(0.005)
+
+    t = threading.Thread(target=tick)
+    t.start()
+    try:
+        time.sleep(0.05)
+        t0 = time.perf_counter()
+        assert binding.call(usleep, 500_000, 0, -1, (None,), None, None, None) == 0
+        t1 = time.perf_counter()
+    finally:
+        stop.set()
+        t.join()
+    assert t1 - t0 >= 0.5
+    assert sum(t0 + 0.02 < s < t1 - 0.02 for s in stamps) >= 10
