@@ -17,8 +17,8 @@
 // Dividing by den is folded into qn and into the row terms, so dO and v enter every product unrounded (both are exact in 16
 // bits); qn, ks, S16, R16, P' and E are two-term 16-bit pairs hi + lo (hi hi + lo hi + hi lo: about 21 bits). Powers of two keep
 // the pairs in the fp16 range and away from its subnormals: 2^kap on ks and S16 (per chunk, from a bound on the state), 2^al on
-// inv (per chunk, from its largest inv and the largest adjoint entry), 2^sc on dO (per head). Chunks whose decay exponents leave
-// +-8 use bf16 pairs.
+// inv (per chunk, from its largest inv and the largest adjoint entry), 2^sc on dO (per head, from its largest |dO| and a bound on
+// E). Chunks whose decay exponents leave +-8, or whose v is beyond the fp16 range, use bf16 pairs.
 //
 // One thread block walks one (batch, query head), lock-step: every phase of a chunk by all threads, products by one thread
 // (tcgen05.mma, fp32 accumulators in tensor memory), bounded waits on mbarriers. What bounds it is that chain of phases:
@@ -40,7 +40,7 @@ using namespace tc;
 using namespace ctc;
 
 constexpr int C = 64, MID = 31;
-constexpr float RMAX_F16 = 8.f;
+constexpr float RMAX_F16 = 8.f, VMAX_F16 = 65504.f;
 constexpr int QSC = 4;       // power of two on qs in the forward sweep
 constexpr int KAP_MAX = 4;   // largest power of two on ks and S16 (ks <= 2^8 in fp16 chunks)
 
@@ -52,7 +52,7 @@ struct Args {
   float* dvh;                           // [B,T,H,D] per-head dv, reduced over the heads of a group afterwards
   bf16* dgate;
   float *inv, *delta;                   // [B,T,H]
-  float* domax;                         // [B*H] largest |dO| of the head
+  float2* domax;                        // [B*H] of the head: largest |dO|, and a bound on |dO . v_i - delta|
   float* z16;                           // [B*H][chunks][D]
   int* meta;                            // [B*H][chunks][2]: kap, operand format
   uint8_t* s16;                         // [B*H][chunks][2 * D * D * 2] operand tiles, hi then lo
@@ -251,14 +251,14 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) sweep_kerne
   float* const s_bm = reinterpret_cast<float*>(sg + F::F_VEC);
   float *const s_ft = s_bm + D, *const s_pe = s_ft + D;  // s_pe: ft of the chunk in front (its state is still 2^-ft short)
   float* const s_row = s_pe + 2 * D;                     // [NCG][C]
-  volatile int* const s_fl = reinterpret_cast<volatile int*>(s_row + F::NCG * C);  // tmem base, abort, rmax, smax, vmax, domax
+  volatile int* const s_fl = reinterpret_cast<volatile int*>(s_row + F::NCG * C);  // tmem base, abort, rmax, smax, vmax, domax, dlmax
   const uint32_t bar = smem_u32(const_cast<int*>(s_fl)) + 32;
   const int bh = blockIdx.x, h = bh % a.H, b = bh / a.H, G = a.H / a.Hkv, j = h / G;
   const int nch = (a.T + C - 1) / C;
   if (tid == 0) {
     mbar_init(bar, 1);
     mbar_fence_init();
-    for (int i = 1; i < 6; ++i) s_fl[i] = 0;
+    for (int i = 1; i < 7; ++i) s_fl[i] = 0;
   }
   if (warp == 0) {
     tmem_alloc(smem_u32(const_cast<int*>(s_fl)), F::COLS);
@@ -314,7 +314,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) sweep_kerne
   smx = warp_max(smx);
   if (lane == 0) atomicMax(const_cast<int*>(&s_fl[3]), __float_as_int(smx));
   __syncthreads();
-  float sbound = __int_as_float(s_fl[3]), domax = 0.f;
+  float sbound = __int_as_float(s_fl[3]), domax = 0.f, dlmax = 0.f, vhead = 0.f;  // (largest |dO|, |delta|, |v| so far)
   int kap_prev = 0;
   Gates<D> gates;
   gates.load(a, b, h, 0, tid);
@@ -327,43 +327,49 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) sweep_kerne
     Rows<D, false> rows;
     rows.load(a, row0, h, j, nvalid, tid);
     gate_pass<D>(a, gates, nvalid, s_x, s_bm, s_ft, const_cast<int*>(&s_fl[2]), tid);
-    const bool f16 = __int_as_float(s_fl[2]) <= RMAX_F16;
-    const int fmt = f16 ? FMT_F16 : FMT_BF16;
+    bool f16 = __int_as_float(s_fl[2]) <= RMAX_F16;
     const int kap = max(-100, min(KAP_MAX, 14 - exp_above(fmaxf(sbound, 1e-30f))));
     const float ksc = pow2i(kap);
-    // ---- operands
-    float vmax = 0.f;
+    // ---- operands (once more in bf16 when v turns out to be beyond the fp16 range: the largest |v| is known behind them)
+#pragma unroll 1
+    for (;;) {
+      float vmax = 0.f;
 #pragma unroll
-    for (int it = 0; it < 2; ++it) {
-      const int idx = tid + it * F::THREADS, o = idx % F::OCT, r = idx / F::OCT;
-      float q[8], k[8], vv[8], x[8];
-      rows.f8(rows.q[it], q);
-      rows.f8(rows.k[it], k);
-      unpack8b(rows.v[it], vv);
-      load_row8(s_x + r * D + o * 8, x);
+      for (int it = 0; it < 2; ++it) {
+        const int idx = tid + it * F::THREADS, o = idx % F::OCT, r = idx / F::OCT;
+        float q[8], k[8], vv[8], x[8];
+        rows.f8(rows.q[it], q);
+        rows.f8(rows.k[it], k);
+        unpack8b(rows.v[it], vv);
+        load_row8(s_x + r * D + o * 8, x);
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        q[i] *= ex2f(x[i]) * (float)(1 << QSC);
-        k[i] *= ex2f(-x[i]) * ksc;
-        vmax = fmaxf(vmax, fabsf(vv[i]));
+        for (int i = 0; i < 8; ++i) {
+          q[i] *= ex2f(x[i]) * (float)(1 << QSC);
+          k[i] *= ex2f(-x[i]) * ksc;
+          vmax = fmaxf(vmax, fabsf(vv[i]));
+        }
+        uint4 hi, lo;
+        const uint32_t at = toff(F::SL_T, r, o * 8);
+        split8h(q, f16, hi, lo);
+        *reinterpret_cast<uint4*>(sg + F::F_QS + at) = hi;
+        *reinterpret_cast<uint4*>(sg + F::F_QS + F::T_TOK + at) = lo;
+        split8h(k, f16, hi, lo);
+        *reinterpret_cast<uint4*>(sg + F::F_KS + at) = hi;
+        *reinterpret_cast<uint4*>(sg + F::F_KS + F::T_TOK + at) = lo;
+        *reinterpret_cast<uint4*>(sg + F::F_V + at) = pack8h(vv, f16);
+        if (o == 0) {
+          const float one[8] = {1.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+          *reinterpret_cast<uint4*>(sg + F::F_V + toff(F::SL_T, r, D)) = pack8h(one, f16);
+        }
       }
-      uint4 hi, lo;
-      const uint32_t at = toff(F::SL_T, r, o * 8);
-      split8h(q, f16, hi, lo);
-      *reinterpret_cast<uint4*>(sg + F::F_QS + at) = hi;
-      *reinterpret_cast<uint4*>(sg + F::F_QS + F::T_TOK + at) = lo;
-      split8h(k, f16, hi, lo);
-      *reinterpret_cast<uint4*>(sg + F::F_KS + at) = hi;
-      *reinterpret_cast<uint4*>(sg + F::F_KS + F::T_TOK + at) = lo;
-      *reinterpret_cast<uint4*>(sg + F::F_V + at) = pack8h(vv, f16);
-      if (o == 0) {
-        const float one[8] = {1.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        *reinterpret_cast<uint4*>(sg + F::F_V + toff(F::SL_T, r, D)) = pack8h(one, f16);
-      }
+      vmax = warp_max(vmax);
+      if (lane == 0) atomicMax(const_cast<int*>(&s_fl[4]), __float_as_int(vmax < 1.0e30f ? vmax : 1.0e30f));
+      __syncthreads();  // (the exponents have been read: the state operand may overwrite them)
+      if (!f16 || __int_as_float(s_fl[4]) <= VMAX_F16) break;
+      f16 = false;
+      rows.load(a, row0, h, j, nvalid, tid);
     }
-    vmax = warp_max(vmax);
-    if (lane == 0) atomicMax(const_cast<int*>(&s_fl[4]), __float_as_int(vmax < 1.0e30f ? vmax : 1.0e30f));
-    __syncthreads();  // (the exponents have been read: the state operand may overwrite them)
+    const int fmt = f16 ? FMT_F16 : FMT_BF16;
     // ---- state pass: W = 2^(bm + ft of the chunk in front) S, kept in tensor memory and as the two-term operand, scaled 2^kap
     smx = 0.f;
     if (st_thr) {
@@ -491,17 +497,22 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) sweep_kerne
       const size_t th = (row0 + row) * a.H + h;
       a.inv[th] = inv;
       a.delta[th] = a.normalize ? d : 0.f;
+      if (a.normalize) dlmax = fmaxf(dlmax, fabsf(d));
     }
     sbound = sm + 64.f * fmaxf(vm, 1.f);
+    vhead = fmaxf(vhead, vm);
     kap_prev = kap;
     __syncthreads();
   }
   domax = warp_max(domax);
   if (lane == 0) atomicMax(const_cast<int*>(&s_fl[5]), __float_as_int(domax < 1.0e30f ? domax : 1.0e30f));
+  dlmax = warp_max(dlmax);
+  if (lane == 0) atomicMax(const_cast<int*>(&s_fl[6]), __float_as_int(dlmax < 1.0e30f ? dlmax : 1.0e30f));
   tc_fence_before_sync();
   __syncthreads();
   if (tid == 0) {
-    a.domax[bh] = __int_as_float(s_fl[5]);
+    domax = __int_as_float(s_fl[5]);
+    a.domax[bh] = make_float2(domax, (float)D * domax * vhead + __int_as_float(s_fl[6]));
     tma_store_wait_all();
   }
   if (warp == 0) {
@@ -564,8 +575,10 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
     for (int c0 = cg * SW; c0 < (cg + 1) * SW; c0 += 8) tmem_st8(lane_base + F::R_R + c0, s);
     tmem_wait_st();
   }
-  // 2^sc: the largest |dO| of the head becomes 2^4 .. 2^5 (every gradient is linear in dO)
-  const int sc = 5 - exp_above(fmaxf(a.domax[bh], 1e-30f));
+  // 2^sc: the largest |dO| of the head becomes 2^4 .. 2^5 (every gradient is linear in dO), or less where |v| is so large (from
+  // about 16 on for d = 128) that an entry of E could leave the fp16 range otherwise
+  const float2 dmx = a.domax[bh];
+  const int sc = min(5 - exp_above(fmaxf(dmx.x, 1e-30f)), 16 - exp_above(fmaxf(1.001f * dmx.y, 1e-30f)));
   const float osc = pow2i(sc);
   int al_prev = 0;
   float wmax = 0.f;
@@ -701,7 +714,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
           for (int i = 0; i < 8; ++i) {
             const bool on = c0 + i8 + i <= row;
             s[i8 + i] = on ? s[i8 + i] : 0.f;
-            e[i8 + i] = on ? fminf(fmaxf(e[i8 + i] - dl, -65000.f), 65000.f) : 0.f;
+            e[i8 + i] = on ? e[i8 + i] - dl : 0.f;
           }
           const uint32_t at = toff(F::SL_U, row, c0 + i8);
           split8h(s + i8, f16, hi, lo);
@@ -1111,7 +1124,7 @@ static Plan plan(const lawcat_params& p) {
   const size_t bth = (size_t)p.B * p.T * p.H, nf = 4 * bth * p.d_k, ch = (size_t)p.B * p.H * ((p.T + C - 1) / C);
   L.qd = take(nf); L.kd = take(nf); L.wq = take(nf); L.wk = take(nf); L.dvh = take(nf);
   L.du_k = take(nf / (p.H / p.H_kv));
-  L.inv = take(4 * bth); L.delta = take(4 * bth); L.domax = take(4 * (size_t)p.B * p.H);
+  L.inv = take(4 * bth); L.delta = take(4 * bth); L.domax = take(8 * (size_t)p.B * p.H);
   L.z16 = take(4 * ch * p.d_k); L.meta = take(8 * ch); L.s16 = take(ch * 4 * p.d_k * p.d_k); L.wmax = take(4);
   L.total = off;
   return L;
@@ -1178,7 +1191,7 @@ int launch_layer_bwd_tc(const Ctx& c, const void* q, const void* k, const void* 
   Args a{};
   a.qd = (float*)(w + L.qd); a.kd = (float*)(w + L.kd); a.v = (const bf16*)v; a.gate = (const bf16*)gate; a.dO = (const bf16*)dO;
   a.S0 = S0; a.z0 = z0; a.wq = (float*)(w + L.wq); a.wk = (float*)(w + L.wk); a.dvh = (float*)(w + L.dvh); a.dgate = (bf16*)dgate;
-  a.inv = (float*)(w + L.inv); a.delta = (float*)(w + L.delta); a.domax = (float*)(w + L.domax); a.z16 = (float*)(w + L.z16);
+  a.inv = (float*)(w + L.inv); a.delta = (float*)(w + L.delta); a.domax = (float2*)(w + L.domax); a.z16 = (float*)(w + L.z16);
   a.meta = (int*)(w + L.meta); a.s16 = (uint8_t*)(w + L.s16); a.wmax = (int*)(w + L.wmax); a.dW = dW; a.dev_status = c.dev_status;
   a.B = p.B; a.T = p.T; a.H = p.H; a.Hkv = p.H_kv; a.gate_dim = p.gate_dim; a.gate_mode = p.gate_mode; a.normalize = p.normalize;
   a.inv_tau = 1.f / p.gate_tau; a.eps = p.eps;

@@ -116,3 +116,25 @@ def test_gradient_scale(api, d, scale):
         check(g[n], ref[n], "bf16", n)
     for n in ("dw_q", "dw_k", "dW"):
         check(g[n], ref[n], "bf16", n, f32_store=True)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("scale", [1e3, 1e5])
+@pytest.mark.parametrize("with_state", [False, True])
+def test_large_values(api, d, scale, with_state):
+    """|v| in the thousands (dO . v and its difference from dO . o leave the fp16 range unless dO is scaled for it), and beyond
+    the fp16 range itself, ordinary and large chunks in one head."""
+    import torch
+    s = I.LayerShape(1, 200, 4, 2, d, d, dtype="bf16", config_id=89)
+    x = I.make(s, NAMES + ["dO"] + (["S0", "z0"] if with_state else []))
+    x["v"][:, 70:] = I.round_to_bf16(x["v"][:, 70:] * np.float32(scale))
+    t = {n: api.to_device(v, "f32" if n in ("S0", "z0") else s.dtype) for n, v in x.items()}
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    g = api.lawcat_layer_bwd(P(api, s), *[t[n] for n in NAMES], t["dO"], None, None, t.get("S0"), t.get("z0"), dev_status=status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    ref = oracle_layer_gradients(s, x)
+    for n in ("dq", "dk", "dv", "dgate"):
+        check(g[n], ref[n], "bf16", n)
+    for n in ("dw_q", "dw_k", "dW"):
+        check(g[n], ref[n], "bf16", n, f32_store=True)
