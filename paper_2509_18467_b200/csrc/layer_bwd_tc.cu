@@ -56,7 +56,7 @@ struct Args {
   float* z16;                           // [B*H][chunks][D]
   int* meta;                            // [B*H][chunks][2]: kap, operand format
   uint8_t* s16;                         // [B*H][chunks][2 * D * D * 2] operand tiles, hi then lo
-  int* wmax;                            // [1] largest |wq|, |wk| of the call as float bits (zeroed by the sweep)
+  float* wmax;                          // [B*H] largest |wq|, |wk| of the head
   float* dW;                            // [H,D,D] weight gradient, accumulated by the mix backward: zeroed by the sweep
   int* dev_status;
   int B, T, H, Hkv, gate_dim, gate_mode, normalize;
@@ -265,10 +265,9 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) sweep_kerne
     tmem_relinquish();
   }
   asm volatile("griddepcontrol.wait;" ::: "memory");  // (each kernel of the step is launched behind the one in front)
-  // zeroed here and not by memset nodes of their own, which cost microseconds each: dW (every block a part), the largest gradient
+  // dW is zeroed here (every block a part) and not by a memset node of its own, which costs microseconds
   for (int i = blockIdx.x * F::THREADS + tid; i < a.H * D * D / 4; i += gridDim.x * F::THREADS)
     reinterpret_cast<float4*>(a.dW)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (blockIdx.x == 0 && tid == 0) *a.wmax = 0;
   // the two extra slabs of [v | 1] (column D: the 1) and of the state operand (column D: z; the rest zero)
   for (int i = tid; i < 2 * C; i += F::THREADS)
     *reinterpret_cast<uint4*>(sg + F::F_V + toff(F::SL_T, i & (C - 1), D + 8 * (i >> 6))) = make_uint4(0u, 0u, 0u, 0u);
@@ -896,9 +895,10 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
     __syncthreads();
   }
   wmax = warp_max(wmax);
-  if (lane == 0) atomicMax(a.wmax, __float_as_int(wmax < 1.0e30f ? wmax : 1.0e30f));
+  if (lane == 0) atomicMax(const_cast<int*>(&s_fl[5]), __float_as_int(wmax < 1.0e30f ? wmax : 1.0e30f));
   tc_fence_before_sync();
   __syncthreads();
+  if (tid == 0) a.wmax[bh] = __int_as_float(s_fl[5]);
   if (warp == 0) {
     tc_fence_after_sync();
     tmem_dealloc(mm.tmem, F::COLS);
@@ -909,14 +909,14 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
 // From w = p * dp of both streams (p the features) back through the softmax and the shared linear layer:
 //   dy = w - p sum(w),   du = dy W_h^T (query stream; key stream summed over the heads of the group),   dW_h += u^T dy
 // One block = one (batch, key head, tile of 128 tokens), walking the group's heads and both streams. dy (scaled by a power of
-// two from the largest |w| of the call) and u, the recomputed conv output, are two-term fp16 pairs; the key stream's du is
-// accumulated over the heads in tensor memory. du of the query stream overwrites wq in place.
+// two from the largest |w| of the head) and u, the recomputed conv output, are two-term fp16 pairs; the key stream's du is
+// summed over the heads in registers, each head on its own scale. du of the query stream overwrites wq in place.
 struct MArgs {
   const bf16 *q, *k, *w_q, *w_k, *W, *cache_q, *cache_k;
   const float *qd, *kd, *wk;
   float *wq;                 // in: wq; out: du of the query stream
   float *du_k, *dW;          // [B,T,Hkv,D]; [H,D,D] (atomic adds into zeros)
-  const int* wmax;
+  const float* wmax;
   int* dev_status;
   int B, T, H, Hkv, K;
 };
@@ -959,22 +959,17 @@ __global__ void __launch_bounds__(MCfg<D>::THREADS, D == 128 ? 1 : 2) mix_bwd_ke
   const int row = (warp & 3) * 32 + lane, cg = warp >> 2;
   constexpr int HC = D / M::NCG, NTH = M::THREADS;
   Waiter wt{sb + M::BAR, 0u, s_fl + 1, a.dev_status};
-  // 2^sg: the largest |w| becomes 2^7 .. 2^8, which leaves |dy| <= |w| + sum |w| below the fp16 maximum for every row
-  const int sgm = 8 - exp_above(fmaxf(__int_as_float(*a.wmax), 1e-30f));
-  const float sc = pow2i(sgm), isc = pow2i(-sgm);
+  float sc = 1.f, isc = 1.f;  // power of two on the head's dy
+  float duk[HC];              // du of the key stream, this thread's row and columns
+#pragma unroll
+  for (int i = 0; i < HC; ++i) duk[i] = 0.f;
   const int o = tid % L::OPR, rr0 = tid / L::OPR;
   constexpr int RSTEP = NTH / L::OPR, RPT = TT / RSTEP;
-  // fp32 [128][D] accumulator to global rows through the (dead) dy tiles
-  auto rows_out = [&](uint32_t col, float* dst, int NH, int head) {
-    float d[8];
-#pragma unroll 1
-    for (int c0 = cg * HC; c0 < (cg + 1) * HC; c0 += 8) {
-      tmem_ld8(lane_base + col + c0, d);
-      tmem_wait_ld();
+  // this thread's row and columns of du to global rows through the (dead) dy tiles
+  auto rows_out = [&](const float (&d)[HC], float* dst, int NH, int head) {
 #pragma unroll
-      for (int i = 0; i < 8; i += 4)
-        *reinterpret_cast<float4*>(sg + M::DY + foff<D>(row, (c0 + i) >> 2)) = make_float4(d[i] * isc, d[i + 1] * isc, d[i + 2] * isc, d[i + 3] * isc);
-    }
+    for (int i = 0; i < HC; i += 4)
+      *reinterpret_cast<float4*>(sg + M::DY + foff<D>(row, (cg * HC + i) >> 2)) = make_float4(d[i], d[i + 1], d[i + 2], d[i + 3]);
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
@@ -988,6 +983,10 @@ __global__ void __launch_bounds__(MCfg<D>::THREADS, D == 128 ? 1 : 2) mix_bwd_ke
 #pragma unroll 1
   for (int g = 0; g < G; ++g) {
     const int h = j * G + g;
+    // the head's largest |w| becomes 2^7 .. 2^8, which leaves |dy| <= |w| + sum |w| below the fp16 maximum for every row
+    const int sgm = 8 - exp_above(fmaxf(a.wmax[b * a.H + h], 1e-30f));
+    sc = pow2i(sgm);
+    isc = pow2i(-sgm);
     load_w_tile<D>(sg + M::WT, a.W + (size_t)h * D * D, tid, NTH);
 #pragma unroll 1
     for (int stream = 0; stream < 2; ++stream) {
@@ -1057,14 +1056,24 @@ __global__ void __launch_bounds__(MCfg<D>::THREADS, D == 128 ? 1 : 2) mix_bwd_ke
       tc_fence_after_sync();
       if (tid == 0) {
         mm.split(stream ? M::DUK : M::DUQ, kview(sb + M::DY, L::SLAB_U), kview(sb + M::DY + L::TILE_U, L::SLAB_U), 2 * L::SLAB_U,
-                 kview(sb + M::WT, L::SLAB_W), 0, 2 * L::SLAB_W, D / 16, instr_desc(128, D, FMT_F16, MAJOR_K, MAJOR_K),
-                 stream == 1 && g > 0);
+                 kview(sb + M::WT, L::SLAB_W), 0, 2 * L::SLAB_W, D / 16, instr_desc(128, D, FMT_F16, MAJOR_K, MAJOR_K), false);
         mm.split(M::DWC, mview(sb + M::U, L::SLAB_U), mview(sb + M::U + L::TILE_U, L::SLAB_U), 256, mview(sb + M::DY, L::SLAB_U),
                  mview(sb + M::DY + L::TILE_U, L::SLAB_U), 256, TT / 16, instr_desc(128, D, FMT_F16, MAJOR_MN, MAJOR_MN), stream == 1);
         mma_commit(sb + M::BAR);
       }
       wt.wait();
-      if (stream == 0) rows_out(M::DUQ, a.wq, a.H, h);
+      static_assert(HC == 32, "one wide load");
+      float du[HC];
+      tmem_ld32(lane_base + (stream ? M::DUK : M::DUQ) + cg * HC, du);
+      tmem_wait_ld();
+      if (stream == 0) {
+#pragma unroll
+        for (int i = 0; i < HC; ++i) du[i] *= isc;
+        rows_out(du, a.wq, a.H, h);
+      } else {
+#pragma unroll
+        for (int i = 0; i < HC; ++i) duk[i] = fmaf(du[i], isc, duk[i]);
+      }
     }
     // dW of the head: row c of the accumulator belongs to lane c
     if (a.dW && row < D) {
@@ -1085,7 +1094,7 @@ __global__ void __launch_bounds__(MCfg<D>::THREADS, D == 128 ? 1 : 2) mix_bwd_ke
     __syncthreads();
     tc_fence_after_sync();
   }
-  rows_out(M::DUK, a.du_k, a.Hkv, j);
+  rows_out(duk, a.du_k, a.Hkv, j);
   tc_fence_before_sync();
   __syncthreads();
   if (warp == 0) {
@@ -1125,7 +1134,7 @@ static Plan plan(const lawcat_params& p) {
   L.qd = take(nf); L.kd = take(nf); L.wq = take(nf); L.wk = take(nf); L.dvh = take(nf);
   L.du_k = take(nf / (p.H / p.H_kv));
   L.inv = take(4 * bth); L.delta = take(4 * bth); L.domax = take(8 * (size_t)p.B * p.H);
-  L.z16 = take(4 * ch * p.d_k); L.meta = take(8 * ch); L.s16 = take(ch * 4 * p.d_k * p.d_k); L.wmax = take(4);
+  L.z16 = take(4 * ch * p.d_k); L.meta = take(8 * ch); L.s16 = take(ch * 4 * p.d_k * p.d_k); L.wmax = take(4 * (size_t)p.B * p.H);
   L.total = off;
   return L;
 }
@@ -1192,7 +1201,7 @@ int launch_layer_bwd_tc(const Ctx& c, const void* q, const void* k, const void* 
   a.qd = (float*)(w + L.qd); a.kd = (float*)(w + L.kd); a.v = (const bf16*)v; a.gate = (const bf16*)gate; a.dO = (const bf16*)dO;
   a.S0 = S0; a.z0 = z0; a.wq = (float*)(w + L.wq); a.wk = (float*)(w + L.wk); a.dvh = (float*)(w + L.dvh); a.dgate = (bf16*)dgate;
   a.inv = (float*)(w + L.inv); a.delta = (float*)(w + L.delta); a.domax = (float2*)(w + L.domax); a.z16 = (float*)(w + L.z16);
-  a.meta = (int*)(w + L.meta); a.s16 = (uint8_t*)(w + L.s16); a.wmax = (int*)(w + L.wmax); a.dW = dW; a.dev_status = c.dev_status;
+  a.meta = (int*)(w + L.meta); a.s16 = (uint8_t*)(w + L.s16); a.wmax = (float*)(w + L.wmax); a.dW = dW; a.dev_status = c.dev_status;
   a.B = p.B; a.T = p.T; a.H = p.H; a.Hkv = p.H_kv; a.gate_dim = p.gate_dim; a.gate_mode = p.gate_mode; a.normalize = p.normalize;
   a.inv_tau = 1.f / p.gate_tau; a.eps = p.eps;
   MArgs m{(const bf16*)q, (const bf16*)k, (const bf16*)w_q, (const bf16*)w_k, (const bf16*)W, (const bf16*)cache_q,

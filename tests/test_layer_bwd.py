@@ -138,3 +138,27 @@ def test_large_values(api, d, scale, with_state):
         check(g[n], ref[n], "bf16", n)
     for n in ("dw_q", "dw_k", "dW"):
         check(g[n], ref[n], "bf16", n, f32_store=True)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_heads_of_very_different_gradients(api, d):
+    """Heads whose upstream gradients lie up to 2^30 apart, inside a group of heads and across groups: each keeps its accuracy."""
+    import torch
+    s = I.LayerShape(2, 150, 6, 2, d, d, dtype="bf16", config_id=98)
+    x = I.make(s, NAMES + ["dO"])
+    x["dO"] = x["dO"] * np.float32([1.0, 2.0**-26, 2.0**-13, 2.0**-30, 2.0**-28, 2.0**-26])[:, None]
+    x["dO"][1] *= np.float32(2.0**-24)   # and the second sequence far below the first
+    t = {n: api.to_device(v, s.dtype) for n, v in x.items()}
+    g = api.lawcat_layer_bwd(P(api, s), *[t[n] for n in NAMES], t["dO"])
+    torch.cuda.synchronize()
+    ref = oracle_layer_gradients(s, x)
+    for b in range(2):
+        for h in range(6):
+            for n in ("dq", "dgate"):
+                check(g[n][b, :, h], ref[n][b, :, h], "bf16", f"{n} of sequence {b}, head {h}")
+        for j in range(2):
+            for n in ("dk", "dv"):
+                check(g[n][b, :, j], ref[n][b, :, j], "bf16", f"{n} of sequence {b}, head {j}")
+    for h in range(6):
+        check(g["dW"][h], ref["dW"][h], "bf16", f"dW of head {h}", f32_store=True)
+        check(g["dw_q"].view(6, -1)[h], ref["dw_q"].reshape(6, -1)[h], "bf16", f"dw_q of head {h}", f32_store=True)
