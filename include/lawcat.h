@@ -113,10 +113,10 @@ int lawcat_trace_begin(void);
 int lawcat_trace_end(char* buf, size_t buf_bytes);
 
 /*
- * Test hook (no counterpart in the paper). Every device-side wait of the tensor-core layer kernels is bounded: after
- * `cycles` clock cycles (default about two seconds) a waiting role gives up, the block leaves its loops, lets its
- * copies land, frees its tensor memory and returns, and dev_status receives LAWCAT_ERR_TIMEOUT. This call sets the bound
- * for the launches that follow (0 restores the default), so that a test can make a wait run out without faulting or
+ * Test hook (no counterpart in the paper). Every device-side wait of the library is bounded. In the kernels whose roles hand
+ * tiles to one another (the chunkwise layer forward, the streaming decode step) a waiting role gives up after `cycles` clock
+ * cycles (default about two seconds), the block leaves its loops, lets its copies land, frees its tensor memory and returns,
+ * and dev_status receives LAWCAT_ERR_TIMEOUT. This call sets their bound for the launches that follow (0 restores the default), so that a test can make a wait run out without faulting or
  * hanging anything. Host-side, process-wide, not meant for production code.
  */
 void lawcat_test_set_wait_limit(long long cycles);

@@ -124,7 +124,7 @@ def trace_end() -> dict:
 
 
 def test_set_wait_limit(cycles: int) -> None:
-    """Test hook: bound (clock cycles) of the device-side waits of the tensor-core layer kernels; 0 = default."""
+    """Test hook: bound (clock cycles) of the device-side waits of the layer forward and streaming decode kernels; 0 = default."""
     f = lib().lawcat_test_set_wait_limit
     f.argtypes, f.restype = [ctypes.c_longlong], None
     f(cycles)

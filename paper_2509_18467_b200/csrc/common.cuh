@@ -77,6 +77,7 @@ size_t decode_workspace_bytes(const lawcat_params& p);
 
 // Host-side check of a parameter block (api.cu): LAWCAT_OK, LAWCAT_ERR_INVALID_ARG or LAWCAT_ERR_UNSUPPORTED.
 int sm_count();  // of the current device (layer_tc.cu)
+long long wait_limit();  // bound of the device-side waits in clock cycles (layer_tc.cu; a test hook may shorten it)
 int validate_params(const lawcat_params* p, bool need_T);
 
 // Chunkwise tensor-core layer forward (layer_tc.cu): whether it takes these parameters, and its launcher.

@@ -31,6 +31,7 @@ struct DecodeArgs {
   int unshared;  // 1: W is [2,H,dk,dk], the key stream's vectors mix with the second set
   float inv_tau, eps;
   int* dev_status;
+  long long wait_limit;  // clock cycles a device-side wait of the streaming kernel may take
 };
 
 constexpr int DEC_THREADS = 256;
@@ -781,11 +782,13 @@ __global__ void __launch_bounds__(4 * D, D == 128 ? 1 : 3) decode_stream_kernel(
   // bounded; once a wait has run out every later one returns at once, so the block runs to its end (with numbers nobody will use)
   auto wait = [&](uint64_t& b, uint32_t parity) {
     const uint32_t bar = smem_u32(&b);
-    if (*s_abort || mbar_try_wait(bar, parity)) return;
+    // (under a limit shorter than a try_wait may take, as a test sets it, the phase is only looked at)
+    auto done = [&]() -> bool { return a.wait_limit < 1000000LL ? mbar_test_wait(bar, parity) : mbar_try_wait(bar, parity); };
+    if (*s_abort || done()) return;
     const long long t0 = clock64();
-    while (!mbar_try_wait(bar, parity)) {
+    while (!done()) {
       if (*s_abort) return;
-      if (clock64() - t0 > 2000000000LL) {
+      if (clock64() - t0 > a.wait_limit) {
         *s_abort = 1;
         if (a.dev_status) atomicMax(a.dev_status, (int)LAWCAT_ERR_TIMEOUT);
         return;
@@ -1124,6 +1127,7 @@ int launch_decode(const Ctx& c, const void* q_t, const void* k_t, const void* v_
   a.B = p.B; a.H = p.H; a.Hkv = p.H_kv; a.dk = p.d_k; a.dv = p.d_v; a.K = p.conv_k; a.gd = p.gate_dim;
   a.phi = p.phi; a.gate_mode = p.gate_mode; a.normalize = p.normalize;
   a.inv_tau = 1.f / p.gate_tau; a.eps = p.eps; a.dev_status = c.dev_status; a.unshared = p.mix_unshared;
+  a.wait_limit = wait_limit();
   if (p.dtype == LAWCAT_F32) return decode_typed<float>(c, a);
   return decode_typed<bf16>(c, a);
 }

@@ -182,6 +182,7 @@ static TcPlan layer_tc_plan(const lawcat_params& p) {
 
 // Limit of the kernels' device-side waits in clock cycles (about two seconds); a test hook may shorten it.
 static std::atomic<long long> g_wait_limit{4000000000LL};
+long long wait_limit() { return g_wait_limit.load(); }
 
 // scratch of a launch with `segs` segments in all (none when every sequence is one segment)
 static size_t layer_tc_scratch(const lawcat_params& p, size_t segs, int nsub) {
@@ -308,7 +309,7 @@ static int run_layer_tc(const Ctx& c, const void* q, const void* k, const void* 
   a.dev_status = c.dev_status;
   a.T = p.T; a.H = p.H; a.Hkv = p.H_kv; a.K = p.conv_k;
   a.gate_mode = p.gate_mode; a.normalize = p.normalize; a.inv_tau = 1.f / p.gate_tau; a.eps = p.eps;
-  a.wait_limit = g_wait_limit.load();
+  a.wait_limit = wait_limit();
   const int nsub = pl.nsub;
   a.nseg = pl.nseg;
   a.seg_len = pl.seg_len;
@@ -414,8 +415,8 @@ int launch_layer_tc_packed(const Ctx& c, const int32_t* cu, int nseq, const void
 
 }  // namespace lawcat
 
-// Test hook: the limit (clock cycles) of every bounded device-side wait of the tensor-core layer kernels launched from
-// now on; 0 restores the default. A limit of a few cycles makes the first unsatisfied wait give up, which exercises the
+// Test hook: the limit (clock cycles) of every bounded device-side wait of the layer forward and streaming decode kernels
+// launched from now on; 0 restores the default. A limit of a few cycles makes the first unsatisfied wait give up, which exercises the
 // path that reports LAWCAT_ERR_TIMEOUT (nothing faults or hangs: the block leaves its loops, lets its copies land, frees
 // its tensor memory and returns).
 extern "C" void lawcat_test_set_wait_limit(long long cycles) {
