@@ -123,15 +123,15 @@ def kernel_bytes_per_step(name: str, kind: str, s: I.LayerShape) -> float:
         "gla_fwd_rec": (f32_feat if kind == "prefill" else 2 * b["q"]) + b["v"] + b["gate"] + b["o"],
         "convmix_fwd": b["q"] + b["k"] + (f32_feat if kind == "prefill" else 2 * b["q"]),
         "convmix_tc_fwd": b["q"] + b["k"] + f32_feat,
-        # chunkwise backward inside layer_bwd: fp32 features in, fp32 feature gradients out, v, gate, dO in, dgate out,
-        # dv per query head out
-        "gla_tc_bwd": 2 * f32_feat + b["v"] + b["gate"] + b["o"] + b["gate"] + f32_dv,
+        # reverse sweep of layer_bwd: fp32 features in, their fp32 products with the feature gradients out, v, gate, dO in,
+        # dgate out, dv per query head out
+        "layer_bwd_reverse": 2 * f32_feat + b["v"] + b["gate"] + b["o"] + b["gate"] + f32_dv,
         "gla_tc_fwd": f32_feat + b["v"] + b["gate"] + b["o"],
-        "gla_tc_bwd_sweep": f32_feat + b["v"] + b["gate"] + b["o"],   # features, v, gate, dO in
-        "dv_reduce": f32_dv + b["v"],
+        "layer_bwd_sweep": f32_feat + b["v"] + b["gate"] + b["o"],   # features, v, gate, dO in
+        "dv_sum": f32_dv + b["v"],
         # raw q, k, the fp32 features and their products with the gradients in, fp32 du out (dW is negligible)
-        "convmix_tc_bwd": b["q"] + b["k"] + 2 * f32_feat + 4 * (s.H + s.H_kv) * s.d_k,
-        "conv_bwd": 4 * (s.H + s.H_kv) * s.d_k + 2 * (b["q"] + b["k"]),
+        "layer_bwd_mix": b["q"] + b["k"] + 2 * f32_feat + 4 * (s.H + s.H_kv) * s.d_k,
+        "conv_bwd4": 4 * (s.H + s.H_kv) * s.d_k + 2 * (b["q"] + b["k"]),
     }
     if name in ("decode_one", "decode_stream", "decode_state", "decode_features"):
         return alg_bytes_per_step("decode", s)

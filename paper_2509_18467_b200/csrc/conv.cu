@@ -630,7 +630,7 @@ static int conv_bwd_both(const Ctx& c, const float* du_q, const float* du_k, con
   const ConvBwd4 a{{du_q, du_k}, {(const bf16*)q, (const bf16*)k}, {(const bf16*)w_q, (const bf16*)w_k},
                    {(const bf16*)cache_q, (const bf16*)cache_k}, {(bf16*)dq, (bf16*)dk}, {dw_q, dw_k}, {Cq, Ck}, p.B, p.T, p.conv_k};
   const dim3 grid((p.B * ((p.T + CB4_SPAN - 1) / CB4_SPAN) + 3) / 4, (Cq / 4 + 31) / 32 + (Ck / 4 + 31) / 32);
-  LaunchScope _ls("conv_bwd", c.stream);
+  LaunchScope _ls("conv_bwd4", c.stream);
   launch_behind(conv_bwd4_kernel, grid, dim3(128), 0, c.stream, a);
   LAWCAT_CHECK_LAUNCH();
   return LAWCAT_OK;

@@ -1158,16 +1158,16 @@ template <int D>
 static int run(const Ctx& c, const Args& a, const MArgs& m) {
   const lawcat_params& p = *c.p;
   {
-    LaunchScope _ls("gla_tc_bwd_sweep", c.stream);
+    LaunchScope _ls("layer_bwd_sweep", c.stream);
     launch_behind(sweep_kernel<D>, dim3(p.B * p.H), dim3(Cfg<D>::THREADS), Cfg<D>::F_BYTES, c.stream, a);
     LAWCAT_CHECK_LAUNCH();
   }
   {
-    LaunchScope _ls("gla_tc_bwd", c.stream);
+    LaunchScope _ls("layer_bwd_reverse", c.stream);
     launch_behind(reverse_kernel<D>, dim3(p.B * p.H), dim3(Cfg<D>::THREADS), Cfg<D>::R_BYTES, c.stream, a);
     LAWCAT_CHECK_LAUNCH();
   }
-  LaunchScope _ls("convmix_tc_bwd", c.stream);
+  LaunchScope _ls("layer_bwd_mix", c.stream);
   // (all blocks along x: the other axes end at 65535)
   launch_behind(mix_bwd_kernel<D>, dim3((unsigned)((p.T + TT - 1) / TT) * (unsigned)(p.B * p.H_kv)), dim3(MCfg<D>::THREADS), MCfg<D>::BYTES,
                 c.stream, m);
@@ -1211,7 +1211,7 @@ int launch_layer_bwd_tc(const Ctx& c, const void* q, const void* k, const void* 
   {
     const int oct = p.d_v / 8;
     const size_t total = (size_t)p.B * p.T * p.H_kv * oct;
-    LaunchScope _ls("dv_reduce", c.stream);
+    LaunchScope _ls("dv_sum", c.stream);
     launch_behind(dv_sum_kernel, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, c.stream, (const float*)a.dvh, (bf16*)dv, total,
                   p.H / p.H_kv, oct, dw_q, dw_q ? p.H * p.d_k * p.conv_k : 0, dw_k, dw_k ? p.H_kv * p.d_k * p.conv_k : 0);
     LAWCAT_CHECK_LAUNCH();

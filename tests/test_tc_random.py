@@ -100,7 +100,7 @@ def test_random_backward(case):
     api.trace_begin()
     g = api.lawcat_layer_bwd(api.params(B, T, H, Hkv, d, d, **kw), *[dv[n] for n in NAMES], dv["dO"], dev_status=status)
     kernels = api.trace_end()
-    assert ("gla_tc_bwd" in kernels) == (T >= 16), kernels
+    assert ("layer_bwd_reverse" in kernels) == (T >= 16), kernels
     assert int(status.item()) == 0
     op = O.OracleParams(B, T, H, Hkv, d, d, **kw)
     fwd = O.layer_fwd(op, *[x[n] for n in NAMES])
