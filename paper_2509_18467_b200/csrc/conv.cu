@@ -494,10 +494,15 @@ static int conv_bwd_stream(const Ctx& c, const TD* du, const TI* x, const TI* w,
   if (dw && cudaMemsetAsync(dw, 0, sizeof(float) * (size_t)C * p.conv_k, c.stream) != cudaSuccess) return LAWCAT_ERR_CUDA;
   dim3 grid(p.B * ((p.T + CBW_SPAN - 1) / CBW_SPAN), (C + 127) / 128);
   LaunchScope _ls("conv_bwd", c.stream);
-  if (p.conv_k <= 4)
-    conv_bwd_kernel<TD, TI, 4><<<grid, 128, 0, c.stream>>>(du, x, w, cache, dx, dw, p.B, p.T, C, p.conv_k);
-  else
+  // (bf16 storage with fp32 du and a width of up to 4 belongs to conv_bwd4_kernel)
+  constexpr bool WIDE_ONLY = std::is_same<TD, float>::value && std::is_same<TI, bf16>::value;
+  if constexpr (WIDE_ONLY) {
     conv_bwd_kernel<TD, TI, 8><<<grid, 128, 0, c.stream>>>(du, x, w, cache, dx, dw, p.B, p.T, C, p.conv_k);
+  } else if (p.conv_k <= 4) {
+    conv_bwd_kernel<TD, TI, 4><<<grid, 128, 0, c.stream>>>(du, x, w, cache, dx, dw, p.B, p.T, C, p.conv_k);
+  } else {
+    conv_bwd_kernel<TD, TI, 8><<<grid, 128, 0, c.stream>>>(du, x, w, cache, dx, dw, p.B, p.T, C, p.conv_k);
+  }
   LAWCAT_CHECK_LAUNCH();
   return LAWCAT_OK;
 }

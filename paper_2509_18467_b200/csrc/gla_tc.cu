@@ -100,7 +100,7 @@ constexpr uint32_t COL_P = 0, COL_A = 64 /* O' | dQ */, COL_ST = 144 /* S' or R 
                    COL_V = 384 /* dV */;
 
 struct GArgs {
-  const void *qdot, *kdot;   // features: bf16, or fp32 when feat_f32 (scratch of a fused layer forward)
+  const void *qdot, *kdot;   // features: bf16, or fp32 when feat_f32 (forward only: scratch of a fused layer forward)
   const bf16 *v, *gate, *dO;
   const float *S0, *z0;
   bf16* o;
@@ -246,13 +246,14 @@ __global__ void __launch_bounds__(THREADS, MODE == 2 ? 1 : 2) gla_tc_kernel(cons
   __syncthreads();
   sbound = __int_as_float(s_flags[3]);
 
+  const bool feat_f32 = MODE == 0 && a.feat_f32;  // (the backward's features are bf16)
   // rows of the next chunk towards L2 (one 128-byte line per row and tensor)
   auto prefetch_chunk = [&](int m) {
     if (m < 0 || m >= nchunks) return;
     const int r = tid >> 2, which = tid & 3, t = m * C + r;
     if (t >= a.T) return;
     const size_t tq = ((size_t)b * a.T + t) * a.H + h, tv = ((size_t)b * a.T + t) * a.Hkv + j;
-    const size_t fb = a.feat_f32 ? 4 : 2;
+    const size_t fb = feat_f32 ? 4 : 2;
     const void* ptr = which == 0 ? (const void*)((const char*)a.qdot + tq * D * fb) : which == 1 ? (const void*)((const char*)a.kdot + tq * D * fb)
                     : which == 2 ? (const void*)(a.v + tv * D)
                     : (a.gate_dim == 1 ? (const void*)(a.gate + tq) : (const void*)(a.gate + tq * D));
@@ -348,7 +349,7 @@ __global__ void __launch_bounds__(THREADS, MODE == 2 ? 1 : 2) gla_tc_kernel(cons
       float inv = 0.f, dl = 0.f;
       if (r < nvalid) {
         const size_t tq = ((size_t)b * a.T + t0 + r) * a.H + h, tv = ((size_t)b * a.T + t0 + r) * a.Hkv + j;
-        if (a.feat_f32) {
+        if (feat_f32) {
           const float* fq = reinterpret_cast<const float*>(a.qdot) + tq * D + o8 * 8;
           const float* fk = reinterpret_cast<const float*>(a.kdot) + tq * D + o8 * 8;
           const float4 q0 = *reinterpret_cast<const float4*>(fq), q1 = *reinterpret_cast<const float4*>(fq + 4);
@@ -366,7 +367,7 @@ __global__ void __launch_bounds__(THREADS, MODE == 2 ? 1 : 2) gla_tc_kernel(cons
           dl = a.ws_delta[tq];
         }
       }
-      if (!a.feat_f32 || r >= nvalid) { unpack8b(zq, q); unpack8b(zk, k); }
+      if (!feat_f32 || r >= nvalid) { unpack8b(zq, q); unpack8b(zk, k); }
       unpack8b(zv, vv);
       const float4 xa = *reinterpret_cast<const float4*>(s_x + r * D + o8 * 8), xb = *reinterpret_cast<const float4*>(s_x + r * D + o8 * 8 + 4);
       x[0] = xa.x; x[1] = xa.y; x[2] = xa.z; x[3] = xa.w; x[4] = xb.x; x[5] = xb.y; x[6] = xb.z; x[7] = xb.w;
