@@ -88,6 +88,13 @@ PyObject* call(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
     }
     if (args[6] != Py_None) st = PyLong_AsVoidPtr(args[6]);
     else if (c10::cuda::device_count() > 0) st = c10::cuda::getCurrentCUDAStream().stream();
+    // the scratch goes back to the allocator when this call returns, and the allocator hands it on in the order of the current
+    // stream: on another one it has to know how long the block is in use
+    if (scratch.defined()) {
+      const c10::DeviceIndex dev = scratch.device().index();
+      if (st != (void*)c10::cuda::getCurrentCUDAStream(dev).stream())
+        scratch.record_stream(c10::cuda::getStreamFromExternal((cudaStream_t)st, dev).unwrap());
+    }
   } catch (const std::exception& e) {
     PyErr_SetString(PyExc_RuntimeError, e.what());
     return nullptr;

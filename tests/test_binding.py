@@ -1,5 +1,5 @@
 """The native module that turns tensors into the pointers of a C entry point: what is not a tensor is a Python error, and other
-Python threads run while the library does. No GPU: nothing here is launched."""
+Python threads run while the library does (no GPU: nothing is launched there); scratch of a call on a stream of its own."""
 import ctypes
 import threading
 import time
@@ -71,3 +71,26 @@ def test_other_threads_run_during_a_call(binding):
         t.join()
     assert t1 - t0 >= 0.5
     assert sum(t0 + 0.02 < s < t1 - 0.02 for s in stamps) >= 10
+
+
+@pytest.mark.gpu
+def test_scratch_of_a_call_on_another_stream_is_not_handed_on_early():
+    """The call's kernels wait behind a delay on a side stream while the current stream allocates and fills blocks of the
+    scratch's size: the result is that of a call on the current stream."""
+    import torch
+    from paper_2509_18467_b200 import inputs as I
+    names = ["q", "k", "v", "gate", "w_q", "w_k", "W"]
+    s = I.LayerShape(1, 300, 4, 2, 64, 64, dtype="bf16", gate_tau=1.0, config_id=131)
+    t = [api.to_device(v, "bf16") for v in I.make(s, names).values()]
+    p = api.params(1, 300, 4, 2, 64, 64, gate_tau=1.0)   # (served by the kernels that keep features in scratch)
+    need = api.workspace_bytes(p, api.OP_LAYER_FWD)
+    assert need > 0
+    ref = api.lawcat_layer_fwd(p, *t)["o"]
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(20_000_000)   # about 10 ms
+    r = api.lawcat_layer_fwd(p, *t, stream=side)["o"]
+    junk = [torch.full((need,), 255, dtype=torch.uint8, device="cuda") for _ in range(4)]
+    torch.cuda.synchronize()
+    assert torch.equal(r, ref) and len(junk) == 4
