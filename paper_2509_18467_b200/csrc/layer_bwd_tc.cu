@@ -581,6 +581,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
   const float osc = pow2i(sc);
   int al_prev = 0;
   float wmax = 0.f;
+  int copied = -1;  // (first thread) the last copy of a state operand that was started
   // what the next chunk's first passes need, fetched while the chunk behind it is computed
   Gates<D> gates;
   int2 nx_meta = make_int2(0, 0);
@@ -674,11 +675,14 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
     publish();
     if (tid == 0) {
       // the state operand of this chunk (needed behind the mask pass), over the exponents
-      mbar_arrive_expect_tx(bar_s, 2 * F::T_C);
-      const uint8_t* src = a.s16 + ((size_t)bh * nch + n) * (2 * F::T_C);
-      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(sb + F::R_S),
-                   "l"(src), "r"(2 * F::T_C), "r"(bar_s)
-                   : "memory");
+      if (!s_fl[1]) {
+        mbar_arrive_expect_tx(bar_s, 2 * F::T_C);
+        const uint8_t* src = a.s16 + ((size_t)bh * nch + n) * (2 * F::T_C);
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(sb + F::R_S),
+                     "l"(src), "r"(2 * F::T_C), "r"(bar_s)
+                     : "memory");
+        copied = nch - 1 - n;
+      }
       mm.split(F::R_P, KV(F::R_QS, F::SL_T), KV(F::R_QS + F::T_TOK, F::SL_T), 2 * F::SL_T, KV(F::R_KS, F::SL_T),
                KV(F::R_KS + F::T_TOK, F::SL_T), 2 * F::SL_T, D / 16, instr_desc(128, C, fmt, MAJOR_K, MAJOR_K), false);
       mm.chain(F::R_EP, KV(F::R_DO, F::SL_T), 2 * F::SL_T, KV(F::R_V, F::SL_T), 2 * F::SL_T, D / 16,
@@ -898,7 +902,10 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
   if (lane == 0) atomicMax(const_cast<int*>(&s_fl[5]), __float_as_int(wmax < 1.0e30f ? wmax : 1.0e30f));
   tc_fence_before_sync();
   __syncthreads();
-  if (tid == 0) a.wmax[bh] = __int_as_float(s_fl[5]);
+  if (tid == 0) {
+    a.wmax[bh] = __int_as_float(s_fl[5]);
+    if (s_fl[1] && copied >= 0) mbar_wait(bar_s, (uint32_t)(copied & 1));  // (after a wait that ran out it may still be under way)
+  }
   if (warp == 0) {
     tc_fence_after_sync();
     tmem_dealloc(mm.tmem, F::COLS);
