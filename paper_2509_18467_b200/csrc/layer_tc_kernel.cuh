@@ -144,6 +144,8 @@ enum {
   B_PH_FULL,       // row warps: masked scores written               -> MMA 3
   B_MMA3,          // MMA 3 complete: O' ready -> row warps; v tile free -> TMA
   B_O_FREE,        // row warps: O' consumed                         -> MMA 2 of the next chunk
+  B_RAW_LAND,      // TMA: raw q|k tile, v tile of a packed sequence's ragged last chunk landed -> TMA warp, which zeroes the
+  B_V_LAND,        //   rows past the end before it passes them on (these two complete once)
   NUM_BARS
 };
 
@@ -370,6 +372,10 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   const int t_begin = min(T, seg * sq.seg_len + (sub * cps / a.nsub) * C);
   const int t_end = min(T, seg * sq.seg_len + ((sub + 1) * cps / a.nsub) * C);
   const int nchunks = max(0, (t_end - t_begin + C - 1) / C);
+  // The last chunk of a packed sequence: behind its last token the tiles hold the next sequence's first tokens, which a factor
+  // of zero further on would not keep out where they are not finite. (Elsewhere the copies fill rows past the end with zeros.)
+  const int last_valid = t_end - t_begin - (nchunks - 1) * C;
+  const bool mixed = MODE == 0 && tab.n != 0 && nchunks > 0 && last_valid < C;
   // index of the state of the real head that owns state row c (rows 64-127 of a pair: the second head): among the caller's
   // states (one per sequence), or among the workspace's (one per segment piece)
   auto head_of_row = [&](int c) -> size_t { return h0 + (pair ? (c >> 6) : 0); };
@@ -388,13 +394,13 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   // sequence spent a third of its time here, most of it in loads that waited for one another (given states 18k cycles, now
   // 2k; W 2k; the first tiles were asked for 3k cycles after the rest).
   const int tt_first = sq.tm_t + t_begin;  // (token coordinate of the first chunk in the tensor maps)
-  auto load_raw = [&](int tt0) {
-    mbar_arrive_expect_tx(bar(B_RAW_FULL), (MODE == 0 ? 16384u : 8192u) * (uint32_t)nslab);
+  auto load_raw = [&](int tt0, int full) {
+    mbar_arrive_expect_tx(bar(full), (MODE == 0 ? 16384u : 8192u) * (uint32_t)nslab);
 #pragma unroll 1
     for (int s = 0; s < nslab; ++s) {
-      if (MODE == 0) tma_load_4d(sb + OFF_AU + s * 16384, &tm_q, bar(B_RAW_FULL), s * 64, h, tt0, sq.tm_b);
+      if (MODE == 0) tma_load_4d(sb + OFF_AU + s * 16384, &tm_q, bar(full), s * 64, h, tt0, sq.tm_b);
       // (pair: the same 64 key channels into both halves of the tile)
-      tma_load_4d(sb + OFF_AU + s * 16384 + 8192, &tm_k, bar(B_RAW_FULL), pair ? 0 : s * 64, j, tt0, sq.tm_b);
+      tma_load_4d(sb + OFF_AU + s * 16384 + 8192, &tm_k, bar(full), pair ? 0 : s * 64, j, tt0, sq.tm_b);
     }
   };
   auto load_gate = [&](int tt0) {
@@ -402,10 +408,10 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     tma_load_4d(sb + OFF_G, &tm_g, bar(B_G_FULL), 0, h, tt0, sq.tm_b);
     if (nslab == 2) tma_load_4d(sb + OFF_G + 8192, &tm_g, bar(B_G_FULL), 64, h, tt0, sq.tm_b);
   };
-  auto load_v = [&](int tt0) {
-    mbar_arrive_expect_tx(bar(B_V_FULL), 8192u * (uint32_t)vslab);
-    tma_load_4d(sb + OFF_V, &tm_v, bar(B_V_FULL), 0, j, tt0, sq.tm_b);
-    if (vslab == 2) tma_load_4d(sb + OFF_V + 8192, &tm_v, bar(B_V_FULL), 64, j, tt0, sq.tm_b);
+  auto load_v = [&](int tt0, int full) {
+    mbar_arrive_expect_tx(bar(full), 8192u * (uint32_t)vslab);
+    tma_load_4d(sb + OFF_V, &tm_v, bar(full), 0, j, tt0, sq.tm_b);
+    if (vslab == 2) tma_load_4d(sb + OFF_V + 8192, &tm_v, bar(full), 64, j, tt0, sq.tm_b);
   };
   // Row warps move states between global memory, where a row is contiguous, and tensor memory, where it belongs to one lane,
   // through 16-byte units in shared memory: a warp's 32 rows x NC columns, units XOR-swizzled with the row so that both
@@ -440,11 +446,14 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       mbar_init(bar(B_PH_FULL), 128);
       mbar_init(bar(B_MMA3), 1);
       mbar_init(bar(B_O_FREE), 128);
+      mbar_init(bar(B_RAW_LAND), 1);
+      mbar_init(bar(B_V_LAND), 1);
       mbar_fence_init();
       if (nchunks > 0) {
-        load_raw(tt_first);
+        const bool land = mixed && nchunks == 1;
+        load_raw(tt_first, land ? B_RAW_LAND : B_RAW_FULL);
         if (a.gate_dim != 1) load_gate(tt_first);
-        load_v(tt_first);
+        load_v(tt_first, land ? B_V_LAND : B_V_FULL);
       }
       s_flags[1] = 0;
       for (int i = 0; i < 7; ++i) s_rmax[i] = 0;
@@ -541,14 +550,15 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
 
   if (warp == TMA_WARP) {
     // ================================================================================================ TMA producer
+    const int cp0 = nchunks > 0 ? 0 : -1;  // (the first chunk's copies were started by the set-up)
+    int ar_raw = cp0, ar_g = a.gate_dim != 1 ? cp0 : -1, ar_v = cp0;  // last chunk whose copies were started, per tile
+    const int plain = mixed ? nchunks - 1 : nchunks;
     if (lane == 0) {
-      const int cp0 = nchunks > 0 ? 0 : -1;  // (the first chunk's copies were started by the set-up)
-      int ar_raw = cp0, ar_g = a.gate_dim != 1 ? cp0 : -1, ar_v = cp0;  // last chunk whose copies were started, per tile
-      for (int n = 1; n < nchunks; ++n) {
+      for (int n = 1; n < plain; ++n) {
         const int tt0 = tt_first + n * C;
         const uint32_t pp = (uint32_t)((n - 1) & 1);
         WAIT(B_MMA1, pp);  // MMA 1 of the previous chunk has read the in-place conv output
-        load_raw(tt0);
+        load_raw(tt0, B_RAW_FULL);
         ar_raw = n;
         if (a.gate_dim != 1) {
           WAIT(B_G_FREE, pp);
@@ -556,15 +566,57 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
           ar_g = n;
         }
         WAIT(MODE == 0 ? B_MMA3 : B_MMA2, pp);  // the last MMA that reads v
-        load_v(tt0);
+        load_v(tt0, B_V_FULL);
         ar_v = n;
       }
-      if (*s_abort) {
-        // leaving early: give the copies that are still in flight a bounded time to land before the CTA exits
-        if (ar_raw >= 0) mbar_wait(bar(B_RAW_FULL), (uint32_t)(ar_raw & 1));
-        if (ar_g >= 0) mbar_wait(bar(B_G_FULL), (uint32_t)(ar_g & 1));
-        if (ar_v >= 0) mbar_wait(bar(B_V_FULL), (uint32_t)(ar_v & 1));
+    }
+    if (mixed) {
+      // the last chunk, by the whole warp: its raw and v tiles land on barriers of their own, the rows past the end are
+      // zeroed, and only then the tiles are passed on
+      __syncwarp();
+      const int n = nchunks - 1, tt0 = tt_first + n * C;
+      const uint32_t pp = (uint32_t)((n - 1) & 1);
+      auto await = [&](int b, uint32_t par) -> bool {
+        return __all_sync(0xffffffffu, wait_or_abort(bar(b), par, s_abort, a.wait_limit));
+      };
+      auto zero_rows = [&](uint32_t tile) {  // rows [last_valid, 64) of a [64 x 128 B] tile
+        for (int u = last_valid * 8 + lane; u < C * 8; u += 32) sts128(sb + tile + (uint32_t)u * 16, make_uint4(0u, 0u, 0u, 0u));
+      };
+      bool ok = __all_sync(0xffffffffu, *s_abort == 0);
+      if (n > 0) {
+        ok = ok && await(B_MMA1, pp);
+        if (ok && lane == 0) load_raw(tt0, B_RAW_LAND);
+        if (ok) ar_raw = n;
+        if (a.gate_dim != 1) {
+          ok = ok && await(B_G_FREE, pp);
+          if (ok && lane == 0) load_gate(tt0);
+          if (ok) ar_g = n;
+        }
       }
+      ok = ok && await(B_RAW_LAND, 0u);
+      if (ok) {
+        for (int t = 0; t < 2 * nslab; ++t) zero_rows(OFF_AU + (uint32_t)t * 8192u);  // (q and k rows of each slab)
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(B_RAW_FULL));
+      }
+      if (n > 0) {
+        ok = ok && await(B_MMA3, pp);
+        if (ok && lane == 0) load_v(tt0, B_V_LAND);
+        if (ok) ar_v = n;
+      }
+      ok = ok && await(B_V_LAND, 0u);
+      if (ok) {
+        for (int t = 0; t < vslab; ++t) zero_rows(OFF_V + (uint32_t)t * 8192u);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(B_V_FULL));
+      }
+    }
+    if (lane == 0 && *s_abort) {
+      // leaving early: give the copies that are still in flight a bounded time to land before the CTA exits
+      const bool lr = mixed && ar_raw == nchunks - 1, lv = mixed && ar_v == nchunks - 1;
+      if (ar_raw >= 0) mbar_wait(bar(lr ? B_RAW_LAND : B_RAW_FULL), lr ? 0u : (uint32_t)(ar_raw & 1));
+      if (ar_g >= 0) mbar_wait(bar(B_G_FULL), (uint32_t)(ar_g & 1));
+      if (ar_v >= 0) mbar_wait(bar(lv ? B_V_LAND : B_V_FULL), lv ? 0u : (uint32_t)(ar_v & 1));
     }
   } else if (warp == MMA_WARP) {
     // ================================================================================================ MMA issuer
@@ -837,13 +889,6 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
 #pragma unroll
           for (int cp = 0; cp < 4; ++cp) { x3[cp] = x2[cp]; x2[cp] = x1[cp]; x1[cp] = x0[cp]; }
         }
-        // Rows past the end of the sequence: zeros. In a pack they hold the next sequence's tokens, and a factor of zero further
-        // on would not keep out what is not finite there.
-        if (MODE == 0 && nvalid < C) {
-#pragma unroll 1
-          for (int i = 0; i < 8; ++i)
-            if (cv_rg * 8 + i >= nvalid) sts128(au + sw128(crow0 + i, cjc), make_uint4(0u, 0u, 0u, 0u));
-        }
         if (cv_rg == 7) {  // the last three raw rows of the chunk are the next chunk's halo (bf16 values: exact repack)
           uint4* hl = reinterpret_cast<uint4*>(sg + OFF_HALO) + cv_stream * 48 + cv_oct;
           hl[0] = pack8p(x3, false); hl[16] = pack8p(x2, false); hl[32] = pack8p(x1, false);
@@ -955,11 +1000,6 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
 #pragma unroll
           for (int e = 0; e < 8; ++e) vm = fmaxf(vm, fabsf(x[e]));
           sts128(ad, pack8(x, true));
-        }
-        if (MODE == 0 && nvalid < C) {  // (rows past the end, as in the conv)
-#pragma unroll 1
-          for (int u = vt; u < vslab * 512; u += vthreads)
-            if (((u >> 3) & (C - 1)) >= nvalid) sts128(sb + OFF_V + (uint32_t)u * 16, make_uint4(0u, 0u, 0u, 0u));
         }
         vm = warp_max(vm);
         if (lane == 0) atomicMax(&s_vmax[p], __float_as_int(vm < 3.0e38f ? vm : 3.0e38f));

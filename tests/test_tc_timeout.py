@@ -45,6 +45,30 @@ def test_wait_that_runs_out_is_reported_and_the_device_stays_usable(T):
     check(r["S_T"], ref["S_T"], "bf16", "S_T", f32_store=True)
 
 
+@pytest.mark.parametrize("d", [128, 64])
+def test_wait_of_a_packed_launch_that_runs_out(d):
+    """(the last chunk of a packed sequence passes through barriers of its own)"""
+    import torch
+    from paper_2509_18467_b200 import api
+    cu = [0, 40, 170, 234, 934]
+    s = I.LayerShape(1, cu[-1], 2, 1, d, d, dtype="bf16", config_id=93)
+    t = [api.to_device(v, "bf16") for v in I.make(s, NAMES).values()]
+    p = api.params(1, s.T, 2, 1, d, d)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    ref = api.lawcat_layer_fwd_varlen(p, cu, *t)
+    try:
+        api.test_set_wait_limit(300)
+        api.lawcat_layer_fwd_varlen(p, cu, *t, dev_status=status)
+        torch.cuda.synchronize()
+    finally:
+        api.test_set_wait_limit(0)
+    assert int(status.item()) == 5
+    status.zero_()
+    r = api.lawcat_layer_fwd_varlen(p, cu, *t, dev_status=status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0 and torch.equal(r["o"], ref["o"]) and torch.equal(r["S_T"], ref["S_T"])
+
+
 @pytest.mark.parametrize("d,B", [(128, 16), (64, 48)])
 def test_wait_of_the_streaming_decode_step_that_runs_out(d, B):
     import torch
