@@ -116,7 +116,8 @@ __global__ void __launch_bounds__(fwd_threads<D, TO>()) convmix_tc_fwd_kernel(co
   volatile int* const s_flags = reinterpret_cast<volatile int*>(sg + OFF_BAR + 16);  // [0] tmem base, [1] abort
   float* const s_taps = reinterpret_cast<float*>(sg + OFF_TAPS);
   float* const s_red = reinterpret_cast<float*>(sg + OFF_RED);  // [max, sum][column group][128 rows]
-  const int tiles = (a.T + TT - 1) / TT, t0 = blockIdx.x % tiles * TT, bh = blockIdx.x / tiles, h = bh % a.H, b = bh / a.H;
+  const int t0 = tile_of_block() * TT, bh = blockIdx.x, h = bh % a.H, b = bh / a.H;
+  if (t0 >= a.T) return;
   const int G = a.H / a.Hkv, j = h / G;
   if (tid == 0) {
     mbar_init(sb + OFF_BAR, 1);
@@ -273,7 +274,8 @@ __global__ void __launch_bounds__(128, 2) convmix_tc_bwd_kernel(const CArgs a) {
   const uint32_t sb = smem_u32(sg);
   const int tid = threadIdx.x, warp = tid >> 5;
   volatile int* const s_flags = reinterpret_cast<volatile int*>(sg + OFF_BAR + 16);
-  const int tiles = (a.T + TT - 1) / TT, t0 = blockIdx.x % tiles * TT, bj = blockIdx.x / tiles, j = bj % a.Hkv, b = bj / a.Hkv;
+  const int t0 = tile_of_block() * TT, bj = blockIdx.x, j = bj % a.Hkv, b = bj / a.Hkv;
+  if (t0 >= a.T) return;
   const int G = a.H / a.Hkv;
   if (tid == 0) {
     mbar_init(sb + OFF_BAR, 1);
@@ -511,8 +513,7 @@ int launch_convmix_tc_fwd(const Ctx& c, const void* q, const void* k, const void
       done[dev] = true;
     }
   }
-  // (all blocks along x: the other axes end at 65535, a batch of many short sequences does not)
-  const dim3 grid((unsigned)((p.T + TT - 1) / TT) * (unsigned)(p.B * p.H));
+  const dim3 grid = tile_grid(p.B * p.H, p.T);
   LaunchScope _ls("convmix_tc_fwd", c.stream);
   if (p.d_k == 64) {
     if (out_f32) launch_behind(convmix_tc_fwd_kernel<64, float>, grid, dim3(fwd_threads<64, float>()), fwd_smem<64, float>(), c.stream, a);
@@ -544,7 +545,7 @@ int launch_convmix_tc_bwd(const Ctx& c, const void* q, const void* k, const void
       done[dev] = true;
     }
   }
-  const dim3 grid((unsigned)((p.T + TT - 1) / TT) * (unsigned)(p.B * p.H_kv));
+  const dim3 grid = tile_grid(p.B * p.H_kv, p.T);
   LaunchScope _ls("convmix_tc_bwd", c.stream);
   convmix_tc_bwd_kernel<<<grid, 128, bwd_smem(), c.stream>>>(a);
   LAWCAT_CHECK_LAUNCH();

@@ -946,7 +946,8 @@ __global__ void __launch_bounds__(MCfg<D>::THREADS, D == 128 ? 1 : 2) mix_bwd_ke
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   volatile int* const s_fl = reinterpret_cast<volatile int*>(sg + M::BAR + 16);  // tmem base, abort
   float* const s_taps = reinterpret_cast<float*>(sg + M::TAPS);
-  const int tiles = (a.T + TT - 1) / TT, t0 = blockIdx.x % tiles * TT, bj = blockIdx.x / tiles, j = bj % a.Hkv, b = bj / a.Hkv, G = a.H / a.Hkv;
+  const int t0 = blockIdx.x * TT, bj = blockIdx.z * gridDim.y + blockIdx.y, j = bj % a.Hkv, b = bj / a.Hkv, G = a.H / a.Hkv;
+  if (b >= a.B) return;
   const int nvalid = min(TT, a.T - t0);
   if (tid == 0) {
     mbar_init(sb + M::BAR, 1);
@@ -1175,8 +1176,10 @@ static int run(const Ctx& c, const Args& a, const MArgs& m) {
     LAWCAT_CHECK_LAUNCH();
   }
   LaunchScope _ls("layer_bwd_mix", c.stream);
-  // (all blocks along x: the other axes end at 65535)
-  launch_behind(mix_bwd_kernel<D>, dim3((unsigned)((p.T + TT - 1) / TT) * (unsigned)(p.B * p.H_kv)), dim3(MCfg<D>::THREADS), MCfg<D>::BYTES,
+  // (tiles along x, with neighbours on the same head: 3 tiles of 8 heads of 128, head by head 92.7 us instead of 90.6; the y axis
+  // ends at 65535, so the heads go on along z)
+  const unsigned heads = (unsigned)(p.B * p.H_kv), ny = heads < 32768u ? heads : 32768u;
+  launch_behind(mix_bwd_kernel<D>, dim3((unsigned)((p.T + TT - 1) / TT), ny, (heads + ny - 1) / ny), dim3(MCfg<D>::THREADS), MCfg<D>::BYTES,
                 c.stream, m);
   LAWCAT_CHECK_LAUNCH();
   return LAWCAT_OK;

@@ -17,6 +17,14 @@ using namespace tc;
 constexpr int TT = 128;   // tokens per tile
 constexpr int HALO = 3;   // raw rows kept in front of a tile (conv width up to 4)
 
+// Grid of the kernels that take one (sequence, head) and one tile of TT tokens per block: x the (sequence, head), whose number
+// may pass the 65535 that end the other axes, y and z the tile.
+inline dim3 tile_grid(int heads, int T) {
+  const unsigned tiles = (unsigned)(T + TT - 1) / TT, y = tiles < 32768u ? tiles : 32768u;
+  return dim3((unsigned)heads, y, (tiles + y - 1) / y);
+}
+__device__ __forceinline__ int tile_of_block() { return (int)(blockIdx.z * gridDim.y + blockIdx.y); }
+
 template <int D>
 struct Lay {
   static constexpr int OPR = D / 8;                         // 16-byte octets per row
