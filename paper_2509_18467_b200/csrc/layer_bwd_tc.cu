@@ -329,9 +329,8 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) sweep_kerne
     bool f16 = __int_as_float(s_fl[2]) <= RMAX_F16;
     const int kap = max(-100, min(KAP_MAX, 14 - exp_above(fmaxf(sbound, 1e-30f))));
     const float ksc = pow2i(kap);
-    // ---- operands (once more in bf16 when v turns out to be beyond the fp16 range: the largest |v| is known behind them)
-#pragma unroll 1
-    for (;;) {
+    // ---- operands
+    auto operands = [&](bool f16) {
       float vmax = 0.f;
 #pragma unroll
       for (int it = 0; it < 2; ++it) {
@@ -363,10 +362,14 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) sweep_kerne
       }
       vmax = warp_max(vmax);
       if (lane == 0) atomicMax(const_cast<int*>(&s_fl[4]), __float_as_int(vmax < 1.0e30f ? vmax : 1.0e30f));
-      __syncthreads();  // (the exponents have been read: the state operand may overwrite them)
-      if (!f16 || __int_as_float(s_fl[4]) <= VMAX_F16) break;
+    };
+    operands(f16);
+    __syncthreads();  // (the exponents have been read: the state operand may overwrite them)
+    if (f16 && __int_as_float(s_fl[4]) > VMAX_F16) {  // v is beyond the fp16 range: once more, in bf16
       f16 = false;
       rows.load(a, row0, h, j, nvalid, tid);
+      operands(false);
+      __syncthreads();
     }
     const int fmt = f16 ? FMT_F16 : FMT_BF16;
     // ---- state pass: W = 2^(bm + ft of the chunk in front) S, kept in tensor memory and as the two-term operand, scaled 2^kap
@@ -916,8 +919,9 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
 // From w = p * dp of both streams (p the features) back through the softmax and the shared linear layer:
 //   dy = w - p sum(w),   du = dy W_h^T (query stream; key stream summed over the heads of the group),   dW_h += u^T dy
 // One block = one (batch, key head, tile of 128 tokens), walking the group's heads and both streams. dy (scaled by a power of
-// two from the largest |w| of the head) and u, the recomputed conv output, are two-term fp16 pairs; the key stream's du is
-// summed over the heads in registers, each head on its own scale. du of the query stream overwrites wq in place.
+// two from the largest |w| of the group, or of the head where that is far smaller) and u, the recomputed conv output, are
+// two-term fp16 pairs; the key stream's du is accumulated over the heads in tensor memory. du of the query stream overwrites wq
+// in place.
 struct MArgs {
   const bf16 *q, *k, *w_q, *w_k, *W, *cache_q, *cache_k;
   const float *qd, *kd, *wk;
@@ -967,17 +971,27 @@ __global__ void __launch_bounds__(MCfg<D>::THREADS, D == 128 ? 1 : 2) mix_bwd_ke
   const int row = (warp & 3) * 32 + lane, cg = warp >> 2;
   constexpr int HC = D / M::NCG, NTH = M::THREADS;
   Waiter wt{sb + M::BAR, 0u, s_fl + 1, a.dev_status};
-  float sc = 1.f, isc = 1.f;  // power of two on the head's dy
-  float duk[HC];              // du of the key stream, this thread's row and columns
-#pragma unroll
-  for (int i = 0; i < HC; ++i) duk[i] = 0.f;
+  // 2^sg on dy. The head's largest |w| becomes 2^7 .. 2^8 by it, which leaves |dy| <= |w| + sum |w| below the fp16 maximum for
+  // every row, or down to 2^3 where the group's own power of two does that: its heads then need no rescaling among themselves.
+  auto sg_of = [](float w) -> int { return 8 - exp_above(fmaxf(w, 1e-30f)); };
+  const float* const wmax = a.wmax + b * a.H + j * G;
+  float wg = 0.f, w_next = wmax[0], sc = 1.f, isc = 1.f;  // (w_next: of the next head, fetched a head ahead)
+  for (int g = lane; g < G; g += 32) wg = fmaxf(wg, wmax[g]);
+  const int sg_group = sg_of(warp_max(wg));
+  int sg_at = 0;
   const int o = tid % L::OPR, rr0 = tid / L::OPR;
   constexpr int RSTEP = NTH / L::OPR, RPT = TT / RSTEP;
-  // this thread's row and columns of du to global rows through the (dead) dy tiles
-  auto rows_out = [&](const float (&d)[HC], float* dst, int NH, int head) {
+  // fp32 [128][D] accumulator to global rows through the (dead) dy tiles
+  auto rows_out = [&](uint32_t col, float* dst, int NH, int head) {
+    float d[8];
+#pragma unroll 1
+    for (int c0 = cg * HC; c0 < (cg + 1) * HC; c0 += 8) {
+      tmem_ld8(lane_base + col + c0, d);
+      tmem_wait_ld();
 #pragma unroll
-    for (int i = 0; i < HC; i += 4)
-      *reinterpret_cast<float4*>(sg + M::DY + foff<D>(row, (cg * HC + i) >> 2)) = make_float4(d[i], d[i + 1], d[i + 2], d[i + 3]);
+      for (int i = 0; i < 8; i += 4)
+        *reinterpret_cast<float4*>(sg + M::DY + foff<D>(row, (c0 + i) >> 2)) = make_float4(d[i] * isc, d[i + 1] * isc, d[i + 2] * isc, d[i + 3] * isc);
+    }
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
@@ -991,10 +1005,26 @@ __global__ void __launch_bounds__(MCfg<D>::THREADS, D == 128 ? 1 : 2) mix_bwd_ke
 #pragma unroll 1
   for (int g = 0; g < G; ++g) {
     const int h = j * G + g;
-    // the head's largest |w| becomes 2^7 .. 2^8, which leaves |dy| <= |w| + sum |w| below the fp16 maximum for every row
-    const int sgm = 8 - exp_above(fmaxf(a.wmax[b * a.H + h], 1e-30f));
-    sc = pow2i(sgm);
-    isc = pow2i(-sgm);
+    {
+      const int own = sg_of(w_next), sgm = own - sg_group <= 4 ? sg_group : min(own, sg_group + 60);
+      if (g > 0 && sgm != sg_at) {  // the key stream's du so far, on this head's scale
+        const float f = pow2i(sgm - sg_at);
+        float d[8];
+#pragma unroll 1
+        for (int c0 = cg * HC; c0 < (cg + 1) * HC; c0 += 8) {
+          tmem_ld8(lane_base + M::DUK + c0, d);
+          tmem_wait_ld();
+#pragma unroll
+          for (int i = 0; i < 8; ++i) d[i] *= f;
+          tmem_st8(lane_base + M::DUK + c0, d);
+        }
+        tmem_wait_st();
+      }
+      sg_at = sgm;
+      if (g + 1 < G) w_next = wmax[g + 1];
+      sc = pow2i(sgm);
+      isc = pow2i(-sgm);
+    }
     load_w_tile<D>(sg + M::WT, a.W + (size_t)h * D * D, tid, NTH);
 #pragma unroll 1
     for (int stream = 0; stream < 2; ++stream) {
@@ -1064,24 +1094,14 @@ __global__ void __launch_bounds__(MCfg<D>::THREADS, D == 128 ? 1 : 2) mix_bwd_ke
       tc_fence_after_sync();
       if (tid == 0) {
         mm.split(stream ? M::DUK : M::DUQ, kview(sb + M::DY, L::SLAB_U), kview(sb + M::DY + L::TILE_U, L::SLAB_U), 2 * L::SLAB_U,
-                 kview(sb + M::WT, L::SLAB_W), 0, 2 * L::SLAB_W, D / 16, instr_desc(128, D, FMT_F16, MAJOR_K, MAJOR_K), false);
+                 kview(sb + M::WT, L::SLAB_W), 0, 2 * L::SLAB_W, D / 16, instr_desc(128, D, FMT_F16, MAJOR_K, MAJOR_K),
+                 stream == 1 && g > 0);
         mm.split(M::DWC, mview(sb + M::U, L::SLAB_U), mview(sb + M::U + L::TILE_U, L::SLAB_U), 256, mview(sb + M::DY, L::SLAB_U),
                  mview(sb + M::DY + L::TILE_U, L::SLAB_U), 256, TT / 16, instr_desc(128, D, FMT_F16, MAJOR_MN, MAJOR_MN), stream == 1);
         mma_commit(sb + M::BAR);
       }
       wt.wait();
-      static_assert(HC == 32, "one wide load");
-      float du[HC];
-      tmem_ld32(lane_base + (stream ? M::DUK : M::DUQ) + cg * HC, du);
-      tmem_wait_ld();
-      if (stream == 0) {
-#pragma unroll
-        for (int i = 0; i < HC; ++i) du[i] *= isc;
-        rows_out(du, a.wq, a.H, h);
-      } else {
-#pragma unroll
-        for (int i = 0; i < HC; ++i) duk[i] = fmaf(du[i], isc, duk[i]);
-      }
+      if (stream == 0) rows_out(M::DUQ, a.wq, a.H, h);
     }
     // dW of the head: row c of the accumulator belongs to lane c
     if (a.dW && row < D) {
@@ -1102,7 +1122,7 @@ __global__ void __launch_bounds__(MCfg<D>::THREADS, D == 128 ? 1 : 2) mix_bwd_ke
     __syncthreads();
     tc_fence_after_sync();
   }
-  rows_out(duk, a.du_k, a.Hkv, j);
+  rows_out(M::DUK, a.du_k, a.Hkv, j);
   tc_fence_before_sync();
   __syncthreads();
   if (warp == 0) {
