@@ -28,6 +28,7 @@
 #include <cuda_fp16.h>
 
 #include <mutex>
+#include <type_traits>
 
 #include "common.cuh"
 #include "octet_tile.cuh"
@@ -971,14 +972,20 @@ __global__ void __launch_bounds__(MCfg<D>::THREADS, D == 128 ? 1 : 2) mix_bwd_ke
   const int row = (warp & 3) * 32 + lane, cg = warp >> 2;
   constexpr int HC = D / M::NCG, NTH = M::THREADS;
   Waiter wt{sb + M::BAR, 0u, s_fl + 1, a.dev_status};
-  // 2^sg on dy. The head's largest |w| becomes 2^7 .. 2^8 by it, which leaves |dy| <= |w| + sum |w| below the fp16 maximum for
-  // every row, or down to 2^3 where the group's own power of two does that: its heads then need no rescaling among themselves.
+  // 2^sg on dy. The group's largest |w| becomes 2^7 .. 2^8 by it, which leaves |dy| <= |w| + sum |w| below the fp16 maximum for
+  // every row. A head more than 2^4 below the others gets a power of two of its own (`spread`: there is one).
   auto sg_of = [](float w) -> int { return 8 - exp_above(fmaxf(w, 1e-30f)); };
   const float* const wmax = a.wmax + b * a.H + j * G;
-  float wg = 0.f, w_next = wmax[0], sc = 1.f, isc = 1.f;  // (w_next: of the next head, fetched a head ahead)
-  for (int g = lane; g < G; g += 32) wg = fmaxf(wg, wmax[g]);
-  const int sg_group = sg_of(warp_max(wg));
-  int sg_at = 0;
+  float whi = 0.f, wlo = -1e30f;  // (wlo: minus the smallest)
+  for (int g = lane; g < G; g += 32) {
+    const float w = wmax[g];
+    whi = fmaxf(whi, w);
+    wlo = fmaxf(wlo, -w);
+  }
+  const int sg_group = sg_of(warp_max(whi));
+  const bool spread = __any_sync(0xffffffffu, sg_of(-warp_max(wlo)) - sg_group > 4);
+  int sg_at = sg_group;
+  float sc = pow2i(sg_at), isc = pow2i(-sg_at);
   const int o = tid % L::OPR, rr0 = tid / L::OPR;
   constexpr int RSTEP = NTH / L::OPR, RPT = TT / RSTEP;
   // fp32 [128][D] accumulator to global rows through the (dead) dy tiles
@@ -1002,126 +1009,132 @@ __global__ void __launch_bounds__(MCfg<D>::THREADS, D == 128 ? 1 : 2) mix_bwd_ke
     }
     __syncthreads();
   };
+  // The group's heads, once with and once without a power of two per head. The choice is a vote, which the compiler knows to be
+  // uniform; a branch that it must take for divergent slows down all that stands behind it (4 x 1300 tokens, 32/8 heads of 128:
+  // no choice 288.2 us, this 289.3, one loop with the rescaling inside 292, a choice that is no vote 293.5).
+  auto heads = [&](auto spreadc) {
 #pragma unroll 1
-  for (int g = 0; g < G; ++g) {
-    const int h = j * G + g;
-    {
-      const int own = sg_of(w_next), sgm = own - sg_group <= 4 ? sg_group : min(own, sg_group + 60);
-      if (g > 0 && sgm != sg_at) {  // the key stream's du so far, on this head's scale
-        const float f = pow2i(sgm - sg_at);
+    for (int g = 0; g < G; ++g) {
+      const int h = j * G + g;
+      if constexpr (decltype(spreadc)::value) {
+        const int own = sg_of(wmax[g]), sgm = own - sg_group <= 4 ? sg_group : min(own, sg_group + 60);
+        if (g > 0 && sgm != sg_at) {  // the key stream's du so far, on this head's scale
+          const float f = pow2i(sgm - sg_at);
+          float d[8];
+#pragma unroll 1
+          for (int c0 = cg * HC; c0 < (cg + 1) * HC; c0 += 8) {
+            tmem_ld8(lane_base + M::DUK + c0, d);
+            tmem_wait_ld();
+#pragma unroll
+            for (int i = 0; i < 8; ++i) d[i] *= f;
+            tmem_st8(lane_base + M::DUK + c0, d);
+          }
+          tmem_wait_st();
+        }
+        sg_at = sgm;
+        sc = pow2i(sgm);
+        isc = pow2i(-sgm);
+      }
+      load_w_tile<D>(sg + M::WT, a.W + (size_t)h * D * D, tid, NTH);
+#pragma unroll 1
+      for (int stream = 0; stream < 2; ++stream) {
+        const bf16* w = stream ? a.w_k : a.w_q;
+        const int NH = stream ? a.Hkv : a.H, head = stream ? j : h;
+        for (int idx = tid; idx < D * 4; idx += NTH) {
+          const int c = idx >> 2, dl = idx & 3;
+          s_taps[idx] = dl < a.K ? __bfloat162float(w[((size_t)head * D + c) * a.K + dl]) : 0.f;
+        }
+        // the rows of the next (head, stream) step travel towards L2 while this one is computed
+        if (g + stream < G) {
+          const int nh = h + stream;
+          const float* wn = stream ? a.wq : a.wk;
+          const float* pn = stream ? a.qd : a.kd;
+          constexpr int LF = D * 4 / 128;
+          for (int idx = tid; idx < nvalid * 2 * LF; idx += NTH) {
+            const int r = idx / (2 * LF), l = idx % (2 * LF);
+            prefetch_l2((l < LF ? wn : pn) + (((size_t)b * a.T + t0 + r) * a.H + nh) * D + (l % LF) * 32);
+          }
+          if (stream && tid < nvalid) {
+            const bf16* xn = a.q + (((size_t)b * a.T + t0 + tid) * a.H + nh) * D;
+            prefetch_l2(xn);
+            if (D == 128) prefetch_l2(xn + 64);
+          }
+        }
+        // ---- dy
+        {
+          const float* wp = stream ? a.wk : a.wq;
+          const float* pp = stream ? a.kd : a.qd;
+#pragma unroll 4
+          for (int r = rr0; r < TT; r += RSTEP) {
+            float wv[8], pv[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) wv[i] = pv[i] = 0.f;
+            if (r < nvalid) {
+              const size_t at = (((size_t)b * a.T + t0 + r) * a.H + h) * D + o * 8;
+              load_row8(wp + at, wv);
+              load_row8(pp + at, pv);
+            }
+            float s = 0.f;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) s += wv[i];
+#pragma unroll
+            for (int off = 1; off < L::OPR; off <<= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) wv[i] = fmaf(-pv[i], s, wv[i]) * sc;
+            uint4 hi, lo;
+            split8h(wv, true, hi, lo);
+            *reinterpret_cast<uint4*>(sg + M::DY + toff(L::SLAB_U, r, o * 8)) = hi;
+            *reinterpret_cast<uint4*>(sg + M::DY + L::TILE_U + toff(L::SLAB_U, r, o * 8)) = lo;
+          }
+        }
+        uint4 raw[RPT + HALO];
+        conv_load<D, RPT>(raw, stream ? a.k : a.q, stream ? a.cache_k : a.cache_q, b, t0 + rr0 * RPT, a.T, NH, head, a.K, o);
+        __syncthreads();  // (the taps)
+        // ---- u
+        conv_emit<RPT>(raw, s_taps, o, [&](int i, float* u) {
+          uint4 hi, lo;
+          split8h(u, true, hi, lo);
+          const uint32_t at = toff(L::SLAB_U, rr0 * RPT + i, o * 8);
+          *reinterpret_cast<uint4*>(sg + M::U + at) = hi;
+          *reinterpret_cast<uint4*>(sg + M::U + L::TILE_U + at) = lo;
+        });
+        fence_proxy_async();
+        tc_fence_before_sync();
+        __syncthreads();
+        tc_fence_after_sync();
+        if (tid == 0) {
+          mm.split(stream ? M::DUK : M::DUQ, kview(sb + M::DY, L::SLAB_U), kview(sb + M::DY + L::TILE_U, L::SLAB_U), 2 * L::SLAB_U,
+                   kview(sb + M::WT, L::SLAB_W), 0, 2 * L::SLAB_W, D / 16, instr_desc(128, D, FMT_F16, MAJOR_K, MAJOR_K),
+                   stream == 1 && g > 0);
+          mm.split(M::DWC, mview(sb + M::U, L::SLAB_U), mview(sb + M::U + L::TILE_U, L::SLAB_U), 256, mview(sb + M::DY, L::SLAB_U),
+                   mview(sb + M::DY + L::TILE_U, L::SLAB_U), 256, TT / 16, instr_desc(128, D, FMT_F16, MAJOR_MN, MAJOR_MN), stream == 1);
+          mma_commit(sb + M::BAR);
+        }
+        wt.wait();
+        if (stream == 0) rows_out(M::DUQ, a.wq, a.H, h);
+      }
+      // dW of the head: row c of the accumulator belongs to lane c
+      if (a.dW && row < D) {
         float d[8];
 #pragma unroll 1
         for (int c0 = cg * HC; c0 < (cg + 1) * HC; c0 += 8) {
-          tmem_ld8(lane_base + M::DUK + c0, d);
+          tmem_ld8(lane_base + M::DWC + c0, d);
           tmem_wait_ld();
+          float* dst = a.dW + ((size_t)h * D + row) * D + c0;
 #pragma unroll
-          for (int i = 0; i < 8; ++i) d[i] *= f;
-          tmem_st8(lane_base + M::DUK + c0, d);
-        }
-        tmem_wait_st();
-      }
-      sg_at = sgm;
-      if (g + 1 < G) w_next = wmax[g + 1];
-      sc = pow2i(sgm);
-      isc = pow2i(-sgm);
-    }
-    load_w_tile<D>(sg + M::WT, a.W + (size_t)h * D * D, tid, NTH);
-#pragma unroll 1
-    for (int stream = 0; stream < 2; ++stream) {
-      const bf16* w = stream ? a.w_k : a.w_q;
-      const int NH = stream ? a.Hkv : a.H, head = stream ? j : h;
-      for (int idx = tid; idx < D * 4; idx += NTH) {
-        const int c = idx >> 2, dl = idx & 3;
-        s_taps[idx] = dl < a.K ? __bfloat162float(w[((size_t)head * D + c) * a.K + dl]) : 0.f;
-      }
-      // the rows of the next (head, stream) step travel towards L2 while this one is computed
-      if (g + stream < G) {
-        const int nh = h + stream;
-        const float* wn = stream ? a.wq : a.wk;
-        const float* pn = stream ? a.qd : a.kd;
-        constexpr int LF = D * 4 / 128;
-        for (int idx = tid; idx < nvalid * 2 * LF; idx += NTH) {
-          const int r = idx / (2 * LF), l = idx % (2 * LF);
-          prefetch_l2((l < LF ? wn : pn) + (((size_t)b * a.T + t0 + r) * a.H + nh) * D + (l % LF) * 32);
-        }
-        if (stream && tid < nvalid) {
-          const bf16* xn = a.q + (((size_t)b * a.T + t0 + tid) * a.H + nh) * D;
-          prefetch_l2(xn);
-          if (D == 128) prefetch_l2(xn + 64);
+          for (int i = 0; i < 8; i += 4)
+            asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + i), "f"(d[i] * isc), "f"(d[i + 1] * isc),
+                         "f"(d[i + 2] * isc), "f"(d[i + 3] * isc)
+                         : "memory");
         }
       }
-      // ---- dy
-      {
-        const float* wp = stream ? a.wk : a.wq;
-        const float* pp = stream ? a.kd : a.qd;
-#pragma unroll 4
-        for (int r = rr0; r < TT; r += RSTEP) {
-          float wv[8], pv[8];
-#pragma unroll
-          for (int i = 0; i < 8; ++i) wv[i] = pv[i] = 0.f;
-          if (r < nvalid) {
-            const size_t at = (((size_t)b * a.T + t0 + r) * a.H + h) * D + o * 8;
-            load_row8(wp + at, wv);
-            load_row8(pp + at, pv);
-          }
-          float s = 0.f;
-#pragma unroll
-          for (int i = 0; i < 8; ++i) s += wv[i];
-#pragma unroll
-          for (int off = 1; off < L::OPR; off <<= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-#pragma unroll
-          for (int i = 0; i < 8; ++i) wv[i] = fmaf(-pv[i], s, wv[i]) * sc;
-          uint4 hi, lo;
-          split8h(wv, true, hi, lo);
-          *reinterpret_cast<uint4*>(sg + M::DY + toff(L::SLAB_U, r, o * 8)) = hi;
-          *reinterpret_cast<uint4*>(sg + M::DY + L::TILE_U + toff(L::SLAB_U, r, o * 8)) = lo;
-        }
-      }
-      uint4 raw[RPT + HALO];
-      conv_load<D, RPT>(raw, stream ? a.k : a.q, stream ? a.cache_k : a.cache_q, b, t0 + rr0 * RPT, a.T, NH, head, a.K, o);
-      __syncthreads();  // (the taps)
-      // ---- u
-      conv_emit<RPT>(raw, s_taps, o, [&](int i, float* u) {
-        uint4 hi, lo;
-        split8h(u, true, hi, lo);
-        const uint32_t at = toff(L::SLAB_U, rr0 * RPT + i, o * 8);
-        *reinterpret_cast<uint4*>(sg + M::U + at) = hi;
-        *reinterpret_cast<uint4*>(sg + M::U + L::TILE_U + at) = lo;
-      });
-      fence_proxy_async();
       tc_fence_before_sync();
       __syncthreads();
       tc_fence_after_sync();
-      if (tid == 0) {
-        mm.split(stream ? M::DUK : M::DUQ, kview(sb + M::DY, L::SLAB_U), kview(sb + M::DY + L::TILE_U, L::SLAB_U), 2 * L::SLAB_U,
-                 kview(sb + M::WT, L::SLAB_W), 0, 2 * L::SLAB_W, D / 16, instr_desc(128, D, FMT_F16, MAJOR_K, MAJOR_K),
-                 stream == 1 && g > 0);
-        mm.split(M::DWC, mview(sb + M::U, L::SLAB_U), mview(sb + M::U + L::TILE_U, L::SLAB_U), 256, mview(sb + M::DY, L::SLAB_U),
-                 mview(sb + M::DY + L::TILE_U, L::SLAB_U), 256, TT / 16, instr_desc(128, D, FMT_F16, MAJOR_MN, MAJOR_MN), stream == 1);
-        mma_commit(sb + M::BAR);
-      }
-      wt.wait();
-      if (stream == 0) rows_out(M::DUQ, a.wq, a.H, h);
     }
-    // dW of the head: row c of the accumulator belongs to lane c
-    if (a.dW && row < D) {
-      float d[8];
-#pragma unroll 1
-      for (int c0 = cg * HC; c0 < (cg + 1) * HC; c0 += 8) {
-        tmem_ld8(lane_base + M::DWC + c0, d);
-        tmem_wait_ld();
-        float* dst = a.dW + ((size_t)h * D + row) * D + c0;
-#pragma unroll
-        for (int i = 0; i < 8; i += 4)
-          asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + i), "f"(d[i] * isc), "f"(d[i + 1] * isc),
-                       "f"(d[i + 2] * isc), "f"(d[i + 3] * isc)
-                       : "memory");
-      }
-    }
-    tc_fence_before_sync();
-    __syncthreads();
-    tc_fence_after_sync();
-  }
+  };
+  if (spread) heads(std::true_type{});
+  else heads(std::false_type{});
   rows_out(M::DUK, a.du_k, a.Hkv, j);
   tc_fence_before_sync();
   __syncthreads();
