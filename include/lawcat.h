@@ -219,7 +219,7 @@ int lawcat_gla_bwd(const lawcat_params* p, const void* qdot, const void* kdot, c
  * chooses the decays and the kernel cannot know them in advance: when a half chunk's accumulated log2-decay exceeds 8 in
  * magnitude (a state that loses about a sixth or more at every token), or a state entry exceeds 3e4, the affected chunks run
  * on 8-bit-mantissa operands, the result is delivered, and dev_status reports LAWCAT_ERR_NUMERIC: the result may miss
- * the tolerance; chunk = 1 has no such limit.
+ * the tolerance; chunk = 1 has no such limit. Its v operand is fp16: |v| above 65504 is out of its range (chunk = 1 again).
  * Asynchronous conditions arrive through dev_status (largest code wins): LAWCAT_ERR_NUMERIC, as above, or a decay
  * exponent within half a chunk left the range +-120 and was clamped; LAWCAT_ERR_TIMEOUT, a bounded device-side wait ran
  * out (the kernel has released its resources and returned; the outputs are undefined).
@@ -263,6 +263,7 @@ int lawcat_layer_fwd_varlen(const lawcat_params* p, const int32_t* cu_seqlens, i
  *   in:  the inputs of lawcat_layer_fwd (caches and initial state nullable) and dO
  *   out: dq [B,T,H,d_k], dk [B,T,H_kv,d_k], dv [B,T,H_kv,d_v], dgate [B,T,H,gate_dim] in p->dtype;
  *        dw_q, dw_k, dW in fp32, shaped like w_q, w_k, W, overwritten. All outputs are required.
+ * v and dO may have any size: the tensor-core path scales its 16-bit operands per chunk, per head and per group of heads.
  * No gradient flows into the conv caches or the initial state.
  */
 int lawcat_layer_bwd(const lawcat_params* p, const void* q, const void* k, const void* v, const void* gate,

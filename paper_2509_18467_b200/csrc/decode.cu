@@ -743,9 +743,9 @@ __global__ void __launch_bounds__(DEC_THREADS) decode_one_kernel(const DecodeArg
 // next sequence while the other passes over the tile of this one in shared memory, and tiles travel as bulk copies: two on
 // their way in and one on its way out at any time. W_h stays in registers; the small inputs are fetched two sequences ahead,
 // because they queue behind the tiles (any head per block, W_h read again for each and inputs one ahead: 49.8 us at B = 64,
-// d = 128). decode_one -> this, 32 heads, us per step:
-//   d = 64:  B = 24 10.0 -> 8.1    B = 32 10.5 -> 9.4    B = 64 22.1 -> 15.5
-//   d = 128: B = 12 13.5 -> 12.3   B = 16 16.7 -> 16.2   B = 32 31.8 -> 27.9   B = 64 59.1 -> 48.4 (268 MB of state: 5.5 TB/s)
+// d = 128). decode_one -> this, 32 heads, us per step, states from memory (several sets in turn):
+//   d = 64:  B = 20 9.9 -> 8.6     B = 32 12.1 -> 11.0   B = 64 22.0 -> 15.8
+//   d = 128: B = 16 17.0 -> 17.5   B = 20 21.6 -> 20.0   B = 32 31.7 -> 27.5   B = 64 59.8 -> 47.9 (268 MB of state: 5.6 TB/s)
 // The key stream's cache has readers in several blocks: key_cache_shift_kernel moves it when this kernel is over.
 // Feature threads: 2 D (thread = (stream, channel) for conv and phi; (row group, output octet) for the mix). State threads: 2 D
 // (thread = (row group of 8, column quad)). For d = 64 three blocks share an SM.
@@ -1016,7 +1016,13 @@ static bool decode_one_supported(const lawcat_params& p) {
 
 // More heads than decode_one blocks run at once (2 per SM for d = 128, 4 for d = 64): up to there its single round is the
 // shorter chain (B = 8, d = 128: 7.3 us against 9.0; B = 16, d = 64: 6.0 against 6.7). Groups that decode_one does not take come
-// here whatever their number (24 heads in groups of 3: 11.6 us as two launches, 6.2 here, d = 128, B = 1). Every query head needs a block at once.
+// here whatever their number (24 heads in groups of 3: 11.6 us as two launches, 6.2 here, d = 128, B = 1). Every query head
+// needs a block at once. Both sides over 32 to 148 heads, groups of 2 and 4, states from memory, us (decode_one / this):
+//   d = 64: this ahead by 8 to 61 % everywhere.
+//   d = 128: level or up to 12 % behind between 2 and about 4 (sequence, head) pairs per SM (32 heads, B = 16: 17.0 / 17.5; 80
+//   heads, B = 6: 16.8 / 19.0), ahead by 5 to 32 % from there on (32 heads, B = 32: 31.7 / 27.5; 144 heads, B = 64: 254 / 202).
+//   With 75 to 85 heads, where a head gets one block and up to half of the SMs none, only level from there on (76 heads,
+//   B = 8: 21.3 / 22.7, B = 32: 69.8 / 69.8, B = 64: 134.4 / 132.6).
 static bool decode_stream_supported(const lawcat_params& p) {
   const int sms = sm_count();
   if (!decode_tc_supported(p) || p.d_v != p.d_k || p.H > sms) return false;

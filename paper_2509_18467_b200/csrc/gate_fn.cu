@@ -535,9 +535,10 @@ static int launch_tc(const Ctx& c, int d_model, const void* x, const void* A1, c
   ysplit = std::min(ysplit, ntile_all);
   ysplit = (ntile_all + ((ntile_all + ysplit - 1) / ysplit) - 1) / ((ntile_all + ysplit - 1) / ysplit);  // (no empty block)
   // With one block per tile the tiles come in whole rounds of the blocks that fit: 32768 tokens are 256 tiles of 128, which
-  // leave 40 SMs with one block where the others have two, or 293 tiles of 112 (114.2 -> 112.5 us at rank 32 and the 7B widths;
-  // 26000 tokens 103 -> 99.7, rank 16 92.2 -> 84.9; rank 64, one block per SM, 19000 tokens 136 -> 129.6). Not when the only round is hardly more than half full: blocks of half the
-  // height read A1 and A2 twice as often (19000 tokens, rank 32: 87.9 -> 89.7).
+  // leave 40 SMs with one block where the others have two, or 293 tiles of 112. Tiles of 128 -> this, 7B widths, medians of
+  // nine alternating runs whose ranges do not overlap: rank 32, 26000 tokens 101.9 -> 98.7 us, 32768 110.4 -> 108.5, 50000
+  // 195.6 -> 184.9; rank 16, 26000 90.2 -> 83.1; rank 64 (one block per SM), 19000 133.8 -> 127.7. Not when the only round is
+  // hardly more than half full: blocks of half the height read A1 and A2 twice as often (19000 tokens, rank 32: 86.1 -> 87.8).
   int tt = TT;
   const size_t slots = (tiles + room - 1) / room * room;
   if (ysplit == 1 && (tiles > (size_t)room || tiles * 20 > slots * 11)) {
