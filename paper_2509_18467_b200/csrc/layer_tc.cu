@@ -4,6 +4,7 @@
 #include <mutex>
 #include <vector>
 
+#include "layer_state_kernel.cuh"
 #include "layer_tc_kernel.cuh"
 
 namespace lawcat {
@@ -149,8 +150,10 @@ struct TcPlan {
 
 // Segments per sequence: enough thread blocks to fill the SMs (one block per SM), but at least MIN_SEG_CHUNKS chunks per
 // segment (a thread block spends about three chunk times on its set-up and on filling its pipeline). Pieces per segment
-// in the state-only pre-pass: its thread blocks are independent, so cutting the segments finer lets them fill the SMs in
-// whole waves; the split with the fewest chunks per SM wins (a small charge per extra piece).
+// in the state-only pre-pass: its thread blocks are independent, so cutting the segments finer lets them fill the SMs, two to
+// an SM, in whole waves; the split with the fewest chunks per SM wins (a set-up is two chunk times). Measured over 1 to 8 pieces:
+// 32768 tokens, 32 heads of 128: 460 us as one piece, 337, 232 as three (96 blocks each), 275 as four, 237 as six; 1223 tokens
+// (five chunks a segment): the call 66.6 us, 67.8, 64.6 as three, 73.8 as four.
 // Two 64-wide heads share a thread block when they can: an even number of query heads per key/value head (the two heads
 // of a block read the same k and v) and one decay per key channel.
 static bool layer_tc_paired(const lawcat_params& p) {
@@ -171,9 +174,9 @@ static TcPlan layer_tc_plan(const lawcat_params& p) {
   if (pl.nseg < 1) pl.nseg = 1;
   const int cps = pl.seg_len / tc::C;
   int best = 1, best_cost = 1 << 30;
-  for (int ns = 1; ns <= 8 && ns * 4 <= cps; ++ns) {
+  for (int ns = 1; ns <= 8 && ns * 2 <= cps + 1; ++ns) {
     const int ctas = seqs * (pl.nseg - 1) * ns;
-    const int cost = ((ctas + sms - 1) / sms) * ((cps + ns - 1) / ns + 2);
+    const int cost = ((ctas + 2 * sms - 1) / (2 * sms)) * ((cps + ns - 1) / ns + 2);
     if (cost < best_cost) { best_cost = cost; best = ns; }
   }
   pl.nsub = best;
@@ -316,7 +319,7 @@ static int run_layer_tc(const Ctx& c, const void* q, const void* k, const void* 
   a.nsub = 1;
   a.S0 = S0; a.z0 = z0; a.S_T = S_T; a.z_T = z_T;
   auto* const k_layer = paired ? layer_tc_kernel<0, 2> : dh == 64 ? layer_tc_kernel<0, 1> : layer_tc_kernel<0, 0>;
-  auto* const k_state = paired ? layer_tc_kernel<1, 2> : dh == 64 ? layer_tc_kernel<1, 1> : layer_tc_kernel<1, 0>;
+  auto* const k_state = paired ? st::layer_state_kernel<2> : dh == 64 ? st::layer_state_kernel<1> : st::layer_state_kernel<0>;
   const int threads = threads_of(paired ? 2 : dh == 64 ? 1 : 0);
   {
     // the kernels' shared-memory limit is raised once per device
@@ -329,9 +332,9 @@ static int run_layer_tc(const Ctx& c, const void* q, const void* k, const void* 
       if (cudaFuncSetAttribute(layer_tc_kernel<0, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_ALLOC) != cudaSuccess ||
           cudaFuncSetAttribute(layer_tc_kernel<0, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_ALLOC) != cudaSuccess ||
           cudaFuncSetAttribute(layer_tc_kernel<0, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_ALLOC) != cudaSuccess ||
-          cudaFuncSetAttribute(layer_tc_kernel<1, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_ALLOC) != cudaSuccess ||
-          cudaFuncSetAttribute(layer_tc_kernel<1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_ALLOC) != cudaSuccess ||
-          cudaFuncSetAttribute(layer_tc_kernel<1, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_ALLOC) != cudaSuccess)
+          cudaFuncSetAttribute(st::layer_state_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)st::SMEM_BYTES) != cudaSuccess ||
+          cudaFuncSetAttribute(st::layer_state_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)st::SMEM_BYTES) != cudaSuccess ||
+          cudaFuncSetAttribute(st::layer_state_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)st::SMEM_BYTES) != cudaSuccess)
         return LAWCAT_ERR_CUDA;
       done[dev] = true;
     }
@@ -356,7 +359,7 @@ static int run_layer_tc(const Ctx& c, const void* q, const void* k, const void* 
     TcArgs b1 = a;
     b1.S_T = loc_S; b1.z_T = loc_z; b1.dtot = dtot; b1.nsub = nsub;
     LaunchScope _ls("layer_tc_state", c.stream);
-    launch_behind(k_state, dim3(Hn * (segs - nseq) * nsub), dim3(threads), SMEM_ALLOC, c.stream, tq, tk, tv, tg, b1, tab);
+    launch_behind(k_state, dim3(Hn * (segs - nseq) * nsub), dim3(st::THREADS), st::SMEM_BYTES, c.stream, tk, tv, tg, b1, tab);
     LAWCAT_CHECK_LAUNCH();
   }
   cudaLaunchAttribute at[1];
