@@ -318,7 +318,7 @@ static int run_layer_tc(const Ctx& c, const void* q, const void* k, const void* 
   a.seg_len = pl.seg_len;
   a.nsub = 1;
   a.S0 = S0; a.z0 = z0; a.S_T = S_T; a.z_T = z_T;
-  auto* const k_layer = paired ? layer_tc_kernel<0, 2> : dh == 64 ? layer_tc_kernel<0, 1> : layer_tc_kernel<0, 0>;
+  auto* const k_layer = paired ? layer_tc_kernel<2> : dh == 64 ? layer_tc_kernel<1> : layer_tc_kernel<0>;
   auto* const k_state = paired ? st::layer_state_kernel<2> : dh == 64 ? st::layer_state_kernel<1> : st::layer_state_kernel<0>;
   const int threads = threads_of(paired ? 2 : dh == 64 ? 1 : 0);
   {
@@ -329,9 +329,9 @@ static int run_layer_tc(const Ctx& c, const void* q, const void* k, const void* 
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return LAWCAT_ERR_CUDA;
     std::lock_guard<std::mutex> lk(mu);
     if (!done[dev]) {
-      if (cudaFuncSetAttribute(layer_tc_kernel<0, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_ALLOC) != cudaSuccess ||
-          cudaFuncSetAttribute(layer_tc_kernel<0, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_ALLOC) != cudaSuccess ||
-          cudaFuncSetAttribute(layer_tc_kernel<0, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_ALLOC) != cudaSuccess ||
+      if (cudaFuncSetAttribute(layer_tc_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_ALLOC) != cudaSuccess ||
+          cudaFuncSetAttribute(layer_tc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_ALLOC) != cudaSuccess ||
+          cudaFuncSetAttribute(layer_tc_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_ALLOC) != cudaSuccess ||
           cudaFuncSetAttribute(st::layer_state_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)st::SMEM_BYTES) != cudaSuccess ||
           cudaFuncSetAttribute(st::layer_state_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)st::SMEM_BYTES) != cudaSuccess ||
           cudaFuncSetAttribute(st::layer_state_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)st::SMEM_BYTES) != cudaSuccess)

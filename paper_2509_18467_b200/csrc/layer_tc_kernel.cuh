@@ -51,9 +51,6 @@ namespace tc {
 // Optional time line (profiling builds only, -DLAWCAT_TIMELINE): one lane per role of thread block 0 stamps the clock at
 // fixed points of four consecutive chunks into a device array that lawcat_timeline_read copies out.
 #ifdef LAWCAT_TIMELINE
-#ifndef LAWCAT_TIMELINE_MODE
-#define LAWCAT_TIMELINE_MODE 0   // which kernel mode stamps: 0 the layer, 1 the state-only pass
-#endif
 #ifndef LAWCAT_TIMELINE_N0
 #define LAWCAT_TIMELINE_N0 40    // first of the four chunks that stamp
 #endif
@@ -64,7 +61,7 @@ constexpr int TL_ROLES = 6, TL_IDS = 16, TL_N0 = LAWCAT_TIMELINE_N0, TL_NCH = 4;
 __device__ long long g_timeline[TL_ROLES * TL_IDS * TL_NCH];
 #define TL(role, id, n, who)                                                                        \
   do {                                                                                              \
-    if (MODE == LAWCAT_TIMELINE_MODE && blockIdx.x == 0 && (who) && (n) >= TL_N0 && (n) < TL_N0 + TL_NCH) \
+    if (blockIdx.x == 0 && (who) && (n) >= TL_N0 && (n) < TL_N0 + TL_NCH) \
       g_timeline[((role) * TL_IDS + (id)) * TL_NCH + ((n) - TL_N0)] = clock64();                    \
   } while (0)
 #else
@@ -180,15 +177,15 @@ struct TcArgs {
                          // zeroed once and never loaded, and the feature map leaves the padded outputs out
   const bf16 *w_q, *w_k, *W, *cache_q, *cache_k;
   const float *S0, *z0;  // [seq,H,..]: state in front of each sequence (nullable: zero)
-  const float *seg_S, *seg_z;  // (MODE 0) [segment,H,..]: state in front of every segment but a sequence's first
-  float *S_T, *z_T;      // MODE 0: [seq,H,..] state after the last token; MODE 1: [segment piece,H,..] state of the piece
-  float* dtot;           // (MODE 1) [segment piece,H,128]: log2 of the total decay of the piece per key channel
+  const float *seg_S, *seg_z;  // [segment,H,..]: state in front of every segment but a sequence's first
+  float *S_T, *z_T;      // [seq,H,..] state after the last token; state-only pass: [segment piece,H,..] state of the piece
+  float* dtot;           // (state-only pass) [segment piece,H,dh]: log2 of the total decay of the piece per key channel
   bf16* o;               // [B,T,H,128]
   bf16 *cache_q_out, *cache_k_out;  // conv caches after the last token (nullable): [B,K-1,H*dh], [B,K-1,Hkv*dh]
   int* dev_status;
   int T, H, Hkv, K;
   int nseg, seg_len;     // uniform batch: segments per sequence and tokens per segment (a multiple of C)
-  int nsub;              // MODE 1: pieces each segment is cut into (whole chunks); MODE 0: 1
+  int nsub;              // (state-only pass) pieces each segment is cut into (whole chunks)
   int gate_mode;
   int normalize;         // 1: Eq. 8; 0: the numerator alone (the query features then carry their softmax normalizer)
   float inv_tau, eps;
@@ -196,7 +193,7 @@ struct TcArgs {
 };
 
 // The sequence that block `blk` of a launch works on, with `per_seg` blocks per segment and `skip` segments of each sequence
-// left out (MODE 1 leaves out the last); blk becomes the block's index inside the sequence.
+// left out (the state-only pass leaves out the last); blk becomes the block's index inside the sequence.
 __device__ __forceinline__ SeqView seq_of_block(const TcArgs& a, const PackTab& tab, int per_seg, int skip, int& blk) {
   SeqView v;
   if (tab.n == 0) {
@@ -320,11 +317,9 @@ __device__ __forceinline__ bool wait_set_or_abort(uint32_t bar0, uint32_t mask, 
   }
 }
 
-// MODE 0: the layer forward. MODE 1: state only (no query stream, no output): the end state of a segment that starts
-// from the given state, used to hand the state across segments of one sequence.
 // WIDTH: 0 = heads of 128 channels; 1 = one head of 64 channels per block (padded to 128); 2 = two 64-wide heads of one
 // key/value group per block. A compile-time switch, so that the 128-wide kernel carries none of the others' tests.
-template <int MODE, int WIDTH>
+template <int WIDTH>
 __global__ void __launch_bounds__(threads_of(WIDTH), 1)
 layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                 const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_g, const TcArgs a,
@@ -359,28 +354,23 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   constexpr uint32_t cS = COL_S, cSZ = pair ? 192u : COL_SZ, cO = pair ? 208u : COL_O, cO2 = 288u;
   constexpr uint32_t cP = pair ? 368u : COL_P, cP2 = 432u, cMAIL = pair ? 496u : COL_MAIL;
   const int Hn = pair ? a.H / 2 : a.H;   // heads as addressed (units of dh channels)
-  // blocks of a sequence: head (outer), segment, piece
+  // blocks of a sequence: head (outer), segment
   int blk = blockIdx.x;
-  const SeqView sq = seq_of_block(a, tab, Hn * a.nsub, MODE == 1 ? 1 : 0, blk);
-  const int segs_run = sq.nseg - (MODE == 1 ? 1 : 0);
-  const int sub = blk % a.nsub;
-  const int seg = (blk / a.nsub) % segs_run;
-  const int h = blk / (a.nsub * segs_run), b = sq.seq, T = sq.T;
+  const SeqView sq = seq_of_block(a, tab, Hn, 0, blk);
+  const int seg = blk % sq.nseg, h = blk / sq.nseg, b = sq.seq, T = sq.T;
   const int h0 = pair ? 2 * h : h;       // first real head of this block
   const int G = a.H / a.Hkv, j = h0 / G;
-  const int cps = sq.seg_len / C;  // chunks per segment; piece `sub` covers chunks [sub cps / nsub, (sub + 1) cps / nsub)
-  const int t_begin = min(T, seg * sq.seg_len + (sub * cps / a.nsub) * C);
-  const int t_end = min(T, seg * sq.seg_len + ((sub + 1) * cps / a.nsub) * C);
+  const int t_begin = min(T, seg * sq.seg_len), t_end = min(T, t_begin + sq.seg_len);
   const int nchunks = max(0, (t_end - t_begin + C - 1) / C);
   // The last chunk of a packed sequence: behind its last token the tiles hold the next sequence's first tokens, which a factor
   // of zero further on would not keep out where they are not finite. (Elsewhere the copies fill rows past the end with zeros.)
   const int last_valid = t_end - t_begin - (nchunks - 1) * C;
-  const bool mixed = MODE == 0 && tab.n != 0 && nchunks > 0 && last_valid < C;
+  const bool mixed = tab.n != 0 && nchunks > 0 && last_valid < C;
   // index of the state of the real head that owns state row c (rows 64-127 of a pair: the second head): among the caller's
   // states (one per sequence), or among the workspace's (one per segment piece)
   auto head_of_row = [&](int c) -> size_t { return h0 + (pair ? (c >> 6) : 0); };
   auto seq_state = [&](int c) -> size_t { return (size_t)b * a.H + head_of_row(c); };
-  auto seg_state = [&](int c) -> size_t { return ((size_t)(sq.seg0 + seg) * a.nsub + sub) * a.H + head_of_row(c); };
+  auto seg_state = [&](int c) -> size_t { return ((size_t)(sq.seg0 + seg)) * a.H + head_of_row(c); };
 
   if ((sb & 1023u) != 0) {  // the swizzled tiles need a 1024-byte aligned base
     if (tid == 0 && a.dev_status) atomicMax(a.dev_status, (int)LAWCAT_ERR_CUDA);
@@ -388,17 +378,16 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   }
 
   // ---- one-time setup --------------------------------------------------------------------------------------------
-  if (MODE == 1) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // (the scan may be scheduled behind)
   asm volatile("griddepcontrol.wait;" ::: "memory");  // (launched behind the kernel in front on the stream)
   // Three groups of warps prepare side by side, with all their loads in flight before the first is used: a block of a short
   // sequence spent a third of its time here, most of it in loads that waited for one another (given states 18k cycles, now
   // 2k; W 2k; the first tiles were asked for 3k cycles after the rest).
   const int tt_first = sq.tm_t + t_begin;  // (token coordinate of the first chunk in the tensor maps)
   auto load_raw = [&](int tt0, int full) {
-    mbar_arrive_expect_tx(bar(full), (MODE == 0 ? 16384u : 8192u) * (uint32_t)nslab);
+    mbar_arrive_expect_tx(bar(full), 16384u * (uint32_t)nslab);
 #pragma unroll 1
     for (int s = 0; s < nslab; ++s) {
-      if (MODE == 0) tma_load_4d(sb + OFF_AU + s * 16384, &tm_q, bar(full), s * 64, h, tt0, sq.tm_b);
+      tma_load_4d(sb + OFF_AU + s * 16384, &tm_q, bar(full), s * 64, h, tt0, sq.tm_b);
       // (pair: the same 64 key channels into both halves of the tile)
       tma_load_4d(sb + OFF_AU + s * 16384 + 8192, &tm_k, bar(full), pair ? 0 : s * 64, j, tt0, sq.tm_b);
     }
@@ -424,11 +413,10 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   const uint32_t rw_stage = sb + (pair ? OFF_QK + (uint32_t)rw * 4096u : (rw < 4 ? OFF_QK : OFF_SBF) + (uint32_t)(rw & 3) * 8192u);
   auto stage_at = [&](int r, int unit) -> uint32_t { return rw_stage + (uint32_t)(r * NC * 4 + ((unit ^ (r & 7)) << 4)); };
   const bool first = seg == 0;  // a sequence's first segment starts from the caller's state, the others from the scan's
-  const float* const srcS = MODE == 1 ? nullptr : first ? a.S0 : a.seg_S;
-  const float* const srcz = MODE == 1 ? nullptr : first ? a.z0 : a.seg_z;
+  const float* const srcS = first ? a.S0 : a.seg_S;
+  const float* const srcz = first ? a.z0 : a.seg_z;
   if (warp == TMA_WARP) {
     if (lane == 0) {
-      const int nphi = MODE == 0 ? 256 : 128;  // threads of the phi pass: all row threads, or the key rows only
       mbar_init(bar(B_RAW_FULL), 1);
       mbar_init(bar(B_G_FULL), 1);
       mbar_init(bar(B_V_FULL), 1);
@@ -437,9 +425,9 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       mbar_init(bar(B_X_FULL), PREP_THREADS);
       mbar_init(bar(B_VH_FULL), PREP_THREADS);
       mbar_init(bar(B_MMA1), 1);
-      mbar_init(bar(B_Y_FREE), nphi);
-      mbar_init(bar(B_X_FREE), 256);  // every row thread: it reads bm, ft and (phi threads) the exponents
-      mbar_init(bar(B_QK_FULL), nphi);
+      mbar_init(bar(B_Y_FREE), 256);
+      mbar_init(bar(B_X_FREE), 256);
+      mbar_init(bar(B_QK_FULL), 256);
       mbar_init(bar(B_SBF_FULL), 256);
       mbar_init(bar(B_P), 1);
       mbar_init(bar(B_MMA2), 1);
@@ -565,7 +553,7 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
           load_gate(tt0);
           ar_g = n;
         }
-        WAIT(MODE == 0 ? B_MMA3 : B_MMA2, pp);  // the last MMA that reads v
+        WAIT(B_MMA3, pp);  // the last MMA that reads v
         load_v(tt0, B_V_FULL);
         ar_v = n;
       }
@@ -623,7 +611,7 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     // First, while the operands of the first chunk are made, the conv caches after the last token (Section 4.1: the last K - 1
     // raw rows of [cache_in, x]): they depend on the raw inputs alone, so the block of a head's last segment writes them
     // (the key stream by the first head of a group).
-    if (MODE == 0 && seg == sq.nseg - 1 && sub == 0 && a.K > 1) {
+    if (seg == sq.nseg - 1 && a.K > 1) {
       const int per = (a.K - 1) * (dh / 8);  // 16-byte units per stream (the key stream of a pair uses the first hd / 8 per row)
       for (int idx = lane; idx < 2 * per; idx += 32) {
         const int st = idx / per, r = (idx % per) / (dh / 8), oc = idx % (dh / 8);
@@ -680,12 +668,12 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       }
       for (int n = 0; ok && n < nchunks; ++n) {
         const uint32_t p = (uint32_t)(n & 1), pp = p ^ 1u;
-        WAITSET(BIT(B_QK_FULL) | BIT(B_SBF_FULL) | BIT(B_VH_FULL) | (MODE == 0 && n > 0 ? BIT(B_O_FREE) : 0u),
+        WAITSET(BIT(B_QK_FULL) | BIT(B_SBF_FULL) | BIT(B_VH_FULL) | (n > 0 ? BIT(B_O_FREE) : 0u),
                 PAR(B_QK_FULL, p) | PAR(B_SBF_FULL, p) | PAR(B_VH_FULL, p) | PAR(B_O_FREE, pp));
         TL(0, 0, n, lane == 0);
         const bool f16 = __int_as_float(s_rmax[p]) <= RMAX_F16 && __int_as_float(s_sbound[p]) < SMAX_F16;
         const int fmt = f16 ? FMT_F16 : FMT_BF16;
-        if (MODE == 0 && lane == 0) {
+        if (lane == 0) {
           // the scores first: their mask pass is the longest chain behind this hand-over
           tc_fence_after_sync();
           // (pair: channels 0-63 give the first head's scores, channels 64-127 the second head's, in accumulators of their own)
@@ -709,16 +697,14 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         TL(0, 2, n, lane == 0);
         if (lane == 0) {
           tc_fence_after_sync();
-          if (MODE == 0) {
-            // read-out O' | denominator = qs [2^b_mid S | 2^b_mid z] in one product per K step
-            // (pair: the first head's read-out contracts channels 0-63 with state rows 0-63, the second head's the rest)
-            const uint32_t ID_O = instr_desc(128, NV + 16, fmt, MAJOR_K, MAJOR_MN);
+          // read-out O' | denominator = qs [2^b_mid S | 2^b_mid z] in one product per K step
+          // (pair: the first head's read-out contracts channels 0-63 with state rows 0-63, the second head's the rest)
+          const uint32_t ID_O = instr_desc(128, NV + 16, fmt, MAJOR_K, MAJOR_MN);
 #pragma unroll
-            for (int k = 0; k < 8; ++k)
-              if (k < ksteps)
-                mma_f16(tmem + ((pair && k >= 4) ? cO2 : cO), adv(dsc_qk, kstep(k)), adv(dsc_s, k * (256 >> 4)), ID_O,
-                        pair ? (k & 3) > 0 : k > 0);
-          }
+          for (int k = 0; k < 8; ++k)
+            if (k < ksteps)
+              mma_f16(tmem + ((pair && k >= 4) ? cO2 : cO), adv(dsc_qk, kstep(k)), adv(dsc_s, k * (256 >> 4)), ID_O,
+                      pair ? (k & 3) > 0 : k > 0);
           const uint32_t ID_S = instr_desc(128, NV, FMT_F16, MAJOR_MN, MAJOR_MN);
           constexpr uint32_t ID_SZ = instr_desc(128, 16, FMT_F16, MAJOR_MN, MAJOR_MN);
 #pragma unroll
@@ -730,25 +716,23 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
           mma_commit(bar(B_MMA2));
         }
         TL(0, 3, n, lane == 0);
-        if (MODE == 0) {
-          WAITSET(BIT(B_PH_FULL), PAR(B_PH_FULL, p));
-          TL(0, 4, n, lane == 0);
-          if (lane == 0) {
-            // O' += P v  (the scores' part of the denominator is summed by the mask pass)
-            tc_fence_after_sync();
-            const uint32_t ID_O = instr_desc(128, NV, FMT_F16, MAJOR_K, MAJOR_MN);
+        WAITSET(BIT(B_PH_FULL), PAR(B_PH_FULL, p));
+        TL(0, 4, n, lane == 0);
+        if (lane == 0) {
+          // O' += P v  (the scores' part of the denominator is summed by the mask pass)
+          tc_fence_after_sync();
+          const uint32_t ID_O = instr_desc(128, NV, FMT_F16, MAJOR_K, MAJOR_MN);
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            mma_f16(tmem + cO, adv(dsc_p, k * 2), adv(dsc_v, k * (2048 >> 4)), ID_O, 1);
+          if (pair) {
 #pragma unroll
             for (int k = 0; k < 4; ++k)
-              mma_f16(tmem + cO, adv(dsc_p, k * 2), adv(dsc_v, k * (2048 >> 4)), ID_O, 1);
-            if (pair) {
-#pragma unroll
-              for (int k = 0; k < 4; ++k)
-                mma_f16(tmem + cO2, adv(dsc_p2, k * 2), adv(dsc_v, k * (2048 >> 4)), ID_O, 1);
-            }
-            mma_commit(bar(B_MMA3));
+              mma_f16(tmem + cO2, adv(dsc_p2, k * 2), adv(dsc_v, k * (2048 >> 4)), ID_O, 1);
           }
-          TL(0, 5, n, lane == 0);
+          mma_commit(bar(B_MMA3));
         }
+        TL(0, 5, n, lane == 0);
       }
     }
   } else if (mixw && warp == MIX_WARP) {
@@ -774,7 +758,7 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     // ================================================================================================ prep warps
     // conv mapping: thread = (stream, channel octet, 8 consecutive tokens); gate mapping: thread = (channel, half chunk)
     const int cv_stream = tid >> 7, cv_oct = tid & 15, cv_rg = (tid >> 4) & 7;
-    const bool cv_on = (MODE == 0 || cv_stream == 1) && cv_oct * 8 < dh;
+    const bool cv_on = cv_oct * 8 < dh;
     uint64_t cw[4][4];  // [channel pair][tap], packed pairs of fp32
     {
       const bf16* w = cv_stream ? a.w_k : a.w_q;
@@ -977,7 +961,7 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       TL(warp == 0 ? 3 : 4, 5, n, (warp == 0 || warp == 2) && lane == 0);
 
       // ---- output of the previous chunk (its last product completes about now; the v tile is loaded after it) -----------
-      if (MODE == 0 && n > 0) {
+      if (n > 0) {
         WAITF(B_MMA3, pp);
         TL(warp == 0 ? 3 : 4, 6, n, (warp == 0 || warp == 2) && lane == 0);
         if (!fail) out_pass(n - 1);
@@ -987,10 +971,10 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       // ---- v: bf16 -> fp16 in place (exact for |v| in the fp16 normal range) ------------------------------------------
       WAITF(B_V_FULL, p);
       TL(warp == 0 ? 3 : 4, 8, n, (warp == 0 || warp == 2) && lane == 0);
-      // (layer mode: by the warps of TMEM quadrants 2-3 only; those of quadrants 0-1 carry the output pass)
-      if (!fail && (MODE == 1 || (warp & 3) >= 2)) {
-        const int vthreads = MODE == 1 ? PREP_THREADS : PREP_THREADS / 2;
-        const int vt = MODE == 1 ? tid : (tid >> 7) * 64 + ((warp & 3) - 2) * 32 + lane;
+      // (by the warps of TMEM quadrants 2-3 only; those of quadrants 0-1 carry the output pass)
+      if (!fail && (warp & 3) >= 2) {
+        constexpr int vthreads = PREP_THREADS / 2;
+        const int vt = (tid >> 7) * 64 + ((warp & 3) - 2) * 32 + lane;
         float vm = 0.f;
 #pragma unroll 2
         for (int i = 0; i < vslab * 512 / vthreads; ++i) {
@@ -1008,7 +992,7 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       mbar_arrive(bar(B_VH_FULL));
       TL(warp == 0 ? 3 : 4, 9, n, (warp == 0 || warp == 2) && lane == 0);
     }
-    if (MODE == 0 && nchunks > 0 && !fail && !*s_abort &&
+    if (nchunks > 0 && !fail && !*s_abort &&
         wait_or_abort(bar(B_MMA3), (uint32_t)((nchunks - 1) & 1), s_abort, a.wait_limit))
       out_pass(nchunks - 1);
   } else {
@@ -1053,7 +1037,6 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     const int r128 = (tw & 127);                  // row of Y and of the state (= TMEM lane)
     const bool is_q = r128 < C;
     const int row = is_q ? r128 : r128 - C;       // token inside the chunk
-    const bool phi_on = MODE == 0 || !is_q;       // the state-only pass has no query rows
     const bool padded = ch >= nslab;              // this thread's 64 columns are the zero padding of a 64-wide head
     const int phi_bar = is_q ? 3 : 4;             // the query rows and the key rows meet among themselves (128 threads each)
     const float L2E = 1.4426950408889634f;
@@ -1061,7 +1044,6 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     const bool need_qsum = a.eps != 0.f || !a.normalize;
     const uint32_t mail_mine = lane_base + cMAIL + 2 + ch, mail_other = lane_base + cMAIL + 2 + (ch ^ 1);
     const uint32_t ycol = lane_base + COL_Y + ch * 64;
-    float dsum = 0.f;  // log2 of this state row's total decay over the segment
     bool fail = false;
     // ---- causal mask of chunk m, fp16 scores: this (query-row) thread's 32 columns of row `row`. It runs behind the
     // reading sweeps of chunk m + 1, which do not have to wait for MMA 2 of chunk m.
@@ -1108,70 +1090,68 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       TL(warp == 8 ? 1 : 2, 0, n, (warp == 8 || warp == 10) && lane == 0);
       // ---- mask of the previous chunk: its scores are the first product issued after the hand-over, ahead of this
       // chunk's mix ---------------------------------------------------------------------------------------------------
-      if (MODE == 0 && is_q && n > 0) mask_chunk(n - 1);
+      if (is_q && n > 0) mask_chunk(n - 1);
       TL(warp == 8 ? 1 : 2, 1, n, (warp == 8 || warp == 10) && lane == 0);
       // ---- phi, reading sweeps ----------------------------------------------------------------------------------------
-      if (phi_on) {
-        WAITF(B_MMA1, p);
-        fail = __any_sync(0xffffffffu, fail);  // (the collective waits below need the whole warp)
-        TL(warp == 8 ? 1 : 2, 2, n, (warp == 8 || warp == 10) && lane == 0);
-        tc_fence_after_sync();
-        float m = -INFINITY;
-        // (64-wide head: the threads of the upper 64 columns have no outputs: they skip every sweep, and the two threads
-        // of a row have nothing to exchange)
-        if (!fail && !padded) {
-          tmem_ld16(ycol, ya);  // 16 columns at a time, the next load in flight while a block is processed
+      WAITF(B_MMA1, p);
+      fail = __any_sync(0xffffffffu, fail);  // (the collective waits below need the whole warp)
+      TL(warp == 8 ? 1 : 2, 2, n, (warp == 8 || warp == 10) && lane == 0);
+      tc_fence_after_sync();
+      float m = -INFINITY;
+      // (64-wide head: the threads of the upper 64 columns have no outputs: they skip every sweep, and the two threads
+      // of a row have nothing to exchange)
+      if (!fail && !padded) {
+        tmem_ld16(ycol, ya);  // 16 columns at a time, the next load in flight while a block is processed
 #pragma unroll 1
-          for (int b2 = 0; b2 < 2; ++b2) {
-            tmem_wait_ld();
-            tmem_ld16(ycol + b2 * 32 + 16, yb);
+        for (int b2 = 0; b2 < 2; ++b2) {
+          tmem_wait_ld();
+          tmem_ld16(ycol + b2 * 32 + 16, yb);
 #pragma unroll
-            for (int i = 0; i < 16; ++i) m = fmaxf(m, ya[i]);
-            tmem_wait_ld();
-            tmem_ld16(ycol + ((b2 * 32 + 32) & 63), ya);  // wraps to the first block: the next sweep starts there
+          for (int i = 0; i < 16; ++i) m = fmaxf(m, ya[i]);
+          tmem_wait_ld();
+          tmem_ld16(ycol + ((b2 * 32 + 32) & 63), ya);  // wraps to the first block: the next sweep starts there
 #pragma unroll
-            for (int i = 0; i < 16; ++i) m = fmaxf(m, yb[i]);
+          for (int i = 0; i < 16; ++i) m = fmaxf(m, yb[i]);
+        }
+      }
+      if (wide) {  // (narrow, pair: a row's softmax lives in one thread's 64 columns)
+        if (!fail) {
+          tmem_st1(mail_mine, m);
+          tmem_wait_st();
+        }
+        named_bar_sync(phi_bar, 128);
+        if (!fail) {
+          m = fmaxf(m, tmem_ld1(mail_other));  // (the load of `ya` issued above completes with this wait as well)
+          tmem_wait_ld();
+        }
+      }
+      mb = m * L2E;
+      TL(warp == 8 ? 1 : 2, 3, n, (warp == 8 || warp == 10) && lane == 0);
+      if (!is_q) {
+        // key rows: e = exp(y - max) and its sum; e is parked in Y's own columns for the writing sweep
+        if (!fail && !padded) {
+#pragma unroll 1
+          for (int b4 = 0; b4 < 4; ++b4) {
+            tmem_wait_ld();
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+              yb[i] = ex2f(fmaf(ya[i], L2E, -mb));
+              sum += yb[i];
+            }
+            if (b4 < 3) tmem_ld16(ycol + b4 * 16 + 16, ya);
+            tmem_st16(ycol + b4 * 16, yb);
           }
         }
-        if (wide) {  // (narrow, pair: a row's softmax lives in one thread's 64 columns)
+        if (wide) {
+          named_bar_sync(phi_bar, 128);  // the partner has read the row max out of the mailbox
           if (!fail) {
-            tmem_st1(mail_mine, m);
+            tmem_st1(mail_mine, sum);
             tmem_wait_st();
           }
           named_bar_sync(phi_bar, 128);
           if (!fail) {
-            m = fmaxf(m, tmem_ld1(mail_other));  // (the load of `ya` issued above completes with this wait as well)
+            sum += tmem_ld1(mail_other);
             tmem_wait_ld();
-          }
-        }
-        mb = m * L2E;
-        TL(warp == 8 ? 1 : 2, 3, n, (warp == 8 || warp == 10) && lane == 0);
-        if (!is_q) {
-          // key rows: e = exp(y - max) and its sum; e is parked in Y's own columns for the writing sweep
-          if (!fail && !padded) {
-#pragma unroll 1
-            for (int b4 = 0; b4 < 4; ++b4) {
-              tmem_wait_ld();
-#pragma unroll
-              for (int i = 0; i < 16; ++i) {
-                yb[i] = ex2f(fmaf(ya[i], L2E, -mb));
-                sum += yb[i];
-              }
-              if (b4 < 3) tmem_ld16(ycol + b4 * 16 + 16, ya);
-              tmem_st16(ycol + b4 * 16, yb);
-            }
-          }
-          if (wide) {
-            named_bar_sync(phi_bar, 128);  // the partner has read the row max out of the mailbox
-            if (!fail) {
-              tmem_st1(mail_mine, sum);
-              tmem_wait_st();
-            }
-            named_bar_sync(phi_bar, 128);
-            if (!fail) {
-              sum += tmem_ld1(mail_other);
-              tmem_wait_ld();
-            }
           }
         }
       }
@@ -1182,7 +1162,7 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       tc_fence_after_sync();
       const bool f16 = __int_as_float(s_rmax[p]) <= RMAX_F16 && __int_as_float(s_sbound[p]) < SMAX_F16;
       // (the 8-bit-mantissa operands keep the range but not the accuracy bound: the caller is told)
-      if (MODE == 0 && !f16 && tw == 0 && a.dev_status) atomicMax(a.dev_status, (int)LAWCAT_ERR_NUMERIC);
+      if (!f16 && tw == 0 && a.dev_status) atomicMax(a.dev_status, (int)LAWCAT_ERR_NUMERIC);
       // The passes that write operands exist once per operand type and with or without the dropped softmax sum, picked by one
       // branch: with the choice at every conversion the code that runs was strewn over twice its size.
       const bool track = (n & 7) == 0;
@@ -1193,12 +1173,10 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         const bool s_on = !narrow || (!padded && r128 < dh);
         // The largest state entry (which decides between fp16 and bf16 operands) is measured every 8th chunk; in between
         // its bound grows by 64 max|v| per chunk (kh <= 1), a few thousand at most against the threshold of 3e4.
-        if (!fail && !s_on && !phi_on) mbar_arrive(bar(B_X_FREE));  // (see the end of the pass)
         if (!fail && s_on) {
           const int c = r128;
           const float bm = vec(p, 0)[c], ft = vec(p, 1)[c];
           const float dm = ex2f(bm), dC = ex2f(bm + ft);
-          if (ch == 0) dsum += bm + ft;
           float mx = 0.f;
           // (pair: 64 value columns, 32 per thread)
 #pragma unroll 1
@@ -1206,47 +1184,39 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             const int blk = pair ? ch : ch * 2 + b2;
             tmem_ld32(lane_base + cS + blk * 32, y);
             tmem_wait_ld();
-            if (MODE == 0) {
-              if (track) {
+            if (track) {
 #pragma unroll
-                for (int i = 0; i < 32; ++i) mx = fmaxf(mx, fabsf(y[i]));
-              }
-              const uint64_t dm2 = f2_pack(dm, dm);
-#pragma unroll
-              for (int q4 = 0; q4 < 4; ++q4) {
-                uint64_t w[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) w[i] = f2_mul(dm2, f2_pack(y[8 * q4 + 2 * i], y[8 * q4 + 2 * i + 1]));
-                // columns [8 nb, 8 nb + 8) of row c: block nb of the unswizzled operand (a warp's 32 rows: 512 contiguous bytes)
-                sts128(sb + OFF_SBF + (uint32_t)(blk * 4 + q4) * 2048u + (uint32_t)c * 16u, pack8p(w, F16));
-              }
+              for (int i = 0; i < 32; ++i) mx = fmaxf(mx, fabsf(y[i]));
             }
-            {
-              const uint64_t dC2 = f2_pack(dC, dC);
+            const uint64_t dm2 = f2_pack(dm, dm), dC2 = f2_pack(dC, dC);
 #pragma unroll
-              for (int i = 0; i < 32; i += 2) f2_unpack(f2_mul(dC2, f2_pack(y[i], y[i + 1])), y[i], y[i + 1]);
+            for (int q4 = 0; q4 < 4; ++q4) {
+              uint64_t w[4];
+#pragma unroll
+              for (int i = 0; i < 4; ++i) w[i] = f2_mul(dm2, f2_pack(y[8 * q4 + 2 * i], y[8 * q4 + 2 * i + 1]));
+              // columns [8 nb, 8 nb + 8) of row c: block nb of the unswizzled operand (a warp's 32 rows: 512 contiguous bytes)
+              sts128(sb + OFF_SBF + (uint32_t)(blk * 4 + q4) * 2048u + (uint32_t)c * 16u, pack8p(w, F16));
             }
+#pragma unroll
+            for (int i = 0; i < 32; i += 2) f2_unpack(f2_mul(dC2, f2_pack(y[i], y[i + 1])), y[i], y[i + 1]);
             tmem_st32(lane_base + cS + blk * 32, y);
           }
           if (ch == (narrow ? 0 : 1)) {  // (the thread of the row's last existing column half also carries z)
             const float z = tmem_ld1(lane_base + cSZ);
             tmem_wait_ld();
-            if (MODE == 0) {
-              *reinterpret_cast<uint16_t*>(sg + OFF_SBF + (hd >> 3) * 2048 + c * 16) = to16(dm * z, F16);
-              if (track) mx = fmaxf(mx, fabsf(z));
-            }
+            *reinterpret_cast<uint16_t*>(sg + OFF_SBF + (hd >> 3) * 2048 + c * 16) = to16(dm * z, F16);
+            if (track) mx = fmaxf(mx, fabsf(z));
             tmem_st1(lane_base + cSZ, dC * z);
           }
-          if (MODE == 0 && track) {
+          if (track) {
             mx = warp_max(mx);
             if (lane == 0) atomicMax(s_smax, __float_as_int(mx < 3.0e38f ? mx : 3.0e38f));
           }
           tmem_wait_st();
-          if (!phi_on) mbar_arrive(bar(B_X_FREE));  // (state-only pass) this thread has read bm, ft and reads no exponents
         }
         TL(warp == 8 ? 1 : 2, 6, n, (warp == 8 || warp == 10) && lane == 0);
         // ---- phi, writing sweep -------------------------------------------------------------------------------------------
-        if (phi_on && !fail && !padded) {
+        if (!fail && !padded) {
           if (is_q) {
             float qsum = 0.f;
             auto q_block = [&](const float* yy, int jj0) {  // 16 columns = channel groups jj0, jj0 + 1
@@ -1292,7 +1262,7 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 const float e63[8] = {ea.x, ea.y, ea.z, ea.w, eb.x, eb.y, eb.z, eb.w};
 #pragma unroll
                 for (int i = 0; i < 8; ++i) ks[i] = ee[h2 * 8 + i] * inv * ex2f(-x[i]);
-                if (MODE == 0) sts128(sb + OFF_QK + ch * 16384 + sw128(C + row, jj & 7), pack8(ks, F16));
+                sts128(sb + OFF_QK + ch * 16384 + sw128(C + row, jj & 7), pack8(ks, F16));
 #pragma unroll
                 for (int i = 0; i < 8; ++i) ks[i] *= e63[i];
                 // kh: row = token, MN-major A operand of the state update (slab = column half)
@@ -1300,31 +1270,18 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
               }
             };
             tmem_ld16(ycol, ya);
-            if (MODE == 0) {
 #pragma unroll 1
-              for (int b4 = 0; b4 < 4; ++b4) {
-                tmem_wait_ld();
+            for (int b4 = 0; b4 < 4; ++b4) {
+              tmem_wait_ld();
 #pragma unroll
-                for (int i = 0; i < 16; ++i) yb[i] = ya[i];
-                if (b4 < 3) tmem_ld16(ycol + b4 * 16 + 16, ya);
-                k_block(yb, ch * 8 + b4 * 2);
-              }
-            } else {  // (the state-only pass is small enough to afford two copies, with a load in flight across both)
-#pragma unroll 1
-              for (int b2 = 0; b2 < 2; ++b2) {
-                tmem_wait_ld();
-                tmem_ld16(ycol + b2 * 32 + 16, yb);
-                k_block(ya, ch * 8 + b2 * 4);
-                tmem_wait_ld();
-                if (b2 < 1) tmem_ld16(ycol + b2 * 32 + 32, ya);
-                k_block(yb, ch * 8 + b2 * 4 + 2);
-              }
+              for (int i = 0; i < 16; ++i) yb[i] = ya[i];
+              if (b4 < 3) tmem_ld16(ycol + b4 * 16 + 16, ya);
+              k_block(yb, ch * 8 + b4 * 2);
             }
           }
         }
       };
-      if (MODE == 1) write_operands(std::true_type{}, std::false_type{});  // (no operand of a choosable type)
-      else if (f16 && !need_qsum) write_operands(std::true_type{}, std::false_type{});
+      if (f16 && !need_qsum) write_operands(std::true_type{}, std::false_type{});
       else if (f16) write_operands(std::true_type{}, std::true_type{});
       else if (!need_qsum) write_operands(std::false_type{}, std::false_type{});
       else write_operands(std::false_type{}, std::true_type{});
@@ -1337,20 +1294,18 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       fail = named_bar_or(2, 256, fail);
       TL(warp == 8 ? 1 : 2, 9, n, (warp == 8 || warp == 10) && lane == 0);
       if (fail) break;
-      if (MODE == 0 && tw == 0) {
+      if (tw == 0) {
         // |S_new| <= |S_old| + 64 max|v|: the next chunk's choice of operand type
         s_sbound[pp] = __float_as_int(__int_as_float(track ? *s_smax : s_sbound[p]) + 64.f * fmaxf(__int_as_float(s_vmax[p]), 1.f));
         *s_smax = 0;
         __threadfence_block();
       }
       mbar_arrive(bar(B_SBF_FULL));
-      if (phi_on) {
-        mbar_arrive(bar(B_Y_FREE));
-        mbar_arrive(bar(B_X_FREE));
-        mbar_arrive(bar(B_QK_FULL));
-      }
+      mbar_arrive(bar(B_Y_FREE));
+      mbar_arrive(bar(B_X_FREE));
+      mbar_arrive(bar(B_QK_FULL));
     }
-    if (MODE == 0 && is_q && nchunks > 0) mask_chunk(nchunks - 1);
+    if (is_q && nchunks > 0) mask_chunk(nchunks - 1);
     // ---- final state -------------------------------------------------------------------------------------------------
     if (!fail && !*s_abort && (nchunks == 0 || wait_or_abort(bar(B_MMA2), (uint32_t)((nchunks - 1) & 1), s_abort, a.wait_limit))) {
       tc_fence_after_sync();
@@ -1358,12 +1313,11 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       // (the block's place among the sequences is worked out again: kept across the chunk loop it would cost spills)
       int blk2 = blockIdx.x;
       asm volatile("" : "+r"(blk2));
-      const SeqView sv = seq_of_block(a, tab, Hn * a.nsub, MODE == 1 ? 1 : 0, blk2);
-      const int nrun = sv.nseg - (MODE == 1 ? 1 : 0), seg2 = (blk2 / a.nsub) % nrun, hh = blk2 / (a.nsub * nrun);
+      const SeqView sv = seq_of_block(a, tab, Hn, 0, blk2);
+      const int seg2 = blk2 % sv.nseg, hh = blk2 / sv.nseg;
       const size_t hr = (pair ? 2 * hh : hh) + (pair ? (c >> 6) : 0);
-      const size_t out_idx = (MODE == 1 ? (size_t)(sv.seg0 + seg2) * a.nsub + blk2 % a.nsub : (size_t)sv.seq) * a.H + hr;
-      if (MODE == 1 && ch == 0 && c < dh) a.dtot[out_idx * hd + cr] = dsum;
-      const bool last = MODE == 1 || seg2 == sv.nseg - 1;  // (each of the two outputs is optional on its own)
+      const size_t out_idx = (size_t)sv.seq * a.H + hr;
+      const bool last = seg2 == sv.nseg - 1;  // (each of the two outputs is optional on its own)
       if (a.S_T != nullptr && last) {
         if (rw_on) {
           float s[32];
