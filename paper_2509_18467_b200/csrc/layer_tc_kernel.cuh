@@ -340,7 +340,7 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     return reinterpret_cast<float*>(sg + OFF_VEC + parity * 1536 + which * 512);
   };
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;  // (warp: uniform to the compiler)
   // WIDTH 0: heads of 128 channels. WIDTH 1 (narrow): one head of 64 channels, run as a 128-wide one whose upper 64
   // channels are zero. WIDTH 2 (pair): two 64-wide heads of one key/value group side by side -- channels 0-63 belong to head
   // 2 h, channels 64-127 to head 2 h + 1; q, gate and o of the two are contiguous in memory and are addressed as one head
@@ -629,7 +629,7 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       }
       __syncwarp();
     }
-    // The whole warp walks the loop and waits (one lane per barrier of a set); lane 0 issues.
+    // The whole warp walks the loop and waits (one lane per barrier of a set); one elected lane issues.
     {
       // shared-memory descriptors of the operands (all tiles sit at fixed addresses); a K step adds a constant to the
       // start-address field (units of 16 bytes): K-major operand 32 B per step and 16 KB to the second 64-column slab;
@@ -662,7 +662,7 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       };
       bool ok = nchunks > 0;
       if (!mixw && ok) ok = wait_set_or_abort(bar(0), BIT(B_U_FULL), 0u, lane, s_abort, a.wait_limit);
-      if (!mixw && ok && lane == 0) {
+      if (!mixw && ok && elect_one()) {
         tc_fence_after_sync();
         issue_mma1();
       }
@@ -673,7 +673,7 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         TL(0, 0, n, lane == 0);
         const bool f16 = __int_as_float(s_rmax[p]) <= RMAX_F16 && __int_as_float(s_sbound[p]) < SMAX_F16;
         const int fmt = f16 ? FMT_F16 : FMT_BF16;
-        if (lane == 0) {
+        if (elect_one()) {
           // the scores first: their mask pass is the longest chain behind this hand-over
           tc_fence_after_sync();
           // (pair: channels 0-63 give the first head's scores, channels 64-127 the second head's, in accumulators of their own)
@@ -689,13 +689,13 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         if (!mixw && n + 1 < nchunks) {
           // then the mix of the next chunk: its phi sweeps read Y while this chunk's read-out and state update execute
           WAITSET(BIT(B_U_FULL) | BIT(B_Y_FREE), PAR(B_U_FULL, pp) | PAR(B_Y_FREE, p));
-          if (lane == 0) {
+          if (elect_one()) {
             tc_fence_after_sync();
             issue_mma1();
           }
         }
         TL(0, 2, n, lane == 0);
-        if (lane == 0) {
+        if (elect_one()) {
           tc_fence_after_sync();
           // read-out O' | denominator = qs [2^b_mid S | 2^b_mid z] in one product per K step
           // (pair: the first head's read-out contracts channels 0-63 with state rows 0-63, the second head's the rest)
@@ -718,7 +718,7 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         TL(0, 3, n, lane == 0);
         WAITSET(BIT(B_PH_FULL), PAR(B_PH_FULL, p));
         TL(0, 4, n, lane == 0);
-        if (lane == 0) {
+        if (elect_one()) {
           // O' += P v  (the scores' part of the denominator is summed by the mask pass)
           tc_fence_after_sync();
           const uint32_t ID_O = instr_desc(128, NV, FMT_F16, MAJOR_K, MAJOR_MN);
@@ -742,7 +742,7 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     constexpr uint32_t ID = instr_desc(128, narrow ? 64 : 128, FMT_F16, MAJOR_K, MAJOR_K);
     for (int n = 0; n < nchunks; ++n) {
       WAITSET(BIT(B_U_FULL) | (n > 0 ? BIT(B_Y_FREE) : 0u), PAR(B_U_FULL, n & 1) | PAR(B_Y_FREE, (n - 1) & 1));
-      if (lane == 0) {
+      if (elect_one()) {
         tc_fence_after_sync();
 #pragma unroll
         for (int k = 0; k < (narrow ? 4 : 8); ++k) {

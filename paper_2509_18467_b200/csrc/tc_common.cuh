@@ -214,6 +214,14 @@ __host__ __device__ constexpr uint32_t instr_desc(int M, int N, int fmt, int a_m
   return (1u << 4) | ((uint32_t)fmt << 7) | ((uint32_t)fmt << 10) | ((uint32_t)a_major << 15) |
          ((uint32_t)b_major << 16) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
+// True in one lane of a converged warp. A branch on it, inside a warp-uniform branch, leaves descriptors and addresses of what the
+// lane issues in uniform registers; behind `lane == 0` every product first moves its own there, and among sixteen busy warps each
+// such instruction waits its turn (8 score products of the layer kernel: 1.6k cycles to their completion, 0.9k so).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+  return r != 0;
+}
 // D[tmem] (+)= A[smem] * B[smem]; issued by one thread.
 __device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
