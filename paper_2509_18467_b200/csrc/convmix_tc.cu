@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(fwd_threads<D, TO>()) convmix_tc_fwd_kernel(co
   const uint32_t sb = smem_u32(sg);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   volatile int* const s_flags = reinterpret_cast<volatile int*>(sg + OFF_BAR + 16);  // [0] tmem base, [1] abort
-  float* const s_taps = reinterpret_cast<float*>(sg + OFF_TAPS);
+  uint8_t* const s_taps = sg + OFF_TAPS;
   float* const s_red = reinterpret_cast<float*>(sg + OFF_RED);  // [max, sum][column group][128 rows]
   const int t0 = tile_of_block() * TT, bh = blockIdx.x, h = bh % a.H, b = bh / a.H;
   if (t0 >= a.T) return;
@@ -154,10 +154,7 @@ __global__ void __launch_bounds__(fwd_threads<D, TO>()) convmix_tc_fwd_kernel(co
     const int head = stream ? j : h;
     // (a separate linear layer per stream: the product that read the query stream's W_h has completed)
     if (stream == 1 && a.unshared) load_w(a.W + ((size_t)a.H + h) * D * D);
-    for (int idx = tid; idx < D * 4; idx += NTH) {
-      const int c = idx >> 2, dl = idx & 3;
-      s_taps[idx] = dl < a.K ? __bfloat162float(w[((size_t)head * D + c) * a.K + dl]) : 0.f;
-    }
+    load_taps<D>(s_taps, w, head, a.K, tid, NTH);
     if (stream == 0 && tid < TT && t0 + tid < a.T) {  // the key stream's raw row of this thread, towards L2 meanwhile
       const bf16* kr = a.k + (((size_t)b * a.T + t0 + tid) * a.Hkv + j) * D;
       prefetch_l2(kr);
@@ -166,14 +163,17 @@ __global__ void __launch_bounds__(fwd_threads<D, TO>()) convmix_tc_fwd_kernel(co
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    conv_emit<RPT>(raw, s_taps, co, [&](int i, float* u) {
+    conv_emit<D, RPT>(raw, s_taps, co, [&](int i, uint64_t* u) {
       uint8_t* dst = sg + OFF_U + toff(L::SLAB_U, cr0 + i, co * 8);
+      float f[8];
       if (NT == 1) {
-        *reinterpret_cast<uint4*>(dst) = pack8f16(u);
+        pairs_to_floats(u, f);
+        *reinterpret_cast<uint4*>(dst) = pack8f16(f);
       } else {
         *reinterpret_cast<uint4*>(dst) = take_bf16(u);
         *reinterpret_cast<uint4*>(dst + L::TILE_U) = take_bf16(u);
-        *reinterpret_cast<uint4*>(dst + 2 * L::TILE_U) = pack8bf16(u);
+        pairs_to_floats(u, f);
+        *reinterpret_cast<uint4*>(dst + 2 * L::TILE_U) = pack8bf16(f);
       }
     });
     fence_proxy_async();

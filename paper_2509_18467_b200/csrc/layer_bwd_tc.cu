@@ -950,7 +950,7 @@ __global__ void __launch_bounds__(MCfg<D>::THREADS, D == 128 ? 1 : 2) mix_bwd_ke
   const uint32_t sb = smem_u32(sg);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   volatile int* const s_fl = reinterpret_cast<volatile int*>(sg + M::BAR + 16);  // tmem base, abort
-  float* const s_taps = reinterpret_cast<float*>(sg + M::TAPS);
+  uint8_t* const s_taps = sg + M::TAPS;
   const int t0 = blockIdx.x * TT, bj = blockIdx.z * gridDim.y + blockIdx.y, j = bj % a.Hkv, b = bj / a.Hkv, G = a.H / a.Hkv;
   if (b >= a.B) return;
   const int nvalid = min(TT, a.T - t0);
@@ -1040,10 +1040,7 @@ __global__ void __launch_bounds__(MCfg<D>::THREADS, D == 128 ? 1 : 2) mix_bwd_ke
       for (int stream = 0; stream < 2; ++stream) {
         const bf16* w = stream ? a.w_k : a.w_q;
         const int NH = stream ? a.Hkv : a.H, head = stream ? j : h;
-        for (int idx = tid; idx < D * 4; idx += NTH) {
-          const int c = idx >> 2, dl = idx & 3;
-          s_taps[idx] = dl < a.K ? __bfloat162float(w[((size_t)head * D + c) * a.K + dl]) : 0.f;
-        }
+        load_taps<D>(s_taps, w, head, a.K, tid, NTH);
         // the rows of the next (head, stream) step travel towards L2 while this one is computed
         if (g + stream < G) {
           const int nh = h + stream;
@@ -1091,8 +1088,10 @@ __global__ void __launch_bounds__(MCfg<D>::THREADS, D == 128 ? 1 : 2) mix_bwd_ke
         conv_load<D, RPT>(raw, stream ? a.k : a.q, stream ? a.cache_k : a.cache_q, b, t0 + rr0 * RPT, a.T, NH, head, a.K, o);
         __syncthreads();  // (the taps)
         // ---- u
-        conv_emit<RPT>(raw, s_taps, o, [&](int i, float* u) {
+        conv_emit<D, RPT>(raw, s_taps, o, [&](int i, const uint64_t* u2) {
           uint4 hi, lo;
+          float u[8];
+          pairs_to_floats(u2, u);
           split8h(u, true, hi, lo);
           const uint32_t at = toff(L::SLAB_U, rr0 * RPT + i, o * 8);
           *reinterpret_cast<uint4*>(sg + M::U + at) = hi;

@@ -167,36 +167,60 @@ __device__ __forceinline__ void conv_load(uint4 (&raw)[N + HALO], const bf16* x,
       raw[i] = *reinterpret_cast<const uint4*>(cache + (((size_t)b * (K - 1) + tt + (K - 1)) * NH + head) * D + o * 8);
   }
 }
-// ... and the sums; emit(i, u) takes token t + i. s_w: the head's taps, fp32 [D][4], in shared memory.
-template <int N, typename F>
-__device__ __forceinline__ void conv_emit(const uint4 (&raw)[N + HALO], const float* s_w, int o, F emit) {
-  float w[8][4];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const float4 t4 = *reinterpret_cast<const float4*>(s_w + (o * 8 + i) * 4);
-    w[i][0] = t4.x; w[i][1] = t4.y; w[i][2] = t4.z; w[i][3] = t4.w;
+// A head's taps as packed pairs of channels, fp32 (zero beyond the conv width): the pairs of taps (dl, dl + 1) of channel pair cp
+// of octet o are the 16 bytes at ((2 cp + dl / 2) * D / 8 + o) * 16, so that neighbouring octets lie side by side. (As [D][4] rows
+// the eight lanes of a quarter warp met in four banks: more than half of all shared-memory wavefronts of these kernels.)
+template <int D>
+__device__ __forceinline__ void load_taps(uint8_t* s_taps, const bf16* w, int head, int K, int tid, int nthreads) {
+  for (int idx = tid; idx < D * 2; idx += nthreads) {
+    const int o = idx % (D / 8), cp = idx / (D / 8) & 3, dl = idx / (D / 2);
+    const bf16* wc = w + ((size_t)head * D + o * 8 + 2 * cp) * K + dl;
+    const uint64_t t = dl < K ? f2_pack(__bfloat162float(wc[0]), __bfloat162float(wc[K])) : f2_pack(0.f, 0.f);
+    *reinterpret_cast<uint64_t*>(s_taps + ((2 * cp + (dl >> 1)) * (D / 8) + o) * 16 + (dl & 1) * 8) = t;
   }
+}
+__device__ __forceinline__ void unpack8p(const uint4& v, uint64_t* f) {  // 8 bf16 values -> 4 packed pairs of fp32
+  f[0] = f2_pack(bf16_lo(v.x), bf16_hi(v.x)); f[1] = f2_pack(bf16_lo(v.y), bf16_hi(v.y));
+  f[2] = f2_pack(bf16_lo(v.z), bf16_hi(v.z)); f[3] = f2_pack(bf16_lo(v.w), bf16_hi(v.w));
+}
+// ... and the sums, in pairs of channels; emit(i, u) takes token t + i. Every raw row is unpacked once.
+template <int D, int N, typename F>
+__device__ __forceinline__ void conv_emit(const uint4 (&raw)[N + HALO], const uint8_t* s_taps, int o, F emit) {
+  uint64_t w[4][4], x0[4], x1[4], x2[4], x3[4];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(s_taps + (u * (D / 8) + o) * 16);
+    w[u >> 1][2 * (u & 1)] = t.x;
+    w[u >> 1][2 * (u & 1) + 1] = t.y;
+  }
+  unpack8p(raw[0], x3); unpack8p(raw[1], x2); unpack8p(raw[2], x1);
 #pragma unroll
   for (int i = 0; i < N; ++i) {
-    float u[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    uint64_t u[4];
+    unpack8p(raw[i + HALO], x0);
 #pragma unroll
-    for (int dl = 0; dl < 4; ++dl) {
-      float xv[8];
-      unpack8b(raw[i + HALO - dl], xv);
-#pragma unroll
-      for (int c = 0; c < 8; ++c) u[c] = fmaf(w[c][dl], xv[c], u[c]);
-    }
+    for (int cp = 0; cp < 4; ++cp)
+      u[cp] = f2_fma(w[cp][3], x3[cp], f2_fma(w[cp][2], x2[cp], f2_fma(w[cp][1], x1[cp], f2_mul(w[cp][0], x0[cp]))));
     emit(i, u);
+#pragma unroll
+    for (int cp = 0; cp < 4; ++cp) { x3[cp] = x2[cp]; x2[cp] = x1[cp]; x1[cp] = x0[cp]; }
   }
+}
+__device__ __forceinline__ void pairs_to_floats(const uint64_t* v, float* f) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) f2_unpack(v[i], f[2 * i], f[2 * i + 1]);
 }
 
 // v rounded to bf16, and v -= the rounded value
-__device__ __forceinline__ uint4 take_bf16(float* v) {
-  const uint4 p = pack8bf16(v);
-  float h[8];
-  unpack8b(p, h);
+__device__ __forceinline__ uint4 take_bf16(uint64_t* v) {
+  float f[8];
+  uint64_t h[4];
+  pairs_to_floats(v, f);
+  const uint4 p = pack8bf16(f);
+  unpack8p(p, h);
+  const uint64_t neg = f2_pack(-1.f, -1.f);
 #pragma unroll
-  for (int i = 0; i < 8; ++i) v[i] -= h[i];
+  for (int i = 0; i < 4; ++i) v[i] = f2_fma(h[i], neg, v[i]);
   return p;
 }
 
