@@ -98,44 +98,49 @@ __device__ __forceinline__ void conv_tile(const uint8_t* s_raw, const float* s_w
 // the conv output as one fp16 operand. fp32 outputs (features that a fused caller keeps in fp32, and those of the exact
 // recurrence) take it as three bf16 terms, u = b1 + b2 + b3 exactly, with W_h exact in bf16: the products are those of
 // fp32 numbers over the full fp32 range, summed in fp32.
-// Bound by HBM writes (fp32 features) and by the dependent phases of a tile: raw rows go from global memory through the
-// conv straight into the operand (no staging tile), and the outputs leave through the drained operand tile as whole rows.
+// Bound by instruction issue and the dependent phases of a tile. The products run behind other work: the key stream's conv (into
+// registers) while the query stream's mix runs, the query stream's features and their way out while the key stream's does. Outputs
+// leave through a staging tile as whole rows.
 template <int D, typename TO>
 __host__ __device__ constexpr int fwd_threads() { return D == 128 && sizeof(TO) == 4 ? 512 : 256; }
+template <int D, typename TO>
+struct FwdMap {  // shared memory
+  using L = Lay<D>;
+  static constexpr int NT = sizeof(TO) == 4 ? 3 : 1, NCG = fwd_threads<D, TO>() / 128;
+  static constexpr uint32_t WT = 0, U = WT + L::TILE_W, ST = U + NT * L::TILE_U, TAPS = ST + TT * D * sizeof(TO);
+  static constexpr uint32_t RED = TAPS + 2 * D * 16, BAR = RED + NCG * TT * 4, BYTES = BAR + 64;
+};
 
 template <int D, typename TO>
 __global__ void __launch_bounds__(fwd_threads<D, TO>()) convmix_tc_fwd_kernel(const CArgs a) {
   using L = Lay<D>;
+  using M = FwdMap<D, TO>;
   extern __shared__ __align__(128) uint8_t sg[];
-  constexpr int NTH = fwd_threads<D, TO>(), NCG = NTH / 128;
-  constexpr int NT = sizeof(TO) == 4 ? 3 : 1, FMT = NT == 3 ? FMT_BF16 : FMT_F16;
-  constexpr uint32_t OFF_WT = 0, OFF_U = OFF_WT + L::TILE_W;
-  constexpr uint32_t OFF_TAPS = OFF_U + NT * L::TILE_U, OFF_RED = OFF_TAPS + D * 16, OFF_BAR = OFF_RED + 2 * NCG * TT * 4;
+  constexpr int NTH = fwd_threads<D, TO>(), NCG = M::NCG, NT = M::NT, FMT = NT == 3 ? FMT_BF16 : FMT_F16;
   const uint32_t sb = smem_u32(sg);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  volatile int* const s_flags = reinterpret_cast<volatile int*>(sg + OFF_BAR + 16);  // [0] tmem base, [1] abort
-  uint8_t* const s_taps = sg + OFF_TAPS;
-  float* const s_red = reinterpret_cast<float*>(sg + OFF_RED);  // [max, sum][column group][128 rows]
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;  // (warp: uniform to the compiler)
+  volatile int* const s_flags = reinterpret_cast<volatile int*>(sg + M::BAR + 16);  // [0] tmem base, [1] abort
+  float* const s_red = reinterpret_cast<float*>(sg + M::RED);  // [column group][128 rows]
   const int t0 = tile_of_block() * TT, bh = blockIdx.x, h = bh % a.H, b = bh / a.H;
   if (t0 >= a.T) return;
   const int G = a.H / a.Hkv, j = h / G;
   if (tid == 0) {
-    mbar_init(sb + OFF_BAR, 1);
+    mbar_init(sb + M::BAR, 1);
     mbar_fence_init();
     s_flags[1] = 0;
   }
   if (warp == 0) {
-    tmem_alloc(sb + OFF_BAR + 16, D);
+    tmem_alloc(sb + M::BAR + 16, 2 * D);
     tmem_relinquish();
   }
   asm volatile("griddepcontrol.wait;" ::: "memory");
   auto load_w = [&](const bf16* Wh) {
     if (NT == 1) {
-      load_w_tile<D>(sg + OFF_WT, Wh, tid, NTH);
+      load_w_tile<D>(sg + M::WT, Wh, tid, NTH);
     } else {
       for (int idx = tid; idx < D * L::OPR; idx += NTH) {
         const int c = idx / L::OPR, o = idx % L::OPR;
-        *reinterpret_cast<uint4*>(sg + OFF_WT + toff(L::SLAB_W, c, o * 8)) = *reinterpret_cast<const uint4*>(Wh + (size_t)c * D + o * 8);
+        *reinterpret_cast<uint4*>(sg + M::WT + toff(L::SLAB_W, c, o * 8)) = *reinterpret_cast<const uint4*>(Wh + (size_t)c * D + o * 8);
       }
     }
   };
@@ -144,89 +149,103 @@ __global__ void __launch_bounds__(fwd_threads<D, TO>()) convmix_tc_fwd_kernel(co
   uint4 raw[RPT + HALO];
   conv_load<D, RPT>(raw, a.q, a.cache_q, b, t0 + cr0, a.T, a.H, h, a.K, co);
   load_w(a.W + (size_t)h * D * D);
+  load_taps<D>(sg + M::TAPS, a.w_q, h, a.K, tid, NTH);
+  load_taps<D>(sg + M::TAPS + D * 16, a.w_k, j, a.K, tid, NTH);
   const int row = (warp & 3) * 32 + lane, cg = warp >> 2;  // epilogue: row of the tile, group of its columns
   constexpr int HC = D / NCG;
-  uint32_t lane_base = 0, tmem = 0;
-  Waiter wt{sb + OFF_BAR, 0u, s_flags + 1, a.dev_status};
-#pragma unroll 1
-  for (int stream = 0; stream < 2; ++stream) {
-    const bf16* w = stream ? a.w_k : a.w_q;
-    const int head = stream ? j : h;
-    // (a separate linear layer per stream: the product that read the query stream's W_h has completed)
-    if (stream == 1 && a.unshared) load_w(a.W + ((size_t)a.H + h) * D * D);
-    load_taps<D>(s_taps, w, head, a.K, tid, NTH);
-    if (stream == 0 && tid < TT && t0 + tid < a.T) {  // the key stream's raw row of this thread, towards L2 meanwhile
-      const bf16* kr = a.k + (((size_t)b * a.T + t0 + tid) * a.Hkv + j) * D;
-      prefetch_l2(kr);
-      if (D * 2 > 128) prefetch_l2(kr + 64);
+  tc_fence_before_sync();
+  __syncthreads();
+  tc_fence_after_sync();
+  const uint32_t tmem = (uint32_t)s_flags[0], lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16) + cg * HC;
+  Waiter wt{sb + M::BAR, 0u, s_flags + 1, a.dev_status};
+  auto put_u = [&](int i, uint64_t* u) {  // operand row of token cr0 + i
+    uint8_t* dst = sg + M::U + toff(L::SLAB_U, cr0 + i, co * 8);
+    float f[8];
+    if (NT == 1) {
+      pairs_to_floats(u, f);
+      *reinterpret_cast<uint4*>(dst) = pack8f16(f);
+    } else {
+      *reinterpret_cast<uint4*>(dst) = take_bf16(u);
+      *reinterpret_cast<uint4*>(dst + L::TILE_U) = take_bf16(u);
+      pairs_to_floats(u, f);
+      *reinterpret_cast<uint4*>(dst + 2 * L::TILE_U) = pack8bf16(f);
     }
-    tc_fence_before_sync();
-    __syncthreads();
-    tc_fence_after_sync();
-    conv_emit<D, RPT>(raw, s_taps, co, [&](int i, uint64_t* u) {
-      uint8_t* dst = sg + OFF_U + toff(L::SLAB_U, cr0 + i, co * 8);
-      float f[8];
-      if (NT == 1) {
-        pairs_to_floats(u, f);
-        *reinterpret_cast<uint4*>(dst) = pack8f16(f);
-      } else {
-        *reinterpret_cast<uint4*>(dst) = take_bf16(u);
-        *reinterpret_cast<uint4*>(dst + L::TILE_U) = take_bf16(u);
-        pairs_to_floats(u, f);
-        *reinterpret_cast<uint4*>(dst + 2 * L::TILE_U) = pack8bf16(f);
-      }
-    });
+  };
+  auto mix = [&](int stream) {  // behind the operand's writes: Y = u W_h
     fence_proxy_async();
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    tmem = (uint32_t)s_flags[0];
-    lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16) + cg * HC;
-    if (tid == 0) {
-      const uint32_t idesc = instr_desc(128, D, FMT, MAJOR_K, MAJOR_MN);
-      const uint64_t db = mview(sb + OFF_WT, L::SLAB_W);
+    if (warp == 0 && elect_one()) {
+      constexpr uint32_t idesc = instr_desc(128, D, FMT, MAJOR_K, MAJOR_MN);
+      const uint64_t db = mview(sb + M::WT, L::SLAB_W);
+#pragma unroll
       for (int term = NT - 1; term >= 0; --term) {  // (smallest terms first)
-        const uint64_t da = kview(sb + OFF_U + term * L::TILE_U, L::SLAB_U);
+        const uint64_t da = kview(sb + M::U + term * L::TILE_U, L::SLAB_U);
+#pragma unroll
         for (int kk = 0; kk < D / 16; ++kk)
-          mma_f16(tmem, dadv(da, 2 * L::SLAB_U * kk), dadv(db, 256 * kk), idesc, term < NT - 1 || kk > 0);
+          mma_f16(tmem + stream * D, dadv(da, 2 * L::SLAB_U * kk), dadv(db, 256 * kk), idesc, term < NT - 1 || kk > 0);
       }
-      mma_commit(sb + OFF_BAR);
+      mma_commit(sb + M::BAR);
     }
-    wt.wait();
-    // phi over the row: softmax (the threads of a row exchange max and sum), or elementwise 1 + ELU / identity
+  };
+  // phi over the row: softmax (the threads of a row exchange the sum), or elementwise 1 + ELU / identity; then out
+  auto features = [&](int stream) {
     float y[HC];
+    auto load_y = [&]() {
 #pragma unroll
-    for (int c0 = 0; c0 < HC; c0 += 32) tmem_ld32(lane_base + c0, y + c0);
-    tmem_wait_ld();
+      for (int c0 = 0; c0 < HC; c0 += 32) tmem_ld32(lane_base + stream * D + c0, y + c0);
+      tmem_wait_ld();
+    };
+    load_y();
     if (a.phi == LAWCAT_PHI_SOFTMAX) {
-      float m = -INFINITY, sum = 0.f;
+      // While every |y| stays below Y_MAX, exp(y) needs no shift by the row's maximum, and the barrier behind which the parts of
+      // the sum meet also tells whether one is missing.
+      float sum, am = 0.f;
+      auto exps = [&](float m) {
+        sum = 0.f;
+        if (NT == 3) {
 #pragma unroll
-      for (int i = 0; i < HC; ++i) m = fmaxf(m, y[i]);
-      s_red[cg * TT + row] = m;
-      __syncthreads();
+          for (int i = 0; i < HC; ++i) { y[i] = expf(y[i] - m); sum += y[i]; }
+        } else {
+          const float mb = m * 1.4426950408889634f;
 #pragma unroll
-      for (int i = 0; i < NCG; ++i) m = fmaxf(m, s_red[i * TT + row]);
-      if (NT == 3) {
+          for (int i = 0; i < HC; ++i) { y[i] = ex2f(fmaf(y[i], 1.4426950408889634f, -mb)); sum += y[i]; }
+        }
+      };
 #pragma unroll
-        for (int i = 0; i < HC; ++i) { y[i] = expf(y[i] - m); sum += y[i]; }
-      } else {
-        const float mb = m * 1.4426950408889634f;
+      for (int i = 0; i < HC; ++i) am = fmaxf(am, fabsf(y[i]));
+      exps(0.f);
+      s_red[cg * TT + row] = sum;
+      if (__syncthreads_or(!(am < Y_MAX))) {
+        __syncthreads();  // (the sums have been seen by nobody; the row's maximum takes their place)
+        load_y();
+        float m = -INFINITY;
 #pragma unroll
-        for (int i = 0; i < HC; ++i) { y[i] = ex2f(fmaf(y[i], 1.4426950408889634f, -mb)); sum += y[i]; }
+        for (int i = 0; i < HC; ++i) m = fmaxf(m, y[i]);
+        s_red[cg * TT + row] = m;
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < NCG; ++i) m = fmaxf(m, s_red[i * TT + row]);
+        exps(m);
+        __syncthreads();
+        s_red[cg * TT + row] = sum;
+        __syncthreads();
       }
-      s_red[(NCG + cg) * TT + row] = sum;
-      __syncthreads();
       float tot = 0.f;
 #pragma unroll
-      for (int i = 0; i < NCG; ++i) tot += s_red[(NCG + i) * TT + row];
+      for (int i = 0; i < NCG; ++i) tot += s_red[i * TT + row];
       const float inv = 1.f / tot;
 #pragma unroll
       for (int i = 0; i < HC; ++i) y[i] *= inv;
-    } else if (a.phi == LAWCAT_PHI_ELU1) {
+    } else {
+      if (a.phi == LAWCAT_PHI_ELU1) {
 #pragma unroll
-      for (int i = 0; i < HC; ++i) y[i] = y[i] > 0.f ? y[i] + 1.f : (NT == 3 ? expf(y[i]) : __expf(y[i]));
+        for (int i = 0; i < HC; ++i) y[i] = y[i] > 0.f ? y[i] + 1.f : (NT == 3 ? expf(y[i]) : __expf(y[i]));
+      }
+      __syncthreads();  // (the staging tile has been read)
     }
-    // out through the drained operand tile: rows of 16-byte pieces, XOR-swizzled, then whole rows to global memory
+    // rows of 16-byte pieces, XOR-swizzled, then whole rows to global memory
     constexpr int EPP = 16 / sizeof(TO), PPR = D / EPP;  // elements per piece, pieces per row
 #pragma unroll
     for (int i = 0; i < HC; i += EPP) {
@@ -234,28 +253,39 @@ __global__ void __launch_bounds__(fwd_threads<D, TO>()) convmix_tc_fwd_kernel(co
       uint4 v;
       if (NT == 3) v = make_uint4(__float_as_uint(y[i]), __float_as_uint(y[i + 1]), __float_as_uint(y[i + 2]), __float_as_uint(y[i + 3]));
       else v = pack8bf16(y + i);
-      *reinterpret_cast<uint4*>(sg + OFF_U + (row * PPR + (pc ^ (row & 7))) * 16) = v;
+      *reinterpret_cast<uint4*>(sg + M::ST + (row * PPR + (pc ^ (row & 7))) * 16) = v;
     }
-    tc_fence_before_sync();
     __syncthreads();
-    tc_fence_after_sync();
-    // (the key stream's rows arrive while the query stream's features leave)
-    if (stream == 0) conv_load<D, RPT>(raw, a.k, a.cache_k, b, t0 + cr0, a.T, a.Hkv, j, a.K, co);
     TO* out = reinterpret_cast<TO*>(stream ? a.kdot : a.qdot);
 #pragma unroll 4
     for (int idx = tid; idx < TT * PPR; idx += NTH) {
       const int r = idx / PPR, pc = idx % PPR;
       if (t0 + r < a.T)
         *reinterpret_cast<uint4*>(out + (((size_t)b * a.T + t0 + r) * a.H + h) * D + pc * EPP) =
-            *reinterpret_cast<const uint4*>(sg + OFF_U + (r * PPR + (pc ^ (r & 7))) * 16);
+            *reinterpret_cast<const uint4*>(sg + M::ST + (r * PPR + (pc ^ (r & 7))) * 16);
     }
-    // (the barrier in front of the next stream's conv keeps its writes behind these reads)
-  }
+  };
+  conv_emit<D, RPT>(raw, sg + M::TAPS, co, put_u);
+  mix(0);
+  uint64_t uk[RPT][4];
+  conv_load<D, RPT>(raw, a.k, a.cache_k, b, t0 + cr0, a.T, a.Hkv, j, a.K, co);
+  conv_emit<D, RPT>(raw, sg + M::TAPS + D * 16, co, [&](int i, uint64_t* u) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) uk[i][c] = u[c];
+  });
+  wt.wait();  // (the operand tile, and W_h, have been read)
+#pragma unroll
+  for (int i = 0; i < RPT; ++i) put_u(i, uk[i]);
+  if (a.unshared) load_w(a.W + ((size_t)a.H + h) * D * D);  // (a separate linear layer per stream)
+  mix(1);
+  features(0);
+  wt.wait();
+  features(1);
   tc_fence_before_sync();
   __syncthreads();
   if (warp == 0) {
     tc_fence_after_sync();
-    tmem_dealloc(tmem, D);
+    tmem_dealloc(tmem, 2 * D);
   }
 }
 
@@ -457,11 +487,6 @@ __global__ void __launch_bounds__(128, 2) convmix_tc_bwd_kernel(const CArgs a) {
   }
 }
 
-template <int D, typename TO>
-constexpr uint32_t fwd_smem() {
-  using L = Lay<D>;
-  return L::TILE_W + (sizeof(TO) == 4 ? 3 : 1) * L::TILE_U + D * 16 + 2 * (fwd_threads<D, TO>() / 128) * TT * 4 + 64;
-}
 constexpr uint32_t bwd_smem() {
   using L = Lay<64>;
   return L::TILE_W + 4 * L::TILE_U + 2048 + (L::RAW_BYTES + 15) / 16 * 16 + 64 * 16 + 64;
@@ -507,8 +532,8 @@ int launch_convmix_tc_fwd(const Ctx& c, const void* q, const void* k, const void
   {
     std::lock_guard<std::mutex> lk(mu);
     if (!done[dev]) {
-      if (raise_smem(convmix_tc_fwd_kernel<64, bf16>, fwd_smem<64, bf16>()) || raise_smem(convmix_tc_fwd_kernel<64, float>, fwd_smem<64, float>()) ||
-          raise_smem(convmix_tc_fwd_kernel<128, bf16>, fwd_smem<128, bf16>()) || raise_smem(convmix_tc_fwd_kernel<128, float>, fwd_smem<128, float>()))
+      if (raise_smem(convmix_tc_fwd_kernel<64, bf16>, FwdMap<64, bf16>::BYTES) || raise_smem(convmix_tc_fwd_kernel<64, float>, FwdMap<64, float>::BYTES) ||
+          raise_smem(convmix_tc_fwd_kernel<128, bf16>, FwdMap<128, bf16>::BYTES) || raise_smem(convmix_tc_fwd_kernel<128, float>, FwdMap<128, float>::BYTES))
         return LAWCAT_ERR_CUDA;
       done[dev] = true;
     }
@@ -516,11 +541,11 @@ int launch_convmix_tc_fwd(const Ctx& c, const void* q, const void* k, const void
   const dim3 grid = tile_grid(p.B * p.H, p.T);
   LaunchScope _ls("convmix_tc_fwd", c.stream);
   if (p.d_k == 64) {
-    if (out_f32) launch_behind(convmix_tc_fwd_kernel<64, float>, grid, dim3(fwd_threads<64, float>()), fwd_smem<64, float>(), c.stream, a);
-    else launch_behind(convmix_tc_fwd_kernel<64, bf16>, grid, dim3(fwd_threads<64, bf16>()), fwd_smem<64, bf16>(), c.stream, a);
+    if (out_f32) launch_behind(convmix_tc_fwd_kernel<64, float>, grid, dim3(fwd_threads<64, float>()), FwdMap<64, float>::BYTES, c.stream, a);
+    else launch_behind(convmix_tc_fwd_kernel<64, bf16>, grid, dim3(fwd_threads<64, bf16>()), FwdMap<64, bf16>::BYTES, c.stream, a);
   } else {
-    if (out_f32) launch_behind(convmix_tc_fwd_kernel<128, float>, grid, dim3(fwd_threads<128, float>()), fwd_smem<128, float>(), c.stream, a);
-    else launch_behind(convmix_tc_fwd_kernel<128, bf16>, grid, dim3(fwd_threads<128, bf16>()), fwd_smem<128, bf16>(), c.stream, a);
+    if (out_f32) launch_behind(convmix_tc_fwd_kernel<128, float>, grid, dim3(fwd_threads<128, float>()), FwdMap<128, float>::BYTES, c.stream, a);
+    else launch_behind(convmix_tc_fwd_kernel<128, bf16>, grid, dim3(fwd_threads<128, bf16>()), FwdMap<128, bf16>::BYTES, c.stream, a);
   }
   LAWCAT_CHECK_LAUNCH();
   return LAWCAT_OK;

@@ -230,6 +230,7 @@ struct Rows {
 struct Mma {
   uint32_t tmem;
   __device__ __forceinline__ void chain(uint32_t col, uint64_t da, uint32_t as, uint64_t db, uint32_t bs, int ks, uint32_t id, bool acc) const {
+#pragma unroll 1
     for (int k = 0; k < ks; ++k) mma_f16(tmem + col, dadv(da, as * k), dadv(db, bs * k), id, (acc || k > 0) ? 1u : 0u);
   }
   __device__ __forceinline__ void split(uint32_t col, uint64_t ah, uint64_t al, uint32_t as, uint64_t bh, uint64_t bl, uint32_t bs,
@@ -247,7 +248,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) sweep_kerne
   constexpr int NV = D + 16;
   extern __shared__ __align__(128) uint8_t sg[];
   const uint32_t sb = smem_u32(sg);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;  // (warp: uniform to the compiler)
   float* const s_x = reinterpret_cast<float*>(sg + F::F_X);
   float* const s_bm = reinterpret_cast<float*>(sg + F::F_VEC);
   float *const s_ft = s_bm + D, *const s_pe = s_ft + D;  // s_pe: ft of the chunk in front (its state is still 2^-ft short)
@@ -421,6 +422,8 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) sweep_kerne
       tma_store_commit();
       a.meta[((size_t)bh * nch + n) * 2] = kap;
       a.meta[((size_t)bh * nch + n) * 2 + 1] = fmt;
+    }
+    if (warp == 0 && elect_one()) {
       mm.split(F::F_P, KV(F::F_QS, F::SL_T), KV(F::F_QS + F::T_TOK, F::SL_T), 2 * F::SL_T, KV(F::F_KS, F::SL_T),
                KV(F::F_KS + F::T_TOK, F::SL_T), 2 * F::SL_T, D / 16, instr_desc(128, C, fmt, MAJOR_K, MAJOR_K), false);
       mm.split(F::F_O, KV(F::F_QS, F::SL_T), KV(F::F_QS + F::T_TOK, F::SL_T), 2 * F::SL_T, MV(F::F_S, F::SL_C),
@@ -452,7 +455,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) sweep_kerne
     }
     for (int i = tid; i < D; i += F::THREADS) s_pe[i] = s_ft[i];
     publish();
-    if (tid == 0) {
+    if (warp == 0 && elect_one()) {
       mm.split(F::F_O, KV(F::F_PM, F::SL_U), KV(F::F_PM + F::T_P, F::SL_U), 2 * F::SL_U, MV(F::F_V, F::SL_T), 0, 256, C / 16,
                instr_desc(128, NV, fmt, MAJOR_K, MAJOR_MN), true);
       mma_commit(bar);
@@ -531,7 +534,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
   constexpr int NW = F::THREADS / 32;
   extern __shared__ __align__(128) uint8_t sg[];
   const uint32_t sb = smem_u32(sg);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;  // (warp: uniform to the compiler)
   float* const s_x = reinterpret_cast<float*>(sg + F::R_X);
   float* const s_bm = reinterpret_cast<float*>(sg + F::R_VEC);
   float *const s_ft = s_bm + D, *const s_pe = s_ft + D;  // s_pe: bm of the chunk behind (its adjoint is still 2^-bm short)
@@ -687,6 +690,8 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
                      : "memory");
         copied = nch - 1 - n;
       }
+    }
+    if (warp == 0 && elect_one()) {
       mm.split(F::R_P, KV(F::R_QS, F::SL_T), KV(F::R_QS + F::T_TOK, F::SL_T), 2 * F::SL_T, KV(F::R_KS, F::SL_T),
                KV(F::R_KS + F::T_TOK, F::SL_T), 2 * F::SL_T, D / 16, instr_desc(128, C, fmt, MAJOR_K, MAJOR_K), false);
       mm.chain(F::R_EP, KV(F::R_DO, F::SL_T), 2 * F::SL_T, KV(F::R_V, F::SL_T), 2 * F::SL_T, D / 16,
@@ -736,8 +741,8 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
     publish();
     const uint32_t ID_KM = instr_desc(128, D, fmt, MAJOR_K, MAJOR_MN), ID_MM = instr_desc(128, D, fmt, MAJOR_MN, MAJOR_MN),
                    ID_KK = instr_desc(128, D, fmt, MAJOR_K, MAJOR_K);
-    if (tid == 0) {
-      ws.wait();  // the state operand has landed
+    if (warp == 0) ws.wait();  // the state operand has landed
+    if (warp == 0 && elect_one()) {
       mm.split(F::R_DQ, KV(F::R_E, F::SL_U), KV(F::R_E + F::T_P, F::SL_U), 2 * F::SL_U, MV(F::R_KS, F::SL_T),
                MV(F::R_KS + F::T_TOK, F::SL_T), 256, C / 16, ID_KM, false);
       mm.split(F::R_DQ, KV(F::R_DO, F::SL_T), 0, 2 * F::SL_T, KV(F::R_S, F::SL_C), KV(F::R_S + F::T_C, F::SL_C), 2 * F::SL_C,
@@ -769,7 +774,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
       tmem_wait_st();
     }
     publish();
-    if (tid == 0) {
+    if (warp == 0 && elect_one()) {
       mm.split(F::R_DK, KV(F::R_V, F::SL_T), 0, 2 * F::SL_T, KV(F::R_S, F::SL_C), KV(F::R_S + F::T_C, F::SL_C), 2 * F::SL_C,
                D / 16, ID_KK, true);
       mm.split(F::R_DVC, KV(F::R_KS, F::SL_T), KV(F::R_KS + F::T_TOK, F::SL_T), 2 * F::SL_T, MV(F::R_S, F::SL_C),

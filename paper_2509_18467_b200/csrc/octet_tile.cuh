@@ -16,6 +16,7 @@ using namespace tc;
 
 constexpr int TT = 128;   // tokens per tile
 constexpr int HALO = 3;   // raw rows kept in front of a tile (conv width up to 4)
+constexpr float Y_MAX = 24.f;  // |y| below which exp(y) is formed without the row's maximum (exp(24) is far from any limit)
 
 // Grid of the kernels that take one (sequence, head) and one tile of TT tokens per block: x the (sequence, head), whose number
 // may pass the 65535 that end the other axes, y and z the tile.
