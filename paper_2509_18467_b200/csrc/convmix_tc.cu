@@ -100,7 +100,8 @@ __device__ __forceinline__ void conv_tile(const uint8_t* s_raw, const float* s_w
 // fp32 numbers over the full fp32 range, summed in fp32.
 // Bound by instruction issue and the dependent phases of a tile. The products run behind other work: the key stream's conv (into
 // registers) while the query stream's mix runs, the query stream's features and their way out while the key stream's does. Outputs
-// leave through a staging tile as whole rows.
+// leave through a staging tile as whole rows. fp32 outputs, 32/8 heads, against one stream after the other: 4 x 1300 tokens of 128
+// channels 148 -> 134 us, 8 x 1024 of 64 84 -> 76, 4096 of 128 107 -> 99.
 template <int D, typename TO>
 __host__ __device__ constexpr int fwd_threads() { return D == 128 && sizeof(TO) == 4 ? 512 : 256; }
 template <int D, typename TO>

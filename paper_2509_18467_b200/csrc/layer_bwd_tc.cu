@@ -226,7 +226,9 @@ struct Rows {
   }
 };
 
-// products on two-term operands, issued by one thread: D (+)= A B with A = ah + al, B = bh + bl (a missing low part is 0)
+// products on two-term operands, issued by one lane: D (+)= A B with A = ah + al, B = bh + bl (a missing low part is 0). (The
+// issuing lane is an elected one of a uniform warp: reverse sweep of 8 x 1024 tokens of 32 heads of 64 255 -> 244 us. Rolled: the 128
+// products of a chunk of the reverse sweep at width 128, unrolled, cost 359 us instead of 350.)
 struct Mma {
   uint32_t tmem;
   __device__ __forceinline__ void chain(uint32_t col, uint64_t da, uint32_t as, uint64_t db, uint32_t bs, int ks, uint32_t id, bool acc) const {
