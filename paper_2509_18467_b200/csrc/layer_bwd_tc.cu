@@ -930,6 +930,10 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
 // two from the largest |w| of the group, or of the head where that is far smaller) and u, the recomputed conv output, are
 // two-term fp16 pairs; the key stream's du is accumulated over the heads in tensor memory. du of the query stream overwrites wq
 // in place.
+// What bounds it is the chain loads -> operands -> products -> gradients out of a step (head, stream). It is folded: while a step's
+// products run, the block works out the next step's operands in registers (its loads are what waits, not the tensor cores), and the
+// gradients of the step before leave tensor memory (dW has two accumulators, du of the query stream is not needed before the next
+// head's products).
 struct MArgs {
   const bf16 *q, *k, *w_q, *w_k, *W, *cache_q, *cache_k;
   const float *qd, *kd, *wk;
@@ -944,9 +948,10 @@ template <int D>
 struct MCfg {
   using L = Lay<D>;
   static constexpr int THREADS = D == 128 ? 512 : 256, NCG = THREADS / 128;  // (16 warps per SM either way)
-  static constexpr uint32_t WT = 0, U = L::TILE_W, DY = U + 2 * L::TILE_U, TAPS = DY + 2 * L::TILE_U, BAR = TAPS + D * 16;
+  static constexpr uint32_t WT = 0, U = L::TILE_W, DY = U + 2 * L::TILE_U, ST = DY + 2 * L::TILE_U;  // ST: 64 columns of fp32 rows on their way out
+  static constexpr uint32_t ST_ROW = 272, TAPS = ST + TT * ST_ROW, BAR = TAPS + 2 * D * 16;                              // taps of two steps
   static constexpr uint32_t BYTES = BAR + 64;
-  static constexpr uint32_t DUQ = 0, DUK = D, DWC = 2 * D, COLS = D == 128 ? 512 : 256;
+  static constexpr uint32_t DUQ = 0, DUK = D, DWC = 2 * D, COLS = 4 * D;  // (DWC: two accumulators)
 };
 
 template <int D>
@@ -955,9 +960,8 @@ __global__ void __launch_bounds__(MCfg<D>::THREADS, D == 128 ? 1 : 2) mix_bwd_ke
   using M = MCfg<D>;
   extern __shared__ __align__(128) uint8_t sg[];
   const uint32_t sb = smem_u32(sg);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   volatile int* const s_fl = reinterpret_cast<volatile int*>(sg + M::BAR + 16);  // tmem base, abort
-  uint8_t* const s_taps = sg + M::TAPS;
   const int t0 = blockIdx.x * TT, bj = blockIdx.z * gridDim.y + blockIdx.y, j = bj % a.Hkv, b = bj / a.Hkv, G = a.H / a.Hkv;
   if (b >= a.B) return;
   const int nvalid = min(TT, a.T - t0);
@@ -991,157 +995,220 @@ __global__ void __launch_bounds__(MCfg<D>::THREADS, D == 128 ? 1 : 2) mix_bwd_ke
   }
   const int sg_group = sg_of(warp_max(whi));
   const bool spread = __any_sync(0xffffffffu, sg_of(-warp_max(wlo)) - sg_group > 4);
-  int sg_at = sg_group;
-  float sc = pow2i(sg_at), isc = pow2i(-sg_at);
-  const int o = tid % L::OPR, rr0 = tid / L::OPR;
-  constexpr int RSTEP = NTH / L::OPR, RPT = TT / RSTEP;
-  // fp32 [128][D] accumulator to global rows through the (dead) dy tiles
-  auto rows_out = [&](uint32_t col, float* dst, int NH, int head) {
-    float d[8];
-#pragma unroll 1
-    for (int c0 = cg * HC; c0 < (cg + 1) * HC; c0 += 8) {
-      tmem_ld8(lane_base + col + c0, d);
-      tmem_wait_ld();
-#pragma unroll
-      for (int i = 0; i < 8; i += 4)
-        *reinterpret_cast<float4*>(sg + M::DY + foff<D>(row, (c0 + i) >> 2)) = make_float4(d[i] * isc, d[i + 1] * isc, d[i + 2] * isc, d[i + 3] * isc);
-    }
-    tc_fence_before_sync();
-    __syncthreads();
-    tc_fence_after_sync();
-    for (int idx = tid; idx < nvalid * (D / 4); idx += NTH) {
-      const int pc = idx % (D / 4), r = idx / (D / 4);
-      *reinterpret_cast<float4*>(dst + (((size_t)b * a.T + t0 + r) * NH + head) * D + pc * 4) =
-          *reinterpret_cast<const float4*>(sg + M::DY + foff<D>(r, pc));
-    }
-    __syncthreads();
+  auto scale_of = [&](int g) -> int {
+    if (!spread) return sg_group;
+    const int own = sg_of(wmax[g]);
+    return own - sg_group <= 4 ? sg_group : min(own, sg_group + 60);
   };
-  // The group's heads, once with and once without a power of two per head. The choice is a vote, which the compiler knows to be
-  // uniform; a branch that it must take for divergent slows down all that stands behind it (4 x 1300 tokens, 32/8 heads of 128:
-  // no choice 288.2 us, this 289.3, one loop with the rescaling inside 292, a choice that is no vote 293.5).
-  auto heads = [&](auto spreadc) {
+  const int o = tid % L::OPR, rr0 = tid / L::OPR;
+  constexpr int RSTEP = NTH / L::OPR, RPT = TT / RSTEP, WPT = D * L::OPR / NTH;
+  // fp32 accumulators leave 64 columns at a time through the staging tile (rows of 272 bytes: the lanes that write own rows)
+  auto stage = [&](uint32_t col, int h64, float isc) {
+    if (cg * HC >= h64 && cg * HC < h64 + 64) {  // (whole warps)
+      float d[16];
 #pragma unroll 1
-    for (int g = 0; g < G; ++g) {
-      const int h = j * G + g;
-      if constexpr (decltype(spreadc)::value) {
-        const int own = sg_of(wmax[g]), sgm = own - sg_group <= 4 ? sg_group : min(own, sg_group + 60);
-        if (g > 0 && sgm != sg_at) {  // the key stream's du so far, on this head's scale
-          const float f = pow2i(sgm - sg_at);
-          float d[8];
-#pragma unroll 1
-          for (int c0 = cg * HC; c0 < (cg + 1) * HC; c0 += 8) {
-            tmem_ld8(lane_base + M::DUK + c0, d);
-            tmem_wait_ld();
+      for (int c0 = cg * HC; c0 < (cg + 1) * HC; c0 += 16) {
+        tmem_ld16(lane_base + col + c0, d);
+        tmem_wait_ld();
 #pragma unroll
-            for (int i = 0; i < 8; ++i) d[i] *= f;
-            tmem_st8(lane_base + M::DUK + c0, d);
-          }
-          tmem_wait_st();
-        }
-        sg_at = sgm;
-        sc = pow2i(sgm);
-        isc = pow2i(-sgm);
+        for (int i = 0; i < 16; i += 4)
+          *reinterpret_cast<float4*>(sg + M::ST + row * M::ST_ROW + (c0 - h64 + i) * 4) = make_float4(d[i] * isc, d[i + 1] * isc, d[i + 2] * isc, d[i + 3] * isc);
       }
-      load_w_tile<D>(sg + M::WT, a.W + (size_t)h * D * D, tid, NTH);
+    }
+  };
+  // du. Width 64: the bulk-copy engine takes the rows on from the staging tile, behind the block's other work (8 x 1024 tokens: the
+  // kernel 131 us; 138 by the threads). Width 128, where a tile is two trips through staging that would wait for one another: by the
+  // threads (4 x 1300 tokens: 238 us; 244).
+  auto du_out = [&](uint32_t col, float* dst, int NH, int head, float isc) {
+    if constexpr (D == 64) {
+      stage(col, 0, isc);
+      fence_proxy_async();
+      __syncthreads();
+      if (tid < nvalid) {
+        float* const p = dst + (((size_t)b * a.T + t0 + tid) * NH + head) * D;
+        asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], 256;" ::"l"(p), "r"(sb + M::ST + tid * M::ST_ROW) : "memory");
+        tma_store_commit();
+      }
+    } else {
 #pragma unroll 1
-      for (int stream = 0; stream < 2; ++stream) {
-        const bf16* w = stream ? a.w_k : a.w_q;
-        const int NH = stream ? a.Hkv : a.H, head = stream ? j : h;
-        load_taps<D>(s_taps, w, head, a.K, tid, NTH);
-        // the rows of the next (head, stream) step travel towards L2 while this one is computed
-        if (g + stream < G) {
-          const int nh = h + stream;
-          const float* wn = stream ? a.wq : a.wk;
-          const float* pn = stream ? a.qd : a.kd;
-          constexpr int LF = D * 4 / 128;
-          for (int idx = tid; idx < nvalid * 2 * LF; idx += NTH) {
-            const int r = idx / (2 * LF), l = idx % (2 * LF);
-            prefetch_l2((l < LF ? wn : pn) + (((size_t)b * a.T + t0 + r) * a.H + nh) * D + (l % LF) * 32);
-          }
-          if (stream && tid < nvalid) {
-            const bf16* xn = a.q + (((size_t)b * a.T + t0 + tid) * a.H + nh) * D;
-            prefetch_l2(xn);
-            if (D == 128) prefetch_l2(xn + 64);
-          }
-        }
-        // ---- dy
-        {
-          const float* wp = stream ? a.wk : a.wq;
-          const float* pp = stream ? a.kd : a.qd;
-#pragma unroll 4
-          for (int r = rr0; r < TT; r += RSTEP) {
-            float wv[8], pv[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) wv[i] = pv[i] = 0.f;
-            if (r < nvalid) {
-              const size_t at = (((size_t)b * a.T + t0 + r) * a.H + h) * D + o * 8;
-              load_row8(wp + at, wv);
-              load_row8(pp + at, pv);
-            }
-            float s = 0.f;
-#pragma unroll
-            for (int i = 0; i < 8; ++i) s += wv[i];
-#pragma unroll
-            for (int off = 1; off < L::OPR; off <<= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) wv[i] = fmaf(-pv[i], s, wv[i]) * sc;
-            uint4 hi, lo;
-            split8h(wv, true, hi, lo);
-            *reinterpret_cast<uint4*>(sg + M::DY + toff(L::SLAB_U, r, o * 8)) = hi;
-            *reinterpret_cast<uint4*>(sg + M::DY + L::TILE_U + toff(L::SLAB_U, r, o * 8)) = lo;
-          }
-        }
-        uint4 raw[RPT + HALO];
-        conv_load<D, RPT>(raw, stream ? a.k : a.q, stream ? a.cache_k : a.cache_q, b, t0 + rr0 * RPT, a.T, NH, head, a.K, o);
-        __syncthreads();  // (the taps)
-        // ---- u
-        conv_emit<D, RPT>(raw, s_taps, o, [&](int i, const uint64_t* u2) {
-          uint4 hi, lo;
-          float u[8];
-          pairs_to_floats(u2, u);
-          split8h(u, true, hi, lo);
-          const uint32_t at = toff(L::SLAB_U, rr0 * RPT + i, o * 8);
-          *reinterpret_cast<uint4*>(sg + M::U + at) = hi;
-          *reinterpret_cast<uint4*>(sg + M::U + L::TILE_U + at) = lo;
-        });
-        fence_proxy_async();
-        tc_fence_before_sync();
+      for (int h64 = 0; h64 < D; h64 += 64) {
+        stage(col, h64, isc);
         __syncthreads();
-        tc_fence_after_sync();
-        if (tid == 0) {
-          mm.split(stream ? M::DUK : M::DUQ, kview(sb + M::DY, L::SLAB_U), kview(sb + M::DY + L::TILE_U, L::SLAB_U), 2 * L::SLAB_U,
-                   kview(sb + M::WT, L::SLAB_W), 0, 2 * L::SLAB_W, D / 16, instr_desc(128, D, FMT_F16, MAJOR_K, MAJOR_K),
-                   stream == 1 && g > 0);
-          mm.split(M::DWC, mview(sb + M::U, L::SLAB_U), mview(sb + M::U + L::TILE_U, L::SLAB_U), 256, mview(sb + M::DY, L::SLAB_U),
-                   mview(sb + M::DY + L::TILE_U, L::SLAB_U), 256, TT / 16, instr_desc(128, D, FMT_F16, MAJOR_MN, MAJOR_MN), stream == 1);
-          mma_commit(sb + M::BAR);
+#pragma unroll 4
+        for (int idx = tid; idx < nvalid * 16; idx += NTH) {
+          const int pc = idx % 16, r = idx / 16;
+          *reinterpret_cast<float4*>(dst + (((size_t)b * a.T + t0 + r) * NH + head) * D + h64 + pc * 4) =
+              *reinterpret_cast<const float4*>(sg + M::ST + r * M::ST_ROW + pc * 16);
         }
-        wt.wait();
-        if (stream == 0) rows_out(M::DUQ, a.wq, a.H, h);
+        __syncthreads();
       }
-      // dW of the head: row c of the accumulator belongs to lane c
-      if (a.dW && row < D) {
+    }
+  };
+  // dW of a head, row c of the accumulator being row c of dW. Width 64: the bulk-copy engine adds the rows, behind the block's other
+  // work. Width 128, where a row would be two trips through the staging tile: added from where they are.
+  auto dw_out = [&](int g) {
+    if (!a.dW) return;
+    float* const dst = a.dW + ((size_t)(j * G + g) * D + (row < D ? row : 0)) * D;
+    const float isc = pow2i(-scale_of(g));
+    if constexpr (D == 64) {
+      stage(M::DWC + (g & 1) * D, 0, isc);
+      fence_proxy_async();
+      __syncthreads();
+      if (tid < D) {
+        asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], 256;" ::"l"(dst), "r"(sb + M::ST + tid * M::ST_ROW) : "memory");
+        tma_store_commit();
+      }
+    } else {
+      float d[8];
+#pragma unroll 1
+      for (int c0 = cg * HC; c0 < (cg + 1) * HC; c0 += 8) {
+        tmem_ld8(lane_base + M::DWC + (g & 1) * D + c0, d);
+        tmem_wait_ld();
+#pragma unroll
+        for (int i = 0; i < 8; i += 4)
+          asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + c0 + i), "f"(d[i] * isc), "f"(d[i + 1] * isc),
+                       "f"(d[i + 2] * isc), "f"(d[i + 3] * isc)
+                       : "memory");
+      }
+    }
+  };
+  auto taps = [&](int s) {  // of step s into its slot
+    if (s < 2 * G) load_taps<D>(sg + M::TAPS + (s & 1) * D * 16, s & 1 ? a.w_k : a.w_q, s & 1 ? j : j * G + (s >> 1), a.K, tid, NTH);
+  };
+  uint4 dyh[RPT], dyl[RPT], uh[RPT], ul[RPT];  // a step's operands: this thread's octets of dy and u, hi and lo
+  auto operands = [&](int s) {
+    const int g = s >> 1, stream = s & 1, h = j * G + g;
+    const float sc = pow2i(scale_of(g));
+    const float* wp = stream ? a.wk : a.wq;
+    const float* pp = stream ? a.kd : a.qd;
+    float4 wr[RPT][2], pr[RPT][2];  // (all loads of a step in flight together: they are what a step takes longest over)
+#pragma unroll
+    for (int k = 0; k < RPT; ++k) {
+      const int r = rr0 + k * RSTEP;
+      const size_t at = (((size_t)b * a.T + t0 + min(r, nvalid - 1)) * a.H + h) * D + o * 8;
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        wr[k][i] = *reinterpret_cast<const float4*>(wp + at + 4 * i);
+        pr[k][i] = *reinterpret_cast<const float4*>(pp + at + 4 * i);
+      }
+    }
+    uint4 raw[RPT + HALO];
+    conv_load<D, RPT>(raw, stream ? a.k : a.q, stream ? a.cache_k : a.cache_q, b, t0 + rr0 * RPT, a.T, stream ? a.Hkv : a.H, stream ? j : h, a.K, o);
+    // the rows of the step behind travel towards L2 meanwhile
+    if (s + 1 < 2 * G) {
+      const int nh = h + stream;
+      const float* wn = stream ? a.wq : a.wk;
+      const float* pn = stream ? a.qd : a.kd;
+      constexpr int LF = D * 4 / 128;
+      for (int idx = tid; idx < nvalid * 2 * LF; idx += NTH) {
+        const int r = idx / (2 * LF), l = idx % (2 * LF);
+        prefetch_l2((l < LF ? wn : pn) + (((size_t)b * a.T + t0 + r) * a.H + nh) * D + (l % LF) * 32);
+      }
+      if (stream && tid < nvalid) {
+        const bf16* xn = a.q + (((size_t)b * a.T + t0 + tid) * a.H + nh) * D;
+        prefetch_l2(xn);
+        if (D == 128) prefetch_l2(xn + 64);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < RPT; ++k) {
+      const float on = rr0 + k * RSTEP < nvalid ? sc : 0.f;
+      float wv[8] = {wr[k][0].x, wr[k][0].y, wr[k][0].z, wr[k][0].w, wr[k][1].x, wr[k][1].y, wr[k][1].z, wr[k][1].w};
+      const float pv[8] = {pr[k][0].x, pr[k][0].y, pr[k][0].z, pr[k][0].w, pr[k][1].x, pr[k][1].y, pr[k][1].z, pr[k][1].w};
+      float s8 = 0.f;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) s8 += wv[i];
+#pragma unroll
+      for (int off = 1; off < L::OPR; off <<= 1) s8 += __shfl_xor_sync(0xffffffffu, s8, off);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) wv[i] = on != 0.f ? fmaf(-pv[i], s8, wv[i]) * on : 0.f;
+      split8h(wv, true, dyh[k], dyl[k]);
+    }
+    conv_emit<D, RPT>(raw, sg + M::TAPS + stream * D * 16, o, [&](int i, const uint64_t* u2) {
+      float u[8];
+      pairs_to_floats(u2, u);
+      split8h(u, true, uh[i], ul[i]);
+    });
+  };
+  taps(0);
+  load_w_tile<D>(sg + M::WT, a.W + (size_t)j * G * D * D, tid, NTH);
+  __syncthreads();
+  operands(0);
+  int sg_at = scale_of(0);  // power of two on the key stream's du so far
+#pragma unroll 1
+  for (int s = 0; s < 2 * G; ++s) {
+    const int g = s >> 1, stream = s & 1, h = j * G + g;
+    uint4 wreg[WPT];
+    const bool next_w = stream == 0 && s > 0;
+    if (next_w) {
+#pragma unroll
+      for (int k = 0; k < WPT; ++k) wreg[k] = *reinterpret_cast<const uint4*>(a.W + (size_t)h * D * D + (size_t)(tid + k * NTH) * 8);
+    }
+    if (s > 0) wt.wait();  // the products of the step in front: its operands and W_h have been read
+    if (next_w) {
+#pragma unroll
+      for (int k = 0; k < WPT; ++k) {
+        const int idx = tid + k * NTH;
+        float f[8];
+        unpack8b(wreg[k], f);
+        *reinterpret_cast<uint4*>(sg + M::WT + toff(L::SLAB_W, idx / L::OPR, idx % L::OPR * 8)) = pack8f16(f);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < RPT; ++k) {
+      const uint32_t ady = toff(L::SLAB_U, rr0 + k * RSTEP, o * 8), au = toff(L::SLAB_U, rr0 * RPT + k, o * 8);
+      *reinterpret_cast<uint4*>(sg + M::DY + ady) = dyh[k];
+      *reinterpret_cast<uint4*>(sg + M::DY + L::TILE_U + ady) = dyl[k];
+      *reinterpret_cast<uint4*>(sg + M::U + au) = uh[k];
+      *reinterpret_cast<uint4*>(sg + M::U + L::TILE_U + au) = ul[k];
+    }
+    const int sgm = scale_of(g);
+    if (stream == 0 && sgm != sg_at) {  // the key stream's du so far, on this head's scale (the choice of powers is uniform)
+      if (g > 0) {
+        const float f = pow2i(sgm - sg_at);
         float d[8];
 #pragma unroll 1
         for (int c0 = cg * HC; c0 < (cg + 1) * HC; c0 += 8) {
-          tmem_ld8(lane_base + M::DWC + c0, d);
+          tmem_ld8(lane_base + M::DUK + c0, d);
           tmem_wait_ld();
-          float* dst = a.dW + ((size_t)h * D + row) * D + c0;
 #pragma unroll
-          for (int i = 0; i < 8; i += 4)
-            asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + i), "f"(d[i] * isc), "f"(d[i + 1] * isc),
-                         "f"(d[i + 2] * isc), "f"(d[i + 3] * isc)
-                         : "memory");
+          for (int i = 0; i < 8; ++i) d[i] *= f;
+          tmem_st8(lane_base + M::DUK + c0, d);
         }
+        tmem_wait_st();
       }
-      tc_fence_before_sync();
+      sg_at = sgm;
+    }
+    taps(s + 1);
+    if (D == 64 && tid < TT) tma_store_wait_read();  // (the rows of the step in front have left the staging tile)
+    fence_proxy_async();
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+    if (warp == 0 && elect_one()) {
+      mm.split(stream ? M::DUK : M::DUQ, kview(sb + M::DY, L::SLAB_U), kview(sb + M::DY + L::TILE_U, L::SLAB_U), 2 * L::SLAB_U,
+               kview(sb + M::WT, L::SLAB_W), 0, 2 * L::SLAB_W, D / 16, instr_desc(128, D, FMT_F16, MAJOR_K, MAJOR_K),
+               stream == 1 && g > 0);
+      mm.split(M::DWC + (g & 1) * D, mview(sb + M::U, L::SLAB_U), mview(sb + M::U + L::TILE_U, L::SLAB_U), 256, mview(sb + M::DY, L::SLAB_U),
+               mview(sb + M::DY + L::TILE_U, L::SLAB_U), 256, TT / 16, instr_desc(128, D, FMT_F16, MAJOR_MN, MAJOR_MN), stream == 1);
+      mma_commit(sb + M::BAR);
+    }
+    if (stream) du_out(M::DUQ, a.wq, a.H, h, pow2i(-sgm));
+    else if (g > 0) dw_out(g - 1);
+    if (s + 1 < 2 * G) operands(s + 1);
+  }
+  wt.wait();
+  auto staging_free = [&]() {
+    if (D == 64) {
+      if (tid < TT) tma_store_wait_read();
       __syncthreads();
-      tc_fence_after_sync();
     }
   };
-  if (spread) heads(std::true_type{});
-  else heads(std::false_type{});
-  rows_out(M::DUK, a.du_k, a.Hkv, j);
+  staging_free();
+  dw_out(G - 1);
+  staging_free();
+  du_out(M::DUK, a.du_k, a.Hkv, j, pow2i(-sg_at));
+  if (D == 64 && tid < TT) tma_store_wait_all();
   tc_fence_before_sync();
   __syncthreads();
   if (warp == 0) {
