@@ -1,5 +1,6 @@
 // Shared device/host helpers of the LAWCAT CUDA library (sm_100a).
 #pragma once
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -79,6 +80,9 @@ size_t decode_workspace_bytes(const lawcat_params& p);
 int sm_count();  // of the current device (layer_tc.cu)
 long long wait_limit();  // bound of the device-side waits in clock cycles (layer_tc.cu; a test hook may shorten it)
 int validate_params(const lawcat_params* p, bool need_T);
+// [B, T, heads, dh] tensor (fp32 or bf16) as a 4-D map (channel, head, token, batch) with boxes of box_ch channels x rows tokens;
+// kept per host thread for the last few pointers and shapes (layer_tc.cu)
+bool tensor_map(CUtensorMap* m, const void* ptr, bool f32, int heads, int T, int B, int dh, int box_ch, int rows, bool swizzle);
 
 // Chunkwise tensor-core layer forward (layer_tc.cu): whether it takes these parameters, and its launcher.
 bool layer_tc_supported(const lawcat_params& p);

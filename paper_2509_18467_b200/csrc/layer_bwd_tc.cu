@@ -64,6 +64,10 @@ struct Args {
   float inv_tau, eps;
 };
 
+struct Maps {  // tensor maps [B,T,heads,D]: whole rows of 64 tokens for the prefetch, 32 fp32 channels x 64 tokens for the stores
+  CUtensorMap qd, kd, v, dO, wq, wk, dvh;
+};
+
 template <int D>
 struct Cfg {
   static constexpr int THREADS = D == 128 ? 512 : 256, OCT = D / 8, NCG = THREADS / 128;  // NCG: column groups of row threads
@@ -78,7 +82,8 @@ struct Cfg {
   static constexpr uint32_t F_BYTES = F_VEC + 4 * D * 4 + NCG * C * 4 + 64;
   static constexpr uint32_t F_X = F_S;           // exponents, fp32 [C][D]: dead before the state operand is written
   // reverse sweep
-  static constexpr uint32_t R_QS = 0, R_KS = R_QS + 2 * T_TOK, R_V = R_KS + 2 * T_TOK, R_DO = R_V + T_TOK, R_PM = R_DO + T_TOK;
+  static constexpr uint32_t R_QS = 0, R_KS = R_QS + 2 * T_TOK, R_V = R_KS + 2 * T_TOK, R_DO = R_V + T_TOK,
+                            R_PM = (R_DO + T_TOK + 1023) / 1024 * 1024;  // (result tiles that lie here and behind are swizzled)
   static constexpr uint32_t R_E = R_PM + 2 * T_P, R_S = R_E + 2 * T_P, R_VEC = R_S + 2 * T_C;
   static constexpr uint32_t R_BYTES = R_VEC + 8 * D * 4 + 2 * C * 4 + (THREADS / 32) * D * 4 + 96;
   static constexpr uint32_t R_X = R_S;
@@ -94,9 +99,9 @@ struct Cfg {
 __device__ __forceinline__ float pow2i(int e) { return __int_as_float((min(max(e, -126), 127) + 127) << 23); }
 // smallest e with |x| < 2^e (x > 0)
 __device__ __forceinline__ int exp_above(float x) { return ((__float_as_int(x) >> 23) & 0xff) - 126; }
-// piece pc (16 bytes) of row r of an fp32 [C][D] tile, swizzled so that lanes that own rows spread over the banks
-template <int D>
-__device__ __forceinline__ uint32_t foff(int r, int pc) { return (uint32_t)(r * (D * 4) + ((pc ^ (r & 7)) << 4)); }
+// piece pc (16 bytes) of row r of an fp32 [C][D] tile: slabs of 32 columns, 128-byte-swizzled as the copy engine stores them, so that
+// lanes that own rows spread over the banks
+__device__ __forceinline__ uint32_t foff(int r, int pc) { return (uint32_t)((pc >> 3) * (C * 128)) + sw128(r, pc & 7); }
 
 // A chunk's gate entries as they lie in memory, two octets per thread (gate_dim = 1: the token's entry as fp32 bits), fetched
 // while the chunk in front is computed.
@@ -179,24 +184,14 @@ __device__ __forceinline__ void gate_pass(const Args& a, const Gates<D>& raw, in
   __syncthreads();
 }
 
-// One chunk's rows towards L2, issued by the warps that wait for a batch of products (the first warp issues them): the chunk
-// that follows travels while this one is computed. Line by line: the bulk prefetch of a row takes hundreds of cycles to issue.
-template <int D>
-__device__ __forceinline__ void prefetch_chunk(const Args& a, int b, int h, int j, int t0, int tid) {
-  constexpr int LF = D * 4 / 128, LB = D * 2 / 128, PER = 2 * LF + 2 * LB, NT = Cfg<D>::THREADS - 32;  // lines per token
-  if (t0 < 0 || tid < 32) return;
-#pragma unroll 2
-  for (int idx = tid - 32; idx < C * PER; idx += NT) {
-    const int r = idx / PER, l = idx % PER;
-    if (t0 + r >= a.T) return;
-    const size_t th = ((size_t)b * a.T + t0 + r) * a.H + h, tv = ((size_t)b * a.T + t0 + r) * a.Hkv + j;
-    const char* p;
-    if (l < LF) p = (const char*)(a.qd + th * D) + l * 128;
-    else if (l < 2 * LF) p = (const char*)(a.kd + th * D) + (l - LF) * 128;
-    else if (l < 2 * LF + LB) p = (const char*)(a.v + tv * D) + (l - 2 * LF) * 128;
-    else p = (const char*)(a.dO + th * D) + (l - 2 * LF - LB) * 128;
-    prefetch_l2(p);
-  }
+// One chunk's rows towards L2, by one thread and four instructions while a batch of products is under way: the chunk that follows
+// travels while this one is computed. (Line by line, by the warps that wait, it took them 5k cycles a chunk at width 128, longer than
+// the products.)
+__device__ __forceinline__ void prefetch_chunk(const Maps& m, int b, int h, int j, int t0) {
+  tma_prefetch_4d(&m.qd, 0, h, t0, b);
+  tma_prefetch_4d(&m.kd, 0, h, t0, b);
+  tma_prefetch_4d(&m.v, 0, j, t0, b);
+  tma_prefetch_4d(&m.dO, 0, h, t0, b);
 }
 
 // A chunk's rows as they lie in memory, two octets per thread, loaded before the gate pass so that they arrive behind it.
@@ -245,7 +240,7 @@ struct Mma {
 
 // ------------------------------------------------------------------------------------------------ forward sweep
 template <int D>
-__global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) sweep_kernel(const Args a) {
+__global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) sweep_kernel(const Args a, const __grid_constant__ Maps maps) {
   using F = Cfg<D>;
   constexpr int NV = D + 16;
   extern __shared__ __align__(128) uint8_t sg[];
@@ -256,11 +251,12 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) sweep_kerne
   float *const s_ft = s_bm + D, *const s_pe = s_ft + D;  // s_pe: ft of the chunk in front (its state is still 2^-ft short)
   float* const s_row = s_pe + 2 * D;                     // [NCG][C]
   volatile int* const s_fl = reinterpret_cast<volatile int*>(s_row + F::NCG * C);  // tmem base, abort, rmax, smax, vmax, domax, dlmax
-  const uint32_t bar = smem_u32(const_cast<int*>(s_fl)) + 32;
+  const uint32_t bar = smem_u32(const_cast<int*>(s_fl)) + 32, bar_p = bar + 8;
   const int bh = blockIdx.x, h = bh % a.H, b = bh / a.H, G = a.H / a.Hkv, j = h / G;
   const int nch = (a.T + C - 1) / C;
   if (tid == 0) {
     mbar_init(bar, 1);
+    mbar_init(bar_p, 1);
     mbar_fence_init();
     for (int i = 1; i < 7; ++i) s_fl[i] = 0;
   }
@@ -283,7 +279,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) sweep_kerne
   const uint32_t lane_base = mm.tmem + ((uint32_t)((warp & 3) * 32) << 16);
   const int row = (warp & 3) * 32 + lane, cg = warp >> 2;  // TMEM lane, column group
   const bool tok_thr = row < C, st_thr = row < D;          // owns a token row / a state row
-  Waiter wt{bar, 0u, s_fl + 1, a.dev_status};
+  Waiter wt{bar, 0u, s_fl + 1, a.dev_status}, wp{bar_p, 0u, s_fl + 1, a.dev_status};
   constexpr int SW = D / F::NCG, TW = 64 / F::NCG;         // columns per thread of a state row, of a score row
   auto publish = [&]() {
     fence_proxy_async();
@@ -428,15 +424,16 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) sweep_kerne
     if (warp == 0 && elect_one()) {
       mm.split(F::F_P, KV(F::F_QS, F::SL_T), KV(F::F_QS + F::T_TOK, F::SL_T), 2 * F::SL_T, KV(F::F_KS, F::SL_T),
                KV(F::F_KS + F::T_TOK, F::SL_T), 2 * F::SL_T, D / 16, instr_desc(128, C, fmt, MAJOR_K, MAJOR_K), false);
+      mma_commit(bar_p);
       mm.split(F::F_O, KV(F::F_QS, F::SL_T), KV(F::F_QS + F::T_TOK, F::SL_T), 2 * F::SL_T, MV(F::F_S, F::SL_C),
                MV(F::F_S + F::T_SZ, F::SL_C), 256, D / 16, instr_desc(128, NV, fmt, MAJOR_K, MAJOR_MN), false);
       // (the state in tensor memory is 2^kap-scaled like ks)
       mm.split(F::F_ST, MV(F::F_KS, F::SL_T), MV(F::F_KS + F::T_TOK, F::SL_T), 256, MV(F::F_V, F::SL_T), 0, 256, C / 16,
                instr_desc(128, NV, fmt, MAJOR_MN, MAJOR_MN), true);
-      mma_commit(bar);
     }
-    if (n + 1 < nch) prefetch_chunk<D>(a, b, h, j, t0 + C, tid);
-    wt.wait();
+    gates.load(a, b, h, t0 + C, tid);  // (early: these rows are not prefetched)
+    if (tid == 32 && n + 1 < nch) prefetch_chunk(maps, b, h, j, t0 + C);
+    wp.wait();  // (the scores alone: the mask runs behind the read-out and the state update)
     // ---- mask
     if (tok_thr) {
       float s[16];
@@ -463,7 +460,6 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) sweep_kerne
       mma_commit(bar);
     }
     // |next state| <= |2^bm state| + 64 max|v|: every key enters with a factor <= 1
-    gates.load(a, b, h, t0 + C, tid);
     const float vm = __int_as_float(s_fl[4]), sm = __int_as_float(s_fl[3]) * pow2i(-kap);
     wt.wait();
     // ---- 1 / den and dO . o of the chunk's rows
@@ -531,10 +527,10 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) sweep_kerne
 
 // ------------------------------------------------------------------------------------------------ reverse sweep
 template <int D>
-__global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_kernel(const Args a) {
+__global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_kernel(const Args a, const __grid_constant__ Maps maps) {
   using F = Cfg<D>;
   constexpr int NW = F::THREADS / 32;
-  extern __shared__ __align__(128) uint8_t sg[];
+  extern __shared__ __align__(1024) uint8_t sg[];
   const uint32_t sb = smem_u32(sg);
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;  // (warp: uniform to the compiler)
   float* const s_x = reinterpret_cast<float*>(sg + F::R_X);
@@ -755,7 +751,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
                false);
       mma_commit(bar);
     }
-    prefetch_chunk<D>(a, b, h, j, t0 - C, tid);
+    if (tid == 32 && n > 0) prefetch_chunk(maps, b, h, j, t0 - C);
     wt.wait();
     // ---- adjoint pass, over the consumed state operand
     if (st_thr) {
@@ -817,8 +813,8 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
           }
 #pragma unroll
           for (int i = 0; i < 8; i += 4) {
-            *reinterpret_cast<float4*>(sg + F::R_WQ + foff<D>(row, (c0 + i) >> 2)) = make_float4(dq[i8 + i], dq[i8 + i + 1], dq[i8 + i + 2], dq[i8 + i + 3]);
-            *reinterpret_cast<float4*>(sg + F::R_WK + foff<D>(row, (c0 + i) >> 2)) = make_float4(dk[i8 + i], dk[i8 + i + 1], dk[i8 + i + 2], dk[i8 + i + 3]);
+            *reinterpret_cast<float4*>(sg + F::R_WQ + foff(row, (c0 + i) >> 2)) = make_float4(dq[i8 + i], dq[i8 + i + 1], dq[i8 + i + 2], dq[i8 + i + 3]);
+            *reinterpret_cast<float4*>(sg + F::R_WK + foff(row, (c0 + i) >> 2)) = make_float4(dk[i8 + i], dk[i8 + i + 1], dk[i8 + i + 2], dk[i8 + i + 3]);
           }
         }
       }
@@ -828,12 +824,19 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
         tmem_wait_ld();
 #pragma unroll
         for (int i = 0; i < 32; i += 4)
-          *reinterpret_cast<float4*>(sg + F::R_DV + foff<D>(row, (cg * SW + i) >> 2)) = make_float4(d[i] * usc, d[i + 1] * usc, d[i + 2] * usc, d[i + 3] * usc);
+          *reinterpret_cast<float4*>(sg + F::R_DV + foff(row, (cg * SW + i) >> 2)) = make_float4(d[i] * usc, d[i + 1] * usc, d[i + 2] * usc, d[i + 3] * usc);
       }
     }
-    tc_fence_before_sync();
-    __syncthreads();
-    tc_fence_after_sync();
+    publish();
+    if (tid == 0) {  // whole rows to memory by the copy engine (rows past the end are clipped)
+#pragma unroll 1
+      for (int c0 = 0; c0 < D; c0 += 32) {
+        tma_store_4d(&maps.wq, sb + F::R_WQ + c0 * (C * 4), c0, h, t0, b);
+        tma_store_4d(&maps.wk, sb + F::R_WK + c0 * (C * 4), c0, h, t0, b);
+        tma_store_4d(&maps.dvh, sb + F::R_DV + c0 * (C * 4), c0, h, t0, b);
+      }
+      tma_store_commit();
+    }
     uint4 graw[2];  // this chunk's gate again, for the derivative of the log-decays
 #pragma unroll
     for (int it = 0; it < 2; ++it) {
@@ -848,7 +851,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
       float v[RT], acc = 0.f;
 #pragma unroll
       for (int i = RT - 1; i >= 0; --i) {
-        const uint32_t at = foff<D>(run * RT + i, c >> 2) + (c & 3) * 4;
+        const uint32_t at = foff(run * RT + i, c >> 2) + (c & 3) * 4;
         acc += *reinterpret_cast<const float*>(sg + F::R_WQ + at) - *reinterpret_cast<const float*>(sg + F::R_WK + at);
         v[i] = acc;
       }
@@ -862,21 +865,9 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
         all += t;
       }
 #pragma unroll
-      for (int i = 0; i < RT; ++i) *reinterpret_cast<float*>(sg + F::R_DG + foff<D>(run * RT + i, c >> 2) + (c & 3) * 4) = v[i] + off;
+      for (int i = 0; i < RT; ++i) *reinterpret_cast<float*>(sg + F::R_DG + foff(run * RT + i, c >> 2) + (c & 3) * 4) = v[i] + off;
       __syncthreads();
       if (run == 0) s_car[c] = all;
-    }
-    // ---- whole rows to global memory
-#pragma unroll
-    for (int it = 0; it < C * (D / 4) / F::THREADS; ++it) {
-      const int idx = tid + it * F::THREADS, pc = idx % (D / 4), r = idx / (D / 4);
-      const size_t at = ((row0 + r) * a.H + h) * D + pc * 4;
-      const uint32_t so = foff<D>(r, pc);
-      if (r < nvalid) {
-        *reinterpret_cast<float4*>(a.wq + at) = *reinterpret_cast<const float4*>(sg + F::R_WQ + so);
-        *reinterpret_cast<float4*>(a.wk + at) = *reinterpret_cast<const float4*>(sg + F::R_WK + so);
-        *reinterpret_cast<float4*>(a.dvh + at) = *reinterpret_cast<const float4*>(sg + F::R_DV + so);
-      }
     }
     // d(log-decay) / d(gate entry): 1 - sigmoid(a) = 1 / (1 + e^a)
     auto dlog = [&](float av) {
@@ -885,7 +876,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
     if (a.gate_dim == 1) {
       for (int r = warp; r < nvalid; r += NW) {
         float s = 0.f;
-        for (int c = lane; c < D; c += 32) s += *reinterpret_cast<const float*>(sg + F::R_DG + foff<D>(r, c >> 2) + (c & 3) * 4);
+        for (int c = lane; c < D; c += 32) s += *reinterpret_cast<const float*>(sg + F::R_DG + foff(r, c >> 2) + (c & 3) * 4);
         s = warp_sum(s);
         if (lane == 0) {
           const size_t gi = (row0 + r) * a.H + h;
@@ -899,7 +890,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
         if (r >= nvalid) continue;
         float av[8], d[8];
         unpack8b(graw[it], av);
-        const float4 x = *reinterpret_cast<const float4*>(sg + F::R_DG + foff<D>(r, 2 * o)), y = *reinterpret_cast<const float4*>(sg + F::R_DG + foff<D>(r, 2 * o + 1));
+        const float4 x = *reinterpret_cast<const float4*>(sg + F::R_DG + foff(r, 2 * o)), y = *reinterpret_cast<const float4*>(sg + F::R_DG + foff(r, 2 * o + 1));
         d[0] = x.x; d[1] = x.y; d[2] = x.z; d[3] = x.w; d[4] = y.x; d[5] = y.y; d[6] = y.z; d[7] = y.w;
 #pragma unroll
         for (int i = 0; i < 8; ++i) d[i] *= dlog(av[i]);
@@ -907,6 +898,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
       }
     }
     al_prev = al;
+    if (tid == 0) tma_store_wait_read();  // (the next chunk writes over the result tiles)
     __syncthreads();
   }
   wmax = warp_max(wmax);
@@ -915,6 +907,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
   __syncthreads();
   if (tid == 0) {
     a.wmax[bh] = __int_as_float(s_fl[5]);
+    tma_store_wait_all();
     if (s_fl[1] && copied >= 0) mbar_wait(bar_s, (uint32_t)(copied & 1));  // (after a wait that ran out it may still be under way)
   }
   if (warp == 0) {
@@ -1269,16 +1262,16 @@ static int raise_limits() {
 }
 
 template <int D>
-static int run(const Ctx& c, const Args& a, const MArgs& m) {
+static int run(const Ctx& c, const Args& a, const Maps& maps, const MArgs& m) {
   const lawcat_params& p = *c.p;
   {
     LaunchScope _ls("layer_bwd_sweep", c.stream);
-    launch_behind(sweep_kernel<D>, dim3(p.B * p.H), dim3(Cfg<D>::THREADS), Cfg<D>::F_BYTES, c.stream, a);
+    launch_behind(sweep_kernel<D>, dim3(p.B * p.H), dim3(Cfg<D>::THREADS), Cfg<D>::F_BYTES, c.stream, a, maps);
     LAWCAT_CHECK_LAUNCH();
   }
   {
     LaunchScope _ls("layer_bwd_reverse", c.stream);
-    launch_behind(reverse_kernel<D>, dim3(p.B * p.H), dim3(Cfg<D>::THREADS), Cfg<D>::R_BYTES, c.stream, a);
+    launch_behind(reverse_kernel<D>, dim3(p.B * p.H), dim3(Cfg<D>::THREADS), Cfg<D>::R_BYTES, c.stream, a, maps);
     LAWCAT_CHECK_LAUNCH();
   }
   LaunchScope _ls("layer_bwd_mix", c.stream);
@@ -1323,7 +1316,14 @@ int launch_layer_bwd_tc(const Ctx& c, const void* q, const void* k, const void* 
   MArgs m{(const bf16*)q, (const bf16*)k, (const bf16*)w_q, (const bf16*)w_k, (const bf16*)W, (const bf16*)cache_q,
           (const bf16*)cache_k, a.qd, a.kd, a.wk, a.wq, (float*)(w + L.du_k), dW, a.wmax, c.dev_status, p.B, p.T, p.H, p.H_kv, p.conv_k};
   if ((r = launch_convmix_tc_fwd(c, q, k, w_q, w_k, W, cache_q, cache_k, (void*)a.qd, (void*)a.kd, true))) return r;
-  if ((r = p.d_k == 64 ? run<64>(c, a, m) : run<128>(c, a, m))) return r;
+  Maps maps;
+  const int D = p.d_k;
+  if (!tensor_map(&maps.qd, a.qd, true, p.H, p.T, p.B, D, D, C, false) || !tensor_map(&maps.kd, a.kd, true, p.H, p.T, p.B, D, D, C, false) ||
+      !tensor_map(&maps.v, v, false, p.H_kv, p.T, p.B, D, D, C, false) || !tensor_map(&maps.dO, dO, false, p.H, p.T, p.B, D, D, C, false) ||
+      !tensor_map(&maps.wq, a.wq, true, p.H, p.T, p.B, D, 32, C, true) || !tensor_map(&maps.wk, a.wk, true, p.H, p.T, p.B, D, 32, C, true) ||
+      !tensor_map(&maps.dvh, a.dvh, true, p.H, p.T, p.B, D, 32, C, true))
+    return LAWCAT_ERR_CUDA;
+  if ((r = D == 64 ? run<64>(c, a, maps, m) : run<128>(c, a, maps, m))) return r;
   {
     const int oct = p.d_v / 8;
     const size_t total = (size_t)p.B * p.T * p.H_kv * oct;

@@ -27,40 +27,51 @@ static EncodeTiledFn encode_fn() {
   return fn;
 }
 
-// [B, T, heads, dh] bf16 tensor as a 4-D map (channel, head, token, batch) with boxes of 64 channels x rows tokens.
+}  // namespace tc
+
 // A map depends only on the pointer and the shape, so the last few are kept per host thread: a serving loop that calls
 // with the same buffers encodes each map once.
-static bool make_map(CUtensorMap* m, const void* ptr, int heads, int T, int B, int rows, int dh) {
+bool tensor_map(CUtensorMap* m, const void* ptr, bool f32, int heads, int T, int B, int dh, int box_ch, int rows, bool swizzle) {
   struct Slot {
     const void* ptr;
-    int heads, T, B, rows, dh;
-    bool used;
+    int heads, T, B, dh, box_ch, rows;
+    bool f32, swizzle, used;
     CUtensorMap map;
   };
-  constexpr int NSLOT = 16;
+  constexpr int NSLOT = 32;
   thread_local Slot cache[NSLOT] = {};
   thread_local int next = 0;
   for (int i = 0; i < NSLOT; ++i) {
     const Slot& c = cache[i];
-    if (c.used && c.ptr == ptr && c.heads == heads && c.T == T && c.B == B && c.rows == rows && c.dh == dh) {
+    if (c.used && c.ptr == ptr && c.heads == heads && c.T == T && c.B == B && c.dh == dh && c.box_ch == box_ch && c.rows == rows &&
+        c.f32 == f32 && c.swizzle == swizzle) {
       *m = c.map;
       return true;
     }
   }
-  EncodeTiledFn fn = encode_fn();
+  tc::EncodeTiledFn fn = tc::encode_fn();
   if (!fn) return false;
+  const cuuint64_t row = (cuuint64_t)dh * (f32 ? 4 : 2);
   const cuuint64_t dims[4] = {(cuuint64_t)dh, (cuuint64_t)heads, (cuuint64_t)T, (cuuint64_t)B};
-  const cuuint64_t strides[3] = {(cuuint64_t)dh * 2, (cuuint64_t)heads * dh * 2, (cuuint64_t)T * heads * dh * 2};
-  const cuuint32_t box[4] = {64, 1, (cuuint32_t)rows, 1};
+  const cuuint64_t strides[3] = {row, heads * row, T * (heads * row)};
+  const cuuint32_t box[4] = {(cuuint32_t)box_ch, 1, (cuuint32_t)rows, 1};
   const cuuint32_t es[4] = {1, 1, 1, 1};
-  if (fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(ptr), dims, strides, box, es,
-         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+  if (fn(m, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(ptr), dims, strides, box, es,
+         CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
+         CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return false;
   Slot& c = cache[next];
   next = (next + 1) % NSLOT;
-  c.ptr = ptr; c.heads = heads; c.T = T; c.B = B; c.rows = rows; c.dh = dh; c.map = *m; c.used = true;
+  c.ptr = ptr; c.heads = heads; c.T = T; c.B = B; c.dh = dh; c.box_ch = box_ch; c.rows = rows; c.f32 = f32; c.swizzle = swizzle;
+  c.map = *m; c.used = true;
   return true;
+}
+
+namespace tc {
+
+// [B, T, heads, dh] bf16 tensor in boxes of 64 channels x rows tokens, 128-byte-swizzled
+static bool make_map(CUtensorMap* m, const void* ptr, int heads, int T, int B, int rows, int dh) {
+  return tensor_map(m, ptr, false, heads, T, B, dh, 64, rows, true);
 }
 
 // State at the start of every segment but a sequence's first from the end states of the pieces in front (each computed from a
