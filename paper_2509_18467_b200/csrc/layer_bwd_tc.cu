@@ -209,8 +209,8 @@ struct Rows {
       v[it] = g[it] = make_uint4(0u, 0u, 0u, 0u);
       if (r < nvalid) {
         const size_t tq = ((row0 + r) * a.H + h) * D + o * 8;
-        q[it][0] = *reinterpret_cast<const float4*>(a.qd + tq); q[it][1] = *reinterpret_cast<const float4*>(a.qd + tq + 4);
-        k[it][0] = *reinterpret_cast<const float4*>(a.kd + tq); k[it][1] = *reinterpret_cast<const float4*>(a.kd + tq + 4);
+        load_octet(a.qd + tq, q[it]);
+        load_octet(a.kd + tq, k[it]);
         v[it] = *reinterpret_cast<const uint4*>(a.v + ((row0 + r) * a.Hkv + j) * D + o * 8);
         if (REV) g[it] = *reinterpret_cast<const uint4*>(a.dO + tq);
       }
@@ -1079,11 +1079,8 @@ __global__ void __launch_bounds__(MCfg<D>::THREADS, D == 128 ? 1 : 2) mix_bwd_ke
     for (int k = 0; k < RPT; ++k) {
       const int r = rr0 + k * RSTEP;
       const size_t at = (((size_t)b * a.T + t0 + min(r, nvalid - 1)) * a.H + h) * D + o * 8;
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        wr[k][i] = *reinterpret_cast<const float4*>(wp + at + 4 * i);
-        pr[k][i] = *reinterpret_cast<const float4*>(pp + at + 4 * i);
-      }
+      load_octet(wp + at, wr[k]);
+      load_octet(pp + at, pr[k]);
     }
     uint4 raw[RPT + HALO];
     conv_load<D, RPT>(raw, stream ? a.k : a.q, stream ? a.cache_k : a.cache_q, b, t0 + rr0 * RPT, a.T, stream ? a.Hkv : a.H, stream ? j : h, a.K, o);
@@ -1242,7 +1239,7 @@ static Plan plan(const lawcat_params& p) {
   L.du_k = take(nf / (p.H / p.H_kv));
   L.inv = take(4 * bth); L.delta = take(4 * bth); L.domax = take(8 * (size_t)p.B * p.H);
   L.z16 = take(4 * ch * p.d_k); L.meta = take(8 * ch); L.s16 = take(ch * 4 * p.d_k * p.d_k); L.wmax = take(4 * (size_t)p.B * p.H);
-  L.total = off;
+  L.total = off + 256;  // (the base is rounded up: rows are read 32 bytes at a time)
   return L;
 }
 
@@ -1305,7 +1302,7 @@ int launch_layer_bwd_tc(const Ctx& c, const void* q, const void* k, const void* 
   int r = raise_limits();
   if (r) return r;
   const Plan L = plan(p);
-  char* w = (char*)ws;
+  char* w = (char*)align_up((size_t)ws, 256);
   Args a{};
   a.qd = (float*)(w + L.qd); a.kd = (float*)(w + L.kd); a.v = (const bf16*)v; a.gate = (const bf16*)gate; a.dO = (const bf16*)dO;
   a.S0 = S0; a.z0 = z0; a.wq = (float*)(w + L.wq); a.wk = (float*)(w + L.wk); a.dvh = (float*)(w + L.dvh); a.dgate = (bf16*)dgate;

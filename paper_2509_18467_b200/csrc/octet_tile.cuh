@@ -63,6 +63,14 @@ __device__ __forceinline__ void load_row8(const float* p, float* v) {
   v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
 }
 
+// eight consecutive floats at a 32-byte boundary by one load: as two, each would take half of every sector it touches
+__device__ __forceinline__ void load_octet(const float* p, float4 (&v)[2]) {
+  asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=f"(v[0].x), "=f"(v[0].y), "=f"(v[0].z), "=f"(v[0].w), "=f"(v[1].x), "=f"(v[1].y), "=f"(v[1].z), "=f"(v[1].w)
+               : "l"(p)
+               : "memory");
+}
+
 __device__ __forceinline__ float log2_sigmoid(float a) {
   const float x = -a * 1.4426950408889634f;
   return -fmaxf(x, lg2f(1.f + ex2f(fminf(x, 126.f))));
