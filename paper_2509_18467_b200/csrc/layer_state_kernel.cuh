@@ -377,8 +377,10 @@ layer_state_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
           f2_unpack(f2_add(f2_pack(x[i], x[i + 1]), off2), e0, e1);
           const uint64_t k2 = f2_mul(f2_mul(f2_pack(y[i], y[i + 1]), i & 2 ? iv.y : iv.x), f2_pack(ex2f(e0), ex2f(e1)));
           f2_unpack(k2, k0, k1);
-          kh[i / 2] = pack_f16(k0, k1);
-          zs = f2_add(zs, k2);
+          const __half2 h2 = __floats2half2_rn(k0, k1);
+          kh[i / 2] = *reinterpret_cast<const uint32_t*>(&h2);
+          const float2 kr = __half22float2(h2);  // (z as the layer kernel has it: the sum of the keys AS ROUNDED)
+          zs = f2_add(zs, f2_pack(kr.x, kr.y));
         }
       }
       float z0, z1;
