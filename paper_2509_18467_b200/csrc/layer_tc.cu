@@ -331,7 +331,6 @@ static int run_layer_tc(const Ctx& c, const void* q, const void* k, const void* 
   a.S0 = S0; a.z0 = z0; a.S_T = S_T; a.z_T = z_T;
   auto* const k_layer = paired ? layer_tc_kernel<2> : dh == 64 ? layer_tc_kernel<1> : layer_tc_kernel<0>;
   auto* const k_state = paired ? st::layer_state_kernel<2> : dh == 64 ? st::layer_state_kernel<1> : st::layer_state_kernel<0>;
-  const int threads = threads_of(paired ? 2 : dh == 64 ? 1 : 0);
   {
     // the kernels' shared-memory limit is raised once per device
     static std::mutex mu;
@@ -353,7 +352,7 @@ static int run_layer_tc(const Ctx& c, const void* q, const void* k, const void* 
   const int Hn = paired ? p.H / 2 : p.H;          // thread blocks per segment
   if (segs == nseq) {
     LaunchScope _ls("layer_tc", c.stream);
-    launch_behind(k_layer, dim3(Hn * segs), dim3(threads), SMEM_ALLOC, c.stream, tq, tk, tv, tg, a, tab);
+    launch_behind(k_layer, dim3(Hn * segs), dim3(LAYER_THREADS), SMEM_ALLOC, c.stream, tq, tk, tv, tg, a, tab);
     LAWCAT_CHECK_LAUNCH();
     return LAWCAT_OK;
   }
@@ -394,7 +393,7 @@ static int run_layer_tc(const Ctx& c, const void* q, const void* k, const void* 
     // (the scan gives no early start: with one, blocks land while scan blocks still hold registers of most SMs,
     // and the call at T = 32768 took 1.34 ms instead of 1.11)
     LaunchScope _ls("layer_tc", c.stream);
-    launch_behind(k_layer, dim3(Hn * segs), dim3(threads), SMEM_ALLOC, c.stream, tq, tk, tv, tg, a, tab);
+    launch_behind(k_layer, dim3(Hn * segs), dim3(LAYER_THREADS), SMEM_ALLOC, c.stream, tq, tk, tv, tg, a, tab);
   }
   LAWCAT_CHECK_LAUNCH();
   return LAWCAT_OK;

@@ -11,13 +11,9 @@
 //               gate: g = log2 sigmoid(a) / tau per entry, then a scan outwards from the middle token gives the
 //               exponents x_t = b_t - b_mid (b the running sum of g) in fp32 (the middle reference keeps every factor
 //               2^x within 2^(+-32 max|g|)); v: bf16 -> fp16 in place (exact)
-//   MMA warp    MMA 1: Y = [u_q; u_k] W_h  (fp16 operands, fp32 accumulate in TMEM). For 64-wide heads a warp of its own
-//               issues it: a thread issues a product every hundred cycles or so, about twice what the tensor pipe needs for
-//               one, and the products of the next chunk's mix stand in the middle of the chain score -> read-out -> state
-//               that the next chunk waits for (32 heads of 64, 8192 tokens: 187 -> 178 us, 65536 tokens: 1205 -> 1066 us).
-//               At width 128 the blocks of a long sequence then fall into periods of 9.7k or 11.5k cycles a chunk, both SMs
-//               of a pair alike and differently from launch to launch, where they otherwise all take 10.0k (32768 tokens:
-//               1080 -> 1180 us): there the MMA warp issues it
+//   mix warp    MMA 1: Y = [u_q; u_k] W_h  (fp16 operands, fp32 accumulate in TMEM), by a warp of its own: the products of the
+//               next chunk's mix would stand in the middle of the chain score -> read-out -> state that the next chunk waits for
+//               (32 heads of 64, 8192 tokens: 187 -> 178 us; 32 heads of 128, 32768 tokens: 703 -> 677)
 //   row warps   (two threads per token row, 64 columns each, straight from tensor memory)
 //               phi: row softmax. Query rows keep exp(y - max) unnormalized: a positive per-token factor cancels in
 //               Eq. 8. The decay factors ride in the exponent of the softmax: qs = 2^(y' + x_t), ks = phi_k 2^(-x_i),
@@ -74,10 +70,10 @@ constexpr int MID = 31;      // reference token of the in-chunk decay factorizat
 constexpr int HALO = 3;      // raw rows in front of a chunk that the conv needs (conv width up to 4)
 
 // warps: 0-7 prep, 8-15 row warps (TMEM quadrant = warp & 3, column half = (warp - 8) >> 2), 16 TMA, 17 MMA,
-// 18 mix (64-wide heads only)
+// 18 mix
 constexpr int PREP_THREADS = 256;
 constexpr int ROW_WARP0 = 8, TMA_WARP = 16, MMA_WARP = 17, MIX_WARP = 18;
-__host__ __device__ constexpr int threads_of(int width) { return (width != 0 ? 19 : 18) * 32; }
+constexpr int LAYER_THREADS = 19 * 32;
 
 // shared memory map (byte offsets from a 1024-byte aligned base)
 constexpr uint32_t OFF_W = 0;                     // W_h^T fp16, K-major, 2 slabs x [128 x 128 B]
@@ -320,7 +316,7 @@ __device__ __forceinline__ bool wait_set_or_abort(uint32_t bar0, uint32_t mask, 
 // WIDTH: 0 = heads of 128 channels; 1 = one head of 64 channels per block (padded to 128); 2 = two 64-wide heads of one
 // key/value group per block. A compile-time switch, so that the 128-wide kernel carries none of the others' tests.
 template <int WIDTH>
-__global__ void __launch_bounds__(threads_of(WIDTH), 1)
+__global__ void __launch_bounds__(LAYER_THREADS, 1)
 layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                 const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_g, const TcArgs a,
                 const __grid_constant__ PackTab tab) {
@@ -347,7 +343,6 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   // of 128 channels, the shared k is loaded into both halves, W is block-diagonal, and everything that contracts over the
   // channels (scores, read-out) is issued per half into accumulators of its own.
   constexpr bool narrow = WIDTH == 1, pair = WIDTH == 2, wide = WIDTH == 0;
-  constexpr bool mixw = WIDTH != 0;  // MMA 1 issued by a warp of its own
   constexpr int dh = narrow ? 64 : 128, nslab = dh >> 6;  // width of the q / gate / o tiles as addressed, and their slabs
   constexpr int hd = wide ? 128 : 64, vslab = hd >> 6;    // width of a real head: of k and v as stored, of the state's value side
   // tensor memory columns (the pair keeps two read-out and two score accumulators where the state needs half the columns)
@@ -650,23 +645,9 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         return (d & 0xFFFFFFFF00000000ull) | (uint64_t)((uint32_t)d + off16);
       };
       auto kstep = [](int k) -> uint32_t { return (uint32_t)((k >> 2) * (16384 >> 4) + (k & 3) * 2); };
-      // (a 64-wide head: 4 instead of 8 K steps over the channels, 64 instead of 128 output columns)
-      const int ksteps = narrow ? 4 : 8, NW = narrow ? 64 : 128;  // (the mix: channels contracted, output columns)
+      const int ksteps = narrow ? 4 : 8;  // (a 64-wide head: 4 instead of 8 K steps over the channels)
       constexpr int NV = hd;  // value columns of the state and of the read-out
-      [[maybe_unused]] auto issue_mma1 = [&]() {
-        const uint32_t ID = instr_desc(128, NW, FMT_F16, MAJOR_K, MAJOR_K);
-#pragma unroll
-        for (int k = 0; k < 8; ++k)
-          if (k < ksteps) mma_f16(tmem + COL_Y, adv(dsc_u, kstep(k)), adv(dsc_w, kstep(k)), ID, k > 0);
-        mma_commit(bar(B_MMA1));
-      };
-      bool ok = nchunks > 0;
-      if (!mixw && ok) ok = wait_set_or_abort(bar(0), BIT(B_U_FULL), 0u, lane, s_abort, a.wait_limit);
-      if (!mixw && ok && elect_one()) {
-        tc_fence_after_sync();
-        issue_mma1();
-      }
-      for (int n = 0; ok && n < nchunks; ++n) {
+      for (int n = 0; n < nchunks; ++n) {
         const uint32_t p = (uint32_t)(n & 1), pp = p ^ 1u;
         WAITSET(BIT(B_QK_FULL) | BIT(B_SBF_FULL) | BIT(B_VH_FULL) | (n > 0 ? BIT(B_O_FREE) : 0u),
                 PAR(B_QK_FULL, p) | PAR(B_SBF_FULL, p) | PAR(B_VH_FULL, p) | PAR(B_O_FREE, pp));
@@ -686,14 +667,6 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
           mma_commit(bar(B_P));
         }
         TL(0, 1, n, lane == 0);
-        if (!mixw && n + 1 < nchunks) {
-          // then the mix of the next chunk: its phi sweeps read Y while this chunk's read-out and state update execute
-          WAITSET(BIT(B_U_FULL) | BIT(B_Y_FREE), PAR(B_U_FULL, pp) | PAR(B_Y_FREE, p));
-          if (elect_one()) {
-            tc_fence_after_sync();
-            issue_mma1();
-          }
-        }
         TL(0, 2, n, lane == 0);
         if (elect_one()) {
           tc_fence_after_sync();
@@ -735,7 +708,7 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         TL(0, 5, n, lane == 0);
       }
     }
-  } else if (mixw && warp == MIX_WARP) {
+  } else if (warp == MIX_WARP) {
     // ================================================================================================ mix issuer
     const uint64_t dsc_u = smem_desc(sb + OFF_AU, 16, 1024, LAYOUT_SW128);
     const uint64_t dsc_w = smem_desc(sb + OFF_W, 16, 1024, LAYOUT_SW128);
