@@ -510,14 +510,14 @@ static int conv_bwd_stream(const Ctx& c, const TD* du, const TI* x, const TI* w,
 // The same for bf16 storage, conv width up to 4 and fp32 du (whole-layer and mix backward), both streams in one launch, four
 // channels per thread: 16-byte loads of du and 8-byte loads of x, a group of 8 tokens in flight. Bound by HBM: du and x in, dx
 // out. One channel per thread, a launch per stream: 129 us at 8 x 1024 tokens, 32/8 heads of 64 (166 MB); this form 50 us.
-constexpr int CB4_SPAN = 32;
+// A warp walks `span` tokens (a multiple of 8).
 struct ConvBwd4 {
   const float* du[2];
   const bf16 *x[2], *w[2], *cache[2];
   bf16* dx[2];
   float* dw[2];
   int C[2];      // channels per stream
-  int B, T, K;
+  int B, T, K, span;
 };
 __device__ __forceinline__ void bf16x4(const uint2& r, float* f) {
   f[0] = __uint_as_float(r.x << 16); f[1] = __uint_as_float(r.x & 0xffff0000u);
@@ -530,7 +530,7 @@ __global__ void __launch_bounds__(128) conv_bwd4_kernel(const ConvBwd4 a) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, qb = (a.C[0] / 4 + 31) / 32;
   const int st = (int)blockIdx.y >= qb;
   const int C = st ? a.C[1] : a.C[0], ch = 4 * (((int)blockIdx.y - (st ? qb : 0)) * 32 + lane), K = a.K, T = a.T;
-  const int spans = (T + CB4_SPAN - 1) / CB4_SPAN, sg = (int)blockIdx.x * 4 + warp;
+  const int spans = (T + a.span - 1) / a.span, sg = (int)blockIdx.x * 4 + warp;
   const bool on = ch < C && sg < a.B * spans;
   const float* du = st ? a.du[1] : a.du[0];
   const bf16* x = st ? a.x[1] : a.x[0];
@@ -538,7 +538,7 @@ __global__ void __launch_bounds__(128) conv_bwd4_kernel(const ConvBwd4 a) {
   const bf16* cache = st ? a.cache[1] : a.cache[0];
   bf16* dx = st ? a.dx[1] : a.dx[0];
   float* dw = st ? a.dw[1] : a.dw[0];
-  const int b = on ? sg / spans : 0, t0 = on ? sg % spans * CB4_SPAN : 0, t1 = on ? min(T, t0 + CB4_SPAN) : 0;
+  const int b = on ? sg / spans : 0, t0 = on ? sg % spans * a.span : 0, t1 = on ? min(T, t0 + a.span) : 0;
   const float* dub = du + (size_t)b * T * C + ch;
   const bf16* xb = x + (size_t)b * T * C + ch;
   float tap[4][4], acc[4][4], xw[3][4], dwin[3][4];  // [delta][channel]; x[t - 1 - i], du[t + i]
@@ -632,9 +632,20 @@ static int conv_bwd_both(const Ctx& c, const float* du_q, const float* du_k, con
   const int Cq = p.H * p.d_k, Ck = p.H_kv * p.d_k;
   if (!zeroed && dw_q && cudaMemsetAsync(dw_q, 0, sizeof(float) * (size_t)Cq * p.conv_k, c.stream) != cudaSuccess) return LAWCAT_ERR_CUDA;
   if (!zeroed && dw_k && cudaMemsetAsync(dw_k, 0, sizeof(float) * (size_t)Ck * p.conv_k, c.stream) != cudaSuccess) return LAWCAT_ERR_CUDA;
+  // The span is the one with the least work on an SM: two blocks are resident (191 registers; held to 128, four are and take longer,
+  // 51 -> 62 us), a span's first loads are worth about four tokens. 8 x 1024 tokens, 32/8 heads of 64: 60 us at 16 tokens, 51 at 32,
+  // 45.5 at 48, 52 at 64; 4 x 1300 of 128: 71, 62, 58, 56.
+  const int cols = (Cq / 4 + 31) / 32 + (Ck / 4 + 31) / 32;
+  int span = 16;
+  long long best = 0;
+  for (int s = 16; s <= 64; s += 8) {
+    const long long blocks = (((long long)p.B * ((p.T + s - 1) / s) + 3) / 4) * cols, slots = 2LL * sm_count();
+    const long long cost = (blocks + slots - 1) / slots * (s + 4);
+    if (best == 0 || cost < best) { best = cost; span = s; }
+  }
   const ConvBwd4 a{{du_q, du_k}, {(const bf16*)q, (const bf16*)k}, {(const bf16*)w_q, (const bf16*)w_k},
-                   {(const bf16*)cache_q, (const bf16*)cache_k}, {(bf16*)dq, (bf16*)dk}, {dw_q, dw_k}, {Cq, Ck}, p.B, p.T, p.conv_k};
-  const dim3 grid((p.B * ((p.T + CB4_SPAN - 1) / CB4_SPAN) + 3) / 4, (Cq / 4 + 31) / 32 + (Ck / 4 + 31) / 32);
+                   {(const bf16*)cache_q, (const bf16*)cache_k}, {(bf16*)dq, (bf16*)dk}, {dw_q, dw_k}, {Cq, Ck}, p.B, p.T, p.conv_k, span};
+  const dim3 grid((p.B * ((p.T + span - 1) / span) + 3) / 4, cols);
   LaunchScope _ls("conv_bwd4", c.stream);
   launch_behind(conv_bwd4_kernel, grid, dim3(128), 0, c.stream, a);
   LAWCAT_CHECK_LAUNCH();
