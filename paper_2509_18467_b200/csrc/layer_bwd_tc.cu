@@ -59,6 +59,7 @@ struct Args {
   uint8_t* s16;                         // [B*H][chunks][2 * D * D * 2] operand tiles, hi then lo
   float* wmax;                          // [B*H] largest |wq|, |wk| of the head
   float* dW;                            // [H,D,D] weight gradient, accumulated by the mix backward: zeroed by the sweep
+  float* du_k;                          // [B,T,Hkv,D], zeroed as well where several blocks of the mix backward add to it (else null)
   int* dev_status;
   int B, T, H, Hkv, gate_dim, gate_mode, normalize;
   float inv_tau, eps;
@@ -268,6 +269,11 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) sweep_kerne
   // dW is zeroed here (every block a part) and not by a memset node of its own, which costs microseconds
   for (int i = blockIdx.x * F::THREADS + tid; i < a.H * D * D / 4; i += gridDim.x * F::THREADS)
     reinterpret_cast<float4*>(a.dW)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (a.du_k) {
+    const size_t n4 = (size_t)a.B * a.T * a.Hkv * (D / 4);
+    for (size_t i = (size_t)blockIdx.x * F::THREADS + tid; i < n4; i += (size_t)gridDim.x * F::THREADS)
+      reinterpret_cast<float4*>(a.du_k)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
   // the two extra slabs of [v | 1] (column D: the 1) and of the state operand (column D: z; the rest zero)
   for (int i = tid; i < 2 * C; i += F::THREADS)
     *reinterpret_cast<uint4*>(sg + F::F_V + toff(F::SL_T, i & (C - 1), D + 8 * (i >> 6))) = make_uint4(0u, 0u, 0u, 0u);
@@ -935,6 +941,7 @@ struct MArgs {
   const float* wmax;
   int* dev_status;
   int B, T, H, Hkv, K;
+  int parts;                 // blocks that share a group's heads; more than one: du_k is added to (zeroed by the sweep)
 };
 
 template <int D>
@@ -955,7 +962,7 @@ __global__ void __launch_bounds__(MCfg<D>::THREADS, D == 128 ? 1 : 2) mix_bwd_ke
   const uint32_t sb = smem_u32(sg);
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   volatile int* const s_fl = reinterpret_cast<volatile int*>(sg + M::BAR + 16);  // tmem base, abort
-  const int t0 = blockIdx.x * TT, bj = blockIdx.z * gridDim.y + blockIdx.y, j = bj % a.Hkv, b = bj / a.Hkv, G = a.H / a.Hkv;
+  const int part = blockIdx.x % a.parts, t0 = blockIdx.x / a.parts * TT, bj = blockIdx.z * gridDim.y + blockIdx.y, j = bj % a.Hkv, b = bj / a.Hkv, G = a.H / a.Hkv;
   if (b >= a.B) return;
   const int nvalid = min(TT, a.T - t0);
   if (tid == 0) {
@@ -1012,14 +1019,15 @@ __global__ void __launch_bounds__(MCfg<D>::THREADS, D == 128 ? 1 : 2) mix_bwd_ke
   // du. Width 64: the bulk-copy engine takes the rows on from the staging tile, behind the block's other work (8 x 1024 tokens: the
   // kernel 131 us; 138 by the threads). Width 128, where a tile is two trips through staging that would wait for one another: by the
   // threads (4 x 1300 tokens: 238 us; 244).
-  auto du_out = [&](uint32_t col, float* dst, int NH, int head, float isc) {
+  auto du_out = [&](uint32_t col, float* dst, int NH, int head, float isc, bool add) {
     if constexpr (D == 64) {
       stage(col, 0, isc);
       fence_proxy_async();
       __syncthreads();
       if (tid < nvalid) {
         float* const p = dst + (((size_t)b * a.T + t0 + tid) * NH + head) * D;
-        asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], 256;" ::"l"(p), "r"(sb + M::ST + tid * M::ST_ROW) : "memory");
+        if (add) asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], 256;" ::"l"(p), "r"(sb + M::ST + tid * M::ST_ROW) : "memory");
+        else asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], 256;" ::"l"(p), "r"(sb + M::ST + tid * M::ST_ROW) : "memory");
         tma_store_commit();
       }
     } else {
@@ -1030,8 +1038,10 @@ __global__ void __launch_bounds__(MCfg<D>::THREADS, D == 128 ? 1 : 2) mix_bwd_ke
 #pragma unroll 4
         for (int idx = tid; idx < nvalid * 16; idx += NTH) {
           const int pc = idx % 16, r = idx / 16;
-          *reinterpret_cast<float4*>(dst + (((size_t)b * a.T + t0 + r) * NH + head) * D + h64 + pc * 4) =
-              *reinterpret_cast<const float4*>(sg + M::ST + r * M::ST_ROW + pc * 16);
+          float* const p = dst + (((size_t)b * a.T + t0 + r) * NH + head) * D + h64 + pc * 4;
+          const float4 v = *reinterpret_cast<const float4*>(sg + M::ST + r * M::ST_ROW + pc * 16);
+          if (add) asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+          else *reinterpret_cast<float4*>(p) = v;
         }
         __syncthreads();
       }
@@ -1065,8 +1075,10 @@ __global__ void __launch_bounds__(MCfg<D>::THREADS, D == 128 ? 1 : 2) mix_bwd_ke
       }
     }
   };
+  // this block's steps: those of heads [G part / parts, G (part + 1) / parts) of the group
+  const int s_begin = 2 * (G * part / a.parts), s_end = 2 * (G * (part + 1) / a.parts);
   auto taps = [&](int s) {  // of step s into its slot
-    if (s < 2 * G) load_taps<D>(sg + M::TAPS + (s & 1) * D * 16, s & 1 ? a.w_k : a.w_q, s & 1 ? j : j * G + (s >> 1), a.K, tid, NTH);
+    if (s < s_end) load_taps<D>(sg + M::TAPS + (s & 1) * D * 16, s & 1 ? a.w_k : a.w_q, s & 1 ? j : j * G + (s >> 1), a.K, tid, NTH);
   };
   uint4 dyh[RPT], dyl[RPT], uh[RPT], ul[RPT];  // a step's operands: this thread's octets of dy and u, hi and lo
   auto operands = [&](int s) {
@@ -1085,7 +1097,7 @@ __global__ void __launch_bounds__(MCfg<D>::THREADS, D == 128 ? 1 : 2) mix_bwd_ke
     uint4 raw[RPT + HALO];
     conv_load<D, RPT>(raw, stream ? a.k : a.q, stream ? a.cache_k : a.cache_q, b, t0 + rr0 * RPT, a.T, stream ? a.Hkv : a.H, stream ? j : h, a.K, o);
     // the rows of the step behind travel towards L2 meanwhile
-    if (s + 1 < 2 * G) {
+    if (s + 1 < s_end) {
       const int nh = h + stream;
       const float* wn = stream ? a.wq : a.wk;
       const float* pn = stream ? a.qd : a.kd;
@@ -1120,21 +1132,21 @@ __global__ void __launch_bounds__(MCfg<D>::THREADS, D == 128 ? 1 : 2) mix_bwd_ke
       split8h(u, true, uh[i], ul[i]);
     });
   };
-  taps(0);
-  load_w_tile<D>(sg + M::WT, a.W + (size_t)j * G * D * D, tid, NTH);
+  taps(s_begin);
+  load_w_tile<D>(sg + M::WT, a.W + ((size_t)j * G + (s_begin >> 1)) * D * D, tid, NTH);
   __syncthreads();
-  operands(0);
-  int sg_at = scale_of(0);  // power of two on the key stream's du so far
+  operands(s_begin);
+  int sg_at = scale_of(s_begin >> 1);  // power of two on the key stream's du so far
 #pragma unroll 1
-  for (int s = 0; s < 2 * G; ++s) {
+  for (int s = s_begin; s < s_end; ++s) {
     const int g = s >> 1, stream = s & 1, h = j * G + g;
     uint4 wreg[WPT];
-    const bool next_w = stream == 0 && s > 0;
+    const bool next_w = stream == 0 && s > s_begin;
     if (next_w) {
 #pragma unroll
       for (int k = 0; k < WPT; ++k) wreg[k] = *reinterpret_cast<const uint4*>(a.W + (size_t)h * D * D + (size_t)(tid + k * NTH) * 8);
     }
-    if (s > 0) wt.wait();  // the products of the step in front: its operands and W_h have been read
+    if (s > s_begin) wt.wait();  // the products of the step in front: its operands and W_h have been read
     if (next_w) {
 #pragma unroll
       for (int k = 0; k < WPT; ++k) {
@@ -1154,7 +1166,7 @@ __global__ void __launch_bounds__(MCfg<D>::THREADS, D == 128 ? 1 : 2) mix_bwd_ke
     }
     const int sgm = scale_of(g);
     if (stream == 0 && sgm != sg_at) {  // the key stream's du so far, on this head's scale (the choice of powers is uniform)
-      if (g > 0) {
+      if (s > s_begin) {
         const float f = pow2i(sgm - sg_at);
         float d[8];
 #pragma unroll 1
@@ -1178,14 +1190,14 @@ __global__ void __launch_bounds__(MCfg<D>::THREADS, D == 128 ? 1 : 2) mix_bwd_ke
     if (warp == 0 && elect_one()) {
       mm.split(stream ? M::DUK : M::DUQ, kview(sb + M::DY, L::SLAB_U), kview(sb + M::DY + L::TILE_U, L::SLAB_U), 2 * L::SLAB_U,
                kview(sb + M::WT, L::SLAB_W), 0, 2 * L::SLAB_W, D / 16, instr_desc(128, D, FMT_F16, MAJOR_K, MAJOR_K),
-               stream == 1 && g > 0);
+               stream == 1 && s > s_begin + 1);
       mm.split(M::DWC + (g & 1) * D, mview(sb + M::U, L::SLAB_U), mview(sb + M::U + L::TILE_U, L::SLAB_U), 256, mview(sb + M::DY, L::SLAB_U),
                mview(sb + M::DY + L::TILE_U, L::SLAB_U), 256, TT / 16, instr_desc(128, D, FMT_F16, MAJOR_MN, MAJOR_MN), stream == 1);
       mma_commit(sb + M::BAR);
     }
-    if (stream) du_out(M::DUQ, a.wq, a.H, h, pow2i(-sgm));
-    else if (g > 0) dw_out(g - 1);
-    if (s + 1 < 2 * G) operands(s + 1);
+    if (stream) du_out(M::DUQ, a.wq, a.H, h, pow2i(-sgm), false);
+    else if (s > s_begin) dw_out(g - 1);
+    if (s + 1 < s_end) operands(s + 1);
   }
   wt.wait();
   auto staging_free = [&]() {
@@ -1195,9 +1207,9 @@ __global__ void __launch_bounds__(MCfg<D>::THREADS, D == 128 ? 1 : 2) mix_bwd_ke
     }
   };
   staging_free();
-  dw_out(G - 1);
+  dw_out((s_end >> 1) - 1);
   staging_free();
-  du_out(M::DUK, a.du_k, a.Hkv, j, pow2i(-sg_at));
+  du_out(M::DUK, a.du_k, a.Hkv, j, pow2i(-sg_at), a.parts > 1);
   if (D == 64 && tid < TT) tma_store_wait_all();
   tc_fence_before_sync();
   __syncthreads();
@@ -1243,6 +1255,21 @@ static Plan plan(const lawcat_params& p) {
   return L;
 }
 
+// How many blocks of the mix backward share the heads of a group: two where that fills the last round of blocks better (one per SM at
+// width 128, two at 64; a block's first operands and last gradients, which nothing hides, are worth about half a head). 4 x 1300 tokens,
+// 32/8 heads of 128 (352 blocks, 2.4 rounds): 236 us as one, 219 as two; 8 x 1024 of 64 (512 blocks, 1.7 rounds) stays one.
+static int mix_parts(const lawcat_params& p) {
+  const int G = p.H / p.H_kv, slots = sm_count() * (p.d_k == 128 ? 1 : 2);
+  const long long blocks = (long long)p.B * p.H_kv * ((p.T + TT - 1) / TT);
+  int best = 1;
+  long long cost = 0;
+  for (int n = 1; n <= 2 && n <= G; ++n) {
+    const long long c = (blocks * n + slots - 1) / slots * (2 * ((G + n - 1) / n) + 1);
+    if (n == 1 || c < cost) { cost = c; best = n; }
+  }
+  return best;
+}
+
 static int raise_limits() {
   static std::mutex mu;
   static bool done[64] = {};
@@ -1275,7 +1302,7 @@ static int run(const Ctx& c, const Args& a, const Maps& maps, const MArgs& m) {
   // (tiles along x, with neighbours on the same head: 3 tiles of 8 heads of 128, head by head 92.7 us instead of 90.6; the y axis
   // ends at 65535, so the heads go on along z)
   const unsigned heads = (unsigned)(p.B * p.H_kv), ny = heads < 32768u ? heads : 32768u;
-  launch_behind(mix_bwd_kernel<D>, dim3((unsigned)((p.T + TT - 1) / TT), ny, (heads + ny - 1) / ny), dim3(MCfg<D>::THREADS), MCfg<D>::BYTES,
+  launch_behind(mix_bwd_kernel<D>, dim3((unsigned)((p.T + TT - 1) / TT * m.parts), ny, (heads + ny - 1) / ny), dim3(MCfg<D>::THREADS), MCfg<D>::BYTES,
                 c.stream, m);
   LAWCAT_CHECK_LAUNCH();
   return LAWCAT_OK;
@@ -1311,7 +1338,9 @@ int launch_layer_bwd_tc(const Ctx& c, const void* q, const void* k, const void* 
   a.B = p.B; a.T = p.T; a.H = p.H; a.Hkv = p.H_kv; a.gate_dim = p.gate_dim; a.gate_mode = p.gate_mode; a.normalize = p.normalize;
   a.inv_tau = 1.f / p.gate_tau; a.eps = p.eps;
   MArgs m{(const bf16*)q, (const bf16*)k, (const bf16*)w_q, (const bf16*)w_k, (const bf16*)W, (const bf16*)cache_q,
-          (const bf16*)cache_k, a.qd, a.kd, a.wk, a.wq, (float*)(w + L.du_k), dW, a.wmax, c.dev_status, p.B, p.T, p.H, p.H_kv, p.conv_k};
+          (const bf16*)cache_k, a.qd, a.kd, a.wk, a.wq, (float*)(w + L.du_k), dW, a.wmax, c.dev_status, p.B, p.T, p.H, p.H_kv, p.conv_k,
+          mix_parts(p)};
+  a.du_k = m.parts > 1 ? m.du_k : nullptr;
   if ((r = launch_convmix_tc_fwd(c, q, k, w_q, w_k, W, cache_q, cache_k, (void*)a.qd, (void*)a.kd, true))) return r;
   Maps maps;
   const int D = p.d_k;
