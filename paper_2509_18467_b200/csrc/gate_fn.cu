@@ -114,7 +114,7 @@ gate_fn_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
   using L = Lay<R>;
   extern __shared__ __align__(1024) uint8_t smem[];
   const uint32_t sb = smem_u32(smem);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;  // (warp: uniform to the compiler)
   const uint32_t bars = sb + L::OFF_BAR;
   volatile int* const s_flags = reinterpret_cast<volatile int*>(smem + L::OFF_BAR + 8 * NUM_BARS);  // [0] tmem base, [1] abort
   volatile int* const s_abort = s_flags + 1;
@@ -161,7 +161,9 @@ gate_fn_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------------------------------------ products
-    if (lane == 0) {
+    // (an elected lane: its descriptors stay in uniform registers. 32768 tokens, rank 32, 4096 wide: 106.5 -> 100.2 us, 3000 tokens,
+    // rank 64: 28.3 -> 24.2)
+    if (elect_one()) {
       constexpr uint32_t idesc1 = instr_desc(128, R, FMT_BF16, MAJOR_K, MAJOR_K);
       constexpr uint32_t idesc2 = instr_desc(128, NT, FMT_BF16, MAJOR_K, MAJOR_K);
       bool ok = true;
