@@ -76,7 +76,7 @@ layer_state_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
   volatile int* const s_flags = reinterpret_cast<volatile int*>(sg + OFF_BAR + 8 * NUM_BARS);  // [0] tmem base, [1] abort
   volatile int* const s_abort = s_flags + 1;
   auto bar = [&](int i) -> uint32_t { return sb + OFF_BAR + 8 * i; };
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;  // (warp: uniform to the compiler)
   constexpr bool narrow = WIDTH == 1, pair = WIDTH == 2, wide = WIDTH == 0;
   constexpr int hd = wide ? 128 : 64, slabs = hd >> 6;  // width of a head; slabs of k and v
   constexpr int gslabs = narrow ? 1 : 2;                // slabs of the gate tile (pair: 128 channels of two heads)
@@ -215,8 +215,8 @@ layer_state_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
     for (int k = 0; k < hd / 16; ++k)
       mma_f16(tmem + COL_Y, adv(dsc_w, (uint32_t)((k >> 2) * 1024 + (k & 3) * 2)), adv(dsc_u, (uint32_t)((k >> 2) * 512 + (k & 3) * 2)), ID, k > 0);
     mma_commit(bar(B_MIX));
-    is_mix = n;
   };
+  auto go = [&]() -> bool { return __shfl_sync(0xffffffffu, (int)!*s_abort, 0) != 0; };  // (whole warp)
   auto publish = [&]() {
     fence_proxy_async();
     tc_fence_before_sync();
@@ -232,9 +232,13 @@ layer_state_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
   if (nchunks > 0) {
     conv(0);
     publish();
-    if (tid == 0 && !*s_abort) {
-      issue_mix(0);
-      if (1 < nchunks) { load_raw(1); is_raw = 1; }
+    if (warp == 0 && go()) {
+      if (elect_one()) {
+        issue_mix(0);
+        if (1 < nchunks) load_raw(1);
+      }
+      is_mix = 0;
+      if (1 < nchunks) is_raw = 1;
     }
   }
 #pragma unroll 1
@@ -400,15 +404,19 @@ layer_state_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
       sts128(ad, pack8(f, true));
     }
     publish();
-    if (tid == 0 && !*s_abort) {
-      constexpr uint32_t ID = instr_desc(128, hd, FMT_F16, MAJOR_K, MAJOR_MN);
+    if (warp == 0 && go()) {
+      if (elect_one()) {
+        constexpr uint32_t ID = instr_desc(128, hd, FMT_F16, MAJOR_K, MAJOR_MN);
 #pragma unroll
-      for (int k = 0; k < C / 16; ++k)
-        mma_f16_ta(tmem + COL_S, tmem + COL_KH + 8 * k, adv(dsc_v, (uint32_t)k * (2048 >> 4)), ID, n > 0 || k > 0);
-      mma_commit(bar(B_UPD));
+        for (int k = 0; k < C / 16; ++k)
+          mma_f16_ta(tmem + COL_S, tmem + COL_KH + 8 * k, adv(dsc_v, (uint32_t)k * (2048 >> 4)), ID, n > 0 || k > 0);
+        mma_commit(bar(B_UPD));
+        if (n + 1 < nchunks) issue_mix(n + 1);
+        if (n + 2 < nchunks) load_raw(n + 2);
+      }
       is_upd = n;
-      if (n + 1 < nchunks) issue_mix(n + 1);
-      if (n + 2 < nchunks) { load_raw(n + 2); is_raw = n + 2; }
+      if (n + 1 < nchunks) is_mix = n + 1;
+      if (n + 2 < nchunks) is_raw = n + 2;
     }
   }
   // ---- end state, as whole rows through the dead tiles
