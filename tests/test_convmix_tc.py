@@ -4,7 +4,7 @@ tile boundaries (128 tokens), ragged tails, conv caches, conv widths 1-4, groupe
 import numpy as np
 import pytest
 
-from helpers import check
+from helpers import check, oracle_params
 from oracle import lawcat_oracle as O
 from paper_2509_18467_b200 import inputs as I
 
@@ -44,6 +44,35 @@ def test_forward_lengths_around_the_tile(api, d, T, with_cache):
     rq, rk = features(s, x)
     check(qd, rq, "bf16", "qdot")
     check(kd, rk, "bf16", "kdot")
+
+
+@pytest.mark.parametrize("d,T", [(64, 127), (64, 300), (128, 129), (128, 300)])
+def test_forward_mix_outputs_too_large_to_exponentiate_as_they_are(api, d, T):
+    """Some rows' mix outputs y exceed what is exponentiated without the row's maximum. bf16 features: the conv output goes in as
+    fp16, off by up to 2^-11 of itself, so y is off by at most e = 2^-11 max_j sum_c |u_c W_cj| and a softmax by exp(2 e), then
+    rounded to bf16 (2^-8). fp32 features (in front of a plain sigmoid gate) hold the conv output exactly."""
+    s = I.LayerShape(1, T, 4, 2, d, d, dtype="bf16", gate_tau=1.0, config_id=74)
+    x = I.make(s, ["q", "k", "v", "gate", "w_q", "w_k", "W"])
+    for n in ("q", "k"):
+        x[n] = I.round_to_bf16(x[n] * np.where(np.arange(T) % 5 == 0, 30.0, 1.0)[None, :, None, None].astype(np.float32))
+    dv = {n: api.to_device(v, "bf16") for n, v in x.items()}
+    got = api.lawcat_conv_fwd(P(api, s), dv["q"], dv["k"], dv["w_q"], dv["w_k"], dv["W"])
+    for g, r, n, w in zip(got, features(s, x), ("q", "k"), ("w_q", "w_k")):
+        u = np.asarray(O.conv(x[n], x[w], None, s.conv_k)).reshape(1, T, -1, d)
+        u = np.repeat(u, s.H // u.shape[2], axis=2)
+        W = x["W"].astype(np.float64)
+        assert np.abs(np.einsum("bthc,hcj->bthj", u, W)).max() > 48
+        e = 2.0 ** -11 * np.einsum("bthc,hcj->bthj", np.abs(u), np.abs(W)).max(-1, keepdims=True)
+        r = np.asarray(r).reshape(1, T, s.H, d)
+        bound = r * (np.expm1(2 * e) + 2.0 ** -8 + 1e-4) + 1e-30
+        assert (np.abs(g.float().cpu().numpy().reshape(r.shape) - r) <= bound).all()
+    api.trace_begin()
+    out = api.lawcat_layer_fwd(P(api, s), *[dv[n] for n in ("q", "k", "v", "gate", "w_q", "w_k", "W")])
+    assert "convmix_tc_fwd" in api.trace_end()
+    ref = O.layer_fwd(oracle_params(s), *[x[n] for n in ("q", "k", "v", "gate", "w_q", "w_k", "W")], None, None, None, None)
+    check(out["o"], ref["o"], "bf16", "o")
+    for n in ("S_T", "z_T"):
+        check(out[n], ref[n], "bf16", n, f32_store=True)
 
 
 @pytest.mark.parametrize("H,Hkv,conv_k", [(2, 2, 4), (4, 1, 3), (8, 2, 2), (3, 3, 1)])
