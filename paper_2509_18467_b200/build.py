@@ -53,7 +53,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     for s in sources():
         src, obj = os.path.join(CSRC, s), os.path.join(OBJ, s[:-3] + ".o")
         if force or not os.path.exists(obj) or os.path.getmtime(obj) < max(os.path.getmtime(src), hdr):
-            cmd = [NVCC, *FLAGS, "-c", src, "-o", obj] + (["-Xptxas", "-v"] if verbose else [])
+            cmd = [NVCC, *FLAGS, "-Xptxas", "-v", "-c", src, "-o", obj]
             jobs.append(cmd)
 
     def run(cmd):
@@ -62,6 +62,9 @@ def build(force: bool = False, verbose: bool = False) -> str:
             sys.stderr.write(" ".join(cmd) + "\n" + r.stdout + r.stderr)
         if r.returncode:
             raise RuntimeError("compiler failed: " + " ".join(cmd))
+        if "-c" in cmd:  # registers, spills and shared memory of every kernel, beside the object
+            with open(cmd[-1][:-2] + ".ptxas", "w") as f:
+                f.write(r.stderr)
 
     with ThreadPoolExecutor(max_workers=8) as ex:
         list(ex.map(run, jobs + ([_binding_cmd()] if build_binding else [])))

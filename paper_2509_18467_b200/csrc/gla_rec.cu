@@ -122,7 +122,13 @@ __device__ __forceinline__ void copy_rows(uint32_t dst, const void* src, size_t 
   }
 }
 
-template <typename TQ, typename TS, int DK, int MODE>
+// Tokens of a batch that are written out without a loop. LONG (see fwd_long): all sixteen, or eight where sixteen spill (fp32 storage
+// at width 128: 680 bytes of spill stores instead of 40; 4096 tokens, 32 heads: 480 us, eight 476, two 504). Otherwise two, or four
+// (fp32 storage up to width 64).
+template <typename TQ, typename TS, int DK, bool LONG>
+__host__ __device__ constexpr int turn() { return LONG ? (sizeof(TS) == 4 && DK == 128 ? 8 : TBF) : sizeof(TS) == 4 && DK <= 64 ? 4 : 2; }
+
+template <typename TQ, typename TS, int DK, int MODE, bool LONG>
 __global__ void __launch_bounds__(256, 2) gla_fwd_rec_kernel(const GlaArgs a, const SegArgs sgm) {
   using namespace tc;
   extern __shared__ __align__(16) float smem[];
@@ -324,9 +330,7 @@ __global__ void __launch_bounds__(256, 2) gla_fwd_rec_kernel(const GlaArgs a, co
     if (active) {
       auto run = [&](auto plain_c) {
         constexpr bool PLAIN = decltype(plain_c)::value;
-        // (4096 tokens, 32 heads of 128, tau = 1: two tokens a turn 342 + 150 us, eight 325 + 150, all sixteen 326 + 143; with bf16
-        // features sixteen would spill)
-        constexpr int TURN = sizeof(TQ) == 4 ? TBF : 2;
+        constexpr int TURN = turn<TQ, TS, DK, LONG>();
 #pragma unroll TURN
         for (int tok = 0; tok < TBF; ++tok) {
           const float4 vv = *reinterpret_cast<const float4*>(s_v + tok * dv + c0);
@@ -446,6 +450,30 @@ size_t gla_fwd_rec_workspace_bytes(const lawcat_params& p) {
   return sizeof(float) * (size_t)p.B * p.H * (s.nseg - 1) * ((size_t)p.d_k * p.d_v + 2 * p.d_k);
 }
 
+// Whether a call takes the kernels whose batches are written out. Their loop is five times as long, and a call first has to fetch it:
+// that takes up to 1.2 us, and a batch gains 0.2 to 0.4 us (4096 tokens, 32 heads of 128, bf16 storage, tau = 1: 342 + 150 -> 326 + 143
+// us). From about one batch per SM on it pays at width 128 (48 tokens, 32 heads: 37.7 us against 39.1; 64 tokens: 43.0 against 43.0;
+// 256 tokens: 110.8 against 109.3); at the smaller widths, whose batches are shorter, only where the sequence is cut into at least four
+// segments or a segment has at least four batches (width 64, 32 heads: 100 tokens, three segments of three, 30.3 us against 30.9; 128
+// tokens, four of two, 27.7 against 27.3).
+static bool fwd_long(const lawcat_params& p, const SegArgs& s) {
+  const long long batches = (long long)p.B * p.H * ((p.T + TBF - 1) / TBF);
+  return batches >= 128 && (p.d_k == 128 || s.nseg >= 4 || s.seg_len >= 4 * TBF);
+}
+
+template <typename TQ, typename TS, int DK>
+static void fwd_kernels(bool long_form, void (*&k_state)(GlaArgs, SegArgs), void (*&k_full)(GlaArgs, SegArgs)) {
+  if constexpr (sizeof(TQ) == 4) {  // (bf16 features: sixteen tokens spill)
+    if (long_form) {
+      k_state = gla_fwd_rec_kernel<TQ, TS, DK, 1, true>;
+      k_full = gla_fwd_rec_kernel<TQ, TS, DK, 0, true>;
+      return;
+    }
+  }
+  k_state = gla_fwd_rec_kernel<TQ, TS, DK, 1, false>;
+  k_full = gla_fwd_rec_kernel<TQ, TS, DK, 0, false>;
+}
+
 template <typename TQ, typename TS>
 static int gla_fwd_launch(const Ctx& c, GlaArgs& a, void* ws, size_t ws_bytes, const CacheOut* caches) {
   const lawcat_params& p = *c.p;
@@ -465,11 +493,13 @@ static int gla_fwd_launch(const Ctx& c, GlaArgs& a, void* ws, size_t ws_bytes, c
   const size_t raw = (size_t)TBF * (p.d_k * sizeof(TQ) + (p.d_k + p.d_v) * sizeof(TS));
   const size_t smem1 = raw + sizeof(float) * ((size_t)TBF * (2 * p.d_k + p.d_v) + 2 * (p.d_k == 128 ? 256 : 128) + p.d_k);
   const size_t smem0 = smem1 + (size_t)TBF * p.d_k * sizeof(TQ) + sizeof(float) * ((size_t)TBF * (p.d_k + p.d_v) + 5 * TBF);
-  auto* k_state = gla_fwd_rec_kernel<TQ, TS, 128, 1>;
-  auto* k_full = gla_fwd_rec_kernel<TQ, TS, 128, 0>;
-  if (p.d_k == 64) { k_state = gla_fwd_rec_kernel<TQ, TS, 64, 1>; k_full = gla_fwd_rec_kernel<TQ, TS, 64, 0>; }
-  if (p.d_k == 32) { k_state = gla_fwd_rec_kernel<TQ, TS, 32, 1>; k_full = gla_fwd_rec_kernel<TQ, TS, 32, 0>; }
-  if (p.d_k == 16) { k_state = gla_fwd_rec_kernel<TQ, TS, 16, 1>; k_full = gla_fwd_rec_kernel<TQ, TS, 16, 0>; }
+  const bool long_form = fwd_long(p, s);
+  void (*k_state)(GlaArgs, SegArgs) = nullptr;
+  void (*k_full)(GlaArgs, SegArgs) = nullptr;
+  if (p.d_k == 128) fwd_kernels<TQ, TS, 128>(long_form, k_state, k_full);
+  if (p.d_k == 64) fwd_kernels<TQ, TS, 64>(long_form, k_state, k_full);
+  if (p.d_k == 32) fwd_kernels<TQ, TS, 32>(long_form, k_state, k_full);
+  if (p.d_k == 16) fwd_kernels<TQ, TS, 16>(long_form, k_state, k_full);
   if (cudaFuncSetAttribute(k_full, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem0) != cudaSuccess ||
       cudaFuncSetAttribute(k_state, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1) != cudaSuccess)
     return LAWCAT_ERR_CUDA;
