@@ -509,8 +509,9 @@ static int conv_bwd_stream(const Ctx& c, const TD* du, const TI* x, const TI* w,
 
 // The same for bf16 storage, conv width up to 4 and fp32 du (whole-layer and mix backward), both streams in one launch, four
 // channels per thread: 16-byte loads of du and 8-byte loads of x, a group of 8 tokens in flight. Bound by HBM: du and x in, dx
-// out. One channel per thread, a launch per stream: 129 us at 8 x 1024 tokens, 32/8 heads of 64 (166 MB); this form 50 us.
-// A warp walks `span` tokens (a multiple of 8).
+// out. One channel per thread, a launch per stream: 129 us at 8 x 1024 tokens, 32/8 heads of 64 (166 MB); this form 43 us.
+// A warp walks `span` tokens (a multiple of 8). SPAN: its value where it is known (205 registers: two blocks per SM, each faster, loads
+// of the next group run ahead), or 0 (161 registers, three per SM).
 struct ConvBwd4 {
   const float* du[2];
   const bf16 *x[2], *w[2], *cache[2];
@@ -523,14 +524,15 @@ __device__ __forceinline__ void bf16x4(const uint2& r, float* f) {
   f[0] = __uint_as_float(r.x << 16); f[1] = __uint_as_float(r.x & 0xffff0000u);
   f[2] = __uint_as_float(r.y << 16); f[3] = __uint_as_float(r.y & 0xffff0000u);
 }
-__global__ void __launch_bounds__(128) conv_bwd4_kernel(const ConvBwd4 a) {
+template <int SPAN>
+__global__ void __launch_bounds__(128, SPAN ? 2 : 3) conv_bwd4_kernel(const ConvBwd4 a) {
   // warp = one of four neighbouring spans of the same 128 channels (C is a multiple of 16: a lane may be past the end)
   __shared__ float s_dw[3][16][33];
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, qb = (a.C[0] / 4 + 31) / 32;
   const int st = (int)blockIdx.y >= qb;
   const int C = st ? a.C[1] : a.C[0], ch = 4 * (((int)blockIdx.y - (st ? qb : 0)) * 32 + lane), K = a.K, T = a.T;
-  const int spans = (T + a.span - 1) / a.span, sg = (int)blockIdx.x * 4 + warp;
+  const int spans = SPAN ? (T + SPAN - 1) / SPAN : (T + a.span - 1) / a.span, sg = (int)blockIdx.x * 4 + warp;
   const bool on = ch < C && sg < a.B * spans;
   const float* du = st ? a.du[1] : a.du[0];
   const bf16* x = st ? a.x[1] : a.x[0];
@@ -538,7 +540,7 @@ __global__ void __launch_bounds__(128) conv_bwd4_kernel(const ConvBwd4 a) {
   const bf16* cache = st ? a.cache[1] : a.cache[0];
   bf16* dx = st ? a.dx[1] : a.dx[0];
   float* dw = st ? a.dw[1] : a.dw[0];
-  const int b = on ? sg / spans : 0, t0 = on ? sg % spans * a.span : 0, t1 = on ? min(T, t0 + a.span) : 0;
+  const int b = on ? sg / spans : 0, t0 = on ? sg % spans * (SPAN ? SPAN : a.span) : 0, t1 = on ? min(T, t0 + (SPAN ? SPAN : a.span)) : 0;
   const float* dub = du + (size_t)b * T * C + ch;
   const bf16* xb = x + (size_t)b * T * C + ch;
   float tap[4][4], acc[4][4], xw[3][4], dwin[3][4];  // [delta][channel]; x[t - 1 - i], du[t + i]
@@ -618,6 +620,27 @@ __global__ void __launch_bounds__(128) conv_bwd4_kernel(const ConvBwd4 a) {
   }
 }
 
+// Calls whose blocks all fit at two per SM take the shortest span of 16, 24 and 32 tokens that lets them, known to the compiler (700
+// tokens, 32/8 heads of 64: 7.4 us against 6.9; 3 x 500: 10.9 against 9.9). The others take the span with the least work on an SM:
+// whole rounds of three blocks, each as long as its span and about twelve tokens more for the first loads and the end. Against 32
+// tokens throughout, over 98 shapes: never slower, and within 0.3 us of the best span of each. Kernel alone: 8 x 1024 tokens, 32/8 heads
+// of 64: 47 us at 32, 39 at 48; 4 x 1300: 31 at 32, 35 at 48 (which a rule that counted two blocks as resident took), 26 at 64.
+static void launch_conv_bwd4(ConvBwd4 a, int cols, cudaStream_t stream) {
+  auto xblocks = [&](int s) { return ((long long)a.B * ((a.T + s - 1) / s) + 3) / 4; };
+  const int sms = sm_count();
+  a.span = 0;
+  for (int s = 32; s >= 16; s -= 8)
+    if (xblocks(s) * cols <= 2 * sms) a.span = s;
+  const bool known = a.span != 0;
+  long long best = 0;
+  for (int s = 16; s <= 64 && !known; s += 8) {
+    const long long cost = (xblocks(s) * cols + 3 * sms - 1) / (3 * sms) * (s + 12);
+    if (best == 0 || cost < best) { best = cost; a.span = s; }
+  }
+  auto* const kernel = !known ? conv_bwd4_kernel<0> : a.span == 16 ? conv_bwd4_kernel<16> : a.span == 24 ? conv_bwd4_kernel<24> : conv_bwd4_kernel<32>;
+  launch_behind(kernel, dim3((unsigned)xblocks(a.span), cols), dim3(128), 0, stream, a);
+}
+
 // the conv's backward of both streams from fp32 du (zeroed: an earlier kernel of the caller's has cleared dw_q and dw_k)
 template <typename TI>
 static int conv_bwd_both(const Ctx& c, const float* du_q, const float* du_k, const void* q, const void* k, const void* w_q,
@@ -632,22 +655,10 @@ static int conv_bwd_both(const Ctx& c, const float* du_q, const float* du_k, con
   const int Cq = p.H * p.d_k, Ck = p.H_kv * p.d_k;
   if (!zeroed && dw_q && cudaMemsetAsync(dw_q, 0, sizeof(float) * (size_t)Cq * p.conv_k, c.stream) != cudaSuccess) return LAWCAT_ERR_CUDA;
   if (!zeroed && dw_k && cudaMemsetAsync(dw_k, 0, sizeof(float) * (size_t)Ck * p.conv_k, c.stream) != cudaSuccess) return LAWCAT_ERR_CUDA;
-  // The span is the one with the least work on an SM: two blocks are resident (191 registers; held to 128, four are and take longer,
-  // 51 -> 62 us), a span's first loads are worth about four tokens. 8 x 1024 tokens, 32/8 heads of 64: 60 us at 16 tokens, 51 at 32,
-  // 45.5 at 48, 52 at 64; 4 x 1300 of 128: 71, 62, 58, 56.
-  const int cols = (Cq / 4 + 31) / 32 + (Ck / 4 + 31) / 32;
-  int span = 16;
-  long long best = 0;
-  for (int s = 16; s <= 64; s += 8) {
-    const long long blocks = (((long long)p.B * ((p.T + s - 1) / s) + 3) / 4) * cols, slots = 2LL * sm_count();
-    const long long cost = (blocks + slots - 1) / slots * (s + 4);
-    if (best == 0 || cost < best) { best = cost; span = s; }
-  }
   const ConvBwd4 a{{du_q, du_k}, {(const bf16*)q, (const bf16*)k}, {(const bf16*)w_q, (const bf16*)w_k},
-                   {(const bf16*)cache_q, (const bf16*)cache_k}, {(bf16*)dq, (bf16*)dk}, {dw_q, dw_k}, {Cq, Ck}, p.B, p.T, p.conv_k, span};
-  const dim3 grid((p.B * ((p.T + span - 1) / span) + 3) / 4, cols);
+                   {(const bf16*)cache_q, (const bf16*)cache_k}, {(bf16*)dq, (bf16*)dk}, {dw_q, dw_k}, {Cq, Ck}, p.B, p.T, p.conv_k, 0};
   LaunchScope _ls("conv_bwd4", c.stream);
-  launch_behind(conv_bwd4_kernel, grid, dim3(128), 0, c.stream, a);
+  launch_conv_bwd4(a, (Cq / 4 + 31) / 32 + (Ck / 4 + 31) / 32, c.stream);
   LAWCAT_CHECK_LAUNCH();
   return LAWCAT_OK;
 }
