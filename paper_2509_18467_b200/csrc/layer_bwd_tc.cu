@@ -91,6 +91,7 @@ struct Cfg {
   // fp32 [C][D] result tiles over operands that are dead by then
   static constexpr uint32_t R_WQ = R_S, R_WK = D == 128 ? R_S + C * D * 4 : R_PM, R_DV = D == 128 ? R_PM : R_E, R_DG = R_QS;
   static_assert(C * D * 4 <= 2 * T_SZ && C * D * 4 <= 2 * T_TOK && 2 * T_P >= C * 64 * 4, "aliases");
+  static_assert(R_WQ % 1024 == 0 && R_WK % 1024 == 0 && R_DV % 1024 == 0, "the copy engine's swizzle goes by the address");
   static_assert(R_BYTES <= (D == 128 ? 232448 : 115000) && F_BYTES <= (D == 128 ? 232448 : 115000), "shared memory budget");
   // tensor memory
   static constexpr uint32_t F_ST = 0, F_O = D + 16, F_P = 2 * (D + 16), COLS = D == 128 ? 512 : 256;
@@ -550,6 +551,10 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, D == 128 ? 1 : 2) reverse_ker
   const uint32_t bar = smem_u32(const_cast<int*>(s_fl)) + 32, bar_s = bar + 8;
   const int bh = blockIdx.x, h = bh % a.H, b = bh / a.H, G = a.H / a.Hkv, j = h / G;
   const int nch = (a.T + C - 1) / C;
+  if ((sb & 1023u) != 0) {  // (the swizzled result tiles need a 1024-byte aligned base)
+    if (tid == 0 && a.dev_status) atomicMax(a.dev_status, (int)LAWCAT_ERR_CUDA);
+    return;
+  }
   if (tid == 0) {
     mbar_init(bar, 1);
     mbar_init(bar_s, 1);
