@@ -1,8 +1,8 @@
 // Tensor-core kernels for conv -> shared linear layer -> softmax feature map (Section 4.1) and for the chain rule back
 // through them (distillation step, Section 5.1), bf16 storage.
 //
-// Forward: one thread block = one (batch, query head, tile of 128 tokens), both streams one after the other (they share
-// W_h): depthwise causal conv in fp32 -> operand, Y = u W_h by tcgen05 (fp32 accumulator in tensor memory), phi (softmax over
+// Forward: one thread block = one (batch, query head, tile of 128 tokens), both streams (they share W_h), each stream's products
+// behind the other one's work: depthwise causal conv in fp32 -> operand, Y = u W_h by tcgen05 (fp32 accumulator in tensor memory), phi (softmax over
 // the row, or the elementwise 1 + ELU / identity of Section 2) by the threads that own the row's TMEM lane, 16-bit or fp32
 // store.
 // Backward (head width 64): one block = one (batch, key head, tile); for each query head of

@@ -10,9 +10,9 @@
 // warps through shared memory; only the softmax crosses lanes, through a max reduction per token and a folding sum.
 // One block is lock-step with two barriers a chunk; 105 KB of shared memory and 256 tensor-memory columns let two blocks share
 // an SM, and one fills the other's waits: 4.4k cycles a chunk and SM (6.8k as a mode of the layer kernel, one block per SM).
-// Bound by instruction issue (9.8k warp instructions a chunk, 45 to 60 % of the slots) and shared-memory latency; the
-// special-function unit, four operations an entry, is at 39 %. 32 heads of 128, 32768 tokens: 323 -> 232 us; 32 heads of 64, 8192
-// tokens: 62.8 -> 47.7; 32 heads of 128, 1223 tokens: 31.4 -> 24.7. (With the row's maximum in front of the exponentials and four
+// Bound by instruction issue (10.2k warp instructions a chunk, 46 % of the slots) and shared-memory latency; the
+// special-function unit, four operations an entry, is at 38 %. 32 heads of 128, 32768 tokens: 323 -> 232 us; 32 heads of 64, 8192
+// tokens: 62.8 -> 47.7; 32 heads of 128, 1223 tokens: 31.4 -> 24.3. (With the row's maximum in front of the exponentials and four
 // barriers: 247, 49.2, 29.4.)
 #pragma once
 #include "layer_tc_kernel.cuh"
@@ -38,7 +38,9 @@ constexpr uint32_t OFF_BAR = OFF_G1 + 256;
 constexpr uint32_t SMEM_BYTES = OFF_BAR + 64;
 static_assert(SMEM_BYTES <= 115000, "two blocks per SM");
 constexpr uint32_t COL_Y = 0, COL_KH = 64, COL_S = 128, TMEM_COLS = 256;
-constexpr float Y_MAX = 24.f;                    // (exp(24) and the rounding of 24 log2(e), 2^-19, are far from any limit)
+// (exp(24) is far from any limit. The rounding of y log2(e) is up to 2^-19 at 24, 2^-22 at 4: a feature is off by up to 1.3e-6 or 3e-7
+// of itself before it is rounded to fp16, 2.4e-4. End states against 64 bits: the same to four digits as with the maximum taken off.)
+constexpr float Y_MAX = 24.f;
 enum { B_RAW = 0, B_G, B_V, B_MIX, B_UPD, NUM_BARS };
 
 // one value in all lanes: the largest (NaN counts as nothing)

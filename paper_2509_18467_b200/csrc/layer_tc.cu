@@ -213,7 +213,11 @@ size_t layer_tc_workspace_bytes(const lawcat_params& p) {
 // it takes to keep the longest from being the tail: L, the longest segment allowed, is the one with the smallest estimate of
 // chunk times over {longest / 1 .. longest / 8}: per block its chunks and about three more for set-up and pipeline fill, the
 // total spread over the SMs but never less than the longest block and half a block of unevenness; when something is cut, the
-// state-only pass over all but the last segments (0.65 of a chunk time each) and its two extra launches (about two).
+// state-only pass over all but the last segments and its two extra launches (about two). The pass is charged 0.65 of a chunk time a
+// chunk, one block per SM, in pieces of at least four chunks, which is dearer than it is (0.44, two blocks per SM; the price is of the
+// time when it was a mode of the layer kernel). The surplus stands in for what the estimate of the main launch leaves out, a last
+// round of a few blocks: at the true price 2 sequences of together 2500 tokens, 32 heads of 128, are cut into 160 blocks and take 122 us,
+// not 103. Over 70 batches of 2 to 32 sequences this rule is 3.6 % behind the best cut and piece count on average, 28 % at most.
 static void layer_tc_pack(const lawcat_params& p, const int32_t* cu, const int* order, int n, tc::PackTab& t, int& nsub) {
   const double sms = sm_count(), Hn = layer_tc_paired(p) ? p.H / 2 : p.H;
   auto chunks = [&](int i) { return (cu[order[i] + 1] - cu[order[i]] + tc::C - 1) / tc::C; };

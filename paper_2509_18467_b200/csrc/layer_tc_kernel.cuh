@@ -667,7 +667,6 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
           mma_commit(bar(B_P));
         }
         TL(0, 1, n, lane == 0);
-        TL(0, 2, n, lane == 0);
         if (elect_one()) {
           tc_fence_after_sync();
           // read-out O' | denominator = qs [2^b_mid S | 2^b_mid z] in one product per K step
@@ -1061,8 +1060,7 @@ layer_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       float y[32], ya[16], yb[16];
       float mb = 0.f, sum = 0.f;
       TL(warp == 8 ? 1 : 2, 0, n, (warp == 8 || warp == 10) && lane == 0);
-      // ---- mask of the previous chunk: its scores are the first product issued after the hand-over, ahead of this
-      // chunk's mix ---------------------------------------------------------------------------------------------------
+      // ---- mask of the previous chunk: its scores are the first product that the MMA warp issues after the hand-over ----
       if (is_q && n > 0) mask_chunk(n - 1);
       TL(warp == 8 ? 1 : 2, 1, n, (warp == 8 || warp == 10) && lane == 0);
       // ---- phi, reading sweeps ----------------------------------------------------------------------------------------

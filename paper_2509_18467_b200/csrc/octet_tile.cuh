@@ -16,7 +16,9 @@ using namespace tc;
 
 constexpr int TT = 128;   // tokens per tile
 constexpr int HALO = 3;   // raw rows kept in front of a tile (conv width up to 4)
-constexpr float Y_MAX = 24.f;  // |y| below which exp(y) is formed without the row's maximum (exp(24) is far from any limit)
+// |y| below which exp(y) is formed without the row's maximum (exp(24) is far from any limit; 16-bit features take 2^(y log2(e)), whose
+// argument is rounded by up to 2^-19: 1.3e-6 of a feature, which is then rounded to bf16, 2e-3)
+constexpr float Y_MAX = 24.f;
 
 // Grid of the kernels that take one (sequence, head) and one tile of TT tokens per block: x the (sequence, head), whose number
 // may pass the 65535 that end the other axes, y and z the tile.
